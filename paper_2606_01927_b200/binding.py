@@ -1,13 +1,15 @@
-"""ctypes binding of ``libalbireo_sample.so`` -- argument marshalling only.
+"""Python binding of ``libalbireo_sample.so`` -- argument marshalling only.
 
 Every step of the sampling path runs inside the CUDA library; this module only turns
 torch tensors (device memory, streams) into the pointers and sizes of the C ABI declared
-in ``include/albireo_sample.h``.  There is no CPU fallback: if the library is missing or
-does not load, importing this module raises.
+in ``include/albireo_sample.h``.  The sampling calls do that in native code
+(``csrc/native_binding.cpp``), the others through ctypes.  There is no CPU fallback: if the
+library is missing or does not load, importing this module raises.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 from dataclasses import dataclass
 from typing import Optional
@@ -77,19 +79,12 @@ def _load() -> C.CDLL:
     lib.albireo_sample_host_staging_bytes.argtypes = [i32, i32, i64]
     lib.albireo_sample_init.restype = C.c_int
     lib.albireo_sample_init.argtypes = [C.POINTER(vp), i32, i32, i32, i64, vp, C.c_size_t]
-    sample_args = [vp, vp, i32, i32, i32, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, u64, vp, vp, vp, C.POINTER(SampleExt)]
-    lib.albireo_sample.restype = C.c_int
-    lib.albireo_sample.argtypes = sample_args
-    lib.albireo_sample_host.restype = C.c_int
-    lib.albireo_sample_host.argtypes = sample_args[:14] + [i64] + sample_args[14:]
     lib.albireo_sample_destroy.restype = C.c_int
     lib.albireo_sample_destroy.argtypes = [vp]
     lib.albireo_last_error.restype = C.c_char_p
     lib.albireo_last_error.argtypes = [vp]
     lib.albireo_sample_launch_count.restype = C.c_uint64
     lib.albireo_sample_launch_count.argtypes = [vp]
-    lib.albireo_sample_fixed_scratch.restype = C.c_int
-    lib.albireo_sample_fixed_scratch.argtypes = sample_args[1:14] + [i64] + sample_args[14:]
     lib.albireo_sample_fixed_scratch_error.restype = C.c_char_p
     lib.albireo_sample_fixed_scratch_error.argtypes = []
     lib.albireo_stream_only.restype = C.c_int
@@ -97,7 +92,20 @@ def _load() -> C.CDLL:
     return lib
 
 
+def _load_native():
+    path = _build.NATIVE_PATH
+    if not os.path.exists(path):
+        raise ImportError(
+            f"{path} is missing: build it with `python -c 'import __graft_entry__ as g; g.build()'`.")
+    spec = importlib.util.spec_from_file_location(__package__ + "._native", path)
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    return mod
+
+
 LIB = _load()
+_sample = _load_native().sample
+_DEVICE, _HOST, _FIXED = 0, 1, 2      # entry points of _native.sample
 
 
 class AlbireoError(RuntimeError):
@@ -112,14 +120,6 @@ def albireo_sample_workspace_bytes(max_rows: int, max_vocab: int, max_history_to
 
 def albireo_sample_host_staging_bytes(max_rows: int, max_vocab: int, max_history_total: int) -> int:
     return int(LIB.albireo_sample_host_staging_bytes(max_rows, max_vocab, max_history_total))
-
-
-def _dp(t: Optional[torch.Tensor], dtype, device_type: str):
-    if t is None:
-        return None
-    if t.dtype != dtype or not t.is_contiguous() or t.device.type != device_type:
-        raise ValueError(f"expected contiguous {dtype} tensor on {device_type}, got {t.dtype} on {t.device}")
-    return C.c_void_p(t.data_ptr())
 
 
 @dataclass
@@ -155,6 +155,7 @@ class Sampler:
                                          max_history_total, C.c_void_p(self._ws_ptr), nbytes)
         if rc != OK:
             raise AlbireoError(rc, "albireo_sample_init failed")
+        self._handle_int = self._handle.value
 
     # -- raw pass-through ------------------------------------------------------------
     def last_error(self) -> str:
@@ -167,48 +168,13 @@ class Sampler:
         if getattr(self, "_handle", None) is not None and self._handle:
             LIB.albireo_sample_destroy(self._handle)
             self._handle = C.c_void_p()
+            self._handle_int = 0
 
     def __del__(self):
         try:
             self.close()
         except Exception:
             pass
-
-    def _ext(self, B, dev_type, device, *, row_base=0, row_stride=0, num_top=0, want_counts=False,
-             dbg_cap=0, want_status=False, flags=0, out_top_ids=None, out_top_logprobs=None):
-        ext = SampleExt()
-        ext.struct_size = C.sizeof(SampleExt)
-        ext.flags = flags
-        ext.row_stride_elems = row_stride
-        ext.row_base = row_base
-        ext.num_top = num_top
-        out = {}
-        kw = dict(device=device) if dev_type == "cuda" else dict(pin_memory=True)
-        if num_top > 0:
-            if out_top_ids is not None and (out_top_ids.dtype != torch.int32 or out_top_ids.numel() < B * num_top
-                                            or not out_top_ids.is_contiguous()):
-                raise ValueError("out_top_ids must be a contiguous int32 tensor of B * num_top entries")
-            if out_top_logprobs is not None and (out_top_logprobs.dtype != torch.float32 or out_top_logprobs.numel() < B * num_top
-                                                 or not out_top_logprobs.is_contiguous()):
-                raise ValueError("out_top_logprobs must be a contiguous float32 tensor of B * num_top entries")
-            out["top_ids"] = torch.empty((B, num_top), dtype=torch.int32, **kw) if out_top_ids is None else out_top_ids
-            out["top_logprobs"] = (torch.empty((B, num_top), dtype=torch.float32, **kw)
-                                   if out_top_logprobs is None else out_top_logprobs)
-            ext.out_top_ids = out["top_ids"].data_ptr()
-            ext.out_top_logprobs = out["top_logprobs"].data_ptr()
-        if want_counts:
-            out["num_kept"] = torch.empty(B, dtype=torch.int32, **kw)
-            out["num_topk"] = torch.empty(B, dtype=torch.int32, **kw)
-            ext.out_num_kept = out["num_kept"].data_ptr()
-            ext.out_num_topk = out["num_topk"].data_ptr()
-        if dbg_cap > 0:
-            out["dbg_topk_ids"] = torch.empty((B, dbg_cap), dtype=torch.int32, **kw)
-            ext.dbg_cap = dbg_cap
-            ext.dbg_topk_ids = out["dbg_topk_ids"].data_ptr()
-        if want_status:
-            out["row_status"] = torch.empty(B, dtype=torch.int32, **kw)
-            ext.out_row_status = out["row_status"].data_ptr()
-        return ext, out
 
     def albireo_sample(self, logits: torch.Tensor, *, temperature=None, top_k=None, top_p=None, min_p=None,
                        repetition_penalty=None, presence_penalty=None, frequency_penalty=None,
@@ -227,80 +193,14 @@ class Sampler:
         ``exp1`` (float32 ``[B, V]``) replaces the counter-based draw by pre-generated Exp(1)
         variates; ``backfill_ids`` / ``backfill_index`` (int32) and ``feedback_ring`` (int64,
         device or pinned host memory) are the early-feedback targets."""
-        nseg = 0
-        if logits.dim() == 3:
-            # rows in pieces, [t, B, V / t]: the receive buffer of the sequence-parallel all-to-all
-            if logits.stride(2) != 1:
-                raise ValueError("logits in pieces must be [t, B, V/t] with unit stride along the last axis")
-            nseg = logits.shape[0]
-            B = logits.shape[1] if B is None else B
-            V = nseg * logits.shape[2] if V is None else V
-        elif logits.dim() != 2 or logits.stride(1) != 1:
-            raise ValueError("logits must be [B, V] with unit stride along V")
-        else:
-            B = logits.shape[0] if B is None else B
-            V = logits.shape[1] if V is None else V
-        dt = _dtype_code(logits)
-        dev = logits.device
-        if out_tokens is None:
-            out_tokens = torch.empty(B, dtype=torch.int32, device=dev)
-        if out_logprobs is None:
-            out_logprobs = torch.empty(B, dtype=torch.float32, device=dev)
-        row_stride = logits.stride(0) if B > 1 else V
-        if nseg:
-            row_stride = logits.stride(1)
-        ext, extra = self._ext(B, "cuda", dev, row_base=row_base, row_stride=0 if row_stride == V else row_stride,
-                               num_top=num_top, want_counts=want_counts, dbg_cap=dbg_cap,
-                               want_status=want_status, flags=flags, out_top_ids=out_top_ids,
-                               out_top_logprobs=out_top_logprobs)
-        if nseg:
-            ext.num_segments = nseg
-            ext.segment_stride_elems = logits.stride(0)
-            ext.row_stride_elems = row_stride
-        if output_start is not None:
-            ext.history_output_start = _dp(output_start, torch.int32, "cuda")
-        if segment_tensors is not None:
-            # one [rows, V/t] buffer per piece (e.g. the peers' vocabulary shards in symmetric memory), read in place
-            t_ = len(segment_tensors)
-            sh0 = segment_tensors[0]
-            if any(x.dim() != 2 or x.stride(1) != 1 or x.dtype != sh0.dtype or x.shape[1] != sh0.shape[1]
-                   or x.stride(0) != sh0.stride(0) for x in segment_tensors):
-                raise ValueError("segment_tensors must be same-shaped [rows, V/t] tensors with unit stride along V/t")
-            ptrs = (C.c_void_p * t_)(*[x.data_ptr() for x in segment_tensors])
-            ext.num_segments = t_
-            ext.segment_ptrs = C.cast(ptrs, C.c_void_p)
-            ext.segment_row_offset = segment_row_offset
-            ext.row_stride_elems = sh0.stride(0)
-            ext._keepalive = ptrs
-        if exp1 is not None:
-            if exp1.dtype != torch.float32 or exp1.dim() != 2 or exp1.stride(1) != 1 or exp1.device != dev:
-                raise ValueError("exp1 must be a float32 [B, V] tensor on the logits' device")
-            ext.exp1 = exp1.data_ptr()
-            ext.exp1_stride_elems = 0 if (B <= 1 or exp1.stride(0) == V) else exp1.stride(0)
-        if backfill_ids is not None:
-            ext.backfill_ids = _dp(backfill_ids, torch.int32, "cuda")
-            ext.backfill_index = _dp(backfill_index, torch.int32, "cuda")
-            ext.backfill_len = backfill_ids.numel()
-        if feedback_ring is not None:
-            if feedback_ring.dtype != torch.int64 or not feedback_ring.is_contiguous():
-                raise ValueError("feedback_ring must be a contiguous int64 tensor (device, or pinned host memory)")
-            ext.feedback_ring = feedback_ring.data_ptr()
-            ext.feedback_cap = feedback_ring.numel()
-            ext.feedback_head = feedback_head
-        st = torch.cuda.current_stream(dev) if stream is None else stream
-        f32, i32 = torch.float32, torch.int32
-        with torch.cuda.device(dev):
-            rc = LIB.albireo_sample(
-                self._handle, C.c_void_p(logits.data_ptr()), B, V, dt,
-                _dp(temperature, f32, "cuda"), _dp(top_k, i32, "cuda"), _dp(top_p, f32, "cuda"), _dp(min_p, f32, "cuda"),
-                _dp(repetition_penalty, f32, "cuda"), _dp(presence_penalty, f32, "cuda"),
-                _dp(frequency_penalty, f32, "cuda"), _dp(history_ids, i32, "cuda"), _dp(history_offsets, i32, "cuda"),
-                _dp(seeds, torch.int64, "cuda"), C.c_uint64(step),
-                C.c_void_p(out_tokens.data_ptr()), C.c_void_p(out_logprobs.data_ptr()),
-                C.c_void_p(st.cuda_stream), C.byref(ext))
-        if rc != OK:
-            raise AlbireoError(rc, self.last_error())
-        return SampleOutputs(out_tokens, out_logprobs, **extra)
+        r = _sample(_DEVICE, self._handle_int, None, logits, temperature, top_k, top_p, min_p, repetition_penalty,
+                    presence_penalty, frequency_penalty, history_ids, history_offsets, seeds, step, out_tokens, out_logprobs,
+                    stream, row_base, num_top, want_counts, dbg_cap, want_status, flags, B, V, exp1, backfill_ids,
+                    backfill_index, feedback_ring, feedback_head, output_start, segment_tensors, segment_row_offset,
+                    out_top_ids, out_top_logprobs, None)
+        if r.__class__ is int:
+            raise AlbireoError(r, self.last_error())
+        return SampleOutputs(*r)
 
     def albireo_stream_only(self, logits: torch.Tensor, sink: torch.Tensor, stream: Optional[torch.cuda.Stream] = None,
                             drop_tile: int = -1):
@@ -323,29 +223,13 @@ class Sampler:
                             row_base: int = 0, num_top: int = 0, want_counts=False, want_status=False,
                             flags: int = 0) -> SampleOutputs:
         """Host-buffer call (CPU tensors, ideally pinned): copies in, samples, copies out, waits."""
-        B, V = logits.shape
-        dt = _dtype_code(logits)
-        if out_tokens is None:
-            out_tokens = torch.empty(B, dtype=torch.int32, pin_memory=True)
-        if out_logprobs is None:
-            out_logprobs = torch.empty(B, dtype=torch.float32, pin_memory=True)
-        ext, extra = self._ext(B, "cpu", None, row_base=row_base, num_top=num_top, want_counts=want_counts,
-                               want_status=want_status, flags=flags)
-        st = torch.cuda.current_stream(self.device) if stream is None else stream
-        f32, i32 = torch.float32, torch.int32
-        htot = int(history_ids.numel()) if history_ids is not None else 0
-        with torch.cuda.device(self.device):
-            rc = LIB.albireo_sample_host(
-                self._handle, C.c_void_p(logits.data_ptr()), B, V, dt,
-                _dp(temperature, f32, "cpu"), _dp(top_k, i32, "cpu"), _dp(top_p, f32, "cpu"), _dp(min_p, f32, "cpu"),
-                _dp(repetition_penalty, f32, "cpu"), _dp(presence_penalty, f32, "cpu"),
-                _dp(frequency_penalty, f32, "cpu"), _dp(history_ids, i32, "cpu"), _dp(history_offsets, i32, "cpu"),
-                C.c_int64(htot), _dp(seeds, torch.int64, "cpu"), C.c_uint64(step),
-                C.c_void_p(out_tokens.data_ptr()), C.c_void_p(out_logprobs.data_ptr()),
-                C.c_void_p(st.cuda_stream), C.byref(ext))
-        if rc != OK:
-            raise AlbireoError(rc, self.last_error())
-        return SampleOutputs(out_tokens, out_logprobs, **extra)
+        r = _sample(_HOST, self._handle_int, self.device.index, logits, temperature, top_k, top_p, min_p, repetition_penalty,
+                    presence_penalty, frequency_penalty, history_ids, history_offsets, seeds, step, out_tokens, out_logprobs,
+                    stream, row_base, num_top, want_counts, 0, want_status, flags, None, None, None, None,
+                    None, None, 0, None, None, 0, None, None, None)
+        if r.__class__ is int:
+            raise AlbireoError(r, self.last_error())
+        return SampleOutputs(*r)
 
 
 def albireo_sample_fixed_scratch(logits: torch.Tensor, *, temperature=None, top_k=None, top_p=None, min_p=None,
@@ -358,40 +242,13 @@ def albireo_sample_fixed_scratch(logits: torch.Tensor, *, temperature=None, top_
     fixed scratch array is used).  The output tensors created here when none are passed (and the
     per-row status / count arrays when asked for) are a convenience of this Python wrapper; the C
     entry point itself allocates nothing."""
-    B, V = logits.shape
-    dt = _dtype_code(logits)
-    dev = logits.device
-    if out_tokens is None:
-        out_tokens = torch.empty(B, dtype=torch.int32, device=dev)
-    if out_logprobs is None:
-        out_logprobs = torch.empty(B, dtype=torch.float32, device=dev)
-    ext = SampleExt()
-    ext.struct_size = C.sizeof(SampleExt)
-    ext.row_base = row_base
-    row_status = num_kept = num_topk = None
-    if want_status:
-        row_status = torch.zeros(B, dtype=torch.int32, device=dev)
-        ext.out_row_status = row_status.data_ptr()
-    if want_counts:
-        num_kept = torch.empty(B, dtype=torch.int32, device=dev)
-        num_topk = torch.empty(B, dtype=torch.int32, device=dev)
-        ext.out_num_kept, ext.out_num_topk = num_kept.data_ptr(), num_topk.data_ptr()
-    if history_total is None:
-        history_total = int(history_ids.numel()) if history_ids is not None else 0
-    st = torch.cuda.current_stream(dev) if stream is None else stream
-    f32, i32 = torch.float32, torch.int32
-    with torch.cuda.device(dev):
-        rc = LIB.albireo_sample_fixed_scratch(
-            C.c_void_p(logits.data_ptr()), B, V, dt,
-            _dp(temperature, f32, "cuda"), _dp(top_k, i32, "cuda"), _dp(top_p, f32, "cuda"), _dp(min_p, f32, "cuda"),
-            _dp(repetition_penalty, f32, "cuda"), _dp(presence_penalty, f32, "cuda"),
-            _dp(frequency_penalty, f32, "cuda"), _dp(history_ids, i32, "cuda"), _dp(history_offsets, i32, "cuda"),
-            C.c_int64(history_total), _dp(seeds, torch.int64, "cuda"), C.c_uint64(step),
-            C.c_void_p(out_tokens.data_ptr()), C.c_void_p(out_logprobs.data_ptr()),
-            C.c_void_p(st.cuda_stream), C.byref(ext))
-    if rc != OK:
-        raise AlbireoError(rc, LIB.albireo_sample_fixed_scratch_error().decode())
-    return SampleOutputs(out_tokens, out_logprobs, num_kept=num_kept, num_topk=num_topk, row_status=row_status)
+    r = _sample(_FIXED, 0, None, logits, temperature, top_k, top_p, min_p, repetition_penalty,
+                presence_penalty, frequency_penalty, history_ids, history_offsets, seeds, step, out_tokens, out_logprobs,
+                stream, row_base, 0, want_counts, 0, want_status, 0, None, None, None, None,
+                None, None, 0, None, None, 0, None, None, history_total)
+    if r.__class__ is int:
+        raise AlbireoError(r, LIB.albireo_sample_fixed_scratch_error().decode())
+    return SampleOutputs(*r)
 
 
 # ------------------------------------------------------------------ workload marshalling
