@@ -89,6 +89,7 @@ struct SampleArgs {
     uint32_t *ws_counts;        // global scratch for history counts of rows with many distinct ids
     int64_t ws_counts_cap;      // entries
     int32_t elem_size;          // host side only: bytes per logit
+    int32_t slice_bytes;        // shared memory of a row's slice (cluster kernel)
     // rows in pieces (vocabulary shards as the all-to-all of sequence-parallel sampling leaves them)
     int32_t seg_ptr_count;      // > 0: the pieces live in buffers of their own, seg_ptr[j]; 0: a stride apart in `logits`
     int64_t seg_stride;         // elements between consecutive pieces of a row
@@ -126,21 +127,7 @@ __device__ __forceinline__ uint32_t race_word(uint64_t seed, uint32_t R, uint64_
     return wsel == 0 ? c0 : wsel == 1 ? c1 : wsel == 2 ? c2 : c3;
 }
 
-// -ln(E) for E = -log1p(-v), v = (w + 1/2) 2^-32, in fp32.  The half of the range near
-// v = 1 is evaluated from 1 - v = (~w + 1/2) 2^-32 so both ends keep full relative accuracy.
-__device__ __forceinline__ float neg_log_exp1_f32(uint32_t w) {
-    float E;
-    if (w < 0x80000000u) {
-        float v = __fmaf_rn((float)w, 2.3283064365386963e-10f, 1.1641532182693481e-10f);
-        E = -log1pf(-v);
-    } else {
-        float omv = __fmaf_rn((float)(~w), 2.3283064365386963e-10f, 1.1641532182693481e-10f);
-        E = -logf(omv);
-    }
-    return -logf(E);
-}
-// The same quantity for the general path, where it is evaluated once per kept element of rows that
-// may keep tens of thousands: branch-free, hardware logarithms.  E = v + v^2/2 + ... for v < 1/4
+// -ln(E) for E = -log1p(-v), v = (w + 1/2) 2^-32: branch-free, hardware logarithms.  E = v + v^2/2 + ... for v < 1/4
 // (the small-E end decides the race and keeps full relative accuracy there), E = -ln(1 - v) above;
 // absolute error of the result about 1e-6, inside the band in which the race counts as a near-tie.
 __device__ __forceinline__ float neg_log_exp1_fast(uint32_t w) {
@@ -156,11 +143,6 @@ __device__ __forceinline__ float neg_log_exp1_fast(uint32_t w) {
 }
 
 __device__ __forceinline__ uint32_t orderable_f32(float g) { return key_of(g); }
-
-// fixed-point mass of an element at distance d = z - zmax <= 0 (deterministic integer sums)
-__device__ __forceinline__ u64 mass_fx(float d) {
-    return __float2ull_rn(expf(d) * FX_SCALE);
-}
 
 // ------------------------------------------------------------------ block primitives
 
@@ -1444,8 +1426,9 @@ __device__ __forceinline__ void cand_append_one(BlockScratch &s, const CandSmem 
 // the comparisons of one candidate when n is small), its mass and its race score, written to its
 // sorted position.  Step 2 (warp 0): the cuts as prefix operations and the argmax of the race.
 // `full_fx` != 0: the log-probabilities are relative to that mass (the whole row's) instead of the kept set's.
+// The top-N list is the head of the first `list_len` candidates (0: of the kept set).
 __device__ void final_stage(BlockScratch &s, const CandSmem &cs, int n, int L6, float zmax, bool has_minp,
-                            const RowParams &rp, const SampleArgs &a, int b, RowOut &out, u64 full_fx) {
+                            const RowParams &rp, const SampleArgs &a, int b, RowOut &out, u64 full_fx, int list_len) {
     const int lane = threadIdx.x & 31;
     // `parts` threads share one candidate's comparisons; the threads after them (from the next warp
     // boundary on) take one candidate each for the race term and the mass, so those long dependent
@@ -1583,10 +1566,11 @@ __device__ void final_stage(BlockScratch &s, const CandSmem &cs, int n, int L6, 
     }
     out.token = tok; out.logprob = lp_tok; out.n_keep = L8;
     if (a.num_top > 0) {
-        for (int q = lane; q < a.num_top && q < L8; q += 32) {
+        const int members = list_len ? list_len : L8;
+        for (int q = lane; q < a.num_top && q < members; q += 32) {
             const int64_t o = (int64_t)b * a.num_top + q;
             a.out_top_ids[o] = comp_idx(sorted[q]);
-            a.out_top_logprobs[o] = (L8 == 1 && !full_fx) ? 0.0f : __fsub_rn(unkey((uint32_t)(sorted[q] >> 32)), zmax) - lnS;
+            a.out_top_logprobs[o] = (members == 1 && !full_fx) ? 0.0f : __fsub_rn(unkey((uint32_t)(sorted[q] >> 32)), zmax) - lnS;
         }
     }
 }
@@ -1667,15 +1651,61 @@ __device__ void candidate_begin(BlockScratch &s, const Ring &rg, const RowCtx &c
 }
 
 // which rows the candidate path takes (decided from the row's parameters alone)
-// (a top-N list over the whole vocabulary is the general path's business: the candidate list ends
-// where the cuts end)
-__device__ __forceinline__ bool candidate_eligible(const RowParams &rp, int V, bool full_list) {
-    if (full_list) return false;
+// (a top-N list over the whole vocabulary needs a top-k threshold that covers it: the list is then the
+// head of the sorted candidates, whatever the cuts keep of them)
+__device__ __forceinline__ bool candidate_eligible(const RowParams &rp, const SampleArgs &a) {
+    const int k = rp.greedy ? 1 : rp.top_k;
+    const bool has_topk = rp.greedy || (k >= 1 && k < a.V);
+    const bool has_minp = !rp.greedy && rp.min_p > 0.0f;
+    if (has_topk && k > KA_MAX) return false;
+    if ((a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) && a.num_top > 0) return has_topk && (rp.greedy || !(a.flags & ALBIREO_FLAG_TOPK_KEEP_TIES));
+    return has_topk || has_minp;
+}
+// which of the others the wide path takes: everything without an active top-k
+__device__ __forceinline__ bool wide_eligible(const RowParams &rp, const SampleArgs &a) {
+    return !(a.flags & ALBIREO_FLAG_FORCE_GENERAL) && !rp.greedy && !(rp.top_k >= 1 && rp.top_k < a.V);
+}
+
+// From the candidate list cand[0..n) (every element of the row with key >= tau_key) to the result.
+// `full_fx` != 0: the mass of the whole row, which the log-probabilities are relative to.  `count_finite`
+// is called, by every thread, only where the number of finite scores is asked for and not known.
+template <class F>
+__device__ __forceinline__ bool candidate_finish(BlockScratch &s, const CandSmem &cs, int n, uint32_t tau_key, uint32_t kmax, const RowParams &rp,
+                                                 const SampleArgs &a, int b, RowOut &out, u64 full_fx, F &&count_finite) {
+    const int V = a.V;
+    const bool full_list = (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) && a.num_top > 0;
     const int k = rp.greedy ? 1 : rp.top_k;
     const bool has_topk = rp.greedy || (k >= 1 && k < V);
     const bool has_minp = !rp.greedy && rp.min_p > 0.0f;
-    if (has_topk && k > KA_MAX) return false;
-    return has_topk || has_minp;
+    const bool stream_minp = has_minp && !full_list && !(has_topk && a.dbg_topk_ids != nullptr);
+    const int k_list = full_list ? max(k, a.num_top) : k;      // the list holds at least this many (or all there are)
+    bool topk_exact_known = true;      // is min(k, #finite) known without counting?
+    // keep-ties mode: the top-k stage keeps every score not below the k-th largest, i.e. exactly the
+    // candidates that are left once the list is cut at the k-th largest key
+    const bool keep_ties = has_topk && !rp.greedy && (a.flags & ALBIREO_FLAG_TOPK_KEEP_TIES);
+    if (has_topk) {
+        if (n > SORT_MAX || n > 2 * k_list + 96 || (keep_ties && n > k)) {
+            uint32_t t = cand_select_exact(s, cs, n, k_list, tau_key, kmax);
+            n = cand_compact(s, cs, n, t);
+        }
+        if (n < k && stream_minp) topk_exact_known = false;
+    } else {
+        n = cand_compact(s, cs, n, minp_key(unkey(kmax), rp.ln_min_p));
+        topk_exact_known = false;
+    }
+    if (n > SORT_MAX || n < 1) return false;
+
+    const int L6 = has_topk ? ((n < k || keep_ties) ? n : k) : n;
+    int n_topk = L6;
+    if (!topk_exact_known && a.out_num_topk) {
+        const u64 nfin = count_finite();
+        n_topk = has_topk ? (int)(nfin < (u64)k ? nfin : (u64)k) : (int)nfin;
+    }
+    out.n_topk = n_topk;
+    // the stream is over: the next kernel in the stream may be scheduled from here on
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    final_stage(s, cs, n, L6, unkey(kmax), has_minp, rp, a, b, out, full_fx, full_list ? n : 0);
+    return true;
 }
 
 // Returns false if the row must be handled by the general path instead.  On success the
@@ -1686,14 +1716,14 @@ __device__ bool candidate_path(BlockScratch &s, const CandSmem &cs, const Ring &
     typedef Elem<DT> E;
     typedef VecTest<DT> T;
     const int V = c.V;
-    const int k = rp.greedy ? 1 : rp.top_k;
-    const bool has_topk = rp.greedy || (k >= 1 && k < V);
+    const bool full_list = (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) && a.num_top > 0;
+    const bool has_topk = rp.greedy || (rp.top_k >= 1 && rp.top_k < V);
+    // the rank the threshold covers: top-k, or the list over the whole vocabulary if that is longer
+    const int k = full_list ? max(rp.greedy ? 1 : rp.top_k, a.num_top) : rp.greedy ? 1 : rp.top_k;
     const bool has_minp = !rp.greedy && rp.min_p > 0.0f;
-    if (has_topk && k > KA_MAX) return false;
-    if (!has_topk && !has_minp) return false;
     // with the debug id list requested, keep the stream's threshold purely top-k so that the
     // top-k stage's set is known exactly
-    const bool stream_minp = has_minp && !(has_topk && a.dbg_topk_ids != nullptr);
+    const bool stream_minp = has_minp && !full_list && !(has_topk && a.dbg_topk_ids != nullptr);
     const int lane = threadIdx.x & 31;
     // Thread -> vector map inside each group of NT vectors: lane l of warp w takes vector
     // 16 l + ((w + l) & 15).  Consecutive vectors land in different warps (the head of the
@@ -1952,37 +1982,68 @@ __device__ bool candidate_path(BlockScratch &s, const CandSmem &cs, const Ring &
     if (ovf || n < 1) return false;
 
     const uint32_t kmax = s.runmax;    // the row's largest score is always a candidate
-    bool topk_exact_known = true;      // is min(k, #finite) known without counting?
-    // keep-ties mode: the top-k stage keeps every score not below the k-th largest, i.e. exactly the
-    // candidates that are left once the list is cut at the k-th largest key
-    const bool keep_ties = has_topk && !rp.greedy && (a.flags & ALBIREO_FLAG_TOPK_KEEP_TIES);
-    if (has_topk) {
-        if (n > SORT_MAX || n > 2 * k + 96 || (keep_ties && n > k)) {
-            uint32_t t = cand_select_exact(s, cs, n, k, tau_key, kmax);
-            n = cand_compact(s, cs, n, t);
-        }
-        if (n < k && stream_minp) topk_exact_known = false;
-    } else {
-        n = cand_compact(s, cs, n, minp_key(unkey(kmax), rp.ln_min_p));
-        topk_exact_known = false;
-    }
-    if (n > SORT_MAX || n < 1) return false;
-
-    const int L6 = has_topk ? ((n < k || keep_ties) ? n : k) : n;
-    int n_topk = L6;
-    if (!topk_exact_known && a.out_num_topk) {
+    const u64 full_fx = (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) ? full_vocab_mass<DT>(s, c, unkey(kmax)) : 0ull;
+    return candidate_finish(s, cs, n, tau_key, kmax, rp, a, b, out, full_fx, [&] {
         // diagnostic only: count the finite scores of the row
         uint32_t local = 0;
         for_each_score<DT>(c, [&](int, float z) { uint32_t kk = key_of(z); local += (kk >= KEY_MIN_FINITE && kk < KEY_POS_INF); });
-        u64 nfin = block_sum_u64(s, local);
-        n_topk = has_topk ? (int)(nfin < (u64)k ? nfin : (u64)k) : (int)nfin;
+        return block_sum_u64(s, local);
+    });
+}
+
+#include "wide_path.cuh"
+
+// ------------------------------------------------------------------ a row's parameters and its results
+
+// The row's parameters and where it lies; the history tables are not looked at here.  Returns the status
+// bits of parameters outside the contract.
+template <int DT>
+__device__ __forceinline__ uint32_t load_row(const SampleArgs &a, int b, const char *const *seg_base, RowParams &rp, RowCtx &c) {
+    rp.T = a.temperature ? a.temperature[b] : 1.0f;
+    rp.top_k = a.top_k ? a.top_k[b] : 0;
+    rp.top_p = a.top_p ? a.top_p[b] : 1.0f;
+    rp.min_p = a.min_p ? a.min_p[b] : 0.0f;
+    rp.seed = a.seeds ? a.seeds[b] : 0ull;
+    c.r = a.rep ? a.rep[b] : 1.0f;
+    c.p = a.pres ? a.pres[b] : 0.0f;
+    c.f = a.freq ? a.freq[b] : 0.0f;
+    rp.R = a.row_base + (uint32_t)b;
+    rp.greedy = !(rp.T > 0.0f);
+    rp.ln_min_p = (!rp.greedy && rp.min_p > 0.0f) ? log((double)rp.min_p) : 0.0;
+    c.invT = rp.greedy ? 1.0f : __fdiv_rn(1.0f, rp.T);
+    c.row = (const char *)a.logits + (size_t)b * (size_t)a.row_stride * Elem<DT>::SIZE;
+    if (a.nseg > 1 && a.seg_ptr_count > 0) c.row = (const char *)a.seg_ptr[0] + (size_t)(a.seg_row_offset + b) * (size_t)a.row_stride * Elem<DT>::SIZE;
+    c.V = a.V; c.nseg = a.nseg; c.Vs = a.Vs; c.seg_base = seg_base;
+    c.has_hist = false; c.bitmap = nullptr; c.coarse = nullptr; c.counts = nullptr; c.n_distinct = 0; c.ncoarse = 0;
+    return ((rp.T < 0.0f || rp.T != rp.T) || !(c.r > 0.0f)) ? ALBIREO_ROW_BAD_PARAM : 0u;
+}
+__device__ __forceinline__ void fill_general_args(GenArgs &ga, const SampleArgs &a) {
+    ga.dbg_topk_ids = a.dbg_topk_ids; ga.exp1 = a.exp1; ga.exp1_stride = a.exp1_stride; ga.out_top_ids = a.out_top_ids;
+    ga.out_top_logprobs = a.out_top_logprobs; ga.step = a.step; ga.flags = a.flags; ga.num_top = a.num_top; ga.dbg_cap = a.dbg_cap;
+}
+__device__ __forceinline__ void store_row(const SampleArgs &a, int b, RowOut &out) {
+    if (threadIdx.x == 0) {
+        a.out_tokens[b] = out.token;
+        a.out_logprobs[b] = out.logprob;
+        if (a.out_num_kept) a.out_num_kept[b] = out.n_keep;
+        if (a.out_num_topk) a.out_num_topk[b] = out.n_topk;
+        // early feedback (section 5.2): the token goes straight into the next iteration's input ids
+        // and to the output processor's ring, without waiting for a host round trip
+        const bool have_token = !(out.status & ALBIREO_ROW_TIMEOUT);
+        if (a.backfill_ids && have_token) {
+            const int64_t slot = a.backfill_index ? (int64_t)a.backfill_index[b] : (int64_t)b;
+            if (slot >= 0) {
+                if (slot < a.backfill_len) a.backfill_ids[slot] = out.token;
+                else out.status |= ALBIREO_ROW_BAD_PARAM;
+            }
+        }
+        if (a.feedback_ring && have_token) {
+            const int64_t slot = (a.feedback_head + b) % a.feedback_cap;
+            const unsigned long long rec = ((unsigned long long)(a.row_base + (uint32_t)b) << 32) | (uint32_t)out.token;
+            *(volatile unsigned long long *)(a.feedback_ring + slot) = rec;      // one 8-byte store
+        }
+        if (a.out_row_status) a.out_row_status[b] = out.status;
     }
-    out.n_topk = n_topk;
-    const u64 full_fx = (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) ? full_vocab_mass<DT>(s, c, unkey(kmax)) : 0ull;
-    // the stream is over: a dependent kernel launched the same way may be scheduled from here on
-    if (a.flags & ALBIREO_FLAG_PROGRAMMATIC_LAUNCH) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    final_stage(s, cs, n, L6, unkey(kmax), has_minp, rp, a, b, out, full_fx);
-    return true;
 }
 
 // ------------------------------------------------------------------ the kernel
@@ -2008,10 +2069,10 @@ __global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const SampleArgs 
     // shared memory.
     const bool ring_started = !(a.flags & ALBIREO_FLAG_FORCE_GENERAL);
     if (ring_started) ring_setup(s, rg);
-    // Under programmatic dependent launch the CTA may have been scheduled while the kernel ahead in the
+    // (Programmatic dependent launch.)  The CTA may have been scheduled while the kernel ahead in the
     // stream (the producer of the logits) was still running: everything above touched only launch
     // arguments and shared memory; nothing below is read or written before that kernel has finished.
-    if (a.flags & ALBIREO_FLAG_PROGRAMMATIC_LAUNCH) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     // The row's own parameters and the first part of its history are asked for before the ring is started: a
     // load issued after the ring's copies (this CTA's and every other's) queues behind megabytes of
     // them; issued before, it is back within an idle round trip, while thread 0 is still setting up.
@@ -2073,7 +2134,7 @@ __global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const SampleArgs 
     c.has_hist = false; c.bitmap = nullptr; c.coarse = nullptr; c.counts = nullptr; c.n_distinct = 0; c.ncoarse = 0;
     if (!(c.r > 0.0f)) out.status |= ALBIREO_ROW_BAD_PARAM;
 
-    const bool try_candidates = ring_started && candidate_eligible(rp, V, (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) && a.num_top > 0);
+    const bool try_candidates = ring_started && candidate_eligible(rp, a);
     if (o1 > o0) {
         bool ok = build_history(s, hs, c, a.hist_ids + o0, o1 - o0, ostart, (const int32_t *)smem, a.ws_counts, a.ws_counts_cap, (int64_t)o0);
         c.has_hist = ok;
@@ -2103,38 +2164,14 @@ __global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const SampleArgs 
         if (__syncthreads_or(!landed)) { out.status |= ALBIREO_ROW_TIMEOUT; out.token = -1; out.logprob = __uint_as_float(0x7FC00000u); done = true; }   // the same in every thread
     }
     if (!done) {
-        if (threadIdx.x == 0) {
-            GenArgs &ga = s.ga;
-            ga.dbg_topk_ids = a.dbg_topk_ids; ga.exp1 = a.exp1; ga.exp1_stride = a.exp1_stride; ga.out_top_ids = a.out_top_ids;
-            ga.out_top_logprobs = a.out_top_logprobs; ga.step = a.step; ga.flags = a.flags; ga.num_top = a.num_top; ga.dbg_cap = a.dbg_cap;
-        }
+        if (threadIdx.x == 0) fill_general_args(s.ga, a);
         __syncthreads();
         out = general_path_call<DT>(&s, smem, c, rp, b, out.status);
     }
-
-    if (threadIdx.x == 0) {
-        a.out_tokens[b] = out.token;
-        a.out_logprobs[b] = out.logprob;
-        if (a.out_num_kept) a.out_num_kept[b] = out.n_keep;
-        if (a.out_num_topk) a.out_num_topk[b] = out.n_topk;
-        // early feedback (section 5.2): the token goes straight into the next iteration's input ids
-        // and to the output processor's ring, without waiting for a host round trip
-        const bool have_token = !(out.status & ALBIREO_ROW_TIMEOUT);
-        if (a.backfill_ids && have_token) {
-            const int64_t slot = a.backfill_index ? (int64_t)a.backfill_index[b] : (int64_t)b;
-            if (slot >= 0) {
-                if (slot < a.backfill_len) a.backfill_ids[slot] = out.token;
-                else out.status |= ALBIREO_ROW_BAD_PARAM;
-            }
-        }
-        if (a.feedback_ring && have_token) {
-            const int64_t slot = (a.feedback_head + b) % a.feedback_cap;
-            const unsigned long long rec = ((unsigned long long)(a.row_base + (uint32_t)b) << 32) | (uint32_t)out.token;
-            *(volatile unsigned long long *)(a.feedback_ring + slot) = rec;      // one 8-byte store
-        }
-        if (a.out_row_status) a.out_row_status[b] = out.status;
-    }
+    store_row(a, b, out);
 }
+
+#include "cluster_kernel.cuh"
 
 // ------------------------------------------------------------------ the stream alone (measurement aid)
 //
@@ -2303,45 +2340,87 @@ int apply_ext(SampleArgs &a, const albireo_sample_ext_t *ext, int B, int V, cons
     return ALBIREO_OK;
 }
 
-void launch_sample_kernel(int dtype, int B, size_t smem, cudaStream_t st, const SampleArgs &a) {
-    if (a.flags & ALBIREO_FLAG_PROGRAMMATIC_LAUNCH) {
-        // programmatic dependent launch: the kernel may be scheduled before the kernel ahead of it in the
-        // stream has finished; it waits for that kernel itself (griddepcontrol.wait) before it touches memory
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)B); cfg.blockDim = dim3(NT); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = at; cfg.numAttrs = 1;
-        if (dtype == ALBIREO_F32) cudaLaunchKernelEx(&cfg, albireo_sample_kernel<ALBIREO_F32>, a);
-        else if (dtype == ALBIREO_BF16) cudaLaunchKernelEx(&cfg, albireo_sample_kernel<ALBIREO_BF16>, a);
-        else cudaLaunchKernelEx(&cfg, albireo_sample_kernel<ALBIREO_F16>, a);
-        return;
+// The launch shape of a batch: a CTA per row (team 1, ring of nstages), or a cluster of `team` CTAs per row.
+struct LaunchShape { int team, nstages, slice_bytes; size_t smem; };
+
+// Rows are shared by clusters where all their CTAs are on the chip at once, one per SM: then every SM
+// works on the batch and a row's slices stay in shared memory.  (Two CTAs per SM, with half the registers,
+// were 10 % slower on the rows without a top-k and the same on the others.)  Of the sizes that fit, the largest whose slices are
+// still at least 8 KB (one vector per thread): below that the exchange costs more than the slice.
+bool pick_team(LaunchShape &ls, int B, int V, int esize, bool with_history, int num_sms, size_t max_smem) {
+    const long row_bytes = (long)(V / (16 / esize)) * 16;
+    for (int team = MAX_TEAM; team >= 2; team >>= 1) {
+        if (row_bytes / team < 8192 || (long)B * team > (long)num_sms) continue;
+        const long per = ((row_bytes / 16 + team - 1) / team) * 16;
+        const long slice = ((per > SLICE_MIN ? per : (long)SLICE_MIN) + 127) & ~127L;
+        long smem = SLICE_OFF + slice + 16 + (with_history ? 4L * slice_table_words((int)(per / esize)) : 8L * X_ENDS);
+        const long general = GENERAL_BYTES + (with_history ? (long)history_smem_bytes(V) : 0);
+        if (general > smem) smem = general;
+        if (smem > (long)max_smem) continue;
+        ls.team = team; ls.slice_bytes = (int)slice; ls.smem = (size_t)smem; ls.nstages = 0;
+        return true;
     }
-    if (dtype == ALBIREO_F32) albireo_sample_kernel<ALBIREO_F32><<<B, NT, smem, st>>>(a);
-    else if (dtype == ALBIREO_BF16) albireo_sample_kernel<ALBIREO_BF16><<<B, NT, smem, st>>>(a);
-    else albireo_sample_kernel<ALBIREO_F16><<<B, NT, smem, st>>>(a);
+    return false;
+}
+// false: the vocabulary is too large for the on-chip tables
+bool pick_shape(LaunchShape &ls, int B, int V, int esize, bool with_history, bool force_general, int num_sms, size_t max_smem) {
+    if (!force_general && pick_team(ls, B, V, esize, with_history, num_sms, max_smem)) return true;
+    ls.team = 1; ls.slice_bytes = 0;
+    ls.nstages = ring_stages_for(V, with_history, B <= num_sms);
+    ls.smem = smem_bytes_for(V, with_history, ls.nstages);
+    while (ls.smem > max_smem && ls.nstages > 2) ls.smem = smem_bytes_for(V, with_history, --ls.nstages);
+    return ls.smem <= max_smem;
+}
+
+template <int DT>
+cudaError_t launch_sample_kernel_as(int B, const LaunchShape &ls, cudaStream_t st, const SampleArgs &a) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(B * ls.team)); cfg.blockDim = dim3(NT); cfg.dynamicSmemBytes = ls.smem; cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    int n = 0;
+    // programmatic dependent launch: the kernel may be scheduled before the kernel ahead of it in the
+    // stream has finished; it waits for that kernel itself (griddepcontrol.wait) before it touches memory.
+    // Back-to-back calls lose the launch gap between them: 1.6 us per call on the metric workload, 3.7 us
+    // of 10.2 on a single row.
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+    if (ls.team > 1) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = (unsigned)ls.team; at[n].val.clusterDim.y = 1; at[n].val.clusterDim.z = 1;
+        ++n;
+    }
+    cfg.attrs = at; cfg.numAttrs = n;
+    return ls.team > 1 ? cudaLaunchKernelEx(&cfg, albireo_cluster_kernel<DT>, a) : cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT>, a);
+}
+cudaError_t launch_sample_kernel(int dtype, int B, const LaunchShape &ls, cudaStream_t st, SampleArgs &a) {
+    a.nstages = ls.nstages; a.slice_bytes = ls.slice_bytes;
+    if (dtype == ALBIREO_F32) return launch_sample_kernel_as<ALBIREO_F32>(B, ls, st, a);
+    if (dtype == ALBIREO_BF16) return launch_sample_kernel_as<ALBIREO_BF16>(B, ls, st, a);
+    return launch_sample_kernel_as<ALBIREO_F16>(B, ls, st, a);
 }
 // Lets every instantiation use the device's opt-in shared memory; gives the dynamic bytes available
 // to a CTA (the opt-in limit less the largest static use), or 0 with *err set.
 size_t enable_large_smem(int device, cudaError_t *err) {
     int optin = 0;
     cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
-    cudaFuncAttributes f0, f1, f2;
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&f0, albireo_sample_kernel<ALBIREO_F32>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&f1, albireo_sample_kernel<ALBIREO_BF16>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&f2, albireo_sample_kernel<ALBIREO_F16>);
+    const void *kernels[] = {
+        (const void *)albireo_cluster_kernel<ALBIREO_F32>, (const void *)albireo_cluster_kernel<ALBIREO_BF16>, (const void *)albireo_cluster_kernel<ALBIREO_F16>,
+        (const void *)albireo_sample_kernel<ALBIREO_F32>, (const void *)albireo_sample_kernel<ALBIREO_BF16>, (const void *)albireo_sample_kernel<ALBIREO_F16>,
+        (const void *)albireo_stream_only_kernel<ALBIREO_F32>, (const void *)albireo_stream_only_kernel<ALBIREO_BF16>, (const void *)albireo_stream_only_kernel<ALBIREO_F16>};
+    size_t st = 0;
+    for (const void *k : kernels) {
+        cudaFuncAttributes f;
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&f, k);
+        if (e == cudaSuccess && f.sharedSizeBytes > st) st = f.sharedSizeBytes;
+    }
     if (e != cudaSuccess) { *err = e; return 0; }
-    size_t st = f0.sharedSizeBytes > f1.sharedSizeBytes ? f0.sharedSizeBytes : f1.sharedSizeBytes;
-    if (f2.sharedSizeBytes > st) st = f2.sharedSizeBytes;
     if ((size_t)optin <= st) { *err = cudaErrorInvalidValue; return 0; }
     const size_t smem = (size_t)optin - st;
-    e = cudaFuncSetAttribute(albireo_sample_kernel<ALBIREO_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(albireo_sample_kernel<ALBIREO_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(albireo_sample_kernel<ALBIREO_F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(albireo_stream_only_kernel<ALBIREO_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(albireo_stream_only_kernel<ALBIREO_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(albireo_stream_only_kernel<ALBIREO_F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    for (const void *k : kernels)
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    for (int i = 0; i < 3; ++i)      // clusters of 16
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernels[i], cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     *err = e;
     return e == cudaSuccess ? smem : 0;
 }
@@ -2453,14 +2532,11 @@ extern "C" int albireo_sample(albireo_sampler_t *h, const void *logits, int32_t 
     int cur = -1;
     if (cudaGetDevice(&cur) != cudaSuccess || cur != h->device) { cudaGetLastError(); set_err(h, "the handle's device is not current%s", ""); return ALBIREO_EINVAL; }
 
-    a.nstages = ring_stages_for(V, history_ids != nullptr, B <= h->num_sms);
-    size_t smem = smem_bytes_for(V, history_ids != nullptr, a.nstages);
-    while (smem > h->max_smem && a.nstages > 2) smem = smem_bytes_for(V, history_ids != nullptr, --a.nstages);
-    if (smem > h->max_smem) { set_err(h, "vocabulary too large for the on-chip tables%s", ""); return ALBIREO_EUNSUPPORTED; }
+    LaunchShape ls;
+    if (!pick_shape(ls, B, V, (int)esize, history_ids != nullptr, (a.flags & ALBIREO_FLAG_FORCE_GENERAL) != 0, h->num_sms, h->max_smem)) { set_err(h, "vocabulary too large for the on-chip tables%s", ""); return ALBIREO_EUNSUPPORTED; }
     cudaStream_t st = (cudaStream_t)stream;
-    launch_sample_kernel(dtype, B, smem, st, a);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) { set_err(h, "kernel launch failed: %s", cudaGetErrorString(e)); return ALBIREO_ECUDA; }
+    const cudaError_t e = launch_sample_kernel(dtype, B, ls, st, a);
+    if (e != cudaSuccess) { cudaGetLastError(); set_err(h, "kernel launch failed: %s", cudaGetErrorString(e)); return ALBIREO_ECUDA; }
     h->launches += 1;
     return ALBIREO_OK;
 }
@@ -2676,14 +2752,11 @@ extern "C" int albireo_sample_fixed_scratch(const void *logits, int32_t B, int32
     a.ws_counts = d->counts;                       // a device address, from cudaGetSymbolAddress
     a.ws_counts_cap = ALBIREO_FIXED_MAX_HISTORY;
 
-    a.nstages = ring_stages_for(V, history_ids != nullptr, B <= d->num_sms);
-    size_t smem = smem_bytes_for(V, history_ids != nullptr, a.nstages);
-    while (smem > d->max_smem && a.nstages > 2) smem = smem_bytes_for(V, history_ids != nullptr, --a.nstages);
-    if (smem > d->max_smem) return fixed_fail(ALBIREO_EUNSUPPORTED, "vocabulary too large for the on-chip tables%s", "");
+    LaunchShape ls;
+    if (!pick_shape(ls, B, V, (int)esize, history_ids != nullptr, (a.flags & ALBIREO_FLAG_FORCE_GENERAL) != 0, d->num_sms, d->max_smem)) return fixed_fail(ALBIREO_EUNSUPPORTED, "vocabulary too large for the on-chip tables%s", "");
     cudaStream_t st = (cudaStream_t)stream;
-    launch_sample_kernel(dtype, B, smem, st, a);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return fixed_fail(ALBIREO_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e));
+    const cudaError_t e = launch_sample_kernel(dtype, B, ls, st, a);
+    if (e != cudaSuccess) { cudaGetLastError(); return fixed_fail(ALBIREO_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e)); }
     return ALBIREO_OK;
 }
 

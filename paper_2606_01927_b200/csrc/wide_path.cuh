@@ -1,0 +1,688 @@
+// Wide rows: rows whose kept set has no small bound (top-p alone, no cut at all, a min-p that keeps
+// thousands).  Included by albireo_sample.cu.
+//
+// What bounds such a row is instruction issue: every element needs an exponential (its mass), and with
+// no cut a share of a Philox block.  So the row is passed over as few times as the definition allows
+// and each pass does one short fixed sequence per element:
+//   mass    e = exp(z - zmax) summed in fixed point, and, where a cut or a list has to be found, one
+//           32-bit shared-memory add per element into a histogram of masses over bins that are linear
+//           in log2 e (32 per octave);
+//   locate  the window of bins in which the wanted mass (or rank) is reached, from prefix sums; a window
+//           that may hold more than the list takes is split again (one more pass that adds only the
+//           window's elements);
+//   final   the elements above the window are kept for sure: their exact mass, their number, the race.
+//           Those in the window go to an on-chip list, in which the cut is found exactly; the exact
+//           masses check that the histogram had located it (otherwise the row goes to the general path).
+// With no cut the first and the last pass are the same pass.  A row may be shared by the CTAs of a
+// cluster (a Team), each holding a slice; what they exchange is the histogram and a few words.
+
+// ------------------------------------------------------------------ teams
+
+constexpr int MAX_TEAM = 16;
+
+// Words that the CTAs of a row exchange: slot r is written by CTA r, in every CTA or only in CTA 0's copy.
+struct TeamWords {
+    uint32_t kmax[MAX_TEAM], tau[MAX_TEAM], tau_part[MAX_TEAM], nfin[MAX_TEAM], flags[MAX_TEAM], ncand[MAX_TEAM];   // in every CTA
+    u64 S[MAX_TEAM], S_all[MAX_TEAM], M[MAX_TEAM], G[MAX_TEAM];                                                    // in CTA 0's
+    uint32_t n[MAX_TEAM];
+    float z[MAX_TEAM];
+    uint32_t far_cand, far_list;      // CTA 0: entries that the others have put at the far end of its lists
+};
+
+struct ClusterTeam {                  // the CTAs of a thread-block cluster
+    TeamWords *x;
+    int rank, size;
+    __device__ __forceinline__ void sync() const {
+        asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    }
+    template <class P> __device__ __forceinline__ P *at(P *p, int r) const { return cg::this_cluster().map_shared_rank(p, r); }
+};
+
+// ------------------------------------------------------------------ reductions with few instructions
+
+// sum of the warp's values, each below 2^58, in every lane: three 32-bit reductions instead of ten shuffles
+__device__ __forceinline__ u64 warp_total(u64 v) {
+    const uint32_t a = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)v & 0x7FFFFFu), b = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)(v >> 23) & 0x7FFFFFu);
+    const uint32_t c = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)(v >> 46));
+    return (u64)a + ((u64)b << 23) + ((u64)c << 46);
+}
+// the largest G of the warp and its z, in every lane
+__device__ __forceinline__ void warp_best(u64 &G, float &z) {
+    const uint32_t hi = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(G >> 32));
+    const uint32_t lo = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(G >> 32) == hi ? (uint32_t)G : 0u);
+    const uint32_t who = __ballot_sync(0xFFFFFFFFu, (uint32_t)(G >> 32) == hi && (uint32_t)G == lo);
+    z = __shfl_sync(0xFFFFFFFFu, z, __ffs(who) - 1);
+    G = ((u64)hi << 32) | lo;
+}
+// what a pass leaves in each thread, added up: masses, number and race of the kept elements
+struct Partial {
+    u64 M, G;
+    uint32_t n;
+    float z;
+    __device__ __forceinline__ void over_warp() { M = warp_total(M); n = __reduce_add_sync(0xFFFFFFFFu, n); warp_best(G, z); }
+};
+// The block's totals, in every lane of warp 0 (the other warps have handed in theirs).  One barrier.
+__device__ __forceinline__ void block_partial(BlockScratch &s, Partial &p) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    p.over_warp();
+    if (lane == 0) { s.red[wid] = p.M; s.red2[wid] = p.G; s.r32a[wid] = p.n; s.r32b[wid] = __float_as_uint(p.z); }
+    __syncthreads();
+    if (wid == 0) {
+        const bool in = lane < NWARPS;
+        p.M = in ? s.red[lane] : 0ull; p.G = in ? s.red2[lane] : 0ull; p.n = in ? s.r32a[lane] : 0u; p.z = in ? __uint_as_float(s.r32b[lane]) : 0.0f;
+        p.over_warp();
+    }
+}
+
+// ------------------------------------------------------------------ what a CTA reads of its row
+
+// element x of a vector, x not known at compile time
+template <int DT>
+__device__ __forceinline__ float pick_element(const uint4 &q, int x) {
+    constexpr int PV = Elem<DT>::PER_VEC;
+    const uint32_t w = x < PV / 2 ? (x < PV / 4 ? q.x : q.y) : (x < 3 * PV / 4 ? q.z : q.w);
+    return Elem<DT>::get(make_uint4(w, w, w, w), PV == 4 ? 0 : (x & 1));
+}
+
+// A slice of the row that lies in shared memory, its penalised tokens already overwritten with -inf;
+// they and the row's unaligned ends are in a list of (id, score).  Both loops have the same trip count
+// in every lane of a warp (lanes past the end see -inf), so that the callee may use warp collectives,
+// but no block barriers.
+template <int DT>
+struct SmemSlice {
+    typedef Elem<DT> E;
+    int vec_off, nvec, id0;       // where the slice and the list lie in the dynamic shared memory
+    int xid_off, xz_off, nx;
+    __device__ __forceinline__ int first_id() const { return id0; }
+    template <class F> __device__ __forceinline__ void vectors(F &&f) const {
+        extern __shared__ __align__(128) unsigned char smem[];
+        const uint4 *vec = (const uint4 *)(smem + vec_off);
+#pragma unroll 1
+        for (int base = 0; base < nvec; base += NT) {
+            const int v = base + (int)threadIdx.x;
+            f(v < nvec ? vec[v] : VecTest<DT>::fill(), id0 + v * E::PER_VEC);
+        }
+    }
+    template <class F> __device__ __forceinline__ void extras(F &&f) const {
+        extern __shared__ __align__(128) unsigned char smem[];
+        const int *xid = (const int *)(smem + xid_off);
+        const float *xz = (const float *)(smem + xz_off);
+#pragma unroll 1
+        for (int r0 = 0; r0 < nx; r0 += NT) {
+            const int r = r0 + (int)threadIdx.x;
+            f(r < nx ? xid[r] : 0, r < nx ? xz[r] : -INFINITY);
+        }
+    }
+};
+
+// ------------------------------------------------------------------ masses and their order codes
+
+// Code of an element: F = -log2(e) in 1/65536 octaves, rounded; a larger z never has a larger F (every
+// step is one monotone rounding).  Kept with the exponent of the magic number added: code(z = zmax) is
+// F_ZERO.  Beyond 128 octaves the sum leaves the integer range of the mantissa and only keeps the order.
+constexpr uint32_t F_ZERO = 0x4B000000u;               // bits of 2^23
+constexpr int W_SHIFT = 11;                            // 65536 / 2^11 = 32 bins per octave
+constexpr int W_BINS = 1344;                           // 42 octaves
+constexpr int W_PER = 4;                               // bins per thread in the scans (one 16-byte load; the last threads have none)
+constexpr int W_LIST = CAND_CAP;                       // entries of the window's list and of the top-N list
+
+__device__ __forceinline__ float ex2_ftz(float t) { float e; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(t)); return e; }
+__device__ __forceinline__ float log2_mass(float z, float zmax) { return __fmul_rn(__fsub_rn(z, zmax), 1.4426950408889634f); }
+__device__ __forceinline__ uint32_t code_of(float t2) { return __float_as_uint(__fmaf_rn(t2, -65536.0f, 8388608.0f)); }
+// A bin's masses are added up as 12-bit fractions of the bin's octave (at most 2^19 elements: no
+// overflow).  `octave_code` = code >> 16 carries the magic exponent, which turns into the sign bit.
+__device__ __forceinline__ uint32_t mass12(float e, uint32_t octave_code) {
+    const float neg = __uint_as_float(__float_as_uint(e) + (octave_code << 23));
+    return __float_as_uint(2048.0f - neg) - 0x45000000u;
+}
+__device__ __forceinline__ u64 mass_of_bin(uint32_t q, uint32_t octave) { return octave < 52u ? ((u64)q << 20) >> octave : 0ull; }   // 2^-32 units
+// hist[bin] += v if bin < W_BINS, without a branch
+__device__ __forceinline__ void hist_add_if(uint32_t hist_addr, uint32_t bin, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p red.shared.add.u32 [%0], %3;\n\t}"
+                 ::"r"(hist_addr + bin * 4u), "r"(bin), "n"(W_BINS), "r"(v) : "memory");
+}
+
+struct WideSmem {
+    u64 *top;             // W_LIST composites: the top-N list
+    u64 *list;            // W_LIST composites: the window
+    uint32_t *hist;       // W_BINS words
+    u64 *queue;           // 64 entries per warp
+};
+// The front of the dynamic shared memory, whatever the kernel keeps behind it
+// (the candidate list and its select bins lie where the top-N list does).
+constexpr int WIDE_LIST_OFF = COMMON_BYTES, WIDE_HIST_OFF = WIDE_LIST_OFF + W_LIST * 8;
+constexpr int WIDE_QUEUE_OFF = WIDE_HIST_OFF + W_BINS * 4, WIDE_BYTES = WIDE_QUEUE_OFF + NWARPS * 64 * 8;
+static_assert(W_LIST <= NWARPS * 64, "the list's masses lie over the queues");
+constexpr int TEAM_OFF = WIDE_BYTES, SLICE_OFF = (TEAM_OFF + (int)sizeof(TeamWords) + 127) & ~127;
+// (taken from the kernel's own shared array, so that the compiler knows the address space)
+__device__ __forceinline__ WideSmem wide_smem() {
+    extern __shared__ __align__(128) unsigned char smem[];
+    WideSmem w;
+    w.top = (u64 *)smem; w.list = (u64 *)(smem + WIDE_LIST_OFF);
+    w.hist = (uint32_t *)(smem + WIDE_HIST_OFF); w.queue = (u64 *)(smem + WIDE_QUEUE_OFF);
+    return w;
+}
+
+// One pass of masses.  FIRST_LEVEL: every element into its bin (1/32 octave; what lies more than 42
+// octaves below the maximum is in none: 2^19 such elements weigh 1e-7 of it).  INSIDE_WINDOW: only
+// elements with code in [lo, lo + (W_BINS << shift)), into bins of 2^shift.  S: the masses of the
+// elements with z >= zfloor, S_all: of all.
+// Bound by issue (about 16 instructions per element) and, on the first level, by the shared-memory
+// adds (one per element, 3 to 5 bank cycles per warp).
+enum MassMode { SUM_ONLY, FIRST_LEVEL, INSIDE_WINDOW };
+template <int DT, int MODE, bool FLOOR, class SRC>
+__device__ __forceinline__ void mass_pass(const SRC &src, float invT, float zmax, float zfloor, uint32_t lo, int shift, u64 &S_out, u64 &S_all_out) {
+    typedef Elem<DT> E;
+    const uint32_t hist = smem_u32(wide_smem().hist);
+    u64 S = 0, S_all = 0;
+    auto add = [&](float z, float &acc, float &all) {
+        const float t2 = log2_mass(z, zmax);
+        const float e = ex2_ftz(t2);
+        uint32_t f = code_of(t2);
+        if (FLOOR) {
+            all += e;
+            const bool in = z >= zfloor;
+            acc += in ? e : 0.0f;
+            f = in ? f : 0xFFFFFFFFu;
+        } else acc += e;
+        if (MODE == FIRST_LEVEL) hist_add_if(hist, (f >> W_SHIFT) - (F_ZERO >> W_SHIFT), mass12(e, f >> 16));
+        if (MODE == INSIDE_WINDOW) hist_add_if(hist, f >= lo ? (f - lo) >> shift : 0xFFFFFFFFu, mass12(e, f >> 16));
+    };
+    const uint32_t thr = VecTest<DT>::raw_threshold(key_of(zmax - 29.5f), invT);
+    src.vectors([&](const uint4 &q, int) {
+        if (!VecTest<DT>::may_pass(q, thr, invT)) return;          // nothing within 42 octaves of the maximum
+        float acc = 0.0f, all = 0.0f;
+#pragma unroll
+        for (int j = 0; j < E::PER_VEC; ++j) add(__fmul_rn(E::get(q, j), invT), acc, all);
+        S += __float2ull_rn(acc * FX_SCALE);
+        if (FLOOR) S_all += __float2ull_rn(all * FX_SCALE);
+    });
+    src.extras([&](int, float z) {
+        float acc = 0.0f, all = 0.0f;
+        add(z, acc, all);
+        S += __float2ull_rn(acc * FX_SCALE);
+        if (FLOOR) S_all += __float2ull_rn(all * FX_SCALE);
+    });
+    S_out = S; S_all_out = FLOOR ? S_all : S;
+}
+
+// One level of the search: where the running total of the team's histogram (masses, or lower bounds of
+// the element counts) reaches its target, with slack on both sides (targets beyond the total are cut
+// down to it).  On the first level of a search by mass the target is the share `frac` of the histogram's
+// own total, so that what its rounding adds or loses everywhere cancels.
+struct Window {
+    uint32_t lo, hi;      // codes, both inclusive
+    u64 before;           // running total ahead of lo
+    uint32_t most;        // no more elements than this lie in [lo, hi]
+    bool found;
+};
+template <class TEAM>
+__device__ __noinline__ Window find_window(BlockScratch *sp, TEAM tm, bool by_count, uint32_t base, int shift, double frac, u64 target, u64 *total) {
+    BlockScratch &s = *sp;
+    uint32_t *hist = wide_smem().hist;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t q[W_PER] = {0, 0, 0, 0};
+    if ((int)threadIdx.x < W_BINS / W_PER) {
+#pragma unroll 4
+        for (int r = 0; r < tm.size; ++r) {
+            const uint4 h = *((const uint4 *)tm.at(hist, r) + threadIdx.x);
+            q[0] += h.x; q[1] += h.y; q[2] += h.z; q[3] += h.w;
+        }
+    }
+    u64 v[W_PER], local = 0;
+    uint32_t cnt = 0;
+#pragma unroll
+    for (int j = 0; j < W_PER; ++j) {
+        const uint32_t code = base + ((uint32_t)(threadIdx.x * W_PER + j) << shift);
+        v[j] = by_count ? (u64)((q[j] + 4095u) >> 12) : mass_of_bin(q[j], (code - F_ZERO) >> 16);
+        local += v[j];
+        q[j] = (q[j] + 2039u) / 2040u;                   // upper bound of the bin's count (a member adds 2047 or more)
+        cnt += q[j];
+    }
+    u64 inc = local;
+    uint32_t cinc = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const u64 t = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+        const uint32_t tc = __shfl_up_sync(0xFFFFFFFFu, cinc, o);
+        if (lane >= o) { inc += t; cinc += tc; }
+    }
+    if (lane == 31) { s.red[wid] = inc; s.r32a[wid] = cinc; }
+    if (threadIdx.x == 0) { s.found_digit = 0xFFFFFFFFu; s.found_cnt = 0xFFFFFFFFu; }
+    __syncthreads();
+    const u64 wt = lane < NWARPS ? s.red[lane] : 0ull;
+    const uint32_t wc = lane < NWARPS ? s.r32a[lane] : 0u;
+    const u64 tot = warp_total(wt);
+    u64 run = warp_total(lane < wid ? wt : 0ull) + inc - local;
+    uint32_t crun = __reduce_add_sync(0xFFFFFFFFu, lane < wid ? wc : 0u) + cinc - cnt;
+    if (frac > 0.0) { *total = tot; target = (u64)(frac * (double)tot); }
+    // (the rounding of the histogram is far inside 2^-14 of the total)
+    const u64 slack = by_count ? 0ull : (*total >> 14) + 1;
+    u64 t_lo = target > slack ? target - slack : 1, t_hi = target + slack;
+    if (t_hi > tot) t_hi = tot;
+    if (t_lo < 1) t_lo = 1;
+    if (t_lo > t_hi) t_lo = t_hi;
+#pragma unroll
+    for (int j = 0; j < W_PER; ++j) {
+        const u64 nx = run + v[j];
+        if (run < t_lo && t_lo <= nx) { s.found_digit = threadIdx.x * W_PER + j; s.found_above = run; s.list_cnt = crun; }
+        if (run < t_hi && t_hi <= nx) { s.found_cnt = threadIdx.x * W_PER + j; s.cand_cnt = crun + q[j]; }
+        run = nx; crun += q[j];
+    }
+    __syncthreads();
+    const uint32_t a = s.found_digit, b2 = s.found_cnt;
+    Window w;
+    w.found = tot > 0 && a != 0xFFFFFFFFu && b2 != 0xFFFFFFFFu;
+    w.lo = base + (a << shift); w.hi = base + (b2 << shift) + ((1u << shift) - 1u);
+    w.before = s.found_above; w.most = s.cand_cnt - s.list_cnt;
+    __syncthreads();
+    return w;
+}
+// Narrows a window until no more than `cap` elements can be in it (or the codes run out).
+template <int DT, bool FLOOR, class SRC, class TEAM>
+__device__ __noinline__ bool narrow_window(BlockScratch *sp, SRC src, TEAM tm, float invT, float zmax, float zfloor, bool by_count, u64 target,
+                                           u64 total, uint32_t cap, Window *wp) {
+    Window w = *wp;
+    uint32_t *hist = wide_smem().hist;
+#pragma unroll 1
+    for (int it = 0; it < 4 && w.most > cap; ++it) {
+        const uint32_t width = w.hi - w.lo + 1;
+        int shift = 0;
+        while (((width - 1) >> shift) >= (uint32_t)W_BINS) ++shift;
+        tm.sync();                                       // everybody has read the histograms
+        for (int i = threadIdx.x; i < W_BINS; i += NT) hist[i] = 0;
+        __syncthreads();
+        u64 d0, d1;
+        mass_pass<DT, INSIDE_WINDOW, FLOOR>(src, invT, zmax, zfloor, w.lo, shift, d0, d1);
+        tm.sync();
+        const u64 before = w.before;
+        w = find_window(sp, tm, by_count, w.lo, shift, 0.0, target - before, &total);
+        if (!w.found) return false;
+        w.before += before;
+        if (shift == 0) break;
+    }
+    *wp = w;
+    return w.most <= cap;
+}
+
+// ------------------------------------------------------------------ the race
+
+// N blocks of the generator at once share its key schedule; each product is one wide multiplication.
+template <int N>
+__device__ __forceinline__ void philox_blocks(uint64_t seed, uint32_t R, uint64_t step, uint32_t block, uint32_t (&w)[4 * N]) {
+    uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+    uint32_t c0[N], c1[N], c2[N], c3[N];
+#pragma unroll
+    for (int n = 0; n < N; ++n) { c0[n] = block + n; c1[n] = R; c2[n] = (uint32_t)step; c3[n] = (uint32_t)(step >> 32); }
+#pragma unroll
+    for (int i = 0; i < 10; ++i) {
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+            const uint64_t p0 = (uint64_t)c0[n] * 0xD2511F53u, p1 = (uint64_t)c2[n] * 0xCD9E8D57u;
+            c0[n] = (uint32_t)(p1 >> 32) ^ c1[n] ^ k0; c1[n] = (uint32_t)p1;
+            c2[n] = (uint32_t)(p0 >> 32) ^ c3[n] ^ k1; c3[n] = (uint32_t)p0;
+        }
+        k0 += 0x9E3779B9u; k1 += 0xBB67AE85u;
+    }
+#pragma unroll
+    for (int n = 0; n < N; ++n) { w[4 * n] = c0[n]; w[4 * n + 1] = c1[n]; w[4 * n + 2] = c2[n]; w[4 * n + 3] = c3[n]; }
+}
+
+// The best race score of this CTA so far is shared by its threads (order code in s.runmax).  An
+// element can only beat it if E < exp(d - best), and E = -log1p(-v) >= v: so a compare of the uniform
+// v with e * exp(-best) decides almost every element without a logarithm.
+struct Racer {
+    float K;              // exp(-best) with a margin for the rounding of e
+    uint32_t seen;        // order code K was computed from
+    u64 G;                // this thread's best: order code of the score, ~id
+    float z;              // and its z
+    __device__ __forceinline__ void start() { K = 3.0e34f; seen = 0; G = 0; z = 0.0f; }
+    __device__ __forceinline__ void refresh(const uint32_t *best) {
+        const uint32_t now = *(const volatile uint32_t *)best;
+        if (now != seen) { seen = now; K = fminf(1.0001f * ex2_ftz(-unkey(now) * 1.4426950408889634f), 3.0e34f); }
+    }
+    __device__ __forceinline__ void take(uint32_t *best, int i, float z_, float g) {
+        const u64 g64 = ((u64)orderable_f32(g) << 32) | (uint32_t)(~(uint32_t)i);
+        if (g64 > G) {
+            G = g64; z = z_;
+            if ((uint32_t)(g64 >> 32) > *(volatile uint32_t *)best) atomicMax(best, (uint32_t)(g64 >> 32));
+        }
+    }
+};
+__device__ __forceinline__ float unit_above(uint32_t w) { return __uint_as_float((w >> 9) | 0x3F800000u); }      // 1 + (v rounded down)
+__device__ __noinline__ float nle_once(uint32_t w) { return neg_log_exp1_fast(w); }      // (where it is rare: one copy of the code)
+
+// No cut: mass and race of every element in one pass.  OFF: id of a vector's first element modulo 4
+// (the generator's blocks are 4 ids).  About 20 instructions per element, half of them Philox; vectors
+// that could not win with the luckiest word skip it.
+template <int DT, int OFF, class SRC>
+__device__ __forceinline__ void race_all(const SRC &src, uint32_t *best, float invT, float zmax, uint64_t seed, uint32_t R, uint64_t step, Partial &p) {
+    typedef Elem<DT> E;
+    constexpr int PV = E::PER_VEC, NB = PV / 4 + (OFF ? 1 : 0);
+    u64 S = 0;
+    Racer rc;
+    rc.start();
+    src.vectors([&](const uint4 &q, int i0) {
+        float e[PV], acc = 0.0f, top = 0.0f;
+#pragma unroll
+        for (int j = 0; j < PV; ++j) {
+            e[j] = ex2_ftz(log2_mass(__fmul_rn(E::get(q, j), invT), zmax));
+            acc += e[j];
+            top = fmaxf(top, e[j]);
+        }
+        S += __float2ull_rn(acc * FX_SCALE);
+        rc.refresh(best);
+        if (!__any_sync(0xFFFFFFFFu, top * rc.K >= 1.16e-10f)) return;      // v is at least 2^-33
+        uint32_t w[4 * NB];
+        philox_blocks<NB>(seed, R, step, (uint32_t)(i0 >> 2), w);
+        uint32_t hits = 0;
+#pragma unroll
+        for (int j = 0; j < PV; ++j) hits |= (uint32_t)(unit_above(w[OFF + j]) <= __fmaf_rn(e[j], rc.K, 1.0f)) << j;
+        // rare after the first vectors: the exact score, one element per lane at a time, the bound renewed in between
+        while (__any_sync(0xFFFFFFFFu, hits != 0)) {
+            if (hits) {
+                const int x = __ffs(hits) - 1;
+                hits &= hits - 1;
+                uint32_t wx = w[OFF];
+#pragma unroll
+                for (int j = 1; j < PV; ++j) wx = x == j ? w[OFF + j] : wx;
+                const float z = __fmul_rn(pick_element<DT>(q, x), invT), d = __fsub_rn(z, zmax);
+                if (d > -3.0e38f && unit_above(wx) <= __fmaf_rn(ex2_ftz(d * 1.4426950408889634f), rc.K, 1.0f)) rc.take(best, i0 + x, z, d + nle_once(wx));
+            }
+            __syncwarp();
+            rc.refresh(best);
+        }
+    });
+    src.extras([&](int i, float z) {
+        const float d = __fsub_rn(z, zmax);
+        if (d > -3.0e38f) {
+            S += __float2ull_rn(ex2_ftz(log2_mass(z, zmax)) * FX_SCALE);
+            rc.take(best, i, z, d + race_nle(seed, R, step, nullptr, i));
+        }
+    });
+    p.M = S; p.n = 0; p.G = rc.G; p.z = rc.z;
+}
+
+struct FinalArgs {
+    float invT, zmax, zfloor;
+    uint32_t sure, win_hi, top_hi;       // codes: below `sure` kept; [sure, win_hi] to the list; <= top_hi to the top-N list
+    uint32_t vec_thr;                    // raw threshold of the vector test
+    uint64_t seed, step;
+    uint32_t R;
+    const float *exp1_row;
+};
+
+// Mass, number and race of the elements kept for sure, and the lists.  Kept elements are scattered over
+// the lanes, and the race term is long: each warp collects them in a queue and works off 32 at a time.
+template <int DT, class SRC>
+__device__ __forceinline__ void final_pass(const SRC &src, BlockScratch &s, const FinalArgs &fa, Partial &p) {
+    typedef Elem<DT> E;
+    const WideSmem ws = wide_smem();
+    const int lane = threadIdx.x & 31;
+    u64 *queue = ws.queue + (threadIdx.x >> 5) * 64;
+    int qn = 0;                                          // the same in every lane
+    u64 S = 0;
+    uint32_t n = 0;
+    Racer rc;
+    rc.start();
+    auto work = [&](int keep) {                          // works the queue off until no more than `keep` are left
+#pragma unroll 1
+        while (qn > keep) {
+            const int cnt = qn < 32 ? qn : 32;
+            qn -= cnt;
+            __syncwarp();
+            rc.refresh(&s.runmax);
+            bool may = false;
+            int i = 0; float z = 0.0f, d = 0.0f;
+            uint32_t w = 0;
+            if (lane < cnt) {
+                const u64 en = queue[qn + lane];
+                i = (int)(uint32_t)en; z = __uint_as_float((uint32_t)(en >> 32));
+                d = __fsub_rn(z, fa.zmax);
+                may = true;
+                if (!fa.exp1_row) {
+                    w = race_word(fa.seed, fa.R, fa.step, i);
+                    may = unit_above(w) <= __fmaf_rn(ex2_ftz(d * 1.4426950408889634f), rc.K, 1.0f);
+                }
+            }
+            if (may) rc.take(&s.runmax, i, z, d + (fa.exp1_row ? -logf(__ldg(fa.exp1_row + i)) : nle_once(w)));
+            __syncwarp();
+        }
+    };
+    auto see = [&](int i, float z) {                     // called by whole warps; z = -inf: nothing
+        const float t2 = log2_mass(z, fa.zmax);
+        const uint32_t f = code_of(t2);
+        const bool alive = z >= fa.zfloor;
+        const bool sure = alive && f < fa.sure;
+        if (sure) { S += __float2ull_rn(ex2_ftz(t2) * FX_SCALE); ++n; }
+        if (alive && f >= fa.sure && f <= fa.win_hi) {
+            const uint32_t slot = atomicAdd(&s.list_cnt, 1u);
+            if (slot < (uint32_t)W_LIST) ws.list[slot] = comp_of(key_of(z), i);
+        }
+        if (alive && f <= fa.top_hi) {
+            const uint32_t slot = atomicAdd(&s.cand_cnt, 1u);
+            if (slot < (uint32_t)W_LIST) ws.top[slot] = comp_of(key_of(z), i);
+        }
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, sure);
+        if (sure) queue[qn + __popc(m & ((1u << lane) - 1u))] = ((u64)__float_as_uint(z) << 32) | (uint32_t)i;
+        qn += __popc(m);
+        if (qn >= 32) work(31);
+    };
+    src.vectors([&](const uint4 &q, int i0) {
+        uint32_t bits = VecTest<DT>::may_pass(q, fa.vec_thr, fa.invT) ? VecTest<DT>::elem_bits(q, fa.vec_thr, fa.invT) : 0u;
+        while (__any_sync(0xFFFFFFFFu, bits != 0)) {     // one element per lane at a time
+            const int x = __ffs(bits | 0x80000000u) - 1;
+            see(i0 + x, bits ? __fmul_rn(pick_element<DT>(q, x), fa.invT) : -INFINITY);
+            bits &= bits - 1u;
+        }
+    });
+    src.extras([&](int i, float z) { see(i, z); });
+    work(0);
+    p.M = S; p.n = n; p.G = rc.G; p.z = rc.z;
+}
+
+// ------------------------------------------------------------------ one wide row
+
+constexpr uint32_t ROW_NOT_DONE = 0x80000000u;      // internal status bit: the general path has to take the row
+
+// CTA 0: moves the entries that the others put at the far end of `buf` behind its own n0; returns the number of all.
+__device__ __forceinline__ int close_gap(u64 *buf, int cap, int n0, int nfar) {
+    if (nfar == 0) return n0;
+    u64 keep[W_LIST / NT];
+#pragma unroll
+    for (int q = 0; q < W_LIST / NT; ++q) { const int j = threadIdx.x + q * NT; keep[q] = j < nfar ? buf[cap - 1 - j] : 0ull; }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < W_LIST / NT; ++q) { const int j = threadIdx.x + q * NT; if (j < nfar && n0 + j < cap) buf[n0 + j] = keep[q]; }
+    __syncthreads();
+    return n0 + nfar;
+}
+
+// The row's kept set, token and log-probability; the result is CTA 0's, in its warp 0.  `kmax`, `n_fin`:
+// the row's largest order key and its number of finite scores (the same in every CTA).
+template <int DT, class SRC, class TEAM>
+__device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, const TEAM &tm, const RowParams &rp, float invT,
+                                           uint32_t kmax, uint32_t n_fin, int b, uint32_t status) {
+    const WideSmem ws = wide_smem();
+    const int lane = threadIdx.x & 31;
+    RowOut out;
+    out.token = 0; out.logprob = 0.0f; out.n_keep = 0; out.n_topk = (int32_t)n_fin; out.status = status | ALBIREO_ROW_GENERAL_PATH;
+    const float zmax = unkey(kmax);
+    const bool full = (s.ga.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) != 0, want_list = s.ga.num_top > 0;
+    const bool topp = rp.top_p < 1.0f, minp = rp.min_p > 0.0f;
+    const float *exp1_row = s.ga.exp1 ? s.ga.exp1 + (int64_t)b * s.ga.exp1_stride : nullptr;
+    const uint32_t kfloor = minp ? minp_key(zmax, rp.ln_min_p) : KEY_MIN_FINITE;
+    if (kfloor > kmax || (minp && full && want_list)) { out.status |= ROW_NOT_DONE; return out; }
+    const float zfloor = unkey(kfloor);
+
+    if (threadIdx.x == 0) { s.runmax = 0; tm.x->far_cand = 0; tm.x->far_list = 0; }
+    const bool need_hist = topp || want_list || (full && minp);
+    Window win, top;
+    win.lo = win.hi = top.lo = top.hi = 0;
+    if (need_hist) {
+        for (int i = threadIdx.x; i < W_BINS; i += NT) ws.hist[i] = 0;
+        __syncthreads();
+        u64 S, S_all;
+        if (minp) mass_pass<DT, FIRST_LEVEL, true>(src, invT, zmax, zfloor, F_ZERO, W_SHIFT, S, S_all);
+        else mass_pass<DT, FIRST_LEVEL, false>(src, invT, zmax, zfloor, F_ZERO, W_SHIFT, S, S_all);
+        S = warp_total(S);
+        S_all = minp ? warp_total(S_all) : S;
+        if (lane == 0) { s.red[threadIdx.x >> 5] = S; s.red2[threadIdx.x >> 5] = S_all; }
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            S = warp_total(lane < NWARPS ? s.red[lane] : 0ull);
+            S_all = warp_total(lane < NWARPS ? s.red2[lane] : 0ull);
+            if (lane == 0) { *tm.at(&tm.x->S[tm.rank], 0) = S; *tm.at(&tm.x->S_all[tm.rank], 0) = S_all; }
+        }
+        tm.sync();
+        bool ok = true;
+        u64 total = 0;
+        const u64 want = (u64)(s.ga.num_top < (int32_t)n_fin ? s.ga.num_top : (int32_t)n_fin);
+        const bool all_listed = want_list && n_fin <= (uint32_t)(W_LIST / 2);
+        if (want_list) {
+            if (all_listed) top.hi = 0xFFFFFFFEu;
+            else {
+                top = find_window(&s, tm, true, F_ZERO, W_SHIFT, 0.0, want, &total);
+                ok = top.found;
+            }
+        }
+        const double share = fmax((double)rp.top_p, 1e-12);
+        if (topp && ok) {
+            win = find_window(&s, tm, false, F_ZERO, W_SHIFT, share, 0ull, &total);
+            ok = win.found;
+        }
+        const u64 target = (u64)(share * (double)total);
+        if (topp && ok && win.most > (uint32_t)W_LIST)
+            ok = minp ? narrow_window<DT, true>(&s, src, tm, invT, zmax, zfloor, false, target, total, W_LIST, &win)
+                      : narrow_window<DT, false>(&s, src, tm, invT, zmax, zfloor, false, target, total, W_LIST, &win);
+        // (ahead of the list's last bin there are fewer than 2 num_top + 1 elements)
+        const uint32_t list_cap = (uint32_t)(W_LIST - 2 * ALBIREO_MAX_NUM_TOP - 32);
+        if (want_list && ok && !all_listed && top.most > list_cap)
+            ok = minp ? narrow_window<DT, true>(&s, src, tm, invT, zmax, zfloor, true, want, 0, list_cap, &top)
+                      : narrow_window<DT, false>(&s, src, tm, invT, zmax, zfloor, true, want, 0, list_cap, &top);
+        if (!ok) { tm.sync(); out.status |= ROW_NOT_DONE; return out; }          // (the same in every CTA)
+    }
+    if (threadIdx.x == 0) { s.list_cnt = 0; s.cand_cnt = 0; }
+    __syncthreads();
+
+    Partial p;
+    if (!topp && !minp && !want_list && !exp1_row) {
+        switch (src.first_id() & 3) {
+            case 0: race_all<DT, 0>(src, &s.runmax, invT, zmax, rp.seed, rp.R, s.ga.step, p); break;
+            case 1: race_all<DT, 1>(src, &s.runmax, invT, zmax, rp.seed, rp.R, s.ga.step, p); break;
+            case 2: race_all<DT, 2>(src, &s.runmax, invT, zmax, rp.seed, rp.R, s.ga.step, p); break;
+            default: race_all<DT, 3>(src, &s.runmax, invT, zmax, rp.seed, rp.R, s.ga.step, p); break;
+        }
+    } else {
+        FinalArgs fa;
+        fa.invT = invT; fa.zmax = zmax; fa.zfloor = zfloor;
+        fa.sure = topp ? win.lo : 0xFFFFFFFFu;
+        fa.win_hi = topp ? win.hi : 0u;
+        fa.top_hi = want_list ? top.hi : 0u;
+        fa.seed = rp.seed; fa.step = s.ga.step; fa.R = rp.R; fa.exp1_row = exp1_row;
+        // the vector test lets through everything with a code up to the largest that matters
+        uint32_t key = kfloor;
+        const uint32_t deepest = fa.win_hi > fa.top_hi ? fa.win_hi : fa.top_hi;
+        if (fa.sure != 0xFFFFFFFFu && deepest < F_ZERO + (128u << 16)) {
+            const float zlow = zmax - ((float)(deepest - F_ZERO + 2) * (0.6931472f / 65536.0f) * 1.00001f + 1e-6f * fabsf(zmax));
+            const uint32_t k2 = key_of(zlow);
+            key = k2 > key ? k2 : key;
+        }
+        fa.vec_thr = VecTest<DT>::raw_threshold(key, invT);
+        final_pass<DT>(src, s, fa, p);
+    }
+    block_partial(s, p);                                 // (its barrier also ends the appends)
+    const int n_list = (int)s.list_cnt, n_top = (int)s.cand_cnt;
+    if (threadIdx.x == 0) {
+        const int r = tm.rank;
+        *tm.at(&tm.x->M[r], 0) = p.M; *tm.at(&tm.x->n[r], 0) = p.n; *tm.at(&tm.x->G[r], 0) = p.G; *tm.at(&tm.x->z[r], 0) = p.z;
+    }
+    if (tm.size > 1 && tm.rank != 0 && (topp || want_list)) {
+        // the lists' entries go to the far ends of CTA 0's lists (each list's sum is within its capacity)
+        if (threadIdx.x == 32) {
+            s.found_digit = n_list ? atomicAdd(tm.at(&tm.x->far_list, 0), (uint32_t)n_list) : 0u;
+            s.found_cnt = n_top ? atomicAdd(tm.at(&tm.x->far_cand, 0), (uint32_t)n_top) : 0u;
+        }
+        __syncthreads();
+        const int at_list = W_LIST - 1 - (int)s.found_digit, at_top = W_LIST - 1 - (int)s.found_cnt;
+        u64 *list0 = tm.at(ws.list, 0), *top0 = tm.at(ws.top, 0);
+        for (int j = threadIdx.x; j < n_list; j += NT) if (at_list - j >= 0) list0[at_list - j] = ws.list[j];
+        for (int j = threadIdx.x; j < n_top; j += NT) if (at_top - j >= 0) top0[at_top - j] = ws.top[j];
+    }
+    tm.sync();
+    if (tm.rank != 0) return out;
+
+    // CTA 0 has everything
+    const TeamWords &x = *tm.x;
+    const bool in = lane < tm.size;
+    p.M = in ? x.M[lane] : 0ull; p.n = in ? x.n[lane] : 0u; p.G = in ? x.G[lane] : 0ull; p.z = in ? x.z[lane] : 0.0f;
+    p.over_warp();
+    u64 S = 0, S_all = p.M;
+    if (need_hist) { S = warp_total(in ? x.S[lane] : 0ull); S_all = warp_total(in ? x.S_all[lane] : 0ull); }
+    else if (!minp) p.n = n_fin;
+    if (topp) {
+        const double t = ceil((double)rp.top_p * (double)S);
+        u64 target = t <= 1.0 ? 1ull : (u64)t;
+        if (target > S) target = S;
+        if (target < 1) target = 1;
+        const int L = close_gap(ws.list, W_LIST, n_list, (int)x.far_list);
+        if (p.M >= target || L < 1 || L > W_LIST) { out.status |= ROW_NOT_DONE; return out; }
+        // Every entry counts the mass ahead of it in the order (masses over the queues, done with by now):
+        // it is kept if that, with the mass kept for sure, is short of the target.
+        u64 *mass = ws.queue;
+        for (int j = threadIdx.x; j < L; j += NT) mass[j] = __float2ull_rn(ex2_ftz(log2_mass(unkey((uint32_t)(ws.list[j] >> 32)), zmax)) * FX_SCALE);
+        __syncthreads();
+        Partial k;
+        k.M = 0; k.n = 0; k.G = 0; k.z = 0.0f;
+        u64 reach = 0;
+#pragma unroll 1
+        for (int j = threadIdx.x; j < L; j += NT) {
+            const u64 C = ws.list[j], own = mass[j];
+            u64 ahead = p.M;
+#pragma unroll 4
+            for (int q = 0; q < L; ++q) ahead += ws.list[q] > C ? mass[q] : 0ull;
+            reach = ahead + own > reach ? ahead + own : reach;
+            if (ahead < target) {
+                k.M += own; ++k.n;
+                const float zq = unkey((uint32_t)(C >> 32));
+                const float g = __fsub_rn(zq, zmax) + race_nle(rp.seed, rp.R, s.ga.step, exp1_row, comp_idx(C));
+                const u64 gq = ((u64)orderable_f32(g) << 32) | (uint32_t)C;
+                if (gq > k.G) { k.G = gq; k.z = zq; }
+            }
+        }
+        // (short of the target by no more than the rounding of the sums: the whole list stays)
+        if (!__syncthreads_or(reach + (1ull << 18) >= target)) { out.status |= ROW_NOT_DONE; return out; }
+        block_partial(s, k);
+        p.M += k.M; p.n += k.n;
+        if (k.G > p.G) { p.G = k.G; p.z = k.z; }
+    }
+    double lnS = 0.0;
+    if (threadIdx.x < 32) {
+        const u64 S_ref = full ? S_all : p.M;
+        lnS = log((double)S_ref) - LN2_40;
+        const int tok = comp_idx(p.G);
+        out.token = tok < 0 ? 0 : tok;                  // (NaN logits: any id in range)
+        out.n_keep = (int32_t)p.n;
+        out.logprob = (p.n == 1 && !full) ? 0.0f : (float)(((double)p.z - (double)zmax) - lnS);
+    }
+    if (want_list) {
+        if (threadIdx.x == 0) { s.bcast[0] = (u64)__double_as_longlong(lnS); s.found_cnt = p.n; }
+        const int n_all = close_gap(ws.top, W_LIST, n_top, (int)x.far_cand);
+        __syncthreads();
+        const double lnS_all = __longlong_as_double((long long)s.bcast[0]);
+        const uint32_t members = full ? n_fin : s.found_cnt;
+#pragma unroll 1
+        for (int j = threadIdx.x; j < n_all; j += NT) {
+            const u64 C = ws.top[j];
+            uint32_t rank = 0;
+#pragma unroll 4
+            for (int q = 0; q < n_all; ++q) rank += ws.top[q] > C;
+            if (rank < (uint32_t)s.ga.num_top && rank < members) {
+                const int64_t o = (int64_t)b * s.ga.num_top + rank;
+                s.ga.out_top_ids[o] = comp_idx(C);
+                s.ga.out_top_logprobs[o] = (members == 1 && !full) ? 0.0f : (float)(((double)unkey((uint32_t)(C >> 32)) - (double)zmax) - lnS_all);
+            }
+        }
+    }
+    return out;
+}

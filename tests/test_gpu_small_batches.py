@@ -1,0 +1,110 @@
+"""Parity of the kernel that shares a row between the CTAs of a cluster (batches of up to 74 rows on a
+148-SM device), at the batch sizes where the number of CTAs per row changes and at row lengths where
+slices, tables and lists have their edges."""
+import os
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import albireo_oracle as O
+from paper_2606_01927_b200 import workloads as W
+
+from parity import compare, compare_top_lists, to_host
+
+pytestmark = pytest.mark.gpu
+
+DBG_CAP = 128
+_CORES = len(os.sched_getaffinity(0))
+
+
+@pytest.fixture(scope="module")
+def binding():
+    from paper_2606_01927_b200 import binding as Bd
+    return Bd
+
+
+@pytest.fixture(scope="module")
+def sampler(binding):
+    s = binding.Sampler(max_rows=128, max_vocab=160000, max_history_total=1 << 21)
+    yield s
+    s.close()
+
+
+def check(binding, sampler, w, flags=0, **kw):
+    ref = O.sample(w, threads=_CORES, topk_cap=DBG_CAP)
+    t = binding.workload_tensors(w, sampler.device)
+    out = sampler.albireo_sample(t.pop("logits"), **t, row_base=w.row_base, num_top=w.num_top, want_counts=True,
+                                 dbg_cap=DBG_CAP, want_status=True, flags=flags, **kw)
+    torch.cuda.synchronize()
+    g = to_host(out)
+    rep = compare(w, g, ref, dbg_cap=DBG_CAP)
+    assert rep.ok() and not rep.excused, (rep.summary(), rep.failures[:3], rep.excused[:3])
+    bad = compare_top_lists(w, g, ref)
+    assert not bad, bad[:3]
+    return g, ref
+
+
+# rows per batch around 148 / 16, 148 / 8, 148 / 4 and 148 / 2; lengths with 0 to 14 unaligned ends, one
+# vector more or less than a slice boundary, and slices that end up empty
+@pytest.mark.parametrize("dtype", [W.F32, W.BF16, W.F16])
+@pytest.mark.parametrize("B,V", [(1, 65536), (9, 65537), (10, 65543), (18, 32775), (19, 16391), (37, 33001), (38, 16384),
+                                 (74, 8191 * 2), (75, 16384), (3, 131073 + 8)])
+def test_mixed_requests_at_the_edges(binding, sampler, B, V, dtype):
+    base = W.random_small(1000 + B, B=B, V=V, dtype=W.F32 if dtype == W.F16 else dtype)
+    w = W.as_f16(base) if dtype == W.F16 else base
+    w.num_top = 5
+    check(binding, sampler, w)
+
+
+@pytest.mark.parametrize("dtype", [W.F32, W.BF16])
+@pytest.mark.parametrize("kind", ["topk", "topk_wide", "minp_wide", "topp", "topp_one", "none", "flat"])
+def test_rows_without_histories(binding, sampler, dtype, kind):
+    """No tables behind the slices; rows off the 16-byte grid, so that CTA 0 lists their ends; rows of
+    ties, whose window of the top-p cut has to be split down to single codes."""
+    B, V = 23, 33271
+    rng = np.random.default_rng(7)
+    x = (rng.standard_normal((B, V)) * 2).astype(np.float32)
+    if kind == "flat":
+        x = np.round(x).astype(np.float32)
+        x[0] = 1.5
+    par = {"topk": dict(top_k=np.full(B, 40, np.int32)),
+           "topk_wide": dict(top_k=np.full(B, 250, np.int32), top_p=np.full(B, 0.9, np.float32)),
+           "minp_wide": dict(min_p=np.full(B, 0.004, np.float32), top_p=np.full(B, 0.9, np.float32)),
+           "topp": dict(top_p=np.linspace(0.05, 0.999, B).astype(np.float32)),
+           "topp_one": dict(top_p=np.zeros(B, np.float32)),
+           "none": dict(), "flat": dict(top_p=np.full(B, 0.7, np.float32))}[kind]
+    w = W.Workload(kind, B, V, dtype, x if dtype == W.F32 else W.f32_to_bf16_bits(x),
+                   temperature=np.full(B, 0.9, np.float32), seeds=np.arange(B, dtype=np.uint64), **par)
+    w.num_top = 0 if kind == "none" else 7
+    if kind == "flat":
+        w.num_top = 0
+    check(binding, sampler, w)
+
+
+def test_a_slice_with_more_distinct_history_ids_than_it_lists(binding, sampler):
+    """Ids packed into the head of the vocabulary: one slice has more of them than its list holds (that row
+    goes to one CTA), another row just fits, a third repeats the row's unaligned ends."""
+    B, V = 4, 120001
+    rng = np.random.default_rng(9)
+    x = (rng.standard_normal((B, V)) * 2).astype(np.float32)
+    rows = [rng.permutation(4000)[:1500], rng.permutation(3500)[:1008], np.array([0, 1, V - 1, V - 1, V - 2, 5, -1, V]), rng.integers(0, V, 9000)]
+    off = np.cumsum([0] + [len(r) for r in rows]).astype(np.int32)
+    w = W.Workload("dense", B, V, W.BF16, W.f32_to_bf16_bits(x), temperature=np.ones(B, np.float32),
+                   top_k=np.array([50, 50, 50, 0], np.int32), top_p=np.full(B, 0.9, np.float32),
+                   repetition_penalty=np.full(B, 1.3, np.float32), presence_penalty=np.full(B, 0.4, np.float32),
+                   frequency_penalty=np.full(B, 0.2, np.float32), history_ids=np.concatenate(rows).astype(np.int32),
+                   history_offsets=off, seeds=np.arange(B, dtype=np.uint64))
+    check(binding, sampler, w)
+
+
+@pytest.mark.parametrize("cut", ["topk", "greedy", "topp", "none"])
+def test_full_vocabulary_list(binding, sampler, cut):
+    w = W.random_small(1100, B=12, V=40003, dtype=W.BF16)
+    w.top_k[:] = 3 if cut == "topk" else 0
+    w.top_p[:] = 0.6 if cut == "topp" else 1.0
+    w.min_p[:] = 0.0
+    w.temperature[:] = 0.0 if cut == "greedy" else 0.8
+    w.logprob_full_vocab = True
+    w.num_top = 128
+    check(binding, sampler, w, flags=binding.FLAG_LOGPROB_FULL_VOCAB)
