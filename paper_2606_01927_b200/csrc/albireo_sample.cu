@@ -1427,7 +1427,8 @@ __device__ __forceinline__ void cand_append_one(BlockScratch &s, const CandSmem 
 // sorted position.  Step 2 (warp 0): the cuts as prefix operations and the argmax of the race.
 // `full_fx` != 0: the log-probabilities are relative to that mass (the whole row's) instead of the kept set's.
 // The top-N list is the head of the first `list_len` candidates (0: of the kept set).
-__device__ void final_stage(BlockScratch &s, const CandSmem &cs, int n, int L6, float zmax, bool has_minp,
+template <bool EXTRA>
+__device__ __forceinline__ void final_stage(BlockScratch &s, const CandSmem &cs, int n, int L6, float zmax, bool has_minp,
                             const RowParams &rp, const SampleArgs &a, int b, RowOut &out, u64 full_fx, int list_len) {
     const int lane = threadIdx.x & 31;
     // `parts` threads share one candidate's comparisons; the threads after them (from the next warp
@@ -1451,7 +1452,7 @@ __device__ void final_stage(BlockScratch &s, const CandSmem &cs, int n, int L6, 
         const int t = dense_ok ? (int)threadIdx.x - dstart : (part == 0 ? j : -1);
         if (t >= 0 && t < n) {
             const u64 Ct = cs.cand[t];
-            nle[t] = a.exp1 ? -logf(__ldg(a.exp1 + (int64_t)b * a.exp1_stride + comp_idx(Ct)))
+            nle[t] = EXTRA && a.exp1 ? -logf(__ldg(a.exp1 + (int64_t)b * a.exp1_stride + comp_idx(Ct)))
                             : neg_log_exp1_fast(race_word(rp.seed, rp.R, a.step, comp_idx(Ct)));
             mass[t] = mass_gen(__fsub_rn(unkey((uint32_t)(Ct >> 32)), zmax));
         }
@@ -1470,7 +1471,7 @@ __device__ void final_stage(BlockScratch &s, const CandSmem &cs, int n, int L6, 
     // min-p keeps a prefix of the order, at least one element (the barrier also publishes step 1)
     int L7 = __syncthreads_count(in7);
     if (L7 < 1) L7 = 1;
-    if (a.dbg_topk_ids && L6 <= a.dbg_cap && (int)threadIdx.x < L6 && (rp.greedy || (rp.top_k >= 1 && rp.top_k < a.V)))
+    if (EXTRA && a.dbg_topk_ids && L6 <= a.dbg_cap && (int)threadIdx.x < L6 && (rp.greedy || (rp.top_k >= 1 && rp.top_k < a.V)))
         a.dbg_topk_ids[(int64_t)b * a.dbg_cap + threadIdx.x] = comp_idx(cs.sorted[threadIdx.x]);
     if (threadIdx.x >= 32) return;
 
@@ -1666,23 +1667,82 @@ __device__ __forceinline__ bool wide_eligible(const RowParams &rp, const SampleA
     return !(a.flags & ALBIREO_FLAG_FORCE_GENERAL) && !rp.greedy && !(rp.top_k >= 1 && rp.top_k < a.V);
 }
 
+#include "wide_path.cuh"
+
+// Sets the passes of one CTA over a row from global memory up (thread 0; a barrier follows): the row's
+// block in shared memory, and the ring's barriers.
+template <int DT>
+__device__ __forceinline__ void passes_begin(BlockScratch &s, const RowCtx &c, int vps, int nstages) {
+    RowShared &r = row_shared();
+    r.c = c; r.vps = vps;
+    const uintptr_t addr = (uintptr_t)c.row;
+    int head = (int)(((16u - (uint32_t)(addr & 15u)) & 15u) / Elem<DT>::SIZE);
+    if (head > c.V) head = c.V;
+    r.head = head; r.nvec = (c.V - head) / Elem<DT>::PER_VEC;
+    r.vp = (const uint4 *)((const char *)c.row + (size_t)head * Elem<DT>::SIZE);
+    r.nst = min(WIDE_MAX_STAGES, (COMMON_BYTES + nstages * STAGE_BYTES - WIDE_RING_OFF) / WIDE_TILE_BYTES);
+#pragma unroll 1
+    for (int q = 0; q < r.nst; ++q) { mbar_init(&r.bar[q], 1); r.done[q] = 0; }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    r.tiles = 0; r.timeout = 0; s.mm_max = 0; s.list_cnt = 0;
+}
+// The row's largest order key (s.mm_max) and the number of its finite scores (s.list_cnt), after passes_begin.
+template <int DT>
+__device__ __noinline__ void max_and_count(BlockScratch *sp) {
+    BlockScratch &s = *sp;
+    const RingSlice<DT> src;
+    const float invT = row_shared().c.invT;
+    uint32_t kbest = 0, nfin = 0;
+    src.vectors([&](const uint4 &q, int) {
+        const uint32_t k = VecTest<DT>::vmax_key(q, invT);
+        kbest = k > kbest ? k : kbest;
+        nfin += (uint32_t)Elem<DT>::PER_VEC - VecTest<DT>::count_neginf(q);
+    });
+    src.extras([&](int, float z) {
+        const uint32_t k = key_of(z);
+        kbest = k > kbest ? k : kbest;
+        nfin += (k >= KEY_MIN_FINITE && k < KEY_POS_INF);
+    });
+    kbest = __reduce_max_sync(0xFFFFFFFFu, kbest);
+    nfin = __reduce_add_sync(0xFFFFFFFFu, nfin);
+    if ((threadIdx.x & 31) == 0) { atomicMax(&s.mm_max, kbest); atomicAdd(&s.list_cnt, nfin); }
+    __syncthreads();
+}
+// The mass of every finite score of the row (s.bcast[0]) and their number (s.bcast[1]), after passes_begin.
+template <int DT>
+__device__ __noinline__ void whole_row_totals(BlockScratch *sp, float zmax) {
+    BlockScratch &s = *sp;
+    max_and_count<DT>(sp);
+    u64 S, S_all;
+    mass_pass<DT, SUM_ONLY, false>(RingSlice<DT>(), row_shared().c.invT, zmax, 0.0f, 0u, 0, S, S_all);
+    S = block_sum_u64(s, S);
+    if (threadIdx.x == 0) {
+        RowShared &r = row_shared();
+        s.bcast[0] = S; s.bcast[1] = s.list_cnt;
+        if (r.timeout) s.timeout = 1u;
+        for (int q = 0; q < r.nst; ++q) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(&r.bar[q])) : "memory");
+    }
+    __syncthreads();
+}
+
 // From the candidate list cand[0..n) (every element of the row with key >= tau_key) to the result.
 // `full_fx` != 0: the mass of the whole row, which the log-probabilities are relative to.  `count_finite`
 // is called, by every thread, only where the number of finite scores is asked for and not known.
-template <class F>
+// EXTRA: see albireo_sample_kernel.
+template <bool EXTRA, class F>
 __device__ __forceinline__ bool candidate_finish(BlockScratch &s, const CandSmem &cs, int n, uint32_t tau_key, uint32_t kmax, const RowParams &rp,
                                                  const SampleArgs &a, int b, RowOut &out, u64 full_fx, F &&count_finite) {
     const int V = a.V;
-    const bool full_list = (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) && a.num_top > 0;
+    const bool full_list = EXTRA && (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) && a.num_top > 0;
     const int k = rp.greedy ? 1 : rp.top_k;
     const bool has_topk = rp.greedy || (k >= 1 && k < V);
     const bool has_minp = !rp.greedy && rp.min_p > 0.0f;
-    const bool stream_minp = has_minp && !full_list && !(has_topk && a.dbg_topk_ids != nullptr);
+    const bool stream_minp = has_minp && !full_list && !(EXTRA && has_topk && a.dbg_topk_ids != nullptr);
     const int k_list = full_list ? max(k, a.num_top) : k;      // the list holds at least this many (or all there are)
     bool topk_exact_known = true;      // is min(k, #finite) known without counting?
     // keep-ties mode: the top-k stage keeps every score not below the k-th largest, i.e. exactly the
     // candidates that are left once the list is cut at the k-th largest key
-    const bool keep_ties = has_topk && !rp.greedy && (a.flags & ALBIREO_FLAG_TOPK_KEEP_TIES);
+    const bool keep_ties = EXTRA && has_topk && !rp.greedy && (a.flags & ALBIREO_FLAG_TOPK_KEEP_TIES);
     if (has_topk) {
         if (n > SORT_MAX || n > 2 * k_list + 96 || (keep_ties && n > k)) {
             uint32_t t = cand_select_exact(s, cs, n, k_list, tau_key, kmax);
@@ -1697,33 +1757,33 @@ __device__ __forceinline__ bool candidate_finish(BlockScratch &s, const CandSmem
 
     const int L6 = has_topk ? ((n < k || keep_ties) ? n : k) : n;
     int n_topk = L6;
-    if (!topk_exact_known && a.out_num_topk) {
+    if (EXTRA && !topk_exact_known && a.out_num_topk) {
         const u64 nfin = count_finite();
         n_topk = has_topk ? (int)(nfin < (u64)k ? nfin : (u64)k) : (int)nfin;
     }
     out.n_topk = n_topk;
     // the stream is over: the next kernel in the stream may be scheduled from here on
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    final_stage(s, cs, n, L6, unkey(kmax), has_minp, rp, a, b, out, full_fx, full_list ? n : 0);
+    final_stage<EXTRA>(s, cs, n, L6, unkey(kmax), has_minp, rp, a, b, out, EXTRA ? full_fx : 0ull, full_list ? n : 0);
     return true;
 }
 
 // Returns false if the row must be handled by the general path instead.  On success the
 // results are in `out` for warp 0 only.
-template <int DT>
-__device__ bool candidate_path(BlockScratch &s, const CandSmem &cs, const Ring &rg, const RowCtx &c,
+template <int DT, bool EXTRA>
+__device__ __forceinline__ bool candidate_path(BlockScratch &s, const CandSmem &cs, const Ring &rg, const RowCtx &c,
                                const RowParams &rp, const SampleArgs &a, int b, RowOut &out) {
     typedef Elem<DT> E;
     typedef VecTest<DT> T;
     const int V = c.V;
-    const bool full_list = (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) && a.num_top > 0;
+    const bool full_list = EXTRA && (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) && a.num_top > 0;
     const bool has_topk = rp.greedy || (rp.top_k >= 1 && rp.top_k < V);
     // the rank the threshold covers: top-k, or the list over the whole vocabulary if that is longer
     const int k = full_list ? max(rp.greedy ? 1 : rp.top_k, a.num_top) : rp.greedy ? 1 : rp.top_k;
     const bool has_minp = !rp.greedy && rp.min_p > 0.0f;
     // with the debug id list requested, keep the stream's threshold purely top-k so that the
     // top-k stage's set is known exactly
-    const bool stream_minp = has_minp && !full_list && !(has_topk && a.dbg_topk_ids != nullptr);
+    const bool stream_minp = has_minp && !full_list && !(EXTRA && has_topk && a.dbg_topk_ids != nullptr);
     const int lane = threadIdx.x & 31;
     // Thread -> vector map inside each group of NT vectors: lane l of warp w takes vector
     // 16 l + ((w + l) & 15).  Consecutive vectors land in different warps (the head of the
@@ -1756,7 +1816,8 @@ __device__ bool candidate_path(BlockScratch &s, const CandSmem &cs, const Ring &
         // (a large k needs a larger sample to give a useful bound: then the whole first tile; so do
         // fp32 rows, whose vectors hold half as many elements, and short rows, which have few tiles
         // over which a loose bound could still be tightened)
-        const int wvecs = (has_topk && (k > 64 || E::PER_VEC < 8 || ntiles <= 6)) ? TILE_VECS : 1;
+        // (and a ring deep enough to bring in twice as much before the list can be looked at)
+        const int wvecs = (has_topk && (k > 64 || E::PER_VEC < 8 || ntiles <= 6 || rg.nstages > 4)) ? TILE_VECS : 1;
         bool bad = !mbar_wait(&rg.bar[MAX_STAGES - 1], 0);
         if (wvecs > 1 && !bad) bad = !mbar_wait(&rg.bar[0], 0);
         uint32_t mk = 0;
@@ -1806,12 +1867,19 @@ __device__ bool candidate_path(BlockScratch &s, const CandSmem &cs, const Ring &
     const bool early_ckpt = ntiles <= rg.nstages + 2;
     const uint32_t low_trig = (uint32_t)(has_topk ? 2 * k + 32 : CAND_CAP / 4);
     bool first_look = true;
+    // A large k: a sample of one tile lets about k elements of every further tile through, which would fill
+    // the list before a rendezvous asked for by its length can take place (such rows then went to the
+    // general path: 130 us instead of 20 at k = 121).  The list is looked at after 2, 4, 8 ... tiles: each
+    // doubling of what has been seen adds 0.7 k entries.
+    int next_look = has_topk && k > 64 ? 2 : 0x7FFFFFFF;
     for (int tile = 0; tile < ntiles; ++tile) {
         // Tile 0 holds the head of the vocabulary and is the densest, and a bound from 4x the warm-up
         // sample is much tighter: if the list is already long after it, it is looked at early --
         // in short rows at a fixed checkpoint before tile 1, in long rows at a rendezvous that the
         // last warp to finish tile 0 asks for (see below), which costs rows with a short list nothing.
-        if ((uint32_t)tile == *(volatile uint32_t *)&s.maint_at || (early_ckpt && tile == 1)) {
+        const bool due = tile == next_look;
+        if ((uint32_t)tile == *(volatile uint32_t *)&s.maint_at || (early_ckpt && tile == 1) || due) {
+            if (due) next_look *= 2;
             __syncthreads();                       // every warp is between tiles: nobody appends
             int n = (int)s.cand_cnt;
             const uint32_t ovf = s.overflow, rmax = s.runmax, tmo = s.timeout;
@@ -1826,7 +1894,7 @@ __device__ bool candidate_path(BlockScratch &s, const CandSmem &cs, const Ring &
             // make the threshold identical in every thread again
             uint32_t tau_new = tau_topk;
             if (stream_minp && rmax) { seen_max = rmax; uint32_t f = minp_key(unkey(rmax), rp.ln_min_p); tau_new = f > tau_new ? f : tau_new; }
-            const uint32_t trig_now = first_look ? min(trig, low_trig) : trig;
+            const uint32_t trig_now = due ? (uint32_t)(k + 32) : first_look ? min(trig, low_trig) : trig;
             first_look = false;
             if ((uint32_t)n + 1u >= trig_now) {
                 if (has_topk && n >= k) {
@@ -1982,16 +2050,25 @@ __device__ bool candidate_path(BlockScratch &s, const CandSmem &cs, const Ring &
     if (ovf || n < 1) return false;
 
     const uint32_t kmax = s.runmax;    // the row's largest score is always a candidate
-    const u64 full_fx = (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) ? full_vocab_mass<DT>(s, c, unkey(kmax)) : 0ull;
-    return candidate_finish(s, cs, n, tau_key, kmax, rp, a, b, out, full_fx, [&] {
-        // diagnostic only: count the finite scores of the row
-        uint32_t local = 0;
-        for_each_score<DT>(c, [&](int, float z) { uint32_t kk = key_of(z); local += (kk >= KEY_MIN_FINITE && kk < KEY_POS_INF); });
-        return block_sum_u64(s, local);
+    // passes over the whole row that only some calls ask for, out of line
+    auto totals = [&]() {
+        if (threadIdx.x == 0) passes_begin<DT>(s, c, a.vps, a.nstages);
+        __syncthreads();
+        whole_row_totals<DT>(&s, unkey(kmax));
+    };
+    u64 full_fx = 0;
+    if (EXTRA && (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB)) {
+        totals();
+        full_fx = s.bcast[0];
+        if (s.timeout) { out.status |= ALBIREO_ROW_TIMEOUT; out.token = -1; out.logprob = __uint_as_float(0x7FC00000u); out.n_keep = 0; out.n_topk = 0; return true; }
+        __syncthreads();
+    }
+    return candidate_finish<EXTRA>(s, cs, n, tau_key, kmax, rp, a, b, out, full_fx, [&]() -> u64 {
+        if (!EXTRA) return 0ull;
+        totals();
+        return s.bcast[1];
     });
 }
-
-#include "wide_path.cuh"
 
 // ------------------------------------------------------------------ a row's parameters and its results
 
@@ -2046,14 +2123,72 @@ __device__ __forceinline__ void store_row(const SampleArgs &a, int b, RowOut &ou
     }
 }
 
+// A row that the candidate path does not take or had to give up, by one CTA from global memory: the wide
+// path where it applies, else the general path.  It starts from the launch arguments alone (and builds
+// the history tables itself): whatever the streaming path would have to keep for it stayed in registers
+// across the stream, and spilled ones come back from memory, behind megabytes of copies, in 1 to 3 us.
+// (Called with the streaming path's structures by value, it cost the metric workload 2 to 4 us of 20.)
+// tab_off: where the history tables lie; no copy is in flight.
+template <int DT>
+__device__ __noinline__ void leftover_row(BlockScratch *sp, const SampleArgs *ap, int tab_off) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    BlockScratch &s = *sp;
+    const SampleArgs &a = *ap;
+    const int b = blockIdx.x;
+    RowParams rp;
+    RowCtx c;
+    uint32_t status = load_row<DT>(a, b, s.seg_base, rp, c);
+    if (a.hist_ids && a.hist_off) {
+        const int o0 = a.hist_off[b], o1 = a.hist_off[b + 1];
+        if (o1 > o0) {
+            HistSmem hs;
+            const int nwords = (a.V + 31) >> 5, ncoarse = (nwords + 7) >> 3;
+            hs.bitmap = (uint32_t *)(smem + tab_off);
+            hs.coarse = hs.bitmap + (nwords + 1);
+            hs.counts = hs.coarse + (ncoarse + 1);
+            hist_prefetch(a.hist_ids + o0, o1 - o0, (int32_t *)smem);
+            c.has_hist = build_history(s, hs, c, a.hist_ids + o0, o1 - o0, a.out_start ? a.out_start[b] : 0, (const int32_t *)smem,
+                                       a.ws_counts, a.ws_counts_cap, (int64_t)o0);
+            if (!c.has_hist) status |= ALBIREO_ROW_HISTORY_OVERFLOW;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        fill_general_args(s.ga, a);
+        passes_begin<DT>(s, c, a.vps, a.nstages);
+        row_shared().rp = rp;
+    }
+    __syncthreads();
+    RowOut out;
+    out.status = status | ROW_NOT_DONE;
+    if (wide_eligible(rp, a)) {
+        const RowShared &r = row_shared();
+        SoloTeam tm;
+        tm.x = (TeamWords *)(smem + TEAM_OFF);
+        max_and_count<DT>(sp);
+        const uint32_t kmax = s.mm_max, n_fin = s.list_cnt;
+        __syncthreads();
+        if (kmax >= KEY_MIN_FINITE) out = wide_row<DT>(s, RingSlice<DT>(), tm, r.rp, r.c.invT, kmax, n_fin, b, status);
+        if (r.timeout) { out.status = (out.status & ~ROW_NOT_DONE) | ALBIREO_ROW_TIMEOUT; out.token = -1; out.logprob = __uint_as_float(0x7FC00000u); out.n_keep = 0; out.n_topk = 0; }
+    }
+    if (out.status & ROW_NOT_DONE) {
+        c = row_shared().c; rp = row_shared().rp;
+        __syncthreads();                                       // the general path lays its own tables over them
+        out = general_path_call<DT>(sp, smem, c, rp, b, status);
+    }
+    store_row(a, b, out);
+}
+
 // ------------------------------------------------------------------ the kernel
 
 // dynamic shared memory layout (bytes): [candidates (8 KiB) + 512 select bins (2 KiB)]
 // [ring: nstages x 32 KiB][mbarriers][bitmap][coarse][counts]; the general path lays its histograms,
 // gather list and search bins (8 + 24 + 16 + 4 KiB) over the first 52 KiB, which it may do because
 // the ring is idle by then
-template <int DT>
-__global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const SampleArgs a) {
+// EXTRA: whether the call asks for something beyond the ordinary (see extras_asked); the ordinary calls'
+// kernel is without the code for it, which would cost it registers.
+template <int DT, bool EXTRA>
+__global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const __grid_constant__ SampleArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ BlockScratch s;
     const int b = blockIdx.x;
@@ -2117,12 +2252,6 @@ __global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const SampleArgs 
     if (ring_started) candidate_begin<DT>(s, rg, c);
     if (!with_hist) load_params();
 
-    HistSmem hs;
-    const int nwords = (V + 31) >> 5, ncoarse = (nwords + 7) >> 3;
-    hs.bitmap = (uint32_t *)((unsigned char *)rg.bar + MAX_STAGES * 8);
-    hs.coarse = hs.bitmap + (nwords + 1);
-    hs.counts = hs.coarse + (ncoarse + 1);
-
     rp.greedy = !(rp.T > 0.0f);
     rp.ln_min_p = (!rp.greedy && rp.min_p > 0.0f) ? log((double)rp.min_p) : 0.0;
 
@@ -2135,40 +2264,46 @@ __global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const SampleArgs 
     if (!(c.r > 0.0f)) out.status |= ALBIREO_ROW_BAD_PARAM;
 
     const bool try_candidates = ring_started && candidate_eligible(rp, a);
-    if (o1 > o0) {
-        bool ok = build_history(s, hs, c, a.hist_ids + o0, o1 - o0, ostart, (const int32_t *)smem, a.ws_counts, a.ws_counts_cap, (int64_t)o0);
-        c.has_hist = ok;
-        if (!ok) out.status |= ALBIREO_ROW_HISTORY_OVERFLOW;
-    }
-
     // dbg / top-N padding first, the paths overwrite what they produce
-    if (a.dbg_topk_ids) for (int j = threadIdx.x; j < a.dbg_cap; j += NT) a.dbg_topk_ids[(int64_t)b * a.dbg_cap + j] = -1;
+    if (EXTRA && a.dbg_topk_ids) for (int j = threadIdx.x; j < a.dbg_cap; j += NT) a.dbg_topk_ids[(int64_t)b * a.dbg_cap + j] = -1;
     if (a.num_top > 0) for (int j = threadIdx.x; j < a.num_top; j += NT) {
         a.out_top_ids[(int64_t)b * a.num_top + j] = -1;
         a.out_top_logprobs[(int64_t)b * a.num_top + j] = __uint_as_float(0xFF800000u);
     }
-    __syncthreads();
 
-    CandSmem cs;
-    cs.cand = (u64 *)smem;                                  // 8 KiB
-    cs.hist = (uint32_t *)(smem + CAND_CAP * 8);            // 2 KiB
-    cs.sorted = (u64 *)rg.buf;                              // 3 x 4 KiB in the ring, used after the stream
-    cs.efx = cs.sorted + SORT_MAX;
-    cs.gsc = cs.efx + SORT_MAX;
+    const int tab_off = COMMON_BYTES + a.nstages * STAGE_BYTES + MAX_STAGES * 8;
     bool done = false;
-    if (try_candidates) done = candidate_path<DT>(s, cs, rg, c, rp, a, b, out);
-    else if (ring_started) {
-        // (the barrier above made s.issued visible)
-        bool landed = mbar_wait(&rg.bar[MAX_STAGES - 1], 0u);
-        for (int t = 0; t < (int)s.issued; ++t) landed = mbar_wait(&rg.bar[t], 0u) && landed;
-        if (__syncthreads_or(!landed)) { out.status |= ALBIREO_ROW_TIMEOUT; out.token = -1; out.logprob = __uint_as_float(0x7FC00000u); done = true; }   // the same in every thread
-    }
-    if (!done) {
-        if (threadIdx.x == 0) fill_general_args(s.ga, a);
+    if (try_candidates) {
+        if (o1 > o0) {
+            HistSmem hs;
+            const int nwords = (V + 31) >> 5, ncoarse = (nwords + 7) >> 3;
+            hs.bitmap = (uint32_t *)(smem + tab_off);
+            hs.coarse = hs.bitmap + (nwords + 1);
+            hs.counts = hs.coarse + (ncoarse + 1);
+            c.has_hist = build_history(s, hs, c, a.hist_ids + o0, o1 - o0, ostart, (const int32_t *)smem, a.ws_counts, a.ws_counts_cap, (int64_t)o0);
+            if (!c.has_hist) out.status |= ALBIREO_ROW_HISTORY_OVERFLOW;
+        }
         __syncthreads();
-        out = general_path_call<DT>(&s, smem, c, rp, b, out.status);
+        CandSmem cs;
+        cs.cand = (u64 *)smem;                                  // 8 KiB
+        cs.hist = (uint32_t *)(smem + CAND_CAP * 8);            // 2 KiB
+        cs.sorted = (u64 *)rg.buf;                              // 3 x 4 KiB in the ring, used after the stream
+        cs.efx = cs.sorted + SORT_MAX;
+        cs.gsc = cs.efx + SORT_MAX;
+        done = candidate_path<DT, EXTRA>(s, cs, rg, c, rp, a, b, out);
+    } else {
+        // (the row's first tiles are on their way: nothing of the shared memory is reused before they are there)
+        asm volatile("cp.async.wait_all;" ::: "memory");        // (the prefetched history ids)
+        __syncthreads();                                        // s.issued is visible
+        if (ring_started) {
+            bool landed = mbar_wait(&rg.bar[MAX_STAGES - 1], 0u);
+            for (int t = 0; t < (int)s.issued; ++t) landed = mbar_wait(&rg.bar[t], 0u) && landed;
+            if (__syncthreads_or(!landed)) { out.status |= ALBIREO_ROW_TIMEOUT; out.token = -1; out.logprob = __uint_as_float(0x7FC00000u); done = true; }   // the same in every thread
+        }
     }
-    store_row(a, b, out);
+    if (done) { store_row(a, b, out); return; }
+    __syncthreads();
+    leftover_row<DT>(&s, &a, tab_off);
 }
 
 #include "cluster_kernel.cuh"
@@ -2265,7 +2400,7 @@ size_t history_smem_bytes(int V) {
 // batch with no more rows than the device has SMs (`alone`: every CTA has an SM to itself), as deep as
 // one CTA's share allows
 int ring_stages_for(int V, bool with_history, bool alone) {
-    const long budget = (alone ? 233472 - 1024 : 233472 / 2 - 1024) - 1024;      // per CTA: dynamic bytes available
+    const long budget = (alone ? 233472 - 1024 : 233472 / 2 - 1024) - 1536;      // per CTA: dynamic bytes available (1 KiB reserved, 1.5 KiB static)
     long fixed = COMMON_BYTES + MAX_STAGES * 8 + (with_history ? (long)history_smem_bytes(V) : 0);
     long n = (budget - fixed) / STAGE_BYTES;
     const long cap = alone ? 6 : 4;
@@ -2362,6 +2497,11 @@ bool pick_team(LaunchShape &ls, int B, int V, int esize, bool with_history, int 
     }
     return false;
 }
+// What the ordinary instantiation of the one-CTA kernel leaves out.
+bool extras_asked(const SampleArgs &a) {
+    return (a.flags & (ALBIREO_FLAG_LOGPROB_FULL_VOCAB | ALBIREO_FLAG_TOPK_KEEP_TIES | ALBIREO_FLAG_FORCE_GENERAL)) || a.dbg_topk_ids || a.out_num_topk || a.exp1;
+}
+
 // false: the vocabulary is too large for the on-chip tables
 bool pick_shape(LaunchShape &ls, int B, int V, int esize, bool with_history, bool force_general, int num_sms, size_t max_smem) {
     if (!force_general && pick_team(ls, B, V, esize, with_history, num_sms, max_smem)) return true;
@@ -2391,7 +2531,8 @@ cudaError_t launch_sample_kernel_as(int B, const LaunchShape &ls, cudaStream_t s
         ++n;
     }
     cfg.attrs = at; cfg.numAttrs = n;
-    return ls.team > 1 ? cudaLaunchKernelEx(&cfg, albireo_cluster_kernel<DT>, a) : cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT>, a);
+    return ls.team > 1 ? cudaLaunchKernelEx(&cfg, albireo_cluster_kernel<DT>, a) 
+           : extras_asked(a) ? cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT, true>, a) : cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT, false>, a);
 }
 cudaError_t launch_sample_kernel(int dtype, int B, const LaunchShape &ls, cudaStream_t st, SampleArgs &a) {
     a.nstages = ls.nstages; a.slice_bytes = ls.slice_bytes;
@@ -2406,7 +2547,8 @@ size_t enable_large_smem(int device, cudaError_t *err) {
     cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
     const void *kernels[] = {
         (const void *)albireo_cluster_kernel<ALBIREO_F32>, (const void *)albireo_cluster_kernel<ALBIREO_BF16>, (const void *)albireo_cluster_kernel<ALBIREO_F16>,
-        (const void *)albireo_sample_kernel<ALBIREO_F32>, (const void *)albireo_sample_kernel<ALBIREO_BF16>, (const void *)albireo_sample_kernel<ALBIREO_F16>,
+        (const void *)albireo_sample_kernel<ALBIREO_F32, false>, (const void *)albireo_sample_kernel<ALBIREO_BF16, false>, (const void *)albireo_sample_kernel<ALBIREO_F16, false>,
+        (const void *)albireo_sample_kernel<ALBIREO_F32, true>, (const void *)albireo_sample_kernel<ALBIREO_BF16, true>, (const void *)albireo_sample_kernel<ALBIREO_F16, true>,
         (const void *)albireo_stream_only_kernel<ALBIREO_F32>, (const void *)albireo_stream_only_kernel<ALBIREO_BF16>, (const void *)albireo_stream_only_kernel<ALBIREO_F16>};
     size_t st = 0;
     for (const void *k : kernels) {

@@ -23,12 +23,19 @@ constexpr int MAX_TEAM = 16;
 // Words that the CTAs of a row exchange: slot r is written by CTA r, in every CTA or only in CTA 0's copy.
 struct TeamWords {
     uint32_t kmax[MAX_TEAM], tau[MAX_TEAM], tau_part[MAX_TEAM], nfin[MAX_TEAM], flags[MAX_TEAM], ncand[MAX_TEAM];   // in every CTA
+    u64 ahead[MAX_TEAM];                                                                                           // in every CTA
     u64 S[MAX_TEAM], S_all[MAX_TEAM], M[MAX_TEAM], G[MAX_TEAM];                                                    // in CTA 0's
     uint32_t n[MAX_TEAM];
     float z[MAX_TEAM];
     uint32_t far_cand, far_list;      // CTA 0: entries that the others have put at the far end of its lists
 };
 
+struct SoloTeam {                     // a CTA that has the row to itself
+    TeamWords *x;
+    static constexpr int rank = 0, size = 1;
+    __device__ __forceinline__ void sync() const { __syncthreads(); }
+    template <class P> __device__ __forceinline__ P *at(P *p, int) const { return p; }
+};
 struct ClusterTeam {                  // the CTAs of a thread-block cluster
     TeamWords *x;
     int rank, size;
@@ -76,6 +83,24 @@ __device__ __forceinline__ void block_partial(BlockScratch &s, Partial &p) {
 
 // ------------------------------------------------------------------ what a CTA reads of its row
 
+template <int DT>
+__device__ __forceinline__ uint4 kill_elements(uint4 q, uint32_t m) {      // elements of the mask become -inf
+    if constexpr (Elem<DT>::PER_VEC == 4) {
+        if (m & 1u) q.x = 0xFF800000u;
+        if (m & 2u) q.y = 0xFF800000u;
+        if (m & 4u) q.z = 0xFF800000u;
+        if (m & 8u) q.w = 0xFF800000u;
+    } else {
+        const uint32_t ninf = VecTest<DT>::fill().x;
+        auto word = [&](uint32_t w, uint32_t mm) {
+            if (mm & 1u) w = (w & 0xFFFF0000u) | (ninf & 0xFFFFu);
+            if (mm & 2u) w = (w & 0x0000FFFFu) | (ninf & 0xFFFF0000u);
+            return w;
+        };
+        q.x = word(q.x, m); q.y = word(q.y, m >> 2); q.z = word(q.z, m >> 4); q.w = word(q.w, m >> 6);
+    }
+    return q;
+}
 // element x of a vector, x not known at compile time
 template <int DT>
 __device__ __forceinline__ float pick_element(const uint4 &q, int x) {
@@ -83,6 +108,112 @@ __device__ __forceinline__ float pick_element(const uint4 &q, int x) {
     const uint32_t w = x < PV / 2 ? (x < PV / 4 ? q.x : q.y) : (x < 3 * PV / 4 ? q.z : q.w);
     return Elem<DT>::get(make_uint4(w, w, w, w), PV == 4 ? 0 : (x & 1));
 }
+
+// The whole row, streamed from global memory (from the L2 after the first pass) through a ring of bulk
+// copies: next to CTAs that stream their own rows a plain load comes back after 1.5 to 3 us, and only the
+// copies of whole tiles keep enough of them in flight.  Penalised tokens are masked out of the vectors
+// and come from the history tables.  Both loops have the same trip count in every lane of a warp (lanes
+// past the end see -inf), so that the callee may use warp collectives, but no block barriers.
+// (A pass needs its registers for the elements: what the loop does not touch per vector stays in shared memory.)
+constexpr int WIDE_TILE_VECS = 2;                              // vectors per thread and tile: 16 KiB
+constexpr int WIDE_TILE_BYTES = NT * WIDE_TILE_VECS * 16;
+constexpr int WIDE_MAX_STAGES = 6;
+struct RowShared {
+    RowCtx c;
+    RowParams rp;
+    const uint4 *vp;
+    int head, nvec, vps, nst;
+    uint32_t tiles;               // tiles of the passes so far
+    uint32_t timeout;             // a wait on a copy expired
+    uint32_t done[WIDE_MAX_STAGES];
+    uint64_t bar[WIDE_MAX_STAGES];
+};
+__device__ __forceinline__ RowShared &row_shared();
+__device__ __forceinline__ unsigned char *wide_stage(int st);
+template <int DT>
+struct RingSlice {
+    typedef Elem<DT> E;
+    __device__ __forceinline__ int first_id() const { return row_shared().head; }
+    __device__ __forceinline__ static void issue(RowShared &r, int t, int st) {
+        Ring rg;
+        rg.vps = r.vps; rg.seg_base = r.c.seg_base;
+        const int v0 = t * (NT * WIDE_TILE_VECS), nv = min(r.nvec - v0, NT * WIDE_TILE_VECS);
+        mbar_expect_tx(&r.bar[st], (uint32_t)nv * 16u);
+        ring_copy(rg, wide_stage(st), r.vp, v0, nv, &r.bar[st]);
+    }
+    // The tiles of all passes are numbered through, which gives stage and phase; the last warp done with a
+    // stage refills it.  A wait that expires marks the row.
+    template <class F> __device__ __forceinline__ void vectors(F &&f) const {
+        RowShared &r = row_shared();
+        const uint32_t first = r.tiles;
+        const int nvec = r.nvec, head = r.head, nst = r.nst, ntiles = (nvec + NT * WIDE_TILE_VECS - 1) / (NT * WIDE_TILE_VECS);
+        const uint32_t *bitmap = r.c.has_hist ? r.c.bitmap : nullptr;
+        int st = (int)(first % (uint32_t)nst);
+        uint32_t parity = (first / (uint32_t)nst) & 1u;
+        if (threadIdx.x == 0) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+#pragma unroll 1
+            for (int t = 0, q = st; t < min(ntiles, nst); ++t) { issue(r, t, q); q = q + 1 == nst ? 0 : q + 1; }
+        }
+        __syncwarp();       // (the other lanes of the issuing warp, spinning on the first copy, could keep the issuing lane from running)
+#pragma unroll 1
+        for (int t = 0; t < ntiles; ++t) {
+            if (*(volatile uint32_t *)&r.timeout == 0u && !mbar_wait(&r.bar[st], parity)) r.timeout = 1u;
+            __syncwarp();
+            const uint4 *stage = (const uint4 *)wide_stage(st);
+#pragma unroll 1
+            for (int u = 0; u < WIDE_TILE_VECS; ++u) {
+                const int v = (t * WIDE_TILE_VECS + u) * NT + (int)threadIdx.x, i0 = head + v * E::PER_VEC;
+                uint4 q = VecTest<DT>::fill();
+                if (v < nvec) {
+                    q = stage[u * NT + threadIdx.x];
+                    if (bitmap) {
+                        const uint32_t m = __funnelshift_r(bitmap[i0 >> 5], bitmap[(i0 >> 5) + 1], i0 & 31) & ((1u << E::PER_VEC) - 1u);
+                        if (m) q = kill_elements<DT>(q, m);
+                    }
+                }
+                f(q, i0);
+            }
+            __syncwarp();
+            if ((threadIdx.x & 31) == 0) {
+                __threadfence_block();
+                if (atomicAdd(&r.done[st], 1u) == (uint32_t)(NWARPS - 1)) {
+                    r.done[st] = 0;
+                    __threadfence_block();
+                    if (t + nst < ntiles) {
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        issue(r, t + nst, st);
+                    }
+                }
+            }
+            __syncwarp();
+            if (++st == nst) { st = 0; parity ^= 1u; }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) r.tiles = first + (uint32_t)ntiles;
+        __syncthreads();
+    }
+    template <class F> __device__ __forceinline__ void extras(F &&f) const {
+        const RowShared &r = row_shared();
+        const RowCtx &c = r.c;
+        const int head = r.head, tail0 = head + r.nvec * E::PER_VEC, nscal = head + (c.V - tail0);
+        const int total = nscal + (c.has_hist ? (int)c.n_distinct : 0);
+#pragma unroll 1
+        for (int base = 0; base < total; base += NT) {
+            const int q = base + (int)threadIdx.x;
+            int i = 0; float z = -INFINITY;
+            if (q < nscal) {
+                i = q < head ? q : tail0 + (q - head);
+                if (!(c.has_hist && ((c.bitmap[i >> 5] >> (i & 31)) & 1u))) z = __fmul_rn(E::load(elem_ptr<DT>(c, i), 0), c.invT);
+            } else if (q < total) {
+                const uint32_t rank = (uint32_t)(q - nscal);
+                i = hist_id_of_rank(c, rank);
+                z = __fmul_rn(penalise_counted(c, E::load(elem_ptr<DT>(c, i), 0), c.counts[rank]), c.invT);
+            }
+            f(i, z);
+        }
+    }
+};
 
 // A slice of the row that lies in shared memory, its penalised tokens already overwritten with -inf;
 // they and the row's unaligned ends are in a list of (id, score).  Both loops have the same trip count
@@ -154,6 +285,10 @@ constexpr int WIDE_LIST_OFF = COMMON_BYTES, WIDE_HIST_OFF = WIDE_LIST_OFF + W_LI
 constexpr int WIDE_QUEUE_OFF = WIDE_HIST_OFF + W_BINS * 4, WIDE_BYTES = WIDE_QUEUE_OFF + NWARPS * 64 * 8;
 static_assert(W_LIST <= NWARPS * 64, "the list's masses lie over the queues");
 constexpr int TEAM_OFF = WIDE_BYTES, SLICE_OFF = (TEAM_OFF + (int)sizeof(TeamWords) + 127) & ~127;
+// (a CTA that has the row to itself: the row's own block and the ring of its passes follow)
+constexpr int ROW_OFF = SLICE_OFF, WIDE_RING_OFF = (ROW_OFF + (int)sizeof(RowShared) + 127) & ~127;
+__device__ __forceinline__ RowShared &row_shared() { extern __shared__ __align__(128) unsigned char smem[]; return *(RowShared *)(smem + ROW_OFF); }
+__device__ __forceinline__ unsigned char *wide_stage(int st) { extern __shared__ __align__(128) unsigned char smem[]; return smem + WIDE_RING_OFF + st * WIDE_TILE_BYTES; }
 // (taken from the kernel's own shared array, so that the compiler knows the address space)
 __device__ __forceinline__ WideSmem wide_smem() {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -166,7 +301,7 @@ __device__ __forceinline__ WideSmem wide_smem() {
 // One pass of masses.  FIRST_LEVEL: every element into its bin (1/32 octave; what lies more than 42
 // octaves below the maximum is in none: 2^19 such elements weigh 1e-7 of it).  INSIDE_WINDOW: only
 // elements with code in [lo, lo + (W_BINS << shift)), into bins of 2^shift.  S: the masses of the
-// elements with z >= zfloor, S_all: of all.
+// elements with z >= zfloor (inside a window: of those ahead of it), S_all: of all.
 // Bound by issue (about 16 instructions per element) and, on the first level, by the shared-memory
 // adds (one per element, 3 to 5 bank cycles per warp).
 enum MassMode { SUM_ONLY, FIRST_LEVEL, INSIDE_WINDOW };
@@ -182,9 +317,10 @@ __device__ __forceinline__ void mass_pass(const SRC &src, float invT, float zmax
         if (FLOOR) {
             all += e;
             const bool in = z >= zfloor;
-            acc += in ? e : 0.0f;
+            if (MODE != INSIDE_WINDOW) acc += in ? e : 0.0f;
             f = in ? f : 0xFFFFFFFFu;
-        } else acc += e;
+        } else if (MODE != INSIDE_WINDOW) acc += e;
+        if (MODE == INSIDE_WINDOW) acc += f < lo ? e : 0.0f;
         if (MODE == FIRST_LEVEL) hist_add_if(hist, (f >> W_SHIFT) - (F_ZERO >> W_SHIFT), mass12(e, f >> 16));
         if (MODE == INSIDE_WINDOW) hist_add_if(hist, f >= lo ? (f - lo) >> shift : 0xFFFFFFFFu, mass12(e, f >> 16));
     };
@@ -207,17 +343,18 @@ __device__ __forceinline__ void mass_pass(const SRC &src, float invT, float zmax
 }
 
 // One level of the search: where the running total of the team's histogram (masses, or lower bounds of
-// the element counts) reaches its target, with slack on both sides (targets beyond the total are cut
-// down to it).  On the first level of a search by mass the target is the share `frac` of the histogram's
-// own total, so that what its rounding adds or loses everywhere cancels.
+// the element counts) reaches its target, give or take the rounding of the histogram: 2^-slack_shift of
+// its total on both sides, or so many elements (targets beyond the total are cut down to it).  On the first level of a search
+// by mass the target is the share `frac` of the histogram's own total.
 struct Window {
     uint32_t lo, hi;      // codes, both inclusive
+    uint32_t id_lo, id_hi;      // of the elements with code lo only ids from id_lo on, of those with code hi only up to id_hi
     u64 before;           // running total ahead of lo
     uint32_t most;        // no more elements than this lie in [lo, hi]
     bool found;
 };
 template <class TEAM>
-__device__ __noinline__ Window find_window(BlockScratch *sp, TEAM tm, bool by_count, uint32_t base, int shift, double frac, u64 target, u64 *total) {
+__device__ __noinline__ Window find_window(BlockScratch *sp, TEAM tm, bool by_count, uint32_t base, int shift, double frac, u64 target, int slack_shift) {
     BlockScratch &s = *sp;
     uint32_t *hist = wide_smem().hist;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -255,9 +392,8 @@ __device__ __noinline__ Window find_window(BlockScratch *sp, TEAM tm, bool by_co
     const u64 tot = warp_total(wt);
     u64 run = warp_total(lane < wid ? wt : 0ull) + inc - local;
     uint32_t crun = __reduce_add_sync(0xFFFFFFFFu, lane < wid ? wc : 0u) + cinc - cnt;
-    if (frac > 0.0) { *total = tot; target = (u64)(frac * (double)tot); }
-    // (the rounding of the histogram is far inside 2^-14 of the total)
-    const u64 slack = by_count ? 0ull : (*total >> 14) + 1;
+    if (frac > 0.0) target = (u64)(frac * (double)tot);
+    const u64 slack = by_count ? (u64)slack_shift : (tot >> slack_shift) + 1;
     u64 t_lo = target > slack ? target - slack : 1, t_hi = target + slack;
     if (t_hi > tot) t_hi = tot;
     if (t_lo < 1) t_lo = 1;
@@ -273,17 +409,51 @@ __device__ __noinline__ Window find_window(BlockScratch *sp, TEAM tm, bool by_co
     const uint32_t a = s.found_digit, b2 = s.found_cnt;
     Window w;
     w.found = tot > 0 && a != 0xFFFFFFFFu && b2 != 0xFFFFFFFFu;
-    w.lo = base + (a << shift); w.hi = base + (b2 << shift) + ((1u << shift) - 1u);
+    w.lo = base + (a << shift); w.hi = base + (b2 << shift) + ((1u << shift) - 1u); w.id_lo = 0; w.id_hi = 0xFFFFFFFFu;
     w.before = s.found_above; w.most = s.cand_cnt - s.list_cnt;
     __syncthreads();
     return w;
 }
-// Narrows a window until no more than `cap` elements can be in it (or the codes run out).
+constexpr int TIE_SHIFT = 9;      // ids per bin when equal scores are told apart by them: 512 (2^19 ids at most: 1024 bins)
+// The elements of one code, counted in bins of their ids (4096 each, the unit of find_window's counts),
+// their smallest and largest order key, and the exact mass of all that are ahead of them.
+template <int DT, class SRC>
+__device__ __noinline__ void tie_pass(SRC src, float invT, float zmax, float zfloor, uint32_t code, u64 &ahead, uint32_t &kmin, uint32_t &kmax) {
+    typedef Elem<DT> E;
+    const uint32_t hist = smem_u32(wide_smem().hist);
+    u64 S = 0;
+    uint32_t mn = 0xFFFFFFFFu, mx = 0;
+    auto see = [&](int i, float z, float &acc) {
+        const float t2 = log2_mass(z, zmax);
+        const uint32_t f = code_of(t2);
+        if (!(z >= zfloor)) return;
+        acc += f < code ? ex2_ftz(t2) : 0.0f;
+        if (f == code) {
+            const uint32_t k = key_of(z);
+            mn = k < mn ? k : mn; mx = k > mx ? k : mx;
+            hist_add_if(hist, (uint32_t)i >> TIE_SHIFT, 4096u);
+        }
+    };
+    src.vectors([&](const uint4 &q, int i0) {
+        float acc = 0.0f;
+#pragma unroll 1
+        for (int j = 0; j < E::PER_VEC; ++j) see(i0 + j, __fmul_rn(pick_element<DT>(q, j), invT), acc);
+        S += __float2ull_rn(acc * FX_SCALE);
+    });
+    src.extras([&](int i, float z) { float acc = 0.0f; see(i, z, acc); S += __float2ull_rn(acc * FX_SCALE); });
+    ahead = S; kmin = mn; kmax = mx;
+}
+// Narrows a window until no more than `cap` elements can be in it (or the codes run out).  The pass over
+// the elements also gives the exact mass ahead of the window, so that the histogram's rounding counts
+// only inside it: without that a cut far down a long tail (top-p 0.999) could not be told apart from
+// thousands of tail elements.  `target`: an exact mass in 2^-40 units, or a count.
 template <int DT, bool FLOOR, class SRC, class TEAM>
 __device__ __noinline__ bool narrow_window(BlockScratch *sp, SRC src, TEAM tm, float invT, float zmax, float zfloor, bool by_count, u64 target,
-                                           u64 total, uint32_t cap, Window *wp) {
+                                           uint32_t cap, Window *wp) {
+    BlockScratch &s = *sp;
     Window w = *wp;
     uint32_t *hist = wide_smem().hist;
+    const int lane = threadIdx.x & 31;
 #pragma unroll 1
     for (int it = 0; it < 4 && w.most > cap; ++it) {
         const uint32_t width = w.hi - w.lo + 1;
@@ -292,14 +462,48 @@ __device__ __noinline__ bool narrow_window(BlockScratch *sp, SRC src, TEAM tm, f
         tm.sync();                                       // everybody has read the histograms
         for (int i = threadIdx.x; i < W_BINS; i += NT) hist[i] = 0;
         __syncthreads();
-        u64 d0, d1;
-        mass_pass<DT, INSIDE_WINDOW, FLOOR>(src, invT, zmax, zfloor, w.lo, shift, d0, d1);
+        u64 ahead, all;
+        mass_pass<DT, INSIDE_WINDOW, FLOOR>(src, invT, zmax, zfloor, w.lo, shift, ahead, all);
+        ahead = block_sum_u64(s, ahead);
+        if ((int)threadIdx.x < tm.size) *tm.at(&tm.x->ahead[tm.rank], (int)threadIdx.x) = ahead;
         tm.sync();
+        ahead = warp_total(lane < tm.size ? tm.x->ahead[lane] : 0ull);
         const u64 before = w.before;
-        w = find_window(sp, tm, by_count, w.lo, shift, 0.0, target - before, &total);
+        const u64 rest = by_count ? target - before : (target > ahead ? (target - ahead) >> 8 : 1ull);
+        w = find_window(sp, tm, by_count, w.lo, shift, 0.0, rest, by_count ? 0 : 11);
         if (!w.found) return false;
-        w.before += before;
+        w.before += before;                              // (a count; by mass the next level measures it anew)
         if (shift == 0) break;
+    }
+    if (!by_count && w.most > cap && w.lo == w.hi) {
+        // Thousands of equal scores at the cut (16-bit logits far from zero: the bulk of a vocabulary falls
+        // on a few hundred values).  They all weigh the same, so the cut among them is a count, and they
+        // are in order of their ids: the window becomes a range of ids.
+        tm.sync();
+        for (int i = threadIdx.x; i < W_BINS; i += NT) hist[i] = 0;
+        __syncthreads();
+        u64 ahead;
+        uint32_t kmin, kmax;
+        tie_pass<DT>(src, invT, zmax, zfloor, w.lo, ahead, kmin, kmax);
+        ahead = block_sum_u64(s, ahead);
+        kmax = (uint32_t)block_max_u64(s, kmax);
+        kmin = ~(uint32_t)block_max_u64(s, ~kmin);
+        if ((int)threadIdx.x < tm.size) {
+            const int r = (int)threadIdx.x;
+            *tm.at(&tm.x->ahead[tm.rank], r) = ahead; *tm.at(&tm.x->kmax[tm.rank], r) = kmax; *tm.at(&tm.x->tau[tm.rank], r) = ~kmin;
+        }
+        tm.sync();
+        const bool in = lane < tm.size;
+        ahead = warp_total(in ? tm.x->ahead[lane] : 0ull);
+        kmax = __reduce_max_sync(0xFFFFFFFFu, in ? tm.x->kmax[lane] : 0u);
+        kmin = ~__reduce_max_sync(0xFFFFFFFFu, in ? tm.x->tau[lane] : 0u);
+        if (kmin != kmax) return false;
+        const u64 each = __float2ull_rn(ex2_ftz(log2_mass(unkey(kmax), zmax)) * FX_SCALE);
+        if (each == 0) return false;
+        const u64 rest = target > ahead ? target - ahead : 1ull;
+        const Window t = find_window(sp, tm, true, 0u, TIE_SHIFT, 0.0, (rest + each - 1) / each, 1);
+        if (!t.found) return false;
+        w.id_lo = t.lo; w.id_hi = t.hi; w.most = t.most;
     }
     *wp = w;
     return w.most <= cap;
@@ -406,6 +610,7 @@ __device__ __forceinline__ void race_all(const SRC &src, uint32_t *best, float i
 struct FinalArgs {
     float invT, zmax, zfloor;
     uint32_t sure, win_hi, top_hi;       // codes: below `sure` kept; [sure, win_hi] to the list; <= top_hi to the top-N list
+    uint32_t id_lo, id_hi;               // (and where the window begins and ends among equal codes, see Window)
     uint32_t vec_thr;                    // raw threshold of the vector test
     uint64_t seed, step;
     uint32_t R;
@@ -432,39 +637,37 @@ __device__ __forceinline__ void final_pass(const SRC &src, BlockScratch &s, cons
             qn -= cnt;
             __syncwarp();
             rc.refresh(&s.runmax);
-            bool may = false;
-            int i = 0; float z = 0.0f, d = 0.0f;
-            uint32_t w = 0;
-            if (lane < cnt) {
-                const u64 en = queue[qn + lane];
-                i = (int)(uint32_t)en; z = __uint_as_float((uint32_t)(en >> 32));
-                d = __fsub_rn(z, fa.zmax);
-                may = true;
+            int i = 0; float z = -INFINITY;
+            if (lane < cnt) { const u64 en = queue[qn + lane]; i = (int)(uint32_t)en; z = __uint_as_float((uint32_t)(en >> 32)); }
+            const float t2 = log2_mass(z, fa.zmax), e = ex2_ftz(t2);
+            const uint32_t f = code_of(t2);
+            const bool alive = z >= fa.zfloor, sure = alive && (f < fa.sure || (f == fa.sure && (uint32_t)i < fa.id_lo));
+            if (alive && !sure && (f < fa.win_hi || (f == fa.win_hi && (uint32_t)i <= fa.id_hi))) {
+                const uint32_t slot = atomicAdd(&s.list_cnt, 1u);
+                if (slot < (uint32_t)W_LIST) ws.list[slot] = comp_of(key_of(z), i);
+            }
+            if (alive && f <= fa.top_hi) {
+                const uint32_t slot = atomicAdd(&s.cand_cnt, 1u);
+                if (slot < (uint32_t)W_LIST) ws.top[slot] = comp_of(key_of(z), i);
+            }
+            if (sure) {
+                S += __float2ull_rn(e * FX_SCALE); ++n;
+                uint32_t w = 0;
+                bool may = true;
                 if (!fa.exp1_row) {
                     w = race_word(fa.seed, fa.R, fa.step, i);
-                    may = unit_above(w) <= __fmaf_rn(ex2_ftz(d * 1.4426950408889634f), rc.K, 1.0f);
+                    may = unit_above(w) <= __fmaf_rn(e, rc.K, 1.0f);
                 }
+                if (may) rc.take(&s.runmax, i, z, __fsub_rn(z, fa.zmax) + (fa.exp1_row ? -logf(__ldg(fa.exp1_row + i)) : nle_once(w)));
             }
-            if (may) rc.take(&s.runmax, i, z, d + (fa.exp1_row ? -logf(__ldg(fa.exp1_row + i)) : nle_once(w)));
             __syncwarp();
         }
     };
-    auto see = [&](int i, float z) {                     // called by whole warps; z = -inf: nothing
-        const float t2 = log2_mass(z, fa.zmax);
-        const uint32_t f = code_of(t2);
-        const bool alive = z >= fa.zfloor;
-        const bool sure = alive && f < fa.sure;
-        if (sure) { S += __float2ull_rn(ex2_ftz(t2) * FX_SCALE); ++n; }
-        if (alive && f >= fa.sure && f <= fa.win_hi) {
-            const uint32_t slot = atomicAdd(&s.list_cnt, 1u);
-            if (slot < (uint32_t)W_LIST) ws.list[slot] = comp_of(key_of(z), i);
-        }
-        if (alive && f <= fa.top_hi) {
-            const uint32_t slot = atomicAdd(&s.cand_cnt, 1u);
-            if (slot < (uint32_t)W_LIST) ws.top[slot] = comp_of(key_of(z), i);
-        }
-        const uint32_t m = __ballot_sync(0xFFFFFFFFu, sure);
-        if (sure) queue[qn + __popc(m & ((1u << lane) - 1u))] = ((u64)__float_as_uint(z) << 32) | (uint32_t)i;
+    // Called by whole warps.  Everything about an element but its place in the queue is worked out 32
+    // elements at a time.
+    auto push = [&](int i, float z, bool in) {
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, in);
+        if (in) queue[qn + __popc(m & ((1u << lane) - 1u))] = ((u64)__float_as_uint(z) << 32) | (uint32_t)i;
         qn += __popc(m);
         if (qn >= 32) work(31);
     };
@@ -472,18 +675,65 @@ __device__ __forceinline__ void final_pass(const SRC &src, BlockScratch &s, cons
         uint32_t bits = VecTest<DT>::may_pass(q, fa.vec_thr, fa.invT) ? VecTest<DT>::elem_bits(q, fa.vec_thr, fa.invT) : 0u;
         while (__any_sync(0xFFFFFFFFu, bits != 0)) {     // one element per lane at a time
             const int x = __ffs(bits | 0x80000000u) - 1;
-            see(i0 + x, bits ? __fmul_rn(pick_element<DT>(q, x), fa.invT) : -INFINITY);
+            push(i0 + x, __fmul_rn(pick_element<DT>(q, x), fa.invT), bits != 0);
             bits &= bits - 1u;
         }
     });
-    src.extras([&](int i, float z) { see(i, z); });
+    src.extras([&](int i, float z) { push(i, z, z >= fa.zfloor); });
     work(0);
     p.M = S; p.n = n; p.G = rc.G; p.z = rc.z;
 }
 
+// The passes out of line, for the kernel that has 64 registers per thread: each gets them all to itself.
+struct PassOut { u64 a, b; };
+template <int DT, int MODE, bool FLOOR>
+__device__ __noinline__ PassOut solo_mass_pass(float invT, float zmax, float zfloor, uint32_t lo, int shift) {
+    PassOut o;
+    mass_pass<DT, MODE, FLOOR>(RingSlice<DT>(), invT, zmax, zfloor, lo, shift, o.a, o.b);
+    return o;
+}
+template <int DT, int OFF>
+__device__ __noinline__ Partial solo_race_all(uint32_t *best, float invT, float zmax, uint64_t seed, uint32_t R, uint64_t step) {
+    Partial p;
+    race_all<DT, OFF>(RingSlice<DT>(), best, invT, zmax, seed, R, step, p);
+    return p;
+}
+template <int DT>
+__device__ __noinline__ Partial solo_final_pass(BlockScratch *sp, FinalArgs fa) {
+    Partial p;
+    final_pass<DT>(RingSlice<DT>(), *sp, fa, p);
+    return p;
+}
+template <int DT, bool FLOOR>
+__device__ __forceinline__ void first_mass_pass(const SmemSlice<DT> &src, float invT, float zmax, float zfloor, u64 &S, u64 &S_all) {
+    mass_pass<DT, FIRST_LEVEL, FLOOR>(src, invT, zmax, zfloor, F_ZERO, W_SHIFT, S, S_all);
+}
+template <int DT, bool FLOOR>
+__device__ __forceinline__ void first_mass_pass(const RingSlice<DT> &, float invT, float zmax, float zfloor, u64 &S, u64 &S_all) {
+    const PassOut o = solo_mass_pass<DT, FIRST_LEVEL, FLOOR>(invT, zmax, zfloor, F_ZERO, W_SHIFT);
+    S = o.a; S_all = o.b;
+}
+template <int DT, int OFF>
+__device__ __forceinline__ void run_race_all(const SmemSlice<DT> &src, uint32_t *best, float invT, float zmax, uint64_t seed, uint32_t R, uint64_t step, Partial &p) {
+    race_all<DT, OFF>(src, best, invT, zmax, seed, R, step, p);
+}
+template <int DT, int OFF>
+__device__ __forceinline__ void run_race_all(const RingSlice<DT> &, uint32_t *best, float invT, float zmax, uint64_t seed, uint32_t R, uint64_t step, Partial &p) {
+    p = solo_race_all<DT, OFF>(best, invT, zmax, seed, R, step);
+}
+template <int DT> __device__ __forceinline__ void run_final_pass(const SmemSlice<DT> &src, BlockScratch &s, const FinalArgs &fa, Partial &p) { final_pass<DT>(src, s, fa, p); }
+template <int DT> __device__ __forceinline__ void run_final_pass(const RingSlice<DT> &, BlockScratch &s, const FinalArgs &fa, Partial &p) { p = solo_final_pass<DT>(&s, fa); }
+
 // ------------------------------------------------------------------ one wide row
 
 constexpr uint32_t ROW_NOT_DONE = 0x80000000u;      // internal status bit: the general path has to take the row
+
+// the mass that the kept prefix has to reach
+__device__ __forceinline__ u64 topp_target(float top_p, u64 S) {
+    const double t = ceil((double)top_p * (double)S);
+    const u64 target = t <= 1.0 ? 1ull : (u64)t;
+    return target > S ? (S < 1 ? 1ull : S) : target;
+}
 
 // CTA 0: moves the entries that the others put at the far end of `buf` behind its own n0; returns the number of all.
 __device__ __forceinline__ int close_gap(u64 *buf, int cap, int n0, int nfar) {
@@ -523,8 +773,8 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
         for (int i = threadIdx.x; i < W_BINS; i += NT) ws.hist[i] = 0;
         __syncthreads();
         u64 S, S_all;
-        if (minp) mass_pass<DT, FIRST_LEVEL, true>(src, invT, zmax, zfloor, F_ZERO, W_SHIFT, S, S_all);
-        else mass_pass<DT, FIRST_LEVEL, false>(src, invT, zmax, zfloor, F_ZERO, W_SHIFT, S, S_all);
+        if (minp) first_mass_pass<DT, true>(src, invT, zmax, zfloor, S, S_all);
+        else first_mass_pass<DT, false>(src, invT, zmax, zfloor, S, S_all);
         S = warp_total(S);
         S_all = minp ? warp_total(S_all) : S;
         if (lane == 0) { s.red[threadIdx.x >> 5] = S; s.red2[threadIdx.x >> 5] = S_all; }
@@ -536,30 +786,30 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
         }
         tm.sync();
         bool ok = true;
-        u64 total = 0;
         const u64 want = (u64)(s.ga.num_top < (int32_t)n_fin ? s.ga.num_top : (int32_t)n_fin);
         const bool all_listed = want_list && n_fin <= (uint32_t)(W_LIST / 2);
         if (want_list) {
             if (all_listed) top.hi = 0xFFFFFFFEu;
             else {
-                top = find_window(&s, tm, true, F_ZERO, W_SHIFT, 0.0, want, &total);
+                top = find_window(&s, tm, true, F_ZERO, W_SHIFT, 0.0, want, 0);
                 ok = top.found;
             }
         }
-        const double share = fmax((double)rp.top_p, 1e-12);
         if (topp && ok) {
-            win = find_window(&s, tm, false, F_ZERO, W_SHIFT, share, 0ull, &total);
+            // (a member's rounding is up to 2^-12 of it, 2^-14 of the total with those of the others)
+            win = find_window(&s, tm, false, F_ZERO, W_SHIFT, fmax((double)rp.top_p, 1e-12), 0ull, 14);
             ok = win.found;
         }
-        const u64 target = (u64)(share * (double)total);
-        if (topp && ok && win.most > (uint32_t)W_LIST)
-            ok = minp ? narrow_window<DT, true>(&s, src, tm, invT, zmax, zfloor, false, target, total, W_LIST, &win)
-                      : narrow_window<DT, false>(&s, src, tm, invT, zmax, zfloor, false, target, total, W_LIST, &win);
+        if (topp && ok && win.most > (uint32_t)W_LIST) {
+            const u64 target = topp_target(rp.top_p, warp_total(lane < tm.size ? *tm.at(&tm.x->S[lane], 0) : 0ull));
+            ok = minp ? narrow_window<DT, true>(&s, src, tm, invT, zmax, zfloor, false, target, W_LIST, &win)
+                      : narrow_window<DT, false>(&s, src, tm, invT, zmax, zfloor, false, target, W_LIST, &win);
+        }
         // (ahead of the list's last bin there are fewer than 2 num_top + 1 elements)
         const uint32_t list_cap = (uint32_t)(W_LIST - 2 * ALBIREO_MAX_NUM_TOP - 32);
         if (want_list && ok && !all_listed && top.most > list_cap)
-            ok = minp ? narrow_window<DT, true>(&s, src, tm, invT, zmax, zfloor, true, want, 0, list_cap, &top)
-                      : narrow_window<DT, false>(&s, src, tm, invT, zmax, zfloor, true, want, 0, list_cap, &top);
+            ok = minp ? narrow_window<DT, true>(&s, src, tm, invT, zmax, zfloor, true, want, list_cap, &top)
+                      : narrow_window<DT, false>(&s, src, tm, invT, zmax, zfloor, true, want, list_cap, &top);
         if (!ok) { tm.sync(); out.status |= ROW_NOT_DONE; return out; }          // (the same in every CTA)
     }
     if (threadIdx.x == 0) { s.list_cnt = 0; s.cand_cnt = 0; }
@@ -568,16 +818,17 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
     Partial p;
     if (!topp && !minp && !want_list && !exp1_row) {
         switch (src.first_id() & 3) {
-            case 0: race_all<DT, 0>(src, &s.runmax, invT, zmax, rp.seed, rp.R, s.ga.step, p); break;
-            case 1: race_all<DT, 1>(src, &s.runmax, invT, zmax, rp.seed, rp.R, s.ga.step, p); break;
-            case 2: race_all<DT, 2>(src, &s.runmax, invT, zmax, rp.seed, rp.R, s.ga.step, p); break;
-            default: race_all<DT, 3>(src, &s.runmax, invT, zmax, rp.seed, rp.R, s.ga.step, p); break;
+            case 0: run_race_all<DT, 0>(src, &s.runmax, invT, zmax, rp.seed, rp.R, s.ga.step, p); break;
+            case 1: run_race_all<DT, 1>(src, &s.runmax, invT, zmax, rp.seed, rp.R, s.ga.step, p); break;
+            case 2: run_race_all<DT, 2>(src, &s.runmax, invT, zmax, rp.seed, rp.R, s.ga.step, p); break;
+            default: run_race_all<DT, 3>(src, &s.runmax, invT, zmax, rp.seed, rp.R, s.ga.step, p); break;
         }
     } else {
         FinalArgs fa;
         fa.invT = invT; fa.zmax = zmax; fa.zfloor = zfloor;
         fa.sure = topp ? win.lo : 0xFFFFFFFFu;
         fa.win_hi = topp ? win.hi : 0u;
+        fa.id_lo = topp ? win.id_lo : 0u; fa.id_hi = topp ? win.id_hi : 0u;
         fa.top_hi = want_list ? top.hi : 0u;
         fa.seed = rp.seed; fa.step = s.ga.step; fa.R = rp.R; fa.exp1_row = exp1_row;
         // the vector test lets through everything with a code up to the largest that matters
@@ -589,7 +840,7 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
             key = k2 > key ? k2 : key;
         }
         fa.vec_thr = VecTest<DT>::raw_threshold(key, invT);
-        final_pass<DT>(src, s, fa, p);
+        run_final_pass<DT>(src, s, fa, p);
     }
     block_partial(s, p);                                 // (its barrier also ends the appends)
     const int n_list = (int)s.list_cnt, n_top = (int)s.cand_cnt;
@@ -621,10 +872,7 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
     if (need_hist) { S = warp_total(in ? x.S[lane] : 0ull); S_all = warp_total(in ? x.S_all[lane] : 0ull); }
     else if (!minp) p.n = n_fin;
     if (topp) {
-        const double t = ceil((double)rp.top_p * (double)S);
-        u64 target = t <= 1.0 ? 1ull : (u64)t;
-        if (target > S) target = S;
-        if (target < 1) target = 1;
+        const u64 target = topp_target(rp.top_p, S);
         const int L = close_gap(ws.list, W_LIST, n_list, (int)x.far_list);
         if (p.M >= target || L < 1 || L > W_LIST) { out.status |= ROW_NOT_DONE; return out; }
         // Every entry counts the mass ahead of it in the order (masses over the queues, done with by now):

@@ -108,3 +108,40 @@ def test_full_vocabulary_list(binding, sampler, cut):
     w.logprob_full_vocab = True
     w.num_top = 128
     check(binding, sampler, w, flags=binding.FLAG_LOGPROB_FULL_VOCAB)
+
+
+# ------------------------------------------------------------------ the same rows by one CTA each (batches above 74 rows)
+
+@pytest.mark.parametrize("dtype", [W.F32, W.BF16])
+@pytest.mark.parametrize("B,V", [(76, 1000), (80, 16385), (100, 33000)])
+def test_mixed_requests_one_cta_per_row(binding, sampler, B, V, dtype):
+    w = W.random_small(1200 + B, B=B, V=V, dtype=dtype)
+    w.num_top = 5
+    check(binding, sampler, w)
+
+
+@pytest.mark.parametrize("B", [2, 76])
+@pytest.mark.parametrize("cut", ["ties", "tail", "none"])
+def test_cuts_among_ties_and_far_down_the_tail(binding, sampler, B, cut):
+    """A vocabulary whose bulk falls on a few dozen bf16 values (thousands of equal scores at the cut), and
+    top-p close to 1 on a long tail."""
+    V = 60001
+    rng = np.random.default_rng(31)
+    x = (rng.standard_normal((B, V)) * 2 - (40.0 if cut == "ties" else 0.0)).astype(np.float32)
+    p = {"ties": np.linspace(0.3, 0.97, B), "tail": 1.0 - np.logspace(-2, -5, B), "none": np.ones(B)}[cut].astype(np.float32)
+    w = W.Workload(cut, B, V, W.BF16, W.f32_to_bf16_bits(x), temperature=np.full(B, 1.2, np.float32), top_p=p,
+                   seeds=np.arange(B, dtype=np.uint64))
+    g, ref = check(binding, sampler, w)
+
+
+@pytest.mark.parametrize("dtype", [W.F32, W.BF16])
+@pytest.mark.parametrize("k", [40, 65, 128, 256])
+def test_large_top_k_on_gaussian_rows(binding, sampler, dtype, k):
+    """Rows without a dense head: the candidate list has to be looked at while it grows."""
+    B, V = 80, 150001
+    rng = np.random.default_rng(33)
+    x = (rng.standard_normal((B, V)) * 3).astype(np.float32)
+    w = W.Workload("gauss", B, V, dtype, x if dtype == W.F32 else W.f32_to_bf16_bits(x), temperature=np.full(B, 0.8, np.float32),
+                   top_k=np.full(B, k, np.int32), seeds=np.arange(B, dtype=np.uint64))
+    g, _ = check(binding, sampler, w)
+    assert (g["row_status"] & 1).sum() == 0            # every row on the single-pass path
