@@ -152,6 +152,17 @@ struct GenArgs {
     uint64_t step; uint32_t flags; int32_t num_top; int32_t dbg_cap;
 };
 
+// what the last pass of the wide path needs (see final_pass)
+struct FinalArgs {
+    float invT, zmax, zfloor;
+    uint32_t sure, win_hi, top_hi;       // codes: below `sure` kept; [sure, win_hi] to the list; <= top_hi to the top-N list
+    uint32_t id_lo, id_hi;               // (and where the window begins and ends among equal codes, see Window)
+    uint32_t vec_thr;                    // raw threshold of the vector test
+    uint64_t seed, step;
+    uint32_t R;
+    const float *exp1_row;
+};
+
 struct BlockScratch {
     u64 red[NWARPS];
     u64 red2[NWARPS];
@@ -167,6 +178,7 @@ struct BlockScratch {
     uint32_t issued;             // tiles whose copy has been issued so far
     const char *seg_base[ALBIREO_MAX_SEGMENTS];   // where this row's pieces start (rows in pieces only)
     uint32_t nfin_cap;           // general path: min(#finite scores, ALBIREO_MAX_NUM_TOP + 1), parked here until the list is written
+    FinalArgs fa;
     GenArgs ga;                  // the general path's copy of the launch arguments it uses
 };
 
@@ -1680,7 +1692,9 @@ __device__ __forceinline__ void passes_begin(BlockScratch &s, const RowCtx &c, i
     if (head > c.V) head = c.V;
     r.head = head; r.nvec = (c.V - head) / Elem<DT>::PER_VEC;
     r.vp = (const uint4 *)((const char *)c.row + (size_t)head * Elem<DT>::SIZE);
-    r.nst = min(WIDE_MAX_STAGES, (COMMON_BYTES + nstages * STAGE_BYTES - WIDE_RING_OFF) / WIDE_TILE_BYTES);
+    const int room = (COMMON_BYTES + nstages * STAGE_BYTES - WIDE_RING_OFF) / WIDE_VEC_BYTES;
+    r.tv = room >= 8 ? 4 : 2;
+    r.nst = min(WIDE_MAX_STAGES, room / r.tv);
 #pragma unroll 1
     for (int q = 0; q < r.nst; ++q) { mbar_init(&r.bar[q], 1); r.done[q] = 0; }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");

@@ -115,14 +115,14 @@ __device__ __forceinline__ float pick_element(const uint4 &q, int x) {
 // and come from the history tables.  Both loops have the same trip count in every lane of a warp (lanes
 // past the end see -inf), so that the callee may use warp collectives, but no block barriers.
 // (A pass needs its registers for the elements: what the loop does not touch per vector stays in shared memory.)
-constexpr int WIDE_TILE_VECS = 2;                              // vectors per thread and tile: 16 KiB
-constexpr int WIDE_TILE_BYTES = NT * WIDE_TILE_VECS * 16;
+// (a tile is 4 vectors per thread, 32 KiB, where two of them fit, else 2: what a tile costs is the hand-shake)
+constexpr int WIDE_VEC_BYTES = NT * 16;
 constexpr int WIDE_MAX_STAGES = 6;
 struct RowShared {
     RowCtx c;
     RowParams rp;
     const uint4 *vp;
-    int head, nvec, vps, nst;
+    int head, nvec, vps, nst, tv; // stages of the ring, vectors per thread and tile
     uint32_t tiles;               // tiles of the passes so far
     uint32_t timeout;             // a wait on a copy expired
     uint32_t done[WIDE_MAX_STAGES];
@@ -133,20 +133,21 @@ __device__ __forceinline__ unsigned char *wide_stage(int st);
 template <int DT>
 struct RingSlice {
     typedef Elem<DT> E;
+    static constexpr bool SPARE_REGISTERS = false;      // 64 per thread
     __device__ __forceinline__ int first_id() const { return row_shared().head; }
     __device__ __forceinline__ static void issue(RowShared &r, int t, int st) {
         Ring rg;
         rg.vps = r.vps; rg.seg_base = r.c.seg_base;
-        const int v0 = t * (NT * WIDE_TILE_VECS), nv = min(r.nvec - v0, NT * WIDE_TILE_VECS);
+        const int v0 = t * (NT * r.tv), nv = min(r.nvec - v0, NT * r.tv);
         mbar_expect_tx(&r.bar[st], (uint32_t)nv * 16u);
-        ring_copy(rg, wide_stage(st), r.vp, v0, nv, &r.bar[st]);
+        ring_copy(rg, wide_stage(st * r.tv), r.vp, v0, nv, &r.bar[st]);
     }
     // The tiles of all passes are numbered through, which gives stage and phase; the last warp done with a
     // stage refills it.  A wait that expires marks the row.
     template <class F> __device__ __forceinline__ void vectors(F &&f) const {
         RowShared &r = row_shared();
         const uint32_t first = r.tiles;
-        const int nvec = r.nvec, head = r.head, nst = r.nst, ntiles = (nvec + NT * WIDE_TILE_VECS - 1) / (NT * WIDE_TILE_VECS);
+        const int nvec = r.nvec, head = r.head, nst = r.nst, tv = r.tv, ntiles = (nvec + NT * tv - 1) / (NT * tv);
         const uint32_t *bitmap = r.c.has_hist ? r.c.bitmap : nullptr;
         int st = (int)(first % (uint32_t)nst);
         uint32_t parity = (first / (uint32_t)nst) & 1u;
@@ -160,10 +161,10 @@ struct RingSlice {
         for (int t = 0; t < ntiles; ++t) {
             if (*(volatile uint32_t *)&r.timeout == 0u && !mbar_wait(&r.bar[st], parity)) r.timeout = 1u;
             __syncwarp();
-            const uint4 *stage = (const uint4 *)wide_stage(st);
+            const uint4 *stage = (const uint4 *)wide_stage(st * tv);
 #pragma unroll 1
-            for (int u = 0; u < WIDE_TILE_VECS; ++u) {
-                const int v = (t * WIDE_TILE_VECS + u) * NT + (int)threadIdx.x, i0 = head + v * E::PER_VEC;
+            for (int u = 0; u < tv; ++u) {
+                const int v = (t * tv + u) * NT + (int)threadIdx.x, i0 = head + v * E::PER_VEC;
                 uint4 q = VecTest<DT>::fill();
                 if (v < nvec) {
                     q = stage[u * NT + threadIdx.x];
@@ -222,6 +223,7 @@ struct RingSlice {
 template <int DT>
 struct SmemSlice {
     typedef Elem<DT> E;
+    static constexpr bool SPARE_REGISTERS = true;       // 128 per thread
     int vec_off, nvec, id0;       // where the slice and the list lie in the dynamic shared memory
     int xid_off, xz_off, nx;
     __device__ __forceinline__ int first_id() const { return id0; }
@@ -288,7 +290,7 @@ constexpr int TEAM_OFF = WIDE_BYTES, SLICE_OFF = (TEAM_OFF + (int)sizeof(TeamWor
 // (a CTA that has the row to itself: the row's own block and the ring of its passes follow)
 constexpr int ROW_OFF = SLICE_OFF, WIDE_RING_OFF = (ROW_OFF + (int)sizeof(RowShared) + 127) & ~127;
 __device__ __forceinline__ RowShared &row_shared() { extern __shared__ __align__(128) unsigned char smem[]; return *(RowShared *)(smem + ROW_OFF); }
-__device__ __forceinline__ unsigned char *wide_stage(int st) { extern __shared__ __align__(128) unsigned char smem[]; return smem + WIDE_RING_OFF + st * WIDE_TILE_BYTES; }
+__device__ __forceinline__ unsigned char *wide_stage(int st) { extern __shared__ __align__(128) unsigned char smem[]; return smem + WIDE_RING_OFF + st * WIDE_VEC_BYTES; }
 // (taken from the kernel's own shared array, so that the compiler knows the address space)
 __device__ __forceinline__ WideSmem wide_smem() {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -342,6 +344,15 @@ __device__ __forceinline__ void mass_pass(const SRC &src, float invT, float zmax
     S_out = S; S_all_out = FLOOR ? S_all : S;
 }
 
+// The passes out of line, for the kernel that has 64 registers per thread: each gets them all to itself.
+struct PassOut { u64 a, b; };
+template <int DT, int MODE, bool FLOOR>
+__device__ __noinline__ PassOut solo_mass_pass(float invT, float zmax, float zfloor, uint32_t lo, int shift) {
+    PassOut o;
+    mass_pass<DT, MODE, FLOOR>(RingSlice<DT>(), invT, zmax, zfloor, lo, shift, o.a, o.b);
+    return o;
+}
+
 // One level of the search: where the running total of the team's histogram (masses, or lower bounds of
 // the element counts) reaches its target, give or take the rounding of the histogram: 2^-slack_shift of
 // its total on both sides, or so many elements (targets beyond the total are cut down to it).  On the first level of a search
@@ -351,6 +362,7 @@ struct Window {
     uint32_t id_lo, id_hi;      // of the elements with code lo only ids from id_lo on, of those with code hi only up to id_hi
     u64 before;           // running total ahead of lo
     uint32_t most;        // no more elements than this lie in [lo, hi]
+    uint32_t ahead_most;  // nor than this ahead of it (first level)
     bool found;
 };
 template <class TEAM>
@@ -410,9 +422,18 @@ __device__ __noinline__ Window find_window(BlockScratch *sp, TEAM tm, bool by_co
     Window w;
     w.found = tot > 0 && a != 0xFFFFFFFFu && b2 != 0xFFFFFFFFu;
     w.lo = base + (a << shift); w.hi = base + (b2 << shift) + ((1u << shift) - 1u); w.id_lo = 0; w.id_hi = 0xFFFFFFFFu;
-    w.before = s.found_above; w.most = s.cand_cnt - s.list_cnt;
+    w.before = s.found_above; w.most = s.cand_cnt - s.list_cnt; w.ahead_most = s.list_cnt;
     __syncthreads();
     return w;
+}
+template <int DT, bool FLOOR>
+__device__ __forceinline__ void window_mass_pass(const SmemSlice<DT> &src, float invT, float zmax, float zfloor, uint32_t lo, int shift, u64 &ahead) {
+    u64 all;
+    mass_pass<DT, INSIDE_WINDOW, FLOOR>(src, invT, zmax, zfloor, lo, shift, ahead, all);
+}
+template <int DT, bool FLOOR>
+__device__ __forceinline__ void window_mass_pass(const RingSlice<DT> &, float invT, float zmax, float zfloor, uint32_t lo, int shift, u64 &ahead) {
+    ahead = solo_mass_pass<DT, INSIDE_WINDOW, FLOOR>(invT, zmax, zfloor, lo, shift).a;
 }
 constexpr int TIE_SHIFT = 9;      // ids per bin when equal scores are told apart by them: 512 (2^19 ids at most: 1024 bins)
 // The elements of one code, counted in bins of their ids (4096 each, the unit of find_window's counts),
@@ -436,8 +457,8 @@ __device__ __noinline__ void tie_pass(SRC src, float invT, float zmax, float zfl
     };
     src.vectors([&](const uint4 &q, int i0) {
         float acc = 0.0f;
-#pragma unroll 1
-        for (int j = 0; j < E::PER_VEC; ++j) see(i0 + j, __fmul_rn(pick_element<DT>(q, j), invT), acc);
+#pragma unroll
+        for (int j = 0; j < E::PER_VEC; ++j) see(i0 + j, __fmul_rn(E::get(q, j), invT), acc);
         S += __float2ull_rn(acc * FX_SCALE);
     });
     src.extras([&](int i, float z) { float acc = 0.0f; see(i, z, acc); S += __float2ull_rn(acc * FX_SCALE); });
@@ -452,6 +473,7 @@ __device__ __noinline__ bool narrow_window(BlockScratch *sp, SRC src, TEAM tm, f
                                            uint32_t cap, Window *wp) {
     BlockScratch &s = *sp;
     Window w = *wp;
+    const uint32_t ahead_most = w.ahead_most;
     uint32_t *hist = wide_smem().hist;
     const int lane = threadIdx.x & 31;
 #pragma unroll 1
@@ -462,8 +484,8 @@ __device__ __noinline__ bool narrow_window(BlockScratch *sp, SRC src, TEAM tm, f
         tm.sync();                                       // everybody has read the histograms
         for (int i = threadIdx.x; i < W_BINS; i += NT) hist[i] = 0;
         __syncthreads();
-        u64 ahead, all;
-        mass_pass<DT, INSIDE_WINDOW, FLOOR>(src, invT, zmax, zfloor, w.lo, shift, ahead, all);
+        u64 ahead;
+        window_mass_pass<DT, FLOOR>(src, invT, zmax, zfloor, w.lo, shift, ahead);
         ahead = block_sum_u64(s, ahead);
         if ((int)threadIdx.x < tm.size) *tm.at(&tm.x->ahead[tm.rank], (int)threadIdx.x) = ahead;
         tm.sync();
@@ -505,6 +527,7 @@ __device__ __noinline__ bool narrow_window(BlockScratch *sp, SRC src, TEAM tm, f
         if (!t.found) return false;
         w.id_lo = t.lo; w.id_hi = t.hi; w.most = t.most;
     }
+    w.ahead_most = ahead_most;
     *wp = w;
     return w.most <= cap;
 }
@@ -556,32 +579,75 @@ struct Racer {
 __device__ __forceinline__ float unit_above(uint32_t w) { return __uint_as_float((w >> 9) | 0x3F800000u); }      // 1 + (v rounded down)
 __device__ __noinline__ float nle_once(uint32_t w) { return neg_log_exp1_fast(w); }      // (where it is rare: one copy of the code)
 
-// No cut: mass and race of every element in one pass.  OFF: id of a vector's first element modulo 4
-// (the generator's blocks are 4 ids).  About 20 instructions per element, half of them Philox; vectors
-// that could not win with the luckiest word skip it.
-template <int DT, int OFF, class SRC>
-__device__ __forceinline__ void race_all(const SRC &src, uint32_t *best, float invT, float zmax, uint64_t seed, uint32_t R, uint64_t step, Partial &p) {
+__device__ __forceinline__ float race_bound(uint32_t best) {      // Racer::K of a best score's order code
+    return best ? fminf(1.0001f * ex2_ftz(-unkey(best) * 1.4426950408889634f), 3.0e34f) : 3.0e34f;
+}
+__device__ __forceinline__ void list_append(u64 *list, uint32_t *cnt, float z, int i) {
+    const uint32_t slot = atomicAdd(cnt, 1u);
+    if (slot < (uint32_t)W_LIST) list[slot] = comp_of(key_of(z), i);
+}
+
+// Mass and race element by element in one pass: of the whole row (no cut), or (CUT, arguments in s.fa) of
+// the elements kept for sure where those are a good part of the row, the window's going to the list.
+// OFF: id of a vector's first element modulo 4 (the generator's blocks are 4 ids).  About 20
+// instructions per element, half of them Philox; vectors that could not win with the luckiest word skip it.
+template <int DT, int OFF, bool CUT, class SRC>
+__device__ __forceinline__ void race_all(const SRC &src, BlockScratch &s, Partial &p) {
     typedef Elem<DT> E;
     constexpr int PV = E::PER_VEC, NB = PV / 4 + (OFF ? 1 : 0);
+    uint32_t *best = &s.runmax;
+    const float invT = s.fa.invT, zmax = s.fa.zmax;
+    const uint64_t seed = s.fa.seed, step = s.fa.step;
+    const uint32_t R = s.fa.R;
+    const uint32_t sure = CUT ? s.fa.sure : 0u, win_hi = CUT ? s.fa.win_hi : 0u;
     u64 S = 0;
+    uint32_t n = 0;
     Racer rc;
     rc.start();
+    // an element at the edge: in the window, or an equal of its first code with a lower id
+    auto edge = [&](int i, float z, float t2, uint32_t f) {
+        const FinalArgs &fa = s.fa;
+        if (!(z >= fa.zfloor)) return;
+        if (f == sure && (uint32_t)i < fa.id_lo) {
+            S += __float2ull_rn(ex2_ftz(t2) * FX_SCALE); ++n;
+            const uint32_t w = race_word(seed, R, step, i);
+            if (unit_above(w) <= __fmaf_rn(ex2_ftz(t2), rc.K, 1.0f)) rc.take(best, i, z, __fsub_rn(z, zmax) + nle_once(w));
+        } else if (f < win_hi || (f == win_hi && (uint32_t)i <= fa.id_hi)) list_append(wide_smem().list, &s.list_cnt, z, i);
+    };
     src.vectors([&](const uint4 &q, int i0) {
         float e[PV], acc = 0.0f, top = 0.0f;
+        uint32_t at_edge = 0;
 #pragma unroll
         for (int j = 0; j < PV; ++j) {
-            e[j] = ex2_ftz(log2_mass(__fmul_rn(E::get(q, j), invT), zmax));
+            const float t2 = log2_mass(__fmul_rn(E::get(q, j), invT), zmax);
+            e[j] = ex2_ftz(t2);
+            if constexpr (CUT) {
+                const uint32_t f = code_of(t2);
+                at_edge |= (uint32_t)(f >= sure && f <= win_hi) << j;
+                const bool in = f < sure;
+                e[j] = in ? e[j] : 0.0f;
+                n += in;
+            }
             acc += e[j];
             top = fmaxf(top, e[j]);
         }
         S += __float2ull_rn(acc * FX_SCALE);
+        if constexpr (CUT) {
+            while (at_edge) {
+                const int x = __ffs(at_edge) - 1;
+                at_edge &= at_edge - 1;
+                const float z = __fmul_rn(pick_element<DT>(q, x), invT), t2 = log2_mass(z, zmax);
+                edge(i0 + x, z, t2, code_of(t2));
+            }
+            __syncwarp();
+        }
         rc.refresh(best);
         if (!__any_sync(0xFFFFFFFFu, top * rc.K >= 1.16e-10f)) return;      // v is at least 2^-33
         uint32_t w[4 * NB];
         philox_blocks<NB>(seed, R, step, (uint32_t)(i0 >> 2), w);
         uint32_t hits = 0;
 #pragma unroll
-        for (int j = 0; j < PV; ++j) hits |= (uint32_t)(unit_above(w[OFF + j]) <= __fmaf_rn(e[j], rc.K, 1.0f)) << j;
+        for (int j = 0; j < PV; ++j) hits |= (uint32_t)((!CUT || e[j] > 0.0f) && unit_above(w[OFF + j]) <= __fmaf_rn(e[j], rc.K, 1.0f)) << j;
         // rare after the first vectors: the exact score, one element per lane at a time, the bound renewed in between
         while (__any_sync(0xFFFFFFFFu, hits != 0)) {
             if (hits) {
@@ -599,66 +665,84 @@ __device__ __forceinline__ void race_all(const SRC &src, uint32_t *best, float i
     });
     src.extras([&](int i, float z) {
         const float d = __fsub_rn(z, zmax);
-        if (d > -3.0e38f) {
-            S += __float2ull_rn(ex2_ftz(log2_mass(z, zmax)) * FX_SCALE);
+        if (!(d > -3.0e38f)) return;
+        const float t2 = log2_mass(z, zmax);
+        const uint32_t f = code_of(t2);
+        bool in = true;
+        if constexpr (CUT) in = f < sure;
+        if (in) {
+            S += __float2ull_rn(ex2_ftz(t2) * FX_SCALE); ++n;
             rc.take(best, i, z, d + race_nle(seed, R, step, nullptr, i));
-        }
+        } else if (f <= win_hi) edge(i, z, t2, f);        // (CUT only)
     });
-    p.M = S; p.n = 0; p.G = rc.G; p.z = rc.z;
+    p.M = S; p.n = CUT ? n : 0; p.G = rc.G; p.z = rc.z;
 }
 
-struct FinalArgs {
-    float invT, zmax, zfloor;
-    uint32_t sure, win_hi, top_hi;       // codes: below `sure` kept; [sure, win_hi] to the list; <= top_hi to the top-N list
-    uint32_t id_lo, id_hi;               // (and where the window begins and ends among equal codes, see Window)
-    uint32_t vec_thr;                    // raw threshold of the vector test
-    uint64_t seed, step;
-    uint32_t R;
-    const float *exp1_row;
-};
-
-// Mass, number and race of the elements kept for sure, and the lists.  Kept elements are scattered over
-// the lanes, and the race term is long: each warp collects them in a queue and works off 32 at a time.
+// Mass, number and race of the elements kept for sure, and the lists (arguments in s.fa).  Kept elements
+// are scattered over the lanes, and the race term is long: each warp collects them in a queue and works
+// off 32 at a time.  Without registers to spare, what has been summed up stays in shared memory, a slot per
+// warp: kept in registers across the scan it was spilled, and local memory of 1024 threads does not fit what the shared memory
+// leaves of the L1 (60 us for a row of 238016 with 64 kept elements, now a third of that).
 template <int DT, class SRC>
-__device__ __forceinline__ void final_pass(const SRC &src, BlockScratch &s, const FinalArgs &fa, Partial &p) {
+__device__ __forceinline__ void final_pass(const SRC &src, BlockScratch &s, Partial &p) {
     typedef Elem<DT> E;
     const WideSmem ws = wide_smem();
-    const int lane = threadIdx.x & 31;
-    u64 *queue = ws.queue + (threadIdx.x >> 5) * 64;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    u64 *queue = ws.queue + wid * 64;
     int qn = 0;                                          // the same in every lane
+    constexpr bool REGS = SRC::SPARE_REGISTERS;
     u64 S = 0;
-    uint32_t n = 0;
+    uint32_t n_kept = 0;
     Racer rc;
     rc.start();
+    if (!REGS && lane == 0) { s.red[wid] = 0; s.red2[wid] = 0; s.r32a[wid] = 0; s.r32b[wid] = 0; }
+    __syncwarp();
     auto work = [&](int keep) {                          // works the queue off until no more than `keep` are left
+        const FinalArgs &fa = s.fa;
 #pragma unroll 1
         while (qn > keep) {
             const int cnt = qn < 32 ? qn : 32;
             qn -= cnt;
             __syncwarp();
-            rc.refresh(&s.runmax);
+            float K;
+            if constexpr (REGS) { rc.refresh(&s.runmax); K = rc.K; }
+            else K = race_bound(*(volatile uint32_t *)&s.runmax);
             int i = 0; float z = -INFINITY;
             if (lane < cnt) { const u64 en = queue[qn + lane]; i = (int)(uint32_t)en; z = __uint_as_float((uint32_t)(en >> 32)); }
             const float t2 = log2_mass(z, fa.zmax), e = ex2_ftz(t2);
             const uint32_t f = code_of(t2);
             const bool alive = z >= fa.zfloor, sure = alive && (f < fa.sure || (f == fa.sure && (uint32_t)i < fa.id_lo));
-            if (alive && !sure && (f < fa.win_hi || (f == fa.win_hi && (uint32_t)i <= fa.id_hi))) {
-                const uint32_t slot = atomicAdd(&s.list_cnt, 1u);
-                if (slot < (uint32_t)W_LIST) ws.list[slot] = comp_of(key_of(z), i);
+            if (alive && !sure && (f < fa.win_hi || (f == fa.win_hi && (uint32_t)i <= fa.id_hi))) list_append(ws.list, &s.list_cnt, z, i);
+            if (alive && f <= fa.top_hi) list_append(ws.top, &s.cand_cnt, z, i);
+            uint32_t w = 0;
+            bool may = sure;
+            if (sure && !fa.exp1_row) {
+                w = race_word(fa.seed, fa.R, fa.step, i);
+                may = unit_above(w) <= __fmaf_rn(e, K, 1.0f);
             }
-            if (alive && f <= fa.top_hi) {
-                const uint32_t slot = atomicAdd(&s.cand_cnt, 1u);
-                if (slot < (uint32_t)W_LIST) ws.top[slot] = comp_of(key_of(z), i);
-            }
-            if (sure) {
-                S += __float2ull_rn(e * FX_SCALE); ++n;
-                uint32_t w = 0;
-                bool may = true;
-                if (!fa.exp1_row) {
-                    w = race_word(fa.seed, fa.R, fa.step, i);
-                    may = unit_above(w) <= __fmaf_rn(e, rc.K, 1.0f);
-                }
+            if constexpr (REGS) {
+                if (sure) { S += __float2ull_rn(e * FX_SCALE); ++n_kept; }
                 if (may) rc.take(&s.runmax, i, z, __fsub_rn(z, fa.zmax) + (fa.exp1_row ? -logf(__ldg(fa.exp1_row + i)) : nle_once(w)));
+                __syncwarp();
+                continue;
+            }
+            const u64 mass = warp_total(sure ? __float2ull_rn(e * FX_SCALE) : 0ull);
+            const uint32_t n = (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, sure));
+            u64 G = 0;
+            if (__any_sync(0xFFFFFFFFu, may)) {
+                if (may) {
+                    const float g = __fsub_rn(z, fa.zmax) + (fa.exp1_row ? -logf(__ldg(fa.exp1_row + i)) : nle_once(w));
+                    G = ((u64)orderable_f32(g) << 32) | (uint32_t)(~(uint32_t)i);
+                }
+                __syncwarp();
+                warp_best(G, z);
+            }
+            if (lane == 0) {
+                s.red[wid] += mass; s.r32a[wid] += n;
+                if (G > s.red2[wid]) {
+                    s.red2[wid] = G; s.r32b[wid] = __float_as_uint(z);
+                    if ((uint32_t)(G >> 32) > *(volatile uint32_t *)&s.runmax) atomicMax(&s.runmax, (uint32_t)(G >> 32));
+                }
             }
             __syncwarp();
         }
@@ -671,37 +755,35 @@ __device__ __forceinline__ void final_pass(const SRC &src, BlockScratch &s, cons
         qn += __popc(m);
         if (qn >= 32) work(31);
     };
-    src.vectors([&](const uint4 &q, int i0) {
-        uint32_t bits = VecTest<DT>::may_pass(q, fa.vec_thr, fa.invT) ? VecTest<DT>::elem_bits(q, fa.vec_thr, fa.invT) : 0u;
-        while (__any_sync(0xFFFFFFFFu, bits != 0)) {     // one element per lane at a time
-            const int x = __ffs(bits | 0x80000000u) - 1;
-            push(i0 + x, __fmul_rn(pick_element<DT>(q, x), fa.invT), bits != 0);
-            bits &= bits - 1u;
-        }
-    });
-    src.extras([&](int i, float z) { push(i, z, z >= fa.zfloor); });
+    {
+        const uint32_t thr = s.fa.vec_thr;
+        const float invT = s.fa.invT;
+        src.vectors([&](const uint4 &q, int i0) {
+            uint32_t bits = VecTest<DT>::may_pass(q, thr, invT) ? VecTest<DT>::elem_bits(q, thr, invT) : 0u;
+            while (__any_sync(0xFFFFFFFFu, bits != 0)) {     // one element per lane at a time
+                const int x = __ffs(bits | 0x80000000u) - 1;
+                push(i0 + x, __fmul_rn(pick_element<DT>(q, x), invT), bits != 0);
+                bits &= bits - 1u;
+            }
+        });
+    }
+    src.extras([&](int i, float z) { push(i, z, z >= s.fa.zfloor); });
     work(0);
-    p.M = S; p.n = n; p.G = rc.G; p.z = rc.z;
+    p.M = S; p.n = n_kept; p.G = rc.G; p.z = rc.z;
+    if (!REGS && lane == 0) { p.M = s.red[wid]; p.n = s.r32a[wid]; p.G = s.red2[wid]; p.z = __uint_as_float(s.r32b[wid]); }
+    __syncwarp();
 }
 
-// The passes out of line, for the kernel that has 64 registers per thread: each gets them all to itself.
-struct PassOut { u64 a, b; };
-template <int DT, int MODE, bool FLOOR>
-__device__ __noinline__ PassOut solo_mass_pass(float invT, float zmax, float zfloor, uint32_t lo, int shift) {
-    PassOut o;
-    mass_pass<DT, MODE, FLOOR>(RingSlice<DT>(), invT, zmax, zfloor, lo, shift, o.a, o.b);
-    return o;
-}
-template <int DT, int OFF>
-__device__ __noinline__ Partial solo_race_all(uint32_t *best, float invT, float zmax, uint64_t seed, uint32_t R, uint64_t step) {
+template <int DT, int OFF, bool CUT>
+__device__ __noinline__ Partial solo_race_all(BlockScratch *sp) {
     Partial p;
-    race_all<DT, OFF>(RingSlice<DT>(), best, invT, zmax, seed, R, step, p);
+    race_all<DT, OFF, CUT>(RingSlice<DT>(), *sp, p);
     return p;
 }
 template <int DT>
-__device__ __noinline__ Partial solo_final_pass(BlockScratch *sp, FinalArgs fa) {
+__device__ __noinline__ Partial solo_final_pass(BlockScratch *sp) {
     Partial p;
-    final_pass<DT>(RingSlice<DT>(), *sp, fa, p);
+    final_pass<DT>(RingSlice<DT>(), *sp, p);
     return p;
 }
 template <int DT, bool FLOOR>
@@ -713,16 +795,30 @@ __device__ __forceinline__ void first_mass_pass(const RingSlice<DT> &, float inv
     const PassOut o = solo_mass_pass<DT, FIRST_LEVEL, FLOOR>(invT, zmax, zfloor, F_ZERO, W_SHIFT);
     S = o.a; S_all = o.b;
 }
+// (out of line in clusters too: code that is fetched only when it runs leaves the other passes' code together)
 template <int DT, int OFF>
-__device__ __forceinline__ void run_race_all(const SmemSlice<DT> &src, uint32_t *best, float invT, float zmax, uint64_t seed, uint32_t R, uint64_t step, Partial &p) {
-    race_all<DT, OFF>(src, best, invT, zmax, seed, R, step, p);
+__device__ __noinline__ Partial team_race_cut(SmemSlice<DT> src, BlockScratch *sp) {
+    Partial p;
+    race_all<DT, OFF, true>(src, *sp, p);
+    return p;
 }
-template <int DT, int OFF>
-__device__ __forceinline__ void run_race_all(const RingSlice<DT> &, uint32_t *best, float invT, float zmax, uint64_t seed, uint32_t R, uint64_t step, Partial &p) {
-    p = solo_race_all<DT, OFF>(best, invT, zmax, seed, R, step);
+template <int DT, int OFF, bool CUT>
+__device__ __forceinline__ void run_race_all(const SmemSlice<DT> &src, BlockScratch &s, Partial &p) {
+    if constexpr (CUT) p = team_race_cut<DT, OFF>(src, &s); else race_all<DT, OFF, CUT>(src, s, p);
 }
-template <int DT> __device__ __forceinline__ void run_final_pass(const SmemSlice<DT> &src, BlockScratch &s, const FinalArgs &fa, Partial &p) { final_pass<DT>(src, s, fa, p); }
-template <int DT> __device__ __forceinline__ void run_final_pass(const RingSlice<DT> &, BlockScratch &s, const FinalArgs &fa, Partial &p) { p = solo_final_pass<DT>(&s, fa); }
+template <int DT, int OFF, bool CUT>
+__device__ __forceinline__ void run_race_all(const RingSlice<DT> &, BlockScratch &s, Partial &p) { p = solo_race_all<DT, OFF, CUT>(&s); }
+template <int DT, bool CUT, class SRC>
+__device__ __forceinline__ void run_race(const SRC &src, BlockScratch &s, Partial &p) {
+    switch (src.first_id() & 3) {
+        case 0: run_race_all<DT, 0, CUT>(src, s, p); break;
+        case 1: run_race_all<DT, 1, CUT>(src, s, p); break;
+        case 2: run_race_all<DT, 2, CUT>(src, s, p); break;
+        default: run_race_all<DT, 3, CUT>(src, s, p); break;
+    }
+}
+template <int DT> __device__ __forceinline__ void run_final_pass(const SmemSlice<DT> &src, BlockScratch &s, Partial &p) { final_pass<DT>(src, s, p); }
+template <int DT> __device__ __forceinline__ void run_final_pass(const RingSlice<DT> &, BlockScratch &s, Partial &p) { p = solo_final_pass<DT>(&s); }
 
 // ------------------------------------------------------------------ one wide row
 
@@ -816,15 +912,12 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
     __syncthreads();
 
     Partial p;
-    if (!topp && !minp && !want_list && !exp1_row) {
-        switch (src.first_id() & 3) {
-            case 0: run_race_all<DT, 0>(src, &s.runmax, invT, zmax, rp.seed, rp.R, s.ga.step, p); break;
-            case 1: run_race_all<DT, 1>(src, &s.runmax, invT, zmax, rp.seed, rp.R, s.ga.step, p); break;
-            case 2: run_race_all<DT, 2>(src, &s.runmax, invT, zmax, rp.seed, rp.R, s.ga.step, p); break;
-            default: run_race_all<DT, 3>(src, &s.runmax, invT, zmax, rp.seed, rp.R, s.ga.step, p); break;
-        }
-    } else {
-        FinalArgs fa;
+    const bool no_cut = !topp && !minp && !want_list && !exp1_row;
+    // kept elements that are a good part of the row are raced in place: 25 instructions per element of the
+    // row against about 40 per kept element through the queues (`ahead_most` is up to twice their number)
+    const bool dense = topp && !minp && !want_list && !exp1_row && win.ahead_most > n_fin / 4;
+    if (threadIdx.x == 0) {
+        FinalArgs &fa = s.fa;
         fa.invT = invT; fa.zmax = zmax; fa.zfloor = zfloor;
         fa.sure = topp ? win.lo : 0xFFFFFFFFu;
         fa.win_hi = topp ? win.hi : 0u;
@@ -840,8 +933,11 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
             key = k2 > key ? k2 : key;
         }
         fa.vec_thr = VecTest<DT>::raw_threshold(key, invT);
-        run_final_pass<DT>(src, s, fa, p);
     }
+    __syncthreads();
+    if (no_cut) run_race<DT, false>(src, s, p);
+    else if (dense) run_race<DT, true>(src, s, p);
+    else run_final_pass<DT>(src, s, p);
     block_partial(s, p);                                 // (its barrier also ends the appends)
     const int n_list = (int)s.list_cnt, n_top = (int)s.cand_cnt;
     if (threadIdx.x == 0) {
