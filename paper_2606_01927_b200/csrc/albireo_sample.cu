@@ -1883,8 +1883,8 @@ __device__ __forceinline__ bool candidate_path(BlockScratch &s, const CandSmem &
     bool first_look = true;
     // A large k: a sample of one tile lets about k elements of every further tile through, which would fill
     // the list before a rendezvous asked for by its length can take place (such rows then went to the
-    // general path: 130 us instead of 20 at k = 121).  The list is looked at after 2, 4, 8 ... tiles: each
-    // doubling of what has been seen adds 0.7 k entries.
+    // general path: 130 us instead of 20 at k = 121).  The list is looked at after two tiles, and where it
+    // grows like that after 4, 8 ... as well: each doubling of what has been seen adds 0.7 k entries.
     int next_look = has_topk && k > 64 ? 2 : 0x7FFFFFFF;
     for (int tile = 0; tile < ntiles; ++tile) {
         // Tile 0 holds the head of the vocabulary and is the densest, and a bound from 4x the warm-up
@@ -1893,7 +1893,7 @@ __device__ __forceinline__ bool candidate_path(BlockScratch &s, const CandSmem &
         // last warp to finish tile 0 asks for (see below), which costs rows with a short list nothing.
         const bool due = tile == next_look;
         if ((uint32_t)tile == *(volatile uint32_t *)&s.maint_at || (early_ckpt && tile == 1) || due) {
-            if (due) next_look *= 2;
+
             __syncthreads();                       // every warp is between tiles: nobody appends
             int n = (int)s.cand_cnt;
             const uint32_t ovf = s.overflow, rmax = s.runmax, tmo = s.timeout;
@@ -1908,7 +1908,9 @@ __device__ __forceinline__ bool candidate_path(BlockScratch &s, const CandSmem &
             // make the threshold identical in every thread again
             uint32_t tau_new = tau_topk;
             if (stream_minp && rmax) { seen_max = rmax; uint32_t f = minp_key(unkey(rmax), rp.ln_min_p); tau_new = f > tau_new ? f : tau_new; }
-            const uint32_t trig_now = due ? (uint32_t)(k + 32) : first_look ? min(trig, low_trig) : trig;
+            // (a list that would not get half full by the time a rendezvous can be had needs no schedule)
+            if (due) next_look = n * (rg.nstages + 3) < CAND_CAP ? 0x7FFFFFFF : 2 * next_look;
+            const uint32_t trig_now = due && next_look != 0x7FFFFFFF ? (uint32_t)(k + 32) : first_look ? min(trig, low_trig) : trig;
             first_look = false;
             if ((uint32_t)n + 1u >= trig_now) {
                 if (has_topk && n >= k) {
@@ -2735,20 +2737,38 @@ extern "C" int albireo_sample_host(albireo_sampler_t *h, const void *logits, int
         return src ? dst : nullptr;
     };
     auto reserve = [&](size_t bytes) -> void * { void *dst = p; p += align256(bytes); return dst; };
+    // The per-row arrays are a few KB: where the caller's memory is pinned, the kernel reads and writes them
+    // there itself (one round trip over the bus, all of them at once) instead of a copy each, which costs
+    // 2 to 4 us apiece (32 rows of 152064 bf16 logits 232.8 -> 229.9 us, most of it the copy of the logits).
+    auto mapped = [&](const void *host) -> void * {
+        cudaPointerAttributes at;
+        if (!host || cudaPointerGetAttributes(&at, host) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+        return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
+    };
+    auto small = [&](const void *src, size_t bytes) -> void * {
+        void *m = mapped(src);
+        return m ? m : stage(src, bytes);
+    };
+    auto result = [&](void *dst, size_t bytes, bool &direct) -> void * {
+        void *m = mapped(dst);
+        direct = m != nullptr;
+        return m ? m : reserve(bytes);
+    };
     const size_t Bs = (size_t)B, esize = dtype == ALBIREO_F32 ? 4 : 2;
     const void *d_logits = stage(logits, Bs * (size_t)V * esize);
-    const float *d_T = (const float *)stage(temperature, Bs * 4);
-    const int32_t *d_k = (const int32_t *)stage(top_k, Bs * 4);
-    const float *d_tp = (const float *)stage(top_p, Bs * 4);
-    const float *d_mp = (const float *)stage(min_p, Bs * 4);
-    const float *d_r = (const float *)stage(repetition_penalty, Bs * 4);
-    const float *d_p = (const float *)stage(presence_penalty, Bs * 4);
-    const float *d_f = (const float *)stage(frequency_penalty, Bs * 4);
+    const float *d_T = (const float *)small(temperature, Bs * 4);
+    const int32_t *d_k = (const int32_t *)small(top_k, Bs * 4);
+    const float *d_tp = (const float *)small(top_p, Bs * 4);
+    const float *d_mp = (const float *)small(min_p, Bs * 4);
+    const float *d_r = (const float *)small(repetition_penalty, Bs * 4);
+    const float *d_p = (const float *)small(presence_penalty, Bs * 4);
+    const float *d_f = (const float *)small(frequency_penalty, Bs * 4);
     const int32_t *d_hid = (const int32_t *)stage(history_ids, (size_t)history_total * 4);
-    const int32_t *d_hoff = (const int32_t *)stage(history_offsets, (Bs + 1) * 4);
-    const uint64_t *d_seeds = (const uint64_t *)stage(seeds, Bs * 8);
-    int32_t *d_tok = (int32_t *)reserve(Bs * 4);
-    float *d_lp = (float *)reserve(Bs * 4);
+    const int32_t *d_hoff = (const int32_t *)small(history_offsets, (Bs + 1) * 4);
+    const uint64_t *d_seeds = (const uint64_t *)small(seeds, Bs * 8);
+    bool tok_direct, lp_direct;
+    int32_t *d_tok = (int32_t *)result(out_tokens, Bs * 4, tok_direct);
+    float *d_lp = (float *)result(out_logprobs, Bs * 4, lp_direct);
     albireo_sample_ext_t dx;
     memset(&dx, 0, sizeof dx);
     dx.struct_size = sizeof dx;
@@ -2769,8 +2789,8 @@ extern "C" int albireo_sample_host(albireo_sampler_t *h, const void *logits, int
     auto back = [&](void *dst, const void *src, size_t bytes) {
         if (dst && src && e == cudaSuccess) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, st);
     };
-    back(out_tokens, d_tok, Bs * 4);
-    back(out_logprobs, d_lp, Bs * 4);
+    if (!tok_direct) back(out_tokens, d_tok, Bs * 4);
+    if (!lp_direct) back(out_logprobs, d_lp, Bs * 4);
     if (ext) {
         back(ext->out_num_kept, dx.out_num_kept, Bs * 4);
         back(ext->out_num_topk, dx.out_num_topk, Bs * 4);

@@ -66,7 +66,8 @@ __device__ void slice_select(BlockScratch &s, const CandSmem &cs, uint32_t mk, i
 // The slice's penalised tokens: how often each occurs (bitmap over the slice, ranks, counts), then
 // their scores from the raw logits in shared memory, which they leave with -inf in their place.
 // Returns how many there are, or -1 if they do not fit.  Ends with a barrier.  The row's unaligned ends
-// (ids below id_lo or from id_hi on, CTA 0 only) are counted in s.red: occurrences, and in the high word all.
+// (ids below id_lo or from id_hi on, CTA 0 only) are counted in s.red: occurrences in the output, and in
+// the high word whether there are any in the prompt.
 // `landed()` waits for the slice; everything before it overlaps the copy.
 template <int DT, class W>
 __device__ __noinline__ int slice_history(BlockScratch *sp, RowCtx c, const int32_t *ids, int len, int out_start, int slice_off, int id0, int nids,
@@ -82,8 +83,12 @@ __device__ __noinline__ int slice_history(BlockScratch *sp, RowCtx c, const int3
     for (int j = threadIdx.x; j < len; j += NT) {
         const int id = __ldg(ids + j);
         const uint32_t t = (uint32_t)(id - id0);
-        if (id < id_lo ? id >= 0 : id >= id_hi && id < c.V)
-            atomicAdd(&s.red[id < id_lo ? id : id_lo + (id - id_hi)], (1ull << 32) | (u64)(j >= out_start));
+        if (id < id_lo ? id >= 0 : id >= id_hi && id < c.V) {
+            // (32-bit adds: the first ids of a vocabulary are most of many a history, and a 64-bit add in shared
+            // memory is a compare-and-swap loop, 18 us for 2700 ids)
+            uint32_t *e = (uint32_t *)&s.red[id < id_lo ? id : id_lo + (id - id_hi)];
+            if (j >= out_start) atomicAdd(e, 1u); else e[1] = 1u;
+        }
         if (t < (uint32_t)nids) {
             const uint32_t bit = 1u << (t & 31);
             if (!(*(volatile uint32_t *)&bitmap[t >> 5] & bit)) atomicOr(&bitmap[t >> 5], bit);

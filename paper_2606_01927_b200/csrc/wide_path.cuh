@@ -436,10 +436,10 @@ __device__ __forceinline__ void window_mass_pass(const RingSlice<DT> &, float in
     ahead = solo_mass_pass<DT, INSIDE_WINDOW, FLOOR>(invT, zmax, zfloor, lo, shift).a;
 }
 constexpr int TIE_SHIFT = 9;      // ids per bin when equal scores are told apart by them: 512 (2^19 ids at most: 1024 bins)
-// The elements of one code, counted in bins of their ids (4096 each, the unit of find_window's counts),
+// The elements of a few codes, counted in bins of their ids (4096 each, the unit of find_window's counts),
 // their smallest and largest order key, and the exact mass of all that are ahead of them.
 template <int DT, class SRC>
-__device__ __noinline__ void tie_pass(SRC src, float invT, float zmax, float zfloor, uint32_t code, u64 &ahead, uint32_t &kmin, uint32_t &kmax) {
+__device__ __noinline__ void tie_pass(SRC src, float invT, float zmax, float zfloor, uint32_t lo, uint32_t hi, u64 &ahead, uint32_t &kmin, uint32_t &kmax) {
     typedef Elem<DT> E;
     const uint32_t hist = smem_u32(wide_smem().hist);
     u64 S = 0;
@@ -448,8 +448,8 @@ __device__ __noinline__ void tie_pass(SRC src, float invT, float zmax, float zfl
         const float t2 = log2_mass(z, zmax);
         const uint32_t f = code_of(t2);
         if (!(z >= zfloor)) return;
-        acc += f < code ? ex2_ftz(t2) : 0.0f;
-        if (f == code) {
+        acc += f < lo ? ex2_ftz(t2) : 0.0f;
+        if (f >= lo && f <= hi) {
             const uint32_t k = key_of(z);
             mn = k < mn ? k : mn; mx = k > mx ? k : mx;
             hist_add_if(hist, (uint32_t)i >> TIE_SHIFT, 4096u);
@@ -476,14 +476,52 @@ __device__ __noinline__ bool narrow_window(BlockScratch *sp, SRC src, TEAM tm, f
     const uint32_t ahead_most = w.ahead_most;
     uint32_t *hist = wide_smem().hist;
     const int lane = threadIdx.x & 31;
+    bool try_ties = !by_count;
 #pragma unroll 1
-    for (int it = 0; it < 4 && w.most > cap; ++it) {
+    for (int it = 0; it < 6 && w.most > cap; ++it) {
         const uint32_t width = w.hi - w.lo + 1;
         int shift = 0;
         while (((width - 1) >> shift) >= (uint32_t)W_BINS) ++shift;
+        const bool ties = try_ties && width <= 16u;
+        if (!ties && width == 1u) return false;
         tm.sync();                                       // everybody has read the histograms
         for (int i = threadIdx.x; i < W_BINS; i += NT) hist[i] = 0;
         __syncthreads();
+        if (ties) {
+            // Thousands of equal scores at the cut (16-bit logits far from zero: the bulk of a vocabulary falls
+            // on a few hundred values).  They all weigh the same, so the cut among them is a count, and they
+            // are in order of their ids: the window becomes a range of ids.
+            try_ties = width > 1u;                       // (once more if they turn out not to be equal)
+            u64 ahead;
+            uint32_t kmin, kmax;
+            tie_pass<DT>(src, invT, zmax, zfloor, w.lo, w.hi, ahead, kmin, kmax);
+            ahead = block_sum_u64(s, ahead);
+            kmax = (uint32_t)block_max_u64(s, kmax);
+            kmin = ~(uint32_t)block_max_u64(s, ~kmin);
+            if ((int)threadIdx.x < tm.size) {
+                const int r = (int)threadIdx.x;
+                *tm.at(&tm.x->ahead[tm.rank], r) = ahead; *tm.at(&tm.x->kmax[tm.rank], r) = kmax; *tm.at(&tm.x->tau[tm.rank], r) = ~kmin;
+            }
+            tm.sync();
+            const bool in = lane < tm.size;
+            ahead = warp_total(in ? tm.x->ahead[lane] : 0ull);
+            kmax = __reduce_max_sync(0xFFFFFFFFu, in ? tm.x->kmax[lane] : 0u);
+            kmin = ~__reduce_max_sync(0xFFFFFFFFu, in ? tm.x->tau[lane] : 0u);
+            const u64 each = __float2ull_rn(ex2_ftz(log2_mass(unkey(kmax), zmax)) * FX_SCALE);
+            if (each == 0) return false;
+            if (kmin == kmax) {
+                const u64 rest = target > ahead ? target - ahead : 1ull;
+                const Window t = find_window(sp, tm, true, 0u, TIE_SHIFT, 0.0, (rest + each - 1) / each, 1);
+                if (!t.found) return false;
+                w.lo = w.hi = code_of(log2_mass(unkey(kmax), zmax));
+                w.id_lo = t.lo; w.id_hi = t.hi; w.most = t.most;
+                break;
+            }
+            if (width == 1u) return false;
+            tm.sync();
+            for (int i = threadIdx.x; i < W_BINS; i += NT) hist[i] = 0;
+            __syncthreads();
+        }
         u64 ahead;
         window_mass_pass<DT, FLOOR>(src, invT, zmax, zfloor, w.lo, shift, ahead);
         ahead = block_sum_u64(s, ahead);
@@ -495,37 +533,6 @@ __device__ __noinline__ bool narrow_window(BlockScratch *sp, SRC src, TEAM tm, f
         w = find_window(sp, tm, by_count, w.lo, shift, 0.0, rest, by_count ? 0 : 11);
         if (!w.found) return false;
         w.before += before;                              // (a count; by mass the next level measures it anew)
-        if (shift == 0) break;
-    }
-    if (!by_count && w.most > cap && w.lo == w.hi) {
-        // Thousands of equal scores at the cut (16-bit logits far from zero: the bulk of a vocabulary falls
-        // on a few hundred values).  They all weigh the same, so the cut among them is a count, and they
-        // are in order of their ids: the window becomes a range of ids.
-        tm.sync();
-        for (int i = threadIdx.x; i < W_BINS; i += NT) hist[i] = 0;
-        __syncthreads();
-        u64 ahead;
-        uint32_t kmin, kmax;
-        tie_pass<DT>(src, invT, zmax, zfloor, w.lo, ahead, kmin, kmax);
-        ahead = block_sum_u64(s, ahead);
-        kmax = (uint32_t)block_max_u64(s, kmax);
-        kmin = ~(uint32_t)block_max_u64(s, ~kmin);
-        if ((int)threadIdx.x < tm.size) {
-            const int r = (int)threadIdx.x;
-            *tm.at(&tm.x->ahead[tm.rank], r) = ahead; *tm.at(&tm.x->kmax[tm.rank], r) = kmax; *tm.at(&tm.x->tau[tm.rank], r) = ~kmin;
-        }
-        tm.sync();
-        const bool in = lane < tm.size;
-        ahead = warp_total(in ? tm.x->ahead[lane] : 0ull);
-        kmax = __reduce_max_sync(0xFFFFFFFFu, in ? tm.x->kmax[lane] : 0u);
-        kmin = ~__reduce_max_sync(0xFFFFFFFFu, in ? tm.x->tau[lane] : 0u);
-        if (kmin != kmax) return false;
-        const u64 each = __float2ull_rn(ex2_ftz(log2_mass(unkey(kmax), zmax)) * FX_SCALE);
-        if (each == 0) return false;
-        const u64 rest = target > ahead ? target - ahead : 1ull;
-        const Window t = find_window(sp, tm, true, 0u, TIE_SHIFT, 0.0, (rest + each - 1) / each, 1);
-        if (!t.found) return false;
-        w.id_lo = t.lo; w.id_hi = t.hi; w.most = t.most;
     }
     w.ahead_most = ahead_most;
     *wp = w;
