@@ -1,16 +1,16 @@
 // Batched token sampler for B200 (sm_100a): kernels and C ABI.
 //
-// One CTA samples one row of the [B, V] logits matrix (rows are independent, paper
-// section 6.1).  Every step of the per-row computation declared in albireo_sample.h runs
-// in this file; there is no host-side arithmetic and no fallback.
+// A CTA, or in small batches a cluster of CTAs (cluster_kernel.cuh), samples one row of the [B, V]
+// logits matrix (rows are independent, paper section 6.1).  Every step of the per-row computation
+// declared in albireo_sample.h runs in these files; there is no host-side arithmetic and no fallback.
 //
-// Two device paths produce the same result:
-//   * general path  -- multi-pass radix selection over the whole row (any parameter mix,
-//                      any kept-set size); the row is re-read from L2 between passes.
+// Three device paths produce the same result:
 //   * candidate path -- one streaming pass that keeps only the few elements that can
 //                      still be among the kept set (rows with a small top-k or a
-//                      selective min-p); falls back to the general path when its
-//                      on-chip buffers would overflow.
+//                      selective min-p); gives a row up when its on-chip buffers would overflow.
+//   * wide path     -- rows without a top-k (wide_path.cuh): a pass of masses, a pass of the race.
+//   * general path  -- multi-pass radix selection over the whole row (any parameter mix,
+//                      any kept-set size); the row is re-read from L2 between passes.
 //
 // Total order used everywhere: composite C(t) = (key(z_t) << 32) | ~t, where key() is
 // the order-preserving map of fp32 bit patterns.  Larger C comes first; all C distinct.
@@ -158,6 +158,8 @@ struct FinalArgs {
     uint32_t sure, win_hi, top_hi;       // codes: below `sure` kept; [sure, win_hi] to the list; <= top_hi to the top-N list
     uint32_t id_lo, id_hi;               // (and where the window begins and ends among equal codes, see Window)
     uint32_t vec_thr;                    // raw threshold of the vector test
+    int list_cap;
+    u64 *list;                           // the window's list
     uint64_t seed, step;
     uint32_t R;
     const float *exp1_row;

@@ -257,7 +257,8 @@ constexpr uint32_t F_ZERO = 0x4B000000u;               // bits of 2^23
 constexpr int W_SHIFT = 11;                            // 65536 / 2^11 = 32 bins per octave
 constexpr int W_BINS = 1344;                           // 42 octaves
 constexpr int W_PER = 4;                               // bins per thread in the scans (one 16-byte load; the last threads have none)
-constexpr int W_LIST = CAND_CAP;                       // entries of the window's list and of the top-N list
+constexpr int W_LIST = CAND_CAP;                       // entries of the top-N list and, beside it, of the window's list
+constexpr int W_LIST_ALONE = 2 * W_LIST;               // entries of the window's list where there is no top-N list
 
 __device__ __forceinline__ float ex2_ftz(float t) { float e; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(t)); return e; }
 __device__ __forceinline__ float log2_mass(float z, float zmax) { return __fmul_rn(__fsub_rn(z, zmax), 1.4426950408889634f); }
@@ -285,7 +286,7 @@ struct WideSmem {
 // (the candidate list and its select bins lie where the top-N list does).
 constexpr int WIDE_LIST_OFF = COMMON_BYTES, WIDE_HIST_OFF = WIDE_LIST_OFF + W_LIST * 8;
 constexpr int WIDE_QUEUE_OFF = WIDE_HIST_OFF + W_BINS * 4, WIDE_BYTES = WIDE_QUEUE_OFF + NWARPS * 64 * 8;
-static_assert(W_LIST <= NWARPS * 64, "the list's masses lie over the queues");
+static_assert(W_LIST_ALONE * 8 <= WIDE_HIST_OFF, "the window's list alone lies over both lists and the select bins");
 constexpr int TEAM_OFF = WIDE_BYTES, SLICE_OFF = (TEAM_OFF + (int)sizeof(TeamWords) + 127) & ~127;
 // (a CTA that has the row to itself: the row's own block and the ring of its passes follow)
 constexpr int ROW_OFF = SLICE_OFF, WIDE_RING_OFF = (ROW_OFF + (int)sizeof(RowShared) + 127) & ~127;
@@ -589,9 +590,9 @@ __device__ __noinline__ float nle_once(uint32_t w) { return neg_log_exp1_fast(w)
 __device__ __forceinline__ float race_bound(uint32_t best) {      // Racer::K of a best score's order code
     return best ? fminf(1.0001f * ex2_ftz(-unkey(best) * 1.4426950408889634f), 3.0e34f) : 3.0e34f;
 }
-__device__ __forceinline__ void list_append(u64 *list, uint32_t *cnt, float z, int i) {
+__device__ __forceinline__ void list_append(u64 *list, int cap, uint32_t *cnt, float z, int i) {
     const uint32_t slot = atomicAdd(cnt, 1u);
-    if (slot < (uint32_t)W_LIST) list[slot] = comp_of(key_of(z), i);
+    if (slot < (uint32_t)cap) list[slot] = comp_of(key_of(z), i);
 }
 
 // Mass and race element by element in one pass: of the whole row (no cut), or (CUT, arguments in s.fa) of
@@ -619,7 +620,7 @@ __device__ __forceinline__ void race_all(const SRC &src, BlockScratch &s, Partia
             S += __float2ull_rn(ex2_ftz(t2) * FX_SCALE); ++n;
             const uint32_t w = race_word(seed, R, step, i);
             if (unit_above(w) <= __fmaf_rn(ex2_ftz(t2), rc.K, 1.0f)) rc.take(best, i, z, __fsub_rn(z, zmax) + nle_once(w));
-        } else if (f < win_hi || (f == win_hi && (uint32_t)i <= fa.id_hi)) list_append(wide_smem().list, &s.list_cnt, z, i);
+        } else if (f < win_hi || (f == win_hi && (uint32_t)i <= fa.id_hi)) list_append(fa.list, fa.list_cap, &s.list_cnt, z, i);
     };
     src.vectors([&](const uint4 &q, int i0) {
         float e[PV], acc = 0.0f, top = 0.0f;
@@ -719,8 +720,8 @@ __device__ __forceinline__ void final_pass(const SRC &src, BlockScratch &s, Part
             const float t2 = log2_mass(z, fa.zmax), e = ex2_ftz(t2);
             const uint32_t f = code_of(t2);
             const bool alive = z >= fa.zfloor, sure = alive && (f < fa.sure || (f == fa.sure && (uint32_t)i < fa.id_lo));
-            if (alive && !sure && (f < fa.win_hi || (f == fa.win_hi && (uint32_t)i <= fa.id_hi))) list_append(ws.list, &s.list_cnt, z, i);
-            if (alive && f <= fa.top_hi) list_append(ws.top, &s.cand_cnt, z, i);
+            if (alive && !sure && (f < fa.win_hi || (f == fa.win_hi && (uint32_t)i <= fa.id_hi))) list_append(fa.list, fa.list_cap, &s.list_cnt, z, i);
+            if (alive && f <= fa.top_hi) list_append(ws.top, W_LIST, &s.cand_cnt, z, i);
             uint32_t w = 0;
             bool may = sure;
             if (sure && !fa.exp1_row) {
@@ -841,14 +842,34 @@ __device__ __forceinline__ u64 topp_target(float top_p, u64 S) {
 // CTA 0: moves the entries that the others put at the far end of `buf` behind its own n0; returns the number of all.
 __device__ __forceinline__ int close_gap(u64 *buf, int cap, int n0, int nfar) {
     if (nfar == 0) return n0;
-    u64 keep[W_LIST / NT];
+    u64 keep[W_LIST_ALONE / NT];
 #pragma unroll
-    for (int q = 0; q < W_LIST / NT; ++q) { const int j = threadIdx.x + q * NT; keep[q] = j < nfar ? buf[cap - 1 - j] : 0ull; }
+    for (int q = 0; q < W_LIST_ALONE / NT; ++q) { const int j = threadIdx.x + q * NT; keep[q] = j < nfar ? buf[cap - 1 - j] : 0ull; }
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < W_LIST / NT; ++q) { const int j = threadIdx.x + q * NT; if (j < nfar && n0 + j < cap) buf[n0 + j] = keep[q]; }
+    for (int q = 0; q < W_LIST_ALONE / NT; ++q) { const int j = threadIdx.x + q * NT; if (j < nfar && n0 + j < cap) buf[n0 + j] = keep[q]; }
     __syncthreads();
     return n0 + nfar;
+}
+
+// Sorts list[0..n) in descending order (a bitonic network over the next power of two, which it returns and
+// up to which the list is filled with zeros): 1 to 4 us where counting every entry's rank took 45 at 540.
+__device__ __noinline__ int list_sort(u64 *list, int n) {
+    int P = 2;
+    while (P < n) P <<= 1;
+    for (int i = n + (int)threadIdx.x; i < P; i += NT) list[i] = 0ull;
+    __syncthreads();
+    for (int k = 2; k <= P; k <<= 1) {
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int t = threadIdx.x; t < (P >> 1); t += NT) {
+                const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1)), l = i | j;
+                const u64 a = list[i], b2 = list[l];
+                if ((i & k) == 0 ? a < b2 : a > b2) { list[i] = b2; list[l] = a; }
+            }
+            __syncthreads();
+        }
+    }
+    return P;
 }
 
 // The row's kept set, token and log-probability; the result is CTA 0's, in its warp 0.  `kmax`, `n_fin`:
@@ -867,6 +888,8 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
     const uint32_t kfloor = minp ? minp_key(zmax, rp.ln_min_p) : KEY_MIN_FINITE;
     if (kfloor > kmax || (minp && full && want_list)) { out.status |= ROW_NOT_DONE; return out; }
     const float zfloor = unkey(kfloor);
+    u64 *const list = want_list ? ws.list : ws.top;
+    const int list_cap = want_list ? W_LIST : W_LIST_ALONE;
 
     if (threadIdx.x == 0) { s.runmax = 0; tm.x->far_cand = 0; tm.x->far_list = 0; }
     const bool need_hist = topp || want_list || (full && minp);
@@ -903,16 +926,16 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
             win = find_window(&s, tm, false, F_ZERO, W_SHIFT, fmax((double)rp.top_p, 1e-12), 0ull, 14);
             ok = win.found;
         }
-        if (topp && ok && win.most > (uint32_t)W_LIST) {
+        if (topp && ok && win.most > (uint32_t)list_cap) {
             const u64 target = topp_target(rp.top_p, warp_total(lane < tm.size ? *tm.at(&tm.x->S[lane], 0) : 0ull));
-            ok = minp ? narrow_window<DT, true>(&s, src, tm, invT, zmax, zfloor, false, target, W_LIST, &win)
-                      : narrow_window<DT, false>(&s, src, tm, invT, zmax, zfloor, false, target, W_LIST, &win);
+            ok = minp ? narrow_window<DT, true>(&s, src, tm, invT, zmax, zfloor, false, target, list_cap, &win)
+                      : narrow_window<DT, false>(&s, src, tm, invT, zmax, zfloor, false, target, list_cap, &win);
         }
         // (ahead of the list's last bin there are fewer than 2 num_top + 1 elements)
-        const uint32_t list_cap = (uint32_t)(W_LIST - 2 * ALBIREO_MAX_NUM_TOP - 32);
-        if (want_list && ok && !all_listed && top.most > list_cap)
-            ok = minp ? narrow_window<DT, true>(&s, src, tm, invT, zmax, zfloor, true, want, list_cap, &top)
-                      : narrow_window<DT, false>(&s, src, tm, invT, zmax, zfloor, true, want, list_cap, &top);
+        const uint32_t top_cap = (uint32_t)(W_LIST - 2 * ALBIREO_MAX_NUM_TOP - 32);
+        if (want_list && ok && !all_listed && top.most > top_cap)
+            ok = minp ? narrow_window<DT, true>(&s, src, tm, invT, zmax, zfloor, true, want, top_cap, &top)
+                      : narrow_window<DT, false>(&s, src, tm, invT, zmax, zfloor, true, want, top_cap, &top);
         if (!ok) { tm.sync(); out.status |= ROW_NOT_DONE; return out; }          // (the same in every CTA)
     }
     if (threadIdx.x == 0) { s.list_cnt = 0; s.cand_cnt = 0; }
@@ -930,6 +953,7 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
         fa.win_hi = topp ? win.hi : 0u;
         fa.id_lo = topp ? win.id_lo : 0u; fa.id_hi = topp ? win.id_hi : 0u;
         fa.top_hi = want_list ? top.hi : 0u;
+        fa.list = list; fa.list_cap = list_cap;
         fa.seed = rp.seed; fa.step = s.ga.step; fa.R = rp.R; fa.exp1_row = exp1_row;
         // the vector test lets through everything with a code up to the largest that matters
         uint32_t key = kfloor;
@@ -958,9 +982,9 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
             s.found_cnt = n_top ? atomicAdd(tm.at(&tm.x->far_cand, 0), (uint32_t)n_top) : 0u;
         }
         __syncthreads();
-        const int at_list = W_LIST - 1 - (int)s.found_digit, at_top = W_LIST - 1 - (int)s.found_cnt;
-        u64 *list0 = tm.at(ws.list, 0), *top0 = tm.at(ws.top, 0);
-        for (int j = threadIdx.x; j < n_list; j += NT) if (at_list - j >= 0) list0[at_list - j] = ws.list[j];
+        const int at_list = list_cap - 1 - (int)s.found_digit, at_top = W_LIST - 1 - (int)s.found_cnt;
+        u64 *list0 = tm.at(list, 0), *top0 = tm.at(ws.top, 0);
+        for (int j = threadIdx.x; j < n_list; j += NT) if (at_list - j >= 0) list0[at_list - j] = list[j];
         for (int j = threadIdx.x; j < n_top; j += NT) if (at_top - j >= 0) top0[at_top - j] = ws.top[j];
     }
     tm.sync();
@@ -976,33 +1000,52 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
     else if (!minp) p.n = n_fin;
     if (topp) {
         const u64 target = topp_target(rp.top_p, S);
-        const int L = close_gap(ws.list, W_LIST, n_list, (int)x.far_list);
-        if (p.M >= target || L < 1 || L > W_LIST) { out.status |= ROW_NOT_DONE; return out; }
-        // Every entry counts the mass ahead of it in the order (masses over the queues, done with by now):
-        // it is kept if that, with the mass kept for sure, is short of the target.
-        u64 *mass = ws.queue;
-        for (int j = threadIdx.x; j < L; j += NT) mass[j] = __float2ull_rn(ex2_ftz(log2_mass(unkey((uint32_t)(ws.list[j] >> 32)), zmax)) * FX_SCALE);
-        __syncthreads();
+        const int L = close_gap(list, list_cap, n_list, (int)x.far_list);
+        if (p.M >= target || L < 1 || L > list_cap) { out.status |= ROW_NOT_DONE; return out; }
+        auto mass_of = [&](u64 C) { return __float2ull_rn(ex2_ftz(log2_mass(unkey((uint32_t)(C >> 32)), zmax)) * FX_SCALE); };
         Partial k;
         k.M = 0; k.n = 0; k.G = 0; k.z = 0.0f;
-        u64 reach = 0;
-#pragma unroll 1
-        for (int j = threadIdx.x; j < L; j += NT) {
-            const u64 C = ws.list[j], own = mass[j];
-            u64 ahead = p.M;
+        auto keep = [&](u64 C, u64 own) {
+            k.M += own; ++k.n;
+            const float zq = unkey((uint32_t)(C >> 32));
+            const float g = __fsub_rn(zq, zmax) + race_nle(rp.seed, rp.R, s.ga.step, exp1_row, comp_idx(C));
+            const u64 gq = ((u64)orderable_f32(g) << 32) | (uint32_t)C;
+            if (gq > k.G) { k.G = gq; k.z = zq; }
+        };
+        // An entry is kept while the mass ahead of it in the order, with the mass kept for sure, is short of
+        // the target.  A short list: every entry adds that mass up (masses over the queues, done with by now),
+        // one barrier in all; from 192 entries on a sort and a prefix sum are faster (2 us against 3 at 300).
+        bool reached;
+        if (L <= 192) {
+            u64 *mass = ws.queue;
+            if ((int)threadIdx.x < L) mass[threadIdx.x] = mass_of(list[threadIdx.x]);
+            __syncthreads();
+            u64 reach = 0;
+            if ((int)threadIdx.x < L) {
+                const u64 C = list[threadIdx.x], own = mass[threadIdx.x];
+                u64 ahead = p.M;
 #pragma unroll 4
-            for (int q = 0; q < L; ++q) ahead += ws.list[q] > C ? mass[q] : 0ull;
-            reach = ahead + own > reach ? ahead + own : reach;
-            if (ahead < target) {
-                k.M += own; ++k.n;
-                const float zq = unkey((uint32_t)(C >> 32));
-                const float g = __fsub_rn(zq, zmax) + race_nle(rp.seed, rp.R, s.ga.step, exp1_row, comp_idx(C));
-                const u64 gq = ((u64)orderable_f32(g) << 32) | (uint32_t)C;
-                if (gq > k.G) { k.G = gq; k.z = zq; }
+                for (int q = 0; q < L; ++q) ahead += list[q] > C ? mass[q] : 0ull;
+                reach = ahead + own;
+                if (ahead < target) keep(C, own);
             }
+            reached = __syncthreads_or(reach + (1ull << 18) >= target) != 0;
+        } else {
+            const int P = list_sort(list, L), per = (P + NT - 1) / NT, q0 = (int)threadIdx.x * per, q1 = min(L, q0 + per);
+            u64 local = 0, tot;
+            for (int q = q0; q < q1; ++q) local += mass_of(list[q]);
+            u64 run = p.M + block_exscan_u64(s, local, tot);
+            reached = p.M + tot + (1ull << 18) >= target;
+#pragma unroll 1
+            for (int q = q0; q < q1 && run < target; ++q) {
+                const u64 C = list[q], own = mass_of(C);
+                run += own;
+                keep(C, own);
+            }
+            __syncthreads();
         }
         // (short of the target by no more than the rounding of the sums: the whole list stays)
-        if (!__syncthreads_or(reach + (1ull << 18) >= target)) { out.status |= ROW_NOT_DONE; return out; }
+        if (!reached) { out.status |= ROW_NOT_DONE; return out; }
         block_partial(s, k);
         p.M += k.M; p.n += k.n;
         if (k.G > p.G) { p.G = k.G; p.z = k.z; }
