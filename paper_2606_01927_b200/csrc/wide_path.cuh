@@ -367,7 +367,7 @@ struct Window {
     bool found;
 };
 template <class TEAM>
-__device__ __noinline__ Window find_window(BlockScratch *sp, TEAM tm, bool by_count, uint32_t base, int shift, double frac, u64 target, int slack_shift) {
+__device__ __noinline__ Window find_window(BlockScratch *sp, TEAM tm, bool by_count, uint32_t base, int shift, double frac, u64 target, int slack_shift, u64 least_slack = 0) {
     BlockScratch &s = *sp;
     uint32_t *hist = wide_smem().hist;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -406,7 +406,8 @@ __device__ __noinline__ Window find_window(BlockScratch *sp, TEAM tm, bool by_co
     u64 run = warp_total(lane < wid ? wt : 0ull) + inc - local;
     uint32_t crun = __reduce_add_sync(0xFFFFFFFFu, lane < wid ? wc : 0u) + cinc - cnt;
     if (frac > 0.0) target = (u64)(frac * (double)tot);
-    const u64 slack = by_count ? (u64)slack_shift : (tot >> slack_shift) + 1;
+    u64 slack = by_count ? (u64)slack_shift : (tot >> slack_shift) + 1;
+    slack = slack > least_slack ? slack : least_slack;
     u64 t_lo = target > slack ? target - slack : 1, t_hi = target + slack;
     if (t_hi > tot) t_hi = tot;
     if (t_lo < 1) t_lo = 1;
@@ -531,7 +532,9 @@ __device__ __noinline__ bool narrow_window(BlockScratch *sp, SRC src, TEAM tm, f
         ahead = warp_total(lane < tm.size ? tm.x->ahead[lane] : 0ull);
         const u64 before = w.before;
         const u64 rest = by_count ? target - before : (target > ahead ? (target - ahead) >> 8 : 1ull);
-        w = find_window(sp, tm, by_count, w.lo, shift, 0.0, rest, by_count ? 0 : 11);
+        // (2^-22 of the whole: a vector's masses are added in fp32 here and one by one in the last pass, and far
+        // down a tail that difference is the mass of many elements)
+        w = find_window(sp, tm, by_count, w.lo, shift, 0.0, rest, by_count ? 0 : 11, by_count ? 0ull : (target >> 30) + 1);
         if (!w.found) return false;
         w.before += before;                              // (a count; by mass the next level measures it anew)
     }
