@@ -920,8 +920,10 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
         if (want_list) {
             if (all_listed) top.hi = 0xFFFFFFFEu;
             else {
+                // (the histogram ends 42 octaves down: a row with fewer entries than wanted ahead of that is the
+                // general path's; what the bounds of the counts leave open shows when the list is there)
                 top = find_window(&s, tm, true, F_ZERO, W_SHIFT, 0.0, want, 0);
-                ok = top.found;
+                ok = top.found && (u64)top.ahead_most + top.most >= want;
             }
         }
         if (topp && ok) {
@@ -1068,6 +1070,7 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
         __syncthreads();
         const double lnS_all = __longlong_as_double((long long)s.bcast[0]);
         const uint32_t members = full ? n_fin : s.found_cnt;
+        if ((uint32_t)n_all < min((uint32_t)s.ga.num_top, members)) { out.status |= ROW_NOT_DONE; return out; }      // (the same in every thread)
 #pragma unroll 1
         for (int j = threadIdx.x; j < n_all; j += NT) {
             const u64 C = ws.top[j];

@@ -145,3 +145,24 @@ def test_large_top_k_on_gaussian_rows(binding, sampler, dtype, k):
                    top_k=np.full(B, k, np.int32), seeds=np.arange(B, dtype=np.uint64))
     g, _ = check(binding, sampler, w)
     assert (g["row_status"] & 1).sum() == 0            # every row on the single-pass path
+
+
+@pytest.mark.parametrize("B", [6, 76])
+@pytest.mark.parametrize("cut", ["none", "topp", "minp", "none_full", "topp_full"])
+@pytest.mark.parametrize("near", [1, 3])
+def test_lists_longer_than_what_carries_mass(binding, sampler, B, cut, near):
+    """Fewer elements than the list wants lie within 2^-42 of the likeliest one's mass: the list goes on with
+    the elements behind the gap wherever they are members."""
+    V = 20011
+    rng = np.random.default_rng(41)
+    x = rng.standard_normal((B, V)).astype(np.float32)
+    for b in range(B):
+        x[b, rng.permutation(V)[:near]] = 14.0 + rng.random(near).astype(np.float32)
+    par = {"topp": dict(top_p=np.full(B, 0.9, np.float32)), "minp": dict(min_p=np.full(B, 1e-30, np.float32))}.get(cut.split("_")[0], {})
+    w = W.Workload(cut, B, V, W.BF16, W.f32_to_bf16_bits(x), temperature=np.full(B, 0.25, np.float32),
+                   seeds=np.arange(B, dtype=np.uint64), **par)
+    w.num_top = 5
+    w.logprob_full_vocab = cut.endswith("full")
+    _, ref = check(binding, sampler, w, flags=binding.FLAG_LOGPROB_FULL_VOCAB if w.logprob_full_vocab else 0)
+    if cut != "topp":
+        assert (ref.top_ids >= 0).all()
