@@ -416,12 +416,18 @@ template <class P> struct VecTest16 {
     static __device__ __forceinline__ uint4 fill() { const uint32_t f = P::NEG_INF | (P::NEG_INF << 16); return make_uint4(f, f, f, f); }
     // the raw threshold that only +inf reaches (NEG_INF without its sign bit), packed twice
     static __device__ __forceinline__ uint32_t pos_inf_threshold() { const uint32_t b = P::NEG_INF & 0x7FFFu; return b | (b << 16); }
-    // how many of the vector's elements are -inf
-    static __device__ __forceinline__ uint32_t count_neginf(const uint4 &q) {
-        const uint32_t f = P::NEG_INF | (P::NEG_INF << 16);
-        const H2 ninf = *reinterpret_cast<const H2 *>(&f);
-        const uint32_t r0 = __heq2_mask(*reinterpret_cast<const H2 *>(&q.x), ninf), r1 = __heq2_mask(*reinterpret_cast<const H2 *>(&q.y), ninf);
-        const uint32_t r2 = __heq2_mask(*reinterpret_cast<const H2 *>(&q.z), ninf), r3 = __heq2_mask(*reinterpret_cast<const H2 *>(&q.w), ninf);
+    // the smallest raw value whose score is finite, packed twice (a lower temperature than 1 takes the lowest logits
+    // out of the fp32 range; where the search does not settle, the lowest finite value)
+    static __device__ __forceinline__ uint32_t finite_threshold(float invT) {
+        constexpr uint32_t LOWEST = (~P::LO & 0xFFFFu) | ((~P::LO & 0xFFFFu) << 16);
+        const uint32_t t = invT > 1.0f ? raw_threshold(KEY_MIN_FINITE, invT) : LOWEST;
+        return t == (P::NEG_INF | (P::NEG_INF << 16)) ? LOWEST : t;
+    }
+    // how many of the vector's elements are below that, i.e. have no finite score
+    static __device__ __forceinline__ uint32_t count_not_finite(const uint4 &q, uint32_t thr, float) {
+        const H2 t2 = *reinterpret_cast<const H2 *>(&thr);
+        const uint32_t r0 = __hlt2_mask(*reinterpret_cast<const H2 *>(&q.x), t2), r1 = __hlt2_mask(*reinterpret_cast<const H2 *>(&q.y), t2);
+        const uint32_t r2 = __hlt2_mask(*reinterpret_cast<const H2 *>(&q.z), t2), r3 = __hlt2_mask(*reinterpret_cast<const H2 *>(&q.w), t2);
         if (!(r0 | r1 | r2 | r3)) return 0u;
         return (uint32_t)(__popc(r0) + __popc(r1) + __popc(r2) + __popc(r3)) >> 4;
     }
@@ -451,8 +457,11 @@ template <> struct VecTest<ALBIREO_F32> {
     static __device__ __forceinline__ uint32_t vmax_key(const uint4 &q, float invT) { return key_of(vmaxz(q, invT)); }
     static __device__ __forceinline__ uint4 fill() { return make_uint4(0xFF800000u, 0xFF800000u, 0xFF800000u, 0xFF800000u); }
     static __device__ __forceinline__ uint32_t pos_inf_threshold() { return 0x7F800000u; }
-    static __device__ __forceinline__ uint32_t count_neginf(const uint4 &q) {
-        return (uint32_t)(q.x == 0xFF800000u) + (uint32_t)(q.y == 0xFF800000u) + (uint32_t)(q.z == 0xFF800000u) + (uint32_t)(q.w == 0xFF800000u);
+    static __device__ __forceinline__ uint32_t finite_threshold(float) { return __float_as_uint(unkey(KEY_MIN_FINITE)); }
+    static __device__ __forceinline__ uint32_t count_not_finite(const uint4 &q, uint32_t thr, float invT) {
+        const float t = __uint_as_float(thr);
+        return (uint32_t)(__fmul_rn(__uint_as_float(q.x), invT) < t) + (uint32_t)(__fmul_rn(__uint_as_float(q.y), invT) < t) +
+               (uint32_t)(__fmul_rn(__uint_as_float(q.z), invT) < t) + (uint32_t)(__fmul_rn(__uint_as_float(q.w), invT) < t);
     }
 };
 
@@ -523,6 +532,7 @@ __device__ __forceinline__ void pass0_max_count(const RowCtx &c, uint32_t &kbest
     if (head > V) head = V;
     const int nvec = (V - head) / E::PER_VEC;
     const uint4 *vp = (const uint4 *)((const char *)c.row + (size_t)head * E::SIZE);
+    const uint32_t fin_thr = T::finite_threshold(c.invT);
     auto one = [&](int, float z) {
         const uint32_t k = key_of(z);
         kbest = k > kbest ? k : kbest;
@@ -542,7 +552,7 @@ __device__ __forceinline__ void pass0_max_count(const RowCtx &c, uint32_t &kbest
             if (m == 0) {
                 const uint32_t k = T::vmax_key(q[u], c.invT);
                 kbest = k > kbest ? k : kbest;
-                nfin += (uint32_t)E::PER_VEC - T::count_neginf(q[u]);
+                nfin += (uint32_t)E::PER_VEC - T::count_not_finite(q[u], fin_thr, c.invT);
             } else {
 #pragma unroll
                 for (int e = 0; e < E::PER_VEC; ++e)
@@ -1708,11 +1718,12 @@ __device__ __noinline__ void max_and_count(BlockScratch *sp) {
     BlockScratch &s = *sp;
     const RingSlice<DT> src;
     const float invT = row_shared().c.invT;
+    const uint32_t fin_thr = VecTest<DT>::finite_threshold(invT);
     uint32_t kbest = 0, nfin = 0;
     src.vectors([&](const uint4 &q, int) {
         const uint32_t k = VecTest<DT>::vmax_key(q, invT);
         kbest = k > kbest ? k : kbest;
-        nfin += (uint32_t)Elem<DT>::PER_VEC - VecTest<DT>::count_neginf(q);
+        nfin += (uint32_t)Elem<DT>::PER_VEC - VecTest<DT>::count_not_finite(q, fin_thr, invT);
     });
     src.extras([&](int, float z) {
         const uint32_t k = key_of(z);

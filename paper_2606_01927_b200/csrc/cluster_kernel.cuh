@@ -210,6 +210,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     if (threadIdx.x == 0) fill_general_args(s.ga, a);
     __syncthreads();
 
+    const uint32_t fin_thr = T::finite_threshold(c.invT);       // (while the slice travels)
     // the slice: penalised tokens and (CTA 0) the row's unaligned ends move to the list of extras
     bool landed = true, fits = true;
     int nx = 0;
@@ -250,7 +251,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
         src.vectors([&](const uint4 &q, int) {
             const uint32_t kk = T::vmax_key(q, c.invT);
             mk = kk > mk ? kk : mk;
-            nfin += (uint32_t)E::PER_VEC - T::count_neginf(q);
+            nfin += (uint32_t)E::PER_VEC - T::count_not_finite(q, fin_thr, c.invT);
         });
         src.extras([&](int, float z) {
             const uint32_t kk = key_of(z);

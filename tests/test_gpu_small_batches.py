@@ -166,3 +166,25 @@ def test_lists_longer_than_what_carries_mass(binding, sampler, B, cut, near):
     _, ref = check(binding, sampler, w, flags=binding.FLAG_LOGPROB_FULL_VOCAB if w.logprob_full_vocab else 0)
     if cut != "topp":
         assert (ref.top_ids >= 0).all()
+
+
+@pytest.mark.parametrize("B", [6, 76])
+@pytest.mark.parametrize("dtype", [W.F32, W.BF16])
+@pytest.mark.parametrize("T", [0.5, 1.0, 1.7])
+@pytest.mark.parametrize("flags", [0, 1], ids=["auto", "general"])
+def test_masks_of_the_lowest_value(binding, sampler, B, dtype, T, flags):
+    """Tokens masked with the type's lowest finite value: below T = 1 their scores leave the fp32 range and are
+    not among the finite ones; sizes of the kept set and of the top-k stage are the oracle's."""
+    V = 20003
+    rng = np.random.default_rng(43)
+    x = rng.standard_normal((B, V)).astype(np.float32)
+    low = np.float32(-3.4028234663852886e38 if dtype == W.F32 else -3.3895313892515355e38)
+    x[rng.random((B, V)) < 0.9] = low
+    x[0] = low
+    x[0, 4321] = 1.0
+    p = np.where(np.arange(B) % 3 == 0, 1.0, 0.9).astype(np.float32)
+    w = W.Workload("masked", B, V, dtype, x if dtype == W.F32 else W.f32_to_bf16_bits(x), temperature=np.full(B, T, np.float32),
+                   top_p=p, seeds=np.arange(B, dtype=np.uint64))
+    g, ref = check(binding, sampler, w, flags=flags)
+    assert (g["num_topk"] == ref.rows["n_topk"]).all()
+    assert (g["num_kept"][p == 1.0] == ref.rows["n_keep"][p == 1.0]).all()
