@@ -995,12 +995,12 @@ __device__ __forceinline__ void general_path(BlockScratch &s, const HistBins &h,
         hist_clear(h);
         __syncthreads();
         for_each_score<DT>(c, [&](int, float z) {
-            const float d = __fsub_rn(zmax, z);               // >= 0 for finite z; inf / NaN otherwise
-            if (d < 3.0e38f) {
-                int q = __float2int_rz(d * BIN_SCALE);
-                q = q > HIST_BINS - 1 ? HIST_BINS - 1 : q;
+            // (every finite score: those furthest down, such as masks of the type's lowest value, are in the last bin)
+            const uint32_t kk = key_of(z);
+            if (kk >= KEY_MIN_FINITE && kk < KEY_POS_INF) {
+                const int q = bin_of(z, zmax);
                 if (with_cnt) atomicAdd(&h.cnt[q], 1u);
-                if (with_mass) { const u64 e = mass_gen(-d); if (e) hist_add_mass(h, q, e); }
+                if (with_mass) { const u64 e = mass_gen(__fsub_rn(z, zmax)); if (e) hist_add_mass(h, q, e); }
             }
         });
         __syncthreads();

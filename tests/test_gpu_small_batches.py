@@ -188,3 +188,22 @@ def test_masks_of_the_lowest_value(binding, sampler, B, dtype, T, flags):
     g, ref = check(binding, sampler, w, flags=flags)
     assert (g["num_topk"] == ref.rows["n_topk"]).all()
     assert (g["num_kept"][p == 1.0] == ref.rows["n_keep"][p == 1.0]).all()
+
+
+@pytest.mark.parametrize("B", [6, 76])
+@pytest.mark.parametrize("dtype", [W.F32, W.BF16])
+@pytest.mark.parametrize("cut", ["none", "topk", "full"])
+@pytest.mark.parametrize("flags", [0, 1], ids=["auto", "general"])
+def test_lists_and_top_k_reach_into_masks_of_the_lowest_value(binding, sampler, B, dtype, cut, flags):
+    """More entries wanted than tokens are left unmasked: the masked ones follow in the order of their ids."""
+    V = 20003
+    rng = np.random.default_rng(44)
+    x = np.full((B, V), -3.4028234663852886e38 if dtype == W.F32 else -3.3895313892515355e38, np.float32)
+    for b in range(B):
+        x[b, rng.permutation(V)[:1 + b % 7]] = rng.standard_normal(1 + b % 7).astype(np.float32)
+    w = W.Workload("masked", B, V, dtype, x if dtype == W.F32 else W.f32_to_bf16_bits(x), temperature=np.ones(B, np.float32),
+                   top_k=np.full(B, 30 if cut == "topk" else 0, np.int32), seeds=np.arange(B, dtype=np.uint64))
+    w.num_top = 20
+    w.logprob_full_vocab = cut == "full"
+    g, ref = check(binding, sampler, w, flags=flags | (binding.FLAG_LOGPROB_FULL_VOCAB if cut == "full" else 0))
+    assert (g["num_kept"] == ref.rows["n_keep"]).all() and (ref.top_ids >= 0).all()
