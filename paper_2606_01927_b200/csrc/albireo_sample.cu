@@ -761,11 +761,33 @@ __device__ __forceinline__ u64 mass_gen(float d) {
     return d < -28.5f ? 0ull : __float2ull_rn(__expf(d) * FX_SCALE);
 }
 
+// A thread's sum of masses, independent of their order and grouping: each mass e <= 1 is rounded to a multiple of
+// 2^-40 by itself (to the integer that mass_gen gives) and added as two integers, multiples of 2^-20 and of 2^-40.
+// Adding a power of two that makes the unit the last place rounds, the difference from it is exact: four additions
+// and two integer ones per mass, where a conversion to 64 bits and its addition would be twice that.  Good for 2^11
+// masses (a thread sees at most 2^20 / NT).
+struct MassSum {
+    uint32_t hi = 0, lo = 0;                     // (lo: signed)
+    __device__ __forceinline__ void add(float e) {
+        const float t = __fadd_rn(e, 8.0f);                                                             // last place 2^-20
+        const float r = __fadd_rn(__fsub_rn(e, __fsub_rn(t, 8.0f)), 1.1444091796875e-5f);               // 1.5 * 2^-17: last place 2^-40
+        hi += __float_as_uint(t) - 0x41000000u;
+        lo += __float_as_uint(r) - 0x37400000u;
+    }
+    __device__ __forceinline__ void add2(float2 e) {      // two at once: the additions in pairs
+        const float2 t = __fadd2_rn(e, make_float2(8.0f, 8.0f));
+        const float2 back = __ffma2_rn(t, make_float2(-1.0f, -1.0f), make_float2(8.0f, 8.0f));
+        const float2 r = __fadd2_rn(__fadd2_rn(e, back), make_float2(1.1444091796875e-5f, 1.1444091796875e-5f));
+        hi += __float_as_uint(t.x) + __float_as_uint(t.y) - 2u * 0x41000000u;
+        lo += __float_as_uint(r.x) + __float_as_uint(r.y) - 2u * 0x37400000u;
+    }
+    __device__ __forceinline__ u64 total() const { return ((u64)hi << 20) + (u64)(int64_t)(int32_t)lo; }
+};
+
 // Mass of the whole row, sum of exp(z - zmax) over its finite scores in 2^40 fixed point: the
 // normaliser of the log-probabilities in the full-vocabulary mode.  One more pass over the row (it
 // was just read, so mostly from L2), four loads in flight; vectors with nothing within 29 of the
-// maximum carry no mass and are skipped by the packed test of the candidate path; the masses of a
-// vector are added in fp32 (a fixed order) and turned into fixed point once.  The same in every thread.
+// maximum carry no mass and are skipped by the packed test of the candidate path.  The same in every thread.
 template <int DT>
 __device__ u64 full_vocab_mass(BlockScratch &s, const RowCtx &c, float zmax) {
     typedef Elem<DT> E;
@@ -777,6 +799,7 @@ __device__ u64 full_vocab_mass(BlockScratch &s, const RowCtx &c, float zmax) {
     const int nvec = (V - head) / E::PER_VEC;
     const uint4 *vp = (const uint4 *)((const char *)c.row + (size_t)head * E::SIZE);
     const uint32_t thr = T::raw_threshold(key_of(zmax - 29.0f), c.invT);
+    MassSum sum;
     u64 local = 0;
     for (int v0 = threadIdx.x; v0 < nvec; v0 += 4 * NT) {
         uint4 q[4];
@@ -790,20 +813,18 @@ __device__ u64 full_vocab_mass(BlockScratch &s, const RowCtx &c, float zmax) {
             const int i0 = head + v * E::PER_VEC;
             uint32_t m = 0;
             if (c.has_hist) m = __funnelshift_r(c.bitmap[i0 >> 5], c.bitmap[(i0 >> 5) + 1], i0 & 31);
-            float acc = 0.0f;
 #pragma unroll
             for (int e = 0; e < E::PER_VEC; ++e) {
                 const float d = __fsub_rn(__fmul_rn(E::get(q[u], e), c.invT), zmax);
-                if (!((m >> e) & 1u) && d >= -28.5f) acc += __expf(d);
+                if (!((m >> e) & 1u) && d >= -28.5f) sum.add(__expf(d));
             }
-            local += __float2ull_rn(acc * FX_SCALE);
         }
     }
     for_each_score_rest<DT>(c, head, nvec, [&](int, float z) {
         const float d = __fsub_rn(z, zmax);
         if (d > -3.0e38f) local += mass_gen(d);         // -inf (and NaN) carry no mass
     });
-    return block_sum_u64(s, local);
+    return block_sum_u64(s, local + sum.total());
 }
 
 // value-linear bin of a finite score z <= zmax; monotone: a larger z never gets a larger bin

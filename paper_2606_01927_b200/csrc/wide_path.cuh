@@ -262,6 +262,14 @@ constexpr int W_LIST_ALONE = 2 * W_LIST;               // entries of the window'
 
 __device__ __forceinline__ float ex2_ftz(float t) { float e; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(t)); return e; }
 __device__ __forceinline__ float log2_mass(float z, float zmax) { return __fmul_rn(__fsub_rn(z, zmax), 1.4426950408889634f); }
+// (of two elements: one rounding per step as well, so the same bits)
+__device__ __forceinline__ float2 log2_mass2(float2 z, float zmax) {
+    return __fmul2_rn(__fadd2_rn(z, make_float2(-zmax, -zmax)), make_float2(1.4426950408889634f, 1.4426950408889634f));
+}
+__device__ __forceinline__ uint2 code_of2(float2 t2) {
+    const float2 c = __ffma2_rn(t2, make_float2(-65536.0f, -65536.0f), make_float2(8388608.0f, 8388608.0f));
+    return make_uint2(__float_as_uint(c.x), __float_as_uint(c.y));
+}
 __device__ __forceinline__ uint32_t code_of(float t2) { return __float_as_uint(__fmaf_rn(t2, -65536.0f, 8388608.0f)); }
 // A bin's masses are added up as 12-bit fractions of the bin's octave (at most 2^19 elements: no
 // overflow).  `octave_code` = code >> 16 carries the magic exponent, which turns into the sign bit.
@@ -269,7 +277,7 @@ __device__ __forceinline__ uint32_t mass12(float e, uint32_t octave_code) {
     const float neg = __uint_as_float(__float_as_uint(e) + (octave_code << 23));
     return __float_as_uint(2048.0f - neg) - 0x45000000u;
 }
-__device__ __forceinline__ u64 mass_of_bin(uint32_t q, uint32_t octave) { return octave < 52u ? ((u64)q << 20) >> octave : 0ull; }   // 2^-32 units
+__device__ __forceinline__ u64 mass_of_bin(uint32_t q, uint32_t octave) { return octave < 60u ? ((u64)q << 28) >> octave : 0ull; }   // 2^-40 units
 // hist[bin] += v if bin < W_BINS, without a branch
 __device__ __forceinline__ void hist_add_if(uint32_t hist_addr, uint32_t bin, uint32_t v) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p red.shared.add.u32 [%0], %3;\n\t}"
@@ -312,37 +320,32 @@ template <int DT, int MODE, bool FLOOR, class SRC>
 __device__ __forceinline__ void mass_pass(const SRC &src, float invT, float zmax, float zfloor, uint32_t lo, int shift, u64 &S_out, u64 &S_all_out) {
     typedef Elem<DT> E;
     const uint32_t hist = smem_u32(wide_smem().hist);
-    u64 S = 0, S_all = 0;
-    auto add = [&](float z, float &acc, float &all) {
-        const float t2 = log2_mass(z, zmax);
-        const float e = ex2_ftz(t2);
-        uint32_t f = code_of(t2);
-        if (FLOOR) {
-            all += e;
-            const bool in = z >= zfloor;
-            if (MODE != INSIDE_WINDOW) acc += in ? e : 0.0f;
-            f = in ? f : 0xFFFFFFFFu;
-        } else if (MODE != INSIDE_WINDOW) acc += e;
-        if (MODE == INSIDE_WINDOW) acc += f < lo ? e : 0.0f;
+    MassSum S, S_all;
+    // an element's place in the histogram, and whether its mass counts towards S
+    auto place = [&](float z, float e, uint32_t f) -> bool {
+        bool in = true;
+        if (FLOOR) { in = z >= zfloor; f = in ? f : 0xFFFFFFFFu; }
+        if (MODE == INSIDE_WINDOW) in = f < lo;
         if (MODE == FIRST_LEVEL) hist_add_if(hist, (f >> W_SHIFT) - (F_ZERO >> W_SHIFT), mass12(e, f >> 16));
         if (MODE == INSIDE_WINDOW) hist_add_if(hist, f >= lo ? (f - lo) >> shift : 0xFFFFFFFFu, mass12(e, f >> 16));
+        return in;
+    };
+    auto add2 = [&](float2 z) {
+        const float2 t2 = log2_mass2(z, zmax);
+        const float2 e = make_float2(ex2_ftz(t2.x), ex2_ftz(t2.y));
+        const uint2 f = code_of2(t2);
+        const bool in0 = place(z.x, e.x, f.x), in1 = place(z.y, e.y, f.y);
+        S.add2(make_float2(in0 ? e.x : 0.0f, in1 ? e.y : 0.0f));
+        if (FLOOR && MODE != INSIDE_WINDOW) S_all.add2(e);
     };
     const uint32_t thr = VecTest<DT>::raw_threshold(key_of(zmax - 29.5f), invT);
     src.vectors([&](const uint4 &q, int) {
         if (!VecTest<DT>::may_pass(q, thr, invT)) return;          // nothing within 42 octaves of the maximum
-        float acc = 0.0f, all = 0.0f;
 #pragma unroll
-        for (int j = 0; j < E::PER_VEC; ++j) add(__fmul_rn(E::get(q, j), invT), acc, all);
-        S += __float2ull_rn(acc * FX_SCALE);
-        if (FLOOR) S_all += __float2ull_rn(all * FX_SCALE);
+        for (int j = 0; j < E::PER_VEC; j += 2) add2(__fmul2_rn(make_float2(E::get(q, j), E::get(q, j + 1)), make_float2(invT, invT)));
     });
-    src.extras([&](int, float z) {
-        float acc = 0.0f, all = 0.0f;
-        add(z, acc, all);
-        S += __float2ull_rn(acc * FX_SCALE);
-        if (FLOOR) S_all += __float2ull_rn(all * FX_SCALE);
-    });
-    S_out = S; S_all_out = FLOOR ? S_all : S;
+    src.extras([&](int, float z) { add2(make_float2(z, -INFINITY)); });
+    S_out = S.total(); S_all_out = FLOOR ? S_all.total() : S_out;
 }
 
 // The passes out of line, for the kernel that has 64 registers per thread: each gets them all to itself.
@@ -357,7 +360,7 @@ __device__ __noinline__ PassOut solo_mass_pass(float invT, float zmax, float zfl
 // One level of the search: where the running total of the team's histogram (masses, or lower bounds of
 // the element counts) reaches its target, give or take the rounding of the histogram: 2^-slack_shift of
 // its total on both sides, or so many elements (targets beyond the total are cut down to it).  On the first level of a search
-// by mass the target is the share `frac` of the histogram's own total.
+// by mass the target is the share `frac` of the histogram's own total.  (A bin's mass is cut off at 2^-40: W_BINS units at most.)
 struct Window {
     uint32_t lo, hi;      // codes, both inclusive
     uint32_t id_lo, id_hi;      // of the elements with code lo only ids from id_lo on, of those with code hi only up to id_hi
@@ -367,7 +370,7 @@ struct Window {
     bool found;
 };
 template <class TEAM>
-__device__ __noinline__ Window find_window(BlockScratch *sp, TEAM tm, bool by_count, uint32_t base, int shift, double frac, u64 target, int slack_shift, u64 least_slack = 0) {
+__device__ __noinline__ Window find_window(BlockScratch *sp, TEAM tm, bool by_count, uint32_t base, int shift, double frac, u64 target, int slack_shift) {
     BlockScratch &s = *sp;
     uint32_t *hist = wide_smem().hist;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -406,8 +409,7 @@ __device__ __noinline__ Window find_window(BlockScratch *sp, TEAM tm, bool by_co
     u64 run = warp_total(lane < wid ? wt : 0ull) + inc - local;
     uint32_t crun = __reduce_add_sync(0xFFFFFFFFu, lane < wid ? wc : 0u) + cinc - cnt;
     if (frac > 0.0) target = (u64)(frac * (double)tot);
-    u64 slack = by_count ? (u64)slack_shift : (tot >> slack_shift) + 1;
-    slack = slack > least_slack ? slack : least_slack;
+    const u64 slack = by_count ? (u64)slack_shift : (tot >> slack_shift) + W_BINS;
     u64 t_lo = target > slack ? target - slack : 1, t_hi = target + slack;
     if (t_hi > tot) t_hi = tot;
     if (t_lo < 1) t_lo = 1;
@@ -444,13 +446,13 @@ template <int DT, class SRC>
 __device__ __noinline__ void tie_pass(SRC src, float invT, float zmax, float zfloor, uint32_t lo, uint32_t hi, u64 &ahead, uint32_t &kmin, uint32_t &kmax) {
     typedef Elem<DT> E;
     const uint32_t hist = smem_u32(wide_smem().hist);
-    u64 S = 0;
+    MassSum S;
     uint32_t mn = 0xFFFFFFFFu, mx = 0;
-    auto see = [&](int i, float z, float &acc) {
+    auto see = [&](int i, float z) {
         const float t2 = log2_mass(z, zmax);
         const uint32_t f = code_of(t2);
         if (!(z >= zfloor)) return;
-        acc += f < lo ? ex2_ftz(t2) : 0.0f;
+        S.add(f < lo ? ex2_ftz(t2) : 0.0f);
         if (f >= lo && f <= hi) {
             const uint32_t k = key_of(z);
             mn = k < mn ? k : mn; mx = k > mx ? k : mx;
@@ -458,13 +460,11 @@ __device__ __noinline__ void tie_pass(SRC src, float invT, float zmax, float zfl
         }
     };
     src.vectors([&](const uint4 &q, int i0) {
-        float acc = 0.0f;
 #pragma unroll
-        for (int j = 0; j < E::PER_VEC; ++j) see(i0 + j, __fmul_rn(E::get(q, j), invT), acc);
-        S += __float2ull_rn(acc * FX_SCALE);
+        for (int j = 0; j < E::PER_VEC; ++j) see(i0 + j, __fmul_rn(E::get(q, j), invT));
     });
-    src.extras([&](int i, float z) { float acc = 0.0f; see(i, z, acc); S += __float2ull_rn(acc * FX_SCALE); });
-    ahead = S; kmin = mn; kmax = mx;
+    src.extras([&](int i, float z) { see(i, z); });
+    ahead = S.total(); kmin = mn; kmax = mx;
 }
 // Narrows a window until no more than `cap` elements can be in it (or the codes run out).  The pass over
 // the elements also gives the exact mass ahead of the window, so that the histogram's rounding counts
@@ -531,10 +531,8 @@ __device__ __noinline__ bool narrow_window(BlockScratch *sp, SRC src, TEAM tm, f
         tm.sync();
         ahead = warp_total(lane < tm.size ? tm.x->ahead[lane] : 0ull);
         const u64 before = w.before;
-        const u64 rest = by_count ? target - before : (target > ahead ? (target - ahead) >> 8 : 1ull);
-        // (2^-22 of the whole: a vector's masses are added in fp32 here and one by one in the last pass, and far
-        // down a tail that difference is the mass of many elements)
-        w = find_window(sp, tm, by_count, w.lo, shift, 0.0, rest, by_count ? 0 : 11, by_count ? 0ull : (target >> 30) + 1);
+        const u64 rest = by_count ? target - before : (target > ahead ? target - ahead : 1ull);
+        w = find_window(sp, tm, by_count, w.lo, shift, 0.0, rest, by_count ? 0 : 11);
         if (!w.found) return false;
         w.before += before;                              // (a count; by mass the next level measures it anew)
     }
@@ -611,7 +609,7 @@ __device__ __forceinline__ void race_all(const SRC &src, BlockScratch &s, Partia
     const uint64_t seed = s.fa.seed, step = s.fa.step;
     const uint32_t R = s.fa.R;
     const uint32_t sure = CUT ? s.fa.sure : 0u, win_hi = CUT ? s.fa.win_hi : 0u;
-    u64 S = 0;
+    MassSum S;
     uint32_t n = 0;
     Racer rc;
     rc.start();
@@ -620,29 +618,27 @@ __device__ __forceinline__ void race_all(const SRC &src, BlockScratch &s, Partia
         const FinalArgs &fa = s.fa;
         if (!(z >= fa.zfloor)) return;
         if (f == sure && (uint32_t)i < fa.id_lo) {
-            S += __float2ull_rn(ex2_ftz(t2) * FX_SCALE); ++n;
+            S.add(ex2_ftz(t2)); ++n;
             const uint32_t w = race_word(seed, R, step, i);
             if (unit_above(w) <= __fmaf_rn(ex2_ftz(t2), rc.K, 1.0f)) rc.take(best, i, z, __fsub_rn(z, zmax) + nle_once(w));
         } else if (f < win_hi || (f == win_hi && (uint32_t)i <= fa.id_hi)) list_append(fa.list, fa.list_cap, &s.list_cnt, z, i);
     };
     src.vectors([&](const uint4 &q, int i0) {
-        float e[PV], acc = 0.0f, top = 0.0f;
+        float e[PV], top = 0.0f;
         uint32_t at_edge = 0;
 #pragma unroll
-        for (int j = 0; j < PV; ++j) {
-            const float t2 = log2_mass(__fmul_rn(E::get(q, j), invT), zmax);
-            e[j] = ex2_ftz(t2);
+        for (int j = 0; j < PV; j += 2) {
+            const float2 t2 = log2_mass2(__fmul2_rn(make_float2(E::get(q, j), E::get(q, j + 1)), make_float2(invT, invT)), zmax);
+            e[j] = ex2_ftz(t2.x); e[j + 1] = ex2_ftz(t2.y);
             if constexpr (CUT) {
-                const uint32_t f = code_of(t2);
-                at_edge |= (uint32_t)(f >= sure && f <= win_hi) << j;
-                const bool in = f < sure;
-                e[j] = in ? e[j] : 0.0f;
-                n += in;
+                const uint2 f = code_of2(t2);
+                at_edge |= (uint32_t)(f.x >= sure && f.x <= win_hi) << j | (uint32_t)(f.y >= sure && f.y <= win_hi) << (j + 1);
+                e[j] = f.x < sure ? e[j] : 0.0f; e[j + 1] = f.y < sure ? e[j + 1] : 0.0f;
+                n += (f.x < sure) + (f.y < sure);
             }
-            acc += e[j];
-            top = fmaxf(top, e[j]);
+            S.add2(make_float2(e[j], e[j + 1]));
+            top = fmaxf(top, fmaxf(e[j], e[j + 1]));
         }
-        S += __float2ull_rn(acc * FX_SCALE);
         if constexpr (CUT) {
             while (at_edge) {
                 const int x = __ffs(at_edge) - 1;
@@ -682,11 +678,11 @@ __device__ __forceinline__ void race_all(const SRC &src, BlockScratch &s, Partia
         bool in = true;
         if constexpr (CUT) in = f < sure;
         if (in) {
-            S += __float2ull_rn(ex2_ftz(t2) * FX_SCALE); ++n;
+            S.add(ex2_ftz(t2)); ++n;
             rc.take(best, i, z, d + race_nle(seed, R, step, nullptr, i));
         } else if (f <= win_hi) edge(i, z, t2, f);        // (CUT only)
     });
-    p.M = S; p.n = CUT ? n : 0; p.G = rc.G; p.z = rc.z;
+    p.M = S.total(); p.n = CUT ? n : 0; p.G = rc.G; p.z = rc.z;
 }
 
 // Mass, number and race of the elements kept for sure, and the lists (arguments in s.fa).  Kept elements
@@ -1034,13 +1030,13 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
                 reach = ahead + own;
                 if (ahead < target) keep(C, own);
             }
-            reached = __syncthreads_or(reach + (1ull << 18) >= target) != 0;
+            reached = __syncthreads_or(reach >= target) != 0;
         } else {
             const int P = list_sort(list, L), per = (P + NT - 1) / NT, q0 = (int)threadIdx.x * per, q1 = min(L, q0 + per);
             u64 local = 0, tot;
             for (int q = q0; q < q1; ++q) local += mass_of(list[q]);
             u64 run = p.M + block_exscan_u64(s, local, tot);
-            reached = p.M + tot + (1ull << 18) >= target;
+            reached = p.M + tot >= target;
 #pragma unroll 1
             for (int q = q0; q < q1 && run < target; ++q) {
                 const u64 C = list[q], own = mass_of(C);
@@ -1049,7 +1045,6 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
             }
             __syncthreads();
         }
-        // (short of the target by no more than the rounding of the sums: the whole list stays)
         if (!reached) { out.status |= ROW_NOT_DONE; return out; }
         block_partial(s, k);
         p.M += k.M; p.n += k.n;

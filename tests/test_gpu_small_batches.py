@@ -207,3 +207,31 @@ def test_lists_and_top_k_reach_into_masks_of_the_lowest_value(binding, sampler, 
     w.logprob_full_vocab = cut == "full"
     g, ref = check(binding, sampler, w, flags=flags | (binding.FLAG_LOGPROB_FULL_VOCAB if cut == "full" else 0))
     assert (g["num_kept"] == ref.rows["n_keep"]).all() and (ref.top_ids >= 0).all()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("cut", ["topp", "none", "minp_topp", "topp_full", "topk_full"])
+def test_results_do_not_depend_on_where_a_row_lies(binding, sampler, dtype, cut):
+    """The same rows in batches of other sizes (one CTA per row, clusters of several sizes) and on other offsets from
+    the 16-byte grid, with cuts down the tail where an element weighs 1e-6 of the sum: sums are of integers, so
+    tokens, kept sizes and log-probabilities are the same bit for bit."""
+    B, V = 96, 40009
+    g = torch.Generator(device=sampler.device).manual_seed(5)
+    x = (torch.randn((B, V), generator=g, device=sampler.device) * 1.5).to(dtype)
+    par = dict(temperature=torch.full((B,), 0.9, device=sampler.device), seeds=torch.arange(B, device=sampler.device) * 7 + 1)
+    if "topp" in cut:
+        par["top_p"] = (1.0 - torch.logspace(-1, -4, B, device=sampler.device)).float()
+    if "minp" in cut:
+        par["min_p"] = torch.full((B,), 1e-4, device=sampler.device)
+    if "topk" in cut:
+        par["top_k"] = torch.full((B,), 30, dtype=torch.int32, device=sampler.device)
+    flags = binding.FLAG_LOGPROB_FULL_VOCAB if cut.endswith("full") else 0
+    whole = to_host(sampler.albireo_sample(x, **par, want_counts=True, flags=flags))
+    for lo, n, shift in [(0, 96, 3), (0, 5, 0), (5, 9, 1), (14, 17, 7), (30, 36, 2), (22, 74, 5)]:
+        buf = torch.zeros((n * (V + shift) + 8,), dtype=dtype, device=sampler.device)
+        view = buf[shift:shift + n * (V + shift)].view(n, V + shift)[:, :V]
+        view.copy_(x[lo:lo + n])
+        part = to_host(sampler.albireo_sample(view, **{k: v[lo:lo + n] for k, v in par.items()}, row_base=lo, want_counts=True, flags=flags))
+        for f in ("tokens", "num_kept", "num_topk"):
+            assert (part[f] == whole[f][lo:lo + n]).all(), (f, lo, n, shift)
+        assert (part["logprobs"].view(np.uint32) == whole["logprobs"][lo:lo + n].view(np.uint32)).all(), (lo, n, shift)
