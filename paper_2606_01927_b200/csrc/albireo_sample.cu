@@ -1773,7 +1773,7 @@ __device__ __noinline__ void whole_row_totals(BlockScratch *sp, float zmax) {
     __syncthreads();
 }
 
-// From the candidate list cand[0..n) (every element of the row with key >= tau_key) to the result.
+// From the candidate list cand[0..n) (every element of the row with key >= tau_key, the same in every thread) to the result.
 // `full_fx` != 0: the mass of the whole row, which the log-probabilities are relative to.  `count_finite`
 // is called, by every thread, only where the number of finite scores is asked for and not known.
 // EXTRA: see albireo_sample_kernel.
@@ -2113,7 +2113,11 @@ __device__ __forceinline__ bool candidate_path(BlockScratch &s, const CandSmem &
         if (s.timeout) { out.status |= ALBIREO_ROW_TIMEOUT; out.token = -1; out.logprob = __uint_as_float(0x7FC00000u); out.n_keep = 0; out.n_topk = 0; return true; }
         __syncthreads();
     }
-    return candidate_finish<EXTRA>(s, cs, n, tau_key, kmax, rp, a, b, out, full_fx, [&]() -> u64 {
+    // (tau_key differs from warp to warp, each with the min-p floor it has seen: the block-wide steps from here on
+    // take the floor of the row's maximum)
+    uint32_t tau = tau_topk;
+    if (has_topk && stream_minp) tau = max(tau, min(kmax, minp_key(unkey(kmax), rp.ln_min_p)));
+    return candidate_finish<EXTRA>(s, cs, n, tau, kmax, rp, a, b, out, full_fx, [&]() -> u64 {
         if (!EXTRA) return 0ull;
         totals();
         return s.bcast[1];

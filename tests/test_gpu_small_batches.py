@@ -235,3 +235,26 @@ def test_results_do_not_depend_on_where_a_row_lies(binding, sampler, dtype, cut)
         for f in ("tokens", "num_kept", "num_topk"):
             assert (part[f] == whole[f][lo:lo + n]).all(), (f, lo, n, shift)
         assert (part["logprobs"].view(np.uint32) == whole["logprobs"][lo:lo + n].view(np.uint32)).all(), (lo, n, shift)
+
+
+@pytest.mark.parametrize("dtype", [W.F32, W.BF16])
+@pytest.mark.parametrize("extras", [True, False])
+def test_top_k_with_a_min_p_floor_that_rises(binding, sampler, dtype, extras):
+    """A long candidate list cut at the k-th largest key while the warps have seen different min-p floors."""
+    B, V = 120, 68066
+    rng = np.random.default_rng(47)
+    x = (rng.standard_normal((B, V))).astype(np.float32)
+    x[rng.random((B, V)) > 0.02] = -np.inf
+    w = W.Workload("topk_minp", B, V, dtype, x if dtype == W.F32 else W.f32_to_bf16_bits(x), temperature=np.ones(B, np.float32),
+                   top_k=np.full(B, 200, np.int32), min_p=np.full(B, 0.04, np.float32), top_p=np.linspace(0.3, 0.95, B).astype(np.float32),
+                   seeds=np.arange(B, dtype=np.uint64))
+    w.num_top = 100
+    if extras:
+        g, ref = check(binding, sampler, w)
+        assert (g["num_kept"] == ref.rows["n_keep"]).sum() >= B - 2
+        return
+    ref = O.sample(w, threads=_CORES)
+    t = binding.workload_tensors(w, sampler.device)
+    g = to_host(sampler.albireo_sample(t.pop("logits"), **t, num_top=w.num_top))
+    rep = compare(w, g, ref)
+    assert rep.ok() and len(rep.excused) <= 1, (rep.summary(), rep.failures[:3])
