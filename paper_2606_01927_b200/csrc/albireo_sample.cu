@@ -761,23 +761,41 @@ __device__ __forceinline__ u64 mass_gen(float d) {
     return d < -28.5f ? 0ull : __float2ull_rn(__expf(d) * FX_SCALE);
 }
 
+// Arithmetic on two values at once.  A product and a sum that follows it are contracted in this form even with
+// explicit rounding (seen in the results, nvcc 12.9); a score is a rounded product, and scores_of makes it as a
+// product plus a -0 that the compiler does not know to be one.
+__device__ __forceinline__ float2 pair_of(float x) { return make_float2(x, x); }
+__device__ __forceinline__ u64 pair_bits(float2 a) { u64 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y)); return r; }
+__device__ __forceinline__ float2 bits_pair(u64 a) { float2 r; asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a)); return r; }
+__device__ __forceinline__ float2 add_pair(float2 a, float2 b) {
+    u64 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pair_bits(a)), "l"(pair_bits(b))); return bits_pair(r);
+}
+__device__ __forceinline__ float2 mul_pair(float2 a, float2 b) {
+    u64 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pair_bits(a)), "l"(pair_bits(b))); return bits_pair(r);
+}
+__device__ __forceinline__ float2 fma_pair(float2 a, float2 b, float2 c) {
+    u64 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pair_bits(a)), "l"(pair_bits(b)), "l"(pair_bits(c))); return bits_pair(r);
+}
+__device__ __forceinline__ float minus_zero(float invT) { return __fmul_rn(fminf(invT, 1.0f), -0.0f); }
+__device__ __forceinline__ float2 scores_of(float x, float y, float invT, float minus0) { return fma_pair(make_float2(x, y), pair_of(invT), pair_of(minus0)); }
+
 // A thread's sum of masses, independent of their order and grouping: each mass e <= 1 is rounded to a multiple of
 // 2^-40 by itself (to the integer that mass_gen gives) and added as two integers, multiples of 2^-20 and of 2^-40.
-// Adding a power of two that makes the unit the last place rounds, the difference from it is exact: four additions
-// and two integer ones per mass, where a conversion to 64 bits and its addition would be twice that.  Good for 2^11
-// masses (a thread sees at most 2^20 / NT).
+// Adding a power of two that makes the unit the last place rounds, the difference from it is exact: three additions
+// (8 + C is a multiple of 2^-20 as well) and two integer ones per mass, in pairs, where a conversion to 64 bits and
+// its addition would be twice that.  Good for 2^11 masses (a thread sees at most 2^20 / NT).
 struct MassSum {
-    uint32_t hi = 0, lo = 0;                     // (lo: signed)
+    static constexpr float C = 1.1444091796875e-5f;       // 1.5 * 2^-17: last place 2^-40
+    uint32_t hi = 0, lo = 0;                             // (lo: signed)
     __device__ __forceinline__ void add(float e) {
-        const float t = __fadd_rn(e, 8.0f);                                                             // last place 2^-20
-        const float r = __fadd_rn(__fsub_rn(e, __fsub_rn(t, 8.0f)), 1.1444091796875e-5f);               // 1.5 * 2^-17: last place 2^-40
+        const float t = __fadd_rn(e, 8.0f);              // last place 2^-20
+        const float r = __fadd_rn(e, __fsub_rn(8.0f + C, t));
         hi += __float_as_uint(t) - 0x41000000u;
         lo += __float_as_uint(r) - 0x37400000u;
     }
-    __device__ __forceinline__ void add2(float2 e) {      // two at once: the additions in pairs
-        const float2 t = __fadd2_rn(e, make_float2(8.0f, 8.0f));
-        const float2 back = __ffma2_rn(t, make_float2(-1.0f, -1.0f), make_float2(8.0f, 8.0f));
-        const float2 r = __fadd2_rn(__fadd2_rn(e, back), make_float2(1.1444091796875e-5f, 1.1444091796875e-5f));
+    __device__ __forceinline__ void add2(float2 e) {
+        const float2 t = add_pair(e, pair_of(8.0f));
+        const float2 r = add_pair(e, fma_pair(t, pair_of(-1.0f), pair_of(8.0f + C)));
         hi += __float_as_uint(t.x) + __float_as_uint(t.y) - 2u * 0x41000000u;
         lo += __float_as_uint(r.x) + __float_as_uint(r.y) - 2u * 0x37400000u;
     }

@@ -264,10 +264,10 @@ __device__ __forceinline__ float ex2_ftz(float t) { float e; asm("ex2.approx.ftz
 __device__ __forceinline__ float log2_mass(float z, float zmax) { return __fmul_rn(__fsub_rn(z, zmax), 1.4426950408889634f); }
 // (of two elements: one rounding per step as well, so the same bits)
 __device__ __forceinline__ float2 log2_mass2(float2 z, float zmax) {
-    return __fmul2_rn(__fadd2_rn(z, make_float2(-zmax, -zmax)), make_float2(1.4426950408889634f, 1.4426950408889634f));
+    return mul_pair(add_pair(z, pair_of(-zmax)), pair_of(1.4426950408889634f));
 }
 __device__ __forceinline__ uint2 code_of2(float2 t2) {
-    const float2 c = __ffma2_rn(t2, make_float2(-65536.0f, -65536.0f), make_float2(8388608.0f, 8388608.0f));
+    const float2 c = fma_pair(t2, pair_of(-65536.0f), pair_of(8388608.0f));
     return make_uint2(__float_as_uint(c.x), __float_as_uint(c.y));
 }
 __device__ __forceinline__ uint32_t code_of(float t2) { return __float_as_uint(__fmaf_rn(t2, -65536.0f, 8388608.0f)); }
@@ -320,6 +320,7 @@ template <int DT, int MODE, bool FLOOR, class SRC>
 __device__ __forceinline__ void mass_pass(const SRC &src, float invT, float zmax, float zfloor, uint32_t lo, int shift, u64 &S_out, u64 &S_all_out) {
     typedef Elem<DT> E;
     const uint32_t hist = smem_u32(wide_smem().hist);
+    const float minus0 = minus_zero(invT);
     MassSum S, S_all;
     // an element's place in the histogram, and whether its mass counts towards S
     auto place = [&](float z, float e, uint32_t f) -> bool {
@@ -342,7 +343,7 @@ __device__ __forceinline__ void mass_pass(const SRC &src, float invT, float zmax
     src.vectors([&](const uint4 &q, int) {
         if (!VecTest<DT>::may_pass(q, thr, invT)) return;          // nothing within 42 octaves of the maximum
 #pragma unroll
-        for (int j = 0; j < E::PER_VEC; j += 2) add2(__fmul2_rn(make_float2(E::get(q, j), E::get(q, j + 1)), make_float2(invT, invT)));
+        for (int j = 0; j < E::PER_VEC; j += 2) add2(scores_of(E::get(q, j), E::get(q, j + 1), invT, minus0));
     });
     src.extras([&](int, float z) { add2(make_float2(z, -INFINITY)); });
     S_out = S.total(); S_all_out = FLOOR ? S_all.total() : S_out;
@@ -605,7 +606,7 @@ __device__ __forceinline__ void race_all(const SRC &src, BlockScratch &s, Partia
     typedef Elem<DT> E;
     constexpr int PV = E::PER_VEC, NB = PV / 4 + (OFF ? 1 : 0);
     uint32_t *best = &s.runmax;
-    const float invT = s.fa.invT, zmax = s.fa.zmax;
+    const float invT = s.fa.invT, zmax = s.fa.zmax, minus0 = minus_zero(invT);
     const uint64_t seed = s.fa.seed, step = s.fa.step;
     const uint32_t R = s.fa.R;
     const uint32_t sure = CUT ? s.fa.sure : 0u, win_hi = CUT ? s.fa.win_hi : 0u;
@@ -628,7 +629,7 @@ __device__ __forceinline__ void race_all(const SRC &src, BlockScratch &s, Partia
         uint32_t at_edge = 0;
 #pragma unroll
         for (int j = 0; j < PV; j += 2) {
-            const float2 t2 = log2_mass2(__fmul2_rn(make_float2(E::get(q, j), E::get(q, j + 1)), make_float2(invT, invT)), zmax);
+            const float2 t2 = log2_mass2(scores_of(E::get(q, j), E::get(q, j + 1), invT, minus0), zmax);
             e[j] = ex2_ftz(t2.x); e[j + 1] = ex2_ftz(t2.y);
             if constexpr (CUT) {
                 const uint2 f = code_of2(t2);

@@ -258,3 +258,20 @@ def test_top_k_with_a_min_p_floor_that_rises(binding, sampler, dtype, extras):
     g = to_host(sampler.albireo_sample(t.pop("logits"), **t, num_top=w.num_top))
     rep = compare(w, g, ref)
     assert rep.ok() and len(rep.excused) <= 1, (rep.summary(), rep.failures[:3])
+
+
+@pytest.mark.parametrize("B", [8, 80])
+@pytest.mark.parametrize("dtype", [W.F32, W.BF16])
+@pytest.mark.parametrize("cut", ["none", "topp", "topk_full"])
+def test_masses_of_scores_far_from_zero(binding, sampler, B, dtype, cut):
+    """Scores around 1000 / T, where the product with 1 / T is rounded by 1e-4 and more: a mass is that of the rounded
+    score (as everywhere else), not of the product before its rounding."""
+    V = 17011
+    rng = np.random.default_rng(53)
+    x = (1000.0 + rng.standard_normal((B, V)) * 3).astype(np.float32)
+    x[:, ::3] = np.round(x[:, ::3])
+    par = dict(none={}, topp=dict(top_p=np.full(B, 0.9, np.float32)), topk_full=dict(top_k=np.full(B, 20, np.int32)))[cut]
+    w = W.Workload("far", B, V, dtype, x if dtype == W.F32 else W.f32_to_bf16_bits(x),
+                   temperature=np.linspace(0.07, 1.3, B).astype(np.float32), seeds=np.arange(B, dtype=np.uint64), **par)
+    w.logprob_full_vocab = cut.endswith("full")
+    check(binding, sampler, w, flags=binding.FLAG_LOGPROB_FULL_VOCAB if w.logprob_full_vocab else 0)
