@@ -1018,7 +1018,7 @@ __device__ __forceinline__ void general_path(BlockScratch &s, const HistBins &h,
     auto top_id = [&]() -> int {
         uint32_t best = 0;
         for_each_score<DT>(c, [&](int i, float z) { if (key_of(z) == kmax) { const uint32_t v = ~(uint32_t)i; best = v > best ? v : best; } });
-        return (int)~(uint32_t)block_max_u64(s, best);
+        return max((int)~(uint32_t)block_max_u64(s, best), 0);         // (NaN: none equals the largest; an id in range all the same)
     };
 
     const bool full_lp = (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) != 0;
@@ -1225,7 +1225,7 @@ __device__ __forceinline__ void general_path(BlockScratch &s, const HistBins &h,
     const u64 S_fx = block_sum_u64(s, S_local);
     const u64 n_keep = block_sum_u64(s, n_local);
     const u64 G = block_max_u64(s, g_best);
-    const int tok = comp_idx(G);
+    const int tok = max(comp_idx(G), 0);                 // (+inf or NaN among the scores: possibly no winner)
     const double lnS = log((double)(full_lp ? full_vocab_mass<DT>(s, c, zmax) : S_fx)) - LN2_40;
     float z_tok = score_of(c, tok, Elem<DT>::load(elem_ptr<DT>(c, tok), 0));
     out.token = tok;                                   // (a single kept element wins its own race)

@@ -839,9 +839,10 @@ __device__ __forceinline__ u64 topp_target(float top_p, u64 S) {
     return target > S ? (S < 1 ? 1ull : S) : target;
 }
 
-// CTA 0: moves the entries that the others put at the far end of `buf` behind its own n0; returns the number of all.
+// CTA 0: moves the entries that the others put at the far end of `buf` behind its own n0; returns the number of all
+// (more than `cap`, which only +inf or NaN among the logits can bring about: nothing is moved).
 __device__ __forceinline__ int close_gap(u64 *buf, int cap, int n0, int nfar) {
-    if (nfar == 0) return n0;
+    if (nfar == 0 || n0 + nfar > cap) return n0 + nfar;
     u64 keep[W_LIST_ALONE / NT];
 #pragma unroll
     for (int q = 0; q < W_LIST_ALONE / NT; ++q) { const int j = threadIdx.x + q * NT; keep[q] = j < nfar ? buf[cap - 1 - j] : 0ull; }
@@ -1066,7 +1067,7 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
         __syncthreads();
         const double lnS_all = __longlong_as_double((long long)s.bcast[0]);
         const uint32_t members = full ? n_fin : s.found_cnt;
-        if ((uint32_t)n_all < min((uint32_t)s.ga.num_top, members)) { out.status |= ROW_NOT_DONE; return out; }      // (the same in every thread)
+        if ((uint32_t)n_all < min((uint32_t)s.ga.num_top, members) || n_all > W_LIST) { out.status |= ROW_NOT_DONE; return out; }      // (the same in every thread)
 #pragma unroll 1
         for (int j = threadIdx.x; j < n_all; j += NT) {
             const u64 C = ws.top[j];

@@ -275,3 +275,33 @@ def test_masses_of_scores_far_from_zero(binding, sampler, B, dtype, cut):
                    temperature=np.linspace(0.07, 1.3, B).astype(np.float32), seeds=np.arange(B, dtype=np.uint64), **par)
     w.logprob_full_vocab = cut.endswith("full")
     check(binding, sampler, w, flags=binding.FLAG_LOGPROB_FULL_VOCAB if w.logprob_full_vocab else 0)
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("cut", ["greedy", "topk", "topp", "minp", "none"])
+@pytest.mark.parametrize("B", [8, 80])
+def test_infinities_and_nan_give_a_token_in_range(binding, sampler, dtype, cut, B):
+    """Rows outside the contract (+inf, NaN, nothing finite): the token is unspecified but an id of the row."""
+    V = 33001
+    g = torch.Generator(device=sampler.device).manual_seed(3)
+    x = torch.randn((B, V), generator=g, device=sampler.device).to(dtype)
+    x[0] = float("nan")
+    x[1] = float("inf")
+    x[2] = -float("inf")
+    x[3, ::2] = float("inf")
+    x[4, ::3] = float("nan")
+    x[5, 7] = float("inf")
+    x[6, 33000] = float("nan")
+    x[7, :100] = float("inf")
+    x[7, 100:] = -float("inf")
+    par = dict(greedy=dict(temperature=torch.zeros(B, device=sampler.device)), none={},
+               topk=dict(top_k=torch.full((B,), 50, dtype=torch.int32, device=sampler.device)),
+               topp=dict(top_p=torch.full((B,), 0.9, device=sampler.device)),
+               minp=dict(min_p=torch.full((B,), 0.01, device=sampler.device)))[cut]
+    pad = torch.zeros((64 + B * V + 64,), dtype=dtype, device=sampler.device)
+    view = pad[64:64 + B * V].view(B, V)
+    view.copy_(x)
+    for flags in (0, binding.FLAG_FORCE_GENERAL, binding.FLAG_LOGPROB_FULL_VOCAB):
+        for num_top in (0, 20):
+            o = to_host(sampler.albireo_sample(view, **par, num_top=num_top, flags=flags))
+            assert ((o["tokens"] >= 0) & (o["tokens"] < V)).all(), (flags, num_top, o["tokens"])
+            if num_top:
+                assert ((o["top_ids"] >= -1) & (o["top_ids"] < V)).all(), (flags, num_top)
