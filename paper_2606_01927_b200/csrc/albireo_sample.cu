@@ -1749,7 +1749,12 @@ __device__ __forceinline__ void passes_begin(BlockScratch &s, const RowCtx &c, i
 #pragma unroll 1
     for (int q = 0; q < r.nst; ++q) { mbar_init(&r.bar[q], 1); r.done[q] = 0; }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    r.tiles = 0; r.timeout = 0; s.mm_max = 0; s.list_cnt = 0;
+    r.tiles = 0; r.issued = 0; r.timeout = 0; s.mm_max = 0; s.list_cnt = 0;
+}
+// The ring's barriers are done with (thread 0): their memory may be used for something else.
+__device__ __forceinline__ void passes_end() {
+    RowShared &r = row_shared();
+    for (int q = 0; q < r.nst; ++q) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(&r.bar[q])) : "memory");
 }
 // The row's largest order key (s.mm_max) and the number of its finite scores (s.list_cnt), after passes_begin.
 template <int DT>
@@ -1786,7 +1791,7 @@ __device__ __noinline__ void whole_row_totals(BlockScratch *sp, float zmax) {
         RowShared &r = row_shared();
         s.bcast[0] = S; s.bcast[1] = s.list_cnt;
         if (r.timeout) s.timeout = 1u;
-        for (int q = 0; q < r.nst; ++q) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(&r.bar[q])) : "memory");
+        passes_end();
     }
     __syncthreads();
 }
@@ -2246,6 +2251,8 @@ __device__ __noinline__ void leftover_row(BlockScratch *sp, const SampleArgs *ap
     if (out.status & ROW_NOT_DONE) {
         c = row_shared().c; rp = row_shared().rp;
         __syncthreads();                                       // the general path lays its own tables over them
+        if (threadIdx.x == 0) passes_end();
+        __syncthreads();
         out = general_path_call<DT>(sp, smem, c, rp, b, status);
     }
     store_row(a, b, out);

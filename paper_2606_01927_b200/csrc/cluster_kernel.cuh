@@ -291,6 +291,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
                             (distinct_row > (uint32_t)CNT_CAP && (int64_t)o0 + distinct_row > a.ws_counts_cap);
     bool done = false;
     if (bad & 0x80000000u) {
+        mbar_wait(bar, 0);                      // (a copy still in flight gets as long again before its memory is given up)
         out.status |= ALBIREO_ROW_TIMEOUT; out.token = -1; out.logprob = __uint_as_float(0x7FC00000u);
         done = true;
     } else if (!to_general) {
@@ -363,6 +364,8 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     if (tm.rank != 0) return;
     if (!done) {
         // the one-CTA path, from global memory, with tables over the whole row
+        __syncthreads();
+        if (threadIdx.x == 0) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
         __syncthreads();
         HistSmem hs;
         const int nw = (V + 31) >> 5, nc = (nw + 7) >> 3;

@@ -124,6 +124,7 @@ struct RowShared {
     const uint4 *vp;
     int head, nvec, vps, nst, tv; // stages of the ring, vectors per thread and tile
     uint32_t tiles;               // tiles of the passes so far
+    uint32_t issued;              // tiles of this pass whose copy has been issued
     uint32_t timeout;             // a wait on a copy expired
     uint32_t done[WIDE_MAX_STAGES];
     uint64_t bar[WIDE_MAX_STAGES];
@@ -143,7 +144,7 @@ struct RingSlice {
         ring_copy(rg, wide_stage(st * r.tv), r.vp, v0, nv, &r.bar[st]);
     }
     // The tiles of all passes are numbered through, which gives stage and phase; the last warp done with a
-    // stage refills it.  A wait that expires marks the row.
+    // stage refills it.  A wait that expires marks the row, and nothing more is copied.
     template <class F> __device__ __forceinline__ void vectors(F &&f) const {
         RowShared &r = row_shared();
         const uint32_t first = r.tiles;
@@ -152,9 +153,11 @@ struct RingSlice {
         int st = (int)(first % (uint32_t)nst);
         uint32_t parity = (first / (uint32_t)nst) & 1u;
         if (threadIdx.x == 0) {
+            const int npre = r.timeout ? 0 : min(ntiles, nst);
+            r.issued = (uint32_t)npre;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 #pragma unroll 1
-            for (int t = 0, q = st; t < min(ntiles, nst); ++t) { issue(r, t, q); q = q + 1 == nst ? 0 : q + 1; }
+            for (int t = 0, q = st; t < npre; ++t) { issue(r, t, q); q = q + 1 == nst ? 0 : q + 1; }
         }
         __syncwarp();       // (the other lanes of the issuing warp, spinning on the first copy, could keep the issuing lane from running)
 #pragma unroll 1
@@ -181,9 +184,10 @@ struct RingSlice {
                 if (atomicAdd(&r.done[st], 1u) == (uint32_t)(NWARPS - 1)) {
                     r.done[st] = 0;
                     __threadfence_block();
-                    if (t + nst < ntiles) {
+                    if (t + nst < ntiles && *(volatile uint32_t *)&r.timeout == 0u) {
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         issue(r, t + nst, st);
+                        atomicMax(&r.issued, (uint32_t)(t + nst + 1));
                     }
                 }
             }
@@ -191,7 +195,13 @@ struct RingSlice {
             if (++st == nst) { st = 0; parity ^= 1u; }
         }
         __syncthreads();
-        if (threadIdx.x == 0) r.tiles = first + (uint32_t)ntiles;
+        if (threadIdx.x == 0) {
+            // (after an expired wait: the copies in flight land, or get as long again, before the CTA moves on)
+            if (r.timeout)
+                for (uint32_t t = r.issued > (uint32_t)nst ? r.issued - (uint32_t)nst : 0u; t < r.issued; ++t)
+                    mbar_wait(&r.bar[(first + t) % (uint32_t)nst], ((first + t) / (uint32_t)nst) & 1u);
+            r.tiles = first + (uint32_t)ntiles;
+        }
         __syncthreads();
     }
     template <class F> __device__ __forceinline__ void extras(F &&f) const {
