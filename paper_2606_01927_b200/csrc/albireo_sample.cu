@@ -1725,6 +1725,13 @@ __device__ __forceinline__ bool candidate_eligible(const RowParams &rp, const Sa
     if ((a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) && a.num_top > 0) return has_topk && (rp.greedy || !(a.flags & ALBIREO_FLAG_TOPK_KEEP_TIES));
     return has_topk || has_minp;
 }
+// Whether the min-p floor may thin out the candidates ahead of the top-k stage: not where that stage's ids are asked
+// for, nor its size with ties, nor a list over the whole vocabulary.
+template <bool EXTRA>
+__device__ __forceinline__ bool floor_while_streaming(const RowParams &rp, const SampleArgs &a, bool has_topk, bool full_list) {
+    if (rp.greedy || !(rp.min_p > 0.0f) || full_list) return false;
+    return !(EXTRA && has_topk && (a.dbg_topk_ids || (a.out_num_topk && (a.flags & ALBIREO_FLAG_TOPK_KEEP_TIES))));
+}
 // which of the others the wide path takes: everything without an active top-k
 __device__ __forceinline__ bool wide_eligible(const RowParams &rp, const SampleArgs &a) {
     return !(a.flags & ALBIREO_FLAG_FORCE_GENERAL) && !rp.greedy && !(rp.top_k >= 1 && rp.top_k < a.V);
@@ -1808,7 +1815,7 @@ __device__ __forceinline__ bool candidate_finish(BlockScratch &s, const CandSmem
     const int k = rp.greedy ? 1 : rp.top_k;
     const bool has_topk = rp.greedy || (k >= 1 && k < V);
     const bool has_minp = !rp.greedy && rp.min_p > 0.0f;
-    const bool stream_minp = has_minp && !full_list && !(EXTRA && has_topk && a.dbg_topk_ids != nullptr);
+    const bool stream_minp = floor_while_streaming<EXTRA>(rp, a, has_topk, full_list);
     const int k_list = full_list ? max(k, a.num_top) : k;      // the list holds at least this many (or all there are)
     bool topk_exact_known = true;      // is min(k, #finite) known without counting?
     // keep-ties mode: the top-k stage keeps every score not below the k-th largest, i.e. exactly the
@@ -1851,10 +1858,7 @@ __device__ __forceinline__ bool candidate_path(BlockScratch &s, const CandSmem &
     const bool has_topk = rp.greedy || (rp.top_k >= 1 && rp.top_k < V);
     // the rank the threshold covers: top-k, or the list over the whole vocabulary if that is longer
     const int k = full_list ? max(rp.greedy ? 1 : rp.top_k, a.num_top) : rp.greedy ? 1 : rp.top_k;
-    const bool has_minp = !rp.greedy && rp.min_p > 0.0f;
-    // with the debug id list requested, keep the stream's threshold purely top-k so that the
-    // top-k stage's set is known exactly
-    const bool stream_minp = has_minp && !full_list && !(EXTRA && has_topk && a.dbg_topk_ids != nullptr);
+    const bool stream_minp = floor_while_streaming<EXTRA>(rp, a, has_topk, full_list);
     const int lane = threadIdx.x & 31;
     // Thread -> vector map inside each group of NT vectors: lane l of warp w takes vector
     // 16 l + ((w + l) & 15).  Consecutive vectors land in different warps (the head of the

@@ -297,8 +297,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     } else if (!to_general) {
         bool wide = !cand_row;
         if (cand_row) {
-            const bool has_minp = !rp.greedy && rp.min_p > 0.0f;
-            const bool stream_minp = has_minp && !full_list && !(has_topk && a.dbg_topk_ids != nullptr);
+            const bool stream_minp = floor_while_streaming<true>(rp, a, has_topk, full_list);
             tau = max(tau, tau_part);
             if (!has_topk || tau < KEY_MIN_FINITE) tau = KEY_MIN_FINITE;
             if (stream_minp) tau = max(tau, min(kmax, minp_key(unkey(kmax), rp.ln_min_p)));

@@ -305,3 +305,21 @@ def test_infinities_and_nan_give_a_token_in_range(binding, sampler, dtype, cut, 
             assert ((o["tokens"] >= 0) & (o["tokens"] < V)).all(), (flags, num_top, o["tokens"])
             if num_top:
                 assert ((o["top_ids"] >= -1) & (o["top_ids"] < V)).all(), (flags, num_top)
+
+
+@pytest.mark.parametrize("B", [8, 80])
+def test_size_of_a_top_k_with_ties_below_the_min_p_floor(binding, sampler, B):
+    """The top-k stage's size with ties kept, where the k-th largest score lies below the min-p floor (no debug
+    list, which changes what the stream may drop)."""
+    V = 17003
+    rng = np.random.default_rng(59)
+    x = np.round(rng.standard_normal((B, V)) * 2).astype(np.float32)
+    x[:, :5] = 20.0
+    w = W.Workload("ties_minp", B, V, W.BF16, W.f32_to_bf16_bits(x), temperature=np.ones(B, np.float32), top_k=np.full(B, 12, np.int32),
+                   min_p=np.full(B, 0.1, np.float32), seeds=np.arange(B, dtype=np.uint64))
+    w.topk_keep_ties = True
+    ref = O.sample(w, threads=_CORES)
+    t = binding.workload_tensors(w, sampler.device)
+    g = to_host(sampler.albireo_sample(t.pop("logits"), **t, want_counts=True, flags=binding.FLAG_TOPK_KEEP_TIES))
+    assert (g["num_topk"] == ref.rows["n_topk"]).all() and (g["num_kept"] == ref.rows["n_keep"]).all()
+    assert compare(w, g, ref).ok()
