@@ -2561,20 +2561,26 @@ int apply_ext(SampleArgs &a, const albireo_sample_ext_t *ext, int B, int V, cons
 // The launch shape of a batch: a CTA per row (team 1, ring of nstages), or a cluster of `team` CTAs per row.
 struct LaunchShape { int team, nstages, slice_bytes; size_t smem; };
 
-// Rows are shared by clusters where all their CTAs are on the chip at once, one per SM: then every SM
-// works on the batch and a row's slices stay in shared memory.  (Two CTAs per SM, with half the registers,
+// What the launch shape depends on: the device's SMs, the dynamic shared memory a CTA may have, and how many
+// clusters of 2^i CTAs (one per SM) are on the device at once.
+struct DeviceShape { int num_sms; size_t max_smem; int teams[5]; };
+
+// Rows are shared by clusters where all of them are on the chip at once, one CTA per SM: then every SM
+// works on the batch and a row's slices stay in shared memory.  That is not B * team <= SMs: a cluster lies within one
+// GPC, and on 148 SMs clusters of 16, 8, 4 and 2 found room 7, 15, 33 and 74 times; with one row more
+// than that a batch took up to twice as long (8 top-p rows of 152064 35.4 us by 16 CTAs each, 21.1 by 8).  (Two CTAs per SM, with half the registers,
 // were 10 % slower on the rows without a top-k and the same on the others.)  Of the sizes that fit, the largest whose slices are
 // still at least 8 KB (one vector per thread): below that the exchange costs more than the slice.
-bool pick_team(LaunchShape &ls, int B, int V, int esize, bool with_history, int num_sms, size_t max_smem) {
+bool pick_team(LaunchShape &ls, int B, int V, int esize, bool with_history, const DeviceShape &d) {
     const long row_bytes = (long)(V / (16 / esize)) * 16;
-    for (int team = MAX_TEAM; team >= 2; team >>= 1) {
-        if (row_bytes / team < 8192 || (long)B * team > (long)num_sms) continue;
+    for (int team = MAX_TEAM, i = 4; team >= 2; team >>= 1, --i) {
+        if (row_bytes / team < 8192 || B > d.teams[i]) continue;
         const long per = ((row_bytes / 16 + team - 1) / team) * 16;
         const long slice = ((per > SLICE_MIN ? per : (long)SLICE_MIN) + 127) & ~127L;
         long smem = SLICE_OFF + slice + 16 + (with_history ? 4L * slice_table_words((int)(per / esize)) : 8L * X_ENDS);
         const long general = GENERAL_BYTES + (with_history ? (long)history_smem_bytes(V) : 0);
         if (general > smem) smem = general;
-        if (smem > (long)max_smem) continue;
+        if (smem > (long)d.max_smem) continue;
         ls.team = team; ls.slice_bytes = (int)slice; ls.smem = (size_t)smem; ls.nstages = 0;
         return true;
     }
@@ -2586,13 +2592,13 @@ bool extras_asked(const SampleArgs &a) {
 }
 
 // false: the vocabulary is too large for the on-chip tables
-bool pick_shape(LaunchShape &ls, int B, int V, int esize, bool with_history, bool force_general, int num_sms, size_t max_smem) {
-    if (!force_general && pick_team(ls, B, V, esize, with_history, num_sms, max_smem)) return true;
+bool pick_shape(LaunchShape &ls, int B, int V, int esize, bool with_history, bool force_general, const DeviceShape &d) {
+    if (!force_general && pick_team(ls, B, V, esize, with_history, d)) return true;
     ls.team = 1; ls.slice_bytes = 0;
-    ls.nstages = ring_stages_for(V, with_history, B <= num_sms);
+    ls.nstages = ring_stages_for(V, with_history, B <= d.num_sms);
     ls.smem = smem_bytes_for(V, with_history, ls.nstages);
-    while (ls.smem > max_smem && ls.nstages > 2) ls.smem = smem_bytes_for(V, with_history, --ls.nstages);
-    return ls.smem <= max_smem;
+    while (ls.smem > d.max_smem && ls.nstages > 2) ls.smem = smem_bytes_for(V, with_history, --ls.nstages);
+    return ls.smem <= d.max_smem;
 }
 
 template <int DT>
@@ -2623,10 +2629,12 @@ cudaError_t launch_sample_kernel(int dtype, int B, const LaunchShape &ls, cudaSt
     if (dtype == ALBIREO_BF16) return launch_sample_kernel_as<ALBIREO_BF16>(B, ls, st, a);
     return launch_sample_kernel_as<ALBIREO_F16>(B, ls, st, a);
 }
-// Lets every instantiation use the device's opt-in shared memory; gives the dynamic bytes available
-// to a CTA (the opt-in limit less the largest static use), or 0 with *err set.
-size_t enable_large_smem(int device, cudaError_t *err) {
+// Lets every instantiation use the device's opt-in shared memory and clusters of 16, and fills in `d` (the dynamic
+// bytes available to a CTA are the opt-in limit less the largest static use).  `device` is current.
+cudaError_t set_up_device(int device, DeviceShape &d) {
     int optin = 0;
+    d = DeviceShape();
+    if (cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) { cudaGetLastError(); d.num_sms = 0; }
     cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
     const void *kernels[] = {
         (const void *)albireo_cluster_kernel<ALBIREO_F32>, (const void *)albireo_cluster_kernel<ALBIREO_BF16>, (const void *)albireo_cluster_kernel<ALBIREO_F16>,
@@ -2639,15 +2647,31 @@ size_t enable_large_smem(int device, cudaError_t *err) {
         if (e == cudaSuccess) e = cudaFuncGetAttributes(&f, k);
         if (e == cudaSuccess && f.sharedSizeBytes > st) st = f.sharedSizeBytes;
     }
-    if (e != cudaSuccess) { *err = e; return 0; }
-    if ((size_t)optin <= st) { *err = cudaErrorInvalidValue; return 0; }
+    if (e != cudaSuccess) return e;
+    if ((size_t)optin <= st) return cudaErrorInvalidValue;
     const size_t smem = (size_t)optin - st;
     for (const void *k : kernels)
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    for (int i = 0; i < 3; ++i)      // clusters of 16
+    for (int i = 0; i < 3; ++i)
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernels[i], cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    *err = e;
-    return e == cudaSuccess ? smem : 0;
+    if (e != cudaSuccess) return e;
+    d.max_smem = smem;
+    // (a size that finds no room at all, on a part of a GPU say, counts 0 and is not used)
+    for (int i = 1; i < 5; ++i) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1u << i); cfg.blockDim = dim3(NT); cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute at;
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = 1u << i; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+        cfg.attrs = &at; cfg.numAttrs = 1;
+        d.teams[i] = d.num_sms >> i;
+        for (int k = 0; k < 3; ++k) {
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, kernels[k], &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+            if (n < d.teams[i]) d.teams[i] = n;
+        }
+    }
+    return cudaSuccess;
 }
 
 }  // namespace
@@ -2660,8 +2684,7 @@ struct albireo_sampler {
     int64_t max_history_total;
     unsigned char *workspace;
     size_t workspace_bytes;
-    size_t max_smem;
-    int num_sms;
+    DeviceShape dev;
     uint64_t launches;
     char err[256];
 };
@@ -2703,20 +2726,18 @@ extern "C" int albireo_sample_init(albireo_sampler_t **out, int32_t device, int3
     if (cudaGetDevice(&prev) != cudaSuccess) return ALBIREO_ECUDA;
     if (cudaSetDevice(device) != cudaSuccess) { cudaGetLastError(); return ALBIREO_ECUDA; }
     // opt in to the largest dynamic shared memory a CTA may have on this device
-    cudaError_t e0 = cudaSuccess;
-    const size_t smem = enable_large_smem(device, &e0);
+    DeviceShape shape;
+    const cudaError_t e0 = set_up_device(device, shape);
     if (prev >= 0 && prev != device) cudaSetDevice(prev);
     if (e0 != cudaSuccess) { cudaGetLastError(); return ALBIREO_ECUDA; }
-    if (smem_bytes_for(max_vocab, true, 2) > smem) return ALBIREO_EUNSUPPORTED;
+    if (smem_bytes_for(max_vocab, true, 2) > shape.max_smem) return ALBIREO_EUNSUPPORTED;
 
     albireo_sampler *h = new (std::nothrow) albireo_sampler();
     if (!h) return ALBIREO_ENOMEM;
     h->device = device; h->max_rows = max_rows; h->max_vocab = max_vocab;
     h->max_history_total = max_history_total;
     h->workspace = (unsigned char *)workspace; h->workspace_bytes = workspace_bytes;
-    h->max_smem = smem; h->launches = 0; h->err[0] = 0;
-    h->num_sms = 0;
-    if (cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) { cudaGetLastError(); h->num_sms = 0; }
+    h->dev = shape; h->launches = 0; h->err[0] = 0;
     *out = h;
     return ALBIREO_OK;
 }
@@ -2758,7 +2779,7 @@ extern "C" int albireo_sample(albireo_sampler_t *h, const void *logits, int32_t 
     if (cudaGetDevice(&cur) != cudaSuccess || cur != h->device) { cudaGetLastError(); set_err(h, "the handle's device is not current%s", ""); return ALBIREO_EINVAL; }
 
     LaunchShape ls;
-    if (!pick_shape(ls, B, V, (int)esize, history_ids != nullptr, (a.flags & ALBIREO_FLAG_FORCE_GENERAL) != 0, h->num_sms, h->max_smem)) { set_err(h, "vocabulary too large for the on-chip tables%s", ""); return ALBIREO_EUNSUPPORTED; }
+    if (!pick_shape(ls, B, V, (int)esize, history_ids != nullptr, (a.flags & ALBIREO_FLAG_FORCE_GENERAL) != 0, h->dev)) { set_err(h, "vocabulary too large for the on-chip tables%s", ""); return ALBIREO_EUNSUPPORTED; }
     cudaStream_t st = (cudaStream_t)stream;
     const cudaError_t e = launch_sample_kernel(dtype, B, ls, st, a);
     if (e != cudaSuccess) { cudaGetLastError(); set_err(h, "kernel launch failed: %s", cudaGetErrorString(e)); return ALBIREO_ECUDA; }
@@ -2889,10 +2910,10 @@ extern "C" int albireo_stream_only(albireo_sampler_t *h, const void *logits, int
     if (B == 0) return ALBIREO_OK;
     if (B < 0 || B > h->max_rows || V < 1 || V > h->max_vocab || !logits || !sink) { set_err(h, "bad arguments%s", ""); return ALBIREO_EINVAL; }
     if (dtype != ALBIREO_F32 && dtype != ALBIREO_BF16 && dtype != ALBIREO_F16) { set_err(h, "unknown dtype%s", ""); return ALBIREO_EINVAL; }
-    int nstages = ring_stages_for(V, false, B <= h->num_sms);
+    int nstages = ring_stages_for(V, false, B <= h->dev.num_sms);
     size_t smem = smem_bytes_for(V, false, nstages);
-    while (smem > h->max_smem && nstages > 2) smem = smem_bytes_for(V, false, --nstages);
-    if (smem > h->max_smem) { set_err(h, "vocabulary too large%s", ""); return ALBIREO_EUNSUPPORTED; }
+    while (smem > h->dev.max_smem && nstages > 2) smem = smem_bytes_for(V, false, --nstages);
+    if (smem > h->dev.max_smem) { set_err(h, "vocabulary too large%s", ""); return ALBIREO_EUNSUPPORTED; }
     cudaStream_t st = (cudaStream_t)stream;
     if (dtype == ALBIREO_F32) albireo_stream_only_kernel<ALBIREO_F32><<<B, NT, smem, st>>>(logits, V, (int64_t)V, nstages, sink, drop_tile);
     else if (dtype == ALBIREO_BF16) albireo_stream_only_kernel<ALBIREO_BF16><<<B, NT, smem, st>>>(logits, V, (int64_t)V, nstages, sink, drop_tile);
@@ -2918,8 +2939,7 @@ constexpr int FIXED_MAX_DEVICES = 64;
 struct FixedDeviceState {
     bool ready;
     uint32_t *counts;     // device address of g_fixed_counts on that device
-    size_t max_smem;
-    int num_sms;
+    DeviceShape shape;
 };
 FixedDeviceState g_fixed_dev[FIXED_MAX_DEVICES];
 std::mutex g_fixed_mutex;
@@ -2941,11 +2961,9 @@ int fixed_setup(int dev, FixedDeviceState **out) {
         void *ptr = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&ptr, g_fixed_counts);
         if (e != cudaSuccess || !ptr) { cudaGetLastError(); return fixed_fail(ALBIREO_ECUDA, "cudaGetSymbolAddress failed: %s", cudaGetErrorString(e)); }
-        const size_t smem = enable_large_smem(dev, &e);
+        e = set_up_device(dev, d.shape);
         if (e != cudaSuccess) { cudaGetLastError(); return fixed_fail(ALBIREO_ECUDA, "kernel set-up failed: %s", cudaGetErrorString(e)); }
-        d.num_sms = 0;
-        if (cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { cudaGetLastError(); d.num_sms = 0; }
-        d.counts = (uint32_t *)ptr; d.max_smem = smem; d.ready = true;
+        d.counts = (uint32_t *)ptr; d.ready = true;
     }
     *out = &d;
     return ALBIREO_OK;
@@ -2996,7 +3014,7 @@ extern "C" int albireo_sample_fixed_scratch(const void *logits, int32_t B, int32
     a.ws_counts_cap = ALBIREO_FIXED_MAX_HISTORY;
 
     LaunchShape ls;
-    if (!pick_shape(ls, B, V, (int)esize, history_ids != nullptr, (a.flags & ALBIREO_FLAG_FORCE_GENERAL) != 0, d->num_sms, d->max_smem)) return fixed_fail(ALBIREO_EUNSUPPORTED, "vocabulary too large for the on-chip tables%s", "");
+    if (!pick_shape(ls, B, V, (int)esize, history_ids != nullptr, (a.flags & ALBIREO_FLAG_FORCE_GENERAL) != 0, d->shape)) return fixed_fail(ALBIREO_EUNSUPPORTED, "vocabulary too large for the on-chip tables%s", "");
     cudaStream_t st = (cudaStream_t)stream;
     const cudaError_t e = launch_sample_kernel(dtype, B, ls, st, a);
     if (e != cudaSuccess) { cudaGetLastError(); return fixed_fail(ALBIREO_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e)); }
