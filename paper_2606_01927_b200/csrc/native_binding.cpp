@@ -248,14 +248,13 @@ PyObject *sample_checked(PyObject *const *a) {
         int32_t *tok = (int32_t *)tokens.data_ptr();
         float *lp = (float *)logprobs.data_ptr();
         const int32_t b32 = (int32_t)B, v32 = (int32_t)V;
-        if (entry == DEVICE) rc = albireo_sample(h, x, b32, v32, dt, T, k, topp, minp, rep, pres, freq, hid, hoff, seeds, step, tok, lp, stream, &ext);
-        else {
-            // the host entry waits for the device; other Python threads run meanwhile
-            PyThreadState *ts = PyEval_SaveThread();
-            rc = entry == HOST ? albireo_sample_host(h, x, b32, v32, dt, T, k, topp, minp, rep, pres, freq, hid, hoff, htot, seeds, step, tok, lp, stream, &ext)
-                               : albireo_sample_fixed_scratch(x, b32, v32, dt, T, k, topp, minp, rep, pres, freq, hid, hoff, htot, seeds, step, tok, lp, stream, &ext);
-            PyEval_RestoreThread(ts);
-        }
+        // other Python threads run meanwhile: the host entry waits for the device, and a launch waits for it where
+        // the queue is full
+        PyThreadState *ts = PyEval_SaveThread();
+        rc = entry == DEVICE ? albireo_sample(h, x, b32, v32, dt, T, k, topp, minp, rep, pres, freq, hid, hoff, seeds, step, tok, lp, stream, &ext)
+             : entry == HOST ? albireo_sample_host(h, x, b32, v32, dt, T, k, topp, minp, rep, pres, freq, hid, hoff, htot, seeds, step, tok, lp, stream, &ext)
+                             : albireo_sample_fixed_scratch(x, b32, v32, dt, T, k, topp, minp, rep, pres, freq, hid, hoff, htot, seeds, step, tok, lp, stream, &ext);
+        PyEval_RestoreThread(ts);
     }
     if (rc != ALBIREO_OK) return PyLong_FromLong(rc);
     // a tensor the caller passed is returned as the object it passed
