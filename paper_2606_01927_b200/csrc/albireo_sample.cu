@@ -90,6 +90,7 @@ struct SampleArgs {
     int64_t ws_counts_cap;      // entries
     int32_t elem_size;          // host side only: bytes per logit
     int32_t slice_bytes;        // shared memory of a row's slice (cluster kernel)
+    int32_t list_words;         // and, behind its tables, 32-bit words for the penalised tokens and the row's ends
     // rows in pieces (vocabulary shards as the all-to-all of sequence-parallel sampling leaves them)
     int32_t seg_ptr_count;      // > 0: the pieces live in buffers of their own, seg_ptr[j]; 0: a stride apart in `logits`
     int64_t seg_stride;         // elements between consecutive pieces of a row
@@ -2559,7 +2560,7 @@ int apply_ext(SampleArgs &a, const albireo_sample_ext_t *ext, int B, int V, cons
 }
 
 // The launch shape of a batch: a CTA per row (team 1, ring of nstages), or a cluster of `team` CTAs per row.
-struct LaunchShape { int team, nstages, slice_bytes; size_t smem; };
+struct LaunchShape { int team, nstages, slice_bytes, list_words; size_t smem; };
 
 // What the launch shape depends on: the device's SMs, the dynamic shared memory a CTA may have, and how many
 // clusters of 2^i CTAs (one per SM) are on the device at once.
@@ -2577,11 +2578,19 @@ bool pick_team(LaunchShape &ls, int B, int V, int esize, bool with_history, cons
         if (row_bytes / team < 8192 || B > d.teams[i]) continue;
         const long per = ((row_bytes / 16 + team - 1) / team) * 16;
         const long slice = ((per > SLICE_MIN ? per : (long)SLICE_MIN) + 127) & ~127L;
-        long smem = SLICE_OFF + slice + 16 + (with_history ? 4L * slice_table_words((int)(per / esize)) : 8L * X_ENDS);
+        const long nids = per / esize, fixed = SLICE_OFF + slice + 16 + (with_history ? 4L * slice_counts_off((int)nids) : 0);
+        long list = 2L * X_ENDS;
+        if (with_history) {
+            list = 2L * (nids + X_ENDS);
+            const long room = ((long)d.max_smem - fixed) / 4;
+            if (room < list) list = room & ~1L;
+            if (list < 2L * X_LEAST && list < 2L * (nids + X_ENDS)) continue;
+        }
+        long smem = fixed + 4 * list;
         const long general = GENERAL_BYTES + (with_history ? (long)history_smem_bytes(V) : 0);
         if (general > smem) smem = general;
         if (smem > (long)d.max_smem) continue;
-        ls.team = team; ls.slice_bytes = (int)slice; ls.smem = (size_t)smem; ls.nstages = 0;
+        ls.team = team; ls.slice_bytes = (int)slice; ls.list_words = (int)list; ls.smem = (size_t)smem; ls.nstages = 0;
         return true;
     }
     return false;
@@ -2594,7 +2603,7 @@ bool extras_asked(const SampleArgs &a) {
 // false: the vocabulary is too large for the on-chip tables
 bool pick_shape(LaunchShape &ls, int B, int V, int esize, bool with_history, bool force_general, const DeviceShape &d) {
     if (!force_general && pick_team(ls, B, V, esize, with_history, d)) return true;
-    ls.team = 1; ls.slice_bytes = 0;
+    ls.team = 1; ls.slice_bytes = 0; ls.list_words = 0;
     ls.nstages = ring_stages_for(V, with_history, B <= d.num_sms);
     ls.smem = smem_bytes_for(V, with_history, ls.nstages);
     while (ls.smem > d.max_smem && ls.nstages > 2) ls.smem = smem_bytes_for(V, with_history, --ls.nstages);
@@ -2624,7 +2633,7 @@ cudaError_t launch_sample_kernel_as(int B, const LaunchShape &ls, cudaStream_t s
            : extras_asked(a) ? cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT, true>, a) : cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT, false>, a);
 }
 cudaError_t launch_sample_kernel(int dtype, int B, const LaunchShape &ls, cudaStream_t st, SampleArgs &a) {
-    a.nstages = ls.nstages; a.slice_bytes = ls.slice_bytes;
+    a.nstages = ls.nstages; a.slice_bytes = ls.slice_bytes; a.list_words = ls.list_words;
     if (dtype == ALBIREO_F32) return launch_sample_kernel_as<ALBIREO_F32>(B, ls, st, a);
     if (dtype == ALBIREO_BF16) return launch_sample_kernel_as<ALBIREO_BF16>(B, ls, st, a);
     return launch_sample_kernel_as<ALBIREO_F16>(B, ls, st, a);

@@ -11,14 +11,14 @@
 // largest of the slices' own k-th largest values, and the smallest of their ceil(k / size)-th largest.
 
 constexpr int SLICE_MIN = 18 * 1024;      // the final stage's scratch lies in CTA 0's slice when that is done with
-constexpr int X_CAP = 1024;               // penalised tokens and unaligned ends of a slice
+constexpr int X_LEAST = 1024;             // penalised tokens and unaligned ends of a slice that are listed on chip, at least
 constexpr int X_ENDS = 16;                // most unaligned ends of a row (14), rounded up
 constexpr int GENERAL_BYTES = HIST_BINS * 16 + GL_CAP * 8 + 4096;      // what the general path lays over the front
 
-// 32-bit words of the tables behind a slice of n elements: bitmap, coarse prefix, counts (then scores) and ids
+// 32-bit words of the tables behind a slice of n elements: bitmap, coarse prefix; then the list_words of the launch for
+// counts (then scores) and ids, as many as there can be of them or as there is room for
 __host__ __device__ constexpr int slice_coarse_off(int n) { return (((n + 31) / 32) + 4) & ~3; }
 __host__ __device__ constexpr int slice_counts_off(int n) { return slice_coarse_off(n) + ((n + 31) / 32 + 7) / 8 + 1; }
-__host__ __device__ constexpr int slice_table_words(int n) { return slice_counts_off(n) + 2 * X_CAP; }
 
 // The k-th and the kp-th largest of the block's per-thread maxima `mk` (0: none), from below: the
 // smallest maximum of the value-linear bin in which the count from the top gets there (see
@@ -65,24 +65,30 @@ __device__ void slice_select(BlockScratch &s, const CandSmem &cs, uint32_t mk, i
 
 // The slice's penalised tokens: how often each occurs (bitmap over the slice, ranks, counts), then
 // their scores from the raw logits in shared memory, which they leave with -inf in their place.
-// Returns how many there are, or -1 if they do not fit.  Ends with a barrier.  The row's unaligned ends
+// Returns how many there are, or -1 if there is no room for them.  Where the list on chip holds the scores but not
+// the ids as well, the ids go to the workspace (`xid` points there then): the row has a word per history id in it, and
+// a slice's part begins after as many words as the history has ids ahead of the slice.  (Such rows went to the general
+// path: 64 rows of 152064 with 8192-id histories and top-k 40 took 260 us.)  Ends with a barrier.  The row's unaligned ends
 // (ids below id_lo or from id_hi on, CTA 0 only) are counted in s.red: occurrences in the output, and in
 // the high word whether there are any in the prompt.
 // `landed()` waits for the slice; everything before it overlaps the copy.
 template <int DT, class W>
 __device__ __noinline__ int slice_history(BlockScratch *sp, RowCtx c, const int32_t *ids, int len, int out_start, int slice_off, int id0, int nids,
-                                          int id_lo, int id_hi, int tab_off, W landed, bool &ok) {
+                                          int id_lo, int id_hi, int tab_off, int list_words, uint32_t *ws, int64_t ws_cap, int64_t ws_off,
+                                          W landed, bool &ok, int *&xid) {
     typedef Elem<DT> E;
     BlockScratch &s = *sp;
     extern __shared__ __align__(128) unsigned char smem[];
     const int nwords = (nids + 31) >> 5, ncoarse = (nwords + 7) >> 3;
     uint32_t *bitmap = (uint32_t *)(smem + tab_off), *coarse = bitmap + slice_coarse_off(nids), *counts = bitmap + slice_counts_off(nids);
-    int *xid = (int *)(counts + X_CAP);
+    uint32_t ahead = 0, own = 0;           // history ids ahead of the slice and in it
     for (int w = threadIdx.x; w <= nwords; w += NT) bitmap[w] = 0;
     __syncthreads();
     for (int j = threadIdx.x; j < len; j += NT) {
         const int id = __ldg(ids + j);
         const uint32_t t = (uint32_t)(id - id0);
+        ahead += id >= 0 && id < id0;
+        own += t < (uint32_t)nids;
         if (id < id_lo ? id >= 0 : id >= id_hi && id < c.V) {
             // (32-bit adds: the first ids of a vocabulary are most of many a history, and a 64-bit add in shared
             // memory is a compare-and-swap loop, 18 us for 2700 ids)
@@ -106,7 +112,14 @@ __device__ __noinline__ int slice_history(BlockScratch *sp, RowCtx c, const int3
         U += tot;
     }
     c.bitmap = bitmap; c.coarse = coarse; c.counts = counts; c.n_distinct = U; c.ncoarse = ncoarse;
-    const bool fits = U <= (uint32_t)(X_CAP - X_ENDS);
+    bool fits = 2u * (U + X_ENDS) <= (uint32_t)list_words;
+    if (!fits && U + X_ENDS <= (uint32_t)list_words) {
+        uint32_t at, n_own;
+        block_exscan_u32(s, ahead, at);
+        block_exscan_u32(s, own, n_own);
+        fits = ws && ws_off >= 0 && U + X_ENDS <= n_own && ws_off + (int64_t)at + (int64_t)n_own <= ws_cap;
+        if (fits) xid = (int *)ws + ws_off + at;
+    }
     if (fits) for (uint32_t u = threadIdx.x; u < U; u += NT) counts[u] = 0;
     __syncthreads();
     if (fits) {
@@ -219,10 +232,11 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     src.vec_off = SLICE_OFF; src.nvec = nv; src.id0 = id0;
     // (a launch without histories has no tables: only the row's unaligned ends are listed)
     src.xz_off = tables ? tab_off + slice_counts_off(n_slice_ids) * 4 : tab_off;
-    src.xid_off = src.xz_off + (tables ? X_CAP : X_ENDS) * 4;
+    int *xid = (int *)(smem + src.xz_off) + (a.list_words >> 1);
     if (o1 > o0) {
         nx = slice_history<DT>(&s, c, a.hist_ids + o0, o1 - o0, ostart, SLICE_OFF, id0, n_slice_ids, tm.rank == 0 ? head : 0,
-                               tm.rank == 0 ? tail0 : V, tab_off, [&] { return mbar_wait(bar, 0); }, landed);
+                               tm.rank == 0 ? tail0 : V, tab_off, a.list_words, a.ws_counts, a.ws_counts_cap, (int64_t)o0,
+                               [&] { return mbar_wait(bar, 0); }, landed, xid);
         if (nx < 0) { nx = 0; fits = false; }
     } else landed = mbar_wait(bar, 0);
     const uint32_t distinct = (uint32_t)nx;
@@ -232,14 +246,14 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
             const int i = q < head ? q : tail0 + (q - head);
             const u64 seen = s.red[q];
             const float x = E::load(elem_ptr<DT>(c, i), 0);
-            ((int *)(smem + src.xid_off))[nx + q] = i;
+            xid[nx + q] = i;
             ((float *)(smem + src.xz_off))[nx + q] = __fmul_rn(seen ? penalise_counted(c, x, (uint32_t)seen) : x, c.invT);
             if (seen) atomicAdd(&tm.x->far_list, 1u);              // (distinct ids among them; far_list starts over below)
         }
         nx += nscal;
         __syncthreads();
     }
-    src.nx = nx;
+    src.nx = nx; src.xid = xid;
 
     // the slice's maximum, its number of finite scores and every thread's own maximum
     const bool full_lp = (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) != 0, full_list = full_lp && a.num_top > 0;

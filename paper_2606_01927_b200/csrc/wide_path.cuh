@@ -235,7 +235,8 @@ struct SmemSlice {
     typedef Elem<DT> E;
     static constexpr bool SPARE_REGISTERS = true;       // 128 per thread
     int vec_off, nvec, id0;       // where the slice and the list lie in the dynamic shared memory
-    int xid_off, xz_off, nx;
+    const int *xid;               // (in the workspace where there are too many for both lists on chip)
+    int xz_off, nx;
     __device__ __forceinline__ int first_id() const { return id0; }
     template <class F> __device__ __forceinline__ void vectors(F &&f) const {
         extern __shared__ __align__(128) unsigned char smem[];
@@ -248,7 +249,6 @@ struct SmemSlice {
     }
     template <class F> __device__ __forceinline__ void extras(F &&f) const {
         extern __shared__ __align__(128) unsigned char smem[];
-        const int *xid = (const int *)(smem + xid_off);
         const float *xz = (const float *)(smem + xz_off);
 #pragma unroll 1
         for (int r0 = 0; r0 < nx; r0 += NT) {

@@ -323,3 +323,26 @@ def test_size_of_a_top_k_with_ties_below_the_min_p_floor(binding, sampler, B):
     g = to_host(sampler.albireo_sample(t.pop("logits"), **t, want_counts=True, flags=binding.FLAG_TOPK_KEEP_TIES))
     assert (g["num_topk"] == ref.rows["n_topk"]).all() and (g["num_kept"] == ref.rows["n_keep"]).all()
     assert compare(w, g, ref).ok()
+
+
+@pytest.mark.parametrize("B", [2, 12, 24, 50])
+@pytest.mark.parametrize("dtype", [W.F32, W.BF16])
+def test_long_histories(binding, sampler, B, dtype):
+    """Histories with more distinct ids in a slice than its list on chip takes, in clusters of every size: the rows stay
+    on their path, with and without a prompt part and with ids outside the vocabulary."""
+    V = 120001
+    rng = np.random.default_rng(61)
+    x = (rng.standard_normal((B, V)) * 2).astype(np.float32)
+    rows = [rng.integers(-3, V + 3, 20000) if b % 3 == 0 else rng.integers(0, 6000, 4000) if b % 3 == 1 else
+            np.minimum(rng.zipf(1.2, 16000), V - 1) for b in range(B)]
+    w = W.Workload("long", B, V, dtype, x if dtype == W.F32 else W.f32_to_bf16_bits(x), temperature=np.ones(B, np.float32),
+                   top_k=np.where(np.arange(B) % 2, 50, 0).astype(np.int32), top_p=np.full(B, 0.9, np.float32),
+                   repetition_penalty=np.full(B, 1.3, np.float32), presence_penalty=np.full(B, 0.4, np.float32),
+                   frequency_penalty=np.full(B, 0.2, np.float32), history_ids=np.concatenate(rows).astype(np.int32),
+                   history_offsets=np.cumsum([0] + [len(r) for r in rows]).astype(np.int32), seeds=np.arange(B, dtype=np.uint64))
+    w.output_start = np.where(np.arange(B) % 4 == 0, 7000, 0).astype(np.int32)
+    w.num_top = 5
+    g, ref = check(binding, sampler, w)
+    assert (g["num_kept"] == ref.rows["n_keep"]).all()
+    assert not (g["row_status"][w.top_k > 0] & binding.ROW_GENERAL_PATH).any()
+    assert not (g["row_status"] & binding.ROW_HISTORY_OVERFLOW).any()
