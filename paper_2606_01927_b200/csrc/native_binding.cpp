@@ -12,6 +12,7 @@
 #include <ATen/ops/empty.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <stdexcept>
@@ -272,17 +273,18 @@ PyObject *sample_checked(PyObject *const *a) {
     return out;
 }
 
+// (torch's own errors reach Python as torch's types: out of memory as torch.OutOfMemoryError)
 PyObject *sample(PyObject *, PyObject *const *args, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
     if (n != A_COUNT) { PyErr_Format(PyExc_TypeError, "sample takes %d positional arguments, got %zd", (int)A_COUNT, n); return nullptr; }
     try {
         return sample_checked(args);
     } catch (const BadArgument &e) {
         PyErr_SetString(PyExc_ValueError, e.what());
     } catch (const PythonError &) {
-    } catch (const std::exception &e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
     }
     return nullptr;
+    END_HANDLE_TH_ERRORS
 }
 
 PyMethodDef methods[] = {

@@ -46,3 +46,11 @@ def test_a_launch_that_waits_for_the_queue_lets_other_threads_run(binding):
     gap = max(b - a for a, b in zip([t0] + seen, seen + [t1]))
     assert longest > 0.2, longest                      # a call did block
     assert gap < 0.5 * longest, (gap, longest)
+
+
+def test_out_of_memory_is_torchs(binding):
+    s = binding.Sampler(max_rows=4, max_vocab=1000)
+    x = torch.zeros((4, 1000), device=s.device)
+    with pytest.raises(torch.cuda.OutOfMemoryError):
+        s.albireo_sample(x, B=1 << 45)                 # the outputs alone are more than any device holds
+    s.close()
