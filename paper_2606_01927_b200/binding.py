@@ -79,6 +79,13 @@ def _load() -> C.CDLL:
     lib.albireo_sample_host_staging_bytes.argtypes = [i32, i32, i64]
     lib.albireo_sample_init.restype = C.c_int
     lib.albireo_sample_init.argtypes = [C.POINTER(vp), i32, i32, i32, i64, vp, C.c_size_t]
+    sample_args = [vp, vp, i32, i32, i32, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, u64, vp, vp, vp, C.POINTER(SampleExt)]
+    lib.albireo_sample.restype = C.c_int
+    lib.albireo_sample.argtypes = sample_args
+    lib.albireo_sample_host.restype = C.c_int
+    lib.albireo_sample_host.argtypes = sample_args[:14] + [i64] + sample_args[14:]
+    lib.albireo_sample_fixed_scratch.restype = C.c_int
+    lib.albireo_sample_fixed_scratch.argtypes = sample_args[1:14] + [i64] + sample_args[14:]
     lib.albireo_sample_destroy.restype = C.c_int
     lib.albireo_sample_destroy.argtypes = [vp]
     lib.albireo_last_error.restype = C.c_char_p

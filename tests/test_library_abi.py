@@ -108,3 +108,10 @@ def test_binding_struct_and_constants_match_the_header(tmp_path):
     assert int(out["ALBIREO_FLAG_LOGPROB_FULL_VOCAB"]) == binding.FLAG_LOGPROB_FULL_VOCAB
     assert int(out["ALBIREO_FLAG_PROGRAMMATIC_LAUNCH"]) == binding.FLAG_PROGRAMMATIC_LAUNCH
     assert int(out["ALBIREO_FIXED_MAX_HISTORY"]) == binding.FIXED_MAX_HISTORY and int(out["ALBIREO_OK"]) == binding.OK
+
+
+def test_every_export_is_declared_to_ctypes():
+    """`binding.LIB` may be called directly: without argument types an integer or a handle would travel as a C int."""
+    from paper_2606_01927_b200 import binding
+    for name in binding.EXPORTS:
+        assert getattr(binding.LIB, name).argtypes is not None, name
