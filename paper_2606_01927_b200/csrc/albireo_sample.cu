@@ -17,6 +17,7 @@
 // A kept set is always a prefix of that order, i.e. { t : C(t) >= threshold }.
 
 #include <cooperative_groups.h>
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -2708,6 +2709,26 @@ extern "C" size_t albireo_sample_workspace_bytes(int32_t max_rows, int32_t max_v
     return (bytes + 255) & ~(size_t)255;
 }
 
+// The device address of a host array that lies in one pinned allocation or registration as a whole, aligned to
+// `align`; null otherwise.
+static void *mapped_host_range(const void *host, size_t bytes, size_t align) {
+    typedef CUresult (*Attributes)(unsigned int, CUpointer_attribute *, void **, CUdeviceptr);
+    static const Attributes attributes = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &f, cudaEnableDefault, &found) != cudaSuccess) { cudaGetLastError(); f = nullptr; }
+        return (Attributes)f;
+    }();
+    if (!host || !attributes) return nullptr;
+    unsigned int type = 0;
+    CUdeviceptr dev = 0, start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *to[] = {&type, &dev, &start, &size};
+    if (attributes(4, what, to, (CUdeviceptr)(uintptr_t)host) != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST || !dev || dev % align) return nullptr;
+    return dev >= start && dev - start <= size && bytes <= size - (dev - start) ? (void *)(uintptr_t)dev : nullptr;
+}
+
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 extern "C" size_t albireo_sample_host_staging_bytes(int32_t max_rows, int32_t max_vocab, int64_t max_history_total) {
@@ -2836,33 +2857,35 @@ extern "C" int albireo_sample_host(albireo_sampler_t *h, const void *logits, int
     auto reserve = [&](size_t bytes) -> void * { void *dst = p; p += align256(bytes); return dst; };
     // The per-row arrays are a few KB: where the caller's memory is pinned, the kernel reads and writes them
     // there itself (one round trip over the bus, all of them at once) instead of a copy each, which costs
-    // 2 to 4 us apiece (32 rows of 152064 bf16 logits 232.8 -> 229.9 us, most of it the copy of the logits).
-    auto mapped = [&](const void *host) -> void * {
-        cudaPointerAttributes at;
-        if (!host || cudaPointerGetAttributes(&at, host) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-        return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
-    };
-    auto small = [&](const void *src, size_t bytes) -> void * {
-        void *m = mapped(src);
+    // 1 to 2 us apiece (32 rows of 152064 bf16 logits 232.6 -> 225.6 us, most of it the copy of the logits).
+    // Only where the whole array is pinned and aligned as the kernel's loads need it; a result only
+    // where it shares no memory with an input, which another row may read after it is written.
+    auto small = [&](const void *src, size_t bytes, size_t align) -> void * {
+        void *m = mapped_host_range(src, bytes, align);
         return m ? m : stage(src, bytes);
     };
+    const size_t Bs = (size_t)B, esize = dtype == ALBIREO_F32 ? 4 : 2;
     auto result = [&](void *dst, size_t bytes, bool &direct) -> void * {
-        void *m = mapped(dst);
+        const struct { const void *at; size_t bytes; } inputs[] = {
+            {temperature, Bs * 4}, {top_k, Bs * 4}, {top_p, Bs * 4}, {min_p, Bs * 4}, {repetition_penalty, Bs * 4}, {presence_penalty, Bs * 4},
+            {frequency_penalty, Bs * 4}, {history_offsets, (Bs + 1) * 4}, {seeds, Bs * 8}};
+        void *m = mapped_host_range(dst, bytes, 4);
+        for (const auto &in : inputs)
+            if (in.at && (uintptr_t)in.at < (uintptr_t)dst + bytes && (uintptr_t)dst < (uintptr_t)in.at + in.bytes) m = nullptr;
         direct = m != nullptr;
         return m ? m : reserve(bytes);
     };
-    const size_t Bs = (size_t)B, esize = dtype == ALBIREO_F32 ? 4 : 2;
     const void *d_logits = stage(logits, Bs * (size_t)V * esize);
-    const float *d_T = (const float *)small(temperature, Bs * 4);
-    const int32_t *d_k = (const int32_t *)small(top_k, Bs * 4);
-    const float *d_tp = (const float *)small(top_p, Bs * 4);
-    const float *d_mp = (const float *)small(min_p, Bs * 4);
-    const float *d_r = (const float *)small(repetition_penalty, Bs * 4);
-    const float *d_p = (const float *)small(presence_penalty, Bs * 4);
-    const float *d_f = (const float *)small(frequency_penalty, Bs * 4);
+    const float *d_T = (const float *)small(temperature, Bs * 4, 4);
+    const int32_t *d_k = (const int32_t *)small(top_k, Bs * 4, 4);
+    const float *d_tp = (const float *)small(top_p, Bs * 4, 4);
+    const float *d_mp = (const float *)small(min_p, Bs * 4, 4);
+    const float *d_r = (const float *)small(repetition_penalty, Bs * 4, 4);
+    const float *d_p = (const float *)small(presence_penalty, Bs * 4, 4);
+    const float *d_f = (const float *)small(frequency_penalty, Bs * 4, 4);
     const int32_t *d_hid = (const int32_t *)stage(history_ids, (size_t)history_total * 4);
-    const int32_t *d_hoff = (const int32_t *)small(history_offsets, (Bs + 1) * 4);
-    const uint64_t *d_seeds = (const uint64_t *)small(seeds, Bs * 8);
+    const int32_t *d_hoff = (const int32_t *)small(history_offsets, (Bs + 1) * 4, 4);
+    const uint64_t *d_seeds = (const uint64_t *)small(seeds, Bs * 8, 8);
     bool tok_direct, lp_direct;
     int32_t *d_tok = (int32_t *)result(out_tokens, Bs * 4, tok_direct);
     float *d_lp = (float *)result(out_logprobs, Bs * 4, lp_direct);

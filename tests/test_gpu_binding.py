@@ -54,3 +54,33 @@ def test_out_of_memory_is_torchs(binding):
     with pytest.raises(torch.cuda.OutOfMemoryError):
         s.albireo_sample(x, B=1 << 45)                 # the outputs alone are more than any device holds
     s.close()
+
+
+def test_host_arrays_off_their_alignment_and_shared_with_results(binding):
+    """Through the C ABI: pinned seeds at a 4-byte offset, and results written over an input array, give what plain
+    arrays give (such arrays are copied, not read in place)."""
+    import ctypes as C
+    B, V = 40, 5000
+    s = binding.Sampler(max_rows=B, max_vocab=V, host_staging=True)
+    g = torch.Generator().manual_seed(1)
+    x = torch.randn((B, V), generator=g).pin_memory()
+    k = torch.randint(1, 60, (B,), generator=g, dtype=torch.int32).pin_memory()
+    seeds = torch.randint(0, 1 << 62, (B,), generator=g).pin_memory()
+    want = s.albireo_sample_host(x, top_k=k, seeds=seeds)
+
+    def call(top_k_at, seeds_at, tok_at, lp_at):
+        st = torch.cuda.current_stream(s.device)
+        rc = binding.LIB.albireo_sample_host(s._handle, x.data_ptr(), B, V, binding.F32, None, top_k_at, None, None, None, None, None,
+                                             None, None, 0, seeds_at, 0, tok_at, lp_at, st.cuda_stream, None)
+        assert rc == binding.OK, s.last_error()
+
+    off = torch.zeros(8 * B + 8, dtype=torch.uint8).pin_memory()
+    C.memmove(off.data_ptr() + 4, seeds.data_ptr(), 8 * B)
+    tok, lp = torch.zeros(B, dtype=torch.int32).pin_memory(), torch.zeros(B).pin_memory()
+    call(k.data_ptr(), off.data_ptr() + 4, tok.data_ptr(), lp.data_ptr())
+    assert (tok == want.tokens).all() and (lp == want.logprobs).all()
+    both = torch.zeros(2 * B, dtype=torch.int32).pin_memory()
+    both[B // 2:B // 2 + B] = k
+    call(both.data_ptr() + 4 * (B // 2), seeds.data_ptr(), both.data_ptr(), lp.data_ptr())      # tokens over half of top_k
+    assert (both[:B] == want.tokens).all() and (lp == want.logprobs).all()
+    s.close()
