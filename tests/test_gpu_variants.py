@@ -376,8 +376,9 @@ def test_full_vocabulary_logprobs_full_size_rows(binding, sampler):
 # ------------------------------------------------------------------ programmatic dependent launch
 
 def test_programmatic_launch_gives_the_same_results(binding, sampler):
-    """Back-to-back calls launched with programmatic stream serialisation, the second reading what the
-    first wrote nowhere: each equals the plain launch bit for bit, also inside a captured graph."""
+    """The flag has no effect (every call is launched with programmatic stream serialisation): with it, back to back and
+    inside a captured graph, a call gives what it gives without.  What the launch mode itself must not break is
+    tested by test_a_call_sees_what_the_kernel_ahead_of_it_wrote."""
     w = W.config3(B=32)
     t = binding.workload_tensors(w, sampler.device)
     lg = t.pop("logits")
