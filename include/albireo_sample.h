@@ -60,7 +60,7 @@ enum {
 #define ALBIREO_MAX_PEER_SEGMENTS 16 /* largest num_segments with segment_ptrs            */
 
 /* bits of out_row_status[b] */
-#define ALBIREO_ROW_GENERAL_PATH 1u  /* informational: row took the multi-pass general path */
+#define ALBIREO_ROW_GENERAL_PATH 1u  /* informational: row took several passes (no top-k, or given up by the single one) */
 #define ALBIREO_ROW_BAD_PARAM 2u     /* T < 0 or NaN, r <= 0, ...: row treated per the clamps */
 #define ALBIREO_ROW_HISTORY_OVERFLOW 4u /* history did not fit the workspace: penalties skipped */
 #define ALBIREO_ROW_TIMEOUT 8u       /* a bounded on-chip wait expired: no result for this row;
@@ -77,10 +77,9 @@ enum {
                                          softmax over every finite score of the row (after penalties
                                          and temperature; greedy rows: over the unscaled scores)
                                          instead of the final kept set; the token drawn does not
-                                         change.  Costs one more pass over the row, from L2.  A
-                                         top-N list (num_top > 0) then holds the first entries of the
-                                         whole row's order, not of the kept set; rows with such a
-                                         list take the general path                               */
+                                         change.  Costs one more pass over the row, on chip or from
+                                         L2.  A top-N list (num_top > 0) then holds the first entries
+                                         of the whole row's order, not of the kept set             */
 #define ALBIREO_FLAG_PROGRAMMATIC_LAUNCH 8u /* accepted and without effect: every call is launched with
                                          programmatic stream serialisation.  The kernel's CTAs may be
                                          scheduled while the kernel ahead of it in the stream is still
@@ -172,8 +171,8 @@ typedef struct albireo_sample_ext {
 
 /*
  * Device bytes the caller must provide as `workspace` to albireo_sample_init.
- * The workspace holds per-row history occurrence counts for rows whose history has more
- * distinct ids than fit on chip (sized by max_history_total, the largest
+ * The workspace holds per-row history occurrence counts, or the ids, of rows whose history
+ * has more distinct ids than fit on chip (sized by max_history_total, the largest
  * history_offsets[B] of any call).  Pure function of its arguments; returns 0 on
  * nonsensical input (negative sizes).
  */
