@@ -223,11 +223,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     if (threadIdx.x == 0) fill_general_args(s.ga, a);
     __syncthreads();
 
-    const bool full_lp = (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) != 0, full_list = full_lp && a.num_top > 0;
-    const bool cand_row = candidate_eligible(rp, a);
-    const bool has_topk = rp.greedy || (rp.top_k >= 1 && rp.top_k < V);
-    // (while the slice travels; nobody asks an ordinary top-k row for the number of its finite scores)
-    const uint32_t fin_thr = T::finite_threshold(cand_row && has_topk && !a.out_num_topk ? 1.0f : c.invT);
+    const uint32_t fin_thr = T::finite_threshold(c.invT);       // (while the slice travels)
     // the slice: penalised tokens and (CTA 0) the row's unaligned ends move to the list of extras
     bool landed = true, fits = true;
     int nx = 0;
@@ -260,6 +256,9 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     src.nx = nx; src.xid = xid;
 
     // the slice's maximum, its number of finite scores and every thread's own maximum
+    const bool full_lp = (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) != 0, full_list = full_lp && a.num_top > 0;
+    const bool cand_row = candidate_eligible(rp, a);
+    const bool has_topk = rp.greedy || (rp.top_k >= 1 && rp.top_k < V);
     const int k = rp.greedy ? 1 : rp.top_k, k_eff = full_list ? max(k, a.num_top) : k;
     uint32_t mk = 0, nfin = 0;
     if (landed) {
