@@ -1805,13 +1805,19 @@ __device__ __noinline__ void whole_row_totals(BlockScratch *sp, float zmax) {
     __syncthreads();
 }
 
+// Whether the size of the top-k stage, asked for, is not to be had from the list: it holds fewer than k because of
+// the min-p floor, or there is no top-k.
+template <bool EXTRA>
+__device__ __forceinline__ bool wants_finite_count(const SampleArgs &a, int n, int k, bool has_topk, bool stream_minp) {
+    return EXTRA && a.out_num_topk && (!has_topk || (n < k && stream_minp));
+}
 // From the candidate list cand[0..n) (every element of the row with key >= tau_key, the same in every thread) to the result.
-// `full_fx` != 0: the mass of the whole row, which the log-probabilities are relative to.  `count_finite`
-// is called, by every thread, only where the number of finite scores is asked for and not known.
+// `full_fx` != 0: the mass of the whole row, which the log-probabilities are relative to.  `n_fin`: the number of
+// finite scores, looked at only where wants_finite_count says so.
 // EXTRA: see albireo_sample_kernel.
-template <bool EXTRA, class F>
+template <bool EXTRA>
 __device__ __forceinline__ bool candidate_finish(BlockScratch &s, const CandSmem &cs, int n, uint32_t tau_key, uint32_t kmax, const RowParams &rp,
-                                                 const SampleArgs &a, int b, RowOut &out, u64 full_fx, F &&count_finite) {
+                                                 const SampleArgs &a, int b, RowOut &out, u64 full_fx, u64 n_fin) {
     const int V = a.V;
     const bool full_list = EXTRA && (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) && a.num_top > 0;
     const int k = rp.greedy ? 1 : rp.top_k;
@@ -1819,7 +1825,8 @@ __device__ __forceinline__ bool candidate_finish(BlockScratch &s, const CandSmem
     const bool has_minp = !rp.greedy && rp.min_p > 0.0f;
     const bool stream_minp = floor_while_streaming<EXTRA>(rp, a, has_topk, full_list);
     const int k_list = full_list ? max(k, a.num_top) : k;      // the list holds at least this many (or all there are)
-    bool topk_exact_known = true;      // is min(k, #finite) known without counting?
+    // (compaction below never takes a list of k and more under k)
+    const bool count_wanted = wants_finite_count<EXTRA>(a, n, k, has_topk, stream_minp);
     // keep-ties mode: the top-k stage keeps every score not below the k-th largest, i.e. exactly the
     // candidates that are left once the list is cut at the k-th largest key
     const bool keep_ties = EXTRA && has_topk && !rp.greedy && (a.flags & ALBIREO_FLAG_TOPK_KEEP_TIES);
@@ -1828,19 +1835,14 @@ __device__ __forceinline__ bool candidate_finish(BlockScratch &s, const CandSmem
             uint32_t t = cand_select_exact(s, cs, n, k_list, tau_key, kmax);
             n = cand_compact(s, cs, n, t);
         }
-        if (n < k && stream_minp) topk_exact_known = false;
     } else {
         n = cand_compact(s, cs, n, minp_key(unkey(kmax), rp.ln_min_p));
-        topk_exact_known = false;
     }
     if (n > SORT_MAX || n < 1) return false;
 
     const int L6 = has_topk ? ((n < k || keep_ties) ? n : k) : n;
     int n_topk = L6;
-    if (EXTRA && !topk_exact_known && a.out_num_topk) {
-        const u64 nfin = count_finite();
-        n_topk = has_topk ? (int)(nfin < (u64)k ? nfin : (u64)k) : (int)nfin;
-    }
+    if (count_wanted) n_topk = has_topk ? (int)(n_fin < (u64)k ? n_fin : (u64)k) : (int)n_fin;
     out.n_topk = n_topk;
     // the stream is over: the next kernel in the stream may be scheduled from here on
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -2129,29 +2131,30 @@ __device__ __forceinline__ bool candidate_path(BlockScratch &s, const CandSmem &
     }
     if (ovf || n < 1) return false;
 
-    const uint32_t kmax = s.runmax;    // the row's largest score is always a candidate
-    // passes over the whole row that only some calls ask for, out of line
-    auto totals = [&]() {
-        if (threadIdx.x == 0) passes_begin<DT>(s, c, a.vps, a.nstages);
-        __syncthreads();
-        whole_row_totals<DT>(&s, unkey(kmax));
-    };
-    u64 full_fx = 0;
-    if (EXTRA && (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB)) {
-        totals();
-        full_fx = s.bcast[0];
-        if (s.timeout) { out.status |= ALBIREO_ROW_TIMEOUT; out.token = -1; out.logprob = __uint_as_float(0x7FC00000u); out.n_keep = 0; out.n_topk = 0; return true; }
-        __syncthreads();
-    }
+    uint32_t kmax = s.runmax;          // the row's largest score is always a candidate
     // (tau_key differs from warp to warp, each with the min-p floor it has seen: the block-wide steps from here on
     // take the floor of the row's maximum)
     uint32_t tau = tau_topk;
     if (has_topk && stream_minp) tau = max(tau, min(kmax, minp_key(unkey(kmax), rp.ln_min_p)));
-    return candidate_finish<EXTRA>(s, cs, n, tau, kmax, rp, a, b, out, full_fx, [&]() -> u64 {
-        if (!EXTRA) return 0ull;
-        totals();
-        return s.bcast[1];
-    });
+    u64 full_fx = 0, n_fin = 0;
+    RowParams rq = rp;
+    if constexpr (EXTRA) {
+        const bool full_lp = (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) != 0;
+        if (full_lp || wants_finite_count<EXTRA>(a, n, rp.greedy ? 1 : rp.top_k, has_topk, stream_minp)) {
+            // A pass over the whole row that only some calls ask for, out of line.  What is needed behind it waits in
+            // shared memory: kept in registers it was spilled ahead of the stream for every call (256 rows with counts
+            // 19.5 -> 23.0 us).
+            if (threadIdx.x == 0) { passes_begin<DT>(s, c, a.vps, a.nstages); row_shared().rp = rp; s.bcast[3] = tau; }
+            __syncthreads();
+            whole_row_totals<DT>(&s, unkey(kmax));
+            rq = row_shared().rp;
+            full_fx = full_lp ? s.bcast[0] : 0ull; n_fin = s.bcast[1];
+            tau = (uint32_t)s.bcast[3]; n = (int)s.cand_cnt; kmax = s.runmax;
+            if (s.timeout) { out.status |= ALBIREO_ROW_TIMEOUT; out.token = -1; out.logprob = __uint_as_float(0x7FC00000u); out.n_keep = 0; out.n_topk = 0; return true; }
+            __syncthreads();
+        }
+    }
+    return candidate_finish<EXTRA>(s, cs, n, tau, kmax, rq, a, b, out, full_fx, n_fin);
 }
 
 // ------------------------------------------------------------------ a row's parameters and its results

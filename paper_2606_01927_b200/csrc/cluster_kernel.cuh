@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
                 n = close_gap(cs.cand, CAND_CAP, n_mine, n - n_mine);
                 u64 full_fx = 0;
                 if (full_lp) for (int r = 0; r < tm.size; ++r) full_fx += tm.x->S_all[r];
-                done = candidate_finish<true>(s, cs, n, tau, kmax, rp, a, b, out, full_fx, [&] { return (u64)n_fin; });
+                done = candidate_finish<true>(s, cs, n, tau, kmax, rp, a, b, out, full_fx, n_fin);
             }
         }
         if (wide) {
