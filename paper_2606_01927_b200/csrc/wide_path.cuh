@@ -1,8 +1,9 @@
 // Wide rows: rows whose kept set has no small bound (top-p alone, no cut at all, a min-p that keeps
 // thousands).  Included by albireo_sample.cu.
 //
-// What bounds such a row is instruction issue: every element needs an exponential (its mass), and with
-// no cut a share of a Philox block.  So the row is passed over as few times as the definition allows
+// What such a row costs is instructions: every element needs an exponential (its mass), and with
+// no cut a share of a Philox block; 41 (no cut) to 65 per logit in all, at 28 to 41 % of the issue slots (the largest
+// stalls are instruction fetch, fixed latencies and barriers).  So the row is passed over as few times as the definition allows
 // and each pass does one short fixed sequence per element:
 //   mass    e = exp(z - zmax) summed in fixed point, and, where a cut or a list has to be found, one
 //           32-bit shared-memory add per element into a histogram of masses over bins that are linear
@@ -323,8 +324,7 @@ __device__ __forceinline__ WideSmem wide_smem() {
 // octaves below the maximum is in none: 2^19 such elements weigh 1e-7 of it).  INSIDE_WINDOW: only
 // elements with code in [lo, lo + (W_BINS << shift)), into bins of 2^shift.  S: the masses of the
 // elements with z >= zfloor (inside a window: of those ahead of it), S_all: of all.
-// Bound by issue (about 16 instructions per element) and, on the first level, by the shared-memory
-// adds (one per element, 3 to 5 bank cycles per warp).
+// About 19 instructions per element and, on the first level, a shared-memory add (3 to 5 bank cycles per warp).
 enum MassMode { SUM_ONLY, FIRST_LEVEL, INSIDE_WINDOW };
 template <int DT, int MODE, bool FLOOR, class SRC>
 __device__ __forceinline__ void mass_pass(const SRC &src, float invT, float zmax, float zfloor, uint32_t lo, int shift, u64 &S_out, u64 &S_all_out) {
