@@ -26,6 +26,8 @@
 #include <string.h>
 #include <mutex>
 #include <new>
+#include <type_traits>
+#include <utility>
 
 #include "albireo_sample.h"
 
@@ -154,7 +156,10 @@ struct GenArgs {
     uint64_t step; uint32_t flags; int32_t num_top; int32_t dbg_cap;
 };
 
-// what the last pass of the wide path needs (see final_pass)
+// what the generator's first two rounds leave that does not depend on the token (see philox_row)
+struct PhiloxRow { uint32_t x0, x1, x2, x3, k0, k1; };
+
+// what the last pass of the wide path needs (see race_all)
 struct FinalArgs {
     float invT, zmax, zfloor;
     uint32_t sure, win_hi, top_hi;       // codes: below `sure` kept; [sure, win_hi] to the list; <= top_hi to the top-N list
@@ -162,6 +167,7 @@ struct FinalArgs {
     uint32_t vec_thr;                    // raw threshold of the vector test
     int list_cap;
     u64 *list;                           // the window's list
+    PhiloxRow philox;
     uint64_t seed, step;
     uint32_t R;
     const float *exp1_row;
@@ -183,8 +189,17 @@ struct BlockScratch {
     const char *seg_base[ALBIREO_MAX_SEGMENTS];   // where this row's pieces start (rows in pieces only)
     uint32_t nfin_cap;           // general path: min(#finite scores, ALBIREO_MAX_NUM_TOP + 1), parked here until the list is written
     FinalArgs fa;
+    u64 cut_words[8];            // CountedCut (wide_path.cuh)
+    u64 race_G[NWARPS];          // the race: each warp's best element, the bound so far (see CountedRacer)
+    float race_z[NWARPS];
+    uint32_t race_bound;
     GenArgs ga;                  // the general path's copy of the launch arguments it uses
 };
+
+static_assert(sizeof(BlockScratch) <= 1536, "static shared memory that ring_stages_for counts on");
+// The block's one scratch structure.  Functions that are not inlined name it anew instead of taking it by a pointer: so the
+// compiler knows that it lies in shared memory (through a generic pointer every load is slower, and an atomic many times).
+__device__ __forceinline__ BlockScratch &block_scratch() { __shared__ BlockScratch s; return s; }
 
 __device__ __forceinline__ u64 warp_max_u64(u64 v) {
 #pragma unroll
@@ -197,7 +212,8 @@ __device__ __forceinline__ u64 warp_sum_u64(u64 v) {
     return v;
 }
 // all threads get the result; contains two barriers
-__device__ u64 block_max_u64(BlockScratch &s, u64 v) {
+__device__ u64 block_max_u64(BlockScratch &, u64 v) {
+    BlockScratch &s = block_scratch();
     v = warp_max_u64(v);
     __syncthreads();
     if ((threadIdx.x & 31) == 0) s.red[threadIdx.x >> 5] = v;
@@ -207,7 +223,8 @@ __device__ u64 block_max_u64(BlockScratch &s, u64 v) {
     for (int w = 1; w < NWARPS; ++w) { u64 t = s.red[w]; r = t > r ? t : r; }
     return r;
 }
-__device__ u64 block_sum_u64(BlockScratch &s, u64 v) {
+__device__ u64 block_sum_u64(BlockScratch &, u64 v) {
+    BlockScratch &s = block_scratch();
     v = warp_sum_u64(v);
     __syncthreads();
     if ((threadIdx.x & 31) == 0) s.red[threadIdx.x >> 5] = v;
@@ -218,7 +235,8 @@ __device__ u64 block_sum_u64(BlockScratch &s, u64 v) {
     return r;
 }
 // exclusive prefix sum over threads in thread order; also returns the block total
-__device__ u64 block_exscan_u64(BlockScratch &s, u64 v, u64 &total) {
+__device__ u64 block_exscan_u64(BlockScratch &, u64 v, u64 &total) {
+    BlockScratch &s = block_scratch();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     u64 inc = v;
 #pragma unroll
@@ -250,6 +268,7 @@ struct RowCtx {
     const uint32_t *counts;   // occurrence count per distinct id, indexed by rank in the bitmap
     uint32_t n_distinct;      // number of distinct history ids (set bits of the bitmap)
     int ncoarse;              // entries of `coarse`
+    bool scored;              // in the place of the counts there are the tokens' scores (the wide path of one CTA, and the general path behind it)
 };
 
 __device__ __forceinline__ uint32_t hist_rank(const RowCtx &c, int i) {
@@ -330,7 +349,10 @@ __device__ __forceinline__ const uint4 *vec_ptr(const RowCtx &c, const uint4 *vp
 
 __device__ __forceinline__ float score_of(const RowCtx &c, int i, float x) {
     float a = x;
-    if (c.has_hist && ((c.bitmap[i >> 5] >> (i & 31)) & 1u)) a = penalise(c, i, x);
+    if (c.has_hist && ((c.bitmap[i >> 5] >> (i & 31)) & 1u)) {
+        if (c.scored) return __uint_as_float(c.counts[hist_rank(c, i)]);
+        a = penalise(c, i, x);
+    }
     return __fmul_rn(a, c.invT);
 }
 
@@ -415,6 +437,11 @@ template <class P> struct VecTest16 {
         H2 m = vmax(q);
         return key_of(__fmul_rn(fmaxf(__low2float(m), __high2float(m)), invT));
     }
+    // the largest element of many vectors: packed maxima, a key only at the end
+    typedef H2 Run;
+    static __device__ __forceinline__ Run run_start() { const uint32_t f = P::NEG_INF | (P::NEG_INF << 16); return *reinterpret_cast<const H2 *>(&f); }
+    static __device__ __forceinline__ void run_take(Run &r, const uint4 &q, float) { r = __hmax2(r, vmax(q)); }
+    static __device__ __forceinline__ uint32_t run_key(const Run &r, float invT) { return key_of(__fmul_rn(fmaxf(__low2float(r), __high2float(r)), invT)); }
     static __device__ __forceinline__ uint4 fill() { const uint32_t f = P::NEG_INF | (P::NEG_INF << 16); return make_uint4(f, f, f, f); }
     // the raw threshold that only +inf reaches (NEG_INF without its sign bit), packed twice
     static __device__ __forceinline__ uint32_t pos_inf_threshold() { const uint32_t b = P::NEG_INF & 0x7FFFu; return b | (b << 16); }
@@ -457,6 +484,10 @@ template <> struct VecTest<ALBIREO_F32> {
                ((uint32_t)(__fmul_rn(__uint_as_float(q.z), invT) >= t) << 2) | ((uint32_t)(__fmul_rn(__uint_as_float(q.w), invT) >= t) << 3);
     }
     static __device__ __forceinline__ uint32_t vmax_key(const uint4 &q, float invT) { return key_of(vmaxz(q, invT)); }
+    typedef float Run;
+    static __device__ __forceinline__ Run run_start() { return -INFINITY; }
+    static __device__ __forceinline__ void run_take(Run &r, const uint4 &q, float invT) { r = fmaxf(r, vmaxz(q, invT)); }
+    static __device__ __forceinline__ uint32_t run_key(Run r, float) { return key_of(r); }
     static __device__ __forceinline__ uint4 fill() { return make_uint4(0xFF800000u, 0xFF800000u, 0xFF800000u, 0xFF800000u); }
     static __device__ __forceinline__ uint32_t pos_inf_threshold() { return 0x7F800000u; }
     static __device__ __forceinline__ uint32_t finite_threshold(float) { return __float_as_uint(unkey(KEY_MIN_FINITE)); }
@@ -482,6 +513,7 @@ __device__ __forceinline__ void for_each_score_rest(const RowCtx &c, int head, i
     if (c.has_hist) {
         for (uint32_t r = threadIdx.x; r < c.n_distinct; r += NT) {
             const int i = hist_id_of_rank(c, r);
+            if (c.scored) { fn(i, __uint_as_float(c.counts[r])); continue; }
             const float x = E::load(elem_ptr<DT>(c, i), 0);
             const float av = penalise_counted(c, x, c.counts[r]);
             fn(i, __fmul_rn(av, c.invT));
@@ -574,7 +606,8 @@ struct HistSmem {
 };
 
 // exclusive prefix sum of 32-bit values over the threads of the block (thread order); block total in `total`
-__device__ uint32_t block_exscan_u32(BlockScratch &s, uint32_t v, uint32_t &total) {
+__device__ uint32_t block_exscan_u32(BlockScratch &, uint32_t v, uint32_t &total) {
+    BlockScratch &s = block_scratch();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t inc = v;
 #pragma unroll
@@ -610,8 +643,9 @@ __device__ __forceinline__ void hist_prefetch(const int32_t *ids, int len, int32
 // Ids before position out_start are the prompt: they set their bit (repetition penalty) but are not counted.
 // Histories repeat a few ids very often: a bit already set is not set again.  (Combining equal ids
 // within a warp first, with match.any, was measured and cost far more than the atomics it saved.)
-__device__ bool build_history(BlockScratch &s, const HistSmem &hs, RowCtx &c, const int32_t *ids, int len, int out_start,
+__device__ bool build_history(BlockScratch &, const HistSmem &hs, RowCtx &c, const int32_t *ids, int len, int out_start,
                               const int32_t *staged, uint32_t *ws, int64_t ws_cap, int64_t ws_off) {
+    BlockScratch &s = block_scratch();
     const int V = c.V;
     const int nwords = (V + 31) >> 5, ncoarse = (nwords + 7) >> 3;
     const int nst = len < HIST_STAGED ? len : HIST_STAGED;
@@ -809,7 +843,8 @@ struct MassSum {
 // was just read, so mostly from L2), four loads in flight; vectors with nothing within 29 of the
 // maximum carry no mass and are skipped by the packed test of the candidate path.  The same in every thread.
 template <int DT>
-__device__ u64 full_vocab_mass(BlockScratch &s, const RowCtx &c, float zmax) {
+__device__ u64 full_vocab_mass(BlockScratch &, const RowCtx &c, float zmax) {
+    BlockScratch &s = block_scratch();
     typedef Elem<DT> E;
     typedef VecTest<DT> T;
     const int V = c.V;
@@ -856,8 +891,9 @@ __device__ __forceinline__ int bitlen64(u64 v) { return 64 - __clzll((long long)
 
 // Finds the first bin (from bin 0) at which the running total of the steering histogram reaches
 // `target` (1 <= target <= grand total).  Gives the totals of both histograms strictly before it.
-__device__ bool find_prefix_bin(BlockScratch &s, const HistBins &h, bool by_mass, bool have_mass, u64 target,
+__device__ bool find_prefix_bin(BlockScratch &, const HistBins &h, bool by_mass, bool have_mass, u64 target,
                                 int &bin, u64 &cnt_before, u64 &mass_before) {
+    BlockScratch &s = block_scratch();
     constexpr int PER = HIST_BINS / NT;
     u64 lc = 0, lm = 0;
 #pragma unroll
@@ -887,7 +923,8 @@ __device__ bool find_prefix_bin(BlockScratch &s, const HistBins &h, bool by_mass
 // Gathers the composites accepted by `take` into h.list (at most GL_CAP are stored); returns how many
 // were accepted, and their smallest and largest composite.
 template <int DT, class F>
-__device__ int gather_if(BlockScratch &s, const HistBins &h, const RowCtx &c, F &&take, u64 &cmin, u64 &cmax) {
+__device__ int gather_if(BlockScratch &, const HistBins &h, const RowCtx &c, F &&take, u64 &cmin, u64 &cmax) {
+    BlockScratch &s = block_scratch();
     if (threadIdx.x == 0) s.list_cnt = 0;
     __syncthreads();
     u64 mn = ~0ull, mx = 0;
@@ -913,7 +950,7 @@ __device__ int gather_if(BlockScratch &s, const HistBins &h, const RowCtx &c, F 
 // (out of line, and given plain pointers only, so that it neither shapes the register allocation of
 // its callers nor forces their structures into local memory)
 __device__ __noinline__ u64 list_resolve(BlockScratch *sp, u64 *list, int n, bool by_mass, u64 target, u64 lo, u64 hi, float zmax) {
-    BlockScratch &s = *sp;
+    BlockScratch &s = block_scratch();
     struct { u64 *list; } h = {list};
     int P = 2;
     while (P < n) P <<= 1;
@@ -963,8 +1000,9 @@ __device__ __noinline__ u64 list_resolve(BlockScratch *sp, u64 *list, int n, boo
 // the order, over elements with C >= floorC) first reaches `target`, given that it falls in value bin
 // `bin` and that `before` of the total lies in the bins ahead of it.
 template <int DT>
-__device__ u64 resolve_cut(BlockScratch &s, const HistBins &h, const RowCtx &c, float zmax, int bin, bool by_mass,
+__device__ u64 resolve_cut(BlockScratch &, const HistBins &h, const RowCtx &c, float zmax, int bin, bool by_mass,
                            u64 target, u64 before, u64 floorC, bool &hist_clobbered) {
+    BlockScratch &s = block_scratch();
     u64 rel = target - before;
     u64 lo, hi;
     int n = gather_if<DT>(s, h, c, [&](u64 C, float z) { return C >= floorC && (C >> 32) < KEY_POS_INF && bin_of(z, zmax) == bin; }, lo, hi);
@@ -1360,8 +1398,9 @@ __device__ __forceinline__ uint32_t warp_incl_scan_u32(uint32_t v) {
 // holds the k-th largest such key.  Returns false if fewer than k keys are in range.
 // On success [lo, hi] is narrowed to that bin and k to the rank inside it; `shift` tells
 // the bin width (0: the bin is a single key, i.e. lo is exactly the k-th largest key).
-__device__ bool cand_select_pass(BlockScratch &s, const CandSmem &cs, int n, uint32_t &k, uint32_t &lo, uint32_t &hi, int &shift,
+__device__ bool cand_select_pass(BlockScratch &, const CandSmem &cs, int n, uint32_t &k, uint32_t &lo, uint32_t &hi, int &shift,
                                  bool zeroed = false) {
+    BlockScratch &s = block_scratch();
     const uint32_t width = hi - lo;
     shift = width < (uint32_t)SEL_BINS ? 0 : (32 - __clz(width)) - 9;
     if (!zeroed) {          // (a caller that zeroed the bins and found_digit before its last barrier skips this)
@@ -1403,7 +1442,8 @@ __device__ bool cand_select_pass(BlockScratch &s, const CandSmem &cs, int n, uin
 // Lower bound t of the k-th largest key in [lo, hi]: count(key >= t) >= k.  One pass when the
 // keys spread over the bins; an outlier that stretches the range leaves most keys in one bin, and
 // then up to two more passes narrow that bin.
-__device__ uint32_t cand_select_approx(BlockScratch &s, const CandSmem &cs, int n, int k, uint32_t lo, uint32_t hi, bool zeroed = false) {
+__device__ uint32_t cand_select_approx(BlockScratch &, const CandSmem &cs, int n, int k, uint32_t lo, uint32_t hi, bool zeroed = false) {
+    BlockScratch &s = block_scratch();
     uint32_t kk = (uint32_t)k; int shift = 1;
     for (int pass = 0; pass < 3 && shift != 0; ++pass) {
         if (!cand_select_pass(s, cs, n, kk, lo, hi, shift, zeroed && pass == 0)) break;   // on failure lo is unchanged
@@ -1414,7 +1454,8 @@ __device__ uint32_t cand_select_approx(BlockScratch &s, const CandSmem &cs, int 
     return lo;
 }
 // The k-th largest key in [lo, hi] exactly (as many passes as the key range needs).
-__device__ uint32_t cand_select_exact(BlockScratch &s, const CandSmem &cs, int n, int k, uint32_t lo, uint32_t hi) {
+__device__ uint32_t cand_select_exact(BlockScratch &, const CandSmem &cs, int n, int k, uint32_t lo, uint32_t hi) {
+    BlockScratch &s = block_scratch();
     uint32_t kk = (uint32_t)k; int shift = 1;
     for (int pass = 0; pass < 5 && shift != 0; ++pass)
         if (!cand_select_pass(s, cs, n, kk, lo, hi, shift)) break;
@@ -1422,7 +1463,8 @@ __device__ uint32_t cand_select_exact(BlockScratch &s, const CandSmem &cs, int n
 }
 
 // keeps the candidates with key >= tkey (and drops empty slots); returns the new count
-__device__ int cand_compact(BlockScratch &s, const CandSmem &cs, int n, uint32_t tkey) {
+__device__ int cand_compact(BlockScratch &, const CandSmem &cs, int n, uint32_t tkey) {
+    BlockScratch &s = block_scratch();
     constexpr int PER = CAND_CAP / NT;
     u64 mine[PER];
     uint32_t cnt = 0;
@@ -1647,7 +1689,8 @@ __device__ __forceinline__ void final_stage(BlockScratch &s, const CandSmem &cs,
 // warp then finds the bin in which the count from the top reaches k and the answer is that bin's
 // smallest key: at least k maxima are not below it.  Returns 0 if there are fewer than k maxima.
 // Needs cs.hist zero and the bin minima 0xFFFFFFFF on entry; contains two barriers, the last at the end.
-__device__ uint32_t warm_select(BlockScratch &s, const CandSmem &cs, uint32_t mk, int k, uint32_t kmin, uint32_t kmax) {
+__device__ uint32_t warm_select(BlockScratch &, const CandSmem &cs, uint32_t mk, int k, uint32_t kmin, uint32_t kmax) {
+    BlockScratch &s = block_scratch();
     uint32_t *binmin = (uint32_t *)(cs.cand + SEL_BINS);
     const float zmin = unkey(kmin), d = unkey(kmax) - zmin;
     const float scale = (d > 0.0f && d <= 3.0e38f) ? __fdividef((float)(SEL_BINS - 1), d) : 0.0f;
@@ -1701,7 +1744,8 @@ __device__ __forceinline__ void ring_setup(BlockScratch &s, const Ring &rg) {
 }
 // The first copies of the row (thread 0 only; after ring_setup).
 template <int DT>
-__device__ void candidate_begin(BlockScratch &s, const Ring &rg, const RowCtx &c) {
+__device__ void candidate_begin(BlockScratch &, const Ring &rg, const RowCtx &c) {
+    BlockScratch &s = block_scratch();
     typedef Elem<DT> E;
     if (threadIdx.x != 0) return;
     const uintptr_t addr = (uintptr_t)c.row;
@@ -1768,7 +1812,7 @@ __device__ __forceinline__ void passes_end() {
 // The row's largest order key (s.mm_max) and the number of its finite scores (s.list_cnt), after passes_begin.
 template <int DT>
 __device__ __noinline__ void max_and_count(BlockScratch *sp) {
-    BlockScratch &s = *sp;
+    BlockScratch &s = block_scratch();
     const RingSlice<DT> src;
     const float invT = row_shared().c.invT;
     const uint32_t fin_thr = VecTest<DT>::finite_threshold(invT);
@@ -1791,7 +1835,7 @@ __device__ __noinline__ void max_and_count(BlockScratch *sp) {
 // The mass of every finite score of the row (s.bcast[0]) and their number (s.bcast[1]), after passes_begin.
 template <int DT>
 __device__ __noinline__ void whole_row_totals(BlockScratch *sp, float zmax) {
-    BlockScratch &s = *sp;
+    BlockScratch &s = block_scratch();
     max_and_count<DT>(sp);
     u64 S, S_all;
     mass_pass<DT, SUM_ONLY, false>(RingSlice<DT>(), row_shared().c.invT, zmax, 0.0f, 0u, 0, S, S_all);
@@ -2178,7 +2222,7 @@ __device__ __forceinline__ uint32_t load_row(const SampleArgs &a, int b, const c
     c.row = (const char *)a.logits + (size_t)b * (size_t)a.row_stride * Elem<DT>::SIZE;
     if (a.nseg > 1 && a.seg_ptr_count > 0) c.row = (const char *)a.seg_ptr[0] + (size_t)(a.seg_row_offset + b) * (size_t)a.row_stride * Elem<DT>::SIZE;
     c.V = a.V; c.nseg = a.nseg; c.Vs = a.Vs; c.seg_base = seg_base;
-    c.has_hist = false; c.bitmap = nullptr; c.coarse = nullptr; c.counts = nullptr; c.n_distinct = 0; c.ncoarse = 0;
+    c.has_hist = false; c.bitmap = nullptr; c.coarse = nullptr; c.counts = nullptr; c.n_distinct = 0; c.ncoarse = 0; c.scored = false;
     return ((rp.T < 0.0f || rp.T != rp.T) || !(c.r > 0.0f)) ? ALBIREO_ROW_BAD_PARAM : 0u;
 }
 __device__ __forceinline__ void fill_general_args(GenArgs &ga, const SampleArgs &a) {
@@ -2210,6 +2254,24 @@ __device__ __forceinline__ void store_row(const SampleArgs &a, int b, RowOut &ou
     }
 }
 
+// The row's context with the history tables of this CTA's row, at tab_off (no copy is in flight, the front of the shared memory is free);
+// without (has_hist) where there is no history, or no room for them.
+__device__ __noinline__ RowCtx row_history(const SampleArgs *ap, int tab_off, RowCtx c) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    const SampleArgs &a = *ap;
+    const int b = blockIdx.x, o0 = a.hist_off[b], o1 = a.hist_off[b + 1];
+    if (o1 <= o0) return c;
+    HistSmem hs;
+    const int nwords = (a.V + 31) >> 5, ncoarse = (nwords + 7) >> 3;
+    hs.bitmap = (uint32_t *)(smem + tab_off);
+    hs.coarse = hs.bitmap + (nwords + 1);
+    hs.counts = hs.coarse + (ncoarse + 1);
+    hist_prefetch(a.hist_ids + o0, o1 - o0, (int32_t *)smem);
+    c.has_hist = build_history(block_scratch(), hs, c, a.hist_ids + o0, o1 - o0, a.out_start ? a.out_start[b] : 0, (const int32_t *)smem,
+                               a.ws_counts, a.ws_counts_cap, (int64_t)o0);
+    return c;
+}
+
 // A row that the candidate path does not take or had to give up, by one CTA from global memory: the wide
 // path where it applies, else the general path.  It starts from the launch arguments alone (and builds
 // the history tables itself): whatever the streaming path would have to keep for it stayed in registers
@@ -2219,43 +2281,87 @@ __device__ __forceinline__ void store_row(const SampleArgs &a, int b, RowOut &ou
 template <int DT>
 __device__ __noinline__ void leftover_row(BlockScratch *sp, const SampleArgs *ap, int tab_off) {
     extern __shared__ __align__(128) unsigned char smem[];
-    BlockScratch &s = *sp;
+    BlockScratch &s = block_scratch();
     const SampleArgs &a = *ap;
     const int b = blockIdx.x;
     RowParams rp;
     RowCtx c;
     uint32_t status = load_row<DT>(a, b, s.seg_base, rp, c);
     if (a.hist_ids && a.hist_off) {
-        const int o0 = a.hist_off[b], o1 = a.hist_off[b + 1];
-        if (o1 > o0) {
-            HistSmem hs;
-            const int nwords = (a.V + 31) >> 5, ncoarse = (nwords + 7) >> 3;
-            hs.bitmap = (uint32_t *)(smem + tab_off);
-            hs.coarse = hs.bitmap + (nwords + 1);
-            hs.counts = hs.coarse + (ncoarse + 1);
-            hist_prefetch(a.hist_ids + o0, o1 - o0, (int32_t *)smem);
-            c.has_hist = build_history(s, hs, c, a.hist_ids + o0, o1 - o0, a.out_start ? a.out_start[b] : 0, (const int32_t *)smem,
-                                       a.ws_counts, a.ws_counts_cap, (int64_t)o0);
-            if (!c.has_hist) status |= ALBIREO_ROW_HISTORY_OVERFLOW;
-        }
+        c = row_history(ap, tab_off, c);
+        if (!c.has_hist && a.hist_off[b + 1] > a.hist_off[b]) status |= ALBIREO_ROW_HISTORY_OVERFLOW;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         fill_general_args(s.ga, a);
         passes_begin<DT>(s, c, a.vps, a.nstages);
         row_shared().rp = rp;
+        s.race_bound = NO_BOUND;
+    }
+    // The penalised tokens' scores take the place of their counts: the passes look them up, where each of them would fetch
+    // their logits again (a scattered load per token and pass, 2 us a round next to CTAs that stream).
+    const bool score = c.has_hist && wide_eligible(rp, a);
+    if (score) {
+        constexpr int PG = 4;
+        for (uint32_t r0 = threadIdx.x; r0 < c.n_distinct; r0 += PG * NT) {
+            float x[PG];
+#pragma unroll
+            for (int u = 0; u < PG; ++u) { const uint32_t r = r0 + u * NT; x[u] = r < c.n_distinct ? Elem<DT>::load(elem_ptr<DT>(c, hist_id_of_rank(c, r)), 0) : 0.0f; }
+#pragma unroll
+            for (int u = 0; u < PG; ++u) {
+                const uint32_t r = r0 + u * NT;
+                uint32_t *at = const_cast<uint32_t *>(c.counts) + r;
+                if (r < c.n_distinct) *at = __float_as_uint(__fmul_rn(penalise_counted(c, x[u], *at), c.invT));
+            }
+        }
     }
     __syncthreads();
+    if (threadIdx.x == 0) row_shared().c.scored = score;
     RowOut out;
     out.status = status | ROW_NOT_DONE;
     if (wide_eligible(rp, a)) {
         const RowShared &r = row_shared();
+        const RingSlice<DT> src;
         SoloTeam tm;
-        tm.x = (TeamWords *)(smem + TEAM_OFF);
-        max_and_count<DT>(sp);
-        const uint32_t kmax = s.mm_max, n_fin = s.list_cnt;
-        __syncthreads();
-        if (kmax >= KEY_MIN_FINITE) out = wide_row<DT>(s, RingSlice<DT>(), tm, r.rp, r.c.invT, kmax, n_fin, b, status);
+        uint32_t kmax = 0, n_fin = 0;
+        out.status = status | ROW_NOT_COUNTED;
+        if constexpr (DT == ALBIREO_BF16) {
+            if (counted_eligible<DT>(rp, c, a)) {
+                // (with no cut the row's first tile is still where the stream put it: its largest score is what the race is run against)
+                const bool race = nothing_cut(rp, a);
+                uint4 q = VecTest<DT>::fill();
+                int ends = 0;
+                if (race && (int)threadIdx.x < r.nvec) {
+                    q = ((const uint4 *)(smem + COMMON_BYTES))[threadIdx.x];
+                    const int i0 = r.head + (int)threadIdx.x * Elem<DT>::PER_VEC;
+                    if (c.has_hist) q = kill_elements<DT>(q, __funnelshift_r(c.bitmap[i0 >> 5], c.bitmap[(i0 >> 5) + 1], i0 & 31));
+                }
+                const float zref = race ? race_reference(s, q, c.invT, rp) : 0.0f;
+                counted_clear();
+                // the penalised tokens among the row's vectors
+                if (c.has_hist) {
+                    const int tail0 = src.end_id(), x = (int)threadIdx.x, i = x < r.head ? x : tail0 + (x - r.head);
+                    ends = __syncthreads_count(x < r.head + (c.V - tail0) && ((c.bitmap[i >> 5] >> (i & 31)) & 1u));
+                } else __syncthreads();
+                const uint32_t killed = c.has_hist ? c.n_distinct - (uint32_t)ends : 0u;
+                run_counting(src, s, race, r.c.invT, zref);
+                __syncthreads();
+                uint32_t flags;
+                n_fin = counted_finite(src, s, r.c.invT, killed, flags) + s.list_cnt;
+                kmax = s.mm_max;
+                __syncthreads();
+                if (kmax >= KEY_MIN_FINITE && !r.timeout) out = counted_row(sp, src, tm, r.rp, r.c.invT, kmax, n_fin, flags, b, status);
+            }
+        }
+        if (out.status & ROW_NOT_COUNTED) {
+            out.status = status | ROW_NOT_DONE;
+            if (kmax == 0) {
+                max_and_count<DT>(sp);
+                kmax = s.mm_max; n_fin = s.list_cnt;
+                __syncthreads();
+            }
+            if (kmax >= KEY_MIN_FINITE) out = wide_row<DT>(s, src, tm, r.rp, r.c.invT, kmax, n_fin, b, status);
+        }
         if (r.timeout) { out.status = (out.status & ~ROW_NOT_DONE) | ALBIREO_ROW_TIMEOUT; out.token = -1; out.logprob = __uint_as_float(0x7FC00000u); out.n_keep = 0; out.n_topk = 0; }
     }
     if (out.status & ROW_NOT_DONE) {
@@ -2279,7 +2385,7 @@ __device__ __noinline__ void leftover_row(BlockScratch *sp, const SampleArgs *ap
 template <int DT, bool EXTRA>
 __global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const __grid_constant__ SampleArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ BlockScratch s;
+    BlockScratch &s = block_scratch();
     const int b = blockIdx.x;
     const int V = a.V;
 
@@ -2349,7 +2455,7 @@ __global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const __grid_cons
     if (rp.T < 0.0f || rp.T != rp.T) out.status |= ALBIREO_ROW_BAD_PARAM;
 
     c.invT = rp.greedy ? 1.0f : __fdiv_rn(1.0f, rp.T);
-    c.has_hist = false; c.bitmap = nullptr; c.coarse = nullptr; c.counts = nullptr; c.n_distinct = 0; c.ncoarse = 0;
+    c.has_hist = false; c.bitmap = nullptr; c.coarse = nullptr; c.counts = nullptr; c.n_distinct = 0; c.ncoarse = 0; c.scored = false;
     if (!(c.r > 0.0f)) out.status |= ALBIREO_ROW_BAD_PARAM;
 
     const bool try_candidates = ring_started && candidate_eligible(rp, a);

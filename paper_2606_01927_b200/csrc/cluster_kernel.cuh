@@ -12,6 +12,7 @@
 
 constexpr int SLICE_MIN = 18 * 1024;      // the final stage's scratch lies in CTA 0's slice when that is done with
 constexpr int X_LEAST = 1024;             // penalised tokens and unaligned ends of a slice that are listed on chip, at least
+constexpr int COUNTED_SLICE = 16384;      // elements of a slice from which on its values are counted (see counted_row)
 constexpr int X_ENDS = 16;                // most unaligned ends of a row (14), rounded up
 constexpr int GENERAL_BYTES = HIST_BINS * 16 + GL_CAP * 8 + 4096;      // what the general path lays over the front
 
@@ -23,8 +24,9 @@ __host__ __device__ constexpr int slice_counts_off(int n) { return slice_coarse_
 // The k-th and the kp-th largest of the block's per-thread maxima `mk` (0: none), from below: the
 // smallest maximum of the value-linear bin in which the count from the top gets there (see
 // warm_select).  0 where there are fewer maxima.
-__device__ void slice_select(BlockScratch &s, const CandSmem &cs, uint32_t mk, int k, int kp, uint32_t kmin, uint32_t kmax,
+__device__ void slice_select(BlockScratch &, const CandSmem &cs, uint32_t mk, int k, int kp, uint32_t kmin, uint32_t kmax,
                              uint32_t &tau, uint32_t &tau_part) {
+    BlockScratch &s = block_scratch();
     uint32_t *binmin = (uint32_t *)(cs.cand + SEL_BINS);
     const float zmin = unkey(kmin), d = unkey(kmax) - zmin;
     const float scale = (d > 0.0f && d <= 3.0e38f) ? __fdividef((float)(SEL_BINS - 1), d) : 0.0f;
@@ -77,7 +79,7 @@ __device__ __noinline__ int slice_history(BlockScratch *sp, RowCtx c, const int3
                                           int id_lo, int id_hi, int tab_off, int list_words, uint32_t *ws, int64_t ws_cap, int64_t ws_off,
                                           W landed, bool &ok, int *&xid) {
     typedef Elem<DT> E;
-    BlockScratch &s = *sp;
+    BlockScratch &s = block_scratch();
     extern __shared__ __align__(128) unsigned char smem[];
     const int nwords = (nids + 31) >> 5, ncoarse = (nwords + 7) >> 3;
     uint32_t *bitmap = (uint32_t *)(smem + tab_off), *coarse = bitmap + slice_coarse_off(nids), *counts = bitmap + slice_counts_off(nids);
@@ -151,9 +153,8 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     typedef Elem<DT> E;
     typedef VecTest<DT> T;
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ BlockScratch s;
+    BlockScratch &s = block_scratch();
     ClusterTeam tm;
-    tm.x = (TeamWords *)(smem + TEAM_OFF);
     tm.rank = (int)cg::this_cluster().block_rank(); tm.size = (int)cg::this_cluster().num_blocks();
     const int b = blockIdx.x / tm.size, V = a.V, lane = threadIdx.x & 31;
     uint64_t *bar = (uint64_t *)(smem + SLICE_OFF + a.slice_bytes);
@@ -170,7 +171,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
         mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        s.cand_cnt = 0; s.runmax = 0; s.mm_max = 0; s.mm_min = 0xFFFFFFFFu; s.list_cnt = 0;
+        s.cand_cnt = 0; s.runmax = 0; s.race_bound = NO_BOUND; s.mm_max = 0; s.mm_min = 0xFFFFFFFFu; s.list_cnt = 0;
         tm.x->far_cand = 0; tm.x->far_list = 0;
     }
     if (threadIdx.x < NWARPS) s.red[threadIdx.x] = 0;
@@ -233,6 +234,11 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     // (a launch without histories has no tables: only the row's unaligned ends are listed)
     src.xz_off = tables ? tab_off + slice_counts_off(n_slice_ids) * 4 : tab_off;
     int *xid = (int *)(smem + src.xz_off) + (a.list_words >> 1);
+    // (Rows are counted by value where a cut or a list has to be found, and in slices that are worth clearing and adding up a
+    // table of 8192 counts: 32 top-p rows of 128256 by 4 CTAs 26.6 -> 23.7 us, but 13 of 50257 by 8 21.2 -> 23.1.  With no cut
+    // the pass of masses and race is faster than counting and race, 22.4 us against 24.5 for 64 rows of 152064.)
+    const bool cand_row = candidate_eligible(rp, a), counted = !cand_row && nv * E::PER_VEC >= COUNTED_SLICE && !nothing_cut(rp, a) && counted_eligible<DT>(rp, c, a);
+    if (counted) counted_clear();
     if (o1 > o0) {
         nx = slice_history<DT>(&s, c, a.hist_ids + o0, o1 - o0, ostart, SLICE_OFF, id0, n_slice_ids, tm.rank == 0 ? head : 0,
                                tm.rank == 0 ? tail0 : V, tab_off, a.list_words, a.ws_counts, a.ws_counts_cap, (int64_t)o0,
@@ -257,16 +263,28 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
 
     // the slice's maximum, its number of finite scores and every thread's own maximum
     const bool full_lp = (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) != 0, full_list = full_lp && a.num_top > 0;
-    const bool cand_row = candidate_eligible(rp, a);
     const bool has_topk = rp.greedy || (rp.top_k >= 1 && rp.top_k < V);
     const int k = rp.greedy ? 1 : rp.top_k, k_eff = full_list ? max(k, a.num_top) : k;
     uint32_t mk = 0, nfin = 0;
-    if (landed) {
-        src.vectors([&](const uint4 &q, int) {
-            const uint32_t kk = T::vmax_key(q, c.invT);
-            mk = kk > mk ? kk : mk;
+    if (counted) {
+        if constexpr (DT == ALBIREO_BF16) {
+            __syncthreads();
+            if (__all_sync(0xFFFFFFFFu, landed)) counting_pass<0, false>(src, &s, c.invT, 0.0f);
+        }
+    } else if (landed) {
+        // (the number of finite scores is wanted for rows that may turn out to be wide, and by calls that ask for the top-k stage's size)
+        const bool count = !cand_row || !has_topk || a.out_num_topk;
+        typename T::Run run = T::run_start();
+        if (count) src.vectors([&](const uint4 &q, int) {
+            T::run_take(run, q, c.invT);
             nfin += (uint32_t)E::PER_VEC - T::count_not_finite(q, fin_thr, c.invT);
         });
+        else {
+            const uint4 *vec = (const uint4 *)(smem + SLICE_OFF);
+#pragma unroll 4
+            for (int v = threadIdx.x; v < nv; v += NT) T::run_take(run, vec[v], c.invT);
+        }
+        mk = T::run_key(run, c.invT);
         src.extras([&](int, float z) {
             const uint32_t kk = key_of(z);
             mk = kk > mk ? kk : mk;
@@ -280,7 +298,8 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
         if (lane == 0) { if (wmx) { atomicMax(&s.mm_max, wmx); atomicMin(&s.mm_min, wmn); } if (wn) atomicAdd(&s.list_cnt, wn); }
     }
     const bool any_late = __syncthreads_or(!landed) != 0;
-    uint32_t kmax = s.mm_max, tau_s = 0, tau_p = 0;
+    uint32_t kmax = s.mm_max, tau_s = 0, tau_p = 0, counted_flags = 0, n_vec = 0;
+    if constexpr (DT == ALBIREO_BF16) { if (counted) n_vec = counted_finite(src, s, c.invT, distinct, counted_flags); }
     if (cand_row && has_topk && kmax) slice_select(s, cs, mk, k_eff, (k_eff + tm.size - 1) / tm.size, s.mm_min, kmax, tau_s, tau_p);
     asm volatile("barrier.cluster.wait;" ::: "memory");            // (the arrival at the start)
     if ((int)threadIdx.x < tm.size) {
@@ -288,8 +307,8 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
         *tm.at(&tm.x->kmax[tm.rank], r) = kmax;
         *tm.at(&tm.x->tau[tm.rank], r) = tau_s;
         *tm.at(&tm.x->tau_part[tm.rank], r) = tau_p;
-        *tm.at(&tm.x->nfin[tm.rank], r) = s.list_cnt;
-        *tm.at(&tm.x->flags[tm.rank], r) = (any_late ? 0x80000000u : 0u) | (fits ? 0u : 0x40000000u) | (distinct + tm.x->far_list);
+        *tm.at(&tm.x->nfin[tm.rank], r) = s.list_cnt + n_vec;
+        *tm.at(&tm.x->flags[tm.rank], r) = (any_late ? 0x80000000u : 0u) | (fits ? 0u : 0x40000000u) | counted_flags | (distinct + tm.x->far_list);
     }
     tm.sync();
     // (a slot per lane: a loop over the slots would be a chain of shared-memory latencies)
@@ -299,7 +318,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     const uint32_t tau_part = __reduce_min_sync(0xFFFFFFFFu, has_slot ? tm.x->tau_part[lane] : 0xFFFFFFFFu);
     const uint32_t n_fin = __reduce_add_sync(0xFFFFFFFFu, has_slot ? tm.x->nfin[lane] : 0u);
     const uint32_t flags_r = has_slot ? tm.x->flags[lane] : 0u;
-    const uint32_t bad = __reduce_or_sync(0xFFFFFFFFu, flags_r) & 0xC0000000u, distinct_row = __reduce_add_sync(0xFFFFFFFFu, flags_r & 0x3FFFFFFFu);
+    const uint32_t bad = __reduce_or_sync(0xFFFFFFFFu, flags_r) & 0xF0000000u, distinct_row = __reduce_add_sync(0xFFFFFFFFu, flags_r & 0x0FFFFFFFu);
     // what only the one-CTA path decides: too many distinct ids for the tables or for the caller's workspace
     const bool to_general = (bad & 0x40000000u) || kmax == 0 || !(cand_row || wide_eligible(rp, a)) ||
                             (distinct_row > (uint32_t)CNT_CAP && (int64_t)o0 + distinct_row > a.ws_counts_cap);
@@ -316,21 +335,17 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
             if (!has_topk || tau < KEY_MIN_FINITE) tau = KEY_MIN_FINITE;
             if (stream_minp) tau = max(tau, min(kmax, minp_key(unkey(kmax), rp.ln_min_p)));
             const uint32_t thr = T::raw_threshold(tau, c.invT);
-            // survivors one per lane at a time (most vectors have none, the rest one or two)
+            // a thread's survivors of a vector (most have none, the rest one or two) take their places in the list together
             src.vectors([&](const uint4 &q, int i0) {
                 uint32_t bits = T::may_pass(q, thr, c.invT) ? T::elem_bits(q, thr, c.invT) : 0u;
-                while (__any_sync(0xFFFFFFFFu, bits != 0)) {
-                    const int x = __ffs(bits | 0x80000000u) - 1;
-                    const uint32_t key = key_of(__fmul_rn(pick_element<DT>(q, x), c.invT));
-                    const bool take = bits != 0 && key >= tau && key < KEY_POS_INF;
-                    const uint32_t m = __ballot_sync(0xFFFFFFFFu, take);
-                    if (m) {
-                        uint32_t base = 0;
-                        if (lane == 0) base = atomicAdd(&s.cand_cnt, (uint32_t)__popc(m));
-                        const uint32_t slot = __shfl_sync(0xFFFFFFFFu, base, 0) + (uint32_t)__popc(m & ((1u << lane) - 1u));
-                        if (take && slot < (uint32_t)CAND_CAP) cs.cand[slot] = comp_of(key, i0 + x);
-                    }
-                    bits &= bits - 1u;
+                if (!bits) return;
+                auto key_at = [&](int x) { return key_of(__fmul_rn(pick_element<DT>(q, x), c.invT)); };
+                uint32_t in = 0;
+                for (uint32_t r = bits; r; r &= r - 1u) { const uint32_t key = key_at(__ffs(r) - 1); in |= key >= tau && key < KEY_POS_INF ? r & -r : 0u; }
+                uint32_t slot = in ? atomicAdd(&s.cand_cnt, (uint32_t)__popc(in)) : 0u;
+                for (; in; in &= in - 1u, ++slot) {
+                    const int x = __ffs(in) - 1;
+                    if (slot < (uint32_t)CAND_CAP) cs.cand[slot] = comp_of(key_at(x), i0 + x);
                 }
             });
             src.extras([&](int i, float z) {
@@ -369,7 +384,9 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
         }
         if (wide) {
             const uint32_t status = out.status;
-            out = wide_row<DT>(s, src, tm, rp, c.invT, kmax, n_fin, b, status);
+            out.status |= ROW_NOT_COUNTED;
+            if constexpr (DT == ALBIREO_BF16) { if (counted) out = counted_row(&s, src, tm, rp, c.invT, kmax, n_fin, bad, b, status); }
+            if (out.status & ROW_NOT_COUNTED) out = wide_row<DT>(s, src, tm, rp, c.invT, kmax, n_fin, b, status);
             done = !(out.status & ROW_NOT_DONE);
             if (!done) out.status = status;
         }

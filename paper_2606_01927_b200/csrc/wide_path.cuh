@@ -1,10 +1,9 @@
 // Wide rows: rows whose kept set has no small bound (top-p alone, no cut at all, a min-p that keeps
 // thousands).  Included by albireo_sample.cu.
 //
-// What such a row costs is instructions: every element needs an exponential (its mass), and with
-// no cut a share of a Philox block; 41 (no cut) to 65 per logit in all, at 28 to 41 % of the issue slots (the largest
-// stalls are instruction fetch, fixed latencies and barriers).  So the row is passed over as few times as the definition allows
-// and each pass does one short fixed sequence per element:
+// What such a row costs is instructions: every element needs its mass, and with no cut a share of a Philox block.  So the row
+// is passed over as few times as the definition allows and each pass does one short fixed sequence per element.  Rows of
+// bfloat16 are counted by value (counted_row, below); in general:
 //   mass    e = exp(z - zmax) summed in fixed point, and, where a cut or a list has to be found, one
 //           32-bit shared-memory add per element into a histogram of masses over bins that are linear
 //           in log2 e (32 per octave);
@@ -23,7 +22,7 @@ constexpr int MAX_TEAM = 16;
 
 // Words that the CTAs of a row exchange: slot r is written by CTA r, in every CTA or only in CTA 0's copy.
 struct TeamWords {
-    uint32_t kmax[MAX_TEAM], tau[MAX_TEAM], tau_part[MAX_TEAM], nfin[MAX_TEAM], flags[MAX_TEAM], ncand[MAX_TEAM];   // in every CTA
+    uint32_t kmax[MAX_TEAM], tau[MAX_TEAM], tau_part[MAX_TEAM], nfin[MAX_TEAM], flags[MAX_TEAM], ncand[MAX_TEAM], fail[MAX_TEAM];   // in every CTA
     u64 ahead[MAX_TEAM];                                                                                           // in every CTA
     u64 S[MAX_TEAM], S_all[MAX_TEAM], M[MAX_TEAM], G[MAX_TEAM];                                                    // in CTA 0's
     uint32_t n[MAX_TEAM];
@@ -31,14 +30,19 @@ struct TeamWords {
     uint32_t far_cand, far_list;      // CTA 0: entries that the others have put at the far end of its lists
 };
 
+__device__ __forceinline__ TeamWords &team_words();
+struct TeamWordsHere {                // this CTA's (named anew at every use, see block_scratch)
+    __device__ __forceinline__ TeamWords *operator->() const { return &team_words(); }
+    __device__ __forceinline__ TeamWords &operator*() const { return team_words(); }
+};
 struct SoloTeam {                     // a CTA that has the row to itself
-    TeamWords *x;
+    TeamWordsHere x;
     static constexpr int rank = 0, size = 1;
     __device__ __forceinline__ void sync() const { __syncthreads(); }
     template <class P> __device__ __forceinline__ P *at(P *p, int) const { return p; }
 };
 struct ClusterTeam {                  // the CTAs of a thread-block cluster
-    TeamWords *x;
+    TeamWordsHere x;
     int rank, size;
     __device__ __forceinline__ void sync() const {
         asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
@@ -110,6 +114,16 @@ __device__ __forceinline__ float pick_element(const uint4 &q, int x) {
     return Elem<DT>::get(make_uint4(w, w, w, w), PV == 4 ? 0 : (x & 1));
 }
 
+// A callee that returns a truth value is called on after the last vector, with id -1, until it returns false (the same in
+// every lane of a warp): what it has put by is worked off by the same code.
+// One that takes two vectors gets two of a thread's at a time from a ring, and elsewhere one and nothing (-inf, id -1).
+template <class F> constexpr bool by_pairs = std::is_invocable<F, uint4, uint4, int, int>::value;
+template <class F> constexpr bool answers() {
+    if constexpr (by_pairs<F>) return std::is_same<std::invoke_result_t<F, uint4, uint4, int, int>, bool>::value;
+    else return std::is_same<std::invoke_result_t<F, uint4, int>, bool>::value;
+}
+template <class F> constexpr bool goes_on = answers<F>();
+
 // The whole row, streamed from global memory (from the L2 after the first pass) through a ring of bulk
 // copies: next to CTAs that stream their own rows a plain load comes back after 1.5 to 3 us, and only the
 // copies of whole tiles keep enough of them in flight.  Penalised tokens are masked out of the vectors
@@ -137,6 +151,9 @@ struct RingSlice {
     typedef Elem<DT> E;
     static constexpr bool SPARE_REGISTERS = false;      // 64 per thread
     __device__ __forceinline__ int first_id() const { return row_shared().head; }
+    __device__ __forceinline__ int end_id() const { return row_shared().head + row_shared().nvec * E::PER_VEC; }
+    __device__ __forceinline__ int elements() const { return row_shared().nvec * E::PER_VEC; }
+    __device__ __forceinline__ int n_extras() const { return row_shared().c.has_hist ? (int)row_shared().c.n_distinct : 0; }
     __device__ __forceinline__ static void issue(RowShared &r, int t, int st) {
         Ring rg;
         rg.vps = r.vps; rg.seg_base = r.c.seg_base;
@@ -147,6 +164,7 @@ struct RingSlice {
     // The tiles of all passes are numbered through, which gives stage and phase; the last warp done with a
     // stage refills it.  A wait that expires marks the row, and nothing more is copied.
     template <class F> __device__ __forceinline__ void vectors(F &&f) const {
+        constexpr bool AFTER = goes_on<F>, PAIRS = by_pairs<F>;
         RowShared &r = row_shared();
         const uint32_t first = r.tiles;
         const int nvec = r.nvec, head = r.head, nst = r.nst, tv = r.tv, ntiles = (nvec + NT * tv - 1) / (NT * tv);
@@ -162,24 +180,36 @@ struct RingSlice {
         }
         __syncwarp();       // (the other lanes of the issuing warp, spinning on the first copy, could keep the issuing lane from running)
 #pragma unroll 1
-        for (int t = 0; t < ntiles; ++t) {
-            if (*(volatile uint32_t *)&r.timeout == 0u && !mbar_wait(&r.bar[st], parity)) r.timeout = 1u;
+        for (int t = 0; AFTER || t < ntiles; ++t) {
+            const bool after = AFTER && t == ntiles;
+            if (!after && *(volatile uint32_t *)&r.timeout == 0u && !mbar_wait(&r.bar[st], parity)) r.timeout = 1u;
             __syncwarp();
             const uint4 *stage = (const uint4 *)wide_stage(st * tv);
-#pragma unroll 1
-            for (int u = 0; u < tv; ++u) {
-                const int v = (t * tv + u) * NT + (int)threadIdx.x, i0 = head + v * E::PER_VEC;
+            auto fetch = [&](int u, int i0) -> uint4 {
                 uint4 q = VecTest<DT>::fill();
-                if (v < nvec) {
+                if (!after && (t * tv + u) * NT + (int)threadIdx.x < nvec) {
                     q = stage[u * NT + threadIdx.x];
                     if (bitmap) {
                         const uint32_t m = __funnelshift_r(bitmap[i0 >> 5], bitmap[(i0 >> 5) + 1], i0 & 31) & ((1u << E::PER_VEC) - 1u);
                         if (m) q = kill_elements<DT>(q, m);
                     }
                 }
-                f(q, i0);
+                return q;
+            };
+#pragma unroll 1
+            for (int u = 0; after || u < tv; u += PAIRS ? 2 : 1) {
+                const int i0 = after ? -1 : head + ((t * tv + u) * NT + (int)threadIdx.x) * E::PER_VEC;
+                if constexpr (PAIRS) {
+                    const int i1 = after ? -1 : i0 + NT * E::PER_VEC;
+                    const uint4 q0 = fetch(u, i0), q1 = fetch(u + 1, i1);
+                    if constexpr (AFTER) { if (!f(q0, q1, i0, i1) && after) break; } else f(q0, q1, i0, i1);
+                } else {
+                    const uint4 q = fetch(u, i0);
+                    if constexpr (AFTER) { if (!f(q, i0) && after) break; } else f(q, i0);
+                }
             }
             __syncwarp();
+            if (after) break;
             if ((threadIdx.x & 31) == 0) {
                 __threadfence_block();
                 if (atomicAdd(&r.done[st], 1u) == (uint32_t)(NWARPS - 1)) {
@@ -220,7 +250,7 @@ struct RingSlice {
             } else if (q < total) {
                 const uint32_t rank = (uint32_t)(q - nscal);
                 i = hist_id_of_rank(c, rank);
-                z = __fmul_rn(penalise_counted(c, E::load(elem_ptr<DT>(c, i), 0), c.counts[rank]), c.invT);
+                z = c.scored ? __uint_as_float(c.counts[rank]) : __fmul_rn(penalise_counted(c, E::load(elem_ptr<DT>(c, i), 0), c.counts[rank]), c.invT);
             }
             f(i, z);
         }
@@ -239,13 +269,23 @@ struct SmemSlice {
     const int *xid;               // (in the workspace where there are too many for both lists on chip)
     int xz_off, nx;
     __device__ __forceinline__ int first_id() const { return id0; }
+    __device__ __forceinline__ int end_id() const { return id0 + nvec * E::PER_VEC; }
+    __device__ __forceinline__ int elements() const { return nvec * E::PER_VEC; }
+    __device__ __forceinline__ int n_extras() const { return nx; }
     template <class F> __device__ __forceinline__ void vectors(F &&f) const {
         extern __shared__ __align__(128) unsigned char smem[];
         const uint4 *vec = (const uint4 *)(smem + vec_off);
+        constexpr bool AFTER = goes_on<F>, PAIRS = by_pairs<F>;
 #pragma unroll 1
-        for (int base = 0; base < nvec; base += NT) {
-            const int v = base + (int)threadIdx.x;
-            f(v < nvec ? vec[v] : VecTest<DT>::fill(), id0 + v * E::PER_VEC);
+        for (int base = 0; AFTER || base < nvec; base += NT) {
+            const int v = base + (int)threadIdx.x, i0 = base < nvec ? id0 + v * E::PER_VEC : -1;
+            const uint4 q = v < nvec ? vec[v] : VecTest<DT>::fill();
+            bool more = false;
+            if constexpr (PAIRS && AFTER) more = f(q, VecTest<DT>::fill(), i0, -1);
+            else if constexpr (PAIRS) f(q, VecTest<DT>::fill(), i0, -1);
+            else if constexpr (AFTER) more = f(q, i0);
+            else f(q, i0);
+            if (AFTER && !more && base >= nvec) break;
         }
     }
     template <class F> __device__ __forceinline__ void extras(F &&f) const {
@@ -299,14 +339,24 @@ struct WideSmem {
     u64 *top;             // W_LIST composites: the top-N list
     u64 *list;            // W_LIST composites: the window
     uint32_t *hist;       // W_BINS words
-    u64 *queue;           // 64 entries per warp
+    u64 *queue;           // 64 entries per warp, later masses of the window's list
 };
 // The front of the dynamic shared memory, whatever the kernel keeps behind it
 // (the candidate list and its select bins lie where the top-N list does).
 constexpr int WIDE_LIST_OFF = COMMON_BYTES, WIDE_HIST_OFF = WIDE_LIST_OFF + W_LIST * 8;
-constexpr int WIDE_QUEUE_OFF = WIDE_HIST_OFF + W_BINS * 4, WIDE_BYTES = WIDE_QUEUE_OFF + NWARPS * 64 * 8;
+constexpr int WIDE_QUEUE_OFF = WIDE_HIST_OFF + W_BINS * 4;
+// (rows of bfloat16 whose values are counted: see counted_row.  The table lies over all of the above, the queues of its
+// last pass behind the lists.)
+constexpr int CT_BINS = 8192, CT_ODD = 254;
+constexpr int RACE_DIRECT = 13;       // so many of a warp's vectors at once are raced in place
+constexpr int RACE_QUEUE = 44;        // vectors that a warp's queue holds: 31 left over and RACE_DIRECT - 1
+constexpr int CT_SEG_OFF = CT_BINS * 4, CT_CNT_OFF = CT_SEG_OFF + NT * 8, CT_ODD_OFF = CT_CNT_OFF + NT * 4;
+constexpr int CT_QUEUE_OFF = WIDE_LIST_OFF + W_LIST * 8;
+constexpr int WIDE_BYTES = CT_ODD_OFF + (CT_ODD + 2) * 4;
+static_assert(WIDE_QUEUE_OFF + NWARPS * 64 * 8 <= CT_SEG_OFF && CT_QUEUE_OFF + NWARPS * RACE_QUEUE * 20 <= CT_SEG_OFF, "queues in front of the segments");
 static_assert(W_LIST_ALONE * 8 <= WIDE_HIST_OFF, "the window's list alone lies over both lists and the select bins");
 constexpr int TEAM_OFF = WIDE_BYTES, SLICE_OFF = (TEAM_OFF + (int)sizeof(TeamWords) + 127) & ~127;
+__device__ __forceinline__ TeamWords &team_words() { extern __shared__ __align__(128) unsigned char smem[]; return *(TeamWords *)(smem + TEAM_OFF); }
 // (a CTA that has the row to itself: the row's own block and the ring of its passes follow)
 constexpr int ROW_OFF = SLICE_OFF, WIDE_RING_OFF = (ROW_OFF + (int)sizeof(RowShared) + 127) & ~127;
 __device__ __forceinline__ RowShared &row_shared() { extern __shared__ __align__(128) unsigned char smem[]; return *(RowShared *)(smem + ROW_OFF); }
@@ -382,7 +432,7 @@ struct Window {
 };
 template <class TEAM>
 __device__ __noinline__ Window find_window(BlockScratch *sp, TEAM tm, bool by_count, uint32_t base, int shift, double frac, u64 target, int slack_shift) {
-    BlockScratch &s = *sp;
+    BlockScratch &s = block_scratch();
     uint32_t *hist = wide_smem().hist;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t q[W_PER] = {0, 0, 0, 0};
@@ -484,7 +534,7 @@ __device__ __noinline__ void tie_pass(SRC src, float invT, float zmax, float zfl
 template <int DT, bool FLOOR, class SRC, class TEAM>
 __device__ __noinline__ bool narrow_window(BlockScratch *sp, SRC src, TEAM tm, float invT, float zmax, float zfloor, bool by_count, u64 target,
                                            uint32_t cap, Window *wp) {
-    BlockScratch &s = *sp;
+    BlockScratch &s = block_scratch();
     Window w = *wp;
     const uint32_t ahead_most = w.ahead_most;
     uint32_t *hist = wide_smem().hist;
@@ -554,15 +604,31 @@ __device__ __noinline__ bool narrow_window(BlockScratch *sp, SRC src, TEAM tm, f
 
 // ------------------------------------------------------------------ the race
 
-// N blocks of the generator at once share its key schedule; each product is one wide multiplication.
+// What the generator's first two rounds leave that does not depend on the token (two of their four products), and
+// the keys of the third.
+__device__ __forceinline__ PhiloxRow philox_row(uint64_t seed, uint32_t R, uint64_t step) {
+    PhiloxRow r;
+    const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+    const uint64_t p1 = (uint64_t)(uint32_t)step * 0xCD9E8D57u;
+    const uint64_t p0 = (uint64_t)((uint32_t)(p1 >> 32) ^ R ^ k0) * 0xD2511F53u;
+    r.x0 = (uint32_t)p1 ^ (k0 + 0x9E3779B9u); r.x1 = (uint32_t)(step >> 32) ^ k1;
+    r.x2 = (uint32_t)(p0 >> 32) ^ (k1 + 0xBB67AE85u); r.x3 = (uint32_t)p0;
+    r.k0 = k0 + 2u * 0x9E3779B9u; r.k1 = k1 + 2u * 0xBB67AE85u;
+    return r;
+}
+// N blocks of the generator at once share its key schedule; each product is one wide multiplication, and those are
+// what the race is bound by (a quarter of the rate of other instructions: 18 a block, 5 cycles each measured).
 template <int N>
-__device__ __forceinline__ void philox_blocks(uint64_t seed, uint32_t R, uint64_t step, uint32_t block, uint32_t (&w)[4 * N]) {
-    uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+__device__ __forceinline__ void philox_blocks(const PhiloxRow &r, uint32_t block, uint32_t (&w)[4 * N]) {
+    uint32_t k0 = r.k0, k1 = r.k1;
     uint32_t c0[N], c1[N], c2[N], c3[N];
 #pragma unroll
-    for (int n = 0; n < N; ++n) { c0[n] = block + n; c1[n] = R; c2[n] = (uint32_t)step; c3[n] = (uint32_t)(step >> 32); }
+    for (int n = 0; n < N; ++n) {
+        const uint64_t p0 = (uint64_t)(block + n) * 0xD2511F53u, p1 = (uint64_t)((uint32_t)(p0 >> 32) ^ r.x1) * 0xCD9E8D57u;
+        c0[n] = (uint32_t)(p1 >> 32) ^ r.x0; c1[n] = (uint32_t)p1; c2[n] = (uint32_t)p0 ^ r.x2; c3[n] = r.x3;
+    }
 #pragma unroll
-    for (int i = 0; i < 10; ++i) {
+    for (int i = 2; i < 10; ++i) {
 #pragma unroll
         for (int n = 0; n < N; ++n) {
             const uint64_t p0 = (uint64_t)c0[n] * 0xD2511F53u, p1 = (uint64_t)c2[n] * 0xCD9E8D57u;
@@ -583,10 +649,10 @@ struct Racer {
     uint32_t seen;        // order code K was computed from
     u64 G;                // this thread's best: order code of the score, ~id
     float z;              // and its z
-    __device__ __forceinline__ void start() { K = 3.0e34f; seen = 0; G = 0; z = 0.0f; }
+    __device__ __forceinline__ void start(float K0 = 3.0e34f) { K = K0; seen = 0; G = 0; z = 0.0f; }
     __device__ __forceinline__ void refresh(const uint32_t *best) {
         const uint32_t now = *(const volatile uint32_t *)best;
-        if (now != seen) { seen = now; K = fminf(1.0001f * ex2_ftz(-unkey(now) * 1.4426950408889634f), 3.0e34f); }
+        if (now != seen) { seen = now; K = fminf(1.0001f * ex2_ftz(-unkey(now) * 1.4426950408889634f), K); }
     }
     __device__ __forceinline__ void take(uint32_t *best, int i, float z_, float g) {
         const u64 g64 = ((u64)orderable_f32(g) << 32) | (uint32_t)(~(uint32_t)i);
@@ -595,8 +661,11 @@ struct Racer {
             if ((uint32_t)(g64 >> 32) > *(volatile uint32_t *)best) atomicMax(best, (uint32_t)(g64 >> 32));
         }
     }
+    // no larger word lets an element of mass e win
+    __device__ __forceinline__ uint32_t word_bound(float e) const { return __float2uint_ru(e * K * 4294967296.0f); }
 };
 __device__ __forceinline__ float unit_above(uint32_t w) { return __uint_as_float((w >> 9) | 0x3F800000u); }      // 1 + (v rounded down)
+constexpr float RACE_LUCK = 24.5f;    // exp(3.2): the winner of a row of mass S has a score above ln S - 3.2 (ln S - ln E) but for 2e-11 of all rows
 __device__ __noinline__ float nle_once(uint32_t w) { return neg_log_exp1_fast(w); }      // (where it is rare: one copy of the code)
 
 __device__ __forceinline__ float race_bound(uint32_t best) {      // Racer::K of a best score's order code
@@ -609,30 +678,34 @@ __device__ __forceinline__ void list_append(u64 *list, int cap, uint32_t *cnt, f
 
 // Mass and race element by element in one pass: of the whole row (no cut), or (CUT, arguments in s.fa) of
 // the elements kept for sure where those are a good part of the row, the window's going to the list.
-// OFF: id of a vector's first element modulo 4 (the generator's blocks are 4 ids).  About 20
-// instructions per element, half of them Philox; vectors that could not win with the luckiest word skip it.
+// OFF: id of a vector's first element modulo 4 (the generator's blocks are 4 ids).
+// What decides is the smallest of a vector's words against the bound of its largest mass: 9 wide multiplications per
+// 2 elements, 8 instructions an element for its mass, and little else.
 template <int DT, int OFF, bool CUT, class SRC>
 __device__ __forceinline__ void race_all(const SRC &src, BlockScratch &s, Partial &p) {
     typedef Elem<DT> E;
     constexpr int PV = E::PER_VEC, NB = PV / 4 + (OFF ? 1 : 0);
     uint32_t *best = &s.runmax;
     const float invT = s.fa.invT, zmax = s.fa.zmax, minus0 = minus_zero(invT);
-    const uint64_t seed = s.fa.seed, step = s.fa.step;
-    const uint32_t R = s.fa.R;
     const uint32_t sure = CUT ? s.fa.sure : 0u, win_hi = CUT ? s.fa.win_hi : 0u;
     MassSum S;
     uint32_t n = 0;
     Racer rc;
-    rc.start();
+    rc.start(RACE_LUCK);
+    const PhiloxRow pr = s.fa.philox;
+    // an element by itself
+    auto race_one = [&](int i, float z, float e) {
+        uint32_t w[4];
+        philox_blocks<1>(pr, (uint32_t)i >> 2, w);
+        const uint32_t x = (i & 3) == 0 ? w[0] : (i & 3) == 1 ? w[1] : (i & 3) == 2 ? w[2] : w[3];
+        if (e > 0.0f && x <= rc.word_bound(e)) rc.take(best, i, z, __fsub_rn(z, zmax) + nle_once(x));
+    };
     // an element at the edge: in the window, or an equal of its first code with a lower id
     auto edge = [&](int i, float z, float t2, uint32_t f) {
         const FinalArgs &fa = s.fa;
         if (!(z >= fa.zfloor)) return;
-        if (f == sure && (uint32_t)i < fa.id_lo) {
-            S.add(ex2_ftz(t2)); ++n;
-            const uint32_t w = race_word(seed, R, step, i);
-            if (unit_above(w) <= __fmaf_rn(ex2_ftz(t2), rc.K, 1.0f)) rc.take(best, i, z, __fsub_rn(z, zmax) + nle_once(w));
-        } else if (f < win_hi || (f == win_hi && (uint32_t)i <= fa.id_hi)) list_append(fa.list, fa.list_cap, &s.list_cnt, z, i);
+        if (f == sure && (uint32_t)i < fa.id_lo) { const float e = ex2_ftz(t2); S.add(e); ++n; race_one(i, z, e); }
+        else if (f < win_hi || (f == win_hi && (uint32_t)i <= fa.id_hi)) list_append(fa.list, fa.list_cap, &s.list_cnt, z, i);
     };
     src.vectors([&](const uint4 &q, int i0) {
         float e[PV], top = 0.0f;
@@ -661,11 +734,14 @@ __device__ __forceinline__ void race_all(const SRC &src, BlockScratch &s, Partia
         }
         rc.refresh(best);
         if (!__any_sync(0xFFFFFFFFu, top * rc.K >= 1.16e-10f)) return;      // v is at least 2^-33
-        uint32_t w[4 * NB];
-        philox_blocks<NB>(seed, R, step, (uint32_t)(i0 >> 2), w);
+        uint32_t w[4 * NB], least = 0xFFFFFFFFu;
+        philox_blocks<NB>(pr, (uint32_t)(i0 >> 2), w);
+#pragma unroll
+        for (int j = 0; j < PV; ++j) least = min(least, w[OFF + j]);
+        if (!__any_sync(0xFFFFFFFFu, least <= rc.word_bound(top))) return;
         uint32_t hits = 0;
 #pragma unroll
-        for (int j = 0; j < PV; ++j) hits |= (uint32_t)((!CUT || e[j] > 0.0f) && unit_above(w[OFF + j]) <= __fmaf_rn(e[j], rc.K, 1.0f)) << j;
+        for (int j = 0; j < PV; ++j) hits |= (uint32_t)(e[j] > 0.0f && w[OFF + j] <= rc.word_bound(e[j])) << j;
         // rare after the first vectors: the exact score, one element per lane at a time, the bound renewed in between
         while (__any_sync(0xFFFFFFFFu, hits != 0)) {
             if (hits) {
@@ -675,7 +751,7 @@ __device__ __forceinline__ void race_all(const SRC &src, BlockScratch &s, Partia
 #pragma unroll
                 for (int j = 1; j < PV; ++j) wx = x == j ? w[OFF + j] : wx;
                 const float z = __fmul_rn(pick_element<DT>(q, x), invT), d = __fsub_rn(z, zmax);
-                if (d > -3.0e38f && unit_above(wx) <= __fmaf_rn(ex2_ftz(d * 1.4426950408889634f), rc.K, 1.0f)) rc.take(best, i0 + x, z, d + nle_once(wx));
+                if (wx <= rc.word_bound(ex2_ftz(d * 1.4426950408889634f))) rc.take(best, i0 + x, z, d + nle_once(wx));
             }
             __syncwarp();
             rc.refresh(best);
@@ -688,10 +764,9 @@ __device__ __forceinline__ void race_all(const SRC &src, BlockScratch &s, Partia
         const uint32_t f = code_of(t2);
         bool in = true;
         if constexpr (CUT) in = f < sure;
-        if (in) {
-            S.add(ex2_ftz(t2)); ++n;
-            rc.take(best, i, z, d + race_nle(seed, R, step, nullptr, i));
-        } else if (f <= win_hi) edge(i, z, t2, f);        // (CUT only)
+        rc.refresh(best);
+        if (in) { const float e = ex2_ftz(t2); S.add(e); ++n; race_one(i, z, e); }
+        else if (f <= win_hi) edge(i, z, t2, f);        // (CUT only)
     });
     p.M = S.total(); p.n = CUT ? n : 0; p.G = rc.G; p.z = rc.z;
 }
@@ -883,6 +958,156 @@ __device__ __noinline__ int list_sort(u64 *list, int n) {
     return P;
 }
 
+// What the passes of a wide row leave behind, apart from each thread's sums and the lists.
+struct WideEnd {
+    u64 M0; uint32_t n0;                 // mass and number of elements kept for sure that the sums do not contain
+    u64 S, S_all;                        // the mass that top-p is a share of, the whole row's
+    float zmax;
+    uint32_t n_fin;
+    bool summed, in_team, all_kept, topp, full;   // the sums contain the whole row's mass; S and S_all are in the team's words; every finite score is kept
+    float race_from;                     // a winner's score below this: one that was passed over may be ahead of it (-infinity: none was)
+};
+constexpr float RACE_FROM = -3.1977f;    // for a race whose bound started from RACE_LUCK: 0.001 - 3.1987 (ln 24.5)
+// From there to the result, which is CTA 0's, in its warp 0.
+template <class TEAM>
+__device__ __forceinline__ RowOut wide_finish_in(TEAM tm, float top_p, uint64_t seed, uint32_t R, Partial p, const WideEnd &w, u64 *list, int list_cap,
+                                                 const float *exp1_row, int b, RowOut out) {
+    BlockScratch &s = block_scratch();
+    const WideSmem ws = wide_smem();
+    const int lane = threadIdx.x & 31;
+    const bool want_list = s.ga.num_top > 0, topp = w.topp, full = w.full;
+    const float zmax = w.zmax;
+    block_partial(s, p);                                 // (its barrier also ends the appends)
+    const int n_list = (int)s.list_cnt, n_top = (int)s.cand_cnt;
+    if (threadIdx.x == 0) {
+        const int r = tm.rank;
+        *tm.at(&tm.x->M[r], 0) = p.M; *tm.at(&tm.x->n[r], 0) = p.n; *tm.at(&tm.x->G[r], 0) = p.G; *tm.at(&tm.x->z[r], 0) = p.z;
+    }
+    if (tm.size > 1 && tm.rank != 0 && (topp || want_list)) {
+        // the lists' entries go to the far ends of CTA 0's lists (each list's sum is within its capacity)
+        if (threadIdx.x == 32) {
+            s.found_digit = n_list ? atomicAdd(tm.at(&tm.x->far_list, 0), (uint32_t)n_list) : 0u;
+            s.found_cnt = n_top ? atomicAdd(tm.at(&tm.x->far_cand, 0), (uint32_t)n_top) : 0u;
+        }
+        __syncthreads();
+        const int at_list = list_cap - 1 - (int)s.found_digit, at_top = W_LIST - 1 - (int)s.found_cnt;
+        u64 *list0 = tm.at(list, 0), *top0 = tm.at(ws.top, 0);
+        for (int j = threadIdx.x; j < n_list; j += NT) if (at_list - j >= 0) list0[at_list - j] = list[j];
+        for (int j = threadIdx.x; j < n_top; j += NT) if (at_top - j >= 0) top0[at_top - j] = ws.top[j];
+    }
+    tm.sync();
+    if (tm.rank != 0) return out;
+
+    // CTA 0 has everything
+    const TeamWords &x = *tm.x;
+    const bool in = lane < tm.size;
+    p.M = in ? x.M[lane] : 0ull; p.n = in ? x.n[lane] : 0u; p.G = in ? x.G[lane] : 0ull; p.z = in ? x.z[lane] : 0.0f;
+    p.over_warp();
+    p.M += w.M0; p.n = w.all_kept ? w.n_fin : p.n + w.n0;
+    u64 S = w.S, S_all = w.summed ? p.M : w.S_all;
+    if (w.in_team) { S = warp_total(in ? x.S[lane] : 0ull); S_all = warp_total(in ? x.S_all[lane] : 0ull); }
+    if (topp) {
+        const u64 target = topp_target(top_p, S);
+        const int L = close_gap(list, list_cap, n_list, (int)x.far_list);
+        if (p.M >= target || L < 1 || L > list_cap) { out.status |= ROW_NOT_DONE; return out; }
+        auto mass_of = [&](u64 C) { return __float2ull_rn(ex2_ftz(log2_mass(unkey((uint32_t)(C >> 32)), zmax)) * FX_SCALE); };
+        Partial k;
+        k.M = 0; k.n = 0; k.G = 0; k.z = 0.0f;
+        auto keep = [&](u64 C, u64 own) {
+            k.M += own; ++k.n;
+            const float zq = unkey((uint32_t)(C >> 32));
+            const float g = __fsub_rn(zq, zmax) + race_nle(seed, R, s.ga.step, exp1_row, comp_idx(C));
+            const u64 gq = ((u64)orderable_f32(g) << 32) | (uint32_t)C;
+            if (gq > k.G) { k.G = gq; k.z = zq; }
+        };
+        // An entry is kept while the mass ahead of it in the order, with the mass kept for sure, is short of
+        // the target.  A short list: every entry adds that mass up (masses over the queues, done with by now),
+        // one barrier in all; from 192 entries on a sort and a prefix sum are faster (2 us against 3 at 300).
+        bool reached;
+        if (L <= 192) {
+            // (two or four threads share an entry's comparisons where there are more than 64)
+            u64 *mass = ws.queue;
+            if ((int)threadIdx.x < L) mass[threadIdx.x] = mass_of(list[threadIdx.x]);
+            __syncthreads();
+            const int sh = L <= 64 ? 0 : L <= 128 ? 2 : 1, j = (int)threadIdx.x >> sh, part = (int)threadIdx.x & ((1 << sh) - 1);
+            const u64 C = j < L ? list[j] : 0ull;
+            u64 ahead = 0, reach = 0;
+            if (j < L) {
+#pragma unroll 4
+                for (int q = part; q < L; q += 1 << sh) ahead += list[q] > C ? mass[q] : 0ull;
+            }
+            for (int o = 1; o < 1 << sh; o <<= 1) ahead += __shfl_xor_sync(0xFFFFFFFFu, ahead, o);
+            ahead += p.M;
+            if (j < L) {
+                const u64 own = mass[j];
+                reach = ahead + own;
+                if (part == 0 && ahead < target) keep(C, own);
+            }
+            reached = __syncthreads_or(reach >= target) != 0;
+        } else {
+            const int P = list_sort(list, L), per = (P + NT - 1) / NT, q0 = (int)threadIdx.x * per, q1 = min(L, q0 + per);
+            u64 local = 0, tot;
+            for (int q = q0; q < q1; ++q) local += mass_of(list[q]);
+            u64 run = p.M + block_exscan_u64(s, local, tot);
+            reached = p.M + tot >= target;
+#pragma unroll 1
+            for (int q = q0; q < q1 && run < target; ++q) {
+                const u64 C = list[q], own = mass_of(C);
+                run += own;
+                keep(C, own);
+            }
+            __syncthreads();
+        }
+        if (!reached) { out.status |= ROW_NOT_DONE; return out; }
+        block_partial(s, k);
+        p.M += k.M; p.n += k.n;
+        if (k.G > p.G) { p.G = k.G; p.z = k.z; }
+    }
+    if (w.race_from > -INFINITY && __syncthreads_or(threadIdx.x == 0 && !(unkey((uint32_t)(p.G >> 32)) >= w.race_from))) { out.status |= ROW_NOT_DONE; return out; }
+    double lnS = 0.0;
+    if (threadIdx.x < 32) {
+        const u64 S_ref = full ? S_all : p.M;
+        lnS = log((double)S_ref) - LN2_40;
+        const int tok = comp_idx(p.G);
+        out.token = tok < 0 ? 0 : tok;                  // (NaN logits: any id in range)
+        out.n_keep = (int32_t)p.n;
+        out.logprob = (p.n == 1 && !full) ? 0.0f : (float)(((double)p.z - (double)zmax) - lnS);
+    }
+    if (want_list) {
+        if (threadIdx.x == 0) { s.bcast[0] = (u64)__double_as_longlong(lnS); s.found_cnt = p.n; }
+        const int n_all = close_gap(ws.top, W_LIST, n_top, (int)x.far_cand);
+        __syncthreads();
+        const double lnS_all = __longlong_as_double((long long)s.bcast[0]);
+        const uint32_t members = full ? w.n_fin : s.found_cnt;
+        if ((uint32_t)n_all < min((uint32_t)s.ga.num_top, members) || n_all > W_LIST) { out.status |= ROW_NOT_DONE; return out; }      // (the same in every thread)
+#pragma unroll 1
+        for (int j = threadIdx.x; j < n_all; j += NT) {
+            const u64 C = ws.top[j];
+            uint32_t rank = 0;
+#pragma unroll 4
+            for (int q = 0; q < n_all; ++q) rank += ws.top[q] > C;
+            if (rank < (uint32_t)s.ga.num_top && rank < members) {
+                const int64_t o = (int64_t)b * s.ga.num_top + rank;
+                s.ga.out_top_ids[o] = comp_idx(C);
+                s.ga.out_top_logprobs[o] = (members == 1 && !full) ? 0.0f : (float)(((double)unkey((uint32_t)(C >> 32)) - (double)zmax) - lnS_all);
+            }
+        }
+    }
+    return out;
+}
+
+__device__ __noinline__ RowOut wide_finish_call(float top_p, uint64_t seed, uint32_t R, Partial p, WideEnd w, u64 *list, int list_cap, const float *exp1_row,
+                                                int b, RowOut out) {
+    return wide_finish_in(SoloTeam(), top_p, seed, R, p, w, list, list_cap, exp1_row, b, out);
+}
+// (with 64 registers per thread out of line)
+template <class TEAM>
+__device__ __forceinline__ RowOut wide_finish(const TEAM &tm, float top_p, uint64_t seed, uint32_t R, const Partial &p, const WideEnd &w, u64 *list, int list_cap,
+                                              const float *exp1_row, int b, const RowOut &out) {
+    if constexpr (std::is_same<TEAM, SoloTeam>::value) return wide_finish_call(top_p, seed, R, p, w, list, list_cap, exp1_row, b, out);
+    else return wide_finish_in(tm, top_p, seed, R, p, w, list, list_cap, exp1_row, b, out);
+}
+
 // The row's kept set, token and log-probability; the result is CTA 0's, in its warp 0.  `kmax`, `n_fin`:
 // the row's largest order key and its number of finite scores (the same in every CTA).
 template <int DT, class SRC, class TEAM>
@@ -954,11 +1179,11 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
     if (threadIdx.x == 0) { s.list_cnt = 0; s.cand_cnt = 0; }
     __syncthreads();
 
-    Partial p;
     const bool no_cut = !topp && !minp && !want_list && !exp1_row;
     // kept elements that are a good part of the row are raced in place: 25 instructions per element of the
     // row against about 40 per kept element through the queues (`ahead_most` is up to twice their number)
     const bool dense = topp && !minp && !want_list && !exp1_row && win.ahead_most > n_fin / 4;
+    if ((no_cut || dense) && threadIdx.x == 32) s.fa.philox = philox_row(rp.seed, rp.R, s.ga.step);
     if (threadIdx.x == 0) {
         FinalArgs &fa = s.fa;
         fa.invT = invT; fa.zmax = zmax; fa.zfloor = zfloor;
@@ -979,117 +1204,631 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
         fa.vec_thr = VecTest<DT>::raw_threshold(key, invT);
     }
     __syncthreads();
+    Partial p;
     if (no_cut) run_race<DT, false>(src, s, p);
     else if (dense) run_race<DT, true>(src, s, p);
     else run_final_pass<DT>(src, s, p);
-    block_partial(s, p);                                 // (its barrier also ends the appends)
-    const int n_list = (int)s.list_cnt, n_top = (int)s.cand_cnt;
-    if (threadIdx.x == 0) {
-        const int r = tm.rank;
-        *tm.at(&tm.x->M[r], 0) = p.M; *tm.at(&tm.x->n[r], 0) = p.n; *tm.at(&tm.x->G[r], 0) = p.G; *tm.at(&tm.x->z[r], 0) = p.z;
-    }
-    if (tm.size > 1 && tm.rank != 0 && (topp || want_list)) {
-        // the lists' entries go to the far ends of CTA 0's lists (each list's sum is within its capacity)
-        if (threadIdx.x == 32) {
-            s.found_digit = n_list ? atomicAdd(tm.at(&tm.x->far_list, 0), (uint32_t)n_list) : 0u;
-            s.found_cnt = n_top ? atomicAdd(tm.at(&tm.x->far_cand, 0), (uint32_t)n_top) : 0u;
-        }
-        __syncthreads();
-        const int at_list = list_cap - 1 - (int)s.found_digit, at_top = W_LIST - 1 - (int)s.found_cnt;
-        u64 *list0 = tm.at(list, 0), *top0 = tm.at(ws.top, 0);
-        for (int j = threadIdx.x; j < n_list; j += NT) if (at_list - j >= 0) list0[at_list - j] = list[j];
-        for (int j = threadIdx.x; j < n_top; j += NT) if (at_top - j >= 0) top0[at_top - j] = ws.top[j];
-    }
-    tm.sync();
-    if (tm.rank != 0) return out;
+    WideEnd w;
+    w.M0 = 0; w.n0 = 0; w.S = 0; w.S_all = 0; w.zmax = zmax; w.n_fin = n_fin; w.summed = !need_hist; w.in_team = need_hist; w.all_kept = !need_hist && !minp;
+    w.topp = topp; w.full = full; w.race_from = no_cut || dense ? RACE_FROM : -INFINITY;
+    return wide_finish_in(tm, rp.top_p, rp.seed, rp.R, p, w, list, list_cap, exp1_row, b, out);
+}
 
-    // CTA 0 has everything
-    const TeamWords &x = *tm.x;
-    const bool in = lane < tm.size;
-    p.M = in ? x.M[lane] : 0ull; p.n = in ? x.n[lane] : 0u; p.G = in ? x.G[lane] : 0ull; p.z = in ? x.z[lane] : 0.0f;
-    p.over_warp();
-    u64 S = 0, S_all = p.M;
-    if (need_hist) { S = warp_total(in ? x.S[lane] : 0ull); S_all = warp_total(in ? x.S_all[lane] : 0ull); }
-    else if (!minp) p.n = n_fin;
-    if (topp) {
-        const u64 target = topp_target(rp.top_p, S);
-        const int L = close_gap(list, list_cap, n_list, (int)x.far_list);
-        if (p.M >= target || L < 1 || L > list_cap) { out.status |= ROW_NOT_DONE; return out; }
-        auto mass_of = [&](u64 C) { return __float2ull_rn(ex2_ftz(log2_mass(unkey((uint32_t)(C >> 32)), zmax)) * FX_SCALE); };
-        Partial k;
-        k.M = 0; k.n = 0; k.G = 0; k.z = 0.0f;
-        auto keep = [&](u64 C, u64 own) {
-            k.M += own; ++k.n;
-            const float zq = unkey((uint32_t)(C >> 32));
-            const float g = __fsub_rn(zq, zmax) + race_nle(rp.seed, rp.R, s.ga.step, exp1_row, comp_idx(C));
-            const u64 gq = ((u64)orderable_f32(g) << 32) | (uint32_t)C;
-            if (gq > k.G) { k.G = gq; k.z = zq; }
+// ------------------------------------------------------------------ rows of bfloat16: counted by value
+//
+// A bfloat16 logit has few values: from 2^-26 up to 64 either sign has 4096, and elements of one value have one mass.
+// So the row's masses are a count per value - one shared-memory increment per element, 4 instructions, where the
+// exponential, its exact sum and a histogram of masses take 19 - times an exponential per value, worked out
+// afterwards, when the maximum is known.  One pass gives the maximum, the number of finite scores, the exact
+// mass and, from prefix sums, the very value at which a cut or a list ends; with no cut the race is in the same
+// pass.  (Increments of one warp meet in 3.5 bank cycles on average, which bounds the pass: 3620 cycles per 32768 elements
+// in one SM against 6940 for the pass of masses and 690 for the maximum.)
+// What has no place in the table: values of 64 and more, and more than CT_ODD values nearer to zero than 2^-26 (the
+// row is then done as rows of other types are); all from -63.75 down are counted together, and weigh nothing unless the
+// maximum is as low.  The scores of the extras (penalised tokens, unaligned ends) lie between those of the values:
+// they are added to the segment of 16 values that they belong to, and stay open in the segment of the cut.
+
+constexpr int CT_PER = CT_BINS / NT;                   // values per thread: a segment
+constexpr uint32_t CT_LOW = 0xC27Fu;                   // -63.75: this value and everything below
+constexpr uint32_t ROW_NOT_COUNTED = 0x40000000u;      // internal status bit: the table does not hold the row (the same in every CTA)
+static_assert(CT_PER == 16, "a segment is 16 values");
+
+struct CountedSmem { uint32_t *count; u64 *seg_mass; uint32_t *seg_cnt, *odd; };     // odd: their number, whether there are values of 64 or more, codes
+__device__ __forceinline__ CountedSmem counted_smem() {
+    extern __shared__ __align__(128) unsigned char smem[];
+    CountedSmem c;
+    c.count = (uint32_t *)smem; c.seg_mass = (u64 *)(smem + CT_SEG_OFF); c.seg_cnt = (uint32_t *)(smem + CT_CNT_OFF); c.odd = (uint32_t *)(smem + CT_ODD_OFF);
+    return c;
+}
+__device__ __forceinline__ uint32_t ct_index(uint32_t c) { return (c & 0xFFFu) | ((c >> 3) & 0x1000u); }
+// the j-th value in descending order, and one step up from a value
+__device__ __forceinline__ uint32_t ct_code(int j) { return j < 4096 ? 0x427Fu - (uint32_t)j : 0xB280u + (uint32_t)(j - 4096); }
+__device__ __forceinline__ uint32_t ct_above(uint32_t c) { return c & 0x8000u ? c - 1u : c + 1u; }
+// which place an element takes whose score lies above that of the next lower value than c and not above that of c
+__device__ __forceinline__ int ct_place(uint32_t c) {
+    const uint32_t mag = c & 0x7FFFu;
+    if (mag < 0x3280u) return 4095;
+    if (mag >= 0x4280u) return c & 0x8000u ? CT_BINS - 1 : 0;
+    return c & 0x8000u ? 4096 + (int)(mag - 0x3280u) : (int)(0x427Fu - mag);
+}
+__device__ __forceinline__ float ct_score(uint32_t c, float invT) { return __fmul_rn(__uint_as_float(c << 16), invT); }
+__device__ __forceinline__ u64 mass_fx(float z, float zmax) { return __float2ull_rn(ex2_ftz(log2_mass(z, zmax)) * FX_SCALE); }
+
+// (by whole blocks; a barrier must follow)
+__device__ __forceinline__ void counted_clear() {
+    const CountedSmem c = counted_smem();
+#pragma unroll
+    for (int i = 0; i < CT_PER / 4; ++i) ((uint4 *)c.count)[i * NT + threadIdx.x] = make_uint4(0, 0, 0, 0);
+    c.seg_mass[threadIdx.x] = 0ull; c.seg_cnt[threadIdx.x] = 0u;
+    if (threadIdx.x < 2) c.odd[threadIdx.x] = 0u;
+}
+__device__ __noinline__ void count_odd_vector(uint4 q) {
+    const CountedSmem c = counted_smem();
+#pragma unroll 1
+    for (int j = 0; j < 8; ++j) {
+        const uint32_t v = __float_as_uint(pick_element<ALBIREO_BF16>(q, j)) >> 16, mag = v & 0x7FFFu;
+        if (mag >= 0x4280u) c.odd[1] = 1u;
+        else if (mag >= 0x3280u) atomicAdd(&c.count[ct_index(v)], 1u);
+        else { const uint32_t at = atomicAdd(&c.odd[0], 1u); if (at < (uint32_t)CT_ODD) c.odd[2 + at] = v; }
+    }
+}
+// counts the vector's values; `top` is its largest of each half
+__device__ __forceinline__ void count_vector(uint4 q, __nv_bfloat162 top) {
+    typedef __nv_bfloat162 H2;
+    uint32_t *count = counted_smem().count;
+    const uint32_t low2 = CT_LOW | (CT_LOW << 16), high2 = 0x42804280u, tiny2 = 0x32803280u;
+    auto h = [](const uint32_t &w) { return *reinterpret_cast<const H2 *>(&w); };
+    const H2 least = __hmin2(__hmin2(__habs2(h(q.x)), __habs2(h(q.y))), __hmin2(__habs2(h(q.z)), __habs2(h(q.w))));
+    const bool plain = (__hlt2_mask(top, h(high2)) & __hge2_mask(least, h(tiny2))) == 0xFFFFFFFFu;
+    auto clamp = [&](uint32_t &w) { const H2 x = __hmax2(h(w), h(low2)); w = *reinterpret_cast<const uint32_t *>(&x); };
+    clamp(q.x); clamp(q.y); clamp(q.z); clamp(q.w);
+    if (!plain) { count_odd_vector(q); return; }
+    auto add = [&](uint32_t w) {
+        const uint32_t i = ((w & 0x0FFF0FFFu) | ((w >> 3) & 0xF000F000u)) & 0x1FFF1FFFu;
+        atomicAdd(&count[i & 0xFFFFu], 1u);
+        atomicAdd(&count[i >> 16], 1u);
+    };
+    add(q.x); add(q.y); add(q.z); add(q.w);
+}
+// An element of mass e can only beat a score g if E < e exp(-g), and E = -log1p(-v) >= v: so comparing v / e with
+// K = exp(-g) decides almost every element without a logarithm.  Nor does K take one: an element's own E / e is an upper
+// bound of it, and E <= v (1 + v) up to v = 1/2.  The smallest K of a CTA so far is shared by its threads (s.race_bound,
+// the float's bits).  It starts from a score that the winner of a row of mass S reaches but for 2e-11 of all rows, ln S - 3.2 (the winner's
+// score is ln S - ln E); a row in which none did goes to the general path.
+// (With K from the exact scores alone batches of vectors stopped for several of them, a few hundred cycles each, while the first
+// batches of all warps were under way: 32 top-p rows of 128256 spent 6.0 us in the last pass, 5.4 so.)
+constexpr uint32_t NO_BOUND = 0x7F7FFFFFu;
+__device__ __forceinline__ float unit_below(uint32_t w) { return __uint_as_float((w >> 9) | 0x3F800000u) - 1.0f; }      // v rounded down to 2^-23
+// an upper bound of E / e from v (rounded down) and 1 / e
+__device__ __forceinline__ float race_cap(float v, float inv_e) {
+    const float up = v + 1.1920929e-7f;
+    return v < 0.5f ? 1.0002f * (__fmaf_rn(up, up, up) * inv_e) : 3.0e38f;
+}
+// What the race needs across the vectors of a pass: the generator's row and each thread's best element (order code of the score, ~id, and its z) in
+// registers where there are some to spare (REGS: 128 per thread), else in shared memory, the best by warps in s.race_G and s.race_z -
+// held across the passes' loops they were spilled, and what is spilled comes back from the L2.  (By the other kernel's way
+// 64 rows of 152064 without a cut took 24.5 us instead of 21.9.)
+template <bool REGS>
+struct CountedRacer {
+    BlockScratch &s;
+    PhiloxRow kept;
+    u64 G;
+    float z;
+    __device__ __forceinline__ explicit CountedRacer(BlockScratch &s_) : s(s_), G(0), z(0.0f) {
+        if constexpr (REGS) { kept = s.fa.philox; return; }
+        if ((threadIdx.x & 31) == 0) { s.race_G[threadIdx.x >> 5] = 0; s.race_z[threadIdx.x >> 5] = 0.0f; }
+        __syncwarp();
+    }
+    __device__ __forceinline__ PhiloxRow row() const {
+        if constexpr (REGS) return kept;
+        const volatile PhiloxRow &v = s.fa.philox;
+        PhiloxRow r;
+        r.x0 = v.x0; r.x1 = v.x1; r.x2 = v.x2; r.x3 = v.x3; r.k0 = v.k0; r.k1 = v.k1;
+        return r;
+    }
+    __device__ __forceinline__ float K() const { return __uint_as_float(*(const volatile uint32_t *)&s.race_bound); }
+    // no larger word lets an element of mass e win
+    __device__ __forceinline__ static uint32_t word_bound(float e, float K) { return __float2uint_ru(e * K * 4294967296.0f); }
+    // by whole warps: the lanes' bounds; gives the smallest of all.  (Never 0: masses relative to a reference far below the maximum can be infinite.)
+    __device__ __forceinline__ float tighten(float cap) const {
+        const uint32_t least = __reduce_min_sync(0xFFFFFFFFu, __float_as_uint(fminf(fmaxf(cap, 1e-37f), 3.0e38f)));
+        const float now = K();
+        if (__uint_as_float(least) < now && (threadIdx.x & 31) == 0) atomicMin(&s.race_bound, least);
+        return fminf(__uint_as_float(least), now);
+    }
+    // by whole warps: the lanes' best elements (0: none)
+    __device__ __forceinline__ void take(u64 g, float zg) {
+        if constexpr (REGS) { if (g > G) { G = g; z = zg; } return; }
+        if (!__any_sync(0xFFFFFFFFu, g != 0)) return;
+        warp_best(g, zg);
+        const int wid = threadIdx.x >> 5;
+        if ((threadIdx.x & 31) == 0 && g > s.race_G[wid]) { s.race_G[wid] = g; s.race_z[wid] = zg; }
+        __syncwarp();
+    }
+    __device__ __forceinline__ static u64 code_of_score(float g, int i) { return ((u64)orderable_f32(g) << 32) | (uint32_t)(~(uint32_t)i); }
+    // One element per lane by itself, by whole warps: of log2 mass t2 and d = z - reference (`in`: if it is there at all).
+    __device__ __forceinline__ void race(bool in, int i, float zi, float d, float t2) {
+        uint32_t w[4];
+        philox_blocks<1>(row(), (uint32_t)i >> 2, w);
+        const uint32_t x = (i & 3) == 0 ? w[0] : (i & 3) == 1 ? w[1] : (i & 3) == 2 ? w[2] : w[3];
+        const float v = unit_below(x), inv_e = in ? ex2_ftz(-t2) : INFINITY;
+        if (!__any_sync(0xFFFFFFFFu, v * inv_e <= K())) return;                         // (0 x infinity is no hit)
+        const float least = tighten(in ? race_cap(v, inv_e) : 3.0e38f);
+        take(v * inv_e <= least ? code_of_score(d + nle_once(x), i) : 0ull, zi);
+    }
+    // The elements of a vector, their words w[OFF ..], by whole warps: `inv_mass` of element j gives 1 / e, infinity for one that does not take part.
+    template <int DT, int OFF, int N, class F>
+    __device__ __forceinline__ void race_hits(const uint32_t (&w)[N], const uint4 &q, int i0, float invT, float zref, F &&inv_mass) {
+        constexpr int PV = Elem<DT>::PER_VEC;
+        float cap = 3.0e38f;
+#pragma unroll
+        for (int j = 0; j < PV; ++j) cap = fminf(cap, race_cap(unit_below(w[OFF + j]), inv_mass(j)));
+        const float K = tighten(cap);
+        uint32_t hits = 0;
+#pragma unroll
+        for (int j = 0; j < PV; ++j) hits |= (uint32_t)(unit_below(w[OFF + j]) * inv_mass(j) <= K) << j;
+        u64 best = 0;
+        float zbest = 0.0f;
+        while (hits) {
+            const int x = __ffs(hits) - 1;
+            hits &= hits - 1;
+            uint32_t wx = w[OFF];
+#pragma unroll
+            for (int j = 1; j < PV; ++j) wx = x == j ? w[OFF + j] : wx;
+            const float zx = __fmul_rn(pick_element<DT>(q, x), invT);
+            const u64 g = code_of_score(__fsub_rn(zx, zref) + nle_once(wx), i0 + x);
+            if (g > best) { best = g; zbest = zx; }
+        }
+        __syncwarp();
+        take(best, zbest);
+    }
+    __device__ __forceinline__ void finish(Partial &p) const {
+        if constexpr (REGS) { p.G = G; p.z = z; return; }
+        __syncwarp();
+        warp_result(s, p);
+        __syncwarp();
+    }
+    // what a pass without registers to spare has left, in the warps' first lanes
+    __device__ __forceinline__ static void warp_result(BlockScratch &s, Partial &p) {
+        const bool first = (threadIdx.x & 31) == 0;
+        p.G = first ? s.race_G[threadIdx.x >> 5] : 0ull; p.z = first ? s.race_z[threadIdx.x >> 5] : 0.0f;
+    }
+};
+
+// The race of a vector's elements from `from` on (see race_all), by whole warps.
+template <int OFF, class RACER>
+__device__ __forceinline__ void race_vector(RACER &rc, const uint4 &q, int i0, __nv_bfloat162 top2, float from, float invT, float zref) {
+    constexpr int NB = 2 + (OFF ? 1 : 0);
+    const float xtop = fmaxf(__low2float(top2), __high2float(top2)), top = xtop >= from ? ex2_ftz(log2_mass(__fmul_rn(xtop, invT), zref)) : 0.0f;
+    const float K = rc.K();
+    if (!__any_sync(0xFFFFFFFFu, top * K >= 1.16e-10f)) return;
+    uint32_t w[4 * NB], least = 0xFFFFFFFFu;
+    philox_blocks<NB>(rc.row(), (uint32_t)(i0 >> 2), w);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) least = min(least, w[OFF + j]);
+    if (!__any_sync(0xFFFFFFFFu, least <= rc.word_bound(top, K))) return;
+    rc.template race_hits<ALBIREO_BF16, OFF>(w, q, i0, invT, zref, [&](int j) {
+        const float x = Elem<ALBIREO_BF16>::get(q, j);
+        return x >= from ? ex2_ftz(-log2_mass(__fmul_rn(x, invT), zref)) : INFINITY;
+    });
+}
+
+// The first pass: values counted, s.mm_max the largest order key, s.list_cnt the finite scores among the extras.
+// RACE (no cut; see race_reference): the race as well, against zref in the place of the maximum.
+template <int OFF, bool RACE, class SRC>
+__device__ __noinline__ void counting_pass(SRC src, BlockScratch *sp, float invT, float zref) {
+    BlockScratch &s = block_scratch();
+    const int end = src.end_id();
+    __nv_bfloat162 most = __halves2bfloat162(__ushort_as_bfloat16(0xFF80), __ushort_as_bfloat16(0xFF80));
+    [[maybe_unused]] CountedRacer<false> rc(s);
+    if constexpr (!RACE) src.vectors([&](const uint4 &q0, const uint4 &q1, int i0, int i1) {
+        const __nv_bfloat162 top0 = VecTest<ALBIREO_BF16>::vmax(q0), top1 = VecTest<ALBIREO_BF16>::vmax(q1);
+        most = __hmax2(most, __hmax2(top0, top1));
+        if (i0 < end) count_vector(q0, top0);
+        if (i1 >= 0 && i1 < end) count_vector(q1, top1);
+    });
+    else src.vectors([&](const uint4 &q, int i0) {
+        const __nv_bfloat162 top = VecTest<ALBIREO_BF16>::vmax(q);
+        most = __hmax2(most, top);
+        if (i0 < end) count_vector(q, top);
+        if constexpr (RACE) { __syncwarp(); race_vector<OFF>(rc, q, i0, top, -INFINITY, invT, zref); }
+    });
+    uint32_t kbest = key_of(__fmul_rn(fmaxf(__low2float(most), __high2float(most)), invT)), nfin = 0;
+    src.extras([&](int i, float z) {
+        const uint32_t k = key_of(z);
+        kbest = k > kbest ? k : kbest;
+        nfin += (k >= KEY_MIN_FINITE && k < KEY_POS_INF);
+        if constexpr (RACE) {
+            const float d = __fsub_rn(z, zref);
+            rc.race(d > -3.0e38f, i, z, d, d * 1.4426950408889634f);
+        }
+    });
+    if (kbest < KEY_MIN_FINITE || kbest >= KEY_POS_INF) kbest = 0;
+    kbest = __reduce_max_sync(0xFFFFFFFFu, kbest);
+    nfin = __reduce_add_sync(0xFFFFFFFFu, nfin);
+    if ((threadIdx.x & 31) == 0) { atomicMax(&s.mm_max, kbest); if (nfin) atomicAdd(&s.list_cnt, nfin); }
+}
+template <class SRC>
+__device__ __forceinline__ void run_counting(const SRC &src, BlockScratch &s, bool race, float invT, float zref) {
+    if (!race) { counting_pass<0, false>(src, &s, invT, 0.0f); return; }
+    switch (src.first_id() & 3) {
+        case 0: counting_pass<0, true>(src, &s, invT, zref); break;
+        case 1: counting_pass<1, true>(src, &s, invT, zref); break;
+        case 2: counting_pass<2, true>(src, &s, invT, zref); break;
+        default: counting_pass<3, true>(src, &s, invT, zref); break;
+    }
+}
+// What the race of a row without a cut is run against in the place of the maximum, which is not known yet: the largest score of the block's
+// vectors `q`, one per thread (0 where they have none, and then no bound to start from).  The generator and the race's bound
+// are set up as well.  Contains a barrier, and one has to follow.
+__device__ __forceinline__ float race_reference(BlockScratch &s, const uint4 &q, float invT, const RowParams &rp) {
+    const uint32_t k = __reduce_max_sync(0xFFFFFFFFu, VecTest<ALBIREO_BF16>::vmax_key(q, invT));
+    if ((threadIdx.x & 31) == 0) s.r32a[threadIdx.x >> 5] = k;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const float top = unkey(__reduce_max_sync(0xFFFFFFFFu, lane < NWARPS ? s.r32a[lane] : 0u));
+    const bool some = fabsf(top) < 3.0e38f;
+    if (threadIdx.x == 0) { s.fa.philox = philox_row(rp.seed, rp.R, s.ga.step); s.race_bound = some ? __float_as_uint(RACE_LUCK) : NO_BOUND; }
+    return some ? top : 0.0f;
+}
+// which wide rows are counted (the temperature's bound keeps the scores of different values apart)
+template <int DT>
+__device__ __forceinline__ bool counted_eligible(const RowParams &rp, const RowCtx &c, const SampleArgs &a) {
+    return DT == ALBIREO_BF16 && wide_eligible(rp, a) && !a.exp1 && !(rp.min_p > 0.0f && (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB)) &&
+           c.invT > 1e-18f && c.invT < 1e18f;
+}
+__device__ __forceinline__ bool nothing_cut(const RowParams &rp, const SampleArgs &a) { return !(rp.top_p < 1.0f) && !(rp.min_p > 0.0f) && a.num_top <= 0; }
+// How many of the vectors' elements have a finite score, where not all of those counted at CT_LOW are the `killed`
+// penalised tokens.  Ends with a barrier.
+template <class SRC>
+__device__ __noinline__ uint32_t count_finite(SRC src, BlockScratch *sp, float invT) {
+    BlockScratch &s = block_scratch();
+    const uint32_t thr = VecTest<ALBIREO_BF16>::finite_threshold(invT);
+    uint32_t n = 0;
+    src.vectors([&](const uint4 &q, int) { n += 8u - VecTest<ALBIREO_BF16>::count_not_finite(q, thr, invT); });
+    return (uint32_t)block_sum_u64(s, n);
+}
+// Row (or slice) after the counting pass and a barrier: the number of finite scores among the vectors' elements, and what
+// the table cannot tell (bit 29), or only if the maximum is far above -63.75 (bit 28).  The same in every thread.
+template <class SRC>
+__device__ __forceinline__ uint32_t counted_finite(const SRC &src, BlockScratch &s, float invT, uint32_t killed, uint32_t &flags) {
+    const CountedSmem c = counted_smem();
+    const uint32_t low = c.count[ct_index(CT_LOW)];
+    flags = (c.odd[1] || c.odd[0] > (uint32_t)CT_ODD) ? 0x20000000u : 0u;
+    const uint32_t rest = (uint32_t)src.elements() - low;
+    if (low == killed) return rest;
+    const uint32_t n = count_finite(src, &s, invT);
+    if (n != rest) flags |= 0x10000000u;
+    return n;
+}
+
+// Where the cut and the list end, the same in every CTA.
+struct CountedCut {
+    uint32_t thr_any, thr_win, thr_sure, thr_top;     // raw, packed twice: values from there on matter, are in the window or kept, are kept, are listed
+    uint32_t key_lo, key_hi;                          // the window's order keys, both inclusive: above it kept
+    uint32_t key_seg;                                 // extras above it are in M and n
+    uint32_t key_top;
+    u64 M; uint32_t n;                                // kept for sure, all but the extras above the window and not above key_seg
+    uint32_t fail;
+};
+__device__ __forceinline__ CountedCut &counted_cut(BlockScratch &s) { return *(CountedCut *)s.cut_words; }
+
+// which halves of a word are in the window
+__device__ __forceinline__ uint32_t edge_mask(uint32_t w, uint32_t thr_win, uint32_t thr_sure) {
+    typedef __nv_bfloat162 H2;
+    const H2 h = *reinterpret_cast<const H2 *>(&w);
+    return __hge2_mask(h, *reinterpret_cast<const H2 *>(&thr_win)) & ~__hge2_mask(h, *reinterpret_cast<const H2 *>(&thr_sure));
+}
+// Mass, number and lists of the extras, the race of all that is kept for sure, the window's elements to their list.
+// Vectors with nothing that matters are passed over; the others are worked on by full warps: where only few of a
+// warp's have something they wait in a queue.
+template <int OFF, class SRC>
+__device__ __noinline__ Partial counted_final_pass(SRC src, BlockScratch *sp) {
+    typedef VecTest<ALBIREO_BF16> T;
+    extern __shared__ __align__(128) unsigned char smem[];
+    BlockScratch &s = block_scratch();
+    const CountedCut &cut = counted_cut(s);
+    const WideSmem ws = wide_smem();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint4 *qvec = (uint4 *)(smem + CT_QUEUE_OFF) + wid * RACE_QUEUE;
+    int *qid = (int *)((uint4 *)(smem + CT_QUEUE_OFF) + NWARPS * RACE_QUEUE) + wid * RACE_QUEUE;
+    int qn = 0;                                        // the same in every lane
+    const uint32_t thr_any = cut.thr_any;
+    CountedRacer<SRC::SPARE_REGISTERS> rc(s);
+    src.vectors([&](const uint4 &q0, const uint4 &q1, int i01, int i1) -> bool {
+        uint32_t m0 = 0, m1 = 0;
+        bool in0 = false, in1 = false;
+        if (i01 >= 0) {
+            in0 = T::may_pass(q0, thr_any, 1.0f); in1 = i1 >= 0 && T::may_pass(q1, thr_any, 1.0f);
+            m0 = __ballot_sync(0xFFFFFFFFu, in0); m1 = __ballot_sync(0xFFFFFFFFu, in1);
+            if ((m0 | m1) == 0) return true;
+        } else if (qn == 0) return false;
+#pragma unroll 1
+        do {
+        uint4 q = T::fill();
+        int i0 = i01;
+        bool waiting = i01 < 0;
+        if (!waiting) {
+            const uint32_t m = m0 ? m0 : m1;
+            const bool in = m0 ? in0 : in1;
+            q = m0 ? q0 : q1;
+            if (!m0) { m1 = 0; i0 = i1; }
+            m0 = 0;
+            if (__popc(m) < RACE_DIRECT) {
+                if (in) { const int at = qn + __popc(m & ((1u << lane) - 1u)); qvec[at] = q; qid[at] = i0; }
+                qn += __popc(m);
+                if (qn < 32) continue;
+                waiting = true;
+            }
+        }
+        if (waiting) {
+            const int cnt = qn < 32 ? qn : 32;
+            qn -= cnt;
+            __syncwarp();
+            q = T::fill();
+            i0 = 0;
+            if (lane < cnt) { q = qvec[qn + lane]; i0 = qid[qn + lane]; }
+            __syncwarp();
+        }
+        const volatile CountedCut &c = cut;
+        const float invT = *(const volatile float *)&s.fa.invT;
+        auto append = [&](u64 *list, int cap, uint32_t *cnt, uint32_t bits) {
+            while (bits) { const int x = __ffs(bits) - 1; bits &= bits - 1u; list_append(list, cap, cnt, __fmul_rn(pick_element<ALBIREO_BF16>(q, x), invT), i0 + x); }
+            __syncwarp();
         };
-        // An entry is kept while the mass ahead of it in the order, with the mass kept for sure, is short of
-        // the target.  A short list: every entry adds that mass up (masses over the queues, done with by now),
-        // one barrier in all; from 192 entries on a sort and a prefix sum are faster (2 us against 3 at 300).
-        bool reached;
-        if (L <= 192) {
-            u64 *mass = ws.queue;
-            if ((int)threadIdx.x < L) mass[threadIdx.x] = mass_of(list[threadIdx.x]);
-            __syncthreads();
-            u64 reach = 0;
-            if ((int)threadIdx.x < L) {
-                const u64 C = list[threadIdx.x], own = mass[threadIdx.x];
-                u64 ahead = p.M;
-#pragma unroll 4
-                for (int q = 0; q < L; ++q) ahead += list[q] > C ? mass[q] : 0ull;
-                reach = ahead + own;
-                if (ahead < target) keep(C, own);
-            }
-            reached = __syncthreads_or(reach >= target) != 0;
-        } else {
-            const int P = list_sort(list, L), per = (P + NT - 1) / NT, q0 = (int)threadIdx.x * per, q1 = min(L, q0 + per);
-            u64 local = 0, tot;
-            for (int q = q0; q < q1; ++q) local += mass_of(list[q]);
-            u64 run = p.M + block_exscan_u64(s, local, tot);
-            reached = p.M + tot >= target;
-#pragma unroll 1
-            for (int q = q0; q < q1 && run < target; ++q) {
-                const u64 C = list[q], own = mass_of(C);
-                run += own;
-                keep(C, own);
-            }
-            __syncthreads();
+        const uint32_t thr_sure = c.thr_sure, thr_win = c.thr_win;
+        const uint4 at_edge = make_uint4(edge_mask(q.x, thr_win, thr_sure), edge_mask(q.y, thr_win, thr_sure), edge_mask(q.z, thr_win, thr_sure), edge_mask(q.w, thr_win, thr_sure));
+        if (s.ga.num_top > 0) append(ws.top, W_LIST, &s.cand_cnt, T::elem_bits(q, c.thr_top, invT));
+        if (__any_sync(0xFFFFFFFFu, (at_edge.x | at_edge.y | at_edge.z | at_edge.w) != 0u))
+            append(s.fa.list, s.fa.list_cap, &s.list_cnt, T::elem_bits(q, thr_win, invT) & ~T::elem_bits(q, thr_sure, invT));
+        race_vector<OFF>(rc, q, i0, T::vmax(q), __uint_as_float(thr_sure << 16), invT, *(const volatile float *)&s.fa.zmax);
+        } while (m0 | m1);
+        return true;
+    });
+    Partial p;
+    p.M = 0; p.n = 0;
+    const float zmax = s.fa.zmax;
+    const bool listed = s.ga.num_top > 0;
+    src.extras([&](int i, float z) {
+        const uint32_t k = key_of(z);
+        const bool finite = k < KEY_POS_INF && k >= KEY_MIN_FINITE, sure = finite && k > cut.key_hi;
+        if (listed && finite && k >= cut.key_top) list_append(ws.top, W_LIST, &s.cand_cnt, z, i);
+        if (sure && k <= cut.key_seg) { p.M += mass_fx(z, zmax); ++p.n; }
+        if (finite && !sure && k >= cut.key_lo) list_append(s.fa.list, s.fa.list_cap, &s.list_cnt, z, i);
+        __syncwarp();
+        const float d = __fsub_rn(z, zmax);
+        if (__any_sync(0xFFFFFFFFu, sure)) rc.race(sure, i, z, d, d * 1.4426950408889634f);
+    });
+    rc.finish(p);
+    return p;
+}
+
+// A segment's 16 values by one warp: where the running total from the top of the order (masses, or counts) reaches `need` of what the
+// segment adds.  Which values are ahead of that for sure, which may be the one: lo <= hi, 16 for what follows the segment's last value.
+struct SegmentEnd { int lo, hi; u64 mass_ahead; uint32_t cnt_ahead, cnt_most; };
+template <class TEAM>
+__device__ __forceinline__ SegmentEnd end_in_segment(const TEAM &tm, int seg, bool by_mass, u64 need, u64 seg_mass, uint32_t seg_cnt, float invT, float zmax, float zfloor) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t code = ct_code(seg * CT_PER + (lane & 15));
+    const float z = ct_score(code, invT);
+    uint32_t cnt = 0;
+    if (lane < CT_PER && z >= zfloor)
+        for (int r = 0; r < tm.size; ++r) cnt += *tm.at(&counted_smem().count[ct_index(code)], r);
+    u64 mass = (u64)cnt * mass_fx(z, zmax);
+#pragma unroll
+    for (int o = 1; o < CT_PER; o <<= 1) {
+        const u64 t = __shfl_up_sync(0xFFFFFFFFu, mass, o);
+        const uint32_t tc = __shfl_up_sync(0xFFFFFFFFu, cnt, o);
+        if (lane >= o) { mass += t; cnt += tc; }
+    }
+    const u64 open_mass = seg_mass - __shfl_sync(0xFFFFFFFFu, mass, CT_PER - 1);
+    const uint32_t open_cnt = seg_cnt - __shfl_sync(0xFFFFFFFFu, cnt, CT_PER - 1);
+    const u64 have = by_mass ? mass : (u64)cnt, open = by_mass ? open_mass : (u64)open_cnt;
+    const uint32_t lo = __ballot_sync(0xFFFFFFFFu, lane < CT_PER && have + open >= need), hi = __ballot_sync(0xFFFFFFFFu, lane < CT_PER && have >= need);
+    SegmentEnd e;
+    e.lo = lo ? __ffs(lo) - 1 : CT_PER - 1; e.hi = hi ? __ffs(hi) - 1 : CT_PER;
+    e.mass_ahead = __shfl_sync(0xFFFFFFFFu, mass, max(e.lo - 1, 0)); e.cnt_ahead = __shfl_sync(0xFFFFFFFFu, cnt, max(e.lo - 1, 0));
+    if (e.lo == 0) { e.mass_ahead = 0; e.cnt_ahead = 0; }
+    e.cnt_most = __shfl_sync(0xFFFFFFFFu, cnt, min(e.hi, CT_PER - 1)) + open_cnt;
+    return e;
+}
+// the order key from which on elements belong to the first hi + 1 values of a segment (hi = 16: to the whole of it)
+__device__ __forceinline__ uint32_t ct_key_down_to(int seg, int hi, float invT) {
+    const int j = seg * CT_PER + hi;
+    if (j >= CT_BINS) return KEY_MIN_FINITE;
+    return key_of(ct_score(ct_code(j), invT)) + (hi == CT_PER ? 1u : 0u);
+}
+
+// The masses of a counted row: its extras' and its values', by segments (in shared memory; cut.fail set where an extra has no place), or, with no
+// cut, each thread's share of the sum.
+template <class SRC>
+__device__ __noinline__ u64 counted_masses(SRC src, BlockScratch *sp, float invT, float zmax, uint32_t kfloor, bool no_cut) {
+    BlockScratch &s = block_scratch();
+    const CountedSmem ct = counted_smem();
+    CountedCut &cut = counted_cut(s);
+    const int t = threadIdx.x, n_odd = (int)ct.odd[0];
+    const float zfloor = unkey(kfloor);
+    u64 sum = 0;
+    auto in_segment = [&](int seg, u64 m) {              // (until the thread of the segment turns them into one number)
+        uint32_t *w = (uint32_t *)&ct.seg_mass[seg];
+        atomicAdd(&w[0], (uint32_t)m & 0xFFFFFu); atomicAdd(&w[1], (uint32_t)(m >> 20)); atomicAdd(&ct.seg_cnt[seg], 1u);
+    };
+    src.extras([&](int, float z) {
+        const uint32_t k = key_of(z);
+        if (k >= KEY_POS_INF || k < kfloor) return;
+        const u64 m = mass_fx(z, zmax);
+        if (no_cut) { sum += m; return; }
+        const uint32_t raw = VecTest<ALBIREO_BF16>::raw_threshold(k, invT) & 0xFFFFu;
+        if (raw == 0xFF80u) cut.fail = 1u; else in_segment(ct_place(raw) / CT_PER, m);
+    });
+    for (int j = t; j < n_odd; j += NT) {
+        const float z = ct_score(ct.odd[2 + j], invT);
+        if (!(z >= zfloor)) continue;
+        if (no_cut) sum += mass_fx(z, zmax); else in_segment(4095 / CT_PER, mass_fx(z, zmax));
+    }
+    __syncthreads();
+    const uint32_t first = t < 256 ? 0x4270u - 16u * (uint32_t)t : 0xB280u + 16u * (uint32_t)(t - 256);      // the smallest magnitude
+    const uint4 *words = (const uint4 *)&ct.count[ct_index(first)];
+    u64 mass = 0;
+    uint32_t cnt = 0;
+#pragma unroll
+    for (int i = 0; i < CT_PER / 4; ++i) {
+        const uint4 w = words[i];
+        if ((w.x | w.y | w.z | w.w) == 0u) continue;
+        const uint32_t v[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float z = ct_score(first + 4 * i + j, invT);
+            if (z >= zfloor) { cnt += v[j]; mass += (u64)v[j] * mass_fx(z, zmax); }
         }
-        if (!reached) { out.status |= ROW_NOT_DONE; return out; }
-        block_partial(s, k);
-        p.M += k.M; p.n += k.n;
-        if (k.G > p.G) { p.G = k.G; p.z = k.z; }
     }
-    double lnS = 0.0;
-    if (threadIdx.x < 32) {
-        const u64 S_ref = full ? S_all : p.M;
-        lnS = log((double)S_ref) - LN2_40;
-        const int tok = comp_idx(p.G);
-        out.token = tok < 0 ? 0 : tok;                  // (NaN logits: any id in range)
-        out.n_keep = (int32_t)p.n;
-        out.logprob = (p.n == 1 && !full) ? 0.0f : (float)(((double)p.z - (double)zmax) - lnS);
-    }
-    if (want_list) {
-        if (threadIdx.x == 0) { s.bcast[0] = (u64)__double_as_longlong(lnS); s.found_cnt = p.n; }
-        const int n_all = close_gap(ws.top, W_LIST, n_top, (int)x.far_cand);
-        __syncthreads();
-        const double lnS_all = __longlong_as_double((long long)s.bcast[0]);
-        const uint32_t members = full ? n_fin : s.found_cnt;
-        if ((uint32_t)n_all < min((uint32_t)s.ga.num_top, members) || n_all > W_LIST) { out.status |= ROW_NOT_DONE; return out; }      // (the same in every thread)
-#pragma unroll 1
-        for (int j = threadIdx.x; j < n_all; j += NT) {
-            const u64 C = ws.top[j];
-            uint32_t rank = 0;
+    if (no_cut) return sum + mass;
+    const uint2 x = *(const uint2 *)&ct.seg_mass[t];
+    ct.seg_mass[t] = mass + (u64)x.x + ((u64)x.y << 20);
+    ct.seg_cnt[t] += cnt;
+    return 0;
+}
+// From the segments of all CTAs to the cut (see CountedCut), the same in every CTA; s.bcast[2] and [3]: the mass above the floor and the one to
+// be reached.  False: the table does not tell.
+template <class TEAM>
+__device__ __noinline__ bool counted_locate(BlockScratch *sp, TEAM tm, float invT, float zmax, uint32_t kfloor, bool minp, float top_p, uint32_t n_fin, int list_cap) {
+    typedef VecTest<ALBIREO_BF16> T;
+    BlockScratch &s = block_scratch();
+    const CountedSmem ct = counted_smem();
+    CountedCut &cut = counted_cut(s);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, t = threadIdx.x;
+    const bool topp = top_p < 1.0f, listed = s.ga.num_top > 0;
+    const float zfloor = unkey(kfloor);
+    u64 mass = 0;
+    uint32_t cnt = 0;
 #pragma unroll 4
-            for (int q = 0; q < n_all; ++q) rank += ws.top[q] > C;
-            if (rank < (uint32_t)s.ga.num_top && rank < members) {
-                const int64_t o = (int64_t)b * s.ga.num_top + rank;
-                s.ga.out_top_ids[o] = comp_idx(C);
-                s.ga.out_top_logprobs[o] = (members == 1 && !full) ? 0.0f : (float)(((double)unkey((uint32_t)(C >> 32)) - (double)zmax) - lnS_all);
+    for (int r = 0; r < tm.size; ++r) { mass += *tm.at(&ct.seg_mass[t], r); cnt += *tm.at(&ct.seg_cnt[t], r); }
+    u64 run = mass;
+    uint32_t crun = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const u64 tt = __shfl_up_sync(0xFFFFFFFFu, run, o);
+        const uint32_t tc = __shfl_up_sync(0xFFFFFFFFu, crun, o);
+        if (lane >= o) { run += tt; crun += tc; }
+    }
+    if (lane == 31) { s.red[wid] = run; s.r32a[wid] = crun; }
+    __syncthreads();
+    const u64 wt = lane < NWARPS ? s.red[lane] : 0ull;
+    const uint32_t wc = lane < NWARPS ? s.r32a[lane] : 0u;
+    const u64 S = warp_total(wt);
+    run += warp_total(lane < wid ? wt : 0ull) - mass;
+    crun += __reduce_add_sync(0xFFFFFFFFu, lane < wid ? wc : 0u) - cnt;
+    const u64 target = topp ? topp_target(top_p, S) : S;
+    const u64 want = (u64)min((uint32_t)s.ga.num_top, n_fin);
+    if (topp && run < target && target <= run + mass) { s.found_digit = (uint32_t)t; s.found_above = run; s.bcast[0] = mass; s.r32b[0] = crun; s.r32b[1] = cnt; }
+    if (listed && (u64)crun < want && want <= (u64)crun + cnt) { s.found_cnt = (uint32_t)t; s.bcast[1] = mass; s.r32b[2] = crun; s.r32b[3] = cnt; }
+    __syncthreads();
+    if (wid == 0) {
+        // the cut: the window's values, and those above it
+        const uint32_t n_all = __reduce_add_sync(0xFFFFFFFFu, wc);
+        CountedCut c;
+        c.M = S; c.n = n_all; c.key_lo = 0xFFFFFFFFu; c.key_hi = kfloor - 1u; c.key_seg = c.key_hi; c.fail = 0;
+        c.thr_sure = c.thr_win = T::fill().x;             // (everything: -inf has no mass and does not win)
+        if (minp && !topp) c.thr_sure = c.thr_win = T::raw_threshold(kfloor, invT);
+        if (topp) {
+            const int seg = (int)s.found_digit;
+            if (seg < 0) c.fail = 1u;
+            else {
+                const SegmentEnd e = end_in_segment(tm, seg, true, target - s.found_above, s.bcast[0], s.r32b[1], invT, zmax, zfloor);
+                const uint32_t above = ct_code(seg * CT_PER + e.lo);
+                c.M = s.found_above + e.mass_ahead; c.n = s.r32b[0] + e.cnt_ahead;
+                c.key_hi = key_of(ct_score(above, invT));
+                c.key_lo = max(ct_key_down_to(seg, e.hi, invT), kfloor);
+                c.key_seg = seg == 0 ? 0xFFFFFFFFu : key_of(ct_score(ct_code(seg * CT_PER), invT));
+                c.thr_sure = ct_above(above) * 0x10001u;
+                c.thr_win = e.hi < CT_PER ? ct_code(seg * CT_PER + e.hi) * 0x10001u : T::raw_threshold(c.key_lo, invT);
+                if (e.cnt_most - e.cnt_ahead > (uint32_t)list_cap) c.fail = 1u;
             }
         }
+        if (lane == 0) {
+            cut.M = c.M; cut.n = c.n; cut.key_lo = c.key_lo; cut.key_hi = c.key_hi; cut.key_seg = c.key_seg;
+            cut.thr_sure = c.thr_sure; cut.thr_win = c.thr_win; cut.fail = c.fail;
+        }
+    } else if (wid == 1) {
+        // the list: everything down to the value at which the wanted number is reached
+        uint32_t key_top = kfloor, fail = 0;
+        if (listed && n_fin > (uint32_t)(W_LIST / 2)) {
+            const int seg = (int)s.found_cnt;
+            if (seg < 0) fail = !(minp || topp);         // (fewer than wanted: all that are kept)
+            else {
+                const SegmentEnd e = end_in_segment(tm, seg, false, want - s.r32b[2], s.bcast[1], s.r32b[3], invT, zmax, zfloor);
+                key_top = max(ct_key_down_to(seg, e.hi, invT), kfloor);
+                if (s.r32b[2] + e.cnt_most > (uint32_t)W_LIST) fail = 1u;
+            }
+        }
+        if (lane == 0) { cut.key_top = key_top; cut.thr_top = listed ? T::raw_threshold(key_top, invT) : 0u; s.r32b[8] = fail; }
+    } else if (t == 64) {
+        s.fa.invT = invT; s.fa.zmax = zmax; s.fa.list_cap = list_cap; s.fa.exp1_row = nullptr;
+        s.fa.list = listed ? wide_smem().list : wide_smem().top;
+        s.race_bound = __float_as_uint(RACE_LUCK / ((float)target * (1.0f / FX_SCALE)));
+        s.bcast[2] = S; s.bcast[3] = target;
     }
-    return out;
+    tm.sync();                                           // (everybody has read the tables; lists and queues lie over them)
+    if (cut.fail | s.r32b[8]) return false;
+    if (t == 0) {
+        const float win = __uint_as_float(cut.thr_win << 16), top = __uint_as_float(cut.thr_top << 16);
+        cut.thr_any = listed && top < win ? cut.thr_top : cut.thr_win;
+    }
+    __syncthreads();
+    return true;
+}
+
+// A row (or a team's slices of it) whose values have been counted; with no cut, it has been raced as well.
+// `flags`: see counted_finite, of all CTAs.  As wide_row otherwise.
+template <class SRC, class TEAM>
+__device__ __noinline__ RowOut counted_row(BlockScratch *sp, SRC src, TEAM tm, const RowParams rp, float invT, uint32_t kmax, uint32_t n_fin,
+                                           uint32_t flags, int b, uint32_t status) {
+    BlockScratch &s = block_scratch();
+    const int lane = threadIdx.x & 31, t = threadIdx.x;
+    RowOut out;
+    out.token = 0; out.logprob = 0.0f; out.n_keep = 0; out.n_topk = (int32_t)n_fin; out.status = status | ALBIREO_ROW_GENERAL_PATH;
+    const float zmax = unkey(kmax);
+    const bool topp = rp.top_p < 1.0f, minp = rp.min_p > 0.0f, listed = s.ga.num_top > 0, no_cut = !topp && !minp && !listed;
+    const uint32_t kfloor = minp ? minp_key(zmax, rp.ln_min_p) : KEY_MIN_FINITE;
+    const float zlow = ct_score(CT_LOW, invT);
+    // (values that are counted together must weigh nothing and be below the floor)
+    if ((flags & 0x20000000u) || kfloor > kmax || ((flags & 0x10000000u) && (!(zmax - zlow > 29.0f) || (minp && unkey(kfloor) <= zlow)))) {
+        out.status |= ROW_NOT_COUNTED;
+        return out;
+    }
+    CountedCut &cut = counted_cut(s);
+    if (t == 0) {
+        counted_smem().count[ct_index(CT_LOW)] = 0;
+        cut.fail = src.n_extras() > 4000;                  // (their sums in 32 bits)
+        tm.x->far_cand = 0; tm.x->far_list = 0;
+    }
+    Partial p;
+    p.M = counted_masses(src, sp, invT, zmax, kfloor, no_cut);
+    p.n = 0; p.G = 0; p.z = 0.0f;
+    WideEnd w;
+    w.M0 = 0; w.n0 = 0; w.S = 0; w.S_all = 0; w.zmax = zmax; w.n_fin = n_fin; w.summed = no_cut; w.in_team = false; w.all_kept = !topp && !minp; w.topp = topp;
+    w.full = (s.ga.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) != 0;
+    w.race_from = RACE_FROM;
+    const int list_cap = listed ? W_LIST : W_LIST_ALONE;
+    if (no_cut) {
+        // (raced against a reference of this CTA's own: the score by the row's maximum)
+        CountedRacer<false>::warp_result(s, p);
+        if (p.G) p.G = CountedRacer<false>::code_of_score(__fsub_rn(p.z, zmax) + race_nle(rp.seed, rp.R, s.ga.step, nullptr, comp_idx(p.G)), comp_idx(p.G));
+    } else {
+        if (t < tm.size) *tm.at(&tm.x->fail[tm.rank], t) = cut.fail;       // (a barrier has ended the extras)
+        if (t == 0) { s.found_digit = 0xFFFFFFFFu; s.found_cnt = 0xFFFFFFFFu; s.list_cnt = 0; s.cand_cnt = 0; s.fa.philox = philox_row(rp.seed, rp.R, s.ga.step); }
+        tm.sync();
+        if (__reduce_or_sync(0xFFFFFFFFu, lane < tm.size ? tm.x->fail[lane] : 0u) ||
+            !counted_locate(sp, tm, invT, zmax, kfloor, minp, rp.top_p, n_fin, list_cap)) { out.status |= ROW_NOT_COUNTED; return out; }
+        w.S = w.S_all = s.bcast[2];
+        w.race_from = 0.001f - logf(RACE_LUCK / ((float)s.bcast[3] * (1.0f / FX_SCALE)));
+        switch (src.first_id() & 3) {
+            case 0: p = counted_final_pass<0>(src, &s); break;
+            case 1: p = counted_final_pass<1>(src, &s); break;
+            case 2: p = counted_final_pass<2>(src, &s); break;
+            default: p = counted_final_pass<3>(src, &s); break;
+        }
+        w.M0 = cut.M; w.n0 = cut.n;
+    }
+    return wide_finish(tm, rp.top_p, rp.seed, rp.R, p, w, listed ? wide_smem().list : wide_smem().top, list_cap, nullptr, b, out);
 }

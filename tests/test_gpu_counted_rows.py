@@ -1,0 +1,107 @@
+"""Rows of bfloat16 logits whose values are counted (top-p, min-p that keeps many, lists): the ends of the table of values,
+what has no place in it, cuts in the segments that penalised tokens share, against the oracle."""
+import os
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import albireo_oracle as O
+from paper_2606_01927_b200 import workloads as W
+
+from parity import compare, compare_top_lists, to_host
+
+pytestmark = pytest.mark.gpu
+
+_CORES = len(os.sched_getaffinity(0))
+
+
+@pytest.fixture(scope="module")
+def binding():
+    from paper_2606_01927_b200 import binding as Bd
+    return Bd
+
+
+@pytest.fixture(scope="module")
+def sampler(binding):
+    s = binding.Sampler(max_rows=80, max_vocab=140000, max_history_total=1 << 20)
+    yield s
+    s.close()
+
+
+def rows(kind, B, V, rng):
+    x = rng.standard_normal((B, V)) * 3 - 1.1 * np.log(np.arange(1, V + 1))
+    if kind == "ends":                       # the table's last values, and those just outside it
+        for b in range(B):
+            for v in (-63.75, -63.5, -64.0, -1e4, 2.0 ** -26, -(2.0 ** -26), 2.0 ** -27, -(2.0 ** -27), 1e-39, 0.0, -0.0, 63.75 if b % 3 else 3.0):
+                x[b, rng.integers(0, V, 5)] = v
+            if b % 4 == 1:
+                x[b, rng.integers(0, V)] = 64.0
+    elif kind == "zeros":                    # padding logits: up to 254 of them are listed, more are not
+        for b in range(B):
+            x[b, V - (253 + b % 3):] = 0.0
+            x[b, :V // 2] -= 6.0
+    elif kind == "masked":
+        x[rng.random((B, V)) < 0.6] = -np.inf
+    elif kind == "below":                    # all of the row where values are counted together
+        x = np.minimum(x - 70.0, -60.0)
+    elif kind == "ties":                     # thousands of equal scores at the cut
+        x = np.round(rng.standard_normal((B, V)) * 0.7) + 40.0
+    elif kind == "flat":
+        x = rng.standard_normal((B, V)) * 0.01
+    elif kind == "high":
+        x = x + 50.0
+    return x.astype(np.float32)
+
+
+# 40 rows: two CTAs to a row, 16: eight (slices just large enough to be counted); 80: a CTA to each
+@pytest.mark.parametrize("B,V", [(40, 33007), (16, 131080), (80, 8211)])
+@pytest.mark.parametrize("kind", ["plain", "ends", "zeros", "masked", "below", "ties", "flat", "high"])
+@pytest.mark.parametrize("history", [False, True])
+def test_counted_rows(binding, sampler, B, V, kind, history):
+    rng = np.random.default_rng(500 + B)
+    x = rows(kind, B, V, rng)
+    cls = np.arange(B) % 5
+    w = W.Workload(kind, B, V, W.BF16, W.f32_to_bf16_bits(x), temperature=rng.choice([0.4, 0.9, 1.0, 1.6], B).astype(np.float32),
+                   top_p=np.where(cls == 4, 1.0, 1.0 - 10.0 ** rng.uniform(-3, -0.2, B)).astype(np.float32),
+                   min_p=np.where(cls >= 3, 10.0 ** rng.uniform(-12, -2, B), 0.0).astype(np.float32),
+                   seeds=rng.integers(0, 1 << 62, B).astype(np.uint64), step=9)
+    if history:
+        lens = rng.integers(0, 1200, B)
+        w.history_offsets = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+        w.history_ids = np.minimum(rng.zipf(1.15, int(lens.sum())) - 1, V - 1).astype(np.int32)
+        w.repetition_penalty, w.presence_penalty, w.frequency_penalty = (np.full(B, v, np.float32) for v in (1.13, 0.21, 0.07))
+    for num_top, full in ((0, False), (6, False), (6, True)):
+        w.num_top, w.logprob_full_vocab = num_top, full
+        if full:
+            w.min_p = None
+        ref = O.sample(w, threads=_CORES)
+        t = binding.workload_tensors(w, sampler.device)
+        g = to_host(sampler.albireo_sample(t.pop("logits"), **t, num_top=num_top, want_counts=True, want_status=True,
+                                           flags=binding.FLAG_LOGPROB_FULL_VOCAB if full else 0))
+        rep = compare(w, g, ref)
+        assert rep.ok() and len(rep.excused) <= 1, (rep.summary(), rep.failures[:3], rep.excused[:3])
+        bad = compare_top_lists(w, g, ref)
+        assert not bad, bad[:3]
+
+
+@pytest.mark.parametrize("B", [40, 80])
+def test_no_cut_and_extreme_temperatures(binding, sampler, B):
+    """The race against a reference that is not the maximum: rows whose largest score comes late, and rows whose first
+    vectors hold no finite score; temperatures at which the scores of different values meet."""
+    V = 40003
+    rng = np.random.default_rng(77)
+    x = rng.standard_normal((B, V)).astype(np.float32)
+    late = np.arange(B) % 4 == 1
+    x[late, :20000] -= 50.0
+    x[late, 30001] = 60.0
+    x[np.arange(B) % 4 == 2, :20000] = -np.inf
+    T = np.where(np.arange(B) % 4 == 3, 10.0 ** rng.uniform(-19, 19, B), 1.0).astype(np.float32)
+    for top_p in (1.0, 0.7):
+        w = W.Workload("none", B, V, W.BF16, W.f32_to_bf16_bits(x), temperature=T, top_p=np.full(B, top_p, np.float32),
+                       seeds=np.arange(B, dtype=np.uint64))
+        ref = O.sample(w, threads=_CORES)
+        t = binding.workload_tensors(w, sampler.device)
+        g = to_host(sampler.albireo_sample(t.pop("logits"), **t, want_counts=True, want_status=True))
+        rep = compare(w, g, ref)
+        assert rep.ok() and len(rep.excused) <= 1, (rep.summary(), rep.failures[:3], rep.excused[:3])
