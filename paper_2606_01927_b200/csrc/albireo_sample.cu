@@ -2671,11 +2671,15 @@ int apply_ext(SampleArgs &a, const albireo_sample_ext_t *ext, int B, int V, cons
 }
 
 // The launch shape of a batch: a CTA per row (team 1, ring of nstages), or a cluster of `team` CTAs per row.
-struct LaunchShape { int team, nstages, slice_bytes, list_words; size_t smem; };
+struct LaunchShape { int team, nstages, slice_bytes, list_words; size_t smem; bool counted; };
 
 // What the launch shape depends on: the device's SMs, the dynamic shared memory a CTA may have, and how many
 // clusters of 2^i CTAs (one per SM) are on the device at once.
 struct DeviceShape { int num_sms; size_t max_smem; int teams[5]; };
+
+// Elements of a slice of bfloat16 from which on values are counted (32 top-p rows of 128256 by 4 CTAs 26.6 -> 23.7 us, 74 of 48000 by 2 22.8 -> 21.8;
+// 30 of 64000 by 4 21.4 -> 23.1, so not there: clearing and adding up a table of 8192 counts has to be worth it).
+constexpr long COUNTED_SLICE = 16384;
 
 // Rows are shared by clusters where all of them are on the chip at once, one CTA per SM: then every SM
 // works on the batch and a row's slices stay in shared memory.  That is not B * team <= SMs: a cluster lies within one
@@ -2701,6 +2705,7 @@ bool pick_team(LaunchShape &ls, int B, int V, int esize, bool with_history, cons
         const long general = GENERAL_BYTES + (with_history ? (long)history_smem_bytes(V) : 0);
         if (general > smem) smem = general;
         if (smem > (long)d.max_smem) continue;
+        ls.counted = nids >= COUNTED_SLICE;
         ls.team = team; ls.slice_bytes = (int)slice; ls.list_words = (int)list; ls.smem = (size_t)smem; ls.nstages = 0;
         return true;
     }
@@ -2714,7 +2719,7 @@ bool extras_asked(const SampleArgs &a) {
 // false: the vocabulary is too large for the on-chip tables
 bool pick_shape(LaunchShape &ls, int B, int V, int esize, bool with_history, bool force_general, const DeviceShape &d) {
     if (!force_general && pick_team(ls, B, V, esize, with_history, d)) return true;
-    ls.team = 1; ls.slice_bytes = 0; ls.list_words = 0;
+    ls.team = 1; ls.slice_bytes = 0; ls.list_words = 0; ls.counted = false;
     ls.nstages = ring_stages_for(V, with_history, B <= d.num_sms);
     ls.smem = smem_bytes_for(V, with_history, ls.nstages);
     while (ls.smem > d.max_smem && ls.nstages > 2) ls.smem = smem_bytes_for(V, with_history, --ls.nstages);
@@ -2740,7 +2745,8 @@ cudaError_t launch_sample_kernel_as(int B, const LaunchShape &ls, cudaStream_t s
         ++n;
     }
     cfg.attrs = at; cfg.numAttrs = n;
-    return ls.team > 1 ? cudaLaunchKernelEx(&cfg, albireo_cluster_kernel<DT>, a) 
+    if constexpr (DT == ALBIREO_BF16) { if (ls.counted) return cudaLaunchKernelEx(&cfg, albireo_cluster_kernel<DT, true>, a); }
+    return ls.team > 1 ? cudaLaunchKernelEx(&cfg, albireo_cluster_kernel<DT, false>, a)
            : extras_asked(a) ? cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT, true>, a) : cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT, false>, a);
 }
 cudaError_t launch_sample_kernel(int dtype, int B, const LaunchShape &ls, cudaStream_t st, SampleArgs &a) {
@@ -2756,8 +2762,10 @@ cudaError_t set_up_device(int device, DeviceShape &d) {
     d = DeviceShape();
     if (cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) { cudaGetLastError(); d.num_sms = 0; }
     cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    constexpr int CLUSTER_KERNELS = 4;
     const void *kernels[] = {
-        (const void *)albireo_cluster_kernel<ALBIREO_F32>, (const void *)albireo_cluster_kernel<ALBIREO_BF16>, (const void *)albireo_cluster_kernel<ALBIREO_F16>,
+        (const void *)albireo_cluster_kernel<ALBIREO_F32, false>, (const void *)albireo_cluster_kernel<ALBIREO_BF16, false>,
+        (const void *)albireo_cluster_kernel<ALBIREO_F16, false>, (const void *)albireo_cluster_kernel<ALBIREO_BF16, true>,
         (const void *)albireo_sample_kernel<ALBIREO_F32, false>, (const void *)albireo_sample_kernel<ALBIREO_BF16, false>, (const void *)albireo_sample_kernel<ALBIREO_F16, false>,
         (const void *)albireo_sample_kernel<ALBIREO_F32, true>, (const void *)albireo_sample_kernel<ALBIREO_BF16, true>, (const void *)albireo_sample_kernel<ALBIREO_F16, true>,
         (const void *)albireo_stream_only_kernel<ALBIREO_F32>, (const void *)albireo_stream_only_kernel<ALBIREO_BF16>, (const void *)albireo_stream_only_kernel<ALBIREO_F16>};
@@ -2772,7 +2780,7 @@ cudaError_t set_up_device(int device, DeviceShape &d) {
     const size_t smem = (size_t)optin - st;
     for (const void *k : kernels)
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    for (int i = 0; i < 3; ++i)
+    for (int i = 0; i < CLUSTER_KERNELS; ++i)
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernels[i], cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     d.max_smem = smem;
@@ -2785,7 +2793,7 @@ cudaError_t set_up_device(int device, DeviceShape &d) {
         at.val.clusterDim.x = 1u << i; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
         cfg.attrs = &at; cfg.numAttrs = 1;
         d.teams[i] = d.num_sms >> i;
-        for (int k = 0; k < 3; ++k) {
+        for (int k = 0; k < CLUSTER_KERNELS; ++k) {
             int n = 0;
             if (cudaOccupancyMaxActiveClusters(&n, kernels[k], &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
             if (n < d.teams[i]) d.teams[i] = n;

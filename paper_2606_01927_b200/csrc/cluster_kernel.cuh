@@ -12,7 +12,6 @@
 
 constexpr int SLICE_MIN = 18 * 1024;      // the final stage's scratch lies in CTA 0's slice when that is done with
 constexpr int X_LEAST = 1024;             // penalised tokens and unaligned ends of a slice that are listed on chip, at least
-constexpr int COUNTED_SLICE = 16384;      // elements of a slice from which on its values are counted (see counted_row)
 constexpr int X_ENDS = 16;                // most unaligned ends of a row (14), rounded up
 constexpr int GENERAL_BYTES = HIST_BINS * 16 + GL_CAP * 8 + 4096;      // what the general path lays over the front
 
@@ -148,7 +147,9 @@ __device__ __noinline__ int slice_history(BlockScratch *sp, RowCtx c, const int3
     return (int)U;
 }
 
-template <int DT>
+// COUNTED: with the code for rows counted by value (see counted_row); the launches whose slices are too small for that do
+// without it (counted_slices): beside it their top-p rows took 1.4 us longer, 18.7 against 17.2 for 8 rows of 32000.
+template <int DT, bool COUNTED>
 __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_constant__ SampleArgs a) {
     typedef Elem<DT> E;
     typedef VecTest<DT> T;
@@ -237,7 +238,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     // (Rows are counted by value where a cut or a list has to be found, and in slices that are worth clearing and adding up a
     // table of 8192 counts: 32 top-p rows of 128256 by 4 CTAs 26.6 -> 23.7 us, but 13 of 50257 by 8 21.2 -> 23.1.  With no cut
     // the pass of masses and race is faster than counting and race, 22.4 us against 24.5 for 64 rows of 152064.)
-    const bool cand_row = candidate_eligible(rp, a), counted = !cand_row && nv * E::PER_VEC >= COUNTED_SLICE && !nothing_cut(rp, a) && counted_eligible<DT>(rp, c, a);
+    const bool cand_row = candidate_eligible(rp, a), counted = COUNTED && !cand_row && !nothing_cut(rp, a) && counted_eligible<DT>(rp, c, a);
     if (counted) counted_clear();
     if (o1 > o0) {
         nx = slice_history<DT>(&s, c, a.hist_ids + o0, o1 - o0, ostart, SLICE_OFF, id0, n_slice_ids, tm.rank == 0 ? head : 0,
@@ -267,7 +268,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     const int k = rp.greedy ? 1 : rp.top_k, k_eff = full_list ? max(k, a.num_top) : k;
     uint32_t mk = 0, nfin = 0;
     if (counted) {
-        if constexpr (DT == ALBIREO_BF16) {
+        if constexpr (COUNTED) {
             __syncthreads();
             if (__all_sync(0xFFFFFFFFu, landed)) counting_pass<0, false>(src, &s, c.invT, 0.0f);
         }
@@ -299,7 +300,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     }
     const bool any_late = __syncthreads_or(!landed) != 0;
     uint32_t kmax = s.mm_max, tau_s = 0, tau_p = 0, counted_flags = 0, n_vec = 0;
-    if constexpr (DT == ALBIREO_BF16) { if (counted) n_vec = counted_finite(src, s, c.invT, distinct, counted_flags); }
+    if constexpr (COUNTED) { if (counted) n_vec = counted_finite(src, s, c.invT, distinct, counted_flags); }
     if (cand_row && has_topk && kmax) slice_select(s, cs, mk, k_eff, (k_eff + tm.size - 1) / tm.size, s.mm_min, kmax, tau_s, tau_p);
     asm volatile("barrier.cluster.wait;" ::: "memory");            // (the arrival at the start)
     if ((int)threadIdx.x < tm.size) {
@@ -385,7 +386,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
         if (wide) {
             const uint32_t status = out.status;
             out.status |= ROW_NOT_COUNTED;
-            if constexpr (DT == ALBIREO_BF16) { if (counted) out = counted_row(&s, src, tm, rp, c.invT, kmax, n_fin, bad, b, status); }
+            if constexpr (COUNTED) { if (counted) out = counted_row(&s, src, tm, rp, c.invT, kmax, n_fin, bad, b, status); }
             if (out.status & ROW_NOT_COUNTED) out = wide_row<DT>(s, src, tm, rp, c.invT, kmax, n_fin, b, status);
             done = !(out.status & ROW_NOT_DONE);
             if (!done) out.status = status;

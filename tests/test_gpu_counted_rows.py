@@ -54,8 +54,9 @@ def rows(kind, B, V, rng):
     return x.astype(np.float32)
 
 
-# 40 rows: two CTAs to a row, 16: eight (slices just large enough to be counted); 80: a CTA to each
-@pytest.mark.parametrize("B,V", [(40, 33007), (16, 131080), (80, 8211)])
+# 40 rows: two CTAs to a row, 16: eight (slices just large enough to be counted; of 32760 the last one is 8 ids short of
+# that, and of 32752 both are); 80: a CTA to each
+@pytest.mark.parametrize("B,V", [(40, 33007), (40, 32760), (40, 32752), (16, 131080), (80, 8211)])
 @pytest.mark.parametrize("kind", ["plain", "ends", "zeros", "masked", "below", "ties", "flat", "high"])
 @pytest.mark.parametrize("history", [False, True])
 def test_counted_rows(binding, sampler, B, V, kind, history):
