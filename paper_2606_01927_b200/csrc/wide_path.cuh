@@ -185,6 +185,21 @@ struct RingSlice {
             if (!after && *(volatile uint32_t *)&r.timeout == 0u && !mbar_wait(&r.bar[st], parity)) r.timeout = 1u;
             __syncwarp();
             const uint4 *stage = (const uint4 *)wide_stage(st * tv);
+            if constexpr (!PAIRS && !AFTER) {
+#pragma unroll 1
+                for (int u = 0; u < tv; ++u) {
+                    const int v = (t * tv + u) * NT + (int)threadIdx.x, i0 = head + v * E::PER_VEC;
+                    uint4 q = VecTest<DT>::fill();
+                    if (v < nvec) {
+                        q = stage[u * NT + threadIdx.x];
+                        if (bitmap) {
+                            const uint32_t m = __funnelshift_r(bitmap[i0 >> 5], bitmap[(i0 >> 5) + 1], i0 & 31) & ((1u << E::PER_VEC) - 1u);
+                            if (m) q = kill_elements<DT>(q, m);
+                        }
+                    }
+                    f(q, i0);
+                }
+            } else {
             auto fetch = [&](int u, int i0) -> uint4 {
                 uint4 q = VecTest<DT>::fill();
                 if (!after && (t * tv + u) * NT + (int)threadIdx.x < nvec) {
@@ -207,6 +222,7 @@ struct RingSlice {
                     const uint4 q = fetch(u, i0);
                     if constexpr (AFTER) { if (!f(q, i0) && after) break; } else f(q, i0);
                 }
+            }
             }
             __syncwarp();
             if (after) break;
@@ -771,6 +787,185 @@ __device__ __forceinline__ void race_all(const SRC &src, BlockScratch &s, Partia
     p.M = S.total(); p.n = CUT ? n : 0; p.G = rc.G; p.z = rc.z;
 }
 
+// An element of mass e can only beat a score g if E < e exp(-g), and E = -log1p(-v) >= v: so comparing v / e with
+// K = exp(-g) decides almost every element without a logarithm.  Nor does K take one: an element's own E / e is an upper
+// bound of it, and E <= v (1 + v) up to v = 1/2.  The smallest K of a CTA so far is shared by its threads (s.race_bound,
+// the float's bits).  It starts from a score that the winner of a row of mass S reaches but for 2e-11 of all rows, ln S - 3.2 (the winner's
+// score is ln S - ln E); a row in which none did goes to the general path.
+// (With K from the exact scores alone batches of vectors stopped for several of them, a few hundred cycles each, while the first
+// batches of all warps were under way: 32 top-p rows of 128256 spent 6.0 us in the last pass, 5.4 so.)
+constexpr uint32_t NO_BOUND = 0x7F7FFFFFu;
+__device__ __forceinline__ float unit_below(uint32_t w) { return __uint_as_float((w >> 9) | 0x3F800000u) - 1.0f; }      // v rounded down to 2^-23
+// an upper bound of E / e from v (rounded down) and 1 / e
+__device__ __forceinline__ float race_cap(float v, float inv_e) {
+    const float up = v + 1.1920929e-7f;
+    return v < 0.5f ? 1.0002f * (__fmaf_rn(up, up, up) * inv_e) : 3.0e38f;
+}
+// What the race needs across the vectors of a pass: the generator's row and each thread's best element (order code of the score, ~id, and its z) in
+// registers where there are some to spare (REGS: 128 per thread), else in shared memory, the best by warps in s.race_G and s.race_z -
+// held across the passes' loops they were spilled, and what is spilled comes back from the L2.  (By the other kernel's way
+// 64 rows of 152064 without a cut took 24.5 us instead of 21.9.)
+template <bool REGS>
+struct CountedRacer {
+    BlockScratch &s;
+    PhiloxRow kept;
+    u64 G;
+    float z;
+    __device__ __forceinline__ explicit CountedRacer(BlockScratch &s_) : s(s_), G(0), z(0.0f) {
+        if constexpr (REGS) { kept = s.fa.philox; return; }
+        if ((threadIdx.x & 31) == 0) { s.race_G[threadIdx.x >> 5] = 0; s.race_z[threadIdx.x >> 5] = 0.0f; }
+        __syncwarp();
+    }
+    __device__ __forceinline__ PhiloxRow row() const {
+        if constexpr (REGS) return kept;
+        const volatile PhiloxRow &v = s.fa.philox;
+        PhiloxRow r;
+        r.x0 = v.x0; r.x1 = v.x1; r.x2 = v.x2; r.x3 = v.x3; r.k0 = v.k0; r.k1 = v.k1;
+        return r;
+    }
+    __device__ __forceinline__ float K() const { return __uint_as_float(*(const volatile uint32_t *)&s.race_bound); }
+    // no larger word lets an element of mass e win
+    __device__ __forceinline__ static uint32_t word_bound(float e, float K) { return __float2uint_ru(e * K * 4294967296.0f); }
+    // by whole warps: the lanes' bounds; gives the smallest of all.  (Never 0: masses relative to a reference far below the maximum can be infinite.)
+    __device__ __forceinline__ float tighten(float cap) const {
+        const uint32_t least = __reduce_min_sync(0xFFFFFFFFu, __float_as_uint(fminf(fmaxf(cap, 1e-37f), 3.0e38f)));
+        const float now = K();
+        if (__uint_as_float(least) < now && (threadIdx.x & 31) == 0) atomicMin(&s.race_bound, least);
+        return fminf(__uint_as_float(least), now);
+    }
+    // by whole warps: the lanes' best elements (0: none)
+    __device__ __forceinline__ void take(u64 g, float zg) {
+        if constexpr (REGS) { if (g > G) { G = g; z = zg; } return; }
+        if (!__any_sync(0xFFFFFFFFu, g != 0)) return;
+        warp_best(g, zg);
+        const int wid = threadIdx.x >> 5;
+        if ((threadIdx.x & 31) == 0 && g > s.race_G[wid]) { s.race_G[wid] = g; s.race_z[wid] = zg; }
+        __syncwarp();
+    }
+    __device__ __forceinline__ static u64 code_of_score(float g, int i) { return ((u64)orderable_f32(g) << 32) | (uint32_t)(~(uint32_t)i); }
+    // One element per lane by itself, by whole warps: of log2 mass t2 and d = z - reference (`in`: if it is there at all).
+    __device__ __forceinline__ void race(bool in, int i, float zi, float d, float t2) {
+        uint32_t w[4];
+        philox_blocks<1>(row(), (uint32_t)i >> 2, w);
+        const uint32_t x = (i & 3) == 0 ? w[0] : (i & 3) == 1 ? w[1] : (i & 3) == 2 ? w[2] : w[3];
+        const float v = unit_below(x), inv_e = in ? ex2_ftz(-t2) : INFINITY;
+        if (!__any_sync(0xFFFFFFFFu, v * inv_e <= K())) return;                         // (0 x infinity is no hit)
+        const float least = tighten(in ? race_cap(v, inv_e) : 3.0e38f);
+        take(v * inv_e <= least ? code_of_score(d + nle_once(x), i) : 0ull, zi);
+    }
+    // The elements of a vector, their words w[OFF ..], by whole warps: `inv_mass` of element j gives 1 / e, infinity for one that does not take part.
+    template <int DT, int OFF, int N, class F>
+    __device__ __forceinline__ void race_hits(const uint32_t (&w)[N], const uint4 &q, int i0, float invT, float zref, F &&inv_mass) {
+        constexpr int PV = Elem<DT>::PER_VEC;
+        float cap = 3.0e38f;
+#pragma unroll
+        for (int j = 0; j < PV; ++j) cap = fminf(cap, race_cap(unit_below(w[OFF + j]), inv_mass(j)));
+        const float K = tighten(cap);
+        uint32_t hits = 0;
+#pragma unroll
+        for (int j = 0; j < PV; ++j) hits |= (uint32_t)(unit_below(w[OFF + j]) * inv_mass(j) <= K) << j;
+        u64 best = 0;
+        float zbest = 0.0f;
+        while (hits) {
+            const int x = __ffs(hits) - 1;
+            hits &= hits - 1;
+            uint32_t wx = w[OFF];
+#pragma unroll
+            for (int j = 1; j < PV; ++j) wx = x == j ? w[OFF + j] : wx;
+            const float zx = __fmul_rn(pick_element<DT>(q, x), invT);
+            const u64 g = code_of_score(__fsub_rn(zx, zref) + nle_once(wx), i0 + x);
+            if (g > best) { best = g; zbest = zx; }
+        }
+        __syncwarp();
+        take(best, zbest);
+    }
+    __device__ __forceinline__ void finish(Partial &p) const {
+        if constexpr (REGS) { p.G = G; p.z = z; return; }
+        __syncwarp();
+        warp_result(s, p);
+        __syncwarp();
+    }
+    // what a pass without registers to spare has left, in the warps' first lanes
+    __device__ __forceinline__ static void warp_result(BlockScratch &s, Partial &p) {
+        const bool first = (threadIdx.x & 31) == 0;
+        p.G = first ? s.race_G[threadIdx.x >> 5] : 0ull; p.z = first ? s.race_z[threadIdx.x >> 5] : 0.0f;
+    }
+};
+
+// The same for the kernel with 64 registers per thread, what the race needs in shared memory. (With the row's words and the bound
+// held across the loop 68 to 104 bytes were spilled, and what is spilled comes back from the L2.)
+template <int DT, int OFF, bool CUT, class SRC>
+__device__ __forceinline__ void race_all_shared(const SRC &src, BlockScratch &s, Partial &p) {
+    typedef Elem<DT> E;
+    constexpr int PV = E::PER_VEC, NB = PV / 4 + (OFF ? 1 : 0);
+    const float invT = s.fa.invT, zmax = s.fa.zmax, minus0 = minus_zero(invT);
+    const uint32_t sure = CUT ? s.fa.sure : 0u, win_hi = CUT ? s.fa.win_hi : 0u;
+    MassSum S;
+    uint32_t n = 0;
+    CountedRacer<false> rc(s);
+    // an element at the edge: in the window, or (true) an equal of its first code with a lower id
+    auto edge = [&](int i, float z, uint32_t f) -> bool {
+        const FinalArgs &fa = s.fa;
+        if (!(z >= fa.zfloor)) return false;
+        if (f == sure && (uint32_t)i < fa.id_lo) return true;
+        if (f < win_hi || (f == win_hi && (uint32_t)i <= fa.id_hi)) list_append(fa.list, fa.list_cap, &s.list_cnt, z, i);
+        return false;
+    };
+    src.vectors([&](const uint4 &q, int i0) {
+        float e[PV], top = 0.0f;
+        uint32_t at_edge = 0;
+#pragma unroll
+        for (int j = 0; j < PV; j += 2) {
+            const float2 t2 = log2_mass2(scores_of(E::get(q, j), E::get(q, j + 1), invT, minus0), zmax);
+            e[j] = ex2_ftz(t2.x); e[j + 1] = ex2_ftz(t2.y);
+            if constexpr (CUT) {
+                const uint2 f = code_of2(t2);
+                at_edge |= (uint32_t)(f.x >= sure && f.x <= win_hi) << j | (uint32_t)(f.y >= sure && f.y <= win_hi) << (j + 1);
+                e[j] = f.x < sure ? e[j] : 0.0f; e[j + 1] = f.y < sure ? e[j + 1] : 0.0f;
+                n += (f.x < sure) + (f.y < sure);
+            }
+            S.add2(make_float2(e[j], e[j + 1]));
+            top = fmaxf(top, fmaxf(e[j], e[j + 1]));
+        }
+        if constexpr (CUT) {
+            // (equals kept for sure are put back among the kept ones)
+            while (at_edge) {
+                const int x = __ffs(at_edge) - 1;
+                at_edge &= at_edge - 1;
+                const float z = __fmul_rn(pick_element<DT>(q, x), invT), t2 = log2_mass(z, zmax);
+                if (edge(i0 + x, z, code_of(t2))) {
+                    const float ex = ex2_ftz(t2);
+                    S.add(ex); ++n;
+                    top = fmaxf(top, ex);
+#pragma unroll
+                    for (int j = 0; j < PV; ++j) e[j] = x == j ? ex : e[j];
+                }
+            }
+            __syncwarp();
+        }
+        const float K = rc.K();
+        if (!__any_sync(0xFFFFFFFFu, top * K >= 1.16e-10f)) return;      // v is at least 2^-33
+        uint32_t w[4 * NB], least = 0xFFFFFFFFu;
+        philox_blocks<NB>(rc.row(), (uint32_t)(i0 >> 2), w);
+#pragma unroll
+        for (int j = 0; j < PV; ++j) least = min(least, w[OFF + j]);
+        if (!__any_sync(0xFFFFFFFFu, least <= rc.word_bound(top, K))) return;
+        rc.template race_hits<DT, OFF>(w, q, i0, invT, zmax, [&](int j) { return e[j] > 0.0f ? __fdividef(1.0f, e[j]) : INFINITY; });
+    });
+    src.extras([&](int i, float z) {
+        const float d = __fsub_rn(z, zmax), t2 = log2_mass(z, zmax);
+        bool in = d > -3.0e38f;
+        if constexpr (CUT) {
+            const uint32_t f = code_of(t2);
+            if (in && f >= sure) in = f <= win_hi && edge(i, z, f);
+        }
+        if (in) { S.add(ex2_ftz(t2)); ++n; }
+        rc.race(in, i, z, d, t2);
+    });
+    p.M = S.total(); p.n = CUT ? n : 0;
+    rc.finish(p);
+}
+
 // Mass, number and race of the elements kept for sure, and the lists (arguments in s.fa).  Kept elements
 // are scattered over the lanes, and the race term is long: each warp collects them in a queue and works
 // off 32 at a time.  Without registers to spare, what has been summed up stays in shared memory, a slot per
@@ -870,7 +1065,7 @@ __device__ __forceinline__ void final_pass(const SRC &src, BlockScratch &s, Part
 template <int DT, int OFF, bool CUT>
 __device__ __noinline__ Partial solo_race_all(BlockScratch *sp) {
     Partial p;
-    race_all<DT, OFF, CUT>(RingSlice<DT>(), *sp, p);
+    race_all_shared<DT, OFF, CUT>(RingSlice<DT>(), *sp, p);
     return p;
 }
 template <int DT>
@@ -1183,7 +1378,7 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
     // kept elements that are a good part of the row are raced in place: 25 instructions per element of the
     // row against about 40 per kept element through the queues (`ahead_most` is up to twice their number)
     const bool dense = topp && !minp && !want_list && !exp1_row && win.ahead_most > n_fin / 4;
-    if ((no_cut || dense) && threadIdx.x == 32) s.fa.philox = philox_row(rp.seed, rp.R, s.ga.step);
+    if ((no_cut || dense) && threadIdx.x == 32) { s.fa.philox = philox_row(rp.seed, rp.R, s.ga.step); s.race_bound = __float_as_uint(RACE_LUCK); }
     if (threadIdx.x == 0) {
         FinalArgs &fa = s.fa;
         fa.invT = invT; fa.zmax = zmax; fa.zfloor = zfloor;
@@ -1290,111 +1485,6 @@ __device__ __forceinline__ void count_vector(uint4 q, __nv_bfloat162 top) {
     };
     add(q.x); add(q.y); add(q.z); add(q.w);
 }
-// An element of mass e can only beat a score g if E < e exp(-g), and E = -log1p(-v) >= v: so comparing v / e with
-// K = exp(-g) decides almost every element without a logarithm.  Nor does K take one: an element's own E / e is an upper
-// bound of it, and E <= v (1 + v) up to v = 1/2.  The smallest K of a CTA so far is shared by its threads (s.race_bound,
-// the float's bits).  It starts from a score that the winner of a row of mass S reaches but for 2e-11 of all rows, ln S - 3.2 (the winner's
-// score is ln S - ln E); a row in which none did goes to the general path.
-// (With K from the exact scores alone batches of vectors stopped for several of them, a few hundred cycles each, while the first
-// batches of all warps were under way: 32 top-p rows of 128256 spent 6.0 us in the last pass, 5.4 so.)
-constexpr uint32_t NO_BOUND = 0x7F7FFFFFu;
-__device__ __forceinline__ float unit_below(uint32_t w) { return __uint_as_float((w >> 9) | 0x3F800000u) - 1.0f; }      // v rounded down to 2^-23
-// an upper bound of E / e from v (rounded down) and 1 / e
-__device__ __forceinline__ float race_cap(float v, float inv_e) {
-    const float up = v + 1.1920929e-7f;
-    return v < 0.5f ? 1.0002f * (__fmaf_rn(up, up, up) * inv_e) : 3.0e38f;
-}
-// What the race needs across the vectors of a pass: the generator's row and each thread's best element (order code of the score, ~id, and its z) in
-// registers where there are some to spare (REGS: 128 per thread), else in shared memory, the best by warps in s.race_G and s.race_z -
-// held across the passes' loops they were spilled, and what is spilled comes back from the L2.  (By the other kernel's way
-// 64 rows of 152064 without a cut took 24.5 us instead of 21.9.)
-template <bool REGS>
-struct CountedRacer {
-    BlockScratch &s;
-    PhiloxRow kept;
-    u64 G;
-    float z;
-    __device__ __forceinline__ explicit CountedRacer(BlockScratch &s_) : s(s_), G(0), z(0.0f) {
-        if constexpr (REGS) { kept = s.fa.philox; return; }
-        if ((threadIdx.x & 31) == 0) { s.race_G[threadIdx.x >> 5] = 0; s.race_z[threadIdx.x >> 5] = 0.0f; }
-        __syncwarp();
-    }
-    __device__ __forceinline__ PhiloxRow row() const {
-        if constexpr (REGS) return kept;
-        const volatile PhiloxRow &v = s.fa.philox;
-        PhiloxRow r;
-        r.x0 = v.x0; r.x1 = v.x1; r.x2 = v.x2; r.x3 = v.x3; r.k0 = v.k0; r.k1 = v.k1;
-        return r;
-    }
-    __device__ __forceinline__ float K() const { return __uint_as_float(*(const volatile uint32_t *)&s.race_bound); }
-    // no larger word lets an element of mass e win
-    __device__ __forceinline__ static uint32_t word_bound(float e, float K) { return __float2uint_ru(e * K * 4294967296.0f); }
-    // by whole warps: the lanes' bounds; gives the smallest of all.  (Never 0: masses relative to a reference far below the maximum can be infinite.)
-    __device__ __forceinline__ float tighten(float cap) const {
-        const uint32_t least = __reduce_min_sync(0xFFFFFFFFu, __float_as_uint(fminf(fmaxf(cap, 1e-37f), 3.0e38f)));
-        const float now = K();
-        if (__uint_as_float(least) < now && (threadIdx.x & 31) == 0) atomicMin(&s.race_bound, least);
-        return fminf(__uint_as_float(least), now);
-    }
-    // by whole warps: the lanes' best elements (0: none)
-    __device__ __forceinline__ void take(u64 g, float zg) {
-        if constexpr (REGS) { if (g > G) { G = g; z = zg; } return; }
-        if (!__any_sync(0xFFFFFFFFu, g != 0)) return;
-        warp_best(g, zg);
-        const int wid = threadIdx.x >> 5;
-        if ((threadIdx.x & 31) == 0 && g > s.race_G[wid]) { s.race_G[wid] = g; s.race_z[wid] = zg; }
-        __syncwarp();
-    }
-    __device__ __forceinline__ static u64 code_of_score(float g, int i) { return ((u64)orderable_f32(g) << 32) | (uint32_t)(~(uint32_t)i); }
-    // One element per lane by itself, by whole warps: of log2 mass t2 and d = z - reference (`in`: if it is there at all).
-    __device__ __forceinline__ void race(bool in, int i, float zi, float d, float t2) {
-        uint32_t w[4];
-        philox_blocks<1>(row(), (uint32_t)i >> 2, w);
-        const uint32_t x = (i & 3) == 0 ? w[0] : (i & 3) == 1 ? w[1] : (i & 3) == 2 ? w[2] : w[3];
-        const float v = unit_below(x), inv_e = in ? ex2_ftz(-t2) : INFINITY;
-        if (!__any_sync(0xFFFFFFFFu, v * inv_e <= K())) return;                         // (0 x infinity is no hit)
-        const float least = tighten(in ? race_cap(v, inv_e) : 3.0e38f);
-        take(v * inv_e <= least ? code_of_score(d + nle_once(x), i) : 0ull, zi);
-    }
-    // The elements of a vector, their words w[OFF ..], by whole warps: `inv_mass` of element j gives 1 / e, infinity for one that does not take part.
-    template <int DT, int OFF, int N, class F>
-    __device__ __forceinline__ void race_hits(const uint32_t (&w)[N], const uint4 &q, int i0, float invT, float zref, F &&inv_mass) {
-        constexpr int PV = Elem<DT>::PER_VEC;
-        float cap = 3.0e38f;
-#pragma unroll
-        for (int j = 0; j < PV; ++j) cap = fminf(cap, race_cap(unit_below(w[OFF + j]), inv_mass(j)));
-        const float K = tighten(cap);
-        uint32_t hits = 0;
-#pragma unroll
-        for (int j = 0; j < PV; ++j) hits |= (uint32_t)(unit_below(w[OFF + j]) * inv_mass(j) <= K) << j;
-        u64 best = 0;
-        float zbest = 0.0f;
-        while (hits) {
-            const int x = __ffs(hits) - 1;
-            hits &= hits - 1;
-            uint32_t wx = w[OFF];
-#pragma unroll
-            for (int j = 1; j < PV; ++j) wx = x == j ? w[OFF + j] : wx;
-            const float zx = __fmul_rn(pick_element<DT>(q, x), invT);
-            const u64 g = code_of_score(__fsub_rn(zx, zref) + nle_once(wx), i0 + x);
-            if (g > best) { best = g; zbest = zx; }
-        }
-        __syncwarp();
-        take(best, zbest);
-    }
-    __device__ __forceinline__ void finish(Partial &p) const {
-        if constexpr (REGS) { p.G = G; p.z = z; return; }
-        __syncwarp();
-        warp_result(s, p);
-        __syncwarp();
-    }
-    // what a pass without registers to spare has left, in the warps' first lanes
-    __device__ __forceinline__ static void warp_result(BlockScratch &s, Partial &p) {
-        const bool first = (threadIdx.x & 31) == 0;
-        p.G = first ? s.race_G[threadIdx.x >> 5] : 0ull; p.z = first ? s.race_z[threadIdx.x >> 5] : 0.0f;
-    }
-};
-
 // The race of a vector's elements from `from` on (see race_all), by whole warps.
 template <int OFF, class RACER>
 __device__ __forceinline__ void race_vector(RACER &rc, const uint4 &q, int i0, __nv_bfloat162 top2, float from, float invT, float zref) {
