@@ -153,7 +153,6 @@ struct RingSlice {
     __device__ __forceinline__ int first_id() const { return row_shared().head; }
     __device__ __forceinline__ int end_id() const { return row_shared().head + row_shared().nvec * E::PER_VEC; }
     __device__ __forceinline__ int elements() const { return row_shared().nvec * E::PER_VEC; }
-    __device__ __forceinline__ int n_extras() const { return row_shared().c.has_hist ? (int)row_shared().c.n_distinct : 0; }
     __device__ __forceinline__ static void issue(RowShared &r, int t, int st) {
         Ring rg;
         rg.vps = r.vps; rg.seg_base = r.c.seg_base;
@@ -287,7 +286,6 @@ struct SmemSlice {
     __device__ __forceinline__ int first_id() const { return id0; }
     __device__ __forceinline__ int end_id() const { return id0 + nvec * E::PER_VEC; }
     __device__ __forceinline__ int elements() const { return nvec * E::PER_VEC; }
-    __device__ __forceinline__ int n_extras() const { return nx; }
     template <class F> __device__ __forceinline__ void vectors(F &&f) const {
         extern __shared__ __align__(128) unsigned char smem[];
         const uint4 *vec = (const uint4 *)(smem + vec_off);
@@ -1739,9 +1737,13 @@ __device__ __noinline__ u64 counted_masses(SRC src, BlockScratch *sp, float invT
     const int t = threadIdx.x, n_odd = (int)ct.odd[0];
     const float zfloor = unkey(kfloor);
     u64 sum = 0;
-    auto in_segment = [&](int seg, u64 m) {              // (until the thread of the segment turns them into one number)
+    // (64 bits as two words, the carry by whoever makes the low one wrap: any number of masses may meet in a segment. A
+    // 64-bit add in shared memory is a compare-and-swap loop.)
+    auto in_segment = [&](int seg, u64 m) {
         uint32_t *w = (uint32_t *)&ct.seg_mass[seg];
-        atomicAdd(&w[0], (uint32_t)m & 0xFFFFFu); atomicAdd(&w[1], (uint32_t)(m >> 20)); atomicAdd(&ct.seg_cnt[seg], 1u);
+        const uint32_t lo = (uint32_t)m, was = atomicAdd(&w[0], lo), hi = (uint32_t)(m >> 32) + (was + lo < lo);
+        if (hi) atomicAdd(&w[1], hi);
+        atomicAdd(&ct.seg_cnt[seg], 1u);
     };
     src.extras([&](int, float z) {
         const uint32_t k = key_of(z);
@@ -1773,8 +1775,7 @@ __device__ __noinline__ u64 counted_masses(SRC src, BlockScratch *sp, float invT
         }
     }
     if (no_cut) return sum + mass;
-    const uint2 x = *(const uint2 *)&ct.seg_mass[t];
-    ct.seg_mass[t] = mass + (u64)x.x + ((u64)x.y << 20);
+    ct.seg_mass[t] += mass;
     ct.seg_cnt[t] += cnt;
     return 0;
 }
@@ -1889,7 +1890,7 @@ __device__ __noinline__ RowOut counted_row(BlockScratch *sp, SRC src, TEAM tm, c
     CountedCut &cut = counted_cut(s);
     if (t == 0) {
         counted_smem().count[ct_index(CT_LOW)] = 0;
-        cut.fail = src.n_extras() > 4000;                  // (their sums in 32 bits)
+        cut.fail = 0;
         tm.x->far_cand = 0; tm.x->far_list = 0;
     }
     Partial p;

@@ -106,3 +106,29 @@ def test_no_cut_and_extreme_temperatures(binding, sampler, B):
         g = to_host(sampler.albireo_sample(t.pop("logits"), **t, want_counts=True, want_status=True))
         rep = compare(w, g, ref)
         assert rep.ok() and len(rep.excused) <= 1, (rep.summary(), rep.failures[:3], rep.excused[:3])
+
+
+@pytest.mark.parametrize("B", [40, 80])
+def test_thousands_of_masses_in_a_segment(binding, sampler, B):
+    """Thousands of penalised tokens and zeros of (nearly) the largest mass, all of them in one segment, and the cut far below:
+    their sum passes 2^52, and its low word wraps many times.  More than 2048 distinct ids by one CTA per row: their scores lie in
+    the workspace."""
+    V = 40003
+    rng = np.random.default_rng(11)
+    x = (-0.5 - 2.5 * rng.random((B, V))).astype(np.float32)
+    n = np.where(np.arange(B) % 2 == 0, 3950, 6000)
+    for b in range(B):
+        x[b, :n[b] + 200] = 0.0
+        if b % 3:
+            x[b, 20000] = 2.0 ** -(b % 7)
+    w = W.Workload("zeros", B, V, W.BF16, W.f32_to_bf16_bits(x), temperature=np.ones(B, np.float32), top_p=np.full(B, 0.9, np.float32),
+                   seeds=rng.integers(0, 1 << 62, B).astype(np.uint64), step=3,
+                   history_ids=np.concatenate([np.arange(k) for k in n]).astype(np.int32), history_offsets=np.concatenate([[0], np.cumsum(n)]).astype(np.int32),
+                   repetition_penalty=np.full(B, 1.1, np.float32), presence_penalty=np.zeros(B, np.float32), frequency_penalty=np.zeros(B, np.float32))
+    ref = O.sample(w, threads=_CORES)
+    t = binding.workload_tensors(w, sampler.device)
+    g = to_host(sampler.albireo_sample(t.pop("logits"), **t, want_counts=True, want_status=True))
+    rep = compare(w, g, ref)
+    assert rep.ok() and len(rep.excused) <= 1, (rep.summary(), rep.failures[:3], rep.excused[:3])
+    # (exponentials to 2^-22: the sum of 8000 to 12000 is off by 0.003 at most, a token at the cut weighs 0.1)
+    assert np.abs(g["num_kept"].astype(np.int64) - ref.rows["n_keep"]).max() <= 2
