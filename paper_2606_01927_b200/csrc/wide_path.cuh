@@ -800,16 +800,25 @@ __device__ __forceinline__ float race_cap(float v, float inv_e) {
     return v < 0.5f ? 1.0002f * (__fmaf_rn(up, up, up) * inv_e) : 3.0e38f;
 }
 // What the race needs across the vectors of a pass: the generator's row and each thread's best element (order code of the score, ~id, and its z) in
-// registers where there are some to spare (REGS: 128 per thread), else in shared memory, the best by warps in s.race_G and s.race_z -
+// registers where there are some to spare (IN_REGS: 128 per thread), else in shared memory, the best by warps in s.race_G and s.race_z -
 // held across the passes' loops they were spilled, and what is spilled comes back from the L2.  (By the other kernel's way
 // 64 rows of 152064 without a cut took 24.5 us instead of 21.9.)
-template <bool REGS>
+// LISTED: the reference is not the row's maximum.  A score is z - maximum + (-ln E), rounded, and an equal one by another reference may be
+// rounded otherwise, so the elements that pass the bound are listed (their score and id) and raced when the maximum is known.  The bound
+// has a margin of 2e-4 in the score: rounding does not reach it where the winner is no more than 88 above the reference, and
+// above that all elements pass, their mass being infinite (and the list, mostly, runs over).
+__device__ __forceinline__ u64 *race_list() { extern __shared__ __align__(128) unsigned char smem[]; return (u64 *)(smem + CT_SEG_OFF); }
+enum RaceBest { IN_REGS, IN_SHARED, LISTED };
+constexpr int RACE_LIST = NT;         // entries, where the segments' masses would lie
+template <RaceBest BEST>
 struct CountedRacer {
+    static constexpr bool REGS = BEST == IN_REGS;
     BlockScratch &s;
     PhiloxRow kept;
     u64 G;
     float z;
     __device__ __forceinline__ explicit CountedRacer(BlockScratch &s_) : s(s_), G(0), z(0.0f) {
+        if constexpr (BEST == LISTED) return;
         if constexpr (REGS) { kept = s.fa.philox; return; }
         if ((threadIdx.x & 31) == 0) { s.race_G[threadIdx.x >> 5] = 0; s.race_z[threadIdx.x >> 5] = 0.0f; }
         __syncwarp();
@@ -840,6 +849,10 @@ struct CountedRacer {
         if ((threadIdx.x & 31) == 0 && g > s.race_G[wid]) { s.race_G[wid] = g; s.race_z[wid] = zg; }
         __syncwarp();
     }
+    __device__ __forceinline__ void list(int i, float z_) {
+        const uint32_t at = atomicAdd(&s.cand_cnt, 1u);
+        if (at < (uint32_t)RACE_LIST) race_list()[at] = comp_of(key_of(z_), i);
+    }
     __device__ __forceinline__ static u64 code_of_score(float g, int i) { return ((u64)orderable_f32(g) << 32) | (uint32_t)(~(uint32_t)i); }
     // One element per lane by itself, by whole warps: of log2 mass t2 and d = z - reference (`in`: if it is there at all).
     __device__ __forceinline__ void race(bool in, int i, float zi, float d, float t2) {
@@ -849,7 +862,10 @@ struct CountedRacer {
         const float v = unit_below(x), inv_e = in ? ex2_ftz(-t2) : INFINITY;
         if (!__any_sync(0xFFFFFFFFu, v * inv_e <= K())) return;                         // (0 x infinity is no hit)
         const float least = tighten(in ? race_cap(v, inv_e) : 3.0e38f);
-        take(v * inv_e <= least ? code_of_score(d + nle_once(x), i) : 0ull, zi);
+        if constexpr (BEST == LISTED) {
+            if (v * inv_e <= least) list(i, zi);
+            __syncwarp();
+        } else take(v * inv_e <= least ? code_of_score(d + nle_once(x), i) : 0ull, zi);
     }
     // The elements of a vector, their words w[OFF ..], by whole warps: `inv_mass` of element j gives 1 / e, infinity for one that does not take part.
     template <int DT, int OFF, int N, class F>
@@ -867,26 +883,23 @@ struct CountedRacer {
         while (hits) {
             const int x = __ffs(hits) - 1;
             hits &= hits - 1;
+            const float zx = __fmul_rn(pick_element<DT>(q, x), invT);
+            if constexpr (BEST == LISTED) { list(i0 + x, zx); continue; }
             uint32_t wx = w[OFF];
 #pragma unroll
             for (int j = 1; j < PV; ++j) wx = x == j ? w[OFF + j] : wx;
-            const float zx = __fmul_rn(pick_element<DT>(q, x), invT);
             const u64 g = code_of_score(__fsub_rn(zx, zref) + nle_once(wx), i0 + x);
             if (g > best) { best = g; zbest = zx; }
         }
         __syncwarp();
-        take(best, zbest);
+        if constexpr (BEST != LISTED) take(best, zbest);
     }
     __device__ __forceinline__ void finish(Partial &p) const {
         if constexpr (REGS) { p.G = G; p.z = z; return; }
         __syncwarp();
-        warp_result(s, p);
-        __syncwarp();
-    }
-    // what a pass without registers to spare has left, in the warps' first lanes
-    __device__ __forceinline__ static void warp_result(BlockScratch &s, Partial &p) {
         const bool first = (threadIdx.x & 31) == 0;
         p.G = first ? s.race_G[threadIdx.x >> 5] : 0ull; p.z = first ? s.race_z[threadIdx.x >> 5] : 0.0f;
+        __syncwarp();
     }
 };
 
@@ -900,7 +913,7 @@ __device__ __forceinline__ void race_all_shared(const SRC &src, BlockScratch &s,
     const uint32_t sure = CUT ? s.fa.sure : 0u, win_hi = CUT ? s.fa.win_hi : 0u;
     MassSum S;
     uint32_t n = 0;
-    CountedRacer<false> rc(s);
+    CountedRacer<IN_SHARED> rc(s);
     // an element at the edge: in the window, or (true) an equal of its first code with a lower id
     auto edge = [&](int i, float z, uint32_t f) -> bool {
         const FinalArgs &fa = s.fa;
@@ -1502,13 +1515,13 @@ __device__ __forceinline__ void race_vector(RACER &rc, const uint4 &q, int i0, _
 }
 
 // The first pass: values counted, s.mm_max the largest order key, s.list_cnt the finite scores among the extras.
-// RACE (no cut; see race_reference): the race as well, against zref in the place of the maximum.
+// RACE (no cut; see race_reference): the race as well, against zref in the place of the maximum: its candidates are listed (see CountedRacer).
 template <int OFF, bool RACE, class SRC>
 __device__ __noinline__ void counting_pass(SRC src, BlockScratch *sp, float invT, float zref) {
     BlockScratch &s = block_scratch();
     const int end = src.end_id();
     __nv_bfloat162 most = __halves2bfloat162(__ushort_as_bfloat16(0xFF80), __ushort_as_bfloat16(0xFF80));
-    [[maybe_unused]] CountedRacer<false> rc(s);
+    [[maybe_unused]] CountedRacer<LISTED> rc(s);
     if constexpr (!RACE) src.vectors([&](const uint4 &q0, const uint4 &q1, int i0, int i1) {
         const __nv_bfloat162 top0 = VecTest<ALBIREO_BF16>::vmax(q0), top1 = VecTest<ALBIREO_BF16>::vmax(q1);
         most = __hmax2(most, __hmax2(top0, top1));
@@ -1519,7 +1532,8 @@ __device__ __noinline__ void counting_pass(SRC src, BlockScratch *sp, float invT
         const __nv_bfloat162 top = VecTest<ALBIREO_BF16>::vmax(q);
         most = __hmax2(most, top);
         if (i0 < end) count_vector(q, top);
-        if constexpr (RACE) { __syncwarp(); race_vector<OFF>(rc, q, i0, top, -INFINITY, invT, zref); }
+        __syncwarp();
+        race_vector<OFF>(rc, q, i0, top, -INFINITY, invT, zref);
     });
     uint32_t kbest = key_of(__fmul_rn(fmaxf(__low2float(most), __high2float(most)), invT)), nfin = 0;
     src.extras([&](int i, float z) {
@@ -1556,7 +1570,7 @@ __device__ __forceinline__ float race_reference(BlockScratch &s, const uint4 &q,
     const int lane = threadIdx.x & 31;
     const float top = unkey(__reduce_max_sync(0xFFFFFFFFu, lane < NWARPS ? s.r32a[lane] : 0u));
     const bool some = fabsf(top) < 3.0e38f;
-    if (threadIdx.x == 0) { s.fa.philox = philox_row(rp.seed, rp.R, s.ga.step); s.race_bound = some ? __float_as_uint(RACE_LUCK) : NO_BOUND; }
+    if (threadIdx.x == 0) { s.fa.philox = philox_row(rp.seed, rp.R, s.ga.step); s.race_bound = some ? __float_as_uint(RACE_LUCK) : NO_BOUND; s.cand_cnt = 0; }
     return some ? top : 0.0f;
 }
 // which wide rows are counted (the temperature's bound keeps the scores of different values apart)
@@ -1622,7 +1636,7 @@ __device__ __noinline__ Partial counted_final_pass(SRC src, BlockScratch *sp) {
     int *qid = (int *)((uint4 *)(smem + CT_QUEUE_OFF) + NWARPS * RACE_QUEUE) + wid * RACE_QUEUE;
     int qn = 0;                                        // the same in every lane
     const uint32_t thr_any = cut.thr_any;
-    CountedRacer<SRC::SPARE_REGISTERS> rc(s);
+    CountedRacer<SRC::SPARE_REGISTERS ? IN_REGS : IN_SHARED> rc(s);
     src.vectors([&](const uint4 &q0, const uint4 &q1, int i01, int i1) -> bool {
         uint32_t m0 = 0, m1 = 0;
         bool in0 = false, in1 = false;
@@ -1869,7 +1883,7 @@ __device__ __noinline__ bool counted_locate(BlockScratch *sp, TEAM tm, float inv
     return true;
 }
 
-// A row (or a team's slices of it) whose values have been counted; with no cut, it has been raced as well.
+// A row (or a team's slices of it) whose values have been counted; by one CTA with no cut, it has been raced as well.
 // `flags`: see counted_finite, of all CTAs.  As wide_row otherwise.
 template <class SRC, class TEAM>
 __device__ __noinline__ RowOut counted_row(BlockScratch *sp, SRC src, TEAM tm, const RowParams rp, float invT, uint32_t kmax, uint32_t n_fin,
@@ -1882,8 +1896,9 @@ __device__ __noinline__ RowOut counted_row(BlockScratch *sp, SRC src, TEAM tm, c
     const bool topp = rp.top_p < 1.0f, minp = rp.min_p > 0.0f, listed = s.ga.num_top > 0, no_cut = !topp && !minp && !listed;
     const uint32_t kfloor = minp ? minp_key(zmax, rp.ln_min_p) : KEY_MIN_FINITE;
     const float zlow = ct_score(CT_LOW, invT);
-    // (values that are counted together must weigh nothing and be below the floor)
-    if ((flags & 0x20000000u) || kfloor > kmax || ((flags & 0x10000000u) && (!(zmax - zlow > 29.0f) || (minp && unkey(kfloor) <= zlow)))) {
+    const bool raced = std::is_same<TEAM, SoloTeam>::value && no_cut;
+    // (values that are counted together must weigh nothing and be below the floor; a race that is listed as a whole)
+    if ((raced && s.cand_cnt > (uint32_t)RACE_LIST) || (flags & 0x20000000u) || kfloor > kmax || ((flags & 0x10000000u) && (!(zmax - zlow > 29.0f) || (minp && unkey(kfloor) <= zlow)))) {
         out.status |= ROW_NOT_COUNTED;
         return out;
     }
@@ -1894,17 +1909,20 @@ __device__ __noinline__ RowOut counted_row(BlockScratch *sp, SRC src, TEAM tm, c
         tm.x->far_cand = 0; tm.x->far_list = 0;
     }
     Partial p;
-    p.M = counted_masses(src, sp, invT, zmax, kfloor, no_cut);
+    p.M = counted_masses(src, sp, invT, zmax, kfloor, raced);
     p.n = 0; p.G = 0; p.z = 0.0f;
     WideEnd w;
-    w.M0 = 0; w.n0 = 0; w.S = 0; w.S_all = 0; w.zmax = zmax; w.n_fin = n_fin; w.summed = no_cut; w.in_team = false; w.all_kept = !topp && !minp; w.topp = topp;
+    w.M0 = 0; w.n0 = 0; w.S = 0; w.S_all = 0; w.zmax = zmax; w.n_fin = n_fin; w.summed = raced; w.in_team = false; w.all_kept = !topp && !minp; w.topp = topp;
     w.full = (s.ga.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) != 0;
     w.race_from = RACE_FROM;
     const int list_cap = listed ? W_LIST : W_LIST_ALONE;
-    if (no_cut) {
-        // (raced against a reference of this CTA's own: the score by the row's maximum)
-        CountedRacer<false>::warp_result(s, p);
-        if (p.G) p.G = CountedRacer<false>::code_of_score(__fsub_rn(p.z, zmax) + race_nle(rp.seed, rp.R, s.ga.step, nullptr, comp_idx(p.G)), comp_idx(p.G));
+    if (raced) {
+        if (t < (int)s.cand_cnt) {
+            const u64 C = race_list()[t];
+            const int i = comp_idx(C);
+            p.z = unkey((uint32_t)(C >> 32));
+            p.G = CountedRacer<LISTED>::code_of_score(__fsub_rn(p.z, zmax) + race_nle(rp.seed, rp.R, s.ga.step, nullptr, i), i);
+        }
     } else {
         if (t < tm.size) *tm.at(&tm.x->fail[tm.rank], t) = cut.fail;       // (a barrier has ended the extras)
         if (t == 0) { s.found_digit = 0xFFFFFFFFu; s.found_cnt = 0xFFFFFFFFu; s.list_cnt = 0; s.cand_cnt = 0; s.fa.philox = philox_row(rp.seed, rp.R, s.ga.step); }

@@ -132,3 +132,35 @@ def test_thousands_of_masses_in_a_segment(binding, sampler, B):
     assert rep.ok() and len(rep.excused) <= 1, (rep.summary(), rep.failures[:3], rep.excused[:3])
     # (exponentials to 2^-22: the sum of 8000 to 12000 is off by 0.003 at most, a token at the cut weighs 0.1)
     assert np.abs(g["num_kept"].astype(np.int64) - ref.rows["n_keep"]).max() <= 2
+
+
+@pytest.mark.parametrize("kind", ["low", "masked", "dense"])
+def test_ties_far_above_the_first_vectors(binding, sampler, kind):
+    """Rows without a cut by one CTA each are raced before their maximum is known: equal maxima behind the first 4096 ids, at
+    temperatures that take them up to 1e9 above all that lies ahead (`low`), behind ids that are masked, and hundreds of thousands of units above
+    rows of which half is at the maximum (`dense`).  Only the generator's words tell them apart; the same rows by clusters give the same bits."""
+    B, V = 80, 40003
+    rng = np.random.default_rng(5)
+    x = rng.standard_normal((B, V)).astype(np.float32)
+    x[:, :4200] = -np.inf if kind == "masked" else -5.0
+    for b in range(B):
+        if kind == "dense":
+            x[b, 4200:][rng.random(V - 4200) < 0.5] = 8.0
+        else:
+            x[b, rng.integers(4200, V, 40)] = 8.0
+            start = 4200 + 8 * int(rng.integers(0, 4000))
+            x[b, start:start + 24] = 8.0
+    T = np.where(np.arange(B) % 2 == 0, 10.0 ** rng.uniform(-8, -4, B), 10.0 ** rng.uniform(-4, 0, B)).astype(np.float32)
+    w = W.Workload("ties", B, V, W.BF16, W.f32_to_bf16_bits(x), temperature=T, seeds=rng.integers(0, 1 << 62, B).astype(np.uint64), step=5)
+    ref = O.sample(w, threads=_CORES)
+    t = binding.workload_tensors(w, sampler.device)
+    logits, step = t.pop("logits"), t.pop("step")
+    g = to_host(sampler.albireo_sample(logits, **t, step=step, want_counts=True, want_status=True))
+    rep = compare(w, g, ref)
+    assert rep.ok() and len(rep.excused) <= 1, (rep.summary(), rep.failures[:3], rep.excused[:3])
+    for lo in (0, 40):
+        part = to_host(sampler.albireo_sample(logits[lo:lo + 40], **{k: v[lo:lo + 40] for k, v in t.items() if v is not None}, step=step, row_base=lo,
+                                              want_counts=True))
+        for f in ("tokens", "num_kept", "num_topk"):
+            assert (part[f] == g[f][lo:lo + 40]).all(), (f, lo)
+        assert (part["logprobs"].view(np.uint32) == g["logprobs"][lo:lo + 40].view(np.uint32)).all(), lo
