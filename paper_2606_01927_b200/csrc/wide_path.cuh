@@ -1460,6 +1460,17 @@ __device__ __forceinline__ int ct_place(uint32_t c) {
 __device__ __forceinline__ float ct_score(uint32_t c, float invT) { return __fmul_rn(__uint_as_float(c << 16), invT); }
 __device__ __forceinline__ u64 mass_fx(float z, float zmax) { return __float2ull_rn(ex2_ftz(log2_mass(z, zmax)) * FX_SCALE); }
 
+// Where the cut and the list end, the same in every CTA.
+struct CountedCut {
+    uint32_t thr_any, thr_win, thr_sure, thr_top;     // raw, packed twice: values from there on matter, are in the window or kept, are kept, are listed
+    uint32_t key_lo, key_hi;                          // the window's order keys, both inclusive: above it kept
+    uint32_t key_seg;                                 // extras above it are in M and n
+    uint32_t key_top;
+    u64 M; uint32_t n;                                // kept for sure, all but the extras above the window and not above key_seg
+    uint32_t fail;                                    // (0 ahead of the counting pass: any thread may set it from there on)
+};
+__device__ __forceinline__ CountedCut &counted_cut(BlockScratch &s) { return *(CountedCut *)s.cut_words; }
+
 // (by whole blocks; a barrier must follow)
 __device__ __forceinline__ void counted_clear() {
     const CountedSmem c = counted_smem();
@@ -1467,6 +1478,7 @@ __device__ __forceinline__ void counted_clear() {
     for (int i = 0; i < CT_PER / 4; ++i) ((uint4 *)c.count)[i * NT + threadIdx.x] = make_uint4(0, 0, 0, 0);
     c.seg_mass[threadIdx.x] = 0ull; c.seg_cnt[threadIdx.x] = 0u;
     if (threadIdx.x < 2) c.odd[threadIdx.x] = 0u;
+    if (threadIdx.x == 0) counted_cut(block_scratch()).fail = 0u;
 }
 __device__ __noinline__ void count_odd_vector(uint4 q) {
     const CountedSmem c = counted_smem();
@@ -1603,17 +1615,6 @@ __device__ __forceinline__ uint32_t counted_finite(const SRC &src, BlockScratch 
     if (n != rest) flags |= 0x10000000u;
     return n;
 }
-
-// Where the cut and the list end, the same in every CTA.
-struct CountedCut {
-    uint32_t thr_any, thr_win, thr_sure, thr_top;     // raw, packed twice: values from there on matter, are in the window or kept, are kept, are listed
-    uint32_t key_lo, key_hi;                          // the window's order keys, both inclusive: above it kept
-    uint32_t key_seg;                                 // extras above it are in M and n
-    uint32_t key_top;
-    u64 M; uint32_t n;                                // kept for sure, all but the extras above the window and not above key_seg
-    uint32_t fail;
-};
-__device__ __forceinline__ CountedCut &counted_cut(BlockScratch &s) { return *(CountedCut *)s.cut_words; }
 
 // which halves of a word are in the window
 __device__ __forceinline__ uint32_t edge_mask(uint32_t w, uint32_t thr_win, uint32_t thr_sure) {
@@ -1905,7 +1906,6 @@ __device__ __noinline__ RowOut counted_row(BlockScratch *sp, SRC src, TEAM tm, c
     CountedCut &cut = counted_cut(s);
     if (t == 0) {
         counted_smem().count[ct_index(CT_LOW)] = 0;
-        cut.fail = 0;
         tm.x->far_cand = 0; tm.x->far_list = 0;
     }
     Partial p;

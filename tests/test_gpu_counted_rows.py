@@ -164,3 +164,23 @@ def test_ties_far_above_the_first_vectors(binding, sampler, kind):
         for f in ("tokens", "num_kept", "num_topk"):
             assert (part[f] == g[f][lo:lo + 40]).all(), (f, lo)
         assert (part["logprobs"].view(np.uint32) == g["logprobs"][lo:lo + 40].view(np.uint32)).all(), lo
+
+
+@pytest.mark.parametrize("B", [40, 80])
+def test_penalised_scores_without_a_place(binding, sampler, B):
+    """Penalties that take scores beyond every value of the logits' type, up (a negative presence penalty) or down: such a token has no place
+    in the table, whichever thread comes upon it."""
+    V = 40003
+    rng = np.random.default_rng(3)
+    x = rng.standard_normal((B, V)).astype(np.float32)
+    n = 1 + np.arange(B) * 37
+    w = W.Workload("beyond", B, V, W.BF16, W.f32_to_bf16_bits(x), temperature=np.ones(B, np.float32), top_p=np.full(B, 0.7, np.float32),
+                   seeds=rng.integers(0, 1 << 62, B).astype(np.uint64), step=3,
+                   history_ids=np.concatenate([rng.permutation(V)[:k] for k in n]).astype(np.int32), history_offsets=np.concatenate([[0], np.cumsum(n)]).astype(np.int32),
+                   repetition_penalty=np.ones(B, np.float32), frequency_penalty=np.zeros(B, np.float32),
+                   presence_penalty=np.where(np.arange(B) % 2 == 0, -3.4e38, 3.4e38).astype(np.float32))
+    ref = O.sample(w, threads=_CORES)
+    t = binding.workload_tensors(w, sampler.device)
+    g = to_host(sampler.albireo_sample(t.pop("logits"), **t, want_counts=True, want_status=True))
+    rep = compare(w, g, ref)
+    assert rep.ok() and len(rep.excused) <= 1, (rep.summary(), rep.failures[:3], rep.excused[:3])
