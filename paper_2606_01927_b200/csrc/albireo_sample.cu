@@ -167,7 +167,6 @@ struct FinalArgs {
     uint32_t vec_thr;                    // raw threshold of the vector test
     int list_cap;
     u64 *list;                           // the window's list
-    PhiloxRow philox;
     uint64_t seed, step;
     uint32_t R;
     const float *exp1_row;
@@ -183,16 +182,15 @@ struct BlockScratch {
     uint32_t cand_cnt, overflow, runmax, timeout;
     uint32_t r32a[NWARPS], r32b[NWARPS];
     uint32_t mm_max, mm_min;
-    uint32_t done[MAX_STAGES];   // warps finished with each ring stage
+    union {
+        uint32_t done[MAX_STAGES];                          // warps finished with each ring stage (candidate path)
+        struct { PhiloxRow philox; uint32_t bound; } race;  // wide path: the generator's row, and the race's bound so far (see CountedRacer)
+    };
     uint32_t maint_at;           // tile index before which every warp meets (0xFFFFFFFF: none)
     uint32_t issued;             // tiles whose copy has been issued so far
     const char *seg_base[ALBIREO_MAX_SEGMENTS];   // where this row's pieces start (rows in pieces only)
     uint32_t nfin_cap;           // general path: min(#finite scores, ALBIREO_MAX_NUM_TOP + 1), parked here until the list is written
     FinalArgs fa;
-    u64 cut_words[8];            // CountedCut (wide_path.cuh)
-    u64 race_G[NWARPS];          // the race: each warp's best element, the bound so far (see CountedRacer)
-    float race_z[NWARPS];
-    uint32_t race_bound;
     GenArgs ga;                  // the general path's copy of the launch arguments it uses
 };
 
@@ -1789,14 +1787,14 @@ __device__ __forceinline__ bool wide_eligible(const RowParams &rp, const SampleA
 // block in shared memory, and the ring's barriers.
 template <int DT>
 __device__ __forceinline__ void passes_begin(BlockScratch &s, const RowCtx &c, int vps, int nstages) {
-    RowShared &r = row_shared();
+    RowShared &r = row_shared<DT>();
     r.c = c; r.vps = vps;
     const uintptr_t addr = (uintptr_t)c.row;
     int head = (int)(((16u - (uint32_t)(addr & 15u)) & 15u) / Elem<DT>::SIZE);
     if (head > c.V) head = c.V;
     r.head = head; r.nvec = (c.V - head) / Elem<DT>::PER_VEC;
     r.vp = (const uint4 *)((const char *)c.row + (size_t)head * Elem<DT>::SIZE);
-    const int room = (COMMON_BYTES + nstages * STAGE_BYTES - WIDE_RING_OFF) / WIDE_VEC_BYTES;
+    const int room = (COMMON_BYTES + nstages * STAGE_BYTES - wide_ring_off(DT)) / WIDE_VEC_BYTES;
     r.tv = room >= 8 ? 4 : 2;
     r.nst = min(WIDE_MAX_STAGES, room / r.tv);
 #pragma unroll 1
@@ -1805,8 +1803,8 @@ __device__ __forceinline__ void passes_begin(BlockScratch &s, const RowCtx &c, i
     r.tiles = 0; r.issued = 0; r.timeout = 0; s.mm_max = 0; s.list_cnt = 0;
 }
 // The ring's barriers are done with (thread 0): their memory may be used for something else.
-__device__ __forceinline__ void passes_end() {
-    RowShared &r = row_shared();
+template <int DT> __device__ __forceinline__ void passes_end() {
+    RowShared &r = row_shared<DT>();
     for (int q = 0; q < r.nst; ++q) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(&r.bar[q])) : "memory");
 }
 // The row's largest order key (s.mm_max) and the number of its finite scores (s.list_cnt), after passes_begin.
@@ -1814,7 +1812,7 @@ template <int DT>
 __device__ __noinline__ void max_and_count(BlockScratch *sp) {
     BlockScratch &s = block_scratch();
     const RingSlice<DT> src;
-    const float invT = row_shared().c.invT;
+    const float invT = row_shared<DT>().c.invT;
     const uint32_t fin_thr = VecTest<DT>::finite_threshold(invT);
     uint32_t kbest = 0, nfin = 0;
     src.vectors([&](const uint4 &q, int) {
@@ -1838,13 +1836,13 @@ __device__ __noinline__ void whole_row_totals(BlockScratch *sp, float zmax) {
     BlockScratch &s = block_scratch();
     max_and_count<DT>(sp);
     u64 S, S_all;
-    mass_pass<DT, SUM_ONLY, false>(RingSlice<DT>(), row_shared().c.invT, zmax, 0.0f, 0u, 0, S, S_all);
+    mass_pass<DT, SUM_ONLY, false>(RingSlice<DT>(), row_shared<DT>().c.invT, zmax, 0.0f, 0u, 0, S, S_all);
     S = block_sum_u64(s, S);
     if (threadIdx.x == 0) {
-        RowShared &r = row_shared();
+        RowShared &r = row_shared<DT>();
         s.bcast[0] = S; s.bcast[1] = s.list_cnt;
         if (r.timeout) s.timeout = 1u;
-        passes_end();
+        passes_end<DT>();
     }
     __syncthreads();
 }
@@ -2188,10 +2186,10 @@ __device__ __forceinline__ bool candidate_path(BlockScratch &s, const CandSmem &
             // A pass over the whole row that only some calls ask for, out of line.  What is needed behind it waits in
             // shared memory: kept in registers it was spilled ahead of the stream for every call (256 rows with counts
             // 19.5 -> 23.0 us).
-            if (threadIdx.x == 0) { passes_begin<DT>(s, c, a.vps, a.nstages); row_shared().rp = rp; s.bcast[3] = tau; }
+            if (threadIdx.x == 0) { passes_begin<DT>(s, c, a.vps, a.nstages); row_shared<DT>().rp = rp; s.bcast[3] = tau; }
             __syncthreads();
             whole_row_totals<DT>(&s, unkey(kmax));
-            rq = row_shared().rp;
+            rq = row_shared<DT>().rp;
             full_fx = full_lp ? s.bcast[0] : 0ull; n_fin = s.bcast[1];
             tau = (uint32_t)s.bcast[3]; n = (int)s.cand_cnt; kmax = s.runmax;
             if (s.timeout) { out.status |= ALBIREO_ROW_TIMEOUT; out.token = -1; out.logprob = __uint_as_float(0x7FC00000u); out.n_keep = 0; out.n_topk = 0; return true; }
@@ -2295,8 +2293,8 @@ __device__ __noinline__ void leftover_row(BlockScratch *sp, const SampleArgs *ap
     if (threadIdx.x == 0) {
         fill_general_args(s.ga, a);
         passes_begin<DT>(s, c, a.vps, a.nstages);
-        row_shared().rp = rp;
-        s.race_bound = NO_BOUND;
+        row_shared<DT>().rp = rp;
+        s.race.bound = NO_BOUND;
     }
     // The penalised tokens' scores take the place of their counts: the passes look them up, where each of them would fetch
     // their logits again (a scattered load per token and pass, 2 us a round next to CTAs that stream).
@@ -2316,13 +2314,13 @@ __device__ __noinline__ void leftover_row(BlockScratch *sp, const SampleArgs *ap
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) row_shared().c.scored = score;
+    if (threadIdx.x == 0) row_shared<DT>().c.scored = score;
     RowOut out;
     out.status = status | ROW_NOT_DONE;
     if (wide_eligible(rp, a)) {
-        const RowShared &r = row_shared();
+        const RowShared &r = row_shared<DT>();
         const RingSlice<DT> src;
-        SoloTeam tm;
+        SoloTeam<counts_rows(DT)> tm;
         uint32_t kmax = 0, n_fin = 0;
         out.status = status | ROW_NOT_COUNTED;
         if constexpr (DT == ALBIREO_BF16) {
@@ -2337,7 +2335,7 @@ __device__ __noinline__ void leftover_row(BlockScratch *sp, const SampleArgs *ap
                     if (c.has_hist) q = kill_elements<DT>(q, __funnelshift_r(c.bitmap[i0 >> 5], c.bitmap[(i0 >> 5) + 1], i0 & 31));
                 }
                 const float zref = race ? race_reference(s, q, c.invT, rp) : 0.0f;
-                counted_clear();
+                counted_clear(src);
                 // the penalised tokens among the row's vectors
                 if (c.has_hist) {
                     const int tail0 = src.end_id(), x = (int)threadIdx.x, i = x < r.head ? x : tail0 + (x - r.head);
@@ -2365,9 +2363,9 @@ __device__ __noinline__ void leftover_row(BlockScratch *sp, const SampleArgs *ap
         if (r.timeout) { out.status = (out.status & ~ROW_NOT_DONE) | ALBIREO_ROW_TIMEOUT; out.token = -1; out.logprob = __uint_as_float(0x7FC00000u); out.n_keep = 0; out.n_topk = 0; }
     }
     if (out.status & ROW_NOT_DONE) {
-        c = row_shared().c; rp = row_shared().rp;
+        c = row_shared<DT>().c; rp = row_shared<DT>().rp;
         __syncthreads();                                       // the general path lays its own tables over them
-        if (threadIdx.x == 0) passes_end();
+        if (threadIdx.x == 0) passes_end<DT>();
         __syncthreads();
         out = general_path_call<DT>(sp, smem, c, rp, b, status);
     }
@@ -2687,27 +2685,32 @@ constexpr long COUNTED_SLICE = 16384;
 // than that a batch took up to twice as long (8 top-p rows of 152064 35.4 us by 16 CTAs each, 21.1 by 8).  (Two CTAs per SM, with half the registers,
 // were 10 % slower on the rows without a top-k and the same on the others.)  Of the sizes that fit, the largest whose slices are
 // still at least 8 KB (one vector per thread): below that the exchange costs more than the slice.
-bool pick_team(LaunchShape &ls, int B, int V, int esize, bool with_history, const DeviceShape &d) {
+bool pick_team(LaunchShape &ls, int B, int V, int dtype, bool with_history, const DeviceShape &d) {
+    const int esize = dtype == ALBIREO_F32 ? 4 : 2;
     const long row_bytes = (long)(V / (16 / esize)) * 16;
     for (int team = MAX_TEAM, i = 4; team >= 2; team >>= 1, --i) {
         if (row_bytes / team < 8192 || B > d.teams[i]) continue;
         const long per = ((row_bytes / 16 + team - 1) / team) * 16;
         const long slice = ((per > SLICE_MIN ? per : (long)SLICE_MIN) + 127) & ~127L;
-        const long nids = per / esize, fixed = SLICE_OFF + slice + 16 + (with_history ? 4L * slice_counts_off((int)nids) : 0);
-        long list = 2L * X_ENDS;
-        if (with_history) {
-            list = 2L * (nids + X_ENDS);
-            const long room = ((long)d.max_smem - fixed) / 4;
-            if (room < list) list = room & ~1L;
-            if (list < 2L * X_LEAST && list < 2L * (nids + X_ENDS)) continue;
+        const long nids = per / esize;
+        // (with the table of values, where there is room for it)
+        for (int counted = dtype == ALBIREO_BF16 && nids >= COUNTED_SLICE; counted >= 0; --counted) {
+            const long fixed = slice_off(counted) + slice + 16 + slice_tables(counted, with_history, (int)nids);
+            long list = 2L * X_ENDS;
+            if (with_history) {
+                list = 2L * (nids + X_ENDS);
+                const long room = ((long)d.max_smem - fixed) / 4;
+                if (room < list) list = room & ~1L;
+                if (list < 2L * X_LEAST && list < 2L * (nids + X_ENDS)) continue;
+            }
+            long smem = fixed + 4 * list;
+            const long general = GENERAL_BYTES + (with_history ? (long)history_smem_bytes(V) : 0);
+            if (general > smem) smem = general;
+            if (smem > (long)d.max_smem) continue;
+            ls.counted = counted != 0;
+            ls.team = team; ls.slice_bytes = (int)slice; ls.list_words = (int)list; ls.smem = (size_t)smem; ls.nstages = 0;
+            return true;
         }
-        long smem = fixed + 4 * list;
-        const long general = GENERAL_BYTES + (with_history ? (long)history_smem_bytes(V) : 0);
-        if (general > smem) smem = general;
-        if (smem > (long)d.max_smem) continue;
-        ls.counted = nids >= COUNTED_SLICE;
-        ls.team = team; ls.slice_bytes = (int)slice; ls.list_words = (int)list; ls.smem = (size_t)smem; ls.nstages = 0;
-        return true;
     }
     return false;
 }
@@ -2717,8 +2720,8 @@ bool extras_asked(const SampleArgs &a) {
 }
 
 // false: the vocabulary is too large for the on-chip tables
-bool pick_shape(LaunchShape &ls, int B, int V, int esize, bool with_history, bool force_general, const DeviceShape &d) {
-    if (!force_general && pick_team(ls, B, V, esize, with_history, d)) return true;
+bool pick_shape(LaunchShape &ls, int B, int V, int dtype, bool with_history, bool force_general, const DeviceShape &d) {
+    if (!force_general && pick_team(ls, B, V, dtype, with_history, d)) return true;
     ls.team = 1; ls.slice_bytes = 0; ls.list_words = 0; ls.counted = false;
     ls.nstages = ring_stages_for(V, with_history, B <= d.num_sms);
     ls.smem = smem_bytes_for(V, with_history, ls.nstages);
@@ -2927,7 +2930,7 @@ extern "C" int albireo_sample(albireo_sampler_t *h, const void *logits, int32_t 
     if (cudaGetDevice(&cur) != cudaSuccess || cur != h->device) { cudaGetLastError(); set_err(h, "the handle's device is not current%s", ""); return ALBIREO_EINVAL; }
 
     LaunchShape ls;
-    if (!pick_shape(ls, B, V, (int)esize, history_ids != nullptr, (a.flags & ALBIREO_FLAG_FORCE_GENERAL) != 0, h->dev)) { set_err(h, "vocabulary too large for the on-chip tables%s", ""); return ALBIREO_EUNSUPPORTED; }
+    if (!pick_shape(ls, B, V, dtype, history_ids != nullptr, (a.flags & ALBIREO_FLAG_FORCE_GENERAL) != 0, h->dev)) { set_err(h, "vocabulary too large for the on-chip tables%s", ""); return ALBIREO_EUNSUPPORTED; }
     cudaStream_t st = (cudaStream_t)stream;
     const cudaError_t e = launch_sample_kernel(dtype, B, ls, st, a);
     if (e != cudaSuccess) { cudaGetLastError(); set_err(h, "kernel launch failed: %s", cudaGetErrorString(e)); return ALBIREO_ECUDA; }
@@ -3164,7 +3167,7 @@ extern "C" int albireo_sample_fixed_scratch(const void *logits, int32_t B, int32
     a.ws_counts_cap = ALBIREO_FIXED_MAX_HISTORY;
 
     LaunchShape ls;
-    if (!pick_shape(ls, B, V, (int)esize, history_ids != nullptr, (a.flags & ALBIREO_FLAG_FORCE_GENERAL) != 0, d->shape)) return fixed_fail(ALBIREO_EUNSUPPORTED, "vocabulary too large for the on-chip tables%s", "");
+    if (!pick_shape(ls, B, V, dtype, history_ids != nullptr, (a.flags & ALBIREO_FLAG_FORCE_GENERAL) != 0, d->shape)) return fixed_fail(ALBIREO_EUNSUPPORTED, "vocabulary too large for the on-chip tables%s", "");
     cudaStream_t st = (cudaStream_t)stream;
     const cudaError_t e = launch_sample_kernel(dtype, B, ls, st, a);
     if (e != cudaSuccess) { cudaGetLastError(); return fixed_fail(ALBIREO_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e)); }

@@ -20,6 +20,12 @@ constexpr int GENERAL_BYTES = HIST_BINS * 16 + GL_CAP * 8 + 4096;      // what t
 __host__ __device__ constexpr int slice_coarse_off(int n) { return (((n + 31) / 32) + 4) & ~3; }
 __host__ __device__ constexpr int slice_counts_off(int n) { return slice_coarse_off(n) + ((n + 31) / 32 + 7) / 8 + 1; }
 
+// Bytes of what lies between a slice and the scores of its penalised tokens: those tables, or, when they are done with, what counted rows need.
+__host__ __device__ constexpr int slice_tables(bool counted, bool with_history, int n) {
+    const int tables = with_history ? 4 * slice_counts_off(n) : 0;
+    return counted && tables < (int)sizeof(CountedSegs) ? (int)sizeof(CountedSegs) : tables;
+}
+
 // The k-th and the kp-th largest of the block's per-thread maxima `mk` (0: none), from below: the
 // smallest maximum of the value-linear bin in which the count from the top gets there (see
 // warm_select).  0 where there are fewer maxima.
@@ -75,13 +81,13 @@ __device__ void slice_select(BlockScratch &, const CandSmem &cs, uint32_t mk, in
 // `landed()` waits for the slice; everything before it overlaps the copy.
 template <int DT, class W>
 __device__ __noinline__ int slice_history(BlockScratch *sp, RowCtx c, const int32_t *ids, int len, int out_start, int slice_off, int id0, int nids,
-                                          int id_lo, int id_hi, int tab_off, int list_words, uint32_t *ws, int64_t ws_cap, int64_t ws_off,
+                                          int id_lo, int id_hi, int tab_off, int xz_off, int list_words, uint32_t *ws, int64_t ws_cap, int64_t ws_off,
                                           W landed, bool &ok, int *&xid) {
     typedef Elem<DT> E;
     BlockScratch &s = block_scratch();
     extern __shared__ __align__(128) unsigned char smem[];
     const int nwords = (nids + 31) >> 5, ncoarse = (nwords + 7) >> 3;
-    uint32_t *bitmap = (uint32_t *)(smem + tab_off), *coarse = bitmap + slice_coarse_off(nids), *counts = bitmap + slice_counts_off(nids);
+    uint32_t *bitmap = (uint32_t *)(smem + tab_off), *coarse = bitmap + slice_coarse_off(nids), *counts = (uint32_t *)(smem + xz_off);
     uint32_t ahead = 0, own = 0;           // history ids ahead of the slice and in it
     for (int w = threadIdx.x; w <= nwords; w += NT) bitmap[w] = 0;
     __syncthreads();
@@ -155,7 +161,8 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     typedef VecTest<DT> T;
     extern __shared__ __align__(128) unsigned char smem[];
     BlockScratch &s = block_scratch();
-    ClusterTeam tm;
+    constexpr int SLICE_OFF = slice_off(COUNTED);
+    ClusterTeam<COUNTED> tm;
     tm.rank = (int)cg::this_cluster().block_rank(); tm.size = (int)cg::this_cluster().num_blocks();
     const int b = blockIdx.x / tm.size, V = a.V, lane = threadIdx.x & 31;
     uint64_t *bar = (uint64_t *)(smem + SLICE_OFF + a.slice_bytes);
@@ -172,7 +179,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
         mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        s.cand_cnt = 0; s.runmax = 0; s.race_bound = NO_BOUND; s.mm_max = 0; s.mm_min = 0xFFFFFFFFu; s.list_cnt = 0;
+        s.cand_cnt = 0; s.runmax = 0; s.race.bound = NO_BOUND; s.mm_max = 0; s.mm_min = 0xFFFFFFFFu; s.list_cnt = 0;
         tm.x->far_cand = 0; tm.x->far_list = 0;
     }
     if (threadIdx.x < NWARPS) s.red[threadIdx.x] = 0;
@@ -231,18 +238,17 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     int nx = 0;
     const int n_slice_ids = nv * E::PER_VEC;
     SmemSlice<DT> src;
-    src.vec_off = SLICE_OFF; src.nvec = nv; src.id0 = id0;
+    src.vec_off = SLICE_OFF; src.nvec = nv; src.id0 = id0; src.seg_off = tab_off;
     // (a launch without histories has no tables: only the row's unaligned ends are listed)
-    src.xz_off = tables ? tab_off + slice_counts_off(n_slice_ids) * 4 : tab_off;
+    src.xz_off = tab_off + slice_tables(COUNTED, tables, n_slice_ids);
     int *xid = (int *)(smem + src.xz_off) + (a.list_words >> 1);
     // (Rows are counted by value where a cut or a list has to be found, and in slices that are worth clearing and adding up a
     // table of 8192 counts: 32 top-p rows of 128256 by 4 CTAs 26.6 -> 23.7 us, but 13 of 50257 by 8 21.2 -> 23.1.  With no cut
     // the pass of masses and race is faster than counting and race, 22.4 us against 24.5 for 64 rows of 152064.)
     const bool cand_row = candidate_eligible(rp, a), counted = COUNTED && !cand_row && !nothing_cut(rp, a) && counted_eligible<DT>(rp, c, a);
-    if (counted) counted_clear();
     if (o1 > o0) {
         nx = slice_history<DT>(&s, c, a.hist_ids + o0, o1 - o0, ostart, SLICE_OFF, id0, n_slice_ids, tm.rank == 0 ? head : 0,
-                               tm.rank == 0 ? tail0 : V, tab_off, a.list_words, a.ws_counts, a.ws_counts_cap, (int64_t)o0,
+                               tm.rank == 0 ? tail0 : V, tab_off, src.xz_off, a.list_words, a.ws_counts, a.ws_counts_cap, (int64_t)o0,
                                [&] { return mbar_wait(bar, 0); }, landed, xid);
         if (nx < 0) { nx = 0; fits = false; }
     } else landed = mbar_wait(bar, 0);
@@ -269,6 +275,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     uint32_t mk = 0, nfin = 0;
     if (counted) {
         if constexpr (COUNTED) {
+            counted_clear(src);
             __syncthreads();
             if (__all_sync(0xFFFFFFFFu, landed)) counting_pass<0, false>(src, &s, c.invT, 0.0f);
         }

@@ -22,7 +22,8 @@ constexpr int MAX_TEAM = 16;
 
 // Words that the CTAs of a row exchange: slot r is written by CTA r, in every CTA or only in CTA 0's copy.
 struct TeamWords {
-    uint32_t kmax[MAX_TEAM], tau[MAX_TEAM], tau_part[MAX_TEAM], nfin[MAX_TEAM], flags[MAX_TEAM], ncand[MAX_TEAM], fail[MAX_TEAM];   // in every CTA
+    uint32_t kmax[MAX_TEAM], tau[MAX_TEAM], tau_part[MAX_TEAM], nfin[MAX_TEAM], flags[MAX_TEAM];   // in every CTA
+    uint32_t ncand[MAX_TEAM];         // (rows counted by value: whether the table cannot tell)
     u64 ahead[MAX_TEAM];                                                                                           // in every CTA
     u64 S[MAX_TEAM], S_all[MAX_TEAM], M[MAX_TEAM], G[MAX_TEAM];                                                    // in CTA 0's
     uint32_t n[MAX_TEAM];
@@ -30,19 +31,25 @@ struct TeamWords {
     uint32_t far_cand, far_list;      // CTA 0: entries that the others have put at the far end of its lists
 };
 
-__device__ __forceinline__ TeamWords &team_words();
+// (COUNTED here and below: in a kernel with the table of rows counted by value, which lies in front of them)
+template <bool COUNTED> __device__ __forceinline__ TeamWords &team_words();
+template <bool COUNTED>
 struct TeamWordsHere {                // this CTA's (named anew at every use, see block_scratch)
-    __device__ __forceinline__ TeamWords *operator->() const { return &team_words(); }
-    __device__ __forceinline__ TeamWords &operator*() const { return team_words(); }
+    __device__ __forceinline__ TeamWords *operator->() const { return &team_words<COUNTED>(); }
+    __device__ __forceinline__ TeamWords &operator*() const { return team_words<COUNTED>(); }
 };
+template <bool COUNTED>
 struct SoloTeam {                     // a CTA that has the row to itself
-    TeamWordsHere x;
+    TeamWordsHere<COUNTED> x;
+    static constexpr bool ALONE = true;
     static constexpr int rank = 0, size = 1;
     __device__ __forceinline__ void sync() const { __syncthreads(); }
     template <class P> __device__ __forceinline__ P *at(P *p, int) const { return p; }
 };
+template <bool COUNTED>
 struct ClusterTeam {                  // the CTAs of a thread-block cluster
-    TeamWordsHere x;
+    TeamWordsHere<COUNTED> x;
+    static constexpr bool ALONE = false;
     int rank, size;
     __device__ __forceinline__ void sync() const {
         asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
@@ -144,27 +151,29 @@ struct RowShared {
     uint32_t done[WIDE_MAX_STAGES];
     uint64_t bar[WIDE_MAX_STAGES];
 };
-__device__ __forceinline__ RowShared &row_shared();
-__device__ __forceinline__ unsigned char *wide_stage(int st);
+template <int DT> __device__ __forceinline__ RowShared &row_shared();
+template <int DT> __device__ __forceinline__ unsigned char *wide_stage(int st);
+template <int DT> __device__ __forceinline__ constexpr int row_segments();
 template <int DT>
 struct RingSlice {
     typedef Elem<DT> E;
     static constexpr bool SPARE_REGISTERS = false;      // 64 per thread
-    __device__ __forceinline__ int first_id() const { return row_shared().head; }
-    __device__ __forceinline__ int end_id() const { return row_shared().head + row_shared().nvec * E::PER_VEC; }
-    __device__ __forceinline__ int elements() const { return row_shared().nvec * E::PER_VEC; }
+    __device__ __forceinline__ int first_id() const { return row_shared<DT>().head; }
+    __device__ __forceinline__ int end_id() const { return row_shared<DT>().head + row_shared<DT>().nvec * E::PER_VEC; }
+    __device__ __forceinline__ int elements() const { return row_shared<DT>().nvec * E::PER_VEC; }
+    __device__ __forceinline__ int segments() const { return row_segments<DT>(); }      // (counted rows: see CountedSegs)
     __device__ __forceinline__ static void issue(RowShared &r, int t, int st) {
         Ring rg;
         rg.vps = r.vps; rg.seg_base = r.c.seg_base;
         const int v0 = t * (NT * r.tv), nv = min(r.nvec - v0, NT * r.tv);
         mbar_expect_tx(&r.bar[st], (uint32_t)nv * 16u);
-        ring_copy(rg, wide_stage(st * r.tv), r.vp, v0, nv, &r.bar[st]);
+        ring_copy(rg, wide_stage<DT>(st * r.tv), r.vp, v0, nv, &r.bar[st]);
     }
     // The tiles of all passes are numbered through, which gives stage and phase; the last warp done with a
     // stage refills it.  A wait that expires marks the row, and nothing more is copied.
     template <class F> __device__ __forceinline__ void vectors(F &&f) const {
         constexpr bool AFTER = goes_on<F>, PAIRS = by_pairs<F>;
-        RowShared &r = row_shared();
+        RowShared &r = row_shared<DT>();
         const uint32_t first = r.tiles;
         const int nvec = r.nvec, head = r.head, nst = r.nst, tv = r.tv, ntiles = (nvec + NT * tv - 1) / (NT * tv);
         const uint32_t *bitmap = r.c.has_hist ? r.c.bitmap : nullptr;
@@ -183,7 +192,7 @@ struct RingSlice {
             const bool after = AFTER && t == ntiles;
             if (!after && *(volatile uint32_t *)&r.timeout == 0u && !mbar_wait(&r.bar[st], parity)) r.timeout = 1u;
             __syncwarp();
-            const uint4 *stage = (const uint4 *)wide_stage(st * tv);
+            const uint4 *stage = (const uint4 *)wide_stage<DT>(st * tv);
             if constexpr (!PAIRS && !AFTER) {
 #pragma unroll 1
                 for (int u = 0; u < tv; ++u) {
@@ -251,7 +260,7 @@ struct RingSlice {
         __syncthreads();
     }
     template <class F> __device__ __forceinline__ void extras(F &&f) const {
-        const RowShared &r = row_shared();
+        const RowShared &r = row_shared<DT>();
         const RowCtx &c = r.c;
         const int head = r.head, tail0 = head + r.nvec * E::PER_VEC, nscal = head + (c.V - tail0);
         const int total = nscal + (c.has_hist ? (int)c.n_distinct : 0);
@@ -281,11 +290,13 @@ struct SmemSlice {
     typedef Elem<DT> E;
     static constexpr bool SPARE_REGISTERS = true;       // 128 per thread
     int vec_off, nvec, id0;       // where the slice and the list lie in the dynamic shared memory
+    int seg_off;                  // (counted rows: see CountedSegs)
     const int *xid;               // (in the workspace where there are too many for both lists on chip)
     int xz_off, nx;
     __device__ __forceinline__ int first_id() const { return id0; }
     __device__ __forceinline__ int end_id() const { return id0 + nvec * E::PER_VEC; }
     __device__ __forceinline__ int elements() const { return nvec * E::PER_VEC; }
+    __device__ __forceinline__ int segments() const { return seg_off; }
     template <class F> __device__ __forceinline__ void vectors(F &&f) const {
         extern __shared__ __align__(128) unsigned char smem[];
         const uint4 *vec = (const uint4 *)(smem + vec_off);
@@ -358,24 +369,43 @@ struct WideSmem {
 // The front of the dynamic shared memory, whatever the kernel keeps behind it
 // (the candidate list and its select bins lie where the top-N list does).
 constexpr int WIDE_LIST_OFF = COMMON_BYTES, WIDE_HIST_OFF = WIDE_LIST_OFF + W_LIST * 8;
-constexpr int WIDE_QUEUE_OFF = WIDE_HIST_OFF + W_BINS * 4;
-// (rows of bfloat16 whose values are counted: see counted_row.  The table lies over all of the above, the queues of its
-// last pass behind the lists.)
-constexpr int CT_BINS = 8192, CT_ODD = 254;
+constexpr int WIDE_QUEUE_OFF = WIDE_HIST_OFF + W_BINS * 4, WIDE_BYTES = WIDE_QUEUE_OFF + NWARPS * 64 * 8;
+static_assert(W_LIST_ALONE * 8 <= WIDE_HIST_OFF, "the window's list alone lies over both lists and the select bins");
+// Rows of bfloat16 whose values are counted (see counted_row): the table of counts lies over all of the above, the queues of the last
+// pass, when it is done with, behind the lists.  What else they need (CountedSegs) lies where the kernel has room: in a cluster
+// over the tables of the history, of which only the scores are still wanted.
+constexpr int CT_BINS = 8192, CT_ODD = 254, CT_BYTES = CT_BINS * 4;
 constexpr int RACE_DIRECT = 13;       // so many of a warp's vectors at once are raced in place
 constexpr int RACE_QUEUE = 44;        // vectors that a warp's queue holds: 31 left over and RACE_DIRECT - 1
-constexpr int CT_SEG_OFF = CT_BINS * 4, CT_CNT_OFF = CT_SEG_OFF + NT * 8, CT_ODD_OFF = CT_CNT_OFF + NT * 4;
 constexpr int CT_QUEUE_OFF = WIDE_LIST_OFF + W_LIST * 8;
-constexpr int WIDE_BYTES = CT_ODD_OFF + (CT_ODD + 2) * 4;
-static_assert(WIDE_QUEUE_OFF + NWARPS * 64 * 8 <= CT_SEG_OFF && CT_QUEUE_OFF + NWARPS * RACE_QUEUE * 20 <= CT_SEG_OFF, "queues in front of the segments");
-static_assert(W_LIST_ALONE * 8 <= WIDE_HIST_OFF, "the window's list alone lies over both lists and the select bins");
-constexpr int TEAM_OFF = WIDE_BYTES, SLICE_OFF = (TEAM_OFF + (int)sizeof(TeamWords) + 127) & ~127;
-__device__ __forceinline__ TeamWords &team_words() { extern __shared__ __align__(128) unsigned char smem[]; return *(TeamWords *)(smem + TEAM_OFF); }
-// (a CTA that has the row to itself: the row's own block and the ring of its passes follow)
-constexpr int ROW_OFF = SLICE_OFF, WIDE_RING_OFF = (ROW_OFF + (int)sizeof(RowShared) + 127) & ~127;
-__device__ __forceinline__ RowShared &row_shared() { extern __shared__ __align__(128) unsigned char smem[]; return *(RowShared *)(smem + ROW_OFF); }
-__device__ __forceinline__ unsigned char *wide_stage(int st) { extern __shared__ __align__(128) unsigned char smem[]; return smem + WIDE_RING_OFF + st * WIDE_VEC_BYTES; }
-// (taken from the kernel's own shared array, so that the compiler knows the address space)
+static_assert(WIDE_BYTES <= CT_BYTES && CT_QUEUE_OFF + NWARPS * RACE_QUEUE * 20 <= CT_BYTES, "lists and queues in front of the team's words");
+// Where the cut and the list end, the same in every CTA.
+struct CountedCut {
+    uint32_t thr_any, thr_win, thr_sure, thr_top;     // raw, packed twice: values from there on matter, are in the window or kept, are kept, are listed
+    uint32_t key_lo, key_hi;                          // the window's order keys, both inclusive: above it kept
+    uint32_t key_seg;                                 // extras above it are in M and n
+    uint32_t key_top;
+    u64 M; uint32_t n;                                // kept for sure, all but the extras above the window and not above key_seg
+    uint32_t fail;                                    // (0 ahead of the counting pass: any thread may set it from there on)
+};
+struct CountedSegs {
+    u64 mass[NT];                     // by segments of 16 values; with no cut the list of the race (RACE_LIST) lies here
+    uint32_t cnt[NT];
+    uint32_t n_odd, lost, odd[CT_ODD];        // values nearer to zero than the table's, and whether there are values above it
+    CountedCut cut;
+};
+// The slices of a cluster begin behind the team's words; by one CTA the row's own block and the ring of its passes do.  (At 128 bytes: 30 rows
+// of 152064 with a top-k took 10.7 us with slices at 16, 10.3 so.)
+__host__ __device__ constexpr int team_off(bool counted) { return counted ? CT_BYTES : WIDE_BYTES; }
+__host__ __device__ constexpr int slice_off(bool counted) { return (team_off(counted) + (int)sizeof(TeamWords) + 127) & ~127; }
+template <bool COUNTED> __device__ __forceinline__ TeamWords &team_words() { extern __shared__ __align__(128) unsigned char smem[]; return *(TeamWords *)(smem + team_off(COUNTED)); }
+__host__ __device__ constexpr bool counts_rows(int dt) { return dt == ALBIREO_BF16; }      // the kernel of one CTA per row
+__host__ __device__ constexpr int row_off(int dt) { return slice_off(counts_rows(dt)) + (counts_rows(dt) ? (int)sizeof(CountedSegs) : 0); }
+__host__ __device__ constexpr int wide_ring_off(int dt) { return (row_off(dt) + (int)sizeof(RowShared) + 127) & ~127; }
+template <int DT> __device__ __forceinline__ constexpr int row_segments() { return slice_off(counts_rows(DT)); }
+template <int DT> __device__ __forceinline__ RowShared &row_shared() { extern __shared__ __align__(128) unsigned char smem[]; return *(RowShared *)(smem + row_off(DT)); }
+template <int DT> __device__ __forceinline__ unsigned char *wide_stage(int st) { extern __shared__ __align__(128) unsigned char smem[]; return smem + wide_ring_off(DT) + st * WIDE_VEC_BYTES; }
+static_assert(sizeof(CountedSegs) % 16 == 0 && sizeof(RowShared) % 8 == 0, "what follows is aligned");
 __device__ __forceinline__ WideSmem wide_smem() {
     extern __shared__ __align__(128) unsigned char smem[];
     WideSmem w;
@@ -706,7 +736,7 @@ __device__ __forceinline__ void race_all(const SRC &src, BlockScratch &s, Partia
     uint32_t n = 0;
     Racer rc;
     rc.start(RACE_LUCK);
-    const PhiloxRow pr = s.fa.philox;
+    const PhiloxRow pr = s.race.philox;
     // an element by itself
     auto race_one = [&](int i, float z, float e) {
         uint32_t w[4];
@@ -787,7 +817,7 @@ __device__ __forceinline__ void race_all(const SRC &src, BlockScratch &s, Partia
 
 // An element of mass e can only beat a score g if E < e exp(-g), and E = -log1p(-v) >= v: so comparing v / e with
 // K = exp(-g) decides almost every element without a logarithm.  Nor does K take one: an element's own E / e is an upper
-// bound of it, and E <= v (1 + v) up to v = 1/2.  The smallest K of a CTA so far is shared by its threads (s.race_bound,
+// bound of it, and E <= v (1 + v) up to v = 1/2.  The smallest K of a CTA so far is shared by its threads (s.race.bound,
 // the float's bits).  It starts from a score that the winner of a row of mass S reaches but for 2e-11 of all rows, ln S - 3.2 (the winner's
 // score is ln S - ln E); a row in which none did goes to the general path.
 // (With K from the exact scores alone batches of vectors stopped for several of them, a few hundred cycles each, while the first
@@ -800,14 +830,14 @@ __device__ __forceinline__ float race_cap(float v, float inv_e) {
     return v < 0.5f ? 1.0002f * (__fmaf_rn(up, up, up) * inv_e) : 3.0e38f;
 }
 // What the race needs across the vectors of a pass: the generator's row and each thread's best element (order code of the score, ~id, and its z) in
-// registers where there are some to spare (IN_REGS: 128 per thread), else in shared memory, the best by warps in s.race_G and s.race_z -
+// registers where there are some to spare (IN_REGS: 128 per thread), else in shared memory, the best by warps where block_partial takes it from -
 // held across the passes' loops they were spilled, and what is spilled comes back from the L2.  (By the other kernel's way
 // 64 rows of 152064 without a cut took 24.5 us instead of 21.9.)
 // LISTED: the reference is not the row's maximum.  A score is z - maximum + (-ln E), rounded, and an equal one by another reference may be
 // rounded otherwise, so the elements that pass the bound are listed (their score and id) and raced when the maximum is known.  The bound
 // has a margin of 2e-4 in the score: rounding does not reach it where the winner is no more than 88 above the reference, and
 // above that all elements pass, their mass being infinite (and the list, mostly, runs over).
-__device__ __forceinline__ u64 *race_list() { extern __shared__ __align__(128) unsigned char smem[]; return (u64 *)(smem + CT_SEG_OFF); }
+__device__ __forceinline__ u64 *race_list() { extern __shared__ __align__(128) unsigned char smem[]; return ((CountedSegs *)(smem + row_segments<ALBIREO_BF16>()))->mass; }
 enum RaceBest { IN_REGS, IN_SHARED, LISTED };
 constexpr int RACE_LIST = NT;         // entries, where the segments' masses would lie
 template <RaceBest BEST>
@@ -819,25 +849,25 @@ struct CountedRacer {
     float z;
     __device__ __forceinline__ explicit CountedRacer(BlockScratch &s_) : s(s_), G(0), z(0.0f) {
         if constexpr (BEST == LISTED) return;
-        if constexpr (REGS) { kept = s.fa.philox; return; }
-        if ((threadIdx.x & 31) == 0) { s.race_G[threadIdx.x >> 5] = 0; s.race_z[threadIdx.x >> 5] = 0.0f; }
+        if constexpr (REGS) { kept = s.race.philox; return; }
+        if ((threadIdx.x & 31) == 0) { s.red2[threadIdx.x >> 5] = 0; s.r32b[threadIdx.x >> 5] = 0; }
         __syncwarp();
     }
     __device__ __forceinline__ PhiloxRow row() const {
         if constexpr (REGS) return kept;
-        const volatile PhiloxRow &v = s.fa.philox;
+        const volatile PhiloxRow &v = s.race.philox;
         PhiloxRow r;
         r.x0 = v.x0; r.x1 = v.x1; r.x2 = v.x2; r.x3 = v.x3; r.k0 = v.k0; r.k1 = v.k1;
         return r;
     }
-    __device__ __forceinline__ float K() const { return __uint_as_float(*(const volatile uint32_t *)&s.race_bound); }
+    __device__ __forceinline__ float K() const { return __uint_as_float(*(const volatile uint32_t *)&s.race.bound); }
     // no larger word lets an element of mass e win
     __device__ __forceinline__ static uint32_t word_bound(float e, float K) { return __float2uint_ru(e * K * 4294967296.0f); }
     // by whole warps: the lanes' bounds; gives the smallest of all.  (Never 0: masses relative to a reference far below the maximum can be infinite.)
     __device__ __forceinline__ float tighten(float cap) const {
         const uint32_t least = __reduce_min_sync(0xFFFFFFFFu, __float_as_uint(fminf(fmaxf(cap, 1e-37f), 3.0e38f)));
         const float now = K();
-        if (__uint_as_float(least) < now && (threadIdx.x & 31) == 0) atomicMin(&s.race_bound, least);
+        if (__uint_as_float(least) < now && (threadIdx.x & 31) == 0) atomicMin(&s.race.bound, least);
         return fminf(__uint_as_float(least), now);
     }
     // by whole warps: the lanes' best elements (0: none)
@@ -846,7 +876,7 @@ struct CountedRacer {
         if (!__any_sync(0xFFFFFFFFu, g != 0)) return;
         warp_best(g, zg);
         const int wid = threadIdx.x >> 5;
-        if ((threadIdx.x & 31) == 0 && g > s.race_G[wid]) { s.race_G[wid] = g; s.race_z[wid] = zg; }
+        if ((threadIdx.x & 31) == 0 && g > s.red2[wid]) { s.red2[wid] = g; s.r32b[wid] = __float_as_uint(zg); }
         __syncwarp();
     }
     __device__ __forceinline__ void list(int i, float z_) {
@@ -898,7 +928,7 @@ struct CountedRacer {
         if constexpr (REGS) { p.G = G; p.z = z; return; }
         __syncwarp();
         const bool first = (threadIdx.x & 31) == 0;
-        p.G = first ? s.race_G[threadIdx.x >> 5] : 0ull; p.z = first ? s.race_z[threadIdx.x >> 5] : 0.0f;
+        p.G = first ? s.red2[threadIdx.x >> 5] : 0ull; p.z = first ? __uint_as_float(s.r32b[threadIdx.x >> 5]) : 0.0f;
         __syncwarp();
     }
 };
@@ -1302,15 +1332,16 @@ __device__ __forceinline__ RowOut wide_finish_in(TEAM tm, float top_p, uint64_t 
     return out;
 }
 
+template <bool COUNTED>
 __device__ __noinline__ RowOut wide_finish_call(float top_p, uint64_t seed, uint32_t R, Partial p, WideEnd w, u64 *list, int list_cap, const float *exp1_row,
                                                 int b, RowOut out) {
-    return wide_finish_in(SoloTeam(), top_p, seed, R, p, w, list, list_cap, exp1_row, b, out);
+    return wide_finish_in(SoloTeam<COUNTED>(), top_p, seed, R, p, w, list, list_cap, exp1_row, b, out);
 }
-// (with 64 registers per thread out of line)
+// (with 64 registers per thread out of line; of rows that have been counted)
 template <class TEAM>
 __device__ __forceinline__ RowOut wide_finish(const TEAM &tm, float top_p, uint64_t seed, uint32_t R, const Partial &p, const WideEnd &w, u64 *list, int list_cap,
                                               const float *exp1_row, int b, const RowOut &out) {
-    if constexpr (std::is_same<TEAM, SoloTeam>::value) return wide_finish_call(top_p, seed, R, p, w, list, list_cap, exp1_row, b, out);
+    if constexpr (TEAM::ALONE) return wide_finish_call<true>(top_p, seed, R, p, w, list, list_cap, exp1_row, b, out);
     else return wide_finish_in(tm, top_p, seed, R, p, w, list, list_cap, exp1_row, b, out);
 }
 
@@ -1389,7 +1420,7 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
     // kept elements that are a good part of the row are raced in place: 25 instructions per element of the
     // row against about 40 per kept element through the queues (`ahead_most` is up to twice their number)
     const bool dense = topp && !minp && !want_list && !exp1_row && win.ahead_most > n_fin / 4;
-    if ((no_cut || dense) && threadIdx.x == 32) { s.fa.philox = philox_row(rp.seed, rp.R, s.ga.step); s.race_bound = __float_as_uint(RACE_LUCK); }
+    if ((no_cut || dense) && threadIdx.x == 32) { s.race.philox = philox_row(rp.seed, rp.R, s.ga.step); s.race.bound = __float_as_uint(RACE_LUCK); }
     if (threadIdx.x == 0) {
         FinalArgs &fa = s.fa;
         fa.invT = invT; fa.zmax = zmax; fa.zfloor = zfloor;
@@ -1439,12 +1470,10 @@ constexpr uint32_t CT_LOW = 0xC27Fu;                   // -63.75: this value and
 constexpr uint32_t ROW_NOT_COUNTED = 0x40000000u;      // internal status bit: the table does not hold the row (the same in every CTA)
 static_assert(CT_PER == 16, "a segment is 16 values");
 
-struct CountedSmem { uint32_t *count; u64 *seg_mass; uint32_t *seg_cnt, *odd; };     // odd: their number, whether there are values of 64 or more, codes
-__device__ __forceinline__ CountedSmem counted_smem() {
+__device__ __forceinline__ uint32_t *counted_table() { extern __shared__ __align__(128) unsigned char smem[]; return (uint32_t *)smem; }
+template <class SRC> __device__ __forceinline__ CountedSegs &counted_segs(const SRC &src) {
     extern __shared__ __align__(128) unsigned char smem[];
-    CountedSmem c;
-    c.count = (uint32_t *)smem; c.seg_mass = (u64 *)(smem + CT_SEG_OFF); c.seg_cnt = (uint32_t *)(smem + CT_CNT_OFF); c.odd = (uint32_t *)(smem + CT_ODD_OFF);
-    return c;
+    return *(CountedSegs *)(smem + src.segments());
 }
 __device__ __forceinline__ uint32_t ct_index(uint32_t c) { return (c & 0xFFFu) | ((c >> 3) & 0x1000u); }
 // the j-th value in descending order, and one step up from a value
@@ -1460,47 +1489,38 @@ __device__ __forceinline__ int ct_place(uint32_t c) {
 __device__ __forceinline__ float ct_score(uint32_t c, float invT) { return __fmul_rn(__uint_as_float(c << 16), invT); }
 __device__ __forceinline__ u64 mass_fx(float z, float zmax) { return __float2ull_rn(ex2_ftz(log2_mass(z, zmax)) * FX_SCALE); }
 
-// Where the cut and the list end, the same in every CTA.
-struct CountedCut {
-    uint32_t thr_any, thr_win, thr_sure, thr_top;     // raw, packed twice: values from there on matter, are in the window or kept, are kept, are listed
-    uint32_t key_lo, key_hi;                          // the window's order keys, both inclusive: above it kept
-    uint32_t key_seg;                                 // extras above it are in M and n
-    uint32_t key_top;
-    u64 M; uint32_t n;                                // kept for sure, all but the extras above the window and not above key_seg
-    uint32_t fail;                                    // (0 ahead of the counting pass: any thread may set it from there on)
-};
-__device__ __forceinline__ CountedCut &counted_cut(BlockScratch &s) { return *(CountedCut *)s.cut_words; }
-
 // (by whole blocks; a barrier must follow)
-__device__ __forceinline__ void counted_clear() {
-    const CountedSmem c = counted_smem();
+template <class SRC>
+__device__ __forceinline__ void counted_clear(const SRC &src) {
+    CountedSegs &c = counted_segs(src);
 #pragma unroll
-    for (int i = 0; i < CT_PER / 4; ++i) ((uint4 *)c.count)[i * NT + threadIdx.x] = make_uint4(0, 0, 0, 0);
-    c.seg_mass[threadIdx.x] = 0ull; c.seg_cnt[threadIdx.x] = 0u;
-    if (threadIdx.x < 2) c.odd[threadIdx.x] = 0u;
-    if (threadIdx.x == 0) counted_cut(block_scratch()).fail = 0u;
+    for (int i = 0; i < CT_PER / 4; ++i) ((uint4 *)counted_table())[i * NT + threadIdx.x] = make_uint4(0, 0, 0, 0);
+    c.mass[threadIdx.x] = 0ull; c.cnt[threadIdx.x] = 0u;
+    if (threadIdx.x == 0) { c.n_odd = 0u; c.lost = 0u; c.cut.fail = 0u; }
 }
-__device__ __noinline__ void count_odd_vector(uint4 q) {
-    const CountedSmem c = counted_smem();
+template <class SRC>
+__device__ __noinline__ void count_odd_vector(SRC src, uint4 q) {
+    CountedSegs &c = counted_segs(src);
 #pragma unroll 1
     for (int j = 0; j < 8; ++j) {
         const uint32_t v = __float_as_uint(pick_element<ALBIREO_BF16>(q, j)) >> 16, mag = v & 0x7FFFu;
-        if (mag >= 0x4280u) c.odd[1] = 1u;
-        else if (mag >= 0x3280u) atomicAdd(&c.count[ct_index(v)], 1u);
-        else { const uint32_t at = atomicAdd(&c.odd[0], 1u); if (at < (uint32_t)CT_ODD) c.odd[2 + at] = v; }
+        if (mag >= 0x4280u) c.lost = 1u;
+        else if (mag >= 0x3280u) atomicAdd(&counted_table()[ct_index(v)], 1u);
+        else { const uint32_t at = atomicAdd(&c.n_odd, 1u); if (at < (uint32_t)CT_ODD) c.odd[at] = v; }
     }
 }
 // counts the vector's values; `top` is its largest of each half
-__device__ __forceinline__ void count_vector(uint4 q, __nv_bfloat162 top) {
+template <class SRC>
+__device__ __forceinline__ void count_vector(const SRC &src, uint4 q, __nv_bfloat162 top) {
     typedef __nv_bfloat162 H2;
-    uint32_t *count = counted_smem().count;
+    uint32_t *count = counted_table();
     const uint32_t low2 = CT_LOW | (CT_LOW << 16), high2 = 0x42804280u, tiny2 = 0x32803280u;
     auto h = [](const uint32_t &w) { return *reinterpret_cast<const H2 *>(&w); };
     const H2 least = __hmin2(__hmin2(__habs2(h(q.x)), __habs2(h(q.y))), __hmin2(__habs2(h(q.z)), __habs2(h(q.w))));
     const bool plain = (__hlt2_mask(top, h(high2)) & __hge2_mask(least, h(tiny2))) == 0xFFFFFFFFu;
     auto clamp = [&](uint32_t &w) { const H2 x = __hmax2(h(w), h(low2)); w = *reinterpret_cast<const uint32_t *>(&x); };
     clamp(q.x); clamp(q.y); clamp(q.z); clamp(q.w);
-    if (!plain) { count_odd_vector(q); return; }
+    if (!plain) { count_odd_vector(src, q); return; }
     auto add = [&](uint32_t w) {
         const uint32_t i = ((w & 0x0FFF0FFFu) | ((w >> 3) & 0xF000F000u)) & 0x1FFF1FFFu;
         atomicAdd(&count[i & 0xFFFFu], 1u);
@@ -1537,13 +1557,13 @@ __device__ __noinline__ void counting_pass(SRC src, BlockScratch *sp, float invT
     if constexpr (!RACE) src.vectors([&](const uint4 &q0, const uint4 &q1, int i0, int i1) {
         const __nv_bfloat162 top0 = VecTest<ALBIREO_BF16>::vmax(q0), top1 = VecTest<ALBIREO_BF16>::vmax(q1);
         most = __hmax2(most, __hmax2(top0, top1));
-        if (i0 < end) count_vector(q0, top0);
-        if (i1 >= 0 && i1 < end) count_vector(q1, top1);
+        if (i0 < end) count_vector(src, q0, top0);
+        if (i1 >= 0 && i1 < end) count_vector(src, q1, top1);
     });
     else src.vectors([&](const uint4 &q, int i0) {
         const __nv_bfloat162 top = VecTest<ALBIREO_BF16>::vmax(q);
         most = __hmax2(most, top);
-        if (i0 < end) count_vector(q, top);
+        if (i0 < end) count_vector(src, q, top);
         __syncwarp();
         race_vector<OFF>(rc, q, i0, top, -INFINITY, invT, zref);
     });
@@ -1582,7 +1602,7 @@ __device__ __forceinline__ float race_reference(BlockScratch &s, const uint4 &q,
     const int lane = threadIdx.x & 31;
     const float top = unkey(__reduce_max_sync(0xFFFFFFFFu, lane < NWARPS ? s.r32a[lane] : 0u));
     const bool some = fabsf(top) < 3.0e38f;
-    if (threadIdx.x == 0) { s.fa.philox = philox_row(rp.seed, rp.R, s.ga.step); s.race_bound = some ? __float_as_uint(RACE_LUCK) : NO_BOUND; s.cand_cnt = 0; }
+    if (threadIdx.x == 0) { s.race.philox = philox_row(rp.seed, rp.R, s.ga.step); s.race.bound = some ? __float_as_uint(RACE_LUCK) : NO_BOUND; s.cand_cnt = 0; }
     return some ? top : 0.0f;
 }
 // which wide rows are counted (the temperature's bound keeps the scores of different values apart)
@@ -1606,9 +1626,9 @@ __device__ __noinline__ uint32_t count_finite(SRC src, BlockScratch *sp, float i
 // the table cannot tell (bit 29), or only if the maximum is far above -63.75 (bit 28).  The same in every thread.
 template <class SRC>
 __device__ __forceinline__ uint32_t counted_finite(const SRC &src, BlockScratch &s, float invT, uint32_t killed, uint32_t &flags) {
-    const CountedSmem c = counted_smem();
-    const uint32_t low = c.count[ct_index(CT_LOW)];
-    flags = (c.odd[1] || c.odd[0] > (uint32_t)CT_ODD) ? 0x20000000u : 0u;
+    const CountedSegs &c = counted_segs(src);
+    const uint32_t low = counted_table()[ct_index(CT_LOW)];
+    flags = (c.lost || c.n_odd > (uint32_t)CT_ODD) ? 0x20000000u : 0u;
     const uint32_t rest = (uint32_t)src.elements() - low;
     if (low == killed) return rest;
     const uint32_t n = count_finite(src, &s, invT);
@@ -1630,7 +1650,7 @@ __device__ __noinline__ Partial counted_final_pass(SRC src, BlockScratch *sp) {
     typedef VecTest<ALBIREO_BF16> T;
     extern __shared__ __align__(128) unsigned char smem[];
     BlockScratch &s = block_scratch();
-    const CountedCut &cut = counted_cut(s);
+    const CountedCut &cut = counted_segs(src).cut;
     const WideSmem ws = wide_smem();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint4 *qvec = (uint4 *)(smem + CT_QUEUE_OFF) + wid * RACE_QUEUE;
@@ -1716,7 +1736,7 @@ __device__ __forceinline__ SegmentEnd end_in_segment(const TEAM &tm, int seg, bo
     const float z = ct_score(code, invT);
     uint32_t cnt = 0;
     if (lane < CT_PER && z >= zfloor)
-        for (int r = 0; r < tm.size; ++r) cnt += *tm.at(&counted_smem().count[ct_index(code)], r);
+        for (int r = 0; r < tm.size; ++r) cnt += *tm.at(&counted_table()[ct_index(code)], r);
     u64 mass = (u64)cnt * mass_fx(z, zmax);
 #pragma unroll
     for (int o = 1; o < CT_PER; o <<= 1) {
@@ -1747,18 +1767,17 @@ __device__ __forceinline__ uint32_t ct_key_down_to(int seg, int hi, float invT) 
 template <class SRC>
 __device__ __noinline__ u64 counted_masses(SRC src, BlockScratch *sp, float invT, float zmax, uint32_t kfloor, bool no_cut) {
     BlockScratch &s = block_scratch();
-    const CountedSmem ct = counted_smem();
-    CountedCut &cut = counted_cut(s);
-    const int t = threadIdx.x, n_odd = (int)ct.odd[0];
+    CountedSegs &ct = counted_segs(src);
+    const int t = threadIdx.x, n_odd = (int)ct.n_odd;
     const float zfloor = unkey(kfloor);
     u64 sum = 0;
     // (64 bits as two words, the carry by whoever makes the low one wrap: any number of masses may meet in a segment. A
     // 64-bit add in shared memory is a compare-and-swap loop.)
     auto in_segment = [&](int seg, u64 m) {
-        uint32_t *w = (uint32_t *)&ct.seg_mass[seg];
+        uint32_t *w = (uint32_t *)&ct.mass[seg];
         const uint32_t lo = (uint32_t)m, was = atomicAdd(&w[0], lo), hi = (uint32_t)(m >> 32) + (was + lo < lo);
         if (hi) atomicAdd(&w[1], hi);
-        atomicAdd(&ct.seg_cnt[seg], 1u);
+        atomicAdd(&ct.cnt[seg], 1u);
     };
     src.extras([&](int, float z) {
         const uint32_t k = key_of(z);
@@ -1766,16 +1785,16 @@ __device__ __noinline__ u64 counted_masses(SRC src, BlockScratch *sp, float invT
         const u64 m = mass_fx(z, zmax);
         if (no_cut) { sum += m; return; }
         const uint32_t raw = VecTest<ALBIREO_BF16>::raw_threshold(k, invT) & 0xFFFFu;
-        if (raw == 0xFF80u) cut.fail = 1u; else in_segment(ct_place(raw) / CT_PER, m);
+        if (raw == 0xFF80u) ct.cut.fail = 1u; else in_segment(ct_place(raw) / CT_PER, m);
     });
     for (int j = t; j < n_odd; j += NT) {
-        const float z = ct_score(ct.odd[2 + j], invT);
+        const float z = ct_score(ct.odd[j], invT);
         if (!(z >= zfloor)) continue;
         if (no_cut) sum += mass_fx(z, zmax); else in_segment(4095 / CT_PER, mass_fx(z, zmax));
     }
     __syncthreads();
     const uint32_t first = t < 256 ? 0x4270u - 16u * (uint32_t)t : 0xB280u + 16u * (uint32_t)(t - 256);      // the smallest magnitude
-    const uint4 *words = (const uint4 *)&ct.count[ct_index(first)];
+    const uint4 *words = (const uint4 *)&counted_table()[ct_index(first)];
     u64 mass = 0;
     uint32_t cnt = 0;
 #pragma unroll
@@ -1790,25 +1809,25 @@ __device__ __noinline__ u64 counted_masses(SRC src, BlockScratch *sp, float invT
         }
     }
     if (no_cut) return sum + mass;
-    ct.seg_mass[t] += mass;
-    ct.seg_cnt[t] += cnt;
+    ct.mass[t] += mass;
+    ct.cnt[t] += cnt;
     return 0;
 }
 // From the segments of all CTAs to the cut (see CountedCut), the same in every CTA; s.bcast[2] and [3]: the mass above the floor and the one to
 // be reached.  False: the table does not tell.
-template <class TEAM>
-__device__ __noinline__ bool counted_locate(BlockScratch *sp, TEAM tm, float invT, float zmax, uint32_t kfloor, bool minp, float top_p, uint32_t n_fin, int list_cap) {
+template <class SRC, class TEAM>
+__device__ __noinline__ bool counted_locate(BlockScratch *sp, SRC src, TEAM tm, float invT, float zmax, uint32_t kfloor, bool minp, float top_p, uint32_t n_fin, int list_cap) {
     typedef VecTest<ALBIREO_BF16> T;
     BlockScratch &s = block_scratch();
-    const CountedSmem ct = counted_smem();
-    CountedCut &cut = counted_cut(s);
+    CountedSegs &ct = counted_segs(src);
+    CountedCut &cut = ct.cut;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, t = threadIdx.x;
     const bool topp = top_p < 1.0f, listed = s.ga.num_top > 0;
     const float zfloor = unkey(kfloor);
     u64 mass = 0;
     uint32_t cnt = 0;
 #pragma unroll 4
-    for (int r = 0; r < tm.size; ++r) { mass += *tm.at(&ct.seg_mass[t], r); cnt += *tm.at(&ct.seg_cnt[t], r); }
+    for (int r = 0; r < tm.size; ++r) { mass += *tm.at(&ct.mass[t], r); cnt += *tm.at(&ct.cnt[t], r); }
     u64 run = mass;
     uint32_t crun = cnt;
 #pragma unroll
@@ -1871,7 +1890,7 @@ __device__ __noinline__ bool counted_locate(BlockScratch *sp, TEAM tm, float inv
     } else if (t == 64) {
         s.fa.invT = invT; s.fa.zmax = zmax; s.fa.list_cap = list_cap; s.fa.exp1_row = nullptr;
         s.fa.list = listed ? wide_smem().list : wide_smem().top;
-        s.race_bound = __float_as_uint(RACE_LUCK / ((float)target * (1.0f / FX_SCALE)));
+        s.race.bound = __float_as_uint(RACE_LUCK / ((float)target * (1.0f / FX_SCALE)));
         s.bcast[2] = S; s.bcast[3] = target;
     }
     tm.sync();                                           // (everybody has read the tables; lists and queues lie over them)
@@ -1897,15 +1916,15 @@ __device__ __noinline__ RowOut counted_row(BlockScratch *sp, SRC src, TEAM tm, c
     const bool topp = rp.top_p < 1.0f, minp = rp.min_p > 0.0f, listed = s.ga.num_top > 0, no_cut = !topp && !minp && !listed;
     const uint32_t kfloor = minp ? minp_key(zmax, rp.ln_min_p) : KEY_MIN_FINITE;
     const float zlow = ct_score(CT_LOW, invT);
-    const bool raced = std::is_same<TEAM, SoloTeam>::value && no_cut;
+    const bool raced = TEAM::ALONE && no_cut;
     // (values that are counted together must weigh nothing and be below the floor; a race that is listed as a whole)
     if ((raced && s.cand_cnt > (uint32_t)RACE_LIST) || (flags & 0x20000000u) || kfloor > kmax || ((flags & 0x10000000u) && (!(zmax - zlow > 29.0f) || (minp && unkey(kfloor) <= zlow)))) {
         out.status |= ROW_NOT_COUNTED;
         return out;
     }
-    CountedCut &cut = counted_cut(s);
+    const CountedCut &cut = counted_segs(src).cut;
     if (t == 0) {
-        counted_smem().count[ct_index(CT_LOW)] = 0;
+        counted_table()[ct_index(CT_LOW)] = 0;
         tm.x->far_cand = 0; tm.x->far_list = 0;
     }
     Partial p;
@@ -1924,11 +1943,11 @@ __device__ __noinline__ RowOut counted_row(BlockScratch *sp, SRC src, TEAM tm, c
             p.G = CountedRacer<LISTED>::code_of_score(__fsub_rn(p.z, zmax) + race_nle(rp.seed, rp.R, s.ga.step, nullptr, i), i);
         }
     } else {
-        if (t < tm.size) *tm.at(&tm.x->fail[tm.rank], t) = cut.fail;       // (a barrier has ended the extras)
-        if (t == 0) { s.found_digit = 0xFFFFFFFFu; s.found_cnt = 0xFFFFFFFFu; s.list_cnt = 0; s.cand_cnt = 0; s.fa.philox = philox_row(rp.seed, rp.R, s.ga.step); }
+        if (t < tm.size) *tm.at(&tm.x->ncand[tm.rank], t) = cut.fail;       // (a barrier has ended the extras)
+        if (t == 0) { s.found_digit = 0xFFFFFFFFu; s.found_cnt = 0xFFFFFFFFu; s.list_cnt = 0; s.cand_cnt = 0; s.race.philox = philox_row(rp.seed, rp.R, s.ga.step); }
         tm.sync();
-        if (__reduce_or_sync(0xFFFFFFFFu, lane < tm.size ? tm.x->fail[lane] : 0u) ||
-            !counted_locate(sp, tm, invT, zmax, kfloor, minp, rp.top_p, n_fin, list_cap)) { out.status |= ROW_NOT_COUNTED; return out; }
+        if (__reduce_or_sync(0xFFFFFFFFu, lane < tm.size ? tm.x->ncand[lane] : 0u) ||
+            !counted_locate(sp, src, tm, invT, zmax, kfloor, minp, rp.top_p, n_fin, list_cap)) { out.status |= ROW_NOT_COUNTED; return out; }
         w.S = w.S_all = s.bcast[2];
         w.race_from = 0.001f - logf(RACE_LUCK / ((float)s.bcast[3] * (1.0f / FX_SCALE)));
         switch (src.first_id() & 3) {
