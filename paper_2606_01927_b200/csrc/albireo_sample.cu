@@ -189,6 +189,7 @@ struct BlockScratch {
     uint32_t maint_at;           // tile index before which every warp meets (0xFFFFFFFF: none)
     uint32_t issued;             // tiles whose copy has been issued so far
     const char *seg_base[ALBIREO_MAX_SEGMENTS];   // where this row's pieces start (rows in pieces only)
+    int32_t seg_off;             // clusters: where a counted slice's CountedSegs lie (wide_path.cuh)
     uint32_t nfin_cap;           // general path: min(#finite scores, ALBIREO_MAX_NUM_TOP + 1), parked here until the list is written
     FinalArgs fa;
     GenArgs ga;                  // the general path's copy of the launch arguments it uses

@@ -153,6 +153,11 @@ __device__ __noinline__ int slice_history(BlockScratch *sp, RowCtx c, const int3
     return (int)U;
 }
 
+template <int DT, class SRC, class TEAM>
+__device__ __noinline__ RowOut team_wide_row(SRC src, TEAM tm, RowParams rp, float invT, uint32_t kmax, uint32_t n_fin, int b, uint32_t status) {
+    return wide_row<DT>(block_scratch(), src, tm, rp, invT, kmax, n_fin, b, status);
+}
+
 // COUNTED: with the code for rows counted by value (see counted_row); the launches whose slices are too small for that do
 // without it (counted_slices): beside it their top-p rows took 1.4 us longer, 18.7 against 17.2 for 8 rows of 32000.
 template <int DT, bool COUNTED>
@@ -179,6 +184,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
         mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        if constexpr (COUNTED) s.seg_off = tab_off;
         s.cand_cnt = 0; s.runmax = 0; s.race.bound = NO_BOUND; s.mm_max = 0; s.mm_min = 0xFFFFFFFFu; s.list_cnt = 0;
         tm.x->far_cand = 0; tm.x->far_list = 0;
     }
@@ -238,7 +244,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     int nx = 0;
     const int n_slice_ids = nv * E::PER_VEC;
     SmemSlice<DT> src;
-    src.vec_off = SLICE_OFF; src.nvec = nv; src.id0 = id0; src.seg_off = tab_off;
+    src.vec_off = SLICE_OFF; src.nvec = nv; src.id0 = id0;
     // (a launch without histories has no tables: only the row's unaligned ends are listed)
     src.xz_off = tab_off + slice_tables(COUNTED, tables, n_slice_ids);
     int *xid = (int *)(smem + src.xz_off) + (a.list_words >> 1);
@@ -392,9 +398,13 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
         }
         if (wide) {
             const uint32_t status = out.status;
-            out.status |= ROW_NOT_COUNTED;
-            if constexpr (COUNTED) { if (counted) out = counted_row(&s, src, tm, rp, c.invT, kmax, n_fin, bad, b, status); }
-            if (out.status & ROW_NOT_COUNTED) out = wide_row<DT>(s, src, tm, rp, c.invT, kmax, n_fin, b, status);
+            if constexpr (COUNTED) out.status |= ROW_NOT_COUNTED;
+            if constexpr (COUNTED) {
+                // (out of line beside the code for counted rows, which else leaves the others spilling: 30 rows of 152064 with a top-k 10.5 us instead
+                // of 10.2.  Top-p rows that are not counted lose by it, 17.5 to 18.0 us for 8 rows of 32000: so not in the other kernel.)
+                if (counted) out = counted_row(&s, src, tm, rp, c.invT, kmax, n_fin, bad, b, status);
+                if (out.status & ROW_NOT_COUNTED) out = team_wide_row<DT>(src, tm, rp, c.invT, kmax, n_fin, b, status);
+            } else out = wide_row<DT>(s, src, tm, rp, c.invT, kmax, n_fin, b, status);
             done = !(out.status & ROW_NOT_DONE);
             if (!done) out.status = status;
         }

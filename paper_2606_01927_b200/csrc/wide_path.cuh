@@ -290,13 +290,12 @@ struct SmemSlice {
     typedef Elem<DT> E;
     static constexpr bool SPARE_REGISTERS = true;       // 128 per thread
     int vec_off, nvec, id0;       // where the slice and the list lie in the dynamic shared memory
-    int seg_off;                  // (counted rows: see CountedSegs)
     const int *xid;               // (in the workspace where there are too many for both lists on chip)
     int xz_off, nx;
     __device__ __forceinline__ int first_id() const { return id0; }
     __device__ __forceinline__ int end_id() const { return id0 + nvec * E::PER_VEC; }
     __device__ __forceinline__ int elements() const { return nvec * E::PER_VEC; }
-    __device__ __forceinline__ int segments() const { return seg_off; }
+    __device__ __forceinline__ int segments() const { return block_scratch().seg_off; }      // (in a register it was spilled)
     template <class F> __device__ __forceinline__ void vectors(F &&f) const {
         extern __shared__ __align__(128) unsigned char smem[];
         const uint4 *vec = (const uint4 *)(smem + vec_off);
@@ -1644,7 +1643,20 @@ __device__ __forceinline__ uint32_t edge_mask(uint32_t w, uint32_t thr_win, uint
 }
 // Mass, number and lists of the extras, the race of all that is kept for sure, the window's elements to their list.
 // Vectors with nothing that matters are passed over; the others are worked on by full warps: where only few of a
-// warp's have something they wait in a queue.
+// warp's have something they wait in a queue.  (One vector of a thread at a time: with two, 52 to 160 bytes were spilled in this loop by the
+// kernel with 64 registers.)
+// (out of line: few vectors have any)
+__device__ __noinline__ void append_elements(uint4 q, int i0, uint32_t bits, float invT, bool listed) {
+    BlockScratch &s = block_scratch();
+    while (bits) {
+        const int x = __ffs(bits) - 1;
+        bits &= bits - 1u;
+        const float z = __fmul_rn(pick_element<ALBIREO_BF16>(q, x), invT);
+        if (listed) list_append(wide_smem().top, W_LIST, &s.cand_cnt, z, i0 + x);
+        else list_append(s.fa.list, s.fa.list_cap, &s.list_cnt, z, i0 + x);
+    }
+    __syncwarp();
+}
 template <int OFF, class SRC>
 __device__ __noinline__ Partial counted_final_pass(SRC src, BlockScratch *sp) {
     typedef VecTest<ALBIREO_BF16> T;
@@ -1652,60 +1664,47 @@ __device__ __noinline__ Partial counted_final_pass(SRC src, BlockScratch *sp) {
     BlockScratch &s = block_scratch();
     const CountedCut &cut = counted_segs(src).cut;
     const WideSmem ws = wide_smem();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint4 *qvec = (uint4 *)(smem + CT_QUEUE_OFF) + wid * RACE_QUEUE;
-    int *qid = (int *)((uint4 *)(smem + CT_QUEUE_OFF) + NWARPS * RACE_QUEUE) + wid * RACE_QUEUE;
+    // (worked out anew where they are used: held across the loop they were spilled)
+    auto lane_now = [] { int l; asm volatile("mov.u32 %0, %%laneid;" : "=r"(l)); return l; };
+    auto warp_now = [] { int t; asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t)); return t >> 5; };
+    auto qvec = [&](int at) -> uint4 & { return ((uint4 *)(smem + CT_QUEUE_OFF))[warp_now() * RACE_QUEUE + at]; };
+    auto qid = [&](int at) -> int & { return ((int *)(smem + CT_QUEUE_OFF + NWARPS * RACE_QUEUE * 16))[warp_now() * RACE_QUEUE + at]; };
     int qn = 0;                                        // the same in every lane
     const uint32_t thr_any = cut.thr_any;
     CountedRacer<SRC::SPARE_REGISTERS ? IN_REGS : IN_SHARED> rc(s);
-    src.vectors([&](const uint4 &q0, const uint4 &q1, int i01, int i1) -> bool {
-        uint32_t m0 = 0, m1 = 0;
-        bool in0 = false, in1 = false;
-        if (i01 >= 0) {
-            in0 = T::may_pass(q0, thr_any, 1.0f); in1 = i1 >= 0 && T::may_pass(q1, thr_any, 1.0f);
-            m0 = __ballot_sync(0xFFFFFFFFu, in0); m1 = __ballot_sync(0xFFFFFFFFu, in1);
-            if ((m0 | m1) == 0) return true;
-        } else if (qn == 0) return false;
-#pragma unroll 1
-        do {
-        uint4 q = T::fill();
+    src.vectors([&](const uint4 &q0, int i01) -> bool {
+        uint4 q = q0;
         int i0 = i01;
         bool waiting = i01 < 0;
         if (!waiting) {
-            const uint32_t m = m0 ? m0 : m1;
-            const bool in = m0 ? in0 : in1;
-            q = m0 ? q0 : q1;
-            if (!m0) { m1 = 0; i0 = i1; }
-            m0 = 0;
+            const bool in = T::may_pass(q, thr_any, 1.0f);
+            const uint32_t m = __ballot_sync(0xFFFFFFFFu, in);
+            if (m == 0) return true;
             if (__popc(m) < RACE_DIRECT) {
-                if (in) { const int at = qn + __popc(m & ((1u << lane) - 1u)); qvec[at] = q; qid[at] = i0; }
+                if (in) { const int at = qn + __popc(m & ((1u << lane_now()) - 1u)); qvec(at) = q; qid(at) = i0; }
                 qn += __popc(m);
-                if (qn < 32) continue;
+                if (qn < 32) return true;
                 waiting = true;
             }
-        }
+        } else if (qn == 0) return false;
         if (waiting) {
             const int cnt = qn < 32 ? qn : 32;
             qn -= cnt;
             __syncwarp();
             q = T::fill();
             i0 = 0;
-            if (lane < cnt) { q = qvec[qn + lane]; i0 = qid[qn + lane]; }
+            const int lane = lane_now();
+            if (lane < cnt) { q = qvec(qn + lane); i0 = qid(qn + lane); }
             __syncwarp();
         }
         const volatile CountedCut &c = cut;
         const float invT = *(const volatile float *)&s.fa.invT;
-        auto append = [&](u64 *list, int cap, uint32_t *cnt, uint32_t bits) {
-            while (bits) { const int x = __ffs(bits) - 1; bits &= bits - 1u; list_append(list, cap, cnt, __fmul_rn(pick_element<ALBIREO_BF16>(q, x), invT), i0 + x); }
-            __syncwarp();
-        };
         const uint32_t thr_sure = c.thr_sure, thr_win = c.thr_win;
         const uint4 at_edge = make_uint4(edge_mask(q.x, thr_win, thr_sure), edge_mask(q.y, thr_win, thr_sure), edge_mask(q.z, thr_win, thr_sure), edge_mask(q.w, thr_win, thr_sure));
-        if (s.ga.num_top > 0) append(ws.top, W_LIST, &s.cand_cnt, T::elem_bits(q, c.thr_top, invT));
+        if (s.ga.num_top > 0) append_elements(q, i0, T::elem_bits(q, c.thr_top, invT), invT, true);
         if (__any_sync(0xFFFFFFFFu, (at_edge.x | at_edge.y | at_edge.z | at_edge.w) != 0u))
-            append(s.fa.list, s.fa.list_cap, &s.list_cnt, T::elem_bits(q, thr_win, invT) & ~T::elem_bits(q, thr_sure, invT));
+            append_elements(q, i0, T::elem_bits(q, thr_win, invT) & ~T::elem_bits(q, thr_sure, invT), invT, false);
         race_vector<OFF>(rc, q, i0, T::vmax(q), __uint_as_float(thr_sure << 16), invT, *(const volatile float *)&s.fa.zmax);
-        } while (m0 | m1);
         return true;
     });
     Partial p;
