@@ -2686,7 +2686,7 @@ constexpr long COUNTED_SLICE = 16384;
 // than that a batch took up to twice as long (8 top-p rows of 152064 35.4 us by 16 CTAs each, 21.1 by 8).  (Two CTAs per SM, with half the registers,
 // were 10 % slower on the rows without a top-k and the same on the others.)  Of the sizes that fit, the largest whose slices are
 // still at least 8 KB (one vector per thread): below that the exchange costs more than the slice.
-bool pick_team(LaunchShape &ls, int B, int V, int dtype, bool with_history, const DeviceShape &d) {
+bool pick_team(LaunchShape &ls, int B, int V, int dtype, bool with_history, bool may_count, const DeviceShape &d) {
     const int esize = dtype == ALBIREO_F32 ? 4 : 2;
     const long row_bytes = (long)(V / (16 / esize)) * 16;
     for (int team = MAX_TEAM, i = 4; team >= 2; team >>= 1, --i) {
@@ -2695,7 +2695,7 @@ bool pick_team(LaunchShape &ls, int B, int V, int dtype, bool with_history, cons
         const long slice = ((per > SLICE_MIN ? per : (long)SLICE_MIN) + 127) & ~127L;
         const long nids = per / esize;
         // (with the table of values, where there is room for it)
-        for (int counted = dtype == ALBIREO_BF16 && nids >= COUNTED_SLICE; counted >= 0; --counted) {
+        for (int counted = may_count && dtype == ALBIREO_BF16 && nids >= COUNTED_SLICE; counted >= 0; --counted) {
             const long fixed = slice_off(counted) + slice + 16 + slice_tables(counted, with_history, (int)nids);
             long list = 2L * X_ENDS;
             if (with_history) {
@@ -2720,9 +2720,15 @@ bool extras_asked(const SampleArgs &a) {
     return (a.flags & (ALBIREO_FLAG_LOGPROB_FULL_VOCAB | ALBIREO_FLAG_TOPK_KEEP_TIES | ALBIREO_FLAG_FORCE_GENERAL)) || a.dbg_topk_ids || a.out_num_topk || a.exp1;
 }
 
+// Whether a row of the call may be counted by value in a cluster: one with a top-p cut or a list, and no min-p (see candidate_eligible, counted_eligible).
+// The others' launches do without the code for it (64 rows of 152064 without a cut 22.5 -> 22.0 us).
+bool may_count_rows(const SampleArgs &a) { return (a.top_p || a.num_top > 0) && !a.exp1; }
+
 // false: the vocabulary is too large for the on-chip tables
-bool pick_shape(LaunchShape &ls, int B, int V, int dtype, bool with_history, bool force_general, const DeviceShape &d) {
-    if (!force_general && pick_team(ls, B, V, dtype, with_history, d)) return true;
+bool pick_shape(LaunchShape &ls, int V, int dtype, const SampleArgs &a, const DeviceShape &d) {
+    const int B = a.B;
+    const bool with_history = a.hist_ids != nullptr;
+    if (!(a.flags & ALBIREO_FLAG_FORCE_GENERAL) && pick_team(ls, B, V, dtype, with_history, may_count_rows(a), d)) return true;
     ls.team = 1; ls.slice_bytes = 0; ls.list_words = 0; ls.counted = false;
     ls.nstages = ring_stages_for(V, with_history, B <= d.num_sms);
     ls.smem = smem_bytes_for(V, with_history, ls.nstages);
@@ -2931,7 +2937,7 @@ extern "C" int albireo_sample(albireo_sampler_t *h, const void *logits, int32_t 
     if (cudaGetDevice(&cur) != cudaSuccess || cur != h->device) { cudaGetLastError(); set_err(h, "the handle's device is not current%s", ""); return ALBIREO_EINVAL; }
 
     LaunchShape ls;
-    if (!pick_shape(ls, B, V, dtype, history_ids != nullptr, (a.flags & ALBIREO_FLAG_FORCE_GENERAL) != 0, h->dev)) { set_err(h, "vocabulary too large for the on-chip tables%s", ""); return ALBIREO_EUNSUPPORTED; }
+    if (!pick_shape(ls, V, dtype, a, h->dev)) { set_err(h, "vocabulary too large for the on-chip tables%s", ""); return ALBIREO_EUNSUPPORTED; }
     cudaStream_t st = (cudaStream_t)stream;
     const cudaError_t e = launch_sample_kernel(dtype, B, ls, st, a);
     if (e != cudaSuccess) { cudaGetLastError(); set_err(h, "kernel launch failed: %s", cudaGetErrorString(e)); return ALBIREO_ECUDA; }
@@ -3168,7 +3174,7 @@ extern "C" int albireo_sample_fixed_scratch(const void *logits, int32_t B, int32
     a.ws_counts_cap = ALBIREO_FIXED_MAX_HISTORY;
 
     LaunchShape ls;
-    if (!pick_shape(ls, B, V, dtype, history_ids != nullptr, (a.flags & ALBIREO_FLAG_FORCE_GENERAL) != 0, d->shape)) return fixed_fail(ALBIREO_EUNSUPPORTED, "vocabulary too large for the on-chip tables%s", "");
+    if (!pick_shape(ls, V, dtype, a, d->shape)) return fixed_fail(ALBIREO_EUNSUPPORTED, "vocabulary too large for the on-chip tables%s", "");
     cudaStream_t st = (cudaStream_t)stream;
     const cudaError_t e = launch_sample_kernel(dtype, B, ls, st, a);
     if (e != cudaSuccess) { cudaGetLastError(); return fixed_fail(ALBIREO_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e)); }

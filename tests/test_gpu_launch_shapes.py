@@ -86,3 +86,13 @@ def test_longest_slices(binding, sampler, dtype, history, B, V):
     t = binding.workload_tensors(w, sampler.device)
     rep = compare(w, to_host(sampler.albireo_sample(t.pop("logits"), **t, want_counts=True, want_status=True)), ref)
     assert rep.ok() and len(rep.excused) <= 1, (rep.summary(), rep.failures[:3], rep.excused[:3])
+
+
+@pytest.mark.parametrize("par,counted", [(("top_p",), True), (("num_top",), True), (("top_k", "top_p"), True), ((), False), (("top_k",), False), (("min_p",), False)])
+def test_table_of_values_only_where_a_row_may_need_it(binding, sampler, par, counted):
+    B, V = 64, 152064
+    dev = sampler.device
+    values = dict(top_p=torch.full((B,), 0.9, device=dev), top_k=torch.full((B,), 40, dtype=torch.int32, device=dev), min_p=torch.full((B,), 0.1, device=dev), num_top=5)
+    logits, rest = batch(sampler, B, V, W.BF16, False, **{k: values[k] for k in par})
+    ctas, name = launched(sampler, logits, **rest)
+    assert ctas == 2 * B and ("ILi1ELb1E" in name) == counted, name
