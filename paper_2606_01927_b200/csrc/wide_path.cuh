@@ -390,7 +390,10 @@ struct CountedCut {
 struct CountedSegs {
     u64 mass[NT];                     // by segments of 16 values; with no cut the list of the race (RACE_LIST) lies here
     uint32_t cnt[NT];
-    uint32_t n_odd, lost, odd[CT_ODD];        // values nearer to zero than the table's, and whether there are values above it
+    uint32_t zeros[2];                // +0 and -0
+    uint32_t n_odd, odd[CT_ODD];      // other values that have no place in the table
+    uint32_t lost;                    // there are more of them than that
+    uint32_t high;                    // some of them are above the table's
     CountedCut cut;
 };
 // The slices of a cluster begin behind the team's words; by one CTA the row's own block and the ring of its passes do.  (At 128 bytes: 30 rows
@@ -1459,15 +1462,15 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
 // mass and, from prefix sums, the very value at which a cut or a list ends; with no cut the race is in the same
 // pass.  (Increments of one warp meet in 3.5 bank cycles on average, which bounds the pass: 3620 cycles per 32768 elements
 // in one SM against 6940 for the pass of masses and 690 for the maximum.)
-// What has no place in the table: values of 64 and more, and more than CT_ODD values nearer to zero than 2^-26 (the
-// row is then done as rows of other types are); all from -63.75 down are counted together, and weigh nothing unless the
-// maximum is as low.  The scores of the extras (penalised tokens, unaligned ends) lie between those of the values:
+// What has no place in the table: zeros, which have counts of their own; values of 64 and more, or nearer to zero than 2^-26, which are
+// listed, up to CT_ODD of them (a row with more is done as rows of other types are); all from -63.75 down are counted together, and
+// weigh nothing unless the maximum is as low.  The scores of the extras (penalised tokens, unaligned ends) lie between those of the values:
 // they are added to the segment of 16 values that they belong to, and stay open in the segment of the cut.
 
 constexpr int CT_PER = CT_BINS / NT;                   // values per thread: a segment
 constexpr uint32_t CT_LOW = 0xC27Fu;                   // -63.75: this value and everything below
 constexpr uint32_t ROW_NOT_COUNTED = 0x40000000u;      // internal status bit: the table does not hold the row (the same in every CTA)
-static_assert(CT_PER == 16, "a segment is 16 values");
+static_assert(CT_PER == 16 && CT_ODD + 2 <= NT, "a segment is 16 values; a thread to each value without a place");
 
 __device__ __forceinline__ uint32_t *counted_table() { extern __shared__ __align__(128) unsigned char smem[]; return (uint32_t *)smem; }
 template <class SRC> __device__ __forceinline__ CountedSegs &counted_segs(const SRC &src) {
@@ -1495,17 +1498,26 @@ __device__ __forceinline__ void counted_clear(const SRC &src) {
 #pragma unroll
     for (int i = 0; i < CT_PER / 4; ++i) ((uint4 *)counted_table())[i * NT + threadIdx.x] = make_uint4(0, 0, 0, 0);
     c.mass[threadIdx.x] = 0ull; c.cnt[threadIdx.x] = 0u;
-    if (threadIdx.x == 0) { c.n_odd = 0u; c.lost = 0u; c.cut.fail = 0u; }
+    if (threadIdx.x == 0) { c.zeros[0] = c.zeros[1] = 0u; c.n_odd = 0u; c.lost = 0u; c.high = 0u; c.cut.fail = 0u; }
 }
 template <class SRC>
 __device__ __noinline__ void count_odd_vector(SRC src, uint4 q) {
     CountedSegs &c = counted_segs(src);
+    if (*(volatile uint32_t *)&c.lost) {               // (then only the values at CT_LOW are still wanted)
+        const uint32_t low = VecTest<ALBIREO_BF16>::count_not_finite(q, (CT_LOW - 1u) * 0x10001u, 1.0f);
+        if (low) atomicAdd(&counted_table()[ct_index(CT_LOW)], low);
+        return;
+    }
 #pragma unroll 1
     for (int j = 0; j < 8; ++j) {
         const uint32_t v = __float_as_uint(pick_element<ALBIREO_BF16>(q, j)) >> 16, mag = v & 0x7FFFu;
-        if (mag >= 0x4280u) c.lost = 1u;
-        else if (mag >= 0x3280u) atomicAdd(&counted_table()[ct_index(v)], 1u);
-        else { const uint32_t at = atomicAdd(&c.n_odd, 1u); if (at < (uint32_t)CT_ODD) c.odd[at] = v; }
+        if (mag == 0u) atomicAdd(&c.zeros[v >> 15], 1u);
+        else if (mag >= 0x3280u && mag < 0x4280u) atomicAdd(&counted_table()[ct_index(v)], 1u);
+        else {
+            const uint32_t at = atomicAdd(&c.n_odd, 1u);
+            if (at < (uint32_t)CT_ODD) c.odd[at] = v; else c.lost = 1u;
+            if (mag >= 0x4280u) { c.high = 1u; if (mag >= 0x7F80u) c.lost = 1u; }
+        }
     }
 }
 // counts the vector's values; `top` is its largest of each half
@@ -1627,7 +1639,7 @@ template <class SRC>
 __device__ __forceinline__ uint32_t counted_finite(const SRC &src, BlockScratch &s, float invT, uint32_t killed, uint32_t &flags) {
     const CountedSegs &c = counted_segs(src);
     const uint32_t low = counted_table()[ct_index(CT_LOW)];
-    flags = (c.lost || c.n_odd > (uint32_t)CT_ODD) ? 0x20000000u : 0u;
+    flags = c.lost ? 0x20000000u : 0u;
     const uint32_t rest = (uint32_t)src.elements() - low;
     if (low == killed) return rest;
     const uint32_t n = count_finite(src, &s, invT);
@@ -1772,11 +1784,11 @@ __device__ __noinline__ u64 counted_masses(SRC src, BlockScratch *sp, float invT
     u64 sum = 0;
     // (64 bits as two words, the carry by whoever makes the low one wrap: any number of masses may meet in a segment. A
     // 64-bit add in shared memory is a compare-and-swap loop.)
-    auto in_segment = [&](int seg, u64 m) {
+    auto in_segment = [&](int seg, u64 m, uint32_t n = 1u) {
         uint32_t *w = (uint32_t *)&ct.mass[seg];
         const uint32_t lo = (uint32_t)m, was = atomicAdd(&w[0], lo), hi = (uint32_t)(m >> 32) + (was + lo < lo);
         if (hi) atomicAdd(&w[1], hi);
-        atomicAdd(&ct.cnt[seg], 1u);
+        atomicAdd(&ct.cnt[seg], n);
     };
     src.extras([&](int, float z) {
         const uint32_t k = key_of(z);
@@ -1786,10 +1798,13 @@ __device__ __noinline__ u64 counted_masses(SRC src, BlockScratch *sp, float invT
         const uint32_t raw = VecTest<ALBIREO_BF16>::raw_threshold(k, invT) & 0xFFFFu;
         if (raw == 0xFF80u) ct.cut.fail = 1u; else in_segment(ct_place(raw) / CT_PER, m);
     });
-    for (int j = t; j < n_odd; j += NT) {
-        const float z = ct_score(ct.odd[j], invT);
-        if (!(z >= zfloor)) continue;
-        if (no_cut) sum += mass_fx(z, zmax); else in_segment(4095 / CT_PER, mass_fx(z, zmax));
+    if (t < n_odd || t >= NT - 2) {
+        const uint32_t code = t < n_odd ? ct.odd[t] : (uint32_t)(t - (NT - 2)) << 15, n = t < n_odd ? 1u : ct.zeros[t - (NT - 2)];
+        const float z = ct_score(code, invT);
+        if (n != 0u && z >= zfloor) {
+            const u64 m = (u64)n * mass_fx(z, zmax);
+            if (no_cut) sum += m; else in_segment(ct_place(code) / CT_PER, m, n);
+        }
     }
     __syncthreads();
     const uint32_t first = t < 256 ? 0x4270u - 16u * (uint32_t)t : 0xB280u + 16u * (uint32_t)(t - 256);      // the smallest magnitude
@@ -1815,7 +1830,7 @@ __device__ __noinline__ u64 counted_masses(SRC src, BlockScratch *sp, float invT
 // From the segments of all CTAs to the cut (see CountedCut), the same in every CTA; s.bcast[2] and [3]: the mass above the floor and the one to
 // be reached.  False: the table does not tell.
 template <class SRC, class TEAM>
-__device__ __noinline__ bool counted_locate(BlockScratch *sp, SRC src, TEAM tm, float invT, float zmax, uint32_t kfloor, bool minp, float top_p, uint32_t n_fin, int list_cap) {
+__device__ __noinline__ bool counted_locate(BlockScratch *sp, SRC src, TEAM tm, float invT, float zmax, uint32_t kfloor, bool minp, float top_p, uint32_t n_fin, int list_cap, bool high) {
     typedef VecTest<ALBIREO_BF16> T;
     BlockScratch &s = block_scratch();
     CountedSegs &ct = counted_segs(src);
@@ -1858,13 +1873,16 @@ __device__ __noinline__ bool counted_locate(BlockScratch *sp, SRC src, TEAM tm, 
             const int seg = (int)s.found_digit;
             if (seg < 0) c.fail = 1u;
             else {
-                const SegmentEnd e = end_in_segment(tm, seg, true, target - s.found_above, s.bcast[0], s.r32b[1], invT, zmax, zfloor);
+                SegmentEnd e = end_in_segment(tm, seg, true, target - s.found_above, s.bcast[0], s.r32b[1], invT, zmax, zfloor);
+                // (values above the table's are in its first segment: where the cut is there too, the window begins with them)
+                const bool from_top = seg == 0 && high;
+                if (from_top) { e.lo = 0; e.mass_ahead = 0; e.cnt_ahead = 0; }
                 const uint32_t above = ct_code(seg * CT_PER + e.lo);
                 c.M = s.found_above + e.mass_ahead; c.n = s.r32b[0] + e.cnt_ahead;
-                c.key_hi = key_of(ct_score(above, invT));
+                c.key_hi = from_top ? 0xFFFFFFFFu : key_of(ct_score(above, invT));
                 c.key_lo = max(ct_key_down_to(seg, e.hi, invT), kfloor);
                 c.key_seg = seg == 0 ? 0xFFFFFFFFu : key_of(ct_score(ct_code(seg * CT_PER), invT));
-                c.thr_sure = ct_above(above) * 0x10001u;
+                c.thr_sure = (from_top ? 0x7F80u : ct_above(above)) * 0x10001u;
                 c.thr_win = e.hi < CT_PER ? ct_code(seg * CT_PER + e.hi) * 0x10001u : T::raw_threshold(c.key_lo, invT);
                 if (e.cnt_most - e.cnt_ahead > (uint32_t)list_cap) c.fail = 1u;
             }
@@ -1942,11 +1960,11 @@ __device__ __noinline__ RowOut counted_row(BlockScratch *sp, SRC src, TEAM tm, c
             p.G = CountedRacer<LISTED>::code_of_score(__fsub_rn(p.z, zmax) + race_nle(rp.seed, rp.R, s.ga.step, nullptr, i), i);
         }
     } else {
-        if (t < tm.size) *tm.at(&tm.x->ncand[tm.rank], t) = cut.fail;       // (a barrier has ended the extras)
+        if (t < tm.size) *tm.at(&tm.x->ncand[tm.rank], t) = cut.fail | (counted_segs(src).high ? 2u : 0u);       // (a barrier has ended the extras)
         if (t == 0) { s.found_digit = 0xFFFFFFFFu; s.found_cnt = 0xFFFFFFFFu; s.list_cnt = 0; s.cand_cnt = 0; s.race.philox = philox_row(rp.seed, rp.R, s.ga.step); }
         tm.sync();
-        if (__reduce_or_sync(0xFFFFFFFFu, lane < tm.size ? tm.x->ncand[lane] : 0u) ||
-            !counted_locate(sp, src, tm, invT, zmax, kfloor, minp, rp.top_p, n_fin, list_cap)) { out.status |= ROW_NOT_COUNTED; return out; }
+        const uint32_t told = __reduce_or_sync(0xFFFFFFFFu, lane < tm.size ? tm.x->ncand[lane] : 0u);
+        if ((told & 1u) || !counted_locate(sp, src, tm, invT, zmax, kfloor, minp, rp.top_p, n_fin, list_cap, (told & 2u) != 0u)) { out.status |= ROW_NOT_COUNTED; return out; }
         w.S = w.S_all = s.bcast[2];
         w.race_from = 0.001f - logf(RACE_LUCK / ((float)s.bcast[3] * (1.0f / FX_SCALE)));
         switch (src.first_id() & 3) {

@@ -184,3 +184,37 @@ def test_penalised_scores_without_a_place(binding, sampler, B):
     g = to_host(sampler.albireo_sample(t.pop("logits"), **t, want_counts=True, want_status=True))
     rep = compare(w, g, ref)
     assert rep.ok() and len(rep.excused) <= 1, (rep.summary(), rep.failures[:3], rep.excused[:3])
+
+
+@pytest.mark.parametrize("B,V", [(40, 33007), (80, 8211)])
+@pytest.mark.parametrize("kind", ["half zeros", "tall", "too many tall", "all tall", "tiny"])
+@pytest.mark.parametrize("history", [False, True])
+def test_values_without_a_place(binding, sampler, B, V, kind, history):
+    """Values that the table does not hold: zeros of both signs by the thousand, up to 254 others that are listed (64 and more; nearer to zero than
+    2^-26), more of them than that; cuts among values of 64 and more, and below them, at temperatures that spread the mass over either."""
+    rng = np.random.default_rng(900 + B)
+    x = (rng.standard_normal((B, V)) * 3).astype(np.float32)
+    for b in range(B):
+        n = {"half zeros": V // 2, "tall": 1 + 31 * (b % 8), "too many tall": 255 + b, "all tall": V, "tiny": 245 + b % 16}[kind]
+        at = rng.permutation(V)[:n]
+        x[b, at] = {"half zeros": np.where(rng.random(n) < 0.5, 0.0, -0.0), "tiny": rng.choice([-1.0, 1.0], n) * 2.0 ** rng.uniform(-60, -27, n)}.get(
+            kind, rng.uniform(56, 100, n))
+        if kind == "tall" and b % 4 == 3:
+            x[b, rng.integers(0, V, 300)] = rng.uniform(57, 63.9, 300)
+    w = W.Workload(kind, B, V, W.BF16, W.f32_to_bf16_bits(x), temperature=np.where(np.arange(B) % 3 == 0, 1.0, rng.choice([8.0, 30.0], B)).astype(np.float32),
+                   top_p=rng.choice([0.01, 0.1, 0.5, 0.9, 0.99], B).astype(np.float32), seeds=rng.integers(0, 1 << 62, B).astype(np.uint64), step=4)
+    if history:
+        lens = rng.integers(0, 1200, B)
+        w.history_offsets = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+        w.history_ids = rng.integers(0, V, int(lens.sum())).astype(np.int32)
+        w.repetition_penalty, w.presence_penalty, w.frequency_penalty = (np.full(B, v, np.float32) for v in (1.13, 0.0, 0.0))
+    for num_top, full in ((0, False), (6, False), (6, True)):
+        w.num_top, w.logprob_full_vocab = num_top, full
+        ref = O.sample(w, threads=_CORES)
+        t = binding.workload_tensors(w, sampler.device)
+        g = to_host(sampler.albireo_sample(t.pop("logits"), **t, num_top=num_top, want_counts=True, want_status=True,
+                                           flags=binding.FLAG_LOGPROB_FULL_VOCAB if full else 0))
+        rep = compare(w, g, ref)
+        assert rep.ok() and len(rep.excused) <= 1, (rep.summary(), rep.failures[:3], rep.excused[:3])
+        bad = compare_top_lists(w, g, ref)
+        assert not bad, bad[:3]
