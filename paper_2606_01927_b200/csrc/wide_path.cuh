@@ -1635,13 +1635,15 @@ __device__ __noinline__ uint32_t count_finite(SRC src, BlockScratch *sp, float i
 }
 // Row (or slice) after the counting pass and a barrier: the number of finite scores among the vectors' elements, and what
 // the table cannot tell (bit 29), or only if the maximum is far above -63.75 (bit 28).  The same in every thread.
+// `exact`: else only those above -63.75 are wanted where there may be others.
 template <class SRC>
-__device__ __forceinline__ uint32_t counted_finite(const SRC &src, BlockScratch &s, float invT, uint32_t killed, uint32_t &flags) {
+__device__ __forceinline__ uint32_t counted_finite(const SRC &src, BlockScratch &s, float invT, uint32_t killed, uint32_t &flags, bool exact = true) {
     const CountedSegs &c = counted_segs(src);
     const uint32_t low = counted_table()[ct_index(CT_LOW)];
     flags = c.lost ? 0x20000000u : 0u;
     const uint32_t rest = (uint32_t)src.elements() - low;
     if (low == killed) return rest;
+    if (!exact) { flags |= 0x10000000u; return rest; }
     const uint32_t n = count_finite(src, &s, invT);
     if (n != rest) flags |= 0x10000000u;
     return n;
