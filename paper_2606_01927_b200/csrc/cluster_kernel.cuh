@@ -20,6 +20,12 @@ constexpr int GENERAL_BYTES = HIST_BINS * 16 + GL_CAP * 8 + 4096;      // what t
 __host__ __device__ constexpr int slice_coarse_off(int n) { return (((n + 31) / 32) + 4) & ~3; }
 __host__ __device__ constexpr int slice_counts_off(int n) { return slice_coarse_off(n) + ((n + 31) / 32 + 7) / 8 + 1; }
 
+// The largest 1 / T at which rows are counted by value.  Top-p rows with a Zipf prior over ids, us without and with counting: 32 of 128256, slices of
+// 64 KB, T = 0.2 16.5 and 18.4, 0.25 17.3 and 18.4, 0.3 17.8 and 18.5, 0.35 18.1 and 18.3, 0.7 19.6 and 19.5, 1 27.5 and 24.1; 64 of 152064, 152 KB,
+// 21.9 and 22.5, 24.4 and 22.6, at 0.3 26.0 and 22.4, 1 42.4 and 32.2.  (A row whose maximum is 29 and more above all else is as quick without at
+// any temperature, 14.3 and 17.7, but that is known too late.)
+__host__ __device__ constexpr float counted_inv_t(int slice_bytes) { return slice_bytes >= 96 * 1024 ? 4.0f : 3.0f; }
+
 // Bytes of what lies between a slice and the scores of its penalised tokens: those tables, or, when they are done with, what counted rows need.
 __host__ __device__ constexpr int slice_tables(bool counted, bool with_history, int n) {
     const int tables = with_history ? 4 * slice_counts_off(n) : 0;
@@ -250,8 +256,9 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     int *xid = (int *)(smem + src.xz_off) + (a.list_words >> 1);
     // (Rows are counted by value where a cut or a list has to be found, and in slices that are worth clearing and adding up a
     // table of 8192 counts: 32 top-p rows of 128256 by 4 CTAs 26.6 -> 23.7 us, but 13 of 50257 by 8 21.2 -> 23.1.  With no cut
-    // the pass of masses and race is faster than counting and race, 22.4 us against 24.5 for 64 rows of 152064.)
-    const bool cand_row = candidate_eligible(rp, a), counted = COUNTED && !cand_row && !nothing_cut(rp, a) && counted_eligible<DT>(rp, c, a);
+    // the pass of masses and race is faster than counting and race, 22.4 us against 24.5 for 64 rows of 152064.  At low temperatures
+    // hardly a vector has any mass, and the pass of masses passes over the others: see counted_inv_t.)
+    const bool cand_row = candidate_eligible(rp, a), counted = COUNTED && !cand_row && !nothing_cut(rp, a) && counted_eligible<DT>(rp, c, a) && c.invT <= counted_inv_t(a.slice_bytes);
     if (o1 > o0) {
         nx = slice_history<DT>(&s, c, a.hist_ids + o0, o1 - o0, ostart, SLICE_OFF, id0, n_slice_ids, tm.rank == 0 ? head : 0,
                                tm.rank == 0 ? tail0 : V, tab_off, src.xz_off, a.list_words, a.ws_counts, a.ws_counts_cap, (int64_t)o0,
