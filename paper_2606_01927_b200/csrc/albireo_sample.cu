@@ -211,7 +211,7 @@ __device__ __forceinline__ u64 warp_sum_u64(u64 v) {
     return v;
 }
 // all threads get the result; contains two barriers
-__device__ u64 block_max_u64(BlockScratch &, u64 v) {
+__device__ u64 block_max_u64(u64 v) {
     BlockScratch &s = block_scratch();
     v = warp_max_u64(v);
     __syncthreads();
@@ -222,7 +222,7 @@ __device__ u64 block_max_u64(BlockScratch &, u64 v) {
     for (int w = 1; w < NWARPS; ++w) { u64 t = s.red[w]; r = t > r ? t : r; }
     return r;
 }
-__device__ u64 block_sum_u64(BlockScratch &, u64 v) {
+__device__ u64 block_sum_u64(u64 v) {
     BlockScratch &s = block_scratch();
     v = warp_sum_u64(v);
     __syncthreads();
@@ -234,7 +234,7 @@ __device__ u64 block_sum_u64(BlockScratch &, u64 v) {
     return r;
 }
 // exclusive prefix sum over threads in thread order; also returns the block total
-__device__ u64 block_exscan_u64(BlockScratch &, u64 v, u64 &total) {
+__device__ u64 block_exscan_u64(u64 v, u64 &total) {
     BlockScratch &s = block_scratch();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     u64 inc = v;
@@ -605,7 +605,7 @@ struct HistSmem {
 };
 
 // exclusive prefix sum of 32-bit values over the threads of the block (thread order); block total in `total`
-__device__ uint32_t block_exscan_u32(BlockScratch &, uint32_t v, uint32_t &total) {
+__device__ uint32_t block_exscan_u32(uint32_t v, uint32_t &total) {
     BlockScratch &s = block_scratch();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t inc = v;
@@ -642,7 +642,7 @@ __device__ __forceinline__ void hist_prefetch(const int32_t *ids, int len, int32
 // Ids before position out_start are the prompt: they set their bit (repetition penalty) but are not counted.
 // Histories repeat a few ids very often: a bit already set is not set again.  (Combining equal ids
 // within a warp first, with match.any, was measured and cost far more than the atomics it saved.)
-__device__ bool build_history(BlockScratch &, const HistSmem &hs, RowCtx &c, const int32_t *ids, int len, int out_start,
+__device__ bool build_history(const HistSmem &hs, RowCtx &c, const int32_t *ids, int len, int out_start,
                               const int32_t *staged, uint32_t *ws, int64_t ws_cap, int64_t ws_off) {
     BlockScratch &s = block_scratch();
     const int V = c.V;
@@ -680,7 +680,7 @@ __device__ bool build_history(BlockScratch &, const HistSmem &hs, RowCtx &c, con
             }
         }
         uint32_t tot;
-        uint32_t ex = block_exscan_u32(s, pc, tot);
+        uint32_t ex = block_exscan_u32(pc, tot);
         if (cb < ncoarse) hs.coarse[cb] = carry + ex;
         carry += tot;
     }
@@ -842,7 +842,7 @@ struct MassSum {
 // was just read, so mostly from L2), four loads in flight; vectors with nothing within 29 of the
 // maximum carry no mass and are skipped by the packed test of the candidate path.  The same in every thread.
 template <int DT>
-__device__ u64 full_vocab_mass(BlockScratch &, const RowCtx &c, float zmax) {
+__device__ u64 full_vocab_mass(const RowCtx &c, float zmax) {
     BlockScratch &s = block_scratch();
     typedef Elem<DT> E;
     typedef VecTest<DT> T;
@@ -878,7 +878,7 @@ __device__ u64 full_vocab_mass(BlockScratch &, const RowCtx &c, float zmax) {
         const float d = __fsub_rn(z, zmax);
         if (d > -3.0e38f) local += mass_gen(d);         // -inf (and NaN) carry no mass
     });
-    return block_sum_u64(s, local + sum.total());
+    return block_sum_u64(local + sum.total());
 }
 
 // value-linear bin of a finite score z <= zmax; monotone: a larger z never gets a larger bin
@@ -890,7 +890,7 @@ __device__ __forceinline__ int bitlen64(u64 v) { return 64 - __clzll((long long)
 
 // Finds the first bin (from bin 0) at which the running total of the steering histogram reaches
 // `target` (1 <= target <= grand total).  Gives the totals of both histograms strictly before it.
-__device__ bool find_prefix_bin(BlockScratch &, const HistBins &h, bool by_mass, bool have_mass, u64 target,
+__device__ bool find_prefix_bin(const HistBins &h, bool by_mass, bool have_mass, u64 target,
                                 int &bin, u64 &cnt_before, u64 &mass_before) {
     BlockScratch &s = block_scratch();
     constexpr int PER = HIST_BINS / NT;
@@ -898,8 +898,8 @@ __device__ bool find_prefix_bin(BlockScratch &, const HistBins &h, bool by_mass,
 #pragma unroll
     for (int q = 0; q < PER; ++q) { lc += h.cnt[threadIdx.x * PER + q]; if (have_mass) lm += hist_mass(h, threadIdx.x * PER + q); }
     u64 totc, totm = 0;
-    u64 runc = block_exscan_u64(s, lc, totc);
-    u64 runm = have_mass ? block_exscan_u64(s, lm, totm) : 0ull;
+    u64 runc = block_exscan_u64(lc, totc);
+    u64 runm = have_mass ? block_exscan_u64(lm, totm) : 0ull;
     if (threadIdx.x == 0) s.found_digit = 0xFFFFFFFFu;
     __syncthreads();
     const u64 run = by_mass ? runm : runc, loc = by_mass ? lm : lc;
@@ -922,7 +922,7 @@ __device__ bool find_prefix_bin(BlockScratch &, const HistBins &h, bool by_mass,
 // Gathers the composites accepted by `take` into h.list (at most GL_CAP are stored); returns how many
 // were accepted, and their smallest and largest composite.
 template <int DT, class F>
-__device__ int gather_if(BlockScratch &, const HistBins &h, const RowCtx &c, F &&take, u64 &cmin, u64 &cmax) {
+__device__ int gather_if(const HistBins &h, const RowCtx &c, F &&take, u64 &cmin, u64 &cmax) {
     BlockScratch &s = block_scratch();
     if (threadIdx.x == 0) s.list_cnt = 0;
     __syncthreads();
@@ -935,8 +935,8 @@ __device__ int gather_if(BlockScratch &, const HistBins &h, const RowCtx &c, F &
             mn = C < mn ? C : mn; mx = C > mx ? C : mx;
         }
     });
-    cmax = block_max_u64(s, mx);
-    cmin = ~block_max_u64(s, ~mn);
+    cmax = block_max_u64(mx);
+    cmin = ~block_max_u64(~mn);
     return (int)s.list_cnt;
 }
 
@@ -948,7 +948,7 @@ __device__ int gather_if(BlockScratch &, const HistBins &h, const RowCtx &c, F &
 // equal keys, which quantised logits produce in their hundreds, cost nothing extra.
 // (out of line, and given plain pointers only, so that it neither shapes the register allocation of
 // its callers nor forces their structures into local memory)
-__device__ __noinline__ u64 list_resolve(BlockScratch *sp, u64 *list, int n, bool by_mass, u64 target, u64 lo, u64 hi, float zmax) {
+__device__ __noinline__ u64 list_resolve(u64 *list, int n, bool by_mass, u64 target, u64 lo, u64 hi, float zmax) {
     BlockScratch &s = block_scratch();
     struct { u64 *list; } h = {list};
     int P = 2;
@@ -978,7 +978,7 @@ __device__ __noinline__ u64 list_resolve(BlockScratch *sp, u64 *list, int n, boo
         if (C) local += by_mass ? mass_gen(__fsub_rn(unkey((uint32_t)(C >> 32)), zmax)) : 1ull;
     }
     u64 tot;
-    u64 run = block_exscan_u64(s, local, tot);
+    u64 run = block_exscan_u64(local, tot);
     if (threadIdx.x == 0) { s.bcast[3] = lo; }                   // target beyond the list: keep all of it
     __syncthreads();
     if (run < target && target <= run + local) {
@@ -999,12 +999,12 @@ __device__ __noinline__ u64 list_resolve(BlockScratch *sp, u64 *list, int n, boo
 // the order, over elements with C >= floorC) first reaches `target`, given that it falls in value bin
 // `bin` and that `before` of the total lies in the bins ahead of it.
 template <int DT>
-__device__ u64 resolve_cut(BlockScratch &, const HistBins &h, const RowCtx &c, float zmax, int bin, bool by_mass,
+__device__ u64 resolve_cut(const HistBins &h, const RowCtx &c, float zmax, int bin, bool by_mass,
                            u64 target, u64 before, u64 floorC, bool &hist_clobbered) {
     BlockScratch &s = block_scratch();
     u64 rel = target - before;
     u64 lo, hi;
-    int n = gather_if<DT>(s, h, c, [&](u64 C, float z) { return C >= floorC && (C >> 32) < KEY_POS_INF && bin_of(z, zmax) == bin; }, lo, hi);
+    int n = gather_if<DT>(h, c, [&](u64 C, float z) { return C >= floorC && (C >> 32) < KEY_POS_INF && bin_of(z, zmax) == bin; }, lo, hi);
     // a bin too full for the list is narrowed with composite-linear histograms over the row
     for (int it = 0; it < 8 && n > GL_CAP; ++it) {
         const u64 width = hi - lo;
@@ -1022,7 +1022,7 @@ __device__ u64 resolve_cut(BlockScratch &, const HistBins &h, const RowCtx &c, f
         });
         __syncthreads();
         int sub; u64 cb, mb;
-        if (!find_prefix_bin(s, h, by_mass, by_mass, rel, sub, cb, mb)) return lo > floorC ? lo : floorC;
+        if (!find_prefix_bin(h, by_mass, by_mass, rel, sub, cb, mb)) return lo > floorC ? lo : floorC;
         rel -= by_mass ? mb : cb;
         const u64 nhi = hi - ((u64)sub << shift);
         if (shift == 0) return nhi;
@@ -1033,13 +1033,13 @@ __device__ u64 resolve_cut(BlockScratch &, const HistBins &h, const RowCtx &c, f
         lo = nlo; hi = nhi;
         if (n <= GL_CAP) {
             u64 l2, h2;
-            n = gather_if<DT>(s, h, c, [&](u64 C, float) { return C >= lo && C <= hi && C >= floorC; }, l2, h2);
+            n = gather_if<DT>(h, c, [&](u64 C, float) { return C >= lo && C <= hi && C >= floorC; }, l2, h2);
             lo = l2; hi = h2;
         }
     }
     if (n > GL_CAP) return lo > floorC ? lo : floorC;        // not reachable: composites are distinct
     if (n < 1) return floorC;
-    return list_resolve(&s, h.list, n, by_mass, rel, lo, hi, zmax);
+    return list_resolve(h.list, n, by_mass, rel, lo, hi, zmax);
 }
 
 template <int DT, class A>
@@ -1049,15 +1049,15 @@ __device__ __forceinline__ void general_path(BlockScratch &s, const HistBins &h,
     // pass 0: the largest key and the number of finite scores
     uint32_t kbest = 0, nfin_local = 0;
     pass0_max_count<DT>(c, kbest, nfin_local);
-    const uint32_t kmax = (uint32_t)block_max_u64(s, kbest);
-    const u64 n_fin = block_sum_u64(s, nfin_local);
+    const uint32_t kmax = (uint32_t)block_max_u64(kbest);
+    const u64 n_fin = block_sum_u64(nfin_local);
     const float zmax = unkey(kmax);
     out.status |= ALBIREO_ROW_GENERAL_PATH;
     // the first element of the order: the lowest id among the largest keys (one more pass, only when asked for)
     auto top_id = [&]() -> int {
         uint32_t best = 0;
         for_each_score<DT>(c, [&](int i, float z) { if (key_of(z) == kmax) { const uint32_t v = ~(uint32_t)i; best = v > best ? v : best; } });
-        return max((int)~(uint32_t)block_max_u64(s, best), 0);         // (NaN: none equals the largest; an id in range all the same)
+        return max((int)~(uint32_t)block_max_u64(best), 0);         // (NaN: none equals the largest; an id in range all the same)
     };
 
     const bool full_lp = (a.flags & ALBIREO_FLAG_LOGPROB_FULL_VOCAB) != 0;
@@ -1093,12 +1093,12 @@ __device__ __forceinline__ void general_path(BlockScratch &s, const HistBins &h,
             if (!have_hist) build_hist(true, false);
             int bin; u64 cb, mb;
             bool clobbered = false;
-            if (find_prefix_bin(s, h, false, false, want, bin, cb, mb))
-                CN = resolve_cut<DT>(s, h, c, zmax, bin, false, want, cb, floorC, clobbered);
+            if (find_prefix_bin(h, false, false, want, bin, cb, mb))
+                CN = resolve_cut<DT>(h, c, zmax, bin, false, want, cb, floorC, clobbered);
             if (clobbered) have_hist = have_mass = false;
         }
         u64 lo, hi;
-        const int n = gather_if<DT>(s, h, c, [&](u64 C, float) { return C >= CN && (C >> 32) < KEY_POS_INF; }, lo, hi);
+        const int n = gather_if<DT>(h, c, [&](u64 C, float) { return C >= CN && (C >> 32) < KEY_POS_INF; }, lo, hi);
         const int m = n < ALBIREO_MAX_NUM_TOP ? n : ALBIREO_MAX_NUM_TOP;
         if ((int)threadIdx.x < m) {
             const u64 C = h.list[threadIdx.x];
@@ -1116,7 +1116,7 @@ __device__ __forceinline__ void general_path(BlockScratch &s, const HistBins &h,
     // the whole vocabulary is wanted: then they go through the cuts below as top_k = 1.
     if ((rp.greedy || n_fin <= 1) && !(full_lp && want_top_list)) {
         out.token = top_id(); out.logprob = 0.0f; out.n_keep = 1; out.n_topk = 1;
-        if (full_lp) out.logprob = (float)-(log((double)full_vocab_mass<DT>(s, c, zmax)) - LN2_40);
+        if (full_lp) out.logprob = (float)-(log((double)full_vocab_mass<DT>(c, zmax)) - LN2_40);
         if (a.dbg_topk_ids && a.dbg_cap >= 1 && threadIdx.x == 0) a.dbg_topk_ids[(int64_t)b * a.dbg_cap] = out.token;
         if (want_top_list && threadIdx.x == 0) {
             a.out_top_ids[(int64_t)b * a.num_top] = out.token;
@@ -1132,9 +1132,9 @@ __device__ __forceinline__ void general_path(BlockScratch &s, const HistBins &h,
     if (want_k) {
         n_topk = (u64)top_k;
         int bin; u64 cb, mb;
-        const bool find_ok = find_prefix_bin(s, h, false, want_topp, n_topk, bin, cb, mb);
+        const bool find_ok = find_prefix_bin(h, false, want_topp, n_topk, bin, cb, mb);
         bool clobbered = false;
-        if (find_ok) C1 = resolve_cut<DT>(s, h, c, zmax, bin, false, n_topk, cb, Cfin, clobbered);
+        if (find_ok) C1 = resolve_cut<DT>(h, c, zmax, bin, false, n_topk, cb, Cfin, clobbered);
         if (clobbered) have_hist = have_mass = false;
         if ((a.flags & ALBIREO_FLAG_TOPK_KEEP_TIES) && !rp.greedy) {
             // every id of the k-th largest key stays; how many that makes takes a count over the row
@@ -1142,7 +1142,7 @@ __device__ __forceinline__ void general_path(BlockScratch &s, const HistBins &h,
             const uint32_t k1 = (uint32_t)(C1 >> 32);
             uint32_t local = 0;
             for_each_score<DT>(c, [&](int, float z) { const uint32_t kk = key_of(z); local += (kk >= k1 && kk < KEY_POS_INF); });
-            n_topk = block_sum_u64(s, local);
+            n_topk = block_sum_u64(local);
         }
         if (want_topp && !have_mass) build_hist(false, true);
     }
@@ -1169,12 +1169,12 @@ __device__ __forceinline__ void general_path(BlockScratch &s, const HistBins &h,
         if (C1 == Cfin) {
             u64 lm = 0;
             for (int q = threadIdx.x; q < HIST_BINS; q += NT) lm += hist_mass(h, q);
-            Sp = block_sum_u64(s, lm);
+            Sp = block_sum_u64(lm);
         } else {
             u64 lm = 0;
             const uint32_t k1 = (uint32_t)(C1 >> 32); const int id1 = comp_idx(C1);
             for_each_score<DT>(c, [&](int i, float z) { const uint32_t k = key_of(z); if (k > k1 || (k == k1 && (uint32_t)i <= (uint32_t)id1)) lm += mass_gen(__fsub_rn(z, zmax)); });
-            Sp = block_sum_u64(s, lm);
+            Sp = block_sum_u64(lm);
         }
         double t = ceil((double)rp.top_p * (double)Sp);
         u64 target = t <= 1.0 ? 1ull : (u64)t;
@@ -1182,8 +1182,8 @@ __device__ __forceinline__ void general_path(BlockScratch &s, const HistBins &h,
         if (target < 1) target = 1;
         int bin; u64 cb, mb;
         bool clobbered = false;
-        if (find_prefix_bin(s, h, true, true, target, bin, cb, mb))
-            C2 = resolve_cut<DT>(s, h, c, zmax, bin, true, target, mb, C1, clobbered);
+        if (find_prefix_bin(h, true, true, target, bin, cb, mb))
+            C2 = resolve_cut<DT>(h, c, zmax, bin, true, target, mb, C1, clobbered);
         if (C2 < C1) C2 = C1;
         if (clobbered) have_hist = have_mass = false;
     }
@@ -1261,11 +1261,11 @@ __device__ __forceinline__ void general_path(BlockScratch &s, const HistBins &h,
         for_each_score_rest<DT>(c, head, nvec, [&](int i, float z) { see(i, z, true); });
         drain(0);
     }
-    const u64 S_fx = block_sum_u64(s, S_local);
-    const u64 n_keep = block_sum_u64(s, n_local);
-    const u64 G = block_max_u64(s, g_best);
+    const u64 S_fx = block_sum_u64(S_local);
+    const u64 n_keep = block_sum_u64(n_local);
+    const u64 G = block_max_u64(g_best);
     const int tok = max(comp_idx(G), 0);                 // (+inf or NaN among the scores: possibly no winner)
-    const double lnS = log((double)(full_lp ? full_vocab_mass<DT>(s, c, zmax) : S_fx)) - LN2_40;
+    const double lnS = log((double)(full_lp ? full_vocab_mass<DT>(c, zmax) : S_fx)) - LN2_40;
     float z_tok = score_of(c, tok, Elem<DT>::load(elem_ptr<DT>(c, tok), 0));
     out.token = tok;                                   // (a single kept element wins its own race)
     out.logprob = (n_keep == 1 && !full_lp) ? 0.0f : (float)(((double)z_tok - (double)zmax) - lnS);
@@ -1397,7 +1397,7 @@ __device__ __forceinline__ uint32_t warp_incl_scan_u32(uint32_t v) {
 // holds the k-th largest such key.  Returns false if fewer than k keys are in range.
 // On success [lo, hi] is narrowed to that bin and k to the rank inside it; `shift` tells
 // the bin width (0: the bin is a single key, i.e. lo is exactly the k-th largest key).
-__device__ bool cand_select_pass(BlockScratch &, const CandSmem &cs, int n, uint32_t &k, uint32_t &lo, uint32_t &hi, int &shift,
+__device__ bool cand_select_pass(const CandSmem &cs, int n, uint32_t &k, uint32_t &lo, uint32_t &hi, int &shift,
                                  bool zeroed = false) {
     BlockScratch &s = block_scratch();
     const uint32_t width = hi - lo;
@@ -1441,11 +1441,11 @@ __device__ bool cand_select_pass(BlockScratch &, const CandSmem &cs, int n, uint
 // Lower bound t of the k-th largest key in [lo, hi]: count(key >= t) >= k.  One pass when the
 // keys spread over the bins; an outlier that stretches the range leaves most keys in one bin, and
 // then up to two more passes narrow that bin.
-__device__ uint32_t cand_select_approx(BlockScratch &, const CandSmem &cs, int n, int k, uint32_t lo, uint32_t hi, bool zeroed = false) {
+__device__ uint32_t cand_select_approx(const CandSmem &cs, int n, int k, uint32_t lo, uint32_t hi, bool zeroed = false) {
     BlockScratch &s = block_scratch();
     uint32_t kk = (uint32_t)k; int shift = 1;
     for (int pass = 0; pass < 3 && shift != 0; ++pass) {
-        if (!cand_select_pass(s, cs, n, kk, lo, hi, shift, zeroed && pass == 0)) break;   // on failure lo is unchanged
+        if (!cand_select_pass(cs, n, kk, lo, hi, shift, zeroed && pass == 0)) break;   // on failure lo is unchanged
         const uint32_t pop = cs.hist[s.found_digit];
         __syncthreads();
         if (pop <= (uint32_t)(k / 4 + 8)) break;
@@ -1453,16 +1453,16 @@ __device__ uint32_t cand_select_approx(BlockScratch &, const CandSmem &cs, int n
     return lo;
 }
 // The k-th largest key in [lo, hi] exactly (as many passes as the key range needs).
-__device__ uint32_t cand_select_exact(BlockScratch &, const CandSmem &cs, int n, int k, uint32_t lo, uint32_t hi) {
+__device__ uint32_t cand_select_exact(const CandSmem &cs, int n, int k, uint32_t lo, uint32_t hi) {
     BlockScratch &s = block_scratch();
     uint32_t kk = (uint32_t)k; int shift = 1;
     for (int pass = 0; pass < 5 && shift != 0; ++pass)
-        if (!cand_select_pass(s, cs, n, kk, lo, hi, shift)) break;
+        if (!cand_select_pass(cs, n, kk, lo, hi, shift)) break;
     return lo;
 }
 
 // keeps the candidates with key >= tkey (and drops empty slots); returns the new count
-__device__ int cand_compact(BlockScratch &, const CandSmem &cs, int n, uint32_t tkey) {
+__device__ int cand_compact(const CandSmem &cs, int n, uint32_t tkey) {
     BlockScratch &s = block_scratch();
     constexpr int PER = CAND_CAP / NT;
     u64 mine[PER];
@@ -1688,7 +1688,7 @@ __device__ __forceinline__ void final_stage(BlockScratch &s, const CandSmem &cs,
 // warp then finds the bin in which the count from the top reaches k and the answer is that bin's
 // smallest key: at least k maxima are not below it.  Returns 0 if there are fewer than k maxima.
 // Needs cs.hist zero and the bin minima 0xFFFFFFFF on entry; contains two barriers, the last at the end.
-__device__ uint32_t warm_select(BlockScratch &, const CandSmem &cs, uint32_t mk, int k, uint32_t kmin, uint32_t kmax) {
+__device__ uint32_t warm_select(const CandSmem &cs, uint32_t mk, int k, uint32_t kmin, uint32_t kmax) {
     BlockScratch &s = block_scratch();
     uint32_t *binmin = (uint32_t *)(cs.cand + SEL_BINS);
     const float zmin = unkey(kmin), d = unkey(kmax) - zmin;
@@ -1743,7 +1743,7 @@ __device__ __forceinline__ void ring_setup(BlockScratch &s, const Ring &rg) {
 }
 // The first copies of the row (thread 0 only; after ring_setup).
 template <int DT>
-__device__ void candidate_begin(BlockScratch &, const Ring &rg, const RowCtx &c) {
+__device__ void candidate_begin(const Ring &rg, const RowCtx &c) {
     BlockScratch &s = block_scratch();
     typedef Elem<DT> E;
     if (threadIdx.x != 0) return;
@@ -1810,7 +1810,7 @@ template <int DT> __device__ __forceinline__ void passes_end() {
 }
 // The row's largest order key (s.mm_max) and the number of its finite scores (s.list_cnt), after passes_begin.
 template <int DT>
-__device__ __noinline__ void max_and_count(BlockScratch *sp) {
+__device__ __noinline__ void max_and_count() {
     BlockScratch &s = block_scratch();
     const RingSlice<DT> src;
     const float invT = row_shared<DT>().c.invT;
@@ -1833,12 +1833,12 @@ __device__ __noinline__ void max_and_count(BlockScratch *sp) {
 }
 // The mass of every finite score of the row (s.bcast[0]) and their number (s.bcast[1]), after passes_begin.
 template <int DT>
-__device__ __noinline__ void whole_row_totals(BlockScratch *sp, float zmax) {
+__device__ __noinline__ void whole_row_totals(float zmax) {
     BlockScratch &s = block_scratch();
-    max_and_count<DT>(sp);
+    max_and_count<DT>();
     u64 S, S_all;
     mass_pass<DT, SUM_ONLY, false>(RingSlice<DT>(), row_shared<DT>().c.invT, zmax, 0.0f, 0u, 0, S, S_all);
-    S = block_sum_u64(s, S);
+    S = block_sum_u64(S);
     if (threadIdx.x == 0) {
         RowShared &r = row_shared<DT>();
         s.bcast[0] = S; s.bcast[1] = s.list_cnt;
@@ -1875,11 +1875,11 @@ __device__ __forceinline__ bool candidate_finish(BlockScratch &s, const CandSmem
     const bool keep_ties = EXTRA && has_topk && !rp.greedy && (a.flags & ALBIREO_FLAG_TOPK_KEEP_TIES);
     if (has_topk) {
         if (n > SORT_MAX || n > 2 * k_list + 96 || (keep_ties && n > k)) {
-            uint32_t t = cand_select_exact(s, cs, n, k_list, tau_key, kmax);
-            n = cand_compact(s, cs, n, t);
+            uint32_t t = cand_select_exact(cs, n, k_list, tau_key, kmax);
+            n = cand_compact(cs, n, t);
         }
     } else {
-        n = cand_compact(s, cs, n, minp_key(unkey(kmax), rp.ln_min_p));
+        n = cand_compact(cs, n, minp_key(unkey(kmax), rp.ln_min_p));
     }
     if (n > SORT_MAX || n < 1) return false;
 
@@ -1969,7 +1969,7 @@ __device__ __forceinline__ bool candidate_path(BlockScratch &s, const CandSmem &
         if (stream_minp && threadIdx.x == 0) s.runmax = kmax;
         // fewer than k valid maxima: the select fails and tau stays at its floor
         if (has_topk && kmax) {
-            const uint32_t t = warm_select(s, cs, mk, k, kmin, kmax);
+            const uint32_t t = warm_select(cs, mk, k, kmin, kmax);
             if (t > tau_topk) tau_topk = t;
         }
         tau_key = tau_topk;
@@ -2023,11 +2023,11 @@ __device__ __forceinline__ bool candidate_path(BlockScratch &s, const CandSmem &
             first_look = false;
             if ((uint32_t)n + 1u >= trig_now) {
                 if (has_topk && n >= k) {
-                    uint32_t t = cand_select_approx(s, cs, n, k, tau_topk, rmax);
+                    uint32_t t = cand_select_approx(cs, n, k, tau_topk, rmax);
                     if (t > tau_topk) tau_topk = t;
                     if (t > tau_new) tau_new = t;
                 }
-                n = cand_compact(s, cs, n, tau_new);
+                n = cand_compact(cs, n, tau_new);
                 // if the list could not be shrunk (ties), look again only after it has grown
                 trig = (uint32_t)n + (uint32_t)(has_topk ? 2 * k + 32 : CAND_CAP / 4);
                 if (trig < trig0) trig = trig0;
@@ -2189,7 +2189,7 @@ __device__ __forceinline__ bool candidate_path(BlockScratch &s, const CandSmem &
             // 19.5 -> 23.0 us).
             if (threadIdx.x == 0) { passes_begin<DT>(s, c, a.vps, a.nstages); row_shared<DT>().rp = rp; s.bcast[3] = tau; }
             __syncthreads();
-            whole_row_totals<DT>(&s, unkey(kmax));
+            whole_row_totals<DT>(unkey(kmax));
             rq = row_shared<DT>().rp;
             full_fx = full_lp ? s.bcast[0] : 0ull; n_fin = s.bcast[1];
             tau = (uint32_t)s.bcast[3]; n = (int)s.cand_cnt; kmax = s.runmax;
@@ -2266,7 +2266,7 @@ __device__ __noinline__ RowCtx row_history(const SampleArgs *ap, int tab_off, Ro
     hs.coarse = hs.bitmap + (nwords + 1);
     hs.counts = hs.coarse + (ncoarse + 1);
     hist_prefetch(a.hist_ids + o0, o1 - o0, (int32_t *)smem);
-    c.has_hist = build_history(block_scratch(), hs, c, a.hist_ids + o0, o1 - o0, a.out_start ? a.out_start[b] : 0, (const int32_t *)smem,
+    c.has_hist = build_history(hs, c, a.hist_ids + o0, o1 - o0, a.out_start ? a.out_start[b] : 0, (const int32_t *)smem,
                                a.ws_counts, a.ws_counts_cap, (int64_t)o0);
     return c;
 }
@@ -2278,7 +2278,7 @@ __device__ __noinline__ RowCtx row_history(const SampleArgs *ap, int tab_off, Ro
 // (Called with the streaming path's structures by value, it cost the metric workload 2 to 4 us of 20.)
 // tab_off: where the history tables lie; no copy is in flight.
 template <int DT>
-__device__ __noinline__ void leftover_row(BlockScratch *sp, const SampleArgs *ap, int tab_off) {
+__device__ __noinline__ void leftover_row(const SampleArgs *ap, int tab_off) {
     extern __shared__ __align__(128) unsigned char smem[];
     BlockScratch &s = block_scratch();
     const SampleArgs &a = *ap;
@@ -2348,11 +2348,11 @@ __device__ __noinline__ void leftover_row(BlockScratch *sp, const SampleArgs *ap
                 uint32_t flags;
                 kmax = s.mm_max;
                 // (masked tokens are counted with all from -63.75 down: how many of those have a finite score takes another pass, which rows whose
-                // maximum is far above them do without where nobody asks for counts: 148 rows of 152064, half of the tokens masked, no cut, 48 us instead of 52)
+                // maximum is far above them do without where nobody asks for counts: 148 rows of 152064, half of the tokens masked, no cut, 47 us instead of 57)
                 const bool exact = a.out_num_kept || a.out_num_topk || a.num_top > 0 || r.rp.min_p > 0.0f || !(unkey(kmax) - ct_score(CT_LOW, r.c.invT) > 29.0f);
                 n_fin = counted_finite(src, s, r.c.invT, killed, flags, exact) + s.list_cnt;
                 __syncthreads();
-                if (kmax >= KEY_MIN_FINITE && !r.timeout) out = counted_row(sp, src, tm, r.rp, r.c.invT, kmax, n_fin, flags, b, status);
+                if (kmax >= KEY_MIN_FINITE && !r.timeout) out = counted_row(src, tm, r.rp, r.c.invT, kmax, n_fin, flags, b, status);
                 if ((out.status & ROW_NOT_COUNTED) && (flags & 0x10000000u) && !exact) kmax = 0;
             }
         }
@@ -2361,7 +2361,7 @@ __device__ __noinline__ void leftover_row(BlockScratch *sp, const SampleArgs *ap
             if (kmax == 0) {
                 if (threadIdx.x == 0) s.list_cnt = 0;
                 __syncthreads();
-                max_and_count<DT>(sp);
+                max_and_count<DT>();
                 kmax = s.mm_max; n_fin = s.list_cnt;
                 __syncthreads();
             }
@@ -2374,7 +2374,7 @@ __device__ __noinline__ void leftover_row(BlockScratch *sp, const SampleArgs *ap
         __syncthreads();                                       // the general path lays its own tables over them
         if (threadIdx.x == 0) passes_end<DT>();
         __syncthreads();
-        out = general_path_call<DT>(sp, smem, c, rp, b, status);
+        out = general_path_call<DT>(&s, smem, c, rp, b, status);
     }
     store_row(a, b, out);
 }
@@ -2449,7 +2449,7 @@ __global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const __grid_cons
                                                     : (const char *)c.row + (size_t)j * (size_t)a.seg_stride * Elem<DT>::SIZE;
         }
     }
-    if (ring_started) candidate_begin<DT>(s, rg, c);
+    if (ring_started) candidate_begin<DT>(rg, c);
     if (!with_hist) load_params();
 
     rp.greedy = !(rp.T > 0.0f);
@@ -2480,7 +2480,7 @@ __global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const __grid_cons
             hs.bitmap = (uint32_t *)(smem + tab_off);
             hs.coarse = hs.bitmap + (nwords + 1);
             hs.counts = hs.coarse + (ncoarse + 1);
-            c.has_hist = build_history(s, hs, c, a.hist_ids + o0, o1 - o0, ostart, (const int32_t *)smem, a.ws_counts, a.ws_counts_cap, (int64_t)o0);
+            c.has_hist = build_history(hs, c, a.hist_ids + o0, o1 - o0, ostart, (const int32_t *)smem, a.ws_counts, a.ws_counts_cap, (int64_t)o0);
             if (!c.has_hist) out.status |= ALBIREO_ROW_HISTORY_OVERFLOW;
         }
         __syncthreads();
@@ -2503,7 +2503,7 @@ __global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const __grid_cons
     }
     if (done) { store_row(a, b, out); return; }
     __syncthreads();
-    leftover_row<DT>(&s, &a, tab_off);
+    leftover_row<DT>(&a, tab_off);
 }
 
 #include "cluster_kernel.cuh"
@@ -2682,8 +2682,9 @@ struct LaunchShape { int team, nstages, slice_bytes, list_words; size_t smem; bo
 // clusters of 2^i CTAs (one per SM) are on the device at once.
 struct DeviceShape { int num_sms; size_t max_smem; int teams[5]; };
 
-// Elements of a slice of bfloat16 from which on values are counted (32 top-p rows of 128256 by 4 CTAs 26.6 -> 23.7 us, 74 of 48000 by 2 22.8 -> 21.8;
-// 30 of 64000 by 4 21.4 -> 23.1, so not there: clearing and adding up a table of 8192 counts has to be worth it).
+// Elements of a slice of bfloat16 from which on values are counted.  Top-p rows at T = 1, us without and with counting: slices of 16416 by 2 CTAs 20.2 and 19.6,
+// by 4 22.3 and 21.4, by 8 23.3 and 22.1; of 18000 20.7 and 20.4, 22.3 and 20.5, 24.1 and 22.3; of 28000 23.7 and 22.2, 25.7 and 23.4.  Half as
+// much is saved at 16416 as at 28000, and clearing and adding up a table of 8192 counts has to be worth it.
 constexpr long COUNTED_SLICE = 16384;
 
 // Rows are shared by clusters where all of them are on the chip at once, one CTA per SM: then every SM

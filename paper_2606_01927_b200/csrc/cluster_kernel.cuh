@@ -35,7 +35,7 @@ __host__ __device__ constexpr int slice_tables(bool counted, bool with_history, 
 // The k-th and the kp-th largest of the block's per-thread maxima `mk` (0: none), from below: the
 // smallest maximum of the value-linear bin in which the count from the top gets there (see
 // warm_select).  0 where there are fewer maxima.
-__device__ void slice_select(BlockScratch &, const CandSmem &cs, uint32_t mk, int k, int kp, uint32_t kmin, uint32_t kmax,
+__device__ void slice_select(const CandSmem &cs, uint32_t mk, int k, int kp, uint32_t kmin, uint32_t kmax,
                              uint32_t &tau, uint32_t &tau_part) {
     BlockScratch &s = block_scratch();
     uint32_t *binmin = (uint32_t *)(cs.cand + SEL_BINS);
@@ -86,7 +86,7 @@ __device__ void slice_select(BlockScratch &, const CandSmem &cs, uint32_t mk, in
 // the high word whether there are any in the prompt.
 // `landed()` waits for the slice; everything before it overlaps the copy.
 template <int DT, class W>
-__device__ __noinline__ int slice_history(BlockScratch *sp, RowCtx c, const int32_t *ids, int len, int out_start, int slice_off, int id0, int nids,
+__device__ __noinline__ int slice_history(RowCtx c, const int32_t *ids, int len, int out_start, int slice_off, int id0, int nids,
                                           int id_lo, int id_hi, int tab_off, int xz_off, int list_words, uint32_t *ws, int64_t ws_cap, int64_t ws_off,
                                           W landed, bool &ok, int *&xid) {
     typedef Elem<DT> E;
@@ -120,7 +120,7 @@ __device__ __noinline__ int slice_history(BlockScratch *sp, RowCtx c, const int3
         uint32_t pc = 0;
         if (cb < ncoarse) for (int w = cb << 3; w < min(nwords, (cb << 3) + 8); ++w) pc += __popc(bitmap[w]);
         uint32_t tot;
-        const uint32_t ex = block_exscan_u32(s, pc, tot);
+        const uint32_t ex = block_exscan_u32(pc, tot);
         if (cb < ncoarse) coarse[cb] = U + ex;
         U += tot;
     }
@@ -128,8 +128,8 @@ __device__ __noinline__ int slice_history(BlockScratch *sp, RowCtx c, const int3
     bool fits = 2u * (U + X_ENDS) <= (uint32_t)list_words;
     if (!fits && U + X_ENDS <= (uint32_t)list_words) {
         uint32_t at, n_own;
-        block_exscan_u32(s, ahead, at);
-        block_exscan_u32(s, own, n_own);
+        block_exscan_u32(ahead, at);
+        block_exscan_u32(own, n_own);
         fits = ws && ws_off >= 0 && U + X_ENDS <= n_own && ws_off + (int64_t)at + (int64_t)n_own <= ws_cap;
         if (fits) xid = (int *)ws + ws_off + at;
     }
@@ -164,8 +164,9 @@ __device__ __noinline__ RowOut team_wide_row(SRC src, TEAM tm, RowParams rp, flo
     return wide_row<DT>(block_scratch(), src, tm, rp, invT, kmax, n_fin, b, status);
 }
 
-// COUNTED: with the code for rows counted by value (see counted_row); the launches whose slices are too small for that do
-// without it (counted_slices): beside it their top-p rows took 1.4 us longer, 18.7 against 17.2 for 8 rows of 32000.
+// COUNTED: with the code for rows counted by value (see counted_row) and the table for it in front of the slice; launches whose slices are too small,
+// or whose rows are not counted, do without (see COUNTED_SLICE, may_count_rows): beside that code their top-p rows took 1.4 us longer, 18.7
+// against 17.2 for 8 rows of 32000.
 template <int DT, bool COUNTED>
 __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_constant__ SampleArgs a) {
     typedef Elem<DT> E;
@@ -260,7 +261,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     // hardly a vector has any mass, and the pass of masses passes over the others: see counted_inv_t.)
     const bool cand_row = candidate_eligible(rp, a), counted = COUNTED && !cand_row && !nothing_cut(rp, a) && counted_eligible<DT>(rp, c, a) && c.invT <= counted_inv_t(a.slice_bytes);
     if (o1 > o0) {
-        nx = slice_history<DT>(&s, c, a.hist_ids + o0, o1 - o0, ostart, SLICE_OFF, id0, n_slice_ids, tm.rank == 0 ? head : 0,
+        nx = slice_history<DT>(c, a.hist_ids + o0, o1 - o0, ostart, SLICE_OFF, id0, n_slice_ids, tm.rank == 0 ? head : 0,
                                tm.rank == 0 ? tail0 : V, tab_off, src.xz_off, a.list_words, a.ws_counts, a.ws_counts_cap, (int64_t)o0,
                                [&] { return mbar_wait(bar, 0); }, landed, xid);
         if (nx < 0) { nx = 0; fits = false; }
@@ -290,7 +291,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
         if constexpr (COUNTED) {
             counted_clear(src);
             __syncthreads();
-            if (__all_sync(0xFFFFFFFFu, landed)) counting_pass<0, false>(src, &s, c.invT, 0.0f);
+            if (__all_sync(0xFFFFFFFFu, landed)) counting_pass<0, false>(src, c.invT, 0.0f);
         }
     } else if (landed) {
         // (the number of finite scores is wanted for rows that may turn out to be wide, and by calls that ask for the top-k stage's size)
@@ -321,7 +322,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
     const bool any_late = __syncthreads_or(!landed) != 0;
     uint32_t kmax = s.mm_max, tau_s = 0, tau_p = 0, counted_flags = 0, n_vec = 0;
     if constexpr (COUNTED) { if (counted) n_vec = counted_finite(src, s, c.invT, distinct, counted_flags); }
-    if (cand_row && has_topk && kmax) slice_select(s, cs, mk, k_eff, (k_eff + tm.size - 1) / tm.size, s.mm_min, kmax, tau_s, tau_p);
+    if (cand_row && has_topk && kmax) slice_select(cs, mk, k_eff, (k_eff + tm.size - 1) / tm.size, s.mm_min, kmax, tau_s, tau_p);
     asm volatile("barrier.cluster.wait;" ::: "memory");            // (the arrival at the start)
     if ((int)threadIdx.x < tm.size) {
         const int r = threadIdx.x;
@@ -379,7 +380,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
             if (full_lp) {
                 u64 S_all, same;
                 mass_pass<DT, SUM_ONLY, false>(src, c.invT, unkey(kmax), 0.0f, 0u, 0, S_all, same);
-                S_all = block_sum_u64(s, S_all);
+                S_all = block_sum_u64(S_all);
                 if (threadIdx.x == 0) *tm.at(&tm.x->S_all[tm.rank], 0) = S_all;
             }
             __syncthreads();
@@ -409,7 +410,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
             if constexpr (COUNTED) {
                 // (out of line beside the code for counted rows, which else leaves the others spilling: 30 rows of 152064 with a top-k 10.5 us instead
                 // of 10.2.  Top-p rows that are not counted lose by it, 17.5 to 18.0 us for 8 rows of 32000: so not in the other kernel.)
-                if (counted) out = counted_row(&s, src, tm, rp, c.invT, kmax, n_fin, bad, b, status);
+                if (counted) out = counted_row(src, tm, rp, c.invT, kmax, n_fin, bad, b, status);
                 if (out.status & ROW_NOT_COUNTED) out = team_wide_row<DT>(src, tm, rp, c.invT, kmax, n_fin, b, status);
             } else out = wide_row<DT>(s, src, tm, rp, c.invT, kmax, n_fin, b, status);
             done = !(out.status & ROW_NOT_DONE);
@@ -429,7 +430,7 @@ __global__ void __launch_bounds__(NT, 1) albireo_cluster_kernel(const __grid_con
         hs.counts = hs.coarse + (nc + 1);
         if (o1 > o0) {
             hist_prefetch(a.hist_ids + o0, o1 - o0, (int32_t *)smem);
-            c.has_hist = build_history(s, hs, c, a.hist_ids + o0, o1 - o0, ostart, (const int32_t *)smem, a.ws_counts, a.ws_counts_cap, (int64_t)o0);
+            c.has_hist = build_history(hs, c, a.hist_ids + o0, o1 - o0, ostart, (const int32_t *)smem, a.ws_counts, a.ws_counts_cap, (int64_t)o0);
             if (!c.has_hist) out.status |= ALBIREO_ROW_HISTORY_OVERFLOW;
         }
         __syncthreads();

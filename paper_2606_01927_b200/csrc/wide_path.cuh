@@ -477,7 +477,7 @@ struct Window {
     bool found;
 };
 template <class TEAM>
-__device__ __noinline__ Window find_window(BlockScratch *sp, TEAM tm, bool by_count, uint32_t base, int shift, double frac, u64 target, int slack_shift) {
+__device__ __noinline__ Window find_window(TEAM tm, bool by_count, uint32_t base, int shift, double frac, u64 target, int slack_shift) {
     BlockScratch &s = block_scratch();
     uint32_t *hist = wide_smem().hist;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -578,7 +578,7 @@ __device__ __noinline__ void tie_pass(SRC src, float invT, float zmax, float zfl
 // only inside it: without that a cut far down a long tail (top-p 0.999) could not be told apart from
 // thousands of tail elements.  `target`: an exact mass in 2^-40 units, or a count.
 template <int DT, bool FLOOR, class SRC, class TEAM>
-__device__ __noinline__ bool narrow_window(BlockScratch *sp, SRC src, TEAM tm, float invT, float zmax, float zfloor, bool by_count, u64 target,
+__device__ __noinline__ bool narrow_window(SRC src, TEAM tm, float invT, float zmax, float zfloor, bool by_count, u64 target,
                                            uint32_t cap, Window *wp) {
     BlockScratch &s = block_scratch();
     Window w = *wp;
@@ -604,9 +604,9 @@ __device__ __noinline__ bool narrow_window(BlockScratch *sp, SRC src, TEAM tm, f
             u64 ahead;
             uint32_t kmin, kmax;
             tie_pass<DT>(src, invT, zmax, zfloor, w.lo, w.hi, ahead, kmin, kmax);
-            ahead = block_sum_u64(s, ahead);
-            kmax = (uint32_t)block_max_u64(s, kmax);
-            kmin = ~(uint32_t)block_max_u64(s, ~kmin);
+            ahead = block_sum_u64(ahead);
+            kmax = (uint32_t)block_max_u64(kmax);
+            kmin = ~(uint32_t)block_max_u64(~kmin);
             if ((int)threadIdx.x < tm.size) {
                 const int r = (int)threadIdx.x;
                 *tm.at(&tm.x->ahead[tm.rank], r) = ahead; *tm.at(&tm.x->kmax[tm.rank], r) = kmax; *tm.at(&tm.x->tau[tm.rank], r) = ~kmin;
@@ -620,7 +620,7 @@ __device__ __noinline__ bool narrow_window(BlockScratch *sp, SRC src, TEAM tm, f
             if (each == 0) return false;
             if (kmin == kmax) {
                 const u64 rest = target > ahead ? target - ahead : 1ull;
-                const Window t = find_window(sp, tm, true, 0u, TIE_SHIFT, 0.0, (rest + each - 1) / each, 1);
+                const Window t = find_window(tm, true, 0u, TIE_SHIFT, 0.0, (rest + each - 1) / each, 1);
                 if (!t.found) return false;
                 w.lo = w.hi = code_of(log2_mass(unkey(kmax), zmax));
                 w.id_lo = t.lo; w.id_hi = t.hi; w.most = t.most;
@@ -633,13 +633,13 @@ __device__ __noinline__ bool narrow_window(BlockScratch *sp, SRC src, TEAM tm, f
         }
         u64 ahead;
         window_mass_pass<DT, FLOOR>(src, invT, zmax, zfloor, w.lo, shift, ahead);
-        ahead = block_sum_u64(s, ahead);
+        ahead = block_sum_u64(ahead);
         if ((int)threadIdx.x < tm.size) *tm.at(&tm.x->ahead[tm.rank], (int)threadIdx.x) = ahead;
         tm.sync();
         ahead = warp_total(lane < tm.size ? tm.x->ahead[lane] : 0ull);
         const u64 before = w.before;
         const u64 rest = by_count ? target - before : (target > ahead ? target - ahead : 1ull);
-        w = find_window(sp, tm, by_count, w.lo, shift, 0.0, rest, by_count ? 0 : 11);
+        w = find_window(tm, by_count, w.lo, shift, 0.0, rest, by_count ? 0 : 11);
         if (!w.found) return false;
         w.before += before;                              // (a count; by mass the next level measures it anew)
     }
@@ -1106,15 +1106,15 @@ __device__ __forceinline__ void final_pass(const SRC &src, BlockScratch &s, Part
 }
 
 template <int DT, int OFF, bool CUT>
-__device__ __noinline__ Partial solo_race_all(BlockScratch *sp) {
+__device__ __noinline__ Partial solo_race_all() {
     Partial p;
-    race_all_shared<DT, OFF, CUT>(RingSlice<DT>(), *sp, p);
+    race_all_shared<DT, OFF, CUT>(RingSlice<DT>(), block_scratch(), p);
     return p;
 }
 template <int DT>
-__device__ __noinline__ Partial solo_final_pass(BlockScratch *sp) {
+__device__ __noinline__ Partial solo_final_pass() {
     Partial p;
-    final_pass<DT>(RingSlice<DT>(), *sp, p);
+    final_pass<DT>(RingSlice<DT>(), block_scratch(), p);
     return p;
 }
 template <int DT, bool FLOOR>
@@ -1129,15 +1129,15 @@ __device__ __forceinline__ void first_mass_pass(const RingSlice<DT> &, float inv
 // (out of line in clusters too: code that is fetched only when it runs leaves the other passes' code together. With the races without a
 // cut inlined 64 such rows of 152064 took 21.9 us instead of 21.5, 13 mixed rows of 50257 21.4 instead of 21.2.)
 template <int DT, int OFF, bool CUT>
-__device__ __noinline__ Partial team_race_all(SmemSlice<DT> src, BlockScratch *sp) {
+__device__ __noinline__ Partial team_race_all(SmemSlice<DT> src) {
     Partial p;
-    race_all<DT, OFF, CUT>(src, *sp, p);
+    race_all<DT, OFF, CUT>(src, block_scratch(), p);
     return p;
 }
 template <int DT, int OFF, bool CUT>
-__device__ __forceinline__ void run_race_all(const SmemSlice<DT> &src, BlockScratch &s, Partial &p) { p = team_race_all<DT, OFF, CUT>(src, &s); }
+__device__ __forceinline__ void run_race_all(const SmemSlice<DT> &src, BlockScratch &s, Partial &p) { p = team_race_all<DT, OFF, CUT>(src); }
 template <int DT, int OFF, bool CUT>
-__device__ __forceinline__ void run_race_all(const RingSlice<DT> &, BlockScratch &s, Partial &p) { p = solo_race_all<DT, OFF, CUT>(&s); }
+__device__ __forceinline__ void run_race_all(const RingSlice<DT> &, BlockScratch &s, Partial &p) { p = solo_race_all<DT, OFF, CUT>(); }
 template <int DT, bool CUT, class SRC>
 __device__ __forceinline__ void run_race(const SRC &src, BlockScratch &s, Partial &p) {
     switch (src.first_id() & 3) {
@@ -1148,7 +1148,7 @@ __device__ __forceinline__ void run_race(const SRC &src, BlockScratch &s, Partia
     }
 }
 template <int DT> __device__ __forceinline__ void run_final_pass(const SmemSlice<DT> &src, BlockScratch &s, Partial &p) { final_pass<DT>(src, s, p); }
-template <int DT> __device__ __forceinline__ void run_final_pass(const RingSlice<DT> &, BlockScratch &s, Partial &p) { p = solo_final_pass<DT>(&s); }
+template <int DT> __device__ __forceinline__ void run_final_pass(const RingSlice<DT> &, BlockScratch &s, Partial &p) { p = solo_final_pass<DT>(); }
 
 // ------------------------------------------------------------------ one wide row
 
@@ -1285,7 +1285,7 @@ __device__ __forceinline__ RowOut wide_finish_in(TEAM tm, float top_p, uint64_t 
             const int P = list_sort(list, L), per = (P + NT - 1) / NT, q0 = (int)threadIdx.x * per, q1 = min(L, q0 + per);
             u64 local = 0, tot;
             for (int q = q0; q < q1; ++q) local += mass_of(list[q]);
-            u64 run = p.M + block_exscan_u64(s, local, tot);
+            u64 run = p.M + block_exscan_u64(local, tot);
             reached = p.M + tot >= target;
 #pragma unroll 1
             for (int q = q0; q < q1 && run < target; ++q) {
@@ -1393,25 +1393,25 @@ __device__ __forceinline__ RowOut wide_row(BlockScratch &s, const SRC &src, cons
             else {
                 // (the histogram ends 42 octaves down: a row with fewer entries than wanted ahead of that is the
                 // general path's; what the bounds of the counts leave open shows when the list is there)
-                top = find_window(&s, tm, true, F_ZERO, W_SHIFT, 0.0, want, 0);
+                top = find_window(tm, true, F_ZERO, W_SHIFT, 0.0, want, 0);
                 ok = top.found && (u64)top.ahead_most + top.most >= want;
             }
         }
         if (topp && ok) {
             // (a member's rounding is up to 2^-12 of it, 2^-14 of the total with those of the others)
-            win = find_window(&s, tm, false, F_ZERO, W_SHIFT, fmax((double)rp.top_p, 1e-12), 0ull, 14);
+            win = find_window(tm, false, F_ZERO, W_SHIFT, fmax((double)rp.top_p, 1e-12), 0ull, 14);
             ok = win.found;
         }
         if (topp && ok && win.most > (uint32_t)list_cap) {
             const u64 target = topp_target(rp.top_p, warp_total(lane < tm.size ? *tm.at(&tm.x->S[lane], 0) : 0ull));
-            ok = minp ? narrow_window<DT, true>(&s, src, tm, invT, zmax, zfloor, false, target, list_cap, &win)
-                      : narrow_window<DT, false>(&s, src, tm, invT, zmax, zfloor, false, target, list_cap, &win);
+            ok = minp ? narrow_window<DT, true>(src, tm, invT, zmax, zfloor, false, target, list_cap, &win)
+                      : narrow_window<DT, false>(src, tm, invT, zmax, zfloor, false, target, list_cap, &win);
         }
         // (ahead of the list's last bin there are fewer than 2 num_top + 1 elements)
         const uint32_t top_cap = (uint32_t)(W_LIST - 2 * ALBIREO_MAX_NUM_TOP - 32);
         if (want_list && ok && !all_listed && top.most > top_cap)
-            ok = minp ? narrow_window<DT, true>(&s, src, tm, invT, zmax, zfloor, true, want, top_cap, &top)
-                      : narrow_window<DT, false>(&s, src, tm, invT, zmax, zfloor, true, want, top_cap, &top);
+            ok = minp ? narrow_window<DT, true>(src, tm, invT, zmax, zfloor, true, want, top_cap, &top)
+                      : narrow_window<DT, false>(src, tm, invT, zmax, zfloor, true, want, top_cap, &top);
         if (!ok) { tm.sync(); out.status |= ROW_NOT_DONE; return out; }          // (the same in every CTA)
     }
     if (threadIdx.x == 0) { s.list_cnt = 0; s.cand_cnt = 0; }
@@ -1559,7 +1559,7 @@ __device__ __forceinline__ void race_vector(RACER &rc, const uint4 &q, int i0, _
 // The first pass: values counted, s.mm_max the largest order key, s.list_cnt the finite scores among the extras.
 // RACE (no cut; see race_reference): the race as well, against zref in the place of the maximum: its candidates are listed (see CountedRacer).
 template <int OFF, bool RACE, class SRC>
-__device__ __noinline__ void counting_pass(SRC src, BlockScratch *sp, float invT, float zref) {
+__device__ __noinline__ void counting_pass(SRC src, float invT, float zref) {
     BlockScratch &s = block_scratch();
     const int end = src.end_id();
     __nv_bfloat162 most = __halves2bfloat162(__ushort_as_bfloat16(0xFF80), __ushort_as_bfloat16(0xFF80));
@@ -1594,12 +1594,12 @@ __device__ __noinline__ void counting_pass(SRC src, BlockScratch *sp, float invT
 }
 template <class SRC>
 __device__ __forceinline__ void run_counting(const SRC &src, BlockScratch &s, bool race, float invT, float zref) {
-    if (!race) { counting_pass<0, false>(src, &s, invT, 0.0f); return; }
+    if (!race) { counting_pass<0, false>(src, invT, 0.0f); return; }
     switch (src.first_id() & 3) {
-        case 0: counting_pass<0, true>(src, &s, invT, zref); break;
-        case 1: counting_pass<1, true>(src, &s, invT, zref); break;
-        case 2: counting_pass<2, true>(src, &s, invT, zref); break;
-        default: counting_pass<3, true>(src, &s, invT, zref); break;
+        case 0: counting_pass<0, true>(src, invT, zref); break;
+        case 1: counting_pass<1, true>(src, invT, zref); break;
+        case 2: counting_pass<2, true>(src, invT, zref); break;
+        default: counting_pass<3, true>(src, invT, zref); break;
     }
 }
 // What the race of a row without a cut is run against in the place of the maximum, which is not known yet: the largest score of the block's
@@ -1625,12 +1625,12 @@ __device__ __forceinline__ bool nothing_cut(const RowParams &rp, const SampleArg
 // How many of the vectors' elements have a finite score, where not all of those counted at CT_LOW are the `killed`
 // penalised tokens.  Ends with a barrier.
 template <class SRC>
-__device__ __noinline__ uint32_t count_finite(SRC src, BlockScratch *sp, float invT) {
+__device__ __noinline__ uint32_t count_finite(SRC src, float invT) {
     BlockScratch &s = block_scratch();
     const uint32_t thr = VecTest<ALBIREO_BF16>::finite_threshold(invT);
     uint32_t n = 0;
     src.vectors([&](const uint4 &q, int) { n += 8u - VecTest<ALBIREO_BF16>::count_not_finite(q, thr, invT); });
-    return (uint32_t)block_sum_u64(s, n);
+    return (uint32_t)block_sum_u64(n);
 }
 // Row (or slice) after the counting pass and a barrier: the number of finite scores among the vectors' elements, and what
 // the table cannot tell (bit 29), or only if the maximum is far above -63.75 (bit 28).  The same in every thread.
@@ -1643,7 +1643,7 @@ __device__ __forceinline__ uint32_t counted_finite(const SRC &src, BlockScratch 
     const uint32_t rest = (uint32_t)src.elements() - low;
     if (low == killed) return rest;
     if (!exact) { flags |= 0x10000000u; return rest; }
-    const uint32_t n = count_finite(src, &s, invT);
+    const uint32_t n = count_finite(src, invT);
     if (n != rest) flags |= 0x10000000u;
     return n;
 }
@@ -1671,7 +1671,7 @@ __device__ __noinline__ void append_elements(uint4 q, int i0, uint32_t bits, flo
     __syncwarp();
 }
 template <int OFF, class SRC>
-__device__ __noinline__ Partial counted_final_pass(SRC src, BlockScratch *sp) {
+__device__ __noinline__ Partial counted_final_pass(SRC src) {
     typedef VecTest<ALBIREO_BF16> T;
     extern __shared__ __align__(128) unsigned char smem[];
     BlockScratch &s = block_scratch();
@@ -1777,7 +1777,7 @@ __device__ __forceinline__ uint32_t ct_key_down_to(int seg, int hi, float invT) 
 // The masses of a counted row: its extras' and its values', by segments (in shared memory; cut.fail set where an extra has no place), or, with no
 // cut, each thread's share of the sum.
 template <class SRC>
-__device__ __noinline__ u64 counted_masses(SRC src, BlockScratch *sp, float invT, float zmax, uint32_t kfloor, bool no_cut) {
+__device__ __noinline__ u64 counted_masses(SRC src, float invT, float zmax, uint32_t kfloor, bool no_cut) {
     BlockScratch &s = block_scratch();
     CountedSegs &ct = counted_segs(src);
     const int t = threadIdx.x, n_odd = (int)ct.n_odd;
@@ -1831,7 +1831,7 @@ __device__ __noinline__ u64 counted_masses(SRC src, BlockScratch *sp, float invT
 // From the segments of all CTAs to the cut (see CountedCut), the same in every CTA; s.bcast[2] and [3]: the mass above the floor and the one to
 // be reached.  False: the table does not tell.
 template <class SRC, class TEAM>
-__device__ __noinline__ bool counted_locate(BlockScratch *sp, SRC src, TEAM tm, float invT, float zmax, uint32_t kfloor, bool minp, float top_p, uint32_t n_fin, int list_cap, bool high) {
+__device__ __noinline__ bool counted_locate(SRC src, TEAM tm, float invT, float zmax, uint32_t kfloor, bool minp, float top_p, uint32_t n_fin, int list_cap, bool high) {
     typedef VecTest<ALBIREO_BF16> T;
     BlockScratch &s = block_scratch();
     CountedSegs &ct = counted_segs(src);
@@ -1924,7 +1924,7 @@ __device__ __noinline__ bool counted_locate(BlockScratch *sp, SRC src, TEAM tm, 
 // A row (or a team's slices of it) whose values have been counted; by one CTA with no cut, it has been raced as well.
 // `flags`: see counted_finite, of all CTAs.  As wide_row otherwise.
 template <class SRC, class TEAM>
-__device__ __noinline__ RowOut counted_row(BlockScratch *sp, SRC src, TEAM tm, const RowParams rp, float invT, uint32_t kmax, uint32_t n_fin,
+__device__ __noinline__ RowOut counted_row(SRC src, TEAM tm, const RowParams rp, float invT, uint32_t kmax, uint32_t n_fin,
                                            uint32_t flags, int b, uint32_t status) {
     BlockScratch &s = block_scratch();
     const int lane = threadIdx.x & 31, t = threadIdx.x;
@@ -1946,7 +1946,7 @@ __device__ __noinline__ RowOut counted_row(BlockScratch *sp, SRC src, TEAM tm, c
         tm.x->far_cand = 0; tm.x->far_list = 0;
     }
     Partial p;
-    p.M = counted_masses(src, sp, invT, zmax, kfloor, raced);
+    p.M = counted_masses(src, invT, zmax, kfloor, raced);
     p.n = 0; p.G = 0; p.z = 0.0f;
     WideEnd w;
     w.M0 = 0; w.n0 = 0; w.S = 0; w.S_all = 0; w.zmax = zmax; w.n_fin = n_fin; w.summed = raced; w.in_team = false; w.all_kept = !topp && !minp; w.topp = topp;
@@ -1965,14 +1965,14 @@ __device__ __noinline__ RowOut counted_row(BlockScratch *sp, SRC src, TEAM tm, c
         if (t == 0) { s.found_digit = 0xFFFFFFFFu; s.found_cnt = 0xFFFFFFFFu; s.list_cnt = 0; s.cand_cnt = 0; s.race.philox = philox_row(rp.seed, rp.R, s.ga.step); }
         tm.sync();
         const uint32_t told = __reduce_or_sync(0xFFFFFFFFu, lane < tm.size ? tm.x->ncand[lane] : 0u);
-        if ((told & 1u) || !counted_locate(sp, src, tm, invT, zmax, kfloor, minp, rp.top_p, n_fin, list_cap, (told & 2u) != 0u)) { out.status |= ROW_NOT_COUNTED; return out; }
+        if ((told & 1u) || !counted_locate(src, tm, invT, zmax, kfloor, minp, rp.top_p, n_fin, list_cap, (told & 2u) != 0u)) { out.status |= ROW_NOT_COUNTED; return out; }
         w.S = w.S_all = s.bcast[2];
         w.race_from = 0.001f - logf(RACE_LUCK / ((float)s.bcast[3] * (1.0f / FX_SCALE)));
         switch (src.first_id() & 3) {
-            case 0: p = counted_final_pass<0>(src, &s); break;
-            case 1: p = counted_final_pass<1>(src, &s); break;
-            case 2: p = counted_final_pass<2>(src, &s); break;
-            default: p = counted_final_pass<3>(src, &s); break;
+            case 0: p = counted_final_pass<0>(src); break;
+            case 1: p = counted_final_pass<1>(src); break;
+            case 2: p = counted_final_pass<2>(src); break;
+            default: p = counted_final_pass<3>(src); break;
         }
         w.M0 = cut.M; w.n0 = cut.n;
     }

@@ -1,5 +1,6 @@
 """Rows of bfloat16 logits whose values are counted (top-p, min-p that keeps many, lists): the ends of the table of values,
-what has no place in it, cuts in the segments that penalised tokens share, against the oracle."""
+what has no place in it, cuts in the segments that penalised tokens share, against the oracle.  Only results are compared: a row that is not
+counted after all gives the same ones by the passes of other rows."""
 import os
 
 import numpy as np

@@ -88,6 +88,26 @@ def test_longest_slices(binding, sampler, dtype, history, B, V):
     assert rep.ok() and len(rep.excused) <= 1, (rep.summary(), rep.failures[:3], rep.excused[:3])
 
 
+@pytest.mark.parametrize("cut", ["top_k", "top_k and top_p"])
+def test_distinct_ids_that_a_slice_holds(binding, cut):
+    """64 rows of 152064 with 8500 distinct ids, some of them twice, in one half of the vocabulary: their scores still lie on chip (the ids in the
+    workspace), in the kernel with the table of values as well, and the rows are done in a single pass."""
+    B, V, n = 64, 152064, 8600
+    s = binding.Sampler(max_rows=B, max_vocab=V, max_history_total=B * n)
+    rng = np.random.default_rng(1)
+    w = W.Workload("many ids", B, V, W.BF16, W.f32_to_bf16_bits((rng.standard_normal((B, V)) * 3).astype(np.float32)), temperature=np.ones(B, np.float32),
+                   top_k=np.full(B, 40, np.int32), top_p=np.full(B, 0.9, np.float32) if "top_p" in cut else None, seeds=np.arange(B, dtype=np.uint64),
+                   history_ids=np.concatenate([np.tile(rng.permutation(V // 2)[:8500], 2)[:n] for _ in range(B)]).astype(np.int32), history_offsets=(np.arange(B + 1) * n).astype(np.int32),
+                   repetition_penalty=np.full(B, 1.2, np.float32), presence_penalty=np.zeros(B, np.float32), frequency_penalty=np.full(B, 0.1, np.float32))
+    ref = O.sample(w, threads=_CORES)
+    t = binding.workload_tensors(w, s.device)
+    g = to_host(s.albireo_sample(t.pop("logits"), **t, want_status=True))
+    rep = compare(w, g, ref)
+    assert rep.ok() and not rep.excused, (rep.summary(), rep.failures[:3], rep.excused[:3])
+    assert not (g["row_status"] & (binding.ROW_GENERAL_PATH | binding.ROW_HISTORY_OVERFLOW)).any()
+    s.close()
+
+
 @pytest.mark.parametrize("par,counted", [(("top_p",), True), (("num_top",), True), (("top_k", "top_p"), True), ((), False), (("top_k",), False), (("min_p",), False)])
 def test_table_of_values_only_where_a_row_may_need_it(binding, sampler, par, counted):
     B, V = 64, 152064
