@@ -123,10 +123,10 @@ __device__ __forceinline__ float pick_element(const uint4 &q, int x) {
 
 // A callee that returns a truth value is called on after the last vector, with id -1, until it returns false (the same in
 // every lane of a warp): what it has put by is worked off by the same code.
-// One that takes two vectors gets two of a thread's at a time from a ring, and elsewhere one and nothing (-inf, id -1).
+// One that takes two vectors (and returns nothing) gets two of a thread's at a time from a ring, and elsewhere one and nothing (-inf, id -1).
 template <class F> constexpr bool by_pairs = std::is_invocable<F, uint4, uint4, int, int>::value;
 template <class F> constexpr bool answers() {
-    if constexpr (by_pairs<F>) return std::is_same<std::invoke_result_t<F, uint4, uint4, int, int>, bool>::value;
+    if constexpr (by_pairs<F>) return false;
     else return std::is_same<std::invoke_result_t<F, uint4, int>, bool>::value;
 }
 template <class F> constexpr bool goes_on = answers<F>();
@@ -223,9 +223,9 @@ struct RingSlice {
             for (int u = 0; after || u < tv; u += PAIRS ? 2 : 1) {
                 const int i0 = after ? -1 : head + ((t * tv + u) * NT + (int)threadIdx.x) * E::PER_VEC;
                 if constexpr (PAIRS) {
-                    const int i1 = after ? -1 : i0 + NT * E::PER_VEC;
+                    const int i1 = i0 + NT * E::PER_VEC;
                     const uint4 q0 = fetch(u, i0), q1 = fetch(u + 1, i1);
-                    if constexpr (AFTER) { if (!f(q0, q1, i0, i1) && after) break; } else f(q0, q1, i0, i1);
+                    f(q0, q1, i0, i1);
                 } else {
                     const uint4 q = fetch(u, i0);
                     if constexpr (AFTER) { if (!f(q, i0) && after) break; } else f(q, i0);
@@ -305,8 +305,7 @@ struct SmemSlice {
             const int v = base + (int)threadIdx.x, i0 = base < nvec ? id0 + v * E::PER_VEC : -1;
             const uint4 q = v < nvec ? vec[v] : VecTest<DT>::fill();
             bool more = false;
-            if constexpr (PAIRS && AFTER) more = f(q, VecTest<DT>::fill(), i0, -1);
-            else if constexpr (PAIRS) f(q, VecTest<DT>::fill(), i0, -1);
+            if constexpr (PAIRS) f(q, VecTest<DT>::fill(), i0, -1);
             else if constexpr (AFTER) more = f(q, i0);
             else f(q, i0);
             if (AFTER && !more && base >= nvec) break;
