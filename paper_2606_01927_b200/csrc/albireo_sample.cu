@@ -1784,35 +1784,24 @@ __device__ __forceinline__ bool wide_eligible(const RowParams &rp, const SampleA
 
 #include "wide_path.cuh"
 
-// Sets the passes of one CTA over a row from global memory up (thread 0; a barrier follows): the row's
-// block in shared memory, and the ring's barriers.
+// Sets the passes of one CTA over a row from global memory up (thread 0; a barrier follows).
 template <int DT>
-__device__ __forceinline__ void passes_begin(BlockScratch &s, const RowCtx &c, int vps, int nstages) {
+__device__ __forceinline__ void passes_begin(BlockScratch &s, const RowCtx &c) {
     RowShared &r = row_shared<DT>();
-    r.c = c; r.vps = vps;
+    r.c = c;
     const uintptr_t addr = (uintptr_t)c.row;
     int head = (int)(((16u - (uint32_t)(addr & 15u)) & 15u) / Elem<DT>::SIZE);
     if (head > c.V) head = c.V;
     r.head = head; r.nvec = (c.V - head) / Elem<DT>::PER_VEC;
     r.vp = (const uint4 *)((const char *)c.row + (size_t)head * Elem<DT>::SIZE);
-    const int room = (COMMON_BYTES + nstages * STAGE_BYTES - wide_ring_off(DT)) / WIDE_VEC_BYTES;
-    r.tv = room >= 8 ? 4 : 2;
-    r.nst = min(WIDE_MAX_STAGES, room / r.tv);
-#pragma unroll 1
-    for (int q = 0; q < r.nst; ++q) { mbar_init(&r.bar[q], 1); r.done[q] = 0; }
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    r.tiles = 0; r.issued = 0; r.timeout = 0; s.mm_max = 0; s.list_cnt = 0;
-}
-// The ring's barriers are done with (thread 0): their memory may be used for something else.
-template <int DT> __device__ __forceinline__ void passes_end() {
-    RowShared &r = row_shared<DT>();
-    for (int q = 0; q < r.nst; ++q) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(&r.bar[q])) : "memory");
+    r.vps = c.Vs / Elem<DT>::PER_VEC;
+    s.mm_max = 0; s.list_cnt = 0;
 }
 // The row's largest order key (s.mm_max) and the number of its finite scores (s.list_cnt), after passes_begin.
 template <int DT>
 __device__ __noinline__ void max_and_count() {
     BlockScratch &s = block_scratch();
-    const RingSlice<DT> src;
+    const RowSlice<DT> src;
     const float invT = row_shared<DT>().c.invT;
     const uint32_t fin_thr = VecTest<DT>::finite_threshold(invT);
     uint32_t kbest = 0, nfin = 0;
@@ -1837,13 +1826,10 @@ __device__ __noinline__ void whole_row_totals(float zmax) {
     BlockScratch &s = block_scratch();
     max_and_count<DT>();
     u64 S, S_all;
-    mass_pass<DT, SUM_ONLY, false>(RingSlice<DT>(), row_shared<DT>().c.invT, zmax, 0.0f, 0u, 0, S, S_all);
+    mass_pass<DT, SUM_ONLY, false>(RowSlice<DT>(), row_shared<DT>().c.invT, zmax, 0.0f, 0u, 0, S, S_all);
     S = block_sum_u64(S);
     if (threadIdx.x == 0) {
-        RowShared &r = row_shared<DT>();
         s.bcast[0] = S; s.bcast[1] = s.list_cnt;
-        if (r.timeout) s.timeout = 1u;
-        passes_end<DT>();
     }
     __syncthreads();
 }
@@ -2187,13 +2173,12 @@ __device__ __forceinline__ bool candidate_path(BlockScratch &s, const CandSmem &
             // A pass over the whole row that only some calls ask for, out of line.  What is needed behind it waits in
             // shared memory: kept in registers it was spilled ahead of the stream for every call (256 rows with counts
             // 19.5 -> 23.0 us).
-            if (threadIdx.x == 0) { passes_begin<DT>(s, c, a.vps, a.nstages); row_shared<DT>().rp = rp; s.bcast[3] = tau; }
+            if (threadIdx.x == 0) { passes_begin<DT>(s, c); row_shared<DT>().rp = rp; s.bcast[3] = tau; }
             __syncthreads();
             whole_row_totals<DT>(unkey(kmax));
             rq = row_shared<DT>().rp;
             full_fx = full_lp ? s.bcast[0] : 0ull; n_fin = s.bcast[1];
             tau = (uint32_t)s.bcast[3]; n = (int)s.cand_cnt; kmax = s.runmax;
-            if (s.timeout) { out.status |= ALBIREO_ROW_TIMEOUT; out.token = -1; out.logprob = __uint_as_float(0x7FC00000u); out.n_keep = 0; out.n_topk = 0; return true; }
             __syncthreads();
         }
     }
@@ -2293,7 +2278,7 @@ __device__ __noinline__ void leftover_row(const SampleArgs *ap, int tab_off) {
     __syncthreads();
     if (threadIdx.x == 0) {
         fill_general_args(s.ga, a);
-        passes_begin<DT>(s, c, a.vps, a.nstages);
+        passes_begin<DT>(s, c);
         row_shared<DT>().rp = rp;
         s.race.bound = NO_BOUND;
     }
@@ -2320,18 +2305,18 @@ __device__ __noinline__ void leftover_row(const SampleArgs *ap, int tab_off) {
     out.status = status | ROW_NOT_DONE;
     if (wide_eligible(rp, a)) {
         const RowShared &r = row_shared<DT>();
-        const RingSlice<DT> src;
+        const RowSlice<DT> src;
         SoloTeam<counts_rows(DT)> tm;
         uint32_t kmax = 0, n_fin = 0;
         out.status = status | ROW_NOT_COUNTED;
         if constexpr (DT == ALBIREO_BF16) {
             if (counted_eligible<DT>(rp, c, a)) {
-                // (with no cut the row's first tile is still where the stream put it: its largest score is what the race is run against)
+                // (with no cut: the largest score of the row's first vectors is what the race is run against)
                 const bool race = nothing_cut(rp, a);
                 uint4 q = VecTest<DT>::fill();
                 int ends = 0;
                 if (race && (int)threadIdx.x < r.nvec) {
-                    q = ((const uint4 *)(smem + COMMON_BYTES))[threadIdx.x];
+                    q = __ldg(vec_ptr<DT>(c, r.vp, (int)threadIdx.x));
                     const int i0 = r.head + (int)threadIdx.x * Elem<DT>::PER_VEC;
                     if (c.has_hist) q = kill_elements<DT>(q, __funnelshift_r(c.bitmap[i0 >> 5], c.bitmap[(i0 >> 5) + 1], i0 & 31));
                 }
@@ -2352,7 +2337,7 @@ __device__ __noinline__ void leftover_row(const SampleArgs *ap, int tab_off) {
                 const bool exact = a.out_num_kept || a.out_num_topk || a.num_top > 0 || r.rp.min_p > 0.0f || !(unkey(kmax) - ct_score(CT_LOW, r.c.invT) > 29.0f);
                 n_fin = counted_finite(src, s, r.c.invT, killed, flags, exact) + s.list_cnt;
                 __syncthreads();
-                if (kmax >= KEY_MIN_FINITE && !r.timeout) out = counted_row(src, tm, r.rp, r.c.invT, kmax, n_fin, flags, b, status);
+                if (kmax >= KEY_MIN_FINITE) out = counted_row(src, tm, r.rp, r.c.invT, kmax, n_fin, flags, b, status);
                 if ((out.status & ROW_NOT_COUNTED) && (flags & 0x10000000u) && !exact) kmax = 0;
             }
         }
@@ -2367,13 +2352,10 @@ __device__ __noinline__ void leftover_row(const SampleArgs *ap, int tab_off) {
             }
             if (kmax >= KEY_MIN_FINITE) out = wide_row<DT>(s, src, tm, r.rp, r.c.invT, kmax, n_fin, b, status);
         }
-        if (r.timeout) { out.status = (out.status & ~ROW_NOT_DONE) | ALBIREO_ROW_TIMEOUT; out.token = -1; out.logprob = __uint_as_float(0x7FC00000u); out.n_keep = 0; out.n_topk = 0; }
     }
     if (out.status & ROW_NOT_DONE) {
         c = row_shared<DT>().c; rp = row_shared<DT>().rp;
         __syncthreads();                                       // the general path lays its own tables over them
-        if (threadIdx.x == 0) passes_end<DT>();
-        __syncthreads();
         out = general_path_call<DT>(&s, smem, c, rp, b, status);
     }
     store_row(a, b, out);

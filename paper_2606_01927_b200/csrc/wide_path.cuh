@@ -121,141 +121,114 @@ __device__ __forceinline__ float pick_element(const uint4 &q, int x) {
     return Elem<DT>::get(make_uint4(w, w, w, w), PV == 4 ? 0 : (x & 1));
 }
 
-// A callee that returns a truth value is called on after the last vector, with id -1, until it returns false (the same in
-// every lane of a warp): what it has put by is worked off by the same code.
-// One that takes two vectors (and returns nothing) gets two of a thread's at a time from a ring, and elsewhere one and nothing (-inf, id -1).
+// A callee that takes two vectors gets two of a thread's at a time from global memory, and elsewhere one and nothing (-inf, id -1).
 template <class F> constexpr bool by_pairs = std::is_invocable<F, uint4, uint4, int, int>::value;
-template <class F> constexpr bool answers() {
-    if constexpr (by_pairs<F>) return false;
-    else return std::is_same<std::invoke_result_t<F, uint4, int>, bool>::value;
-}
-template <class F> constexpr bool goes_on = answers<F>();
+// A callee may come with a test of four vectors at once: where no lane's answer is true the callee is not called for them (it must
+// have nothing to do there).
+struct NoTest {};
 
-// The whole row, streamed from global memory (from the L2 after the first pass) through a ring of bulk
-// copies: next to CTAs that stream their own rows a plain load comes back after 1.5 to 3 us, and only the
-// copies of whole tiles keep enough of them in flight.  Penalised tokens are masked out of the vectors
+// The whole row from global memory (from the L2 after the first pass), in plain 16-byte loads that wait in registers: AHEAD of a thread's
+// vectors are on their way while it works on another.  Penalised tokens are masked out of the vectors
 // and come from the history tables.  Both loops have the same trip count in every lane of a warp (lanes
 // past the end see -inf), so that the callee may use warp collectives, but no block barriers.
-// (A pass needs its registers for the elements: what the loop does not touch per vector stays in shared memory.)
-// (a tile is 4 vectors per thread, 32 KiB, where two of them fit, else 2: what a tile costs is the hand-shake)
-constexpr int WIDE_VEC_BYTES = NT * 16;
-constexpr int WIDE_MAX_STAGES = 6;
+// (What the loop does not touch per vector stays in shared memory: a pass needs its registers for the elements.)
+// What bounds a pass is shared memory and issue slots, not the loads: with the vectors brought into shared memory by bulk copies, as before,
+// both the copies and the reads back were in the way of the callee's own accesses, and each tile of 32 KB cost a hand-shake of all
+// warps.  A row of 152064 bfloat16 logits by one CTA, in the L2, us including the launch, from a ring and from registers: largest element
+// 8.3 and 6.2, counted by value 19.5 and 12.4, exponentials summed 13.2 and 12.4; two rows per SM 10.3 and 8.2, 32.8 and 22.4, 23.7 and 20.5.
 struct RowShared {
     RowCtx c;
     RowParams rp;
     const uint4 *vp;
-    int head, nvec, vps, nst, tv; // stages of the ring, vectors per thread and tile
-    uint32_t tiles;               // tiles of the passes so far
-    uint32_t issued;              // tiles of this pass whose copy has been issued
-    uint32_t timeout;             // a wait on a copy expired
-    uint32_t done[WIDE_MAX_STAGES];
-    uint64_t bar[WIDE_MAX_STAGES];
+    int head, nvec;
+    int vps;                      // vectors per piece
 };
 template <int DT> __device__ __forceinline__ RowShared &row_shared();
-template <int DT> __device__ __forceinline__ unsigned char *wide_stage(int st);
 template <int DT> __device__ __forceinline__ constexpr int row_segments();
+// which of the n elements from i0 on are in the history, from the bitmap's address in shared memory
+template <int N>
+__device__ __forceinline__ uint32_t history_mask(uint32_t bitmap, int i0) {
+    uint32_t w0, w1;
+    asm volatile("ld.shared.u32 %0, [%2];\n\tld.shared.u32 %1, [%2 + 4];" : "=r"(w0), "=r"(w1) : "r"(bitmap + 4u * ((uint32_t)i0 >> 5)));
+    return __funnelshift_r(w0, w1, i0 & 31) & ((1u << N) - 1u);
+}
 template <int DT>
-struct RingSlice {
+struct RowSlice {
     typedef Elem<DT> E;
     static constexpr bool SPARE_REGISTERS = false;      // 64 per thread
     __device__ __forceinline__ int first_id() const { return row_shared<DT>().head; }
     __device__ __forceinline__ int end_id() const { return row_shared<DT>().head + row_shared<DT>().nvec * E::PER_VEC; }
     __device__ __forceinline__ int elements() const { return row_shared<DT>().nvec * E::PER_VEC; }
     __device__ __forceinline__ int segments() const { return row_segments<DT>(); }      // (counted rows: see CountedSegs)
-    __device__ __forceinline__ static void issue(RowShared &r, int t, int st) {
-        Ring rg;
-        rg.vps = r.vps; rg.seg_base = r.c.seg_base;
-        const int v0 = t * (NT * r.tv), nv = min(r.nvec - v0, NT * r.tv);
-        mbar_expect_tx(&r.bar[st], (uint32_t)nv * 16u);
-        ring_copy(rg, wide_stage<DT>(st * r.tv), r.vp, v0, nv, &r.bar[st]);
-    }
-    // The tiles of all passes are numbered through, which gives stage and phase; the last warp done with a
-    // stage refills it.  A wait that expires marks the row, and nothing more is copied.
-    template <class F> __device__ __forceinline__ void vectors(F &&f) const {
-        constexpr bool AFTER = goes_on<F>, PAIRS = by_pairs<F>;
-        RowShared &r = row_shared<DT>();
-        const uint32_t first = r.tiles;
-        const int nvec = r.nvec, head = r.head, nst = r.nst, tv = r.tv, ntiles = (nvec + NT * tv - 1) / (NT * tv);
-        const uint32_t *bitmap = r.c.has_hist ? r.c.bitmap : nullptr;
-        int st = (int)(first % (uint32_t)nst);
-        uint32_t parity = (first / (uint32_t)nst) & 1u;
-        if (threadIdx.x == 0) {
-            const int npre = r.timeout ? 0 : min(ntiles, nst);
-            r.issued = (uint32_t)npre;
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-#pragma unroll 1
-            for (int t = 0, q = st; t < npre; ++t) { issue(r, t, q); q = q + 1 == nst ? 0 : q + 1; }
+    __device__ __forceinline__ int count() const { return row_shared<DT>().nvec; }
+    // vector v by itself (v < 0: none)
+    __device__ __forceinline__ uint4 vector(int v) const {
+        if (v < 0) return VecTest<DT>::fill();
+        const RowShared &r = row_shared<DT>();
+        uint4 q = __ldg(vec_ptr<DT>(r.c, r.vp, v));
+        if (r.c.has_hist) {
+            const uint32_t m = history_mask<E::PER_VEC>(smem_u32(r.c.bitmap), r.head + v * E::PER_VEC);
+            if (m) q = kill_elements<DT>(q, m);
         }
-        __syncwarp();       // (the other lanes of the issuing warp, spinning on the first copy, could keep the issuing lane from running)
+        return q;
+    }
+    // Those of the row's vectors from `first` on and before `end`, piece after piece (lanes past the end of one see -inf and the id behind the last).
+    template <int AHEAD = 4, class F, class T = NoTest> __device__ __forceinline__ void vectors(F &&f, T &&test = T(), int first = 0, int end = 0x7FFFFFFF) const {
+        constexpr bool PAIRS = by_pairs<F>, TESTED = !std::is_same<std::decay_t<T>, NoTest>::value;
+        const RowShared &r = row_shared<DT>();
+        const int head = r.head, end_id = head + r.nvec * E::PER_VEC;
+        const uint32_t bitmap = r.c.has_hist ? smem_u32(r.c.bitmap) : 0u;
+        auto masked = [&](uint4 q, int i0) -> uint4 {
+            if (bitmap && i0 < end_id) {
+                const uint32_t m = history_mask<E::PER_VEC>(bitmap, i0);
+                if (m) q = kill_elements<DT>(q, m);
+            }
+            return q;
+        };
 #pragma unroll 1
-        for (int t = 0; AFTER || t < ntiles; ++t) {
-            const bool after = AFTER && t == ntiles;
-            if (!after && *(volatile uint32_t *)&r.timeout == 0u && !mbar_wait(&r.bar[st], parity)) r.timeout = 1u;
-            __syncwarp();
-            const uint4 *stage = (const uint4 *)wide_stage<DT>(st * tv);
-            if constexpr (!PAIRS && !AFTER) {
+        for (int j = 0; j < r.c.nseg; ++j) {
+            const bool whole = r.c.nseg == 1;
+            const int v_lo = whole ? 0 : j * r.vps, lo = max(first, v_lo), hi = min(min(r.nvec, end), whole ? r.nvec : v_lo + r.vps);
+            const uint4 *const vp = (whole ? r.vp : (const uint4 *)r.c.seg_base[j]) - v_lo;
+            auto load = [&](int v) -> uint4 { return v < hi ? __ldg(vp + v) : VecTest<DT>::fill(); };
+            auto id_of = [&](int v) { return v < hi ? head + v * E::PER_VEC : end_id; };
+            if constexpr (TESTED) {
+                // four at a time, and one after another where some matter
 #pragma unroll 1
-                for (int u = 0; u < tv; ++u) {
-                    const int v = (t * tv + u) * NT + (int)threadIdx.x, i0 = head + v * E::PER_VEC;
-                    uint4 q = VecTest<DT>::fill();
-                    if (v < nvec) {
-                        q = stage[u * NT + threadIdx.x];
-                        if (bitmap) {
-                            const uint32_t m = __funnelshift_r(bitmap[i0 >> 5], bitmap[(i0 >> 5) + 1], i0 & 31) & ((1u << E::PER_VEC) - 1u);
-                            if (m) q = kill_elements<DT>(q, m);
-                        }
+                for (int v0 = lo + (int)threadIdx.x; v0 - (int)threadIdx.x < hi; v0 += 4 * NT) {
+                    uint4 q[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) q[u] = load(v0 + u * NT);
+                    if (!__any_sync(0xFFFFFFFFu, test(q))) continue;
+#pragma unroll 1
+                    for (int u = 0; u < 4; ++u) {
+                        uint4 x = q[0];
+#pragma unroll
+                        for (int w = 1; w < 4; ++w) if (u == w) x = q[w];
+                        const int i0 = id_of(v0 + u * NT);
+                        f(masked(x, i0), i0);
                     }
-                    f(q, i0);
                 }
             } else {
-            auto fetch = [&](int u, int i0) -> uint4 {
-                uint4 q = VecTest<DT>::fill();
-                if (!after && (t * tv + u) * NT + (int)threadIdx.x < nvec) {
-                    q = stage[u * NT + threadIdx.x];
-                    if (bitmap) {
-                        const uint32_t m = __funnelshift_r(bitmap[i0 >> 5], bitmap[(i0 >> 5) + 1], i0 & 31) & ((1u << E::PER_VEC) - 1u);
-                        if (m) q = kill_elements<DT>(q, m);
-                    }
-                }
-                return q;
-            };
+                uint4 q[AHEAD];
+#pragma unroll
+                for (int u = 0; u < AHEAD; ++u) q[u] = load(lo + (int)threadIdx.x + u * NT);
 #pragma unroll 1
-            for (int u = 0; after || u < tv; u += PAIRS ? 2 : 1) {
-                const int i0 = after ? -1 : head + ((t * tv + u) * NT + (int)threadIdx.x) * E::PER_VEC;
-                if constexpr (PAIRS) {
-                    const int i1 = i0 + NT * E::PER_VEC;
-                    const uint4 q0 = fetch(u, i0), q1 = fetch(u + 1, i1);
-                    f(q0, q1, i0, i1);
-                } else {
-                    const uint4 q = fetch(u, i0);
-                    if constexpr (AFTER) { if (!f(q, i0) && after) break; } else f(q, i0);
-                }
-            }
-            }
-            __syncwarp();
-            if (after) break;
-            if ((threadIdx.x & 31) == 0) {
-                __threadfence_block();
-                if (atomicAdd(&r.done[st], 1u) == (uint32_t)(NWARPS - 1)) {
-                    r.done[st] = 0;
-                    __threadfence_block();
-                    if (t + nst < ntiles && *(volatile uint32_t *)&r.timeout == 0u) {
-                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                        issue(r, t + nst, st);
-                        atomicMax(&r.issued, (uint32_t)(t + nst + 1));
+                for (int v0 = lo + (int)threadIdx.x; v0 - (int)threadIdx.x < hi; v0 += AHEAD * NT) {
+#pragma unroll
+                    for (int u = 0; u < AHEAD; u += PAIRS ? 2 : 1) {
+                        const int v = v0 + u * NT, i0 = id_of(v);
+                        const uint4 x = masked(q[u], i0);
+                        q[u] = load(v + AHEAD * NT);
+                        if constexpr (PAIRS) {
+                            const int i1 = id_of(v + NT);
+                            const uint4 y = masked(q[u + 1], i1);
+                            q[u + 1] = load(v + (AHEAD + 1) * NT);
+                            f(x, y, i0, i1);
+                        } else f(x, i0);
                     }
                 }
             }
-            __syncwarp();
-            if (++st == nst) { st = 0; parity ^= 1u; }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            // (after an expired wait: the copies in flight land, or get as long again, before the CTA moves on)
-            if (r.timeout)
-                for (uint32_t t = r.issued > (uint32_t)nst ? r.issued - (uint32_t)nst : 0u; t < r.issued; ++t)
-                    mbar_wait(&r.bar[(first + t) % (uint32_t)nst], ((first + t) / (uint32_t)nst) & 1u);
-            r.tiles = first + (uint32_t)ntiles;
         }
         __syncthreads();
     }
@@ -296,19 +269,22 @@ struct SmemSlice {
     __device__ __forceinline__ int end_id() const { return id0 + nvec * E::PER_VEC; }
     __device__ __forceinline__ int elements() const { return nvec * E::PER_VEC; }
     __device__ __forceinline__ int segments() const { return block_scratch().seg_off; }      // (in a register it was spilled)
-    template <class F> __device__ __forceinline__ void vectors(F &&f) const {
+    __device__ __forceinline__ int count() const { return nvec; }
+    __device__ __forceinline__ uint4 vector(int v) const {
+        extern __shared__ __align__(128) unsigned char smem[];
+        return v < 0 ? VecTest<DT>::fill() : ((const uint4 *)(smem + vec_off))[v];
+    }
+    template <int AHEAD = 4, class F, class T = NoTest> __device__ __forceinline__ void vectors(F &&f, T && = T(), int first = 0, int end = 0x7FFFFFFF) const {
         extern __shared__ __align__(128) unsigned char smem[];
         const uint4 *vec = (const uint4 *)(smem + vec_off);
-        constexpr bool AFTER = goes_on<F>, PAIRS = by_pairs<F>;
+        constexpr bool PAIRS = by_pairs<F>;
+        const int n = min(nvec, end);
 #pragma unroll 1
-        for (int base = 0; AFTER || base < nvec; base += NT) {
-            const int v = base + (int)threadIdx.x, i0 = base < nvec ? id0 + v * E::PER_VEC : -1;
-            const uint4 q = v < nvec ? vec[v] : VecTest<DT>::fill();
-            bool more = false;
+        for (int base = first; base < n; base += NT) {
+            const int v = base + (int)threadIdx.x, i0 = id0 + v * E::PER_VEC;
+            const uint4 q = v < n ? vec[v] : VecTest<DT>::fill();
             if constexpr (PAIRS) f(q, VecTest<DT>::fill(), i0, -1);
-            else if constexpr (AFTER) more = f(q, i0);
             else f(q, i0);
-            if (AFTER && !more && base >= nvec) break;
         }
     }
     template <class F> __device__ __forceinline__ void extras(F &&f) const {
@@ -373,10 +349,9 @@ static_assert(W_LIST_ALONE * 8 <= WIDE_HIST_OFF, "the window's list alone lies o
 // pass, when it is done with, behind the lists.  What else they need (CountedSegs) lies where the kernel has room: in a cluster
 // over the tables of the history, of which only the scores are still wanted.
 constexpr int CT_BINS = 8192, CT_ODD = 254, CT_BYTES = CT_BINS * 4;
-constexpr int RACE_DIRECT = 13;       // so many of a warp's vectors at once are raced in place
-constexpr int RACE_QUEUE = 44;        // vectors that a warp's queue holds: 31 left over and RACE_DIRECT - 1
 constexpr int CT_QUEUE_OFF = WIDE_LIST_OFF + W_LIST * 8;
-static_assert(WIDE_BYTES <= CT_BYTES && CT_QUEUE_OFF + NWARPS * RACE_QUEUE * 20 <= CT_BYTES, "lists and queues in front of the team's words");
+constexpr int FINAL_QUEUE = (CT_BYTES - CT_QUEUE_OFF) / 2 / NT * NT;      // vectors that wait in the last pass, by their numbers (at most 2^16)
+static_assert(WIDE_BYTES <= CT_BYTES && ALBIREO_MAX_VOCAB / 8 <= 65536, "lists and queue in front of the team's words");
 // Where the cut and the list end, the same in every CTA.
 struct CountedCut {
     uint32_t thr_any, thr_win, thr_sure, thr_top;     // raw, packed twice: values from there on matter, are in the window or kept, are kept, are listed
@@ -384,9 +359,10 @@ struct CountedCut {
     uint32_t key_seg;                                 // extras above it are in M and n
     uint32_t key_top;
     u64 M; uint32_t n;                                // kept for sure, all but the extras above the window and not above key_seg
+    uint32_t n_any;                                   // no more elements of vectors than this are at or above thr_any (all ones: not known)
     uint32_t fail;                                    // (0 ahead of the counting pass: any thread may set it from there on)
 };
-struct CountedSegs {
+struct alignas(16) CountedSegs {
     u64 mass[NT];                     // by segments of 16 values; with no cut the list of the race (RACE_LIST) lies here
     uint32_t cnt[NT];
     uint32_t zeros[2];                // +0 and -0
@@ -402,10 +378,9 @@ __host__ __device__ constexpr int slice_off(bool counted) { return (team_off(cou
 template <bool COUNTED> __device__ __forceinline__ TeamWords &team_words() { extern __shared__ __align__(128) unsigned char smem[]; return *(TeamWords *)(smem + team_off(COUNTED)); }
 __host__ __device__ constexpr bool counts_rows(int dt) { return dt == ALBIREO_BF16; }      // the kernel of one CTA per row
 __host__ __device__ constexpr int row_off(int dt) { return slice_off(counts_rows(dt)) + (counts_rows(dt) ? (int)sizeof(CountedSegs) : 0); }
-__host__ __device__ constexpr int wide_ring_off(int dt) { return (row_off(dt) + (int)sizeof(RowShared) + 127) & ~127; }
+__host__ __device__ constexpr int row_front(int dt) { return (row_off(dt) + (int)sizeof(RowShared) + 127) & ~127; }      // what a wide row needs of one CTA
 template <int DT> __device__ __forceinline__ constexpr int row_segments() { return slice_off(counts_rows(DT)); }
 template <int DT> __device__ __forceinline__ RowShared &row_shared() { extern __shared__ __align__(128) unsigned char smem[]; return *(RowShared *)(smem + row_off(DT)); }
-template <int DT> __device__ __forceinline__ unsigned char *wide_stage(int st) { extern __shared__ __align__(128) unsigned char smem[]; return smem + wide_ring_off(DT) + st * WIDE_VEC_BYTES; }
 static_assert(sizeof(CountedSegs) % 16 == 0 && sizeof(RowShared) % 8 == 0, "what follows is aligned");
 __device__ __forceinline__ WideSmem wide_smem() {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -459,7 +434,7 @@ struct PassOut { u64 a, b; };
 template <int DT, int MODE, bool FLOOR>
 __device__ __noinline__ PassOut solo_mass_pass(float invT, float zmax, float zfloor, uint32_t lo, int shift) {
     PassOut o;
-    mass_pass<DT, MODE, FLOOR>(RingSlice<DT>(), invT, zmax, zfloor, lo, shift, o.a, o.b);
+    mass_pass<DT, MODE, FLOOR>(RowSlice<DT>(), invT, zmax, zfloor, lo, shift, o.a, o.b);
     return o;
 }
 
@@ -542,7 +517,7 @@ __device__ __forceinline__ void window_mass_pass(const SmemSlice<DT> &src, float
     mass_pass<DT, INSIDE_WINDOW, FLOOR>(src, invT, zmax, zfloor, lo, shift, ahead, all);
 }
 template <int DT, bool FLOOR>
-__device__ __forceinline__ void window_mass_pass(const RingSlice<DT> &, float invT, float zmax, float zfloor, uint32_t lo, int shift, u64 &ahead) {
+__device__ __forceinline__ void window_mass_pass(const RowSlice<DT> &, float invT, float zmax, float zfloor, uint32_t lo, int shift, u64 &ahead) {
     ahead = solo_mass_pass<DT, INSIDE_WINDOW, FLOOR>(invT, zmax, zfloor, lo, shift).a;
 }
 constexpr int TIE_SHIFT = 9;      // ids per bin when equal scores are told apart by them: 512 (2^19 ids at most: 1024 bins)
@@ -752,7 +727,7 @@ __device__ __forceinline__ void race_all(const SRC &src, BlockScratch &s, Partia
         if (f == sure && (uint32_t)i < fa.id_lo) { const float e = ex2_ftz(t2); S.add(e); ++n; race_one(i, z, e); }
         else if (f < win_hi || (f == win_hi && (uint32_t)i <= fa.id_hi)) list_append(fa.list, fa.list_cap, &s.list_cnt, z, i);
     };
-    src.vectors([&](const uint4 &q, int i0) {
+    src.template vectors<1>([&](const uint4 &q, int i0) {
         float e[PV], top = 0.0f;
         uint32_t at_edge = 0;
 #pragma unroll
@@ -953,7 +928,7 @@ __device__ __forceinline__ void race_all_shared(const SRC &src, BlockScratch &s,
         if (f < win_hi || (f == win_hi && (uint32_t)i <= fa.id_hi)) list_append(fa.list, fa.list_cap, &s.list_cnt, z, i);
         return false;
     };
-    src.vectors([&](const uint4 &q, int i0) {
+    src.template vectors<1>([&](const uint4 &q, int i0) {
         float e[PV], top = 0.0f;
         uint32_t at_edge = 0;
 #pragma unroll
@@ -1095,7 +1070,7 @@ __device__ __forceinline__ void final_pass(const SRC &src, BlockScratch &s, Part
                 push(i0 + x, __fmul_rn(pick_element<DT>(q, x), invT), bits != 0);
                 bits &= bits - 1u;
             }
-        });
+        }, [&](const uint4 (&q)[4]) { return VecTest<DT>::any_may_pass(q, thr, invT); });
     }
     src.extras([&](int i, float z) { push(i, z, z >= s.fa.zfloor); });
     work(0);
@@ -1107,13 +1082,13 @@ __device__ __forceinline__ void final_pass(const SRC &src, BlockScratch &s, Part
 template <int DT, int OFF, bool CUT>
 __device__ __noinline__ Partial solo_race_all() {
     Partial p;
-    race_all_shared<DT, OFF, CUT>(RingSlice<DT>(), block_scratch(), p);
+    race_all_shared<DT, OFF, CUT>(RowSlice<DT>(), block_scratch(), p);
     return p;
 }
 template <int DT>
 __device__ __noinline__ Partial solo_final_pass() {
     Partial p;
-    final_pass<DT>(RingSlice<DT>(), block_scratch(), p);
+    final_pass<DT>(RowSlice<DT>(), block_scratch(), p);
     return p;
 }
 template <int DT, bool FLOOR>
@@ -1121,7 +1096,7 @@ __device__ __forceinline__ void first_mass_pass(const SmemSlice<DT> &src, float 
     mass_pass<DT, FIRST_LEVEL, FLOOR>(src, invT, zmax, zfloor, F_ZERO, W_SHIFT, S, S_all);
 }
 template <int DT, bool FLOOR>
-__device__ __forceinline__ void first_mass_pass(const RingSlice<DT> &, float invT, float zmax, float zfloor, u64 &S, u64 &S_all) {
+__device__ __forceinline__ void first_mass_pass(const RowSlice<DT> &, float invT, float zmax, float zfloor, u64 &S, u64 &S_all) {
     const PassOut o = solo_mass_pass<DT, FIRST_LEVEL, FLOOR>(invT, zmax, zfloor, F_ZERO, W_SHIFT);
     S = o.a; S_all = o.b;
 }
@@ -1136,7 +1111,7 @@ __device__ __noinline__ Partial team_race_all(SmemSlice<DT> src) {
 template <int DT, int OFF, bool CUT>
 __device__ __forceinline__ void run_race_all(const SmemSlice<DT> &src, BlockScratch &s, Partial &p) { p = team_race_all<DT, OFF, CUT>(src); }
 template <int DT, int OFF, bool CUT>
-__device__ __forceinline__ void run_race_all(const RingSlice<DT> &, BlockScratch &s, Partial &p) { p = solo_race_all<DT, OFF, CUT>(); }
+__device__ __forceinline__ void run_race_all(const RowSlice<DT> &, BlockScratch &s, Partial &p) { p = solo_race_all<DT, OFF, CUT>(); }
 template <int DT, bool CUT, class SRC>
 __device__ __forceinline__ void run_race(const SRC &src, BlockScratch &s, Partial &p) {
     switch (src.first_id() & 3) {
@@ -1147,7 +1122,7 @@ __device__ __forceinline__ void run_race(const SRC &src, BlockScratch &s, Partia
     }
 }
 template <int DT> __device__ __forceinline__ void run_final_pass(const SmemSlice<DT> &src, BlockScratch &s, Partial &p) { final_pass<DT>(src, s, p); }
-template <int DT> __device__ __forceinline__ void run_final_pass(const RingSlice<DT> &, BlockScratch &s, Partial &p) { p = solo_final_pass<DT>(); }
+template <int DT> __device__ __forceinline__ void run_final_pass(const RowSlice<DT> &, BlockScratch &s, Partial &p) { p = solo_final_pass<DT>(); }
 
 // ------------------------------------------------------------------ one wide row
 
@@ -1192,6 +1167,44 @@ __device__ __noinline__ int list_sort(u64 *list, int n) {
         }
     }
     return P;
+}
+
+__device__ __forceinline__ bool all_keys_are(const u64 *list, int n, uint32_t key) {
+    bool same = true;
+    for (int i = threadIdx.x; i < n; i += NT) same &= (uint32_t)(list[i] >> 32) == key;
+    return same;
+}
+// The `want`-th lowest id of list[0..n), 1 <= want <= n <= W_LIST_ALONE, the same in every thread: ids counted in bins of 1024, and the entries of one bin by
+// their bits.  (16-bit logits far from zero have hundreds of elements at the score of the cut; sorted, 1250 of them took 20 us.)
+__device__ __noinline__ uint32_t lowest_ids(const u64 *list, int n, uint32_t want) {
+    BlockScratch &s = block_scratch();
+    uint32_t *bins = (uint32_t *)wide_smem().queue;      // NT bins, then 32 words of one bin's ids
+    static_assert(NT * 1024 >= ALBIREO_MAX_VOCAB && NWARPS * 64 * 8 >= (NT + 32) * 4, "a bin per thread, over the queues");
+    bins[threadIdx.x] = 0u;
+    if (threadIdx.x < 32) bins[NT + threadIdx.x] = 0u;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += NT) atomicAdd(&bins[(uint32_t)comp_idx(list[i]) >> 10], 1u);
+    __syncthreads();
+    const uint32_t mine = bins[threadIdx.x];
+    uint32_t tot;
+    const uint32_t ahead = block_exscan_u32(mine, tot);
+    if (ahead < want && want <= ahead + mine) { s.found_digit = threadIdx.x; s.found_cnt = want - ahead; }
+    __syncthreads();
+    const uint32_t bin = s.found_digit;
+    for (int i = threadIdx.x; i < n; i += NT) {
+        const uint32_t id = (uint32_t)comp_idx(list[i]);
+        if (id >> 10 == bin) atomicOr(&bins[NT + ((id >> 5) & 31u)], 1u << (id & 31u));
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const uint32_t w = bins[NT + threadIdx.x], c = __popc(w), k = s.found_cnt;
+        uint32_t inc = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, inc, o); if ((int)threadIdx.x >= o) inc += x; }
+        if (inc - c < k && k <= inc) s.list_cnt = (bin << 10) + (threadIdx.x << 5) + __fns(w, 0, (int)(k - (inc - c)));
+    }
+    __syncthreads();
+    return s.list_cnt;
 }
 
 // What the passes of a wide row leave behind, apart from each thread's sums and the lists.
@@ -1280,6 +1293,15 @@ __device__ __forceinline__ RowOut wide_finish_in(TEAM tm, float top_p, uint64_t 
                 if (part == 0 && ahead < target) keep(C, own);
             }
             reached = __syncthreads_or(reach >= target) != 0;
+        } else if (__syncthreads_and(all_keys_are(list, L, (uint32_t)(list[0] >> 32)))) {
+            // elements of one score: so many of the lowest ids are kept as are short of the target
+            const u64 each = mass_of(list[0]), want = each ? (target - p.M + each - 1) / each : 0ull;
+            reached = want > 0 && want <= (u64)L;
+            if (reached) {
+                const uint32_t last = lowest_ids(list, L, (uint32_t)want);
+                for (int q = threadIdx.x; q < L; q += NT) if ((uint32_t)comp_idx(list[q]) <= last) keep(list[q], each);
+            }
+            __syncthreads();
         } else {
             const int P = list_sort(list, L), per = (P + NT - 1) / NT, q0 = (int)threadIdx.x * per, q1 = min(L, q0 + per);
             u64 local = 0, tot;
@@ -1563,13 +1585,13 @@ __device__ __noinline__ void counting_pass(SRC src, float invT, float zref) {
     const int end = src.end_id();
     __nv_bfloat162 most = __halves2bfloat162(__ushort_as_bfloat16(0xFF80), __ushort_as_bfloat16(0xFF80));
     [[maybe_unused]] CountedRacer<LISTED> rc(s);
-    if constexpr (!RACE) src.vectors([&](const uint4 &q0, const uint4 &q1, int i0, int i1) {
+    if constexpr (!RACE) src.template vectors<4>([&](const uint4 &q0, const uint4 &q1, int i0, int i1) {
         const __nv_bfloat162 top0 = VecTest<ALBIREO_BF16>::vmax(q0), top1 = VecTest<ALBIREO_BF16>::vmax(q1);
         most = __hmax2(most, __hmax2(top0, top1));
         if (i0 < end) count_vector(src, q0, top0);
         if (i1 >= 0 && i1 < end) count_vector(src, q1, top1);
     });
-    else src.vectors([&](const uint4 &q, int i0) {
+    else src.template vectors<1>([&](const uint4 &q, int i0) {
         const __nv_bfloat162 top = VecTest<ALBIREO_BF16>::vmax(q);
         most = __hmax2(most, top);
         if (i0 < end) count_vector(src, q, top);
@@ -1654,9 +1676,8 @@ __device__ __forceinline__ uint32_t edge_mask(uint32_t w, uint32_t thr_win, uint
     return __hge2_mask(h, *reinterpret_cast<const H2 *>(&thr_win)) & ~__hge2_mask(h, *reinterpret_cast<const H2 *>(&thr_sure));
 }
 // Mass, number and lists of the extras, the race of all that is kept for sure, the window's elements to their list.
-// Vectors with nothing that matters are passed over; the others are worked on by full warps: where only few of a
-// warp's have something they wait in a queue.  (One vector of a thread at a time: with two, 52 to 160 bytes were spilled in this loop by the
-// kernel with 64 registers.)
+// Vectors with something that matters are listed by their number, and the list is worked off by all warps alike: where they lie close together (the head of a
+// vocabulary) they would else be a few warps' work.  Where there may be more of them than the list holds, so many vectors at a time.
 // (out of line: few vectors have any)
 __device__ __noinline__ void append_elements(uint4 q, int i0, uint32_t bits, float invT, bool listed) {
     BlockScratch &s = block_scratch();
@@ -1678,47 +1699,52 @@ __device__ __noinline__ Partial counted_final_pass(SRC src) {
     const WideSmem ws = wide_smem();
     // (worked out anew where they are used: held across the loop they were spilled)
     auto lane_now = [] { int l; asm volatile("mov.u32 %0, %%laneid;" : "=r"(l)); return l; };
-    auto warp_now = [] { int t; asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t)); return t >> 5; };
-    auto qvec = [&](int at) -> uint4 & { return ((uint4 *)(smem + CT_QUEUE_OFF))[warp_now() * RACE_QUEUE + at]; };
-    auto qid = [&](int at) -> int & { return ((int *)(smem + CT_QUEUE_OFF + NWARPS * RACE_QUEUE * 16))[warp_now() * RACE_QUEUE + at]; };
-    int qn = 0;                                        // the same in every lane
-    const uint32_t thr_any = cut.thr_any;
+    uint16_t *queue = (uint16_t *)(smem + CT_QUEUE_OFF);
     CountedRacer<SRC::SPARE_REGISTERS ? IN_REGS : IN_SHARED> rc(s);
-    src.vectors([&](const uint4 &q0, int i01) -> bool {
-        uint4 q = q0;
-        int i0 = i01;
-        bool waiting = i01 < 0;
-        if (!waiting) {
-            const bool in = T::may_pass(q, thr_any, 1.0f);
-            const uint32_t m = __ballot_sync(0xFFFFFFFFu, in);
-            if (m == 0) return true;
-            if (__popc(m) < RACE_DIRECT) {
-                if (in) { const int at = qn + __popc(m & ((1u << lane_now()) - 1u)); qvec(at) = q; qid(at) = i0; }
-                qn += __popc(m);
-                if (qn < 32) return true;
-                waiting = true;
-            }
-        } else if (qn == 0) return false;
-        if (waiting) {
-            const int cnt = qn < 32 ? qn : 32;
-            qn -= cnt;
-            __syncwarp();
-            q = T::fill();
-            i0 = 0;
-            const int lane = lane_now();
-            if (lane < cnt) { q = qvec(qn + lane); i0 = qid(qn + lane); }
-            __syncwarp();
+    const int chunk = cut.n_any <= (uint32_t)FINAL_QUEUE ? src.count() : FINAL_QUEUE;
+#pragma unroll 1
+    for (int c0 = 0; c0 < src.count(); c0 += chunk) {
+        if (c0 > 0) {
+            __syncthreads();
+            if (threadIdx.x == 0) s.runmax = 0;
+            __syncthreads();
         }
-        const volatile CountedCut &c = cut;
-        const float invT = *(const volatile float *)&s.fa.invT;
-        const uint32_t thr_sure = c.thr_sure, thr_win = c.thr_win;
-        const uint4 at_edge = make_uint4(edge_mask(q.x, thr_win, thr_sure), edge_mask(q.y, thr_win, thr_sure), edge_mask(q.z, thr_win, thr_sure), edge_mask(q.w, thr_win, thr_sure));
-        if (s.ga.num_top > 0) append_elements(q, i0, T::elem_bits(q, c.thr_top, invT), invT, true);
-        if (__any_sync(0xFFFFFFFFu, (at_edge.x | at_edge.y | at_edge.z | at_edge.w) != 0u))
-            append_elements(q, i0, T::elem_bits(q, thr_win, invT) & ~T::elem_bits(q, thr_sure, invT), invT, false);
-        race_vector<OFF>(rc, q, i0, T::vmax(q), __uint_as_float(thr_sure << 16), invT, *(const volatile float *)&s.fa.zmax);
-        return true;
-    });
+        {
+            const uint32_t thr_any = cut.thr_any;
+            const int first_id = src.first_id(), end = first_id + min(src.count(), c0 + chunk) * 8;
+            src.template vectors<4>([&](const uint4 &q, int i0) {
+                const bool in = T::may_pass(q, thr_any, 1.0f) && i0 < end;
+                const uint32_t m = __ballot_sync(0xFFFFFFFFu, in);
+                if (m == 0) return;
+                const int lane = lane_now();
+                uint32_t at = 0;
+                if (lane == 0) at = atomicAdd(&s.runmax, (uint32_t)__popc(m));
+                at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(m & ((1u << lane) - 1u));
+                if (in && at < (uint32_t)FINAL_QUEUE) queue[at] = (uint16_t)((uint32_t)(i0 - first_id) / 8u);
+            }, NoTest(), c0, c0 + chunk);
+        }
+        __syncthreads();
+        // (never more than there is room for, see n_any; else the row is given up)
+        const int n = (int)min(s.runmax, (uint32_t)FINAL_QUEUE);
+        if (s.runmax > (uint32_t)FINAL_QUEUE) s.list_cnt = 0x10000000u;
+        uint4 ahead = src.vector((int)threadIdx.x < n ? (int)queue[threadIdx.x] : -1);
+#pragma unroll 1
+        for (int at = (int)threadIdx.x, v = at < n ? (int)queue[at] : -1; at - lane_now() < n; at += NT) {
+            // (the next one is fetched while this one is worked on)
+            const uint4 q = ahead;
+            const int i0 = v < 0 ? 0 : src.first_id() + v * 8;
+            v = at + NT < n ? (int)queue[at + NT] : -1;
+            ahead = src.vector(v);
+            const volatile CountedCut &c = cut;
+            const float invT = *(const volatile float *)&s.fa.invT;
+            const uint32_t thr_sure = c.thr_sure, thr_win = c.thr_win;
+            const uint4 at_edge = make_uint4(edge_mask(q.x, thr_win, thr_sure), edge_mask(q.y, thr_win, thr_sure), edge_mask(q.z, thr_win, thr_sure), edge_mask(q.w, thr_win, thr_sure));
+            if (s.ga.num_top > 0) append_elements(q, i0, T::elem_bits(q, c.thr_top, invT), invT, true);
+            if (__any_sync(0xFFFFFFFFu, (at_edge.x | at_edge.y | at_edge.z | at_edge.w) != 0u))
+                append_elements(q, i0, T::elem_bits(q, thr_win, invT) & ~T::elem_bits(q, thr_sure, invT), invT, false);
+            race_vector<OFF>(rc, q, i0, T::vmax(q), __uint_as_float(thr_sure << 16), invT, *(const volatile float *)&s.fa.zmax);
+        }
+    }
     Partial p;
     p.M = 0; p.n = 0;
     const float zmax = s.fa.zmax;
@@ -1866,6 +1892,7 @@ __device__ __noinline__ bool counted_locate(SRC src, TEAM tm, float invT, float 
         // the cut: the window's values, and those above it
         const uint32_t n_all = __reduce_add_sync(0xFFFFFFFFu, wc);
         CountedCut c;
+        c.n_any = 0xFFFFFFFFu;
         c.M = S; c.n = n_all; c.key_lo = 0xFFFFFFFFu; c.key_hi = kfloor - 1u; c.key_seg = c.key_hi; c.fail = 0;
         c.thr_sure = c.thr_win = T::fill().x;             // (everything: -inf has no mass and does not win)
         if (minp && !topp) c.thr_sure = c.thr_win = T::raw_threshold(kfloor, invT);
@@ -1884,26 +1911,28 @@ __device__ __noinline__ bool counted_locate(SRC src, TEAM tm, float invT, float 
                 c.key_seg = seg == 0 ? 0xFFFFFFFFu : key_of(ct_score(ct_code(seg * CT_PER), invT));
                 c.thr_sure = (from_top ? 0x7F80u : ct_above(above)) * 0x10001u;
                 c.thr_win = e.hi < CT_PER ? ct_code(seg * CT_PER + e.hi) * 0x10001u : T::raw_threshold(c.key_lo, invT);
+                c.n_any = s.r32b[0] + e.cnt_most;
                 if (e.cnt_most - e.cnt_ahead > (uint32_t)list_cap) c.fail = 1u;
             }
         }
         if (lane == 0) {
             cut.M = c.M; cut.n = c.n; cut.key_lo = c.key_lo; cut.key_hi = c.key_hi; cut.key_seg = c.key_seg;
-            cut.thr_sure = c.thr_sure; cut.thr_win = c.thr_win; cut.fail = c.fail;
+            cut.thr_sure = c.thr_sure; cut.thr_win = c.thr_win; cut.n_any = c.n_any; cut.fail = c.fail;
         }
     } else if (wid == 1) {
         // the list: everything down to the value at which the wanted number is reached
-        uint32_t key_top = kfloor, fail = 0;
+        uint32_t key_top = kfloor, fail = 0, n_top = 0xFFFFFFFFu;
         if (listed && n_fin > (uint32_t)(W_LIST / 2)) {
             const int seg = (int)s.found_cnt;
             if (seg < 0) fail = !(minp || topp);         // (fewer than wanted: all that are kept)
             else {
                 const SegmentEnd e = end_in_segment(tm, seg, false, want - s.r32b[2], s.bcast[1], s.r32b[3], invT, zmax, zfloor);
                 key_top = max(ct_key_down_to(seg, e.hi, invT), kfloor);
-                if (s.r32b[2] + e.cnt_most > (uint32_t)W_LIST) fail = 1u;
+                n_top = s.r32b[2] + e.cnt_most;
+                if (n_top > (uint32_t)W_LIST) fail = 1u;
             }
         }
-        if (lane == 0) { cut.key_top = key_top; cut.thr_top = listed ? T::raw_threshold(key_top, invT) : 0u; s.r32b[8] = fail; }
+        if (lane == 0) { cut.key_top = key_top; cut.thr_top = listed ? T::raw_threshold(key_top, invT) : 0u; s.r32b[8] = fail; s.r32b[9] = n_top; }
     } else if (t == 64) {
         s.fa.invT = invT; s.fa.zmax = zmax; s.fa.list_cap = list_cap; s.fa.exp1_row = nullptr;
         s.fa.list = listed ? wide_smem().list : wide_smem().top;
@@ -1915,6 +1944,7 @@ __device__ __noinline__ bool counted_locate(SRC src, TEAM tm, float invT, float 
     if (t == 0) {
         const float win = __uint_as_float(cut.thr_win << 16), top = __uint_as_float(cut.thr_top << 16);
         cut.thr_any = listed && top < win ? cut.thr_top : cut.thr_win;
+        if (listed && top < win) cut.n_any = s.r32b[9];
     }
     __syncthreads();
     return true;
@@ -1961,7 +1991,7 @@ __device__ __noinline__ RowOut counted_row(SRC src, TEAM tm, const RowParams rp,
         }
     } else {
         if (t < tm.size) *tm.at(&tm.x->ncand[tm.rank], t) = cut.fail | (counted_segs(src).high ? 2u : 0u);       // (a barrier has ended the extras)
-        if (t == 0) { s.found_digit = 0xFFFFFFFFu; s.found_cnt = 0xFFFFFFFFu; s.list_cnt = 0; s.cand_cnt = 0; s.race.philox = philox_row(rp.seed, rp.R, s.ga.step); }
+        if (t == 0) { s.found_digit = 0xFFFFFFFFu; s.found_cnt = 0xFFFFFFFFu; s.list_cnt = 0; s.cand_cnt = 0; s.runmax = 0; s.race.philox = philox_row(rp.seed, rp.R, s.ga.step); }
         tm.sync();
         const uint32_t told = __reduce_or_sync(0xFFFFFFFFu, lane < tm.size ? tm.x->ncand[lane] : 0u);
         if ((told & 1u) || !counted_locate(src, tm, invT, zmax, kfloor, minp, rp.top_p, n_fin, list_cap, (told & 2u) != 0u)) { out.status |= ROW_NOT_COUNTED; return out; }
