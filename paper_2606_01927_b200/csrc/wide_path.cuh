@@ -1675,18 +1675,22 @@ __device__ __forceinline__ uint32_t edge_mask(uint32_t w, uint32_t thr_win, uint
     const H2 h = *reinterpret_cast<const H2 *>(&w);
     return __hge2_mask(h, *reinterpret_cast<const H2 *>(&thr_win)) & ~__hge2_mask(h, *reinterpret_cast<const H2 *>(&thr_sure));
 }
+// and the elements that they stand for
+__device__ __forceinline__ uint32_t edge_bits(uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
+    auto two = [](uint32_t m) { return (m & 1u) | ((m >> 15) & 2u); };
+    return two(x) | two(y) << 2 | two(z) << 4 | two(w) << 6;
+}
 // Mass, number and lists of the extras, the race of all that is kept for sure, the window's elements to their list.
-// Vectors with something that matters are listed by their number, and the list is worked off by all warps alike: where they lie close together (the head of a
-// vocabulary) they would else be a few warps' work.  Where there may be more of them than the list holds, so many vectors at a time.
+// Where few vectors have something that matters they are listed by their number, and the list is worked off by all warps alike: where they lie close together
+// (the head of a vocabulary) they would else be a few warps' work.  Where they may be more than the list holds every vector is worked on as it comes. (100 rows of 152064,
+// us of this pass, listed in parts and as they come: 49000 kept 53 and 37, 23000 43 and 35.)
 // (out of line: few vectors have any)
-__device__ __noinline__ void append_elements(uint4 q, int i0, uint32_t bits, float invT, bool listed) {
+__device__ __noinline__ void append_elements(uint4 q, int i0, uint32_t bits, float invT) {
     BlockScratch &s = block_scratch();
     while (bits) {
         const int x = __ffs(bits) - 1;
         bits &= bits - 1u;
-        const float z = __fmul_rn(pick_element<ALBIREO_BF16>(q, x), invT);
-        if (listed) list_append(wide_smem().top, W_LIST, &s.cand_cnt, z, i0 + x);
-        else list_append(s.fa.list, s.fa.list_cap, &s.list_cnt, z, i0 + x);
+        list_append(wide_smem().top, W_LIST, &s.cand_cnt, __fmul_rn(pick_element<ALBIREO_BF16>(q, x), invT), i0 + x);
     }
     __syncwarp();
 }
@@ -1701,17 +1705,24 @@ __device__ __noinline__ Partial counted_final_pass(SRC src) {
     auto lane_now = [] { int l; asm volatile("mov.u32 %0, %%laneid;" : "=r"(l)); return l; };
     uint16_t *queue = (uint16_t *)(smem + CT_QUEUE_OFF);
     CountedRacer<SRC::SPARE_REGISTERS ? IN_REGS : IN_SHARED> rc(s);
-    const int chunk = cut.n_any <= (uint32_t)FINAL_QUEUE ? src.count() : FINAL_QUEUE;
-#pragma unroll 1
-    for (int c0 = 0; c0 < src.count(); c0 += chunk) {
-        if (c0 > 0) {
-            __syncthreads();
-            if (threadIdx.x == 0) s.runmax = 0;
-            __syncthreads();
+    auto work = [&](const uint4 &q, int i0) {
+        const volatile CountedCut &c = cut;
+        const float invT = *(const volatile float *)&s.fa.invT;
+        const uint32_t thr_sure = c.thr_sure, thr_win = c.thr_win;
+        if (s.ga.num_top > 0) append_elements(q, i0, T::elem_bits(q, c.thr_top, invT), invT);
+        uint32_t in = edge_bits(edge_mask(q.x, thr_win, thr_sure), edge_mask(q.y, thr_win, thr_sure), edge_mask(q.z, thr_win, thr_sure), edge_mask(q.w, thr_win, thr_sure));
+        while (in) {
+            const int x = __ffs(in) - 1;
+            in &= in - 1u;
+            list_append(s.fa.list, s.fa.list_cap, &s.list_cnt, __fmul_rn(pick_element<ALBIREO_BF16>(q, x), invT), i0 + x);
         }
+        __syncwarp();
+        race_vector<OFF>(rc, q, i0, T::vmax(q), __uint_as_float(thr_sure << 16), invT, *(const volatile float *)&s.fa.zmax);
+    };
+    if (cut.n_any <= (uint32_t)FINAL_QUEUE) {
         {
             const uint32_t thr_any = cut.thr_any;
-            const int first_id = src.first_id(), end = first_id + min(src.count(), c0 + chunk) * 8;
+            const int first_id = src.first_id(), end = src.end_id();
             src.template vectors<4>([&](const uint4 &q, int i0) {
                 const bool in = T::may_pass(q, thr_any, 1.0f) && i0 < end;
                 const uint32_t m = __ballot_sync(0xFFFFFFFFu, in);
@@ -1721,7 +1732,7 @@ __device__ __noinline__ Partial counted_final_pass(SRC src) {
                 if (lane == 0) at = atomicAdd(&s.runmax, (uint32_t)__popc(m));
                 at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(m & ((1u << lane) - 1u));
                 if (in && at < (uint32_t)FINAL_QUEUE) queue[at] = (uint16_t)((uint32_t)(i0 - first_id) / 8u);
-            }, NoTest(), c0, c0 + chunk);
+            });
         }
         __syncthreads();
         // (never more than there is room for, see n_any; else the row is given up)
@@ -1735,16 +1746,9 @@ __device__ __noinline__ Partial counted_final_pass(SRC src) {
             const int i0 = v < 0 ? 0 : src.first_id() + v * 8;
             v = at + NT < n ? (int)queue[at + NT] : -1;
             ahead = src.vector(v);
-            const volatile CountedCut &c = cut;
-            const float invT = *(const volatile float *)&s.fa.invT;
-            const uint32_t thr_sure = c.thr_sure, thr_win = c.thr_win;
-            const uint4 at_edge = make_uint4(edge_mask(q.x, thr_win, thr_sure), edge_mask(q.y, thr_win, thr_sure), edge_mask(q.z, thr_win, thr_sure), edge_mask(q.w, thr_win, thr_sure));
-            if (s.ga.num_top > 0) append_elements(q, i0, T::elem_bits(q, c.thr_top, invT), invT, true);
-            if (__any_sync(0xFFFFFFFFu, (at_edge.x | at_edge.y | at_edge.z | at_edge.w) != 0u))
-                append_elements(q, i0, T::elem_bits(q, thr_win, invT) & ~T::elem_bits(q, thr_sure, invT), invT, false);
-            race_vector<OFF>(rc, q, i0, T::vmax(q), __uint_as_float(thr_sure << 16), invT, *(const volatile float *)&s.fa.zmax);
+            work(q, i0);
         }
-    }
+    } else src.template vectors<1>(work);
     Partial p;
     p.M = 0; p.n = 0;
     const float zmax = s.fa.zmax;
