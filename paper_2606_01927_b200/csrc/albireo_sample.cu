@@ -62,6 +62,7 @@ struct SampleArgs {
     int64_t row_stride;
     int32_t nseg;               // pieces per row (1: rows are contiguous)
     int32_t nstages;            // ring depth chosen by the host for this launch
+    int32_t hashed;             // whether there is room for a hash table of history ids (see build_hashed)
     int32_t vps;                // 16-byte vectors per piece (worked out on the host: no division on the device)
     int32_t Vs;                 // elements per piece
     uint32_t flags;
@@ -705,6 +706,45 @@ __device__ bool build_history(const HistSmem &hs, RowCtx &c, const int32_t *ids,
     __syncthreads();
     return true;
 }
+
+// The tables of the candidate path for a history of more than HASH_LEAST ids and at most HASH_IDS: the bitmap, and in the place of ranks and counts a hash table of ids and their
+// counts, filled in one sweep with one barrier behind it.  (Ranks need the finished bitmap, a prefix sum over it and a second sweep that looks each id's rank up word by
+// word: 256 rows of 128256 with 2048 ids each 34.8 us, hashed 33.6.)  A word is an id and, from bit 19 on, its count; an id seen in the prompt only has count 0.  Whoever puts an id in sets its bit.
+constexpr int HASH_SLOTS = 4096, HASH_IDS = HASH_SLOTS * 7 / 8, HASH_LEAST = 1024;
+constexpr uint32_t HASH_EMPTY = 0xFFFFFFFFu, HASH_ID = (1u << 19) - 1u;      // (no count reaches 2^13 - 1)
+static_assert(ALBIREO_MAX_VOCAB <= 1 << 19 && HASH_IDS < (1 << 13) - 1, "an id and a count in a word");
+// (Not in the kernels of fp32 rows: with the code for it 1024 of them with 1024 ids, which do not use it, took 136.0 us instead of 133.7.)
+__host__ __device__ constexpr bool hashes_history(int dt, bool extra) { return dt != ALBIREO_F32 && !extra; }
+__host__ __device__ constexpr int hash_off(int V) { return ((((V + 31) >> 5) + 1) + 3) & ~3; }      // words from the bitmap to the hash table
+__device__ __forceinline__ void build_hashed(uint32_t *bitmap, RowCtx &c, const int32_t *ids, int len, int out_start, const int32_t *staged) {
+    const int V = c.V, nwords = (V + 31) >> 5, nst = len < HIST_STAGED ? len : HIST_STAGED;
+    uint32_t *slots = bitmap + hash_off(V);
+    for (int w = threadIdx.x; w <= nwords; w += NT) bitmap[w] = 0;
+#pragma unroll
+    for (int i = 0; i < HASH_SLOTS / 4 / NT; ++i) ((uint4 *)slots)[i * NT + threadIdx.x] = make_uint4(HASH_EMPTY, HASH_EMPTY, HASH_EMPTY, HASH_EMPTY);
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+#pragma unroll 1
+    for (int j = threadIdx.x; j < len; j += NT) {
+        const int t = j < nst ? staged[j] : __ldg(ids + j);
+        if (t < 0 || t >= V) continue;
+        const uint32_t once = j >= out_start ? 1u << 19 : 0u;
+        uint32_t h = ((uint32_t)t * 0x9E3779B1u) >> 20;
+#pragma unroll 1
+        for (int it = 0; it < HASH_SLOTS; ++it) {
+            uint32_t cur = *(volatile uint32_t *)&slots[h];
+            if (cur == HASH_EMPTY) {
+                cur = atomicCAS(&slots[h], HASH_EMPTY, (uint32_t)t | once);
+                if (cur == HASH_EMPTY) { atomicOr(&bitmap[t >> 5], 1u << (t & 31)); break; }
+            }
+            if ((cur & HASH_ID) == (uint32_t)t) { if (once) atomicAdd(&slots[h], once); break; }
+            h = (h + 1u) & (uint32_t)(HASH_SLOTS - 1);
+        }
+    }
+    __syncthreads();
+    c.has_hist = true; c.bitmap = bitmap; c.coarse = nullptr; c.counts = slots; c.n_distinct = 0; c.ncoarse = 0;
+}
+static_assert(HASH_SLOTS == 1 << 12, "the upper 12 bits of the hash");
 
 // token id of the r-th distinct history id (r < n_distinct), i.e. the r-th set bit of the bitmap
 __device__ int hist_id_of_rank(const RowCtx &c, uint32_t r) {
@@ -2131,7 +2171,23 @@ __device__ __forceinline__ bool candidate_path(BlockScratch &s, const CandSmem &
     // penalised tokens, straight from the history tables: one distinct id per thread and round,
     // so that a dense head of the vocabulary does not pile up on a few threads; four rounds at a
     // time, so that their scattered loads (a round trip each, behind the other rows' streams) overlap
-    if (c.has_hist) {
+    if (hashes_history(DT, EXTRA) && c.has_hist && !c.coarse) {
+        constexpr int PG = 4;
+#pragma unroll 1
+        for (int at = (int)threadIdx.x; at < HASH_SLOTS; at += PG * NT) {
+            uint32_t w[PG]; float x[PG];
+#pragma unroll
+            for (int u = 0; u < PG; ++u) w[u] = c.counts[at + u * NT];
+#pragma unroll
+            for (int u = 0; u < PG; ++u) x[u] = w[u] != HASH_EMPTY ? E::load(elem_ptr<DT>(c, (int)(w[u] & HASH_ID)), 0) : 0.0f;
+#pragma unroll
+            for (int u = 0; u < PG; ++u) {
+                if (w[u] == HASH_EMPTY) continue;
+                const uint32_t key = key_of(__fmul_rn(penalise_counted(c, x[u], w[u] >> 19), c.invT));
+                if (key >= tau_key) cand_append_one(s, cs, comp_of(key, (int)(w[u] & HASH_ID)));
+            }
+        }
+    } else if (c.has_hist) {
         constexpr int PG = 4;
         for (uint32_t r0 = threadIdx.x; r0 < c.n_distinct; r0 += PG * NT) {
             int id[PG]; float x[PG];
@@ -2524,8 +2580,14 @@ __device__ __forceinline__ void one_row(const SampleArgs &a, const int b) {
             hs.bitmap = (uint32_t *)(smem + tab_off);
             hs.coarse = hs.bitmap + (nwords + 1);
             hs.counts = hs.coarse + (ncoarse + 1);
-            c.has_hist = build_history(hs, c, a.hist_ids + o0, o1 - o0, ostart, (const int32_t *)smem, a.ws_counts, a.ws_counts_cap, (int64_t)o0);
-            if (!c.has_hist) out.status |= ALBIREO_ROW_HISTORY_OVERFLOW;
+            // (a history that could have more distinct ids than the other tables hold, and more than the workspace does, is theirs to refuse)
+            const int len = o1 - o0;
+            if (hashes_history(DT, EXTRA) && a.hashed && len > HASH_LEAST && len <= HASH_IDS && (len <= CNT_CAP || (a.ws_counts && o0 >= 0 && (int64_t)o1 <= a.ws_counts_cap)))
+                build_hashed(hs.bitmap, c, a.hist_ids + o0, len, ostart, (const int32_t *)smem);
+            else {
+                c.has_hist = build_history(hs, c, a.hist_ids + o0, len, ostart, (const int32_t *)smem, a.ws_counts, a.ws_counts_cap, (int64_t)o0);
+                if (!c.has_hist) out.status |= ALBIREO_ROW_HISTORY_OVERFLOW;
+            }
         }
         __syncthreads();
         CandSmem cs;
@@ -2642,6 +2704,7 @@ __global__ void __launch_bounds__(NT, 2) albireo_stream_only_kernel(const void *
     if (threadIdx.x == 0) sink[blockIdx.x] = hits + (dead << 31);
 }
 
+constexpr int SM_SMEM = 233472;         // shared memory of an SM
 size_t history_smem_bytes(int V) {
     size_t nwords = ((size_t)V + 31) / 32, ncoarse = (nwords + 7) / 8;
     return (nwords + 1 + ncoarse + 1 + CNT_CAP) * 4;
@@ -2650,7 +2713,7 @@ size_t history_smem_bytes(int V) {
 // batch with no more rows than the device has SMs (`alone`: every CTA has an SM to itself), as deep as
 // one CTA's share allows
 int ring_stages_for(int V, bool with_history, bool alone) {
-    const long budget = (alone ? 233472 - 1024 : 233472 / 2 - 1024) - 1536;      // per CTA: dynamic bytes available (1 KiB reserved, 1.5 KiB static)
+    const long budget = (alone ? SM_SMEM - 1024 : SM_SMEM / 2 - 1024) - 1536;      // per CTA: dynamic bytes available (1 KiB reserved, 1.5 KiB static)
     long fixed = COMMON_BYTES + MAX_STAGES * 8 + (with_history ? (long)history_smem_bytes(V) : 0);
     long n = (budget - fixed) / STAGE_BYTES;
     const long cap = alone ? 6 : 4;
@@ -2726,7 +2789,7 @@ int apply_ext(SampleArgs &a, const albireo_sample_ext_t *ext, int B, int V, cons
 }
 
 // The launch shape of a batch: a CTA per row (team 1, ring of nstages), or a cluster of `team` CTAs per row.
-struct LaunchShape { int team, nstages, slice_bytes, list_words; size_t smem; bool counted, ordered; };
+struct LaunchShape { int team, nstages, slice_bytes, list_words; size_t smem; bool counted, ordered, hashed; };
 
 // What the launch shape depends on: the device's SMs, the dynamic shared memory a CTA may have, and how many
 // clusters of 2^i CTAs (one per SM) are on the device at once.
@@ -2766,7 +2829,7 @@ bool pick_team(LaunchShape &ls, int B, int V, int dtype, bool with_history, bool
             if (general > smem) smem = general;
             if (smem > (long)d.max_smem) continue;
             ls.counted = counted != 0;
-            ls.ordered = false; ls.team = team; ls.slice_bytes = (int)slice; ls.list_words = (int)list; ls.smem = (size_t)smem; ls.nstages = 0;
+            ls.ordered = false; ls.hashed = false; ls.team = team; ls.slice_bytes = (int)slice; ls.list_words = (int)list; ls.smem = (size_t)smem; ls.nstages = 0;
             return true;
         }
     }
@@ -2793,6 +2856,11 @@ bool pick_shape(LaunchShape &ls, int V, int dtype, const SampleArgs &a, const De
     ls.nstages = ring_stages_for(V, with_history, B <= d.num_sms);
     ls.smem = smem_bytes_for(V, with_history, ls.nstages);
     while (ls.smem > d.max_smem && ls.nstages > 2) ls.smem = smem_bytes_for(V, with_history, --ls.nstages);
+    // (where the hash table costs neither a stage of the ring nor the second CTA of an SM: up to vocabularies of 179000 tokens)
+    const size_t hashed = smem_bytes_for(V, false, ls.nstages) + (size_t)(hash_off(V) + HASH_SLOTS) * 4;
+    const size_t budget = (size_t)(B <= d.num_sms ? SM_SMEM : SM_SMEM / 2) - 1024 - 1536;
+    ls.hashed = with_history && hashes_history(dtype, extras_asked(a)) && hashed <= budget && hashed <= d.max_smem;
+    if (ls.hashed && hashed > ls.smem) ls.smem = (hashed + 127) & ~(size_t)127;
     return ls.smem <= d.max_smem;
 }
 
@@ -2821,7 +2889,7 @@ cudaError_t launch_sample_kernel_as(int B, const LaunchShape &ls, cudaStream_t s
            : ls.ordered ? cudaLaunchKernelEx(&cfg, albireo_ordered_sample_kernel<DT>, a) : cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT, false>, a);
 }
 cudaError_t launch_sample_kernel(int dtype, int B, const LaunchShape &ls, cudaStream_t st, SampleArgs &a) {
-    a.nstages = ls.nstages; a.slice_bytes = ls.slice_bytes; a.list_words = ls.list_words;
+    a.nstages = ls.nstages; a.hashed = ls.hashed; a.slice_bytes = ls.slice_bytes; a.list_words = ls.list_words;
     if (dtype == ALBIREO_F32) return launch_sample_kernel_as<ALBIREO_F32>(B, ls, st, a);
     if (dtype == ALBIREO_BF16) return launch_sample_kernel_as<ALBIREO_BF16>(B, ls, st, a);
     return launch_sample_kernel_as<ALBIREO_F16>(B, ls, st, a);
