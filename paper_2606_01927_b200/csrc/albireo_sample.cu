@@ -2538,7 +2538,7 @@ __device__ __forceinline__ void one_row(const SampleArgs &a, const int b) {
             const int row = row_of_cta(order, a.B, V);          // (its barrier: s.issued is visible)
             if (row != b) {
                 asm volatile("cp.async.wait_all;" ::: "memory");
-                mbar_wait(&rg.bar[MAX_STAGES - 1], 0u);
+                if (s.issued) mbar_wait(&rg.bar[MAX_STAGES - 1], 0u);      // (no copies: nothing arrives there)
                 for (int t = 0; t < (int)s.issued; ++t) mbar_wait(&rg.bar[t], 0u);
                 __syncthreads();
                 if (threadIdx.x == 0) {
@@ -2602,8 +2602,9 @@ __device__ __forceinline__ void one_row(const SampleArgs &a, const int b) {
         asm volatile("cp.async.wait_all;" ::: "memory");        // (the prefetched history ids)
         __syncthreads();                                        // s.issued is visible
         if (ring_started) {
-            bool landed = mbar_wait(&rg.bar[MAX_STAGES - 1], 0u);
-            for (int t = 0; t < (int)s.issued; ++t) landed = mbar_wait(&rg.bar[t], 0u) && landed;
+            const int issued = (int)s.issued;                   // (a row without a whole aligned vector has no copies: nothing arrives on the first one's barrier)
+            bool landed = issued == 0 || mbar_wait(&rg.bar[MAX_STAGES - 1], 0u);
+            for (int t = 0; t < issued; ++t) landed = mbar_wait(&rg.bar[t], 0u) && landed;
             if (__syncthreads_or(!landed)) { out.status |= ALBIREO_ROW_TIMEOUT; out.token = -1; out.logprob = __uint_as_float(0x7FC00000u); done = true; }   // the same in every thread
         }
     }

@@ -1,6 +1,7 @@
 """Passes of one CTA over a row in global memory, and the end of a cut among equal scores: row lengths around whole rounds of the passes' loads, rows in pieces,
 kept sets of more vectors than wait in the last pass at a time, hundreds of elements at the score of the cut, against the oracle."""
 import os
+from contextlib import closing
 
 import numpy as np
 import pytest
@@ -9,7 +10,7 @@ import torch
 from oracle import albireo_oracle as O
 from paper_2606_01927_b200 import workloads as W
 
-from parity import compare, to_host
+from parity import compare, compare_top_lists, to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -55,3 +56,25 @@ def test_wide_rows(binding, sampler, B, V, pieces, dtype, history):
     g = to_host(sampler.albireo_sample(lg, **t, want_counts=True, want_status=True))
     rep = compare(w, g, ref)
     assert rep.ok() and len(rep.excused) <= 1, (rep.summary(), rep.failures[:3], rep.excused[:3])
+
+
+# Rows so short that some or all of them have no whole aligned vector of 16 bytes (and rows of one vector and two among them): nothing is copied for
+# those.  1 and 80 rows are on the device at once, 300 are not.
+@pytest.mark.parametrize("V", [1, 2, 3, 7, 9, 14, 15, 17])
+@pytest.mark.parametrize("dtype", [W.BF16, W.F16, W.F32])
+@pytest.mark.parametrize("history,num_top", [(False, 0), (True, 0), (False, 3)])
+def test_rows_without_a_whole_vector(binding, dtype, V, history, num_top):
+    with closing(binding.Sampler(max_rows=300, max_vocab=32, max_history_total=1 << 16)) as sampler:
+        for B in (1, 80, 300):
+            base = W.random_small(2000 + 16 * B + V, B=B, V=V, dtype=W.F32 if dtype == W.F16 else dtype, with_history=history)
+            if B == 1:
+                base.temperature[:], base.top_k[:], base.top_p[:] = 0.9, 0, 0.8
+            base.num_top = num_top
+            w = W.as_f16(base) if dtype == W.F16 else base
+            ref = O.sample(w, threads=_CORES)
+            t = binding.workload_tensors(w, sampler.device)
+            g = to_host(sampler.albireo_sample(t.pop("logits"), **t, num_top=num_top, want_status=True))
+            rep = compare(w, g, ref)
+            assert rep.ok() and not rep.excused, (B, rep.summary(), rep.failures[:3], rep.excused[:3])
+            assert not (g["row_status"] & binding.ROW_TIMEOUT).any(), B
+            assert not compare_top_lists(w, g, ref), B
