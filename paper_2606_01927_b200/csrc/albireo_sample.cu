@@ -2296,10 +2296,10 @@ __device__ __forceinline__ void store_row(const SampleArgs &a, int b, RowOut &ou
 
 // The row's context with the history tables of this CTA's row, at tab_off (no copy is in flight, the front of the shared memory is free);
 // without (has_hist) where there is no history, or no room for them.
-__device__ __noinline__ RowCtx row_history(const SampleArgs *ap, int b, int tab_off, RowCtx c) {
+__device__ __noinline__ RowCtx row_history(const SampleArgs *ap, int tab_off, RowCtx c) {
     extern __shared__ __align__(128) unsigned char smem[];
     const SampleArgs &a = *ap;
-    const int o0 = a.hist_off[b], o1 = a.hist_off[b + 1];
+    const int b = blockIdx.x, o0 = a.hist_off[b], o1 = a.hist_off[b + 1];
     if (o1 <= o0) return c;
     HistSmem hs;
     const int nwords = (a.V + 31) >> 5, ncoarse = (nwords + 7) >> 3;
@@ -2319,15 +2319,16 @@ __device__ __noinline__ RowCtx row_history(const SampleArgs *ap, int b, int tab_
 // (Called with the streaming path's structures by value, it cost the metric workload 2 to 4 us of 20.)
 // tab_off: where the history tables lie; no copy is in flight.
 template <int DT>
-__device__ __noinline__ void leftover_row(const SampleArgs *ap, int b, int tab_off) {
+__device__ __noinline__ void leftover_row(const SampleArgs *ap, int tab_off) {
     extern __shared__ __align__(128) unsigned char smem[];
     BlockScratch &s = block_scratch();
     const SampleArgs &a = *ap;
+    const int b = blockIdx.x;
     RowParams rp;
     RowCtx c;
     uint32_t status = load_row<DT>(a, b, s.seg_base, rp, c);
     if (a.hist_ids && a.hist_off) {
-        c = row_history(ap, b, tab_off, c);
+        c = row_history(ap, tab_off, c);
         if (!c.has_hist && a.hist_off[b + 1] > a.hist_off[b]) status |= ALBIREO_ROW_HISTORY_OVERFLOW;
     }
     __syncthreads();
@@ -2418,60 +2419,17 @@ __device__ __noinline__ void leftover_row(const SampleArgs *ap, int b, int tab_o
 
 // ------------------------------------------------------------------ the kernel
 
-// Which row this CTA takes in a batch of more rows than are on the device at once, where some may be wide and others not: the wide ones first, otherwise in
-// their order, within 1024 rows.  A wide row takes 40 to 120 us and the others 20: handed out as they come the last wide ones began when the
-// first rows had ended, and the rows of one kind could meet on one SM (CTAs of the first round 148 apart): 512 mixed rows of 152064
-// with histories 141.3 us as they come, 137.7 so (122 and 125 to 128, by the inputs, with the last pass of dense kept sets as it is now).
-// Min-p rows without a top-k count as wide where the floor lies more than 5 below the maximum (in units of the score before its temperature): such rows mostly outgrow
-// the candidate list.  The parameters are looked at while the row's first tiles are on their way; a row that is another CTA's then costs those.  Contains a barrier.
-constexpr int ORDER_ROWS = 1024;
-// (what that is decided by, of this thread's two rows: asked for ahead of the row's copies, looked at when they have all had their latency)
-struct OrderWords { float T[ORDER_ROWS / NT], m[ORDER_ROWS / NT]; int k[ORDER_ROWS / NT]; };
-__device__ __forceinline__ OrderWords order_words(const SampleArgs &a) {
-    OrderWords o;
-    const int base = (int)blockIdx.x & ~(ORDER_ROWS - 1), n = min(ORDER_ROWS, a.B - base);
-#pragma unroll
-    for (int u = 0; u < ORDER_ROWS / NT; ++u) {
-        const int x = base + min(u * NT + (int)threadIdx.x, n - 1);
-        o.T[u] = a.temperature ? a.temperature[x] : 1.0f; o.k[u] = a.top_k ? a.top_k[x] : 0; o.m[u] = a.min_p ? a.min_p[x] : 0.0f;
-    }
-    return o;
-}
-__device__ __noinline__ int row_of_cta(OrderWords o, int B, int V) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    uint32_t *wide_rows = (uint32_t *)(smem + CAND_CAP * 8);       // (the select bins' place)
-    const int lane = threadIdx.x & 31, base = (int)blockIdx.x & ~(ORDER_ROWS - 1), n = min(ORDER_ROWS, B - base);
-    uint32_t any = 0;
-#pragma unroll
-    for (int u = 0; u < ORDER_ROWS / NT; ++u) {
-        const bool wide = u * NT + (int)threadIdx.x < n && o.T[u] > 0.0f && !(o.k[u] >= 1 && o.k[u] < V) && !(o.m[u] > 0.0f && o.T[u] * -__logf(o.m[u]) < 5.0f);
-        const uint32_t w = __ballot_sync(0xFFFFFFFFu, wide);
-        if (lane == 0) wide_rows[(u * NT + (int)threadIdx.x) >> 5] = w;
-        any |= w;
-    }
-    if (!__syncthreads_or(any != 0u)) return (int)blockIdx.x;
-    // Of the CTAs that come first, as many as there are wide rows, those with another row change it for the wide ones of later CTAs; all others keep theirs.
-    const uint32_t w = wide_rows[lane];
-    const int total = (int)__reduce_add_sync(0xFFFFFFFFu, (uint32_t)__popc(w)), j = (int)blockIdx.x - base;
-    auto below = [&](int limit) { const int m = limit - 32 * lane; return m >= 32 ? 0xFFFFFFFFu : m > 0 ? (1u << m) - 1u : 0u; };      // this lane's rows below `limit`
-    const uint32_t early_other = ~w & below(total), late_wide = w & ~below(total);
-    const uint32_t mine = j < total ? early_other : late_wide, theirs = j < total ? late_wide : early_other;
-    const uint32_t own = __shfl_sync(0xFFFFFFFFu, mine, j >> 5);
-    if (!((own >> (j & 31)) & 1u)) return (int)blockIdx.x;
-    const int rank = (int)__reduce_add_sync(0xFFFFFFFFu, (uint32_t)__popc(mine & below(j)));
-    const int c = __popc(theirs), ahead = (int)warp_incl_scan_u32((uint32_t)c) - c;
-    const bool here = ahead <= rank && rank < ahead + c;
-    const int row = here ? base + 32 * lane + (int)__fns(theirs, 0, rank - ahead + 1) : 0;
-    return __shfl_sync(0xFFFFFFFFu, row, __ffs(__ballot_sync(0xFFFFFFFFu, here)) - 1);
-}
-
-template <int DT> __device__ __noinline__ void moved_row(const SampleArgs *ap, int b);
-enum RowStart { OWN, ORDERED, MOVED };
-// ORDERED: the row may turn out to be another one (see row_of_cta). MOVED: by a CTA that has begun with another one; nothing of that is left, and no copies are in flight.
-template <int DT, bool EXTRA, RowStart START>
-__device__ __forceinline__ void one_row(const SampleArgs &a, const int b) {
+// dynamic shared memory layout (bytes): [candidates (8 KiB) + 512 select bins (2 KiB)]
+// [ring: nstages x 32 KiB][mbarriers][bitmap][coarse][counts]; the general path lays its histograms,
+// gather list and search bins (8 + 24 + 16 + 4 KiB) over the first 52 KiB, which it may do because
+// the ring is idle by then
+// EXTRA: whether the call asks for something beyond the ordinary (see extras_asked); the ordinary calls'
+// kernel is without the code for it, which would cost it registers.
+template <int DT, bool EXTRA>
+__global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const __grid_constant__ SampleArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     BlockScratch &s = block_scratch();
+    const int b = blockIdx.x;
     const int V = a.V;
 
     Ring rg;
@@ -2487,7 +2445,7 @@ __device__ __forceinline__ void one_row(const SampleArgs &a, const int b) {
     // (Programmatic dependent launch.)  The CTA may have been scheduled while the kernel ahead in the
     // stream (the producer of the logits) was still running: everything above touched only launch
     // arguments and shared memory; nothing below is read or written before that kernel has finished.
-    if (START != MOVED) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     // The row's own parameters and the first part of its history are asked for before the ring is started: a
     // load issued after the ring's copies (this CTA's and every other's) queues behind megabytes of
     // them; issued before, it is back within an idle round trip, while thread 0 is still setting up.
@@ -2496,8 +2454,6 @@ __device__ __forceinline__ void one_row(const SampleArgs &a, const int b) {
     // reading a dozen more launch arguments first would hold the ring back for nothing.
     RowParams rp;
     RowCtx c;
-    [[maybe_unused]] OrderWords order;
-    if constexpr (START == ORDERED) order = order_words(a);
     int o0 = 0, o1 = 0, ostart = 0;
     const bool with_hist = a.hist_ids && a.hist_off;
     auto load_params = [&]() {
@@ -2533,24 +2489,6 @@ __device__ __forceinline__ void one_row(const SampleArgs &a, const int b) {
     }
     if (ring_started) candidate_begin<DT>(rg, c);
     if (!with_hist) load_params();
-    if constexpr (START == ORDERED) {
-        {
-            const int row = row_of_cta(order, a.B, V);          // (its barrier: s.issued is visible)
-            if (row != b) {
-                asm volatile("cp.async.wait_all;" ::: "memory");
-                if (s.issued) mbar_wait(&rg.bar[MAX_STAGES - 1], 0u);      // (no copies: nothing arrives there)
-                for (int t = 0; t < (int)s.issued; ++t) mbar_wait(&rg.bar[t], 0u);
-                __syncthreads();
-                if (threadIdx.x == 0) {
-                    for (int st = 0; st < rg.nstages; ++st) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(&rg.bar[st])) : "memory");
-                    asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(&rg.bar[MAX_STAGES - 1])) : "memory");
-                }
-                __syncthreads();
-                moved_row<DT>(&a, row);
-                return;
-            }
-        }
-    }
 
     rp.greedy = !(rp.T > 0.0f);
     rp.ln_min_p = (!rp.greedy && rp.min_p > 0.0f) ? log((double)rp.min_p) : 0.0;
@@ -2610,14 +2548,8 @@ __device__ __forceinline__ void one_row(const SampleArgs &a, const int b) {
     }
     if (done) { store_row(a, b, out); return; }
     __syncthreads();
-    leftover_row<DT>(&a, b, tab_off);
+    leftover_row<DT>(&a, tab_off);
 }
-template <int DT> __device__ __noinline__ void moved_row(const SampleArgs *ap, int b) { one_row<DT, false, MOVED>(*ap, b); }
-template <int DT, bool EXTRA>
-__global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const __grid_constant__ SampleArgs a) { one_row<DT, EXTRA, OWN>(a, (int)blockIdx.x); }
-// (a kernel of its own: with the code for it the ordinary one spilled, 256 rows 19.4 -> 19.6 us)
-template <int DT>
-__global__ void __launch_bounds__(NT, 2) albireo_ordered_sample_kernel(const __grid_constant__ SampleArgs a) { one_row<DT, false, ORDERED>(a, (int)blockIdx.x); }
 
 #include "cluster_kernel.cuh"
 
@@ -2790,7 +2722,7 @@ int apply_ext(SampleArgs &a, const albireo_sample_ext_t *ext, int B, int V, cons
 }
 
 // The launch shape of a batch: a CTA per row (team 1, ring of nstages), or a cluster of `team` CTAs per row.
-struct LaunchShape { int team, nstages, slice_bytes, list_words; size_t smem; bool counted, ordered, hashed; };
+struct LaunchShape { int team, nstages, slice_bytes, list_words; size_t smem; bool counted, hashed; };
 
 // What the launch shape depends on: the device's SMs, the dynamic shared memory a CTA may have, and how many
 // clusters of 2^i CTAs (one per SM) are on the device at once.
@@ -2830,7 +2762,7 @@ bool pick_team(LaunchShape &ls, int B, int V, int dtype, bool with_history, bool
             if (general > smem) smem = general;
             if (smem > (long)d.max_smem) continue;
             ls.counted = counted != 0;
-            ls.ordered = false; ls.hashed = false; ls.team = team; ls.slice_bytes = (int)slice; ls.list_words = (int)list; ls.smem = (size_t)smem; ls.nstages = 0;
+            ls.hashed = false; ls.team = team; ls.slice_bytes = (int)slice; ls.list_words = (int)list; ls.smem = (size_t)smem; ls.nstages = 0;
             return true;
         }
     }
@@ -2851,9 +2783,6 @@ bool pick_shape(LaunchShape &ls, int V, int dtype, const SampleArgs &a, const De
     const bool with_history = a.hist_ids != nullptr;
     if (!(a.flags & ALBIREO_FLAG_FORCE_GENERAL) && pick_team(ls, B, V, dtype, with_history, may_count_rows(a), d)) return true;
     ls.team = 1; ls.slice_bytes = 0; ls.list_words = 0; ls.counted = false;
-    // (Where rows of both kinds can be.  With still more rows the last ones weigh less, and the look at the parameters costs every row: 1024 rows of fp32, all with a
-    // top-k, 137.0 us instead of 131.)
-    ls.ordered = B > 2 * d.num_sms && B <= 4 * d.num_sms && (a.top_k || a.min_p) && !extras_asked(a);
     ls.nstages = ring_stages_for(V, with_history, B <= d.num_sms);
     ls.smem = smem_bytes_for(V, with_history, ls.nstages);
     while (ls.smem > d.max_smem && ls.nstages > 2) ls.smem = smem_bytes_for(V, with_history, --ls.nstages);
@@ -2886,8 +2815,7 @@ cudaError_t launch_sample_kernel_as(int B, const LaunchShape &ls, cudaStream_t s
     cfg.attrs = at; cfg.numAttrs = n;
     if constexpr (DT == ALBIREO_BF16) { if (ls.counted) return cudaLaunchKernelEx(&cfg, albireo_cluster_kernel<DT, true>, a); }
     return ls.team > 1 ? cudaLaunchKernelEx(&cfg, albireo_cluster_kernel<DT, false>, a)
-           : extras_asked(a) ? cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT, true>, a)
-           : ls.ordered ? cudaLaunchKernelEx(&cfg, albireo_ordered_sample_kernel<DT>, a) : cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT, false>, a);
+           : extras_asked(a) ? cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT, true>, a) : cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT, false>, a);
 }
 cudaError_t launch_sample_kernel(int dtype, int B, const LaunchShape &ls, cudaStream_t st, SampleArgs &a) {
     a.nstages = ls.nstages; a.hashed = ls.hashed; a.slice_bytes = ls.slice_bytes; a.list_words = ls.list_words;
@@ -2907,7 +2835,6 @@ cudaError_t set_up_device(int device, DeviceShape &d) {
         (const void *)albireo_cluster_kernel<ALBIREO_F32, false>, (const void *)albireo_cluster_kernel<ALBIREO_BF16, false>,
         (const void *)albireo_cluster_kernel<ALBIREO_F16, false>, (const void *)albireo_cluster_kernel<ALBIREO_BF16, true>,
         (const void *)albireo_sample_kernel<ALBIREO_F32, false>, (const void *)albireo_sample_kernel<ALBIREO_BF16, false>, (const void *)albireo_sample_kernel<ALBIREO_F16, false>,
-        (const void *)albireo_ordered_sample_kernel<ALBIREO_F32>, (const void *)albireo_ordered_sample_kernel<ALBIREO_BF16>, (const void *)albireo_ordered_sample_kernel<ALBIREO_F16>,
         (const void *)albireo_sample_kernel<ALBIREO_F32, true>, (const void *)albireo_sample_kernel<ALBIREO_BF16, true>, (const void *)albireo_sample_kernel<ALBIREO_F16, true>,
         (const void *)albireo_stream_only_kernel<ALBIREO_F32>, (const void *)albireo_stream_only_kernel<ALBIREO_BF16>, (const void *)albireo_stream_only_kernel<ALBIREO_F16>};
     size_t st = 0;

@@ -116,3 +116,19 @@ def test_table_of_values_only_where_a_row_may_need_it(binding, sampler, par, cou
     logits, rest = batch(sampler, B, V, W.BF16, False, **{k: values[k] for k in par})
     ctas, name = launched(sampler, logits, **rest)
     assert ctas == 2 * B and ("ILi1ELb1E" in name) == counted, name
+
+
+# Batches around one and two rounds of the rows that are on the device at once: requests that all have a top-k, or a min-p, get the kernel of smaller and larger batches
+@pytest.mark.parametrize("par", [("top_k", "top_p"), ("min_p",), ()])
+@pytest.mark.parametrize("dtype", [W.BF16, W.F16, W.F32])
+def test_one_kernel_for_a_cta_per_row(binding, par, dtype):
+    s = binding.Sampler(max_rows=593, max_vocab=4096)
+    dev, names = s.device, set()
+    for B in (148, 296, 297, 592, 593):
+        values = dict(top_p=torch.full((B,), 0.9, device=dev), top_k=torch.full((B,), 40, dtype=torch.int32, device=dev), min_p=torch.full((B,), 0.1, device=dev))
+        logits, rest = batch(s, B, 4096, dtype, False, **{k: values[k] for k in par})
+        ctas, name = launched(s, logits, **rest)
+        assert ctas == B, (B, ctas, name)
+        names.add(name)
+    s.close()
+    assert len(names) == 1 and "albireo_sample_kernel" in names.pop(), names
