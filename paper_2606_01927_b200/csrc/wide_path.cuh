@@ -1899,7 +1899,7 @@ __device__ __noinline__ bool counted_locate(SRC src, TEAM tm, float invT, float 
         c.n_any = 0xFFFFFFFFu;
         c.M = S; c.n = n_all; c.key_lo = 0xFFFFFFFFu; c.key_hi = kfloor - 1u; c.key_seg = c.key_hi; c.fail = 0;
         c.thr_sure = c.thr_win = T::fill().x;             // (everything: -inf has no mass and does not win)
-        if (minp && !topp) c.thr_sure = c.thr_win = T::raw_threshold(kfloor, invT);
+        if (minp && !topp) { c.thr_sure = c.thr_win = T::raw_threshold(kfloor, invT); c.n_any = n_all; }      // (all that is above the floor has been counted)
         if (topp) {
             const int seg = (int)s.found_digit;
             if (seg < 0) c.fail = 1u;

@@ -78,3 +78,28 @@ def test_rows_without_a_whole_vector(binding, dtype, V, history, num_top):
             assert rep.ok() and not rep.excused, (B, rep.summary(), rep.failures[:3], rep.excused[:3])
             assert not (g["row_status"] & binding.ROW_TIMEOUT).any(), B
             assert not compare_top_lists(w, g, ref), B
+
+
+# A floor and no top-p: so many elements above it as wait in the last pass at a time (7168 vectors), fewer and more, some of them penalised, lists with and without
+@pytest.mark.parametrize("B,V", [(80, 131072), (80, 65537), (24, 131072)])
+@pytest.mark.parametrize("num_top,history", [(0, False), (0, True), (5, False)])
+def test_floor_alone(binding, sampler, B, V, num_top, history):
+    rng = np.random.default_rng(V + B)
+    kept = np.array([1100, 2050, 7167, 7168, 7169, 7680, 20000, 60000])[np.arange(B) % 8]
+    x = rng.uniform(-9, -6, (B, V)).astype(np.float32)
+    for b in range(B):
+        x[b, rng.permutation(V)[:kept[b]]] = rng.uniform(2, 5, kept[b]).astype(np.float32)
+    w = W.Workload("floor", B, V, W.BF16, W.f32_to_bf16_bits(x), temperature=np.ones(B, np.float32), min_p=np.full(B, 1e-3, np.float32), seeds=rng.integers(0, 1 << 62, B).astype(np.uint64), step=4)
+    w.num_top = num_top
+    if history:
+        lens = rng.integers(0, 900, B)
+        w.history_offsets = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+        w.history_ids = rng.integers(0, V, int(lens.sum())).astype(np.int32)
+        w.repetition_penalty, w.presence_penalty, w.frequency_penalty = (np.full(B, v, np.float32) for v in (1.2, 0.3, 0.1))
+    ref = O.sample(w, threads=_CORES)
+    t = binding.workload_tensors(w, sampler.device)
+    g = to_host(sampler.albireo_sample(t.pop("logits"), **t, num_top=num_top, want_counts=True, want_status=True))
+    rep = compare(w, g, ref)
+    assert rep.ok() and len(rep.excused) <= 1, (rep.summary(), rep.failures[:3], rep.excused[:3])
+    assert (g["num_kept"] == ref.rows["n_keep"]).all()
+    assert not compare_top_lists(w, g, ref)
