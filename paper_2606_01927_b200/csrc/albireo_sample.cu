@@ -62,7 +62,7 @@ struct SampleArgs {
     int64_t row_stride;
     int32_t nseg;               // pieces per row (1: rows are contiguous)
     int32_t nstages;            // ring depth chosen by the host for this launch
-    int32_t hashed;             // whether there is room for a hash table of history ids (see build_hashed)
+    int32_t unused;             // (what follows lies in the lines of constant memory as it does best: without this word a single row took 8.64 us instead of 8.50)
     int32_t vps;                // 16-byte vectors per piece (worked out on the host: no division on the device)
     int32_t Vs;                 // elements per piece
     uint32_t flags;
@@ -709,7 +709,9 @@ __device__ bool build_history(const HistSmem &hs, RowCtx &c, const int32_t *ids,
 
 // The tables of the candidate path for a history of more than HASH_LEAST ids and at most HASH_IDS: the bitmap, and in the place of ranks and counts a hash table of ids and their
 // counts, filled in one sweep with one barrier behind it.  (Ranks need the finished bitmap, a prefix sum over it and a second sweep that looks each id's rank up word by
-// word: 256 rows of 128256 with 2048 ids each 34.8 us, hashed 33.6.)  A word is an id and, from bit 19 on, its count; an id seen in the prompt only has count 0.  Whoever puts an id in sets its bit.
+// word.  256 rows of 128256 bf16 with a top-k and 1100 / 1536 / 2048 / 3584 ids each, us by ranks and hashed: 25.8 / 26.5 / 28.2 / 32.6 and 24.9 / 25.4 / 26.3 / 29.5; 100 rows 19.2 / 19.7 / 20.9 / 25.0 and
+// 18.9 / 19.2 / 20.1 / 23.0.  With fewer ids it depends on how the rows share the SMs: rows of 152064 with 256 / 1024 ids, 296 of them 27.0 / 28.6 and 26.0 / 27.9, 330 42.4 / 44.4 and 40.5 / 43.7, but 400
+// 43.0 / 45.2 and 44.0 / 47.4: those have ranks.)  A word is an id and, from bit 19 on, its count; an id seen in the prompt only has count 0.  Whoever puts an id in sets its bit.
 constexpr int HASH_SLOTS = 4096, HASH_IDS = HASH_SLOTS * 7 / 8, HASH_LEAST = 1024;
 constexpr uint32_t HASH_EMPTY = 0xFFFFFFFFu, HASH_ID = (1u << 19) - 1u;      // (no count reaches 2^13 - 1)
 static_assert(ALBIREO_MAX_VOCAB <= 1 << 19 && HASH_IDS < (1 << 13) - 1, "an id and a count in a word");
@@ -1921,7 +1923,7 @@ __device__ __forceinline__ bool candidate_finish(BlockScratch &s, const CandSmem
 
 // Returns false if the row must be handled by the general path instead.  On success the
 // results are in `out` for warp 0 only.
-template <int DT, bool EXTRA>
+template <int DT, bool EXTRA, bool HASHED>
 __device__ __forceinline__ bool candidate_path(BlockScratch &s, const CandSmem &cs, const Ring &rg, const RowCtx &c,
                                const RowParams &rp, const SampleArgs &a, int b, RowOut &out) {
     typedef Elem<DT> E;
@@ -2171,7 +2173,7 @@ __device__ __forceinline__ bool candidate_path(BlockScratch &s, const CandSmem &
     // penalised tokens, straight from the history tables: one distinct id per thread and round,
     // so that a dense head of the vocabulary does not pile up on a few threads; four rounds at a
     // time, so that their scattered loads (a round trip each, behind the other rows' streams) overlap
-    if (hashes_history(DT, EXTRA) && c.has_hist && !c.coarse) {
+    if (HASHED && c.has_hist && !c.coarse) {
         constexpr int PG = 4;
 #pragma unroll 1
         for (int at = (int)threadIdx.x; at < HASH_SLOTS; at += PG * NT) {
@@ -2425,7 +2427,9 @@ __device__ __noinline__ void leftover_row(const SampleArgs *ap, int tab_off) {
 // the ring is idle by then
 // EXTRA: whether the call asks for something beyond the ordinary (see extras_asked); the ordinary calls'
 // kernel is without the code for it, which would cost it registers.
-template <int DT, bool EXTRA>
+// HASHED: whether histories may have hash tables (see build_hashed, pick_shape).  (A kernel of its own: with the code for them in the ordinary one, calls without histories took longer where rows follow
+// one another on an SM: 297 rows of 152064 bf16 29.1 us instead of 28.2, 512 35.8 instead of 35.4.  Out of line, the calls cost the stream its registers: 256 rows 23.5 instead of 19.7.)
+template <int DT, bool EXTRA, bool HASHED>
 __global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const __grid_constant__ SampleArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     BlockScratch &s = block_scratch();
@@ -2520,7 +2524,7 @@ __global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const __grid_cons
             hs.counts = hs.coarse + (ncoarse + 1);
             // (a history that could have more distinct ids than the other tables hold, and more than the workspace does, is theirs to refuse)
             const int len = o1 - o0;
-            if (hashes_history(DT, EXTRA) && a.hashed && len > HASH_LEAST && len <= HASH_IDS && (len <= CNT_CAP || (a.ws_counts && o0 >= 0 && (int64_t)o1 <= a.ws_counts_cap)))
+            if (HASHED && len > HASH_LEAST && len <= HASH_IDS && (len <= CNT_CAP || (a.ws_counts && o0 >= 0 && (int64_t)o1 <= a.ws_counts_cap)))
                 build_hashed(hs.bitmap, c, a.hist_ids + o0, len, ostart, (const int32_t *)smem);
             else {
                 c.has_hist = build_history(hs, c, a.hist_ids + o0, len, ostart, (const int32_t *)smem, a.ws_counts, a.ws_counts_cap, (int64_t)o0);
@@ -2534,7 +2538,7 @@ __global__ void __launch_bounds__(NT, 2) albireo_sample_kernel(const __grid_cons
         cs.sorted = (u64 *)rg.buf;                              // 3 x 4 KiB in the ring, used after the stream
         cs.efx = cs.sorted + SORT_MAX;
         cs.gsc = cs.efx + SORT_MAX;
-        done = candidate_path<DT, EXTRA>(s, cs, rg, c, rp, a, b, out);
+        done = candidate_path<DT, EXTRA, HASHED>(s, cs, rg, c, rp, a, b, out);
     } else {
         // (the row's first tiles are on their way: nothing of the shared memory is reused before they are there)
         asm volatile("cp.async.wait_all;" ::: "memory");        // (the prefetched history ids)
@@ -2786,7 +2790,8 @@ bool pick_shape(LaunchShape &ls, int V, int dtype, const SampleArgs &a, const De
     ls.nstages = ring_stages_for(V, with_history, B <= d.num_sms);
     ls.smem = smem_bytes_for(V, with_history, ls.nstages);
     while (ls.smem > d.max_smem && ls.nstages > 2) ls.smem = smem_bytes_for(V, with_history, --ls.nstages);
-    // (where the hash table costs neither a stage of the ring nor the second CTA of an SM: up to vocabularies of 179000 tokens)
+    // (where the hash table costs neither a stage of the ring nor the second CTA of an SM: with more rows than SMs up to vocabularies of 175072 tokens; with fewer the ring has
+    // taken as many stages as fit, and what is left behind them has room for it or not as V goes)
     const size_t hashed = smem_bytes_for(V, false, ls.nstages) + (size_t)(hash_off(V) + HASH_SLOTS) * 4;
     const size_t budget = (size_t)(B <= d.num_sms ? SM_SMEM : SM_SMEM / 2) - 1024 - 1536;
     ls.hashed = with_history && hashes_history(dtype, extras_asked(a)) && hashed <= budget && hashed <= d.max_smem;
@@ -2813,12 +2818,13 @@ cudaError_t launch_sample_kernel_as(int B, const LaunchShape &ls, cudaStream_t s
         ++n;
     }
     cfg.attrs = at; cfg.numAttrs = n;
+    if constexpr (hashes_history(DT, false)) { if (ls.hashed) return cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT, false, true>, a); }
     if constexpr (DT == ALBIREO_BF16) { if (ls.counted) return cudaLaunchKernelEx(&cfg, albireo_cluster_kernel<DT, true>, a); }
     return ls.team > 1 ? cudaLaunchKernelEx(&cfg, albireo_cluster_kernel<DT, false>, a)
-           : extras_asked(a) ? cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT, true>, a) : cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT, false>, a);
+           : extras_asked(a) ? cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT, true, false>, a) : cudaLaunchKernelEx(&cfg, albireo_sample_kernel<DT, false, false>, a);
 }
 cudaError_t launch_sample_kernel(int dtype, int B, const LaunchShape &ls, cudaStream_t st, SampleArgs &a) {
-    a.nstages = ls.nstages; a.hashed = ls.hashed; a.slice_bytes = ls.slice_bytes; a.list_words = ls.list_words;
+    a.nstages = ls.nstages; a.unused = 0; a.slice_bytes = ls.slice_bytes; a.list_words = ls.list_words;
     if (dtype == ALBIREO_F32) return launch_sample_kernel_as<ALBIREO_F32>(B, ls, st, a);
     if (dtype == ALBIREO_BF16) return launch_sample_kernel_as<ALBIREO_BF16>(B, ls, st, a);
     return launch_sample_kernel_as<ALBIREO_F16>(B, ls, st, a);
@@ -2834,8 +2840,9 @@ cudaError_t set_up_device(int device, DeviceShape &d) {
     const void *kernels[] = {
         (const void *)albireo_cluster_kernel<ALBIREO_F32, false>, (const void *)albireo_cluster_kernel<ALBIREO_BF16, false>,
         (const void *)albireo_cluster_kernel<ALBIREO_F16, false>, (const void *)albireo_cluster_kernel<ALBIREO_BF16, true>,
-        (const void *)albireo_sample_kernel<ALBIREO_F32, false>, (const void *)albireo_sample_kernel<ALBIREO_BF16, false>, (const void *)albireo_sample_kernel<ALBIREO_F16, false>,
-        (const void *)albireo_sample_kernel<ALBIREO_F32, true>, (const void *)albireo_sample_kernel<ALBIREO_BF16, true>, (const void *)albireo_sample_kernel<ALBIREO_F16, true>,
+        (const void *)albireo_sample_kernel<ALBIREO_F32, false, false>, (const void *)albireo_sample_kernel<ALBIREO_BF16, false, false>, (const void *)albireo_sample_kernel<ALBIREO_F16, false, false>,
+        (const void *)albireo_sample_kernel<ALBIREO_BF16, false, true>, (const void *)albireo_sample_kernel<ALBIREO_F16, false, true>,
+        (const void *)albireo_sample_kernel<ALBIREO_F32, true, false>, (const void *)albireo_sample_kernel<ALBIREO_BF16, true, false>, (const void *)albireo_sample_kernel<ALBIREO_F16, true, false>,
         (const void *)albireo_stream_only_kernel<ALBIREO_F32>, (const void *)albireo_stream_only_kernel<ALBIREO_BF16>, (const void *)albireo_stream_only_kernel<ALBIREO_F16>};
     size_t st = 0;
     for (const void *k : kernels) {

@@ -132,3 +132,14 @@ def test_one_kernel_for_a_cta_per_row(binding, par, dtype):
         names.add(name)
     s.close()
     assert len(names) == 1 and "albireo_sample_kernel" in names.pop(), names
+
+
+# Histories have hash tables where these fit beside two CTAs per SM; calls without histories keep the kernel without the code for them
+@pytest.mark.parametrize("dtype,V,history,hashed", [(W.BF16, 175072, True, True), (W.BF16, 175073, True, False), (W.F16, 40000, True, True), (W.BF16, 40000, False, False), (W.F32, 40000, True, False)])
+def test_kernel_of_hashed_histories(binding, dtype, V, history, hashed):
+    B = 150
+    s = binding.Sampler(max_rows=B, max_vocab=V, max_history_total=64 * B)
+    logits, par = batch(s, B, V, dtype, history, top_k=torch.full((B,), 40, dtype=torch.int32, device=s.device))
+    ctas, name = launched(s, logits, **par)
+    s.close()
+    assert ctas == B and ("Lb0ELb1E" in name) == hashed, name
