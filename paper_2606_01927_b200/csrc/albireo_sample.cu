@@ -1847,7 +1847,7 @@ __device__ __noinline__ void max_and_count() {
     const float invT = row_shared<DT>().c.invT;
     const uint32_t fin_thr = VecTest<DT>::finite_threshold(invT);
     uint32_t kbest = 0, nfin = 0;
-    src.vectors([&](const uint4 &q, int) {
+    src.template vectors<4>([&](const uint4 &q, int) {
         const uint32_t k = VecTest<DT>::vmax_key(q, invT);
         kbest = k > kbest ? k : kbest;
         nfin += (uint32_t)Elem<DT>::PER_VEC - VecTest<DT>::count_not_finite(q, fin_thr, invT);

@@ -123,7 +123,7 @@ __device__ __forceinline__ float pick_element(const uint4 &q, int x) {
 
 // A callee that takes two vectors gets two of a thread's at a time from global memory, and elsewhere one and nothing (-inf, id -1).
 template <class F> constexpr bool by_pairs = std::is_invocable<F, uint4, uint4, int, int>::value;
-// A callee may come with a test of four vectors at once: where no lane's answer is true the callee is not called for them (it must
+// A callee may come with a test of two vectors at once: where no lane's answer is true the callee is not called for them (it must
 // have nothing to do there).
 struct NoTest {};
 
@@ -131,6 +131,9 @@ struct NoTest {};
 // vectors are on their way while it works on another.  Penalised tokens are masked out of the vectors
 // and come from the history tables.  Both loops have the same trip count in every lane of a warp (lanes
 // past the end see -inf), so that the callee may use warp collectives, but no block barriers.
+// How many wait is what the registers of the passes leave room for: 4 where the callee keeps a sum or a maximum, else 2 (with 4, the functions around the passes spilled 124 bytes instead of
+// 32 to 60), 1 where whole vectors are raced; 2 and 2 where pairs are tested.  148 rows of 128256, top-p, us with 4 everywhere and so: fp32 98.5 and 93.3, f16 77.8 and 72.8; 256 rows of fp32, which
+// the L2 does not hold, 143.9 and 134.7 (136.9 from a ring); with 2 for the largest element, too, rows without a cut 55.1 -> 59.
 // (What the loop does not touch per vector stays in shared memory: a pass needs its registers for the elements.)
 // What bounds a pass is shared memory and issue slots, not the loads: with the vectors brought into shared memory by bulk copies, as before,
 // both the copies and the reads back were in the way of the callee's own accesses, and each tile of 32 KB cost a hand-shake of all
@@ -173,7 +176,7 @@ struct RowSlice {
         return q;
     }
     // Those of the row's vectors from `first` on and before `end`, piece after piece (lanes past the end of one see -inf and the id behind the last).
-    template <int AHEAD = 4, class F, class T = NoTest> __device__ __forceinline__ void vectors(F &&f, T &&test = T(), int first = 0, int end = 0x7FFFFFFF) const {
+    template <int AHEAD = 2, class F, class T = NoTest> __device__ __forceinline__ void vectors(F &&f, T &&test = T(), int first = 0, int end = 0x7FFFFFFF) const {
         constexpr bool PAIRS = by_pairs<F>, TESTED = !std::is_same<std::decay_t<T>, NoTest>::value;
         const RowShared &r = row_shared<DT>();
         const int head = r.head, end_id = head + r.nvec * E::PER_VEC;
@@ -193,20 +196,17 @@ struct RowSlice {
             auto load = [&](int v) -> uint4 { return v < hi ? __ldg(vp + v) : VecTest<DT>::fill(); };
             auto id_of = [&](int v) { return v < hi ? head + v * E::PER_VEC : end_id; };
             if constexpr (TESTED) {
-                // four at a time, and one after another where some matter
+                // two at a time, the next two on their way
+                uint4 q0 = load(lo + (int)threadIdx.x), q1 = load(lo + (int)threadIdx.x + NT);
 #pragma unroll 1
-                for (int v0 = lo + (int)threadIdx.x; v0 - (int)threadIdx.x < hi; v0 += 4 * NT) {
-                    uint4 q[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) q[u] = load(v0 + u * NT);
-                    if (!__any_sync(0xFFFFFFFFu, test(q))) continue;
+                for (int v0 = lo + (int)threadIdx.x; v0 - (int)threadIdx.x < hi; v0 += 2 * NT) {
+                    const uint4 x = q0, y = q1;
+                    q0 = load(v0 + 2 * NT); q1 = load(v0 + 3 * NT);
+                    if (!__any_sync(0xFFFFFFFFu, test(x, y))) continue;
 #pragma unroll 1
-                    for (int u = 0; u < 4; ++u) {
-                        uint4 x = q[0];
-#pragma unroll
-                        for (int w = 1; w < 4; ++w) if (u == w) x = q[w];
+                    for (int u = 0; u < 2; ++u) {
                         const int i0 = id_of(v0 + u * NT);
-                        f(masked(x, i0), i0);
+                        f(masked(u ? y : x, i0), i0);
                     }
                 }
             } else {
@@ -274,7 +274,7 @@ struct SmemSlice {
         extern __shared__ __align__(128) unsigned char smem[];
         return v < 0 ? VecTest<DT>::fill() : ((const uint4 *)(smem + vec_off))[v];
     }
-    template <int AHEAD = 4, class F, class T = NoTest> __device__ __forceinline__ void vectors(F &&f, T && = T(), int first = 0, int end = 0x7FFFFFFF) const {
+    template <int AHEAD = 2, class F, class T = NoTest> __device__ __forceinline__ void vectors(F &&f, T && = T(), int first = 0, int end = 0x7FFFFFFF) const {
         extern __shared__ __align__(128) unsigned char smem[];
         const uint4 *vec = (const uint4 *)(smem + vec_off);
         constexpr bool PAIRS = by_pairs<F>;
@@ -420,7 +420,7 @@ __device__ __forceinline__ void mass_pass(const SRC &src, float invT, float zmax
         if (FLOOR && MODE != INSIDE_WINDOW) S_all.add2(e);
     };
     const uint32_t thr = VecTest<DT>::raw_threshold(key_of(zmax - 29.5f), invT);
-    src.vectors([&](const uint4 &q, int) {
+    src.template vectors<MODE == SUM_ONLY ? 4 : 2>([&](const uint4 &q, int) {
         if (!VecTest<DT>::may_pass(q, thr, invT)) return;          // nothing within 42 octaves of the maximum
 #pragma unroll
         for (int j = 0; j < E::PER_VEC; j += 2) add2(scores_of(E::get(q, j), E::get(q, j + 1), invT, minus0));
@@ -1070,7 +1070,7 @@ __device__ __forceinline__ void final_pass(const SRC &src, BlockScratch &s, Part
                 push(i0 + x, __fmul_rn(pick_element<DT>(q, x), invT), bits != 0);
                 bits &= bits - 1u;
             }
-        }, [&](const uint4 (&q)[4]) { return VecTest<DT>::any_may_pass(q, thr, invT); });
+        }, [&](const uint4 &x, const uint4 &y) { return VecTest<DT>::may_pass(x, thr, invT) || VecTest<DT>::may_pass(y, thr, invT); });
     }
     src.extras([&](int i, float z) { push(i, z, z >= s.fa.zfloor); });
     work(0);
@@ -1650,7 +1650,7 @@ __device__ __noinline__ uint32_t count_finite(SRC src, float invT) {
     BlockScratch &s = block_scratch();
     const uint32_t thr = VecTest<ALBIREO_BF16>::finite_threshold(invT);
     uint32_t n = 0;
-    src.vectors([&](const uint4 &q, int) { n += 8u - VecTest<ALBIREO_BF16>::count_not_finite(q, thr, invT); });
+    src.template vectors<4>([&](const uint4 &q, int) { n += 8u - VecTest<ALBIREO_BF16>::count_not_finite(q, thr, invT); });
     return (uint32_t)block_sum_u64(n);
 }
 // Row (or slice) after the counting pass and a barrier: the number of finite scores among the vectors' elements, and what
