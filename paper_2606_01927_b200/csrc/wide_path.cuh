@@ -1709,7 +1709,10 @@ __device__ __noinline__ Partial counted_final_pass(SRC src) {
         const volatile CountedCut &c = cut;
         const float invT = *(const volatile float *)&s.fa.invT;
         const uint32_t thr_sure = c.thr_sure, thr_win = c.thr_win;
-        if (s.ga.num_top > 0) append_elements(q, i0, T::elem_bits(q, c.thr_top, invT), invT);
+        if (s.ga.num_top > 0) {
+            const uint32_t bits = T::elem_bits(q, c.thr_top, invT);
+            if (__any_sync(0xFFFFFFFFu, bits != 0u)) append_elements(q, i0, bits, invT);
+        }
         uint32_t in = edge_bits(edge_mask(q.x, thr_win, thr_sure), edge_mask(q.y, thr_win, thr_sure), edge_mask(q.z, thr_win, thr_sure), edge_mask(q.w, thr_win, thr_sure));
         while (in) {
             const int x = __ffs(in) - 1;
