@@ -163,7 +163,6 @@ struct RowSlice {
     __device__ __forceinline__ int end_id() const { return row_shared<DT>().head + row_shared<DT>().nvec * E::PER_VEC; }
     __device__ __forceinline__ int elements() const { return row_shared<DT>().nvec * E::PER_VEC; }
     __device__ __forceinline__ int segments() const { return row_segments<DT>(); }      // (counted rows: see CountedSegs)
-    __device__ __forceinline__ int count() const { return row_shared<DT>().nvec; }
     // vector v by itself (v < 0: none)
     __device__ __forceinline__ uint4 vector(int v) const {
         if (v < 0) return VecTest<DT>::fill();
@@ -175,8 +174,8 @@ struct RowSlice {
         }
         return q;
     }
-    // Those of the row's vectors from `first` on and before `end`, piece after piece (lanes past the end of one see -inf and the id behind the last).
-    template <int AHEAD = 2, class F, class T = NoTest> __device__ __forceinline__ void vectors(F &&f, T &&test = T(), int first = 0, int end = 0x7FFFFFFF) const {
+    // The row's vectors, piece after piece (lanes past the end of one see -inf and the id behind the last).
+    template <int AHEAD = 2, class F, class T = NoTest> __device__ __forceinline__ void vectors(F &&f, T &&test = T()) const {
         constexpr bool PAIRS = by_pairs<F>, TESTED = !std::is_same<std::decay_t<T>, NoTest>::value;
         const RowShared &r = row_shared<DT>();
         const int head = r.head, end_id = head + r.nvec * E::PER_VEC;
@@ -191,8 +190,8 @@ struct RowSlice {
 #pragma unroll 1
         for (int j = 0; j < r.c.nseg; ++j) {
             const bool whole = r.c.nseg == 1;
-            const int v_lo = whole ? 0 : j * r.vps, lo = max(first, v_lo), hi = min(min(r.nvec, end), whole ? r.nvec : v_lo + r.vps);
-            const uint4 *const vp = (whole ? r.vp : (const uint4 *)r.c.seg_base[j]) - v_lo;
+            const int lo = whole ? 0 : j * r.vps, hi = whole ? r.nvec : min(r.nvec, lo + r.vps);
+            const uint4 *const vp = (whole ? r.vp : (const uint4 *)r.c.seg_base[j]) - lo;
             auto load = [&](int v) -> uint4 { return v < hi ? __ldg(vp + v) : VecTest<DT>::fill(); };
             auto id_of = [&](int v) { return v < hi ? head + v * E::PER_VEC : end_id; };
             if constexpr (TESTED) {
@@ -269,20 +268,18 @@ struct SmemSlice {
     __device__ __forceinline__ int end_id() const { return id0 + nvec * E::PER_VEC; }
     __device__ __forceinline__ int elements() const { return nvec * E::PER_VEC; }
     __device__ __forceinline__ int segments() const { return block_scratch().seg_off; }      // (in a register it was spilled)
-    __device__ __forceinline__ int count() const { return nvec; }
     __device__ __forceinline__ uint4 vector(int v) const {
         extern __shared__ __align__(128) unsigned char smem[];
         return v < 0 ? VecTest<DT>::fill() : ((const uint4 *)(smem + vec_off))[v];
     }
-    template <int AHEAD = 2, class F, class T = NoTest> __device__ __forceinline__ void vectors(F &&f, T && = T(), int first = 0, int end = 0x7FFFFFFF) const {
+    template <int AHEAD = 2, class F, class T = NoTest> __device__ __forceinline__ void vectors(F &&f, T && = T()) const {
         extern __shared__ __align__(128) unsigned char smem[];
         const uint4 *vec = (const uint4 *)(smem + vec_off);
         constexpr bool PAIRS = by_pairs<F>;
-        const int n = min(nvec, end);
 #pragma unroll 1
-        for (int base = first; base < n; base += NT) {
+        for (int base = 0; base < nvec; base += NT) {
             const int v = base + (int)threadIdx.x, i0 = id0 + v * E::PER_VEC;
-            const uint4 q = v < n ? vec[v] : VecTest<DT>::fill();
+            const uint4 q = v < nvec ? vec[v] : VecTest<DT>::fill();
             if constexpr (PAIRS) f(q, VecTest<DT>::fill(), i0, -1);
             else f(q, i0);
         }
@@ -371,14 +368,16 @@ struct alignas(16) CountedSegs {
     uint32_t high;                    // some of them are above the table's
     CountedCut cut;
 };
-// The slices of a cluster begin behind the team's words; by one CTA the row's own block and the ring of its passes do.  (At 128 bytes: 30 rows
+// The slices of a cluster begin behind the team's words, by one CTA the row's own block does.  (At 128 bytes: 30 rows
 // of 152064 with a top-k took 10.7 us with slices at 16, 10.3 so.)
 __host__ __device__ constexpr int team_off(bool counted) { return counted ? CT_BYTES : WIDE_BYTES; }
 __host__ __device__ constexpr int slice_off(bool counted) { return (team_off(counted) + (int)sizeof(TeamWords) + 127) & ~127; }
 template <bool COUNTED> __device__ __forceinline__ TeamWords &team_words() { extern __shared__ __align__(128) unsigned char smem[]; return *(TeamWords *)(smem + team_off(COUNTED)); }
 __host__ __device__ constexpr bool counts_rows(int dt) { return dt == ALBIREO_BF16; }      // the kernel of one CTA per row
 __host__ __device__ constexpr int row_off(int dt) { return slice_off(counts_rows(dt)) + (counts_rows(dt) ? (int)sizeof(CountedSegs) : 0); }
-__host__ __device__ constexpr int row_front(int dt) { return (row_off(dt) + (int)sizeof(RowShared) + 127) & ~127; }      // what a wide row needs of one CTA
+// (the tables of the history, which the passes ask, lie behind the ring of at least two stages)
+constexpr int row_end(int dt) { return row_off(dt) + (int)sizeof(RowShared); }
+static_assert(row_end(ALBIREO_F32) <= COMMON_BYTES + 2 * STAGE_BYTES && row_end(ALBIREO_BF16) <= COMMON_BYTES + 2 * STAGE_BYTES && row_end(ALBIREO_F16) <= COMMON_BYTES + 2 * STAGE_BYTES, "a wide row in front of its tables");
 template <int DT> __device__ __forceinline__ constexpr int row_segments() { return slice_off(counts_rows(DT)); }
 template <int DT> __device__ __forceinline__ RowShared &row_shared() { extern __shared__ __align__(128) unsigned char smem[]; return *(RowShared *)(smem + row_off(DT)); }
 static_assert(sizeof(CountedSegs) % 16 == 0 && sizeof(RowShared) % 8 == 0, "what follows is aligned");
